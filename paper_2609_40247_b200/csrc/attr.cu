@@ -609,9 +609,15 @@ __global__ void __launch_bounds__(AT_THREADS, AT_RES_MINB) k_attr_resolve(AttrAr
 #define AT_OPS_ITEMS 4
 #endif
 #define AT_OPS_TILE (AT_THREADS * AT_OPS_ITEMS)
+// adds a group of device records to the row of their window
+__device__ __forceinline__ void attr_emit(ta_attr_summary *sm, const u64 *t) {
+  if (t[0]) atomicAdd((u64 *)&sm->n_attributed, t[0]);
+  if (t[1]) atomicAdd((u64 *)&sm->n_no_launch, t[1]);
+  if (t[2]) atomicAdd((u64 *)&sm->n_no_op, t[2]);
+}
 __global__ void __launch_bounds__(AT_THREADS, AT_OPS_MINB) k_attr_ops(AttrArgs a) {
   constexpr int IT = AT_OPS_ITEMS;
-  __shared__ u64 red[AT_THREADS / 32];
+  __shared__ u64 red[3][AT_THREADS / 32];
   __shared__ int s_lane0, s_lane1;
   if (ta_failed(a.status)) return;
   const int tid = threadIdx.x, lane = tid & 31;
@@ -672,34 +678,35 @@ __global__ void __launch_bounds__(AT_THREADS, AT_OPS_MINB) k_attr_ops(AttrArgs a
 #pragma unroll
   for (int j = 0; j < IT; j++)
     if (p0 + j < a.n_valid && (kd[j] == TA_KIND_KERNEL || kd[j] == TA_KIND_MEMCPY)) pm |= 1u << j;
-  u64 packed = 0;  // attributed | no launch << 20 | no op << 40, for the thread's first lane
-  int lm = -1;
+  u64 acc[3] = {0, 0, 0};  // attributed, no launch, no operator, for the thread's first window
+  int wm = -1;
   {
     int l = l0;
     int64_t next_off = l >= 0 ? (int64_t)a.lane_off[l + 1] : LLONG_MAX;
+    int win = l >= 0 ? a.lane_window[l] : 0;
 #pragma unroll
     for (int j = 0; j < IT; j++) {
       if (!(pm & (1u << j))) { op[j] = -1; continue; }
       const int64_t p = p0 + j;
-      while (p >= next_off) { l++; next_off = a.lane_off[l + 1]; }
-      u64 add;
-      if (lo[j] < 0) add = 1ull << 20;
-      else if (op[j] < 0) add = 1ull << 40;
-      else {
-        add = 1ull;
+      if (p >= next_off) {
+        do { l++; next_off = a.lane_off[l + 1]; } while (p >= next_off);
+        win = a.lane_window[l];
+      }
+      if (lo[j] >= 0 && op[j] >= 0) {
         const int32_t r = op[j];
         // (the kernel count of the operator is accumulated from the launch side, in k_attr_resolve)
         atomicAdd((u64 *)&a.op_ns[r], (u64)(en[j] - st[j]));
         atomicMax(&a.op_first[r], ~((u64)st[j] ^ (1ull << 63)));
         atomicMax(&a.op_last[r], (u64)en[j] ^ (1ull << 63));
       }
-      if (lm < 0) lm = l;
-      if (l == lm && l - l0 <= 1) packed += add;
-      else {
-        ta_attr_summary *sm = &a.sum[a.lane_window[l]];
-        if (add == 1ull) atomicAdd((u64 *)&sm->n_attributed, 1ull);
-        else if (add == (1ull << 20)) atomicAdd((u64 *)&sm->n_no_launch, 1ull);
-        else atomicAdd((u64 *)&sm->n_no_op, 1ull);
+      if (wm < 0) wm = win;
+      if (win == wm) {
+        acc[0] += lo[j] >= 0 && op[j] >= 0;
+        acc[1] += lo[j] < 0;
+        acc[2] += lo[j] >= 0 && op[j] < 0;
+      } else {
+        const u64 one[3] = {lo[j] >= 0 && op[j] >= 0, lo[j] < 0, lo[j] >= 0 && op[j] < 0};
+        attr_emit(&a.sum[win], one);
       }
     }
     const int64_t plast = min(tile_start + AT_OPS_TILE, a.n_valid) - 1;
@@ -718,25 +725,9 @@ __global__ void __launch_bounds__(AT_THREADS, AT_OPS_MINB) k_attr_ops(AttrArgs a
       if (p0 + j < a.n) a.op_of[p0 + j] = op[j];
   }
   __syncthreads();
-  const int l1 = s_lane1;
-  for (int li = 0; li < 2; li++) {
-    const int l = l0 + li;
-    if (l0 < 0 || l > l1) break;
-    if (a.lane_domain[l] != 1) continue;
-    u64 v = warp_reduce(lm == l ? packed : 0, OpAdd());
-    __syncthreads();
-    if (lane == 0) red[tid >> 5] = v;
-    __syncthreads();
-    if (tid == 0) {
-      u64 t = 0;
-      for (int w = 0; w < AT_THREADS / 32; w++) t += red[w];
-      const u64 m = (1ull << 20) - 1;
-      ta_attr_summary *sm = &a.sum[a.lane_window[l]];
-      if (t & m) atomicAdd((u64 *)&sm->n_attributed, t & m);
-      if ((t >> 20) & m) atomicAdd((u64 *)&sm->n_no_launch, (t >> 20) & m);
-      if ((t >> 40) & m) atomicAdd((u64 *)&sm->n_no_op, (t >> 40) & m);
-    }
-  }
+  if (l0 < 0) return;
+  fold_by_window<3, 0, AT_THREADS / 32>(acc, wm, a.lane_window[l0], a.lane_window[s_lane1], red,
+                                        [&](int w, const u64 *t) { attr_emit(&a.sum[w], t); });
 }
 
 // first/last were accumulated in an order-preserving unsigned encoding (0 = untouched)

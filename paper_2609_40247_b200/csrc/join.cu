@@ -47,35 +47,6 @@ struct JoinArgs {
 __device__ __forceinline__ u64 bias64(i64 v) { return (u64)v ^ (1ull << 63); }
 __device__ __forceinline__ i64 unbias64(u64 v) { return (i64)(v ^ (1ull << 63)); }
 
-// block-wide reduction helper (all threads call); smem >= 33 u64
-__device__ __forceinline__ u64 blk_reduce(u64 v, bool is_max, u64 *smem) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  v = is_max ? warp_reduce(v, OpMax()) : warp_reduce(v, OpAdd());
-  __syncthreads();
-  if (lane == 0) smem[warp] = v;
-  __syncthreads();
-  if (warp == 0) {
-    u64 w = lane < (int)(blockDim.x >> 5) ? smem[lane] : 0;
-    w = is_max ? warp_reduce(w, OpMax()) : warp_reduce(w, OpAdd());
-    if (lane == 0) smem[32] = w;
-  }
-  __syncthreads();
-  return smem[32];
-}
-
-// lanes touched by the CTA's selected items -> [l0, l1] (l1 < l0 if none)
-__device__ __forceinline__ void tile_lane_range(int my_lo, int my_hi, int *s_lo, int *s_hi, int *l0,
-                                                int *l1) {
-  if (threadIdx.x == 0) { *s_lo = INT_MAX; *s_hi = -1; }
-  __syncthreads();
-  if (my_hi >= 0) { atomicMin(s_lo, my_lo); atomicMax(s_hi, my_hi); }
-  __syncthreads();
-  *l0 = *s_lo;
-  *l1 = *s_hi;
-  __syncthreads();
-}
-
-
 // ---- direct path: fill the table -------------------------------------------
 __global__ void __launch_bounds__(JN_THREADS) k_join_build(JoinArgs a) {
   __shared__ int s_lane0;
@@ -110,17 +81,6 @@ __global__ void __launch_bounds__(JN_THREADS) k_join_build(JoinArgs a) {
   }
 }
 
-template <bool DIRECT>
-__device__ __forceinline__ int32_t winner_of(const JoinArgs &a, int64_t p, int slot) {
-  if (!DIRECT) return a.found[p];
-  i64 base = a.slot_base[slot];
-  if (base < 0) return -1;
-  i64 c = a.corr[p];
-  if (c < a.slot_min[slot] || c > a.slot_max[slot]) return -1;
-  u32 v = a.table[base + (c - a.slot_min[slot])];
-  return v == EMPTY_U32 ? -1 : (int32_t)v;
-}
-
 // ---- pass 2: probes ----------------------------------------------------------
 // 256 threads x JP_ITEMS consecutive positions; every output column is written once.
 #define JP_THREADS 256
@@ -131,6 +91,19 @@ __device__ __forceinline__ int32_t winner_of(const JoinArgs &a, int64_t p, int s
 #define JP_ITEMS 8
 #endif
 #define JP_TILE (JP_THREADS * JP_ITEMS)
+
+// adds a group of probes to the row of their window
+__device__ __forceinline__ void join_emit(ta_join_summary *sm, const u64 *t) {
+  if (t[0] == 0) return;
+  atomicAdd((u64 *)&sm->n_probe, t[0]);
+  if (t[1] == 0) return;
+  atomicAdd((u64 *)&sm->n_matched, t[1]);
+  atomicAdd((u64 *)&sm->sum_latency, t[2]);
+  atomicAdd((u64 *)&sm->sum_queue, t[3]);
+  atomicMax((i64 *)&sm->max_latency, unbias64(t[4]));
+  atomicMin((i64 *)&sm->min_latency, unbias64(~t[5]));
+  atomicMax((i64 *)&sm->max_queue, (i64)t[6]);
+}
 
 template <bool DIRECT>
 __global__ void __launch_bounds__(JP_THREADS, JP_MINB) k_join_probe(JoinArgs a) {
@@ -172,19 +145,24 @@ __global__ void __launch_bounds__(JP_THREADS, JP_MINB) k_join_probe(JoinArgs a) 
   for (int j = 0; j < IT; j++)
     if (p0 + j < a.n_valid && (kd[j] == TA_KIND_KERNEL || kd[j] == TA_KIND_MEMCPY)) pm |= 1u << j;
   int32_t lo[IT];
-  int ln[IT];
+  int wn[IT];  // window of the probe
   {
     int l = l0;
     int64_t next_off = l >= 0 ? (int64_t)a.lane_off[l + 1] : LLONG_MAX;
     int slot = l >= 0 ? a.lane_slot[l] : 0;
+    int win = l >= 0 ? a.lane_window[l] : 0;
 #pragma unroll
     for (int j = 0; j < IT; j++) {
       lo[j] = -1;
-      ln[j] = -1;
+      wn[j] = -1;
       if (pm & (1u << j)) {
         const int64_t p = p0 + j;
-        while (p >= next_off) { l++; next_off = a.lane_off[l + 1]; slot = a.lane_slot[l]; }
-        ln[j] = l;
+        if (p >= next_off) {
+          do { l++; next_off = a.lane_off[l + 1]; } while (p >= next_off);
+          slot = a.lane_slot[l];
+          win = a.lane_window[l];
+        }
+        wn[j] = win;
         if (DIRECT) {
           const i64 base = a.slot_base[slot];
           if (base >= 0 && c[j] >= a.slot_min[slot] && c[j] <= a.slot_max[slot]) {
@@ -210,8 +188,9 @@ __global__ void __launch_bounds__(JP_THREADS, JP_MINB) k_join_probe(JoinArgs a) 
     if (lo[j] >= 0) { ls[j] = a.ts[lo[j]]; le[j] = a.te[lo[j]]; }
   }
   i64 lat[IT], q[IT];
-  u64 np = 0, nm = 0, sl = 0, sq = 0, mxl = 0, mnl_inv = 0, mxq = 0;
-  int lm = -1;
+  // probes, matches, latencies and delays summed; largest latency, largest complement, largest delay
+  u64 acc[7] = {0, 0, 0, 0, 0, 0, 0};
+  int wm = -1;
 #pragma unroll
   for (int j = 0; j < IT; j++) {
     lat[j] = q[j] = 0;
@@ -223,78 +202,43 @@ __global__ void __launch_bounds__(JP_THREADS, JP_MINB) k_join_probe(JoinArgs a) 
       q[j] = d > 0 ? d : 0;
       atomicAdd(&a.kol[lo[j]], 1);
     }
-    if (lm < 0) lm = ln[j];
-    if (ln[j] == lm && ln[j] - l0 <= 1) {
-      np++;
+    if (wm < 0) wm = wn[j];
+    if (wn[j] == wm) {
+      acc[0]++;
       if (matched) {
-        nm++;
-        sl += (u64)lat[j];
-        sq += (u64)q[j];
-        mxl = max(mxl, bias64(lat[j]));
-        mnl_inv = max(mnl_inv, ~bias64(lat[j]));
-        mxq = max(mxq, (u64)q[j]);
+        acc[1]++;
+        acc[2] += (u64)lat[j];
+        acc[3] += (u64)q[j];
+        acc[4] = max(acc[4], bias64(lat[j]));
+        acc[5] = max(acc[5], ~bias64(lat[j]));
+        acc[6] = max(acc[6], (u64)q[j]);
       }
-    } else {  // a thread that straddles a lane boundary, or a third lane in the tile
-      ta_join_summary *sm = &a.sum[a.lane_window[ln[j]]];
-      atomicAdd((u64 *)&sm->n_probe, 1ull);
-      if (matched) {
-        atomicAdd((u64 *)&sm->n_matched, 1ull);
-        atomicAdd((u64 *)&sm->sum_latency, (u64)lat[j]);
-        atomicAdd((u64 *)&sm->sum_queue, (u64)q[j]);
-        atomicMax((i64 *)&sm->max_latency, lat[j]);
-        atomicMin((i64 *)&sm->min_latency, lat[j]);
-        atomicMax((i64 *)&sm->max_queue, q[j]);
-      }
+    } else {  // a thread that straddles a window boundary
+      const u64 one[7] = {1, matched ? 1ull : 0ull, (u64)lat[j], (u64)q[j], bias64(lat[j]), ~bias64(lat[j]), (u64)q[j]};
+      join_emit(&a.sum[wn[j]], one);
     }
   }
   storen_i32<IT>(a.launch_of, p0, a.n, lo);
   storen_i64<IT>(a.latency, p0, a.n, lat);
   storen_i64<IT>(a.qdelay, p0, a.n, q);
   __syncthreads();
-  const int l1 = s_lane1;
-  for (int li = 0; li < 2; li++) {
-    const int l = l0 + li;
-    if (l0 < 0 || l > l1) break;
-    if (a.lane_domain[l] != 1) continue;  // uniform over the CTA
-    const bool mine = lm == l;
-    u64 r[7] = {mine ? np : 0, mine ? nm : 0, mine ? sl : 0, mine ? sq : 0,
-                mine ? mxl : 0, mine ? mnl_inv : 0, mine ? mxq : 0};
-#pragma unroll
-    for (int k = 0; k < 4; k++) r[k] = warp_reduce(r[k], OpAdd());
-#pragma unroll
-    for (int k = 4; k < 7; k++) r[k] = warp_reduce(r[k], OpMax());
-    __syncthreads();
-    if (lane == 0)
-#pragma unroll
-      for (int k = 0; k < 7; k++) red[k][tid >> 5] = r[k];
-    __syncthreads();
-    if (tid == 0) {
-      u64 t[7] = {0, 0, 0, 0, 0, 0, 0};
-      for (int w = 0; w < JP_THREADS / 32; w++) {
-        for (int k = 0; k < 4; k++) t[k] += red[k][w];
-        for (int k = 4; k < 7; k++) t[k] = max(t[k], red[k][w]);
-      }
-      if (t[0]) {
-        ta_join_summary *sm = &a.sum[a.lane_window[l]];
-        atomicAdd((u64 *)&sm->n_probe, t[0]);
-        if (t[1]) {
-          atomicAdd((u64 *)&sm->n_matched, t[1]);
-          atomicAdd((u64 *)&sm->sum_latency, t[2]);
-          atomicAdd((u64 *)&sm->sum_queue, t[3]);
-          atomicMax((i64 *)&sm->max_latency, unbias64(t[4]));
-          atomicMin((i64 *)&sm->min_latency, unbias64(~t[5]));
-          atomicMax((i64 *)&sm->max_queue, (i64)t[6]);
-        }
-      }
-    }
-  }
+  if (l0 < 0) return;
+  fold_by_window<4, 3, JP_THREADS / 32>(acc, wm, a.lane_window[l0], a.lane_window[s_lane1], red,
+                                        [&](int w, const u64 *t) { join_emit(&a.sum[w], t); });
 }
 
 // ---- pass 3: launch statistics (duplicates, orphans) ---------------------------
 #define JS_TILE (JP_THREADS * 8)
+// adds a group of launches to the row of their window
+__device__ __forceinline__ void launch_emit(ta_join_summary *sm, const u64 *t) {
+  if (t[0]) atomicAdd((u64 *)&sm->n_launch, t[0]);
+  if (t[1]) atomicAdd((u64 *)&sm->n_dup_launch, t[1]);
+  if (t[2]) atomicAdd((u64 *)&sm->n_orphan_launch, t[2]);
+}
+
 template <bool DIRECT>
 __global__ void __launch_bounds__(JP_THREADS) k_join_launch_stats(JoinArgs a) {
-  __shared__ u64 red[JP_THREADS / 32];
+  __shared__ u64 red[3][JP_THREADS / 32];
   __shared__ int s_lane0, s_lane1;
   if (ta_failed(a.status)) return;
   const int tid = threadIdx.x, lane = tid & 31;
@@ -329,21 +273,21 @@ __global__ void __launch_bounds__(JP_THREADS) k_join_launch_stats(JoinArgs a) {
 #pragma unroll
   for (int j = 0; j < 8; j++)
     if (p0 + j < a.n_valid && kd[j] == TA_KIND_LAUNCH) lmask |= 1u << j;
-  u64 packed = 0;  // n_launch | n_dup << 20 | n_orphan << 40 for the thread's first lane
-  int lm = -1;
+  u64 acc[3] = {0, 0, 0};  // launches, duplicates, orphans of the thread's first window
+  int wm = -1;
   {
     int l = l0;
-    int64_t next_off = l >= 0 ? (int64_t)a.lane_off[l + 1] : LLONG_MAX;
-    int ln[8];
+    int64_t next_off = (int64_t)a.lane_off[l + 1];
+    int wn[8];
     int32_t win[8];
 #pragma unroll
     for (int j = 0; j < 8; j++) {
-      ln[j] = -1;
+      wn[j] = -1;
       win[j] = -1;
       if (!(lmask & (1u << j))) continue;
       const int64_t p = p0 + j;
       while (p >= next_off) { l++; next_off = a.lane_off[l + 1]; }
-      ln[j] = l;
+      wn[j] = a.lane_window[l];
       if (DIRECT) {
         const int slot = a.lane_slot[l];
         const i64 base = a.slot_base[slot];
@@ -355,52 +299,30 @@ __global__ void __launch_bounds__(JP_THREADS) k_join_launch_stats(JoinArgs a) {
         win[j] = a.found[p];
       }
     }
-    const int l_end = l;
-    int64_t next_end = next_off;
 #pragma unroll
     for (int j = 0; j < 8; j++) {
       if (!(lmask & (1u << j))) continue;
-      const int64_t p = p0 + j;
-      const int l = ln[j];
-      const bool dup = win[j] != (int32_t)p;
+      const bool dup = win[j] != (int32_t)(p0 + j);
       const bool orphan = !dup && nk[j] == 0;
-      if (lm < 0) lm = l;
-      if (l == lm && l - l0 <= 1) {
-        packed += 1ull + ((u64)dup << 20) + ((u64)orphan << 40);
+      if (wm < 0) wm = wn[j];
+      if (wn[j] == wm) {
+        acc[0]++;
+        acc[1] += dup;
+        acc[2] += orphan;
       } else {
-        ta_join_summary *sm = &a.sum[a.lane_window[l]];
-        atomicAdd((u64 *)&sm->n_launch, 1ull);
-        if (dup) atomicAdd((u64 *)&sm->n_dup_launch, 1ull);
-        if (orphan) atomicAdd((u64 *)&sm->n_orphan_launch, 1ull);
+        const u64 one[3] = {1, dup, orphan};
+        launch_emit(&a.sum[wn[j]], one);
       }
     }
     const int64_t plast = min(tile_start + JS_TILE, a.n_valid) - 1;
     if (plast >= p0 && plast < p0 + 8) {
-      int le = l_end;
-      while (plast >= next_end) { le++; next_end = a.lane_off[le + 1]; }
-      s_lane1 = le;
+      while (plast >= next_off) { l++; next_off = a.lane_off[l + 1]; }
+      s_lane1 = l;
     }
   }
   __syncthreads();
-  const int l1 = s_lane1;
-  for (int li = 0; li < 2; li++) {
-    const int l = l0 + li;
-    if (l0 < 0 || l > l1) break;
-    if (a.lane_domain[l] != 0) continue;
-    u64 v = warp_reduce(lm == l ? packed : 0, OpAdd());
-    __syncthreads();
-    if (lane == 0) red[tid >> 5] = v;
-    __syncthreads();
-    if (tid == 0) {
-      u64 t = 0;
-      for (int w = 0; w < JP_THREADS / 32; w++) t += red[w];
-      const u64 m = (1ull << 20) - 1;
-      ta_join_summary *sm = &a.sum[a.lane_window[l]];
-      if (t & m) atomicAdd((u64 *)&sm->n_launch, t & m);
-      if ((t >> 20) & m) atomicAdd((u64 *)&sm->n_dup_launch, (t >> 20) & m);
-      if ((t >> 40) & m) atomicAdd((u64 *)&sm->n_orphan_launch, (t >> 40) & m);
-    }
-  }
+  fold_by_window<3, 0, JP_THREADS / 32>(acc, wm, a.lane_window[l0], a.lane_window[s_lane1], red,
+                                        [&](int w, const u64 *t) { launch_emit(&a.sum[w], t); });
 }
 
 // ---- general path helpers -----------------------------------------------------
