@@ -23,6 +23,10 @@
 #define GP_MINB 4
 #endif
 #define GP_TILE (GP_THREADS * GP_ITEMS)
+// lanes of a tile whose statistics are folded on chip: in a batch of many windows a lane is a
+// thousand records or so and a tile meets several (a batch of 512 windows of 65 k records: 395 us
+// with two lanes folded and the rest by global atomics per record)
+#define GP_LANES 8
 #define GP_LOW ((1ull << 40) - 1)
 
 struct GapArgs {
@@ -55,7 +59,7 @@ __global__ void __launch_bounds__(GP_THREADS, GP_MINB) k_gaps(GapArgs a) {
   __shared__ u64 tmp[33];
   __shared__ u64 red[4][GP_THREADS / 32];
   __shared__ u64 s_excl_max;
-  __shared__ u32 s_hist[2][TA_NBINS];  // the tile's first two lanes; further lanes go straight to global
+  __shared__ u32 s_hist[GP_LANES][TA_NBINS];  // the tile's first lanes; further lanes go straight to global
   __shared__ int s_tile, s_lane0, s_lane1, s_fail;
   const int tid = threadIdx.x;
   if (tid == 0) {
@@ -63,7 +67,7 @@ __global__ void __launch_bounds__(GP_THREADS, GP_MINB) k_gaps(GapArgs a) {
     s_lane1 = -1;
     s_fail = ta_failed(a.status) ? 1 : 0;
   }
-  if (tid < 2 * TA_NBINS) (&s_hist[0][0])[tid] = 0;
+  for (int i = tid; i < GP_LANES * TA_NBINS; i += GP_THREADS) (&s_hist[0][0])[i] = 0;
   __syncthreads();
   if (s_fail) return;
   const int tile = s_tile;
@@ -231,12 +235,12 @@ __global__ void __launch_bounds__(GP_THREADS, GP_MINB) k_gaps(GapArgs a) {
       if (a.list_only) continue;
       if (lm < 0) lm = l;
       const int li = l - l0;
-      if (l == lm && li <= 1) {
+      if (l == lm && li < GP_LANES) {
         sb += (u64)bz;
         si += (u64)(g + tl);
         if (g > 0) { ng++; mg = max(mg, (u64)g); atomicAdd(&s_hist[li][log2_bin(g)], 1u); }
         if (tl > 0) { ng++; mg = max(mg, (u64)tl); atomicAdd(&s_hist[li][log2_bin(tl)], 1u); }
-      } else {  // a thread that straddles a lane boundary, or a third lane in the tile
+      } else {  // a thread that straddles a lane boundary, or a lane too many in the tile
         ta_lane_gaps *gl = &a.lane_gaps[l];
         const int w = a.lane_window[l];
         if (bz) atomicAdd((u64 *)&gl->busy, (u64)bz);
@@ -271,9 +275,9 @@ __global__ void __launch_bounds__(GP_THREADS, GP_MINB) k_gaps(GapArgs a) {
     for (int j = 0; j < GP_ITEMS; j++)
       if (p0 + j < a.n) a.gap_before[p0 + j] = gap[j];
   }
-  // fold the register statistics of the tile's first two lanes
+  // fold the register statistics of the tile's first lanes
   const int l1 = s_lane1;
-  for (int li = 0; li < 2; li++) {
+  for (int li = 0; li < GP_LANES; li++) {
     const int l = l0 + li;
     if (l0 < 0 || l > l1) break;
     if (a.lane_domain[l] != 1) continue;  // uniform over the CTA
