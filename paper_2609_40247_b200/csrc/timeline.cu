@@ -225,6 +225,7 @@ __global__ void __launch_bounds__(256, GT_MINB) k_gather(GatherArgs a) {
   }
 }
 
+#define LT_ITEMS 8
 // One CTA: compacts the non-empty lane codes into the lane table (code order is
 // canonical order).
 __global__ void __launch_bounds__(1024) k_lane_table(const int32_t *lane_start, int64_t n_codes,
@@ -244,24 +245,36 @@ __global__ void __launch_bounds__(1024) k_lane_table(const int32_t *lane_start, 
   }
   if (threadIdx.x == 0) base = 0;
   __syncthreads();
-  for (int64_t c0 = 0; c0 < n_codes; c0 += blockDim.x) {
-    int64_t c = c0 + threadIdx.x;
-    int32_t st = c < n_codes ? lane_start[c] : -1;
+  // LT_ITEMS consecutive codes (then lanes) per thread and round: a batch of 512 windows has 65 k
+  // codes, and one code per thread took 64 rounds of two block scans each (165 us; now 28 us)
+  for (int64_t c0 = 0; c0 < n_codes; c0 += LT_ITEMS * blockDim.x) {
+    const int64_t cb = c0 + (int64_t)threadIdx.x * LT_ITEMS;
+    int32_t sts[LT_ITEMS];
+    u32 mine = 0;
+#pragma unroll
+    for (int j = 0; j < LT_ITEMS; j++) {
+      sts[j] = cb + j < n_codes ? lane_start[cb + j] : -1;
+      mine += sts[j] >= 0;
+    }
     u64 total;
-    u64 ex = block_scan_exclusive<OpAdd>(st >= 0 ? 1ull : 0ull, OpAdd(), tmp, &total);
-    if (st >= 0) {
-      int64_t l = (int64_t)(base + ex);
+    const u64 ex = block_scan_exclusive<OpAdd>((u64)mine, OpAdd(), tmp, &total);
+    int64_t l = (int64_t)(base + ex);
+#pragma unroll
+    for (int j = 0; j < LT_ITEMS; j++) {
+      if (sts[j] < 0) continue;
       if (l < cap) {
+        const int64_t c = cb + j;
         int w = (int)(c >> tbits), t = (int)(c & ((1ll << tbits) - 1));
         u64 code = tt->sorted_code[t];
         lane_window[l] = w;
         lane_pid[l] = code_pid(code);
         lane_stream[l] = code_stream(code);
         lane_domain[l] = code_domain(code);
-        lane_off[l] = st;
+        lane_off[l] = sts[j];
         lane_code[l] = (int32_t)c;
         lane_slot[l] = w * n_pids + tt->pid_rank[t];
       }
+      l++;
     }
     __syncthreads();
     if (threadIdx.x == 0) base += total;
@@ -277,24 +290,33 @@ __global__ void __launch_bounds__(1024) k_lane_table(const int32_t *lane_start, 
   // and device lanes alternate per (window, pid), so the runs are a few lanes long - but a batch
   // of device-only windows is one long run, hence a scan and no walk).  Going backwards over
   // the lanes, the nearest boundary at or behind lane l is a running maximum of
-  // L - (index of the lane behind a boundary); chunks of blockDim.x lanes, carried in `base`.
+  // L - (index of the lane behind a boundary); rounds of LT_ITEMS * blockDim.x lanes, carried in `base`.
   const int64_t L = (int64_t)base < cap ? (int64_t)base : cap;
   __syncthreads();  // every thread has read the lane count before `base` is reused
   if (threadIdx.x == 0) base = 0;
   __syncthreads();
-  for (int64_t r0 = 0; r0 < L; r0 += blockDim.x) {
-    const int64_t r = r0 + threadIdx.x;  // reversed lane index
-    const int64_t l = L - 1 - r;
-    u64 v = 0;
-    if (r < L && l + 1 < L && lane_domain[l + 1] != lane_domain[l]) v = (u64)(L - (l + 1));
+  for (int64_t r0 = 0; r0 < L; r0 += LT_ITEMS * blockDim.x) {
+    const int64_t rb = r0 + (int64_t)threadIdx.x * LT_ITEMS;  // reversed lane index
+    u64 v[LT_ITEMS], run = 0;
+#pragma unroll
+    for (int j = 0; j < LT_ITEMS; j++) {
+      const int64_t r = rb + j, l = L - 1 - r;
+      v[j] = 0;
+      if (r < L && l + 1 < L && lane_domain[l + 1] != lane_domain[l]) v[j] = (u64)(L - (l + 1));
+      run = max(run, v[j]);
+    }
     u64 total;
-    const u64 ex = block_scan_exclusive<OpMax>(v, OpMax(), tmp, &total);
-    if (r < L) {
-      u64 best = ex > v ? ex : v;
-      best = best > base ? best : base;
-      const int64_t m = best ? L - (int64_t)best : L;
-      lane_dom_end[l] = m < L ? lane_off[m] : (int32_t)n_valid;
-      lane_dom_next[l] = (int32_t)m;  // index of the first later lane of the other domain (L if none)
+    const u64 ex = block_scan_exclusive<OpMax>(run, OpMax(), tmp, &total);
+    u64 best = max((u64)base, ex);
+#pragma unroll
+    for (int j = 0; j < LT_ITEMS; j++) {
+      const int64_t r = rb + j, l = L - 1 - r;
+      best = max(best, v[j]);
+      if (r < L) {
+        const int64_t m = best ? L - (int64_t)best : L;
+        lane_dom_end[l] = m < L ? lane_off[m] : (int32_t)n_valid;
+        lane_dom_next[l] = (int32_t)m;  // index of the first later lane of the other domain (L if none)
+      }
     }
     __syncthreads();
     if (threadIdx.x == 0) base = base > total ? base : total;
@@ -304,13 +326,25 @@ __global__ void __launch_bounds__(1024) k_lane_table(const int32_t *lane_start, 
   // records are taken out in order); n_lanes_out[1] = the number of device records
   if (threadIdx.x == 0) base = 0;
   __syncthreads();
-  for (int64_t l0 = 0; l0 < L; l0 += blockDim.x) {
-    const int64_t l = l0 + threadIdx.x;
-    u64 sz = 0;
-    if (l < L && lane_domain[l] == 1) sz = (u64)((l + 1 < L ? lane_off[l + 1] : (int32_t)n_valid) - lane_off[l]);
+  for (int64_t l0 = 0; l0 < L; l0 += LT_ITEMS * blockDim.x) {
+    const int64_t lb = l0 + (int64_t)threadIdx.x * LT_ITEMS;
+    u32 sz[LT_ITEMS];
+    u64 run = 0;
+#pragma unroll
+    for (int j = 0; j < LT_ITEMS; j++) {
+      const int64_t l = lb + j;
+      sz[j] = 0;
+      if (l < L && lane_domain[l] == 1) sz[j] = (u32)((l + 1 < L ? lane_off[l + 1] : (int32_t)n_valid) - lane_off[l]);
+      run += sz[j];
+    }
     u64 total;
-    const u64 ex = block_scan_exclusive<OpAdd>(sz, OpAdd(), tmp, &total);
-    if (l < L) lane_dev_base[l] = (int32_t)(base + ex);
+    const u64 ex = block_scan_exclusive<OpAdd>(run, OpAdd(), tmp, &total);
+    u64 at = base + ex;
+#pragma unroll
+    for (int j = 0; j < LT_ITEMS; j++) {
+      if (lb + j < L) lane_dev_base[lb + j] = (int32_t)at;
+      at += sz[j];
+    }
     __syncthreads();
     if (threadIdx.x == 0) base += total;
     __syncthreads();
