@@ -4,13 +4,20 @@
 // Per-symbol counts and duration statistics are what Sec. 8.1 compares.
 //
 // Symbol popularity is heavy-tailed (a few names carry most records), so global
-// atomics alone would serialise on the hot rows.  Each CTA takes 16384
+// atomics alone would serialise on the hot rows.  Each CTA takes up to 16384
 // consecutive sorted positions (one process, mostly; CTAs whose lanes cannot
 // hold a selected kind return at once) and folds its records into a
-// shared-memory hash table first; the table is flushed to a dense global table
-// indexed by (window, pid rank, name_id - min name) with one atomic per field.
-// A scan then compacts the non-empty rows in key order.  Symbol ids spread too wide
-// for a dense table take the sort-based path at the end of this file instead.
+// shared-memory hash table first, which is flushed to global rows with one atomic
+// per field.  A cell = (window, pid rank, symbol rank); three ways to give cells rows:
+//   dense   few cells: one row per cell, a scan compacts the non-empty ones in key order;
+//   marked  many cells (a batch of windows), few of them occupied: a first pass over kinds
+//           and symbols sets one bit per occupied cell, a scan over the words of the bitmap
+//           numbers the occupied cells in key order, and the records are folded straight
+//           into the result rows;
+//   sorted  more distinct symbols than the symbol table holds, or more cells than a bitmap:
+//           group by sorting, at the end of this file.
+// Symbol rank = name_id - min name when the ids are close together; symbol ids spread wide
+// (hashes) are ranked through a table of the distinct ones, built once per window.
 // HBM-bound on the column reads: 2 B (kind) for every record, 24 B more for the
 // selected ones.
 #include <climits>
@@ -47,12 +54,90 @@ struct AggArgs {
   int want_domain;  // 0 / 1: the selected kinds all live in lanes of this domain; -1: both
   int64_t chunk;    // positions per CTA, a multiple of AG_STEP
   unsigned n_items, spread, per;
-  // dense table (all zero-initialised; min is kept as the complement of the biased value)
+  const u64 *names;        // symbol table when the ids are spread wide, else null
+  const u32 *name_rank;
+  // rows (all zero-initialised; min is kept as the complement of the biased value)
   u64 *d_cnt, *d_sum, *d_minc, *d_maxb;
   u32 *d_hist;
-  u64 *n_groups;
-  const int32_t *status;
+  // marked cells: row of cell g = rank[g / 32] + set bits of bits[g / 32] below g; null: row = cell
+  u32 *bits;
+  const u32 *rank;
+  int32_t *status;
 };
+
+// ---- symbol table: the distinct symbol ids of the window, open addressing ------------------
+#define NT_SLOTS (1u << 18)
+#define NT_MAX (1u << 17)
+#define NT_PROBES 512
+#define NT_EMPTY 0ull  // entries are biased ids + 1
+__device__ __forceinline__ u32 name_hash(u32 b) {
+  u32 h = b * 0x9E3779B1u;
+  h ^= h >> 15;
+  h *= 0x2C1B3C6Du;
+  return (h ^ (h >> 13)) & (NT_SLOTS - 1);
+}
+__global__ void __launch_bounds__(256) k_name_set(const int32_t *name, int64_t n_valid, u64 *names, u64 *n_names,
+                                                  u64 *list, int32_t *status) {
+  __shared__ u64 cache[2048];  // ids this CTA has seen already (direct mapped, one word each)
+  if (ta_failed(status)) return;
+  for (int i = threadIdx.x; i < 2048; i += 256) cache[i] = NT_EMPTY;
+  __syncthreads();
+  for (int64_t p0 = ((int64_t)blockIdx.x * 256 + threadIdx.x) * 4; p0 < n_valid; p0 += (int64_t)gridDim.x * 1024) {
+    int32_t nm[4];
+    const int cnt = (int)min((int64_t)4, n_valid - p0);
+    if (cnt == 4) {
+      const int4 q = *reinterpret_cast<const int4 *>(name + p0);
+      nm[0] = q.x; nm[1] = q.y; nm[2] = q.z; nm[3] = q.w;
+    } else {
+      for (int j = 0; j < 4; j++) nm[j] = j < cnt ? name[p0 + j] : 0;
+    }
+#pragma unroll
+    for (int j = 0; j < 4; j++) {
+      if (j >= cnt) break;
+      const u64 e = (u64)((u32)nm[j] ^ 0x80000000u) + 1;
+      u32 slot = name_hash((u32)(e - 1));
+      if (cache[slot & 2047] == e) continue;
+      cache[slot & 2047] = e;
+      for (u32 probe = 0;; probe++) {
+        u64 cur = ld_relaxed(&names[slot]);
+        if (cur == NT_EMPTY || probe == NT_PROBES) {
+          // too many symbols (a table half full has no run of NT_PROBES): the caller groups by sorting
+          if (probe == NT_PROBES) atomicAdd(n_names, (u64)NT_MAX + 1);
+          if (ld_relaxed(n_names) > NT_MAX) return;
+          cur = atomicCAS(&names[slot], NT_EMPTY, e);
+          if (cur == NT_EMPTY) {
+            const u64 at = atomicAdd(n_names, 1ull);
+            if (at < NT_MAX) list[at] = (e - 1) << 32 | slot;
+            break;
+          }
+        }
+        if (cur == e) break;
+        slot = (slot + 1) & (NT_SLOTS - 1);
+      }
+    }
+  }
+}
+__global__ void __launch_bounds__(256) k_name_rank(const u64 *sorted, int64_t D, u32 *name_rank, int32_t *name_of,
+                                                   const int32_t *status) {
+  if (ta_failed(status)) return;
+  const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
+  if (i >= D) return;
+  const u64 x = sorted[i];
+  name_rank[(u32)x & (NT_SLOTS - 1)] = (u32)i;
+  name_of[i] = (int32_t)((u32)(x >> 32) ^ 0x80000000u);
+}
+__device__ __forceinline__ int64_t name_rank_of(const AggArgs &a, int32_t nm) {
+  if (!a.names) return (int64_t)nm - a.min_name;
+  const u64 e = (u64)((u32)nm ^ 0x80000000u) + 1;
+  u32 slot = name_hash((u32)(e - 1));
+  // every id of the window is in the table: a bounded probe all the same
+  for (u32 probe = 0; probe < NT_SLOTS && a.names[slot] != e; probe++) slot = (slot + 1) & (NT_SLOTS - 1);
+  return (int64_t)a.name_rank[slot];
+}
+__device__ __forceinline__ int64_t row_of(const AggArgs &a, int64_t g) {
+  if (!a.rank) return g;
+  return (int64_t)a.rank[g >> 5] + __popc(a.bits[g >> 5] & ((1u << (g & 31)) - 1u));
+}
 
 struct AggSmem {
   int32_t key[AG_SLOTS];
@@ -88,11 +173,15 @@ __device__ __forceinline__ void agg_flush(const AggArgs &a, AggSmem &s) {
   __syncthreads();
   for (int i = threadIdx.x; i < AG_SLOTS; i += AG_THREADS) {
     int32_t k = s.key[i];
-    if (k >= 0)
+    if (k >= 0) {
+      k = (int32_t)row_of(a, k);
+      s.key[i] = k;  // the row, for the bins below
       agg_global_add(a, k, s.cnt[i],
                      (u64)s.sum16[0][i] + ((u64)s.sum16[1][i] << 16) + ((u64)s.sum16[2][i] << 32),
                      s.minc[i], s.maxb[i]);
+    }
   }
+  __syncthreads();
   // histogram bins: one thread per (slot, bin)
   for (int i = threadIdx.x; i < AG_SLOTS * TA_NBINS; i += AG_THREADS) {
     const int sl = i / TA_NBINS, b = i - sl * TA_NBINS;
@@ -102,6 +191,108 @@ __device__ __forceinline__ void agg_flush(const AggArgs &a, AggSmem &s) {
   __syncthreads();
   agg_clear(s);
   __syncthreads();
+}
+
+// Which of the thread's four records are selected, their values and symbols (a caller that makes no
+// use of the values pays for no load of them).
+__device__ __forceinline__ void agg_select(const AggArgs &a, int64_t p0, int64_t end, bool (&sel)[AG_ITEMS],
+                                           i64 (&v)[AG_ITEMS], int32_t (&nm)[AG_ITEMS]) {
+  // all loads of the thread's four records are issued before any of them is used; for the
+  // plain duration the times and names are requested with the kinds, not after them (the
+  // step holds lanes of the wanted domain, so most records are selected anyway)
+  int16_t kd[AG_ITEMS];
+  i64 pre_v[AG_ITEMS];
+  int32_t pre_nm[AG_ITEMS];
+#pragma unroll
+  for (int j = 0; j < AG_ITEMS; j++) { pre_v[j] = 0; pre_nm[j] = 0; }
+  if (p0 + AG_ITEMS <= end) {
+    uint2 q = *reinterpret_cast<const uint2 *>(a.kind + p0);
+    if (a.value_sel == 0) {
+      const longlong2 *ps = reinterpret_cast<const longlong2 *>(a.ts + p0);
+      const longlong2 *pe = reinterpret_cast<const longlong2 *>(a.te + p0);
+      const int4 nq = *reinterpret_cast<const int4 *>(a.name + p0);
+#pragma unroll
+      for (int h2 = 0; h2 < AG_ITEMS / 2; h2++) {
+        const longlong2 x = ps[h2], y = pe[h2];
+        pre_v[2 * h2] = y.x - x.x;
+        pre_v[2 * h2 + 1] = y.y - x.y;
+      }
+      pre_nm[0] = nq.x; pre_nm[1] = nq.y; pre_nm[2] = nq.z; pre_nm[3] = nq.w;
+    } else if (a.value_sel == 1) {  // the kernel counts with the kinds (pre_nm holds them)
+      const int4 cq = *reinterpret_cast<const int4 *>(a.op_n + p0);
+      pre_nm[0] = cq.x; pre_nm[1] = cq.y; pre_nm[2] = cq.z; pre_nm[3] = cq.w;
+    }
+    const int16_t *hq = reinterpret_cast<const int16_t *>(&q);
+#pragma unroll
+    for (int j = 0; j < AG_ITEMS; j++) kd[j] = hq[j];
+  } else {
+#pragma unroll
+    for (int j = 0; j < AG_ITEMS; j++) {
+      kd[j] = p0 + j < end ? a.kind[p0 + j] : (int16_t)-1;
+      if (a.value_sel == 0 && p0 + j < end) { pre_v[j] = a.te[p0 + j] - a.ts[p0 + j]; pre_nm[j] = a.name[p0 + j]; }
+      if (a.value_sel == 1 && p0 + j < end) pre_nm[j] = a.op_n[p0 + j];
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < AG_ITEMS; j++) {
+    sel[j] = kd[j] >= 0 && ((a.kind_mask >> kd[j]) & 1u);
+    v[j] = 0;
+    nm[j] = 0;
+  }
+  if (a.value_sel == 0) {
+#pragma unroll
+    for (int j = 0; j < AG_ITEMS; j++)
+      if (sel[j]) { v[j] = pre_v[j]; nm[j] = pre_nm[j]; }
+  } else if (a.value_sel == 1) {
+#pragma unroll
+    for (int j = 0; j < AG_ITEMS; j++)
+      if (sel[j]) sel[j] = pre_nm[j] > 0;
+#pragma unroll
+    for (int j = 0; j < AG_ITEMS; j++)
+      if (sel[j]) { v[j] = a.op_last[p0 + j] - a.op_first[p0 + j]; nm[j] = a.name[p0 + j]; }
+  } else if (a.value_sel == 2) {
+#pragma unroll
+    for (int j = 0; j < AG_ITEMS; j++)
+      if (sel[j]) { v[j] = a.op_gap[p0 + j]; sel[j] = v[j] > 0; }
+#pragma unroll
+    for (int j = 0; j < AG_ITEMS; j++)
+      if (sel[j]) nm[j] = a.name[p0 + j];
+  } else {
+#pragma unroll
+    for (int j = 0; j < AG_ITEMS; j++)
+      if (sel[j]) sel[j] = a.on_path[p0 + j] != 0;
+#pragma unroll
+    for (int j = 0; j < AG_ITEMS; j++)
+      if (sel[j]) { v[j] = a.te[p0 + j] - a.ts[p0 + j]; nm[j] = a.name[p0 + j]; }
+  }
+}
+
+// sets the bit of every cell that holds a selected record
+__global__ void __launch_bounds__(AG_THREADS) k_agg_mark(AggArgs a) {
+  if (ta_failed(a.status)) return;
+  LaneWalker lw(a.lane_off, a.n_lanes, a.n_valid, a.n_valid);
+  const int64_t begin = (int64_t)blockIdx.x * a.chunk, end = min(begin + a.chunk, a.n_valid);
+  if (begin >= end) return;
+  int bl = lane_of_pos(a.lane_off, a.n_lanes, begin);
+  for (int64_t base = begin; base < end; base += AG_STEP) {
+    while (bl + 1 < a.n_lanes && (int64_t)a.lane_off[bl + 1] <= base) bl++;
+    if (a.want_domain >= 0 &&
+        span_outside_domain(a.lane_domain, a.lane_dom_end, bl, min(base + AG_STEP, end), a.want_domain))
+      continue;
+    lw.lane = bl;
+    const int64_t p0 = base + (int64_t)threadIdx.x * AG_ITEMS;
+    bool sel[AG_ITEMS];
+    i64 v[AG_ITEMS];
+    int32_t nm[AG_ITEMS];
+    agg_select(a, p0, end, sel, v, nm);
+#pragma unroll
+    for (int j = 0; j < AG_ITEMS; j++) {
+      if (!sel[j]) continue;
+      const int64_t g = (int64_t)a.lane_slot[lw.at(p0 + j)] * a.R + name_rank_of(a, nm[j]);
+      // a stale word only costs a second atomic: popular cells are set once and then read from L1
+      if (!((a.bits[g >> 5] >> (g & 31)) & 1u)) atomicOr(&a.bits[g >> 5], 1u << (g & 31));
+    }
+  }
 }
 
 __global__ void __launch_bounds__(AG_THREADS, 6) k_agg(AggArgs a) {
@@ -130,82 +321,15 @@ __global__ void __launch_bounds__(AG_THREADS, 6) k_agg(AggArgs a) {
         continue;
       lw.lane = bl;
       const int64_t p0 = base + (int64_t)threadIdx.x * AG_ITEMS;
-      // all loads of the thread's four records are issued before any of them is used; for the
-      // plain duration the times and names are requested with the kinds, not after them (the
-      // step holds lanes of the wanted domain, so most records are selected anyway)
-      int16_t kd[AG_ITEMS];
-      i64 pre_v[AG_ITEMS];
-      int32_t pre_nm[AG_ITEMS];
-#pragma unroll
-      for (int j = 0; j < AG_ITEMS; j++) { pre_v[j] = 0; pre_nm[j] = 0; }
-      if (p0 + AG_ITEMS <= end) {
-        uint2 q = *reinterpret_cast<const uint2 *>(a.kind + p0);
-        if (a.value_sel == 0) {
-          const longlong2 *ps = reinterpret_cast<const longlong2 *>(a.ts + p0);
-          const longlong2 *pe = reinterpret_cast<const longlong2 *>(a.te + p0);
-          const int4 nq = *reinterpret_cast<const int4 *>(a.name + p0);
-#pragma unroll
-          for (int h2 = 0; h2 < AG_ITEMS / 2; h2++) {
-            const longlong2 x = ps[h2], y = pe[h2];
-            pre_v[2 * h2] = y.x - x.x;
-            pre_v[2 * h2 + 1] = y.y - x.y;
-          }
-          pre_nm[0] = nq.x; pre_nm[1] = nq.y; pre_nm[2] = nq.z; pre_nm[3] = nq.w;
-        } else if (a.value_sel == 1) {  // the kernel counts with the kinds (pre_nm holds them)
-          const int4 cq = *reinterpret_cast<const int4 *>(a.op_n + p0);
-          pre_nm[0] = cq.x; pre_nm[1] = cq.y; pre_nm[2] = cq.z; pre_nm[3] = cq.w;
-        }
-        const int16_t *hq = reinterpret_cast<const int16_t *>(&q);
-#pragma unroll
-        for (int j = 0; j < AG_ITEMS; j++) kd[j] = hq[j];
-      } else {
-#pragma unroll
-        for (int j = 0; j < AG_ITEMS; j++) {
-          kd[j] = p0 + j < end ? a.kind[p0 + j] : (int16_t)-1;
-          if (a.value_sel == 0 && p0 + j < end) { pre_v[j] = a.te[p0 + j] - a.ts[p0 + j]; pre_nm[j] = a.name[p0 + j]; }
-          if (a.value_sel == 1 && p0 + j < end) pre_nm[j] = a.op_n[p0 + j];
-        }
-      }
       bool sel[AG_ITEMS];
       i64 v[AG_ITEMS];
       int32_t nm[AG_ITEMS];
-#pragma unroll
-      for (int j = 0; j < AG_ITEMS; j++) {
-        sel[j] = kd[j] >= 0 && ((a.kind_mask >> kd[j]) & 1u);
-        v[j] = 0;
-        nm[j] = 0;
-      }
-      if (a.value_sel == 0) {
-#pragma unroll
-        for (int j = 0; j < AG_ITEMS; j++)
-          if (sel[j]) { v[j] = pre_v[j]; nm[j] = pre_nm[j]; }
-      } else if (a.value_sel == 1) {
-#pragma unroll
-        for (int j = 0; j < AG_ITEMS; j++)
-          if (sel[j]) sel[j] = pre_nm[j] > 0;
-#pragma unroll
-        for (int j = 0; j < AG_ITEMS; j++)
-          if (sel[j]) { v[j] = a.op_last[p0 + j] - a.op_first[p0 + j]; nm[j] = a.name[p0 + j]; }
-      } else if (a.value_sel == 2) {
-#pragma unroll
-        for (int j = 0; j < AG_ITEMS; j++)
-          if (sel[j]) { v[j] = a.op_gap[p0 + j]; sel[j] = v[j] > 0; }
-#pragma unroll
-        for (int j = 0; j < AG_ITEMS; j++)
-          if (sel[j]) nm[j] = a.name[p0 + j];
-      } else {
-#pragma unroll
-        for (int j = 0; j < AG_ITEMS; j++)
-          if (sel[j]) sel[j] = a.on_path[p0 + j] != 0;
-#pragma unroll
-        for (int j = 0; j < AG_ITEMS; j++)
-          if (sel[j]) { v[j] = a.te[p0 + j] - a.ts[p0 + j]; nm[j] = a.name[p0 + j]; }
-      }
+      agg_select(a, p0, end, sel, v, nm);
 #pragma unroll
       for (int j = 0; j < AG_ITEMS; j++) {
         if (!sel[j]) continue;
         const int lane = lw.at(p0 + j);
-        const int64_t g = (int64_t)a.lane_slot[lane] * a.R + ((int64_t)nm[j] - a.min_name);
+        const int64_t g = (int64_t)a.lane_slot[lane] * a.R + name_rank_of(a, nm[j]);
         const u64 vb = (u64)v[j] ^ (1ull << 63);
         const int bin = log2_bin(v[j]);
         u32 hsh = (u32)g * 2654435761u;
@@ -236,8 +360,9 @@ __global__ void __launch_bounds__(AG_THREADS, 6) k_agg(AggArgs a) {
           u32 *hw = reinterpret_cast<u32 *>(&s.hist[slot][0]) + (bin >> 1);
           atomicAdd(hw, (bin & 1) ? 0x10000u : 1u);
         } else {
-          agg_global_add(a, g, 1, (u64)v[j], ~vb, vb);
-          atomicAdd(&a.d_hist[(size_t)g * TA_NBINS + bin], 1u);
+          const int64_t row = row_of(a, g);
+          agg_global_add(a, row, 1, (u64)v[j], ~vb, vb);
+          atomicAdd(&a.d_hist[(size_t)row * TA_NBINS + bin], 1u);
         }
       }
       since_flush += AG_STEP;
@@ -248,15 +373,6 @@ __global__ void __launch_bounds__(AG_THREADS, 6) k_agg(AggArgs a) {
     }
   }
   agg_flush(a, s);
-}
-
-// number of non-empty rows (only needed up front when the output cannot be sized by a bound)
-__global__ void __launch_bounds__(256) k_agg_count_rows(const u64 *cnt, int64_t G, u64 *n_rows) {
-  u64 c = 0;
-  for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < G; g += (int64_t)gridDim.x * blockDim.x)
-    c += cnt[g] ? 1ull : 0ull;
-  c = warp_reduce(c, OpAdd());
-  if ((threadIdx.x & 31) == 0 && c) atomicAdd(n_rows, c);
 }
 
 // compaction of the non-empty rows in dense (= key) order
@@ -270,6 +386,7 @@ struct AggRowOut {
   const TripleTable *tt;
   int n_pids;
   int64_t R, min_name;
+  const int32_t *name_of;  // symbol of a rank, null: rank + min_name
   int32_t *g_window, *g_pid, *g_name;
   int64_t *g_count, *g_sum, *g_min, *g_max;
   u32 *g_hist;
@@ -278,7 +395,7 @@ struct AggRowOut {
     int64_t slot = g / R;
     g_window[row] = (int32_t)(slot / n_pids);
     g_pid[row] = tt->pid_value[slot % n_pids];
-    g_name[row] = (int32_t)(min_name + g % R);
+    g_name[row] = name_of ? name_of[g % R] : (int32_t)(min_name + g % R);
     g_count[row] = (int64_t)cnt[g];
     g_sum[row] = (int64_t)sum[g];
     g_min[row] = (int64_t)((~minc[g]) ^ (1ull << 63));
@@ -295,7 +412,36 @@ struct AggRowOut {
   }
 };
 
-// ---- symbol ids too spread out for the dense table: aggregate by sorting ---------------
+// ---- marked cells: numbering, and what is left to write of a row -----------------------------
+struct AggBitsIn {
+  const u32 *bits;
+  __device__ u64 operator()(int64_t i) const { return (u64)__popc(bits[i]); }
+};
+struct AggBitsOut {
+  u32 *rank;
+  __device__ void operator()(int64_t i, u64 excl, u64) const { rank[i] = (u32)excl; }
+};
+// one thread per word of the bitmap: key and extremes of its rows (the extremes were accumulated
+// in order-preserving codes with 0 as "nothing yet")
+__global__ void __launch_bounds__(256) k_agg_marked_rows(const u32 *bits, const u32 *rank, int64_t words,
+                                                         AggRowOut o, const int32_t *status) {
+  if (ta_failed(status)) return;
+  const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
+  if (i >= words) return;
+  u32 m = bits[i];
+  if (!m) return;
+  for (u32 row = rank[i]; m; row++, m &= m - 1) {
+    const int64_t g = i * 32 + (__ffs((int)m) - 1);
+    const int64_t slot = g / o.R, r = g - slot * o.R;
+    o.g_window[row] = (int32_t)(slot / o.n_pids);
+    o.g_pid[row] = o.tt->pid_value[slot % o.n_pids];
+    o.g_name[row] = o.name_of ? o.name_of[r] : (int32_t)(o.min_name + r);
+    o.g_min[row] = (int64_t)((~(u64)o.g_min[row]) ^ (1ull << 63));
+    o.g_max[row] = (int64_t)((u64)o.g_max[row] ^ (1ull << 63));
+  }
+}
+
+// ---- too many symbols or cells: aggregate by sorting ---------------
 // The selected records are compacted to (key, position) pairs with key = (window, pid) slot
 // << 32 | name_id (order-preserving code), sorted with the pair sorter, cut into groups where
 // the key changes, and reduced with atomics on the group rows - one per run of equal keys
@@ -501,38 +647,74 @@ static ta_status ta_run_aggregate_sorted(ta_window *h, uint32_t kind_mask, int v
   return TA_OK;
 }
 
+// Builds the symbol table of the window (once per handle); h->n_names = number of distinct ids, or
+// -1 if there are more than NT_MAX.
+static ta_status build_names(ta_window *h) {
+  if (h->n_names) return TA_OK;
+  cudaStream_t st = h->stream;
+  void *tmp = ta_dalloc(h, Carver::pad((size_t)NT_MAX * 8));
+  const size_t keep = Carver::pad((size_t)NT_SLOTS * 8) + Carver::pad(64) + Carver::pad((size_t)NT_SLOTS * 4) +
+                      Carver::pad((size_t)NT_MAX * 4);
+  void *kb = ta_dalloc(h, keep);
+  if (!tmp || !kb) return TA_ERR_OOM;
+  u64 *list = (u64 *)tmp;
+  Carver ck(kb);
+  h->d_names = ck.take<u64>(NT_SLOTS);
+  u64 *count = ck.take<u64>(8);
+  TA_CHECK_CUDA(h, cudaMemsetAsync(kb, 0, ck.off, st));
+  h->d_name_rank = ck.take<u32>(NT_SLOTS);
+  h->d_name_of = ck.take<int32_t>(NT_MAX);
+  const int64_t want = (h->n_valid + 1023) / 1024;
+  k_name_set<<<TA_N (unsigned)(want < 148 * 8 ? want : 148 * 8), 256, 0, st>>>(h->sorted.name_id, h->n_valid,
+                                                                               h->d_names, count, list, h->d_status);
+  TA_CHECK_CUDA(h, cudaGetLastError());
+  u64 D = 0;
+  TA_TRY(ta_queue_d2h(h, &D, count, 8));
+  TA_TRY(ta_sync_fetch(h));
+  if (D == 0 || D > NT_MAX) {  // (0: an earlier kernel failed; the caller's status check reports it)
+    h->n_names = -1;
+  } else {
+    void *sb = ta_dalloc(h, 2 * Carver::pad(D * 8) + ta_sort_temp_bytes((int64_t)D) + 256);
+    if (!sb) return TA_ERR_OOM;
+    Carver cs(sb);
+    u64 *scr = cs.take<u64>(D), *sorted = cs.take<u64>(D);
+    TA_TRY(ta_radix_sort_keys(h, list, scr, sorted, (int64_t)D, ta_make_plan(32, 64), nullptr, cs.base + cs.off, false));
+    k_name_rank<<<TA_N (unsigned)((D + 255) / 256), 256, 0, st>>>(sorted, (int64_t)D, h->d_name_rank, h->d_name_of,
+                                                                  h->d_status);
+    TA_CHECK_CUDA(h, cudaGetLastError());
+    h->n_names = (int64_t)D;
+    ta_dfree_later(h, sb);
+  }
+  ta_dfree_later(h, tmp);
+  return TA_OK;
+}
+
 ta_status ta_run_aggregate(ta_window *h, uint32_t kind_mask, int value_sel, ta_agg_result *out) {
   cudaStream_t st = h->stream;
   const int n_pids = h->n_pids > 0 ? h->n_pids : 1;
   memset(out, 0, sizeof(*out));
   if (h->n_valid == 0 || (kind_mask & 63u) == 0) return TA_OK;
-  const unsigned __int128 R128 = (unsigned __int128)((uint64_t)h->max_name - (uint64_t)h->min_name) + 1;
-  const unsigned __int128 G128 = R128 * (unsigned __int128)((uint64_t)h->W * (uint64_t)n_pids);
-  if (G128 > (unsigned __int128)TA_AGG_DENSE_LIMIT) return ta_run_aggregate_sorted(h, kind_mask, value_sel, out);
-  const int64_t R = (int64_t)R128, G = (int64_t)G128;
+  const int64_t n_slots = (int64_t)h->W * n_pids;
+  int64_t R = h->max_name - h->min_name + 1;  // names are 32-bit: no overflow
+  // Ids spread wide (R x slots cells would not fit the dense table): ranks through the symbol table.
+  const bool table = R > TA_AGG_DENSE_LIMIT / n_slots;
+  if (table) {
+    TA_TRY(build_names(h));
+    if (h->n_names < 0 || h->n_names > TA_AGG_MARK_LIMIT / n_slots)
+      return ta_run_aggregate_sorted(h, kind_mask, value_sel, out);
+    R = h->n_names;
+  }
+  const int64_t G = R * n_slots;
 
-  size_t tb = 4 * Carver::pad((size_t)G * 8) + Carver::pad((size_t)G * TA_NBINS * 4) + Carver::pad(64) +
-              scan_temp_bytes(G) + 256;
-  void *tmpb = ta_dalloc(h, tb);
-  if (!tmpb) return TA_ERR_OOM;
-  Carver ct(tmpb);
   AggArgs a;
   memset(&a, 0, sizeof(a));
-  a.d_cnt = ct.take<u64>(G);
-  a.d_sum = ct.take<u64>(G);
-  a.d_minc = ct.take<u64>(G);
-  a.d_maxb = ct.take<u64>(G);
-  a.d_hist = ct.take<u32>((size_t)G * TA_NBINS);
-  a.n_groups = ct.take<u64>(8);
-  TA_CHECK_CUDA(h, cudaMemsetAsync(tmpb, 0, ct.off, st));
-  void *scan_mem = ct.base + ct.off;
-
   a.n_valid = h->n_valid; a.n_lanes = h->sorted.n_lanes;
   a.kind = h->sorted.kind; a.name = h->sorted.name_id; a.ts = h->sorted.ts_start; a.te = h->sorted.ts_end;
   a.lane_off = h->sorted.lane_off; a.lane_slot = h->d_lane_slot;
   a.op_n = h->attr.op_n_kernels; a.op_first = h->attr.op_first_start; a.op_last = h->attr.op_last_end;
   a.op_gap = h->d_op_gap_ns; a.on_path = h->d_on_path;
   a.kind_mask = kind_mask & 63u; a.value_sel = value_sel; a.min_name = h->min_name; a.R = R;
+  a.names = table ? h->d_names : nullptr; a.name_rank = h->d_name_rank;
   a.lane_domain = h->sorted.lane_domain; a.lane_dom_end = h->d_lane_dom_end; a.status = h->d_status;
   const bool host_kinds = (a.kind_mask & 7u) != 0, dev_kinds = (a.kind_mask & 56u) != 0;
   a.want_domain = host_kinds && dev_kinds ? -1 : (dev_kinds ? 1 : 0);
@@ -545,48 +727,88 @@ ta_status ta_run_aggregate(ta_window *h, uint32_t kind_mask, int value_sel, ta_a
   a.spread = a.n_items < 148u * 6u ? a.n_items : 148u * 6u;
   a.per = (a.n_items + a.spread - 1) / a.spread;
   const int64_t blocks = (int64_t)a.spread * a.per;
-  k_agg<<<TA_N (unsigned)blocks, AG_THREADS, 0, st>>>(a);
-  TA_CHECK_CUDA(h, cudaGetLastError());
-  // Rows are compacted without waiting for their count when a bound on it (dense rows, selected
-  // records) keeps the output small; otherwise the count is fetched first.
+
+  AggRowOut ro;
+  memset(&ro, 0, sizeof(ro));
+  ro.tt = h->d_triples; ro.n_pids = n_pids; ro.R = R; ro.min_name = h->min_name;
+  ro.name_of = table ? h->d_name_of : nullptr;
   u64 ng = 0;
-  u64 cap = (u64)G < (u64)h->n_valid ? (u64)G : (u64)h->n_valid;
-  const bool bounded = cap * (28 + 32 + TA_NBINS * 4) <= (256ull << 20);
-  if (!bounded) {
-    const int64_t want = (G + 255) / 256;
-    k_agg_count_rows<<<TA_N (unsigned)(want < 148 * 8 ? want : 148 * 8), 256, 0, st>>>(a.d_cnt, G, a.n_groups);
-    TA_TRY(ta_queue_d2h(h, &ng, a.n_groups, 8));
-    TA_TRY(ta_sync_fetch(h));
-    cap = ng;
-  }
-  u64 *scan_total = nullptr;
-  if (cap > 0) {
-    size_t ob = 3 * Carver::pad(cap * 4) + 4 * Carver::pad(cap * 8) + Carver::pad(cap * TA_NBINS * 4) + 256;
-    void *outb = ta_dalloc(h, ob);
-    if (!outb) return TA_ERR_OOM;
-    Carver co(outb);
-    AggRowOut ro;
-    ro.cnt = a.d_cnt; ro.sum = a.d_sum; ro.minc = a.d_minc; ro.maxb = a.d_maxb; ro.hist = a.d_hist;
-    ro.tt = h->d_triples; ro.n_pids = n_pids; ro.R = R; ro.min_name = h->min_name;
-    ro.g_window = co.take<int32_t>(cap); ro.g_pid = co.take<int32_t>(cap); ro.g_name = co.take<int32_t>(cap);
-    ro.g_count = co.take<int64_t>(cap); ro.g_sum = co.take<int64_t>(cap);
-    ro.g_min = co.take<int64_t>(cap); ro.g_max = co.take<int64_t>(cap);
-    ro.g_hist = co.take<u32>(cap * TA_NBINS);
+  void *tmpb = nullptr, *outb = nullptr;
+  // the three row tables (window, pid, symbol), the four 64-bit columns and the histograms of `rows` rows
+  auto carve_rows = [&](int64_t rows) -> size_t {
+    const size_t b = Carver::pad(rows * 8) * 4 + Carver::pad(rows * TA_NBINS * 4) + Carver::pad(rows * 4) * 3 + 256;
+    outb = ta_dalloc(h, b);
+    if (!outb) return 0;
+    Carver c(outb);
+    ro.g_count = c.take<int64_t>(rows); ro.g_sum = c.take<int64_t>(rows);
+    ro.g_min = c.take<int64_t>(rows); ro.g_max = c.take<int64_t>(rows);
+    ro.g_hist = c.take<u32>(rows * TA_NBINS);
+    const size_t zero = c.off;  // what has to start at zero when records are folded into the rows directly
+    ro.g_window = c.take<int32_t>(rows); ro.g_pid = c.take<int32_t>(rows); ro.g_name = c.take<int32_t>(rows);
+    return zero;
+  };
+  // Dense rows: 192 bytes per cell to clear and a scan over the cells.  Marked cells: one more pass
+  // over kinds and symbols (6 bytes per record) and a round trip for the number of rows.  The line
+  // is drawn where the dense table's bytes reach those of the extra pass plus what some 20 us
+  // (pass, scan, round trip) are worth.  512 windows of 65 k records have 33 M cells, one in
+  // twenty of them occupied: 1.85 ms per call dense.
+  if (G * 232 <= 8 * h->n_valid + (64ll << 20)) {
     ScanTemp t;
-    TA_TRY(scan_temp_init(h, scan_mem, G, &t));
+    size_t tb = 4 * Carver::pad((size_t)G * 8) + Carver::pad((size_t)G * TA_NBINS * 4) + scan_temp_bytes(G) + 256;
+    tmpb = ta_dalloc(h, tb);
+    if (!tmpb) return TA_ERR_OOM;
+    Carver ct(tmpb);
+    a.d_cnt = ct.take<u64>(G);
+    a.d_sum = ct.take<u64>(G);
+    a.d_minc = ct.take<u64>(G);
+    a.d_maxb = ct.take<u64>(G);
+    a.d_hist = ct.take<u32>((size_t)G * TA_NBINS);
+    ct.off += scan_temp_carve(ct.base + ct.off, G, &t);
+    TA_CHECK_CUDA(h, cudaMemsetAsync(tmpb, 0, ct.off, st));
+    k_agg<<<TA_N (unsigned)blocks, AG_THREADS, 0, st>>>(a);
+    // the rows are compacted without waiting for their count: it is bounded by cells and records
+    carve_rows(G < h->n_valid ? G : h->n_valid);
+    if (!outb) return TA_ERR_OOM;
+    ro.cnt = a.d_cnt; ro.sum = a.d_sum; ro.minc = a.d_minc; ro.maxb = a.d_maxb; ro.hist = a.d_hist;
     AggRowIn ri{a.d_cnt};
     TA_TRY((launch_scan<OpAdd, AggRowIn, AggRowOut>(h, G, ri, ro, OpAdd(), t)));
-    scan_total = t.total;
-    out->g_window = ro.g_window; out->g_pid = ro.g_pid; out->g_name = ro.g_name;
-    out->g_count = ro.g_count; out->g_sum = ro.g_sum; out->g_min = ro.g_min; out->g_max = ro.g_max;
-    out->g_hist = ro.g_hist;
+    TA_TRY(ta_queue_d2h(h, &ng, t.total, 8));
+  } else {
+    const int64_t words = (G + 31) / 32;
+    ScanTemp t;
+    tmpb = ta_dalloc(h, 2 * Carver::pad((size_t)words * 4) + scan_temp_bytes(words) + 256);
+    if (!tmpb) return TA_ERR_OOM;
+    Carver ct(tmpb);
+    a.bits = ct.take<u32>(words);
+    ct.off += scan_temp_carve(ct.base + ct.off, words, &t);
+    TA_CHECK_CUDA(h, cudaMemsetAsync(tmpb, 0, ct.off, st));
+    u32 *rank = ct.take<u32>(words);
+    k_agg_mark<<<TA_N a.n_items, AG_THREADS, 0, st>>>(a);
+    AggBitsIn bi{a.bits};
+    AggBitsOut bo{rank};
+    TA_TRY((launch_scan<OpAdd, AggBitsIn, AggBitsOut>(h, words, bi, bo, OpAdd(), t)));
+    TA_TRY(ta_queue_d2h(h, &ng, t.total, 8));
+    TA_TRY(ta_sync_fetch(h));
+    if (ng > 0) {
+      const size_t zero = carve_rows((int64_t)ng);
+      if (!outb) return TA_ERR_OOM;
+      TA_CHECK_CUDA(h, cudaMemsetAsync(outb, 0, zero, st));
+      a.rank = rank;
+      a.d_cnt = (u64 *)ro.g_count; a.d_sum = (u64 *)ro.g_sum; a.d_minc = (u64 *)ro.g_min; a.d_maxb = (u64 *)ro.g_max;
+      a.d_hist = ro.g_hist;
+      k_agg<<<TA_N (unsigned)blocks, AG_THREADS, 0, st>>>(a);
+      k_agg_marked_rows<<<TA_N (unsigned)((words + 255) / 256), 256, 0, st>>>(a.bits, rank, words, ro, h->d_status);
+    }
   }
-  if (bounded && scan_total)  // the scan's total is the number of rows
-    TA_TRY(ta_queue_d2h(h, &ng, scan_total, 8));
+  TA_CHECK_CUDA(h, cudaGetLastError());
   int32_t words[ST_WORDS];
   TA_TRY(ta_read_status(h, words));
-  out->n_groups = (int64_t)ng;
   ta_dfree(h, tmpb);
   if (words[ST_ERR]) return (ta_status)words[ST_ERR];
+  out->n_groups = (int64_t)ng;
+  if (ng == 0) return TA_OK;
+  out->g_window = ro.g_window; out->g_pid = ro.g_pid; out->g_name = ro.g_name;
+  out->g_count = ro.g_count; out->g_sum = ro.g_sum; out->g_min = ro.g_min; out->g_max = ro.g_max;
+  out->g_hist = ro.g_hist;
   return TA_OK;
 }

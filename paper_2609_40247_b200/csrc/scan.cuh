@@ -19,15 +19,19 @@ static inline size_t scan_temp_bytes(int64_t n) {
   int64_t tiles = (n + SC_TILE - 1) / SC_TILE + 1;
   return Carver::pad((size_t)tiles * 8) + Carver::pad(64);
 }
-// carves and zeroes the temp (one memset)
-static inline ta_status scan_temp_init(ta_window *h, void *mem, int64_t n, ScanTemp *t) {
+// carves the temp; returns its size, all of which the caller has to zero
+static inline size_t scan_temp_carve(void *mem, int64_t n, ScanTemp *t) {
   int64_t tiles = (n + SC_TILE - 1) / SC_TILE + 1;
   Carver c(mem);
   t->state = c.take<u64>(tiles);
   u64 *sc = c.take<u64>(8);
   t->counter = (u32 *)(sc + 1);
   t->total = sc;
-  TA_CHECK_CUDA(h, cudaMemsetAsync(mem, 0, c.off, h->stream));
+  return c.off;
+}
+// carves and zeroes the temp (one memset)
+static inline ta_status scan_temp_init(ta_window *h, void *mem, int64_t n, ScanTemp *t) {
+  TA_CHECK_CUDA(h, cudaMemsetAsync(mem, 0, scan_temp_carve(mem, n, t), h->stream));
   return TA_OK;
 }
 

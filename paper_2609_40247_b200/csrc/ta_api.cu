@@ -490,6 +490,10 @@ ta_status ta_load_window(const ta_env *env, const ta_event *events, int64_t n,
   h->d_keys = nullptr;
   h->prekeys = 0;
   h->attr_status = 0;
+  h->n_names = 0;
+  h->d_names = nullptr;
+  h->d_name_rank = nullptr;
+  h->d_name_of = nullptr;
   h->d_op_gap_ns = nullptr;
   h->d_on_path = nullptr;
   h->d_status = nullptr;

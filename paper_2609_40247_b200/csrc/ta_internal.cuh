@@ -24,7 +24,8 @@ typedef unsigned int u32;
 #define TA_SPIN_LIMIT (1 << 22)   // polls of a tile descriptor before giving up
 #define TA_TIE_RUN_MAX 48         // equal-key runs up to this length are fixed in place
 #define TA_PACK_MAX_DROP 12        // low time bits a packed key may give up
-#define TA_AGG_DENSE_LIMIT (1ll << 27)
+#define TA_AGG_DENSE_LIMIT (1ll << 27)  // cells (window, pid, id - min id); beyond it ids go through a symbol table
+#define TA_AGG_MARK_LIMIT (1ll << 30)   // cells (window, pid, symbol rank) a bitmap is made for
 
 // device status word indices (h->d_status)
 // ST_SPIN: polls a device-side wait may make before it gives up (0 = TA_SPIN_LIMIT)
@@ -143,6 +144,12 @@ struct ta_window {
   const int64_t *d_op_gap_ns;  // per sorted position, set by the gap blame (null before)
   const uint8_t *d_on_path;    // per sorted position, set by the critical path (null before)
   int attr_status;
+
+  // symbol table of the aggregates (ids spread wide): 0 = not built, -1 = more symbols than it holds
+  int64_t n_names;
+  u64 *d_names;
+  u32 *d_name_rank;
+  int32_t *d_name_of;
 };
 
 // number of bits needed to write v (0 for 0)
