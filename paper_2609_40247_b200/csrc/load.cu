@@ -544,26 +544,13 @@ __global__ void __launch_bounds__(256) k_top_hist_words(TopHistArgs a) {
     if (sh[i]) atomicAdd(&a.hist[i], sh[i]);
 }
 
-// One CTA: sorts the discovered triples, ranks them and the pids they contain.
-__device__ __forceinline__ void rank_triples(TripleTable *tt, int32_t *status, u64 *buf /* TA_TRIPLE_SLOTS */) {
-  __shared__ u64 tmp[33];
-  __shared__ int n_tr;
+// ascending bitonic sort of buf[0 .. n) in shared memory by the whole CTA; positions up to the next
+// power of two are overwritten with all ones
+__device__ __forceinline__ void block_sort(u64 *buf, int n) {
   const int tid = threadIdx.x;
-  // the occupied slots, packed to the front (a window has tens of triples, not thousands)
-  if (tid == 0) n_tr = 0;
-  __syncthreads();
-  for (int c0 = 0; c0 < TA_TRIPLE_SLOTS; c0 += blockDim.x) {
-    const u64 v = tt->slots[c0 + tid];
-    u64 total;
-    const u64 ex = block_scan_exclusive<OpAdd>(v != TRIPLE_EMPTY ? 1ull : 0ull, OpAdd(), tmp, &total);
-    if (v != TRIPLE_EMPTY) buf[n_tr + (int)ex] = v;
-    __syncthreads();
-    if (tid == 0) n_tr += (int)total;
-    __syncthreads();
-  }
   int padded = 32;
-  while (padded < n_tr) padded <<= 1;
-  for (int i = n_tr + tid; i < padded; i += blockDim.x) buf[i] = TRIPLE_EMPTY;  // sorts last
+  while (padded < n) padded <<= 1;
+  for (int i = n + tid; i < padded; i += blockDim.x) buf[i] = ~0ull;
   __syncthreads();
   for (int k = 2; k <= padded; k <<= 1)
     for (int j = k >> 1; j > 0; j >>= 1) {
@@ -577,81 +564,82 @@ __device__ __forceinline__ void rank_triples(TripleTable *tt, int32_t *status, u
       }
       __syncthreads();
     }
+}
+
+// One CTA: sorts the discovered triples, ranks them and the pids they contain.  A window has tens
+// of triples: the occupied slots are packed to the front in any order, as code << 13 | slot, so
+// that the sorted entry names its slot; the table is read once and only its occupied slots are
+// written (two passes over all slots in block-scan rounds and a serial pid walk took 20 us).
+__device__ __forceinline__ void rank_triples(TripleTable *tt, int32_t *status, u64 *buf /* TA_TRIPLE_SLOTS */) {
+  __shared__ u64 tmp[33];
+  __shared__ int n_tr;
+  const int tid = threadIdx.x;
+  if (tid == 0) n_tr = 0;
+  __syncthreads();
+  for (int s = tid; s < TA_TRIPLE_SLOTS; s += blockDim.x) {
+    const u64 v = tt->slots[s];
+    if (v != TRIPLE_EMPTY) buf[atomicAdd(&n_tr, 1)] = (v << 13) | (u64)s;
+  }
+  __syncthreads();
+  block_sort(buf, n_tr);
   int n = n_tr;
   if (n > TA_MAX_TRIPLES) {
     if (tid == 0) ta_set_err(status, TA_ERR_TOO_LARGE);
     n = TA_MAX_TRIPLES;
   }
-  for (int i = tid; i < n; i += blockDim.x) tt->sorted_code[i] = buf[i];
-  if (tid == 0) {
-    int pr = -1;
-    u64 prev = ~0ull;
-    for (int i = 0; i < n; i++) {
-      u64 pidb = buf[i] >> 17;
-      if (pidb != prev) { pr++; prev = pidb; tt->pid_value[pr] = (int32_t)((u32)pidb ^ 0x80000000u); }
+  int pids = 0;  // pids in front of the round
+  for (int i0 = 0; i0 < n; i0 += blockDim.x) {
+    const int i = i0 + tid;
+    const u64 c = i < n ? buf[i] >> 13 : 0;
+    const bool head = i < n && (i == 0 || (buf[i - 1] >> 30) != (c >> 17));
+    u64 total;
+    const u64 ex = block_scan_exclusive<OpAdd>(head ? 1ull : 0ull, OpAdd(), tmp, &total);
+    const int pr = pids + (int)ex + (head ? 1 : 0) - 1;
+    if (i < n) {
+      tt->sorted_code[i] = c;
+      tt->rank_of_slot[(u32)buf[i] & (TA_TRIPLE_SLOTS - 1)] = i;
       tt->pid_rank[i] = pr;
+      if (head) tt->pid_value[pr] = (int32_t)((u32)(c >> 17) ^ 0x80000000u);
     }
-    status[ST_N_TRIPLES] = n;
-    status[ST_N_PIDS] = pr + 1;
+    pids += (int)total;
   }
-  for (int s = tid; s < TA_TRIPLE_SLOTS; s += blockDim.x) {
-    u64 c = tt->slots[s];
-    int r = -1;
-    if (c != TRIPLE_EMPTY) {
-      int lo = 0, hi = n - 1;
-      while (lo < hi) {
-        int mid = (lo + hi) >> 1;
-        if (buf[mid] < c) lo = mid + 1;
-        else hi = mid;
-      }
-      r = lo;
-    }
-    tt->rank_of_slot[s] = r;
+  if (tid == 0) {
+    status[ST_N_TRIPLES] = n;
+    status[ST_N_PIDS] = pids;
   }
 }
 
 // One CTA: sorts and ranks the communicator ids.
 __device__ __forceinline__ void rank_comms(CommTable *cm, int32_t *status, u64 *buf /* TA_COMM_SLOTS */) {
   __shared__ int n_c;
+  __shared__ u32 slot_of[TA_COMM_SLOTS];
   const int tid = threadIdx.x;
-  for (int i = tid; i < TA_COMM_SLOTS; i += blockDim.x) buf[i] = cm->slots[i];
   if (tid == 0) n_c = 0;
   __syncthreads();
-  for (int k = 2; k <= TA_COMM_SLOTS; k <<= 1)
-    for (int j = k >> 1; j > 0; j >>= 1) {
-      for (int i = tid; i < TA_COMM_SLOTS; i += blockDim.x) {
-        int ixj = i ^ j;
-        if (ixj > i) {
-          u64 a = buf[i], b = buf[ixj];
-          bool up = (i & k) == 0;
-          if ((a > b) == up) { buf[i] = b; buf[ixj] = a; }
-        }
-      }
-      __syncthreads();
+  for (int s = tid; s < TA_COMM_SLOTS; s += blockDim.x) {
+    const u64 v = cm->slots[s];
+    if (v != TRIPLE_EMPTY) {
+      const int at = atomicAdd(&n_c, 1);
+      buf[at] = v;
+      slot_of[at] = (u32)s;
     }
-  for (int i = tid; i < TA_COMM_SLOTS; i += blockDim.x)
-    if (buf[i] != TRIPLE_EMPTY && (i + 1 == TA_COMM_SLOTS || buf[i + 1] == TRIPLE_EMPTY)) n_c = i + 1;
+  }
   __syncthreads();
   int n = n_c;
-  if (n > TA_MAX_COMMS) {
-    if (tid == 0) ta_set_err(status, TA_ERR_TOO_LARGE);
-    n = TA_MAX_COMMS;
-  }
-  for (int i = tid; i < n; i += blockDim.x) cm->sorted_id[i] = buf[i];
-  if (tid == 0) status[ST_N_COMMS] = n;
-  for (int s = tid; s < TA_COMM_SLOTS; s += blockDim.x) {
-    u64 c = cm->slots[s];
-    int r = -1;
-    if (c != TRIPLE_EMPTY) {
-      int lo = 0, hi = n - 1;
-      while (lo < hi) {
-        int mid = (lo + hi) >> 1;
-        if (buf[mid] < c) lo = mid + 1;
-        else hi = mid;
-      }
-      r = lo;
+  if (tid == 0) status[ST_N_COMMS] = n > TA_MAX_COMMS ? TA_MAX_COMMS : n;
+  if (n == 0) return;
+  block_sort(buf, n);
+  if (n > TA_MAX_COMMS && tid == 0) ta_set_err(status, TA_ERR_TOO_LARGE);
+  for (int i = tid; i < n && i < TA_MAX_COMMS; i += blockDim.x) cm->sorted_id[i] = buf[i];
+  for (int i = tid; i < n; i += blockDim.x) {
+    const u64 c = cm->slots[slot_of[i]];
+    int lo = 0, hi = n - 1;
+    while (lo < hi) {
+      int mid = (lo + hi) >> 1;
+      if (buf[mid] < c) lo = mid + 1;
+      else hi = mid;
     }
-    cm->rank_of_slot[s] = r;
+    cm->rank_of_slot[slot_of[i]] = lo;
   }
 }
 
