@@ -7,8 +7,9 @@
 // lane-aware without segment flags: the scanned value is (lane + 1) << 40 |
 // (clipped end - window start), which grows from lane to lane, so a prefix
 // that belongs to an earlier lane is recognised by its upper bits.  Long gaps
-// are rare: they are appended to a list with an atomic cursor and the list is
-// put in (lane, time) order afterwards with the pair sorter.
+// are rare: they are appended to a list with an atomic cursor, each sets the bit of its
+// place in the order (two per record: the gap in front of it, the tail gap behind it) in
+// a bitmap, and a scan over the bitmap's words tells every entry its rank.
 // HBM-bound: 18 B read + 8 B written per device record.
 #include <climits>
 
@@ -46,7 +47,8 @@ struct GapArgs {
   ta_lane_gaps *lane_gaps;
   u32 *lane_hist, *win_hist;
   ta_long_gap *list;  // unordered
-  u64 *list_key;      // lane << 32 | next_event (0xFFFFFFFF for a tail gap)
+  u32 *list_key;      // 2 * position for the gap in front of a record, + 1 for the tail gap behind it
+  u64 *bits;          // bit `list_key` of every entry
   i64 list_cap;
   u64 *st_max;
   u32 *counter;
@@ -219,15 +221,17 @@ __global__ void __launch_bounds__(GP_THREADS, GP_MINB) k_gaps(GapArgs a) {
             const i64 o = (i64)base + __popc(m_g & below);
             if (o < a.list_cap) {
               a.list[o] = ta_long_gap{l, (int32_t)(p0 + j), Pi, g};
-              a.list_key[o] = ((u64)l << 32) | (u64)(u32)(p0 + j);
+              a.list_key[o] = (u32)(p0 + j) << 1;
             }
+            atomicOr(&a.bits[(p0 + j) >> 5], 1ull << (((u32)(p0 + j) & 31u) << 1));
           }
           if (lt) {
             const i64 o = (i64)base + __popc(m_g) + __popc(m_t & below);
             if (o < a.list_cap) {
               a.list[o] = ta_long_gap{l, -1, w1 - tl, tl};
-              a.list_key[o] = ((u64)l << 32) | 0xFFFFFFFFull;
+              a.list_key[o] = (u32)(p0 + j) << 1 | 1u;
             }
+            atomicOr(&a.bits[(p0 + j) >> 5], 2ull << (((u32)(p0 + j) & 31u) << 1));
           }
         }
       }
@@ -307,12 +311,23 @@ __global__ void __launch_bounds__(GP_THREADS, GP_MINB) k_gaps(GapArgs a) {
   }
 }
 
-__global__ void __launch_bounds__(256) k_gap_list_gather(const ta_long_gap *src, const u32 *order,
-                                                         int64_t m, ta_long_gap *dst,
-                                                         const int32_t *status) {
+struct GapBitsIn {
+  const u64 *bits;
+  __device__ u64 operator()(int64_t i) const { return (u64)__popcll(bits[i]); }
+};
+struct GapBitsOut {
+  u32 *rank;
+  __device__ void operator()(int64_t i, u64 excl, u64) const { rank[i] = (u32)excl; }
+};
+// every entry to its place
+__global__ void __launch_bounds__(256) k_gap_list_order(const ta_long_gap *src, const u32 *key, const u64 *bits,
+                                                        const u32 *rank, int64_t m, ta_long_gap *dst,
+                                                        const int32_t *status) {
   if (ta_failed(status)) return;
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < m) dst[i] = src[order[i]];
+  if (i >= m) return;
+  const u32 k = key[i];
+  dst[rank[k >> 6] + __popcll(bits[k >> 6] & ((1ull << (k & 63u)) - 1ull))] = src[i];
 }
 
 ta_status ta_run_gaps(ta_window *h, int64_t min_gap, ta_gap_result *out) {
@@ -325,7 +340,11 @@ ta_status ta_run_gaps(ta_window *h, int64_t min_gap, ta_gap_result *out) {
   int64_t cap = n / 8 > 65536 ? n / 8 : 65536;  // first guess; a longer list is rebuilt below
   size_t bytes = Carver::pad((size_t)(n > 0 ? n : 1) * 8) + Carver::pad((size_t)(L + 1) * sizeof(ta_lane_gaps)) +
                  Carver::pad((size_t)(L + 1) * TA_NBINS * 4) + Carver::pad((size_t)W * TA_NBINS * 4) +
-                 Carver::pad((size_t)(tiles + 1) * 8) + Carver::pad(64) + 512;
+                 512;
+  // temporary: look-back state, scalars, the bitmap of the list's order, its scan
+  const int64_t n_bits = (n + 31) / 32;
+  const size_t tmp_bytes = Carver::pad((size_t)(tiles + 1) * 8) + Carver::pad(64) + Carver::pad((size_t)n_bits * 8) +
+                           scan_temp_bytes(n_bits) + Carver::pad((size_t)n_bits * 4) + 512;
   void *b = ta_dalloc(h, bytes);
   if (!b) return TA_ERR_OOM;
   Carver c(b);
@@ -335,16 +354,26 @@ ta_status ta_run_gaps(ta_window *h, int64_t min_gap, ta_gap_result *out) {
   ta_lane_gaps *lane_gaps = c.take<ta_lane_gaps>(L + 1);
   u32 *lane_hist = c.take<u32>((size_t)(L + 1) * TA_NBINS);
   u32 *win_hist = c.take<u32>((size_t)W * TA_NBINS);
-  u64 *st_max = c.take<u64>(tiles + 1);
-  u64 *scal = c.take<u64>(8);  // [0] list cursor, [1] tile counter
   char *zero_end = c.base + c.off;
   TA_CHECK_CUDA(h, cudaMemsetAsync(zero_begin, 0, zero_end - zero_begin, st));
+  void *tb = ta_dalloc(h, tmp_bytes);
+  if (!tb) return TA_ERR_OOM;
+  Carver ct(tb);
+  u64 *st_max = ct.take<u64>(tiles + 1);
+  u64 *scal = ct.take<u64>(8);  // [0] list cursor, [1] tile counter, [2] not ascending
+  const size_t state_bytes = ct.off;
+  u64 *bits = ct.take<u64>(n_bits);
+  ScanTemp scan;
+  ct.off += scan_temp_carve(ct.base + ct.off, n_bits, &scan);
+  const size_t tmp_zero = ct.off;
+  u32 *rank = ct.take<u32>(n_bits);
+  TA_CHECK_CUDA(h, cudaMemsetAsync(tb, 0, tmp_zero, st));
   // unordered list + keys (temporary)
-  void *lt = ta_dalloc(h, Carver::pad((size_t)cap * sizeof(ta_long_gap)) + Carver::pad((size_t)cap * 8) + 256);
+  void *lt = ta_dalloc(h, Carver::pad((size_t)cap * sizeof(ta_long_gap)) + Carver::pad((size_t)cap * 4) + 256);
   if (!lt) return TA_ERR_OOM;
   Carver cl(lt);
   ta_long_gap *ulist = cl.take<ta_long_gap>(cap);
-  u64 *ukeys = cl.take<u64>(cap);
+  u32 *ukeys = cl.take<u32>(cap);
 
   GapArgs a;
   a.n = n; a.n_valid = h->n_valid; a.n_lanes = L;
@@ -353,7 +382,7 @@ ta_status ta_run_gaps(ta_window *h, int64_t min_gap, ta_gap_result *out) {
   a.lane_domain = h->sorted.lane_domain; a.lane_dom_end = h->d_lane_dom_end; a.t0 = h->d_t0; a.t1 = h->d_t1;
   a.min_gap = min_gap; a.list_only = 0;
   a.gap_before = gap_before; a.lane_gaps = lane_gaps; a.lane_hist = lane_hist; a.win_hist = win_hist;
-  a.list = ulist; a.list_key = ukeys; a.list_cap = cap; a.st_max = st_max;
+  a.list = ulist; a.list_key = ukeys; a.list_cap = cap; a.st_max = st_max; a.bits = bits;
   a.counter = (u32 *)(scal + 1); a.status = h->d_status; a.n_long = scal;
   a.not_ascending = (u32 *)(scal + 2);
   u64 n_long = 0;
@@ -370,17 +399,18 @@ ta_status ta_run_gaps(ta_window *h, int64_t min_gap, ta_gap_result *out) {
     n_long = two[0];
     if (!a.local || !(u32)two[2]) break;
     TA_CHECK_CUDA(h, cudaMemsetAsync(zero_begin, 0, zero_end - zero_begin, st));
+    TA_CHECK_CUDA(h, cudaMemsetAsync(tb, 0, tmp_zero, st));
   }
   if ((int64_t)n_long > cap) {
     // rare: a tiny min_gap made the list longer than the first guess; rebuild it
     ta_dfree(h, lt);
     cap = (int64_t)n_long;
-    lt = ta_dalloc(h, Carver::pad((size_t)cap * sizeof(ta_long_gap)) + Carver::pad((size_t)cap * 8) + 256);
+    lt = ta_dalloc(h, Carver::pad((size_t)cap * sizeof(ta_long_gap)) + Carver::pad((size_t)cap * 4) + 256);
     if (!lt) return TA_ERR_OOM;
     Carver cl2(lt);
     ulist = cl2.take<ta_long_gap>(cap);
-    ukeys = cl2.take<u64>(cap);
-    TA_CHECK_CUDA(h, cudaMemsetAsync(st_max, 0, (char *)zero_end - (char *)st_max, st));
+    ukeys = cl2.take<u32>(cap);
+    TA_CHECK_CUDA(h, cudaMemsetAsync(tb, 0, state_bytes, st));
     a.list = ulist; a.list_key = ukeys; a.list_cap = cap; a.list_only = 1;
     k_gaps<<<TA_N (unsigned)tiles, GP_THREADS, 0, st>>>(a);
     TA_CHECK_CUDA(h, cudaGetLastError());
@@ -393,23 +423,18 @@ ta_status ta_run_gaps(ta_window *h, int64_t min_gap, ta_gap_result *out) {
   if (m > 0) {
     list = (ta_long_gap *)ta_dalloc(h, (size_t)m * sizeof(ta_long_gap));
     if (!list) return TA_ERR_OOM;
-    void *stb = ta_dalloc(h, 2 * Carver::pad((size_t)m * 8) + 2 * Carver::pad((size_t)m * 4) +
-                                 ta_sort_temp_bytes(m) + 256);
-    if (!stb) return TA_ERR_OOM;
-    Carver cs(stb);
-    u64 *ks = cs.take<u64>(m), *kf = cs.take<u64>(m);
-    u32 *vs = cs.take<u32>(m), *order = cs.take<u32>(m);
-    TA_TRY(ta_radix_sort_pairs(h, ukeys, nullptr, ks, vs, kf, order, m,
-                               ta_make_plan(0, 32 + ta_bit_len((uint64_t)(L > 1 ? L - 1 : 1))), nullptr,
-                               cs.base + cs.off));
-    k_gap_list_gather<<<TA_N (unsigned)((m + 255) / 256), 256, 0, st>>>(ulist, order, m, list, h->d_status);
+    GapBitsIn bi{bits};
+    GapBitsOut bo{rank};
+    TA_TRY((launch_scan<OpAdd, GapBitsIn, GapBitsOut>(h, n_bits, bi, bo, OpAdd(), scan)));
+    k_gap_list_order<<<TA_N (unsigned)((m + 255) / 256), 256, 0, st>>>(ulist, ukeys, bits, rank, m, list, h->d_status);
     TA_CHECK_CUDA(h, cudaGetLastError());
-    // the sort and the gather are still queued: their temporaries go back after the handle's
-    // next synchronisation (the list itself is used in stream order like every other result)
-    ta_dfree_later(h, stb);
+    // both kernels are still queued: their temporaries go back after the handle's next
+    // synchronisation (the list itself is used in stream order like every other result)
+    ta_dfree_later(h, tb);
     ta_dfree_later(h, lt);
-    lt = nullptr;
+    tb = lt = nullptr;
   }
+  if (tb) ta_dfree(h, tb);
   if (lt) ta_dfree(h, lt);
   out->gap_before = gap_before;
   out->lane_gaps = lane_gaps;
