@@ -14,6 +14,7 @@
 #include <climits>
 
 #include "records.cuh"
+#include "scan.cuh"
 #include "ta_internal.cuh"
 
 // ---- pair path: equal-key runs -------------------------------------------
@@ -225,9 +226,8 @@ __global__ void __launch_bounds__(256, GT_MINB) k_gather(GatherArgs a) {
   }
 }
 
-#define LT_ITEMS 8
 // One CTA: compacts the non-empty lane codes into the lane table (code order is
-// canonical order).
+// canonical order).  For few codes; k_scan with the functors below does the same for many.
 __global__ void __launch_bounds__(1024) k_lane_table(const int32_t *lane_start, int64_t n_codes,
                                                      int tbits, int n_pids, const TripleTable *tt,
                                                      int64_t n_valid, int32_t *lane_window,
@@ -245,36 +245,24 @@ __global__ void __launch_bounds__(1024) k_lane_table(const int32_t *lane_start, 
   }
   if (threadIdx.x == 0) base = 0;
   __syncthreads();
-  // LT_ITEMS consecutive codes (then lanes) per thread and round: a batch of 512 windows has 65 k
-  // codes, and one code per thread took 64 rounds of two block scans each (165 us; now 28 us)
-  for (int64_t c0 = 0; c0 < n_codes; c0 += LT_ITEMS * blockDim.x) {
-    const int64_t cb = c0 + (int64_t)threadIdx.x * LT_ITEMS;
-    int32_t sts[LT_ITEMS];
-    u32 mine = 0;
-#pragma unroll
-    for (int j = 0; j < LT_ITEMS; j++) {
-      sts[j] = cb + j < n_codes ? lane_start[cb + j] : -1;
-      mine += sts[j] >= 0;
-    }
+  for (int64_t c0 = 0; c0 < n_codes; c0 += blockDim.x) {
+    int64_t c = c0 + threadIdx.x;
+    int32_t st = c < n_codes ? lane_start[c] : -1;
     u64 total;
-    const u64 ex = block_scan_exclusive<OpAdd>((u64)mine, OpAdd(), tmp, &total);
-    int64_t l = (int64_t)(base + ex);
-#pragma unroll
-    for (int j = 0; j < LT_ITEMS; j++) {
-      if (sts[j] < 0) continue;
+    u64 ex = block_scan_exclusive<OpAdd>(st >= 0 ? 1ull : 0ull, OpAdd(), tmp, &total);
+    if (st >= 0) {
+      int64_t l = (int64_t)(base + ex);
       if (l < cap) {
-        const int64_t c = cb + j;
         int w = (int)(c >> tbits), t = (int)(c & ((1ll << tbits) - 1));
         u64 code = tt->sorted_code[t];
         lane_window[l] = w;
         lane_pid[l] = code_pid(code);
         lane_stream[l] = code_stream(code);
         lane_domain[l] = code_domain(code);
-        lane_off[l] = sts[j];
+        lane_off[l] = st;
         lane_code[l] = (int32_t)c;
         lane_slot[l] = w * n_pids + tt->pid_rank[t];
       }
-      l++;
     }
     __syncthreads();
     if (threadIdx.x == 0) base += total;
@@ -290,33 +278,24 @@ __global__ void __launch_bounds__(1024) k_lane_table(const int32_t *lane_start, 
   // and device lanes alternate per (window, pid), so the runs are a few lanes long - but a batch
   // of device-only windows is one long run, hence a scan and no walk).  Going backwards over
   // the lanes, the nearest boundary at or behind lane l is a running maximum of
-  // L - (index of the lane behind a boundary); rounds of LT_ITEMS * blockDim.x lanes, carried in `base`.
+  // L - (index of the lane behind a boundary); chunks of blockDim.x lanes, carried in `base`.
   const int64_t L = (int64_t)base < cap ? (int64_t)base : cap;
   __syncthreads();  // every thread has read the lane count before `base` is reused
   if (threadIdx.x == 0) base = 0;
   __syncthreads();
-  for (int64_t r0 = 0; r0 < L; r0 += LT_ITEMS * blockDim.x) {
-    const int64_t rb = r0 + (int64_t)threadIdx.x * LT_ITEMS;  // reversed lane index
-    u64 v[LT_ITEMS], run = 0;
-#pragma unroll
-    for (int j = 0; j < LT_ITEMS; j++) {
-      const int64_t r = rb + j, l = L - 1 - r;
-      v[j] = 0;
-      if (r < L && l + 1 < L && lane_domain[l + 1] != lane_domain[l]) v[j] = (u64)(L - (l + 1));
-      run = max(run, v[j]);
-    }
+  for (int64_t r0 = 0; r0 < L; r0 += blockDim.x) {
+    const int64_t r = r0 + threadIdx.x;  // reversed lane index
+    const int64_t l = L - 1 - r;
+    u64 v = 0;
+    if (r < L && l + 1 < L && lane_domain[l + 1] != lane_domain[l]) v = (u64)(L - (l + 1));
     u64 total;
-    const u64 ex = block_scan_exclusive<OpMax>(run, OpMax(), tmp, &total);
-    u64 best = max((u64)base, ex);
-#pragma unroll
-    for (int j = 0; j < LT_ITEMS; j++) {
-      const int64_t r = rb + j, l = L - 1 - r;
-      best = max(best, v[j]);
-      if (r < L) {
-        const int64_t m = best ? L - (int64_t)best : L;
-        lane_dom_end[l] = m < L ? lane_off[m] : (int32_t)n_valid;
-        lane_dom_next[l] = (int32_t)m;  // index of the first later lane of the other domain (L if none)
-      }
+    const u64 ex = block_scan_exclusive<OpMax>(v, OpMax(), tmp, &total);
+    if (r < L) {
+      u64 best = ex > v ? ex : v;
+      best = best > base ? best : base;
+      const int64_t m = best ? L - (int64_t)best : L;
+      lane_dom_end[l] = m < L ? lane_off[m] : (int32_t)n_valid;
+      lane_dom_next[l] = (int32_t)m;  // index of the first later lane of the other domain (L if none)
     }
     __syncthreads();
     if (threadIdx.x == 0) base = base > total ? base : total;
@@ -326,31 +305,91 @@ __global__ void __launch_bounds__(1024) k_lane_table(const int32_t *lane_start, 
   // records are taken out in order); n_lanes_out[1] = the number of device records
   if (threadIdx.x == 0) base = 0;
   __syncthreads();
-  for (int64_t l0 = 0; l0 < L; l0 += LT_ITEMS * blockDim.x) {
-    const int64_t lb = l0 + (int64_t)threadIdx.x * LT_ITEMS;
-    u32 sz[LT_ITEMS];
-    u64 run = 0;
-#pragma unroll
-    for (int j = 0; j < LT_ITEMS; j++) {
-      const int64_t l = lb + j;
-      sz[j] = 0;
-      if (l < L && lane_domain[l] == 1) sz[j] = (u32)((l + 1 < L ? lane_off[l + 1] : (int32_t)n_valid) - lane_off[l]);
-      run += sz[j];
-    }
+  for (int64_t l0 = 0; l0 < L; l0 += blockDim.x) {
+    const int64_t l = l0 + threadIdx.x;
+    u64 sz = 0;
+    if (l < L && lane_domain[l] == 1) sz = (u64)((l + 1 < L ? lane_off[l + 1] : (int32_t)n_valid) - lane_off[l]);
     u64 total;
-    const u64 ex = block_scan_exclusive<OpAdd>(run, OpAdd(), tmp, &total);
-    u64 at = base + ex;
-#pragma unroll
-    for (int j = 0; j < LT_ITEMS; j++) {
-      if (lb + j < L) lane_dev_base[lb + j] = (int32_t)at;
-      at += sz[j];
-    }
+    const u64 ex = block_scan_exclusive<OpAdd>(sz, OpAdd(), tmp, &total);
+    if (l < L) lane_dev_base[l] = (int32_t)(base + ex);
     __syncthreads();
     if (threadIdx.x == 0) base += total;
     __syncthreads();
   }
   if (threadIdx.x == 0) n_lanes_out[1] = (int32_t)base;
 }
+
+// The same for many codes (a batch of 512 windows has 65 k of them, and one CTA was bound by the
+// scattered writes it has to make alone: 165 us): three scans over as many CTAs as it takes.
+struct LaneRows {
+  const int32_t *lane_start;
+  int tbits, n_pids;
+  const TripleTable *tt;
+  int64_t n_valid;
+  int32_t *lane_window, *lane_pid;
+  int16_t *lane_stream, *lane_domain;
+  int32_t *lane_off, *lane_code, *lane_slot, *lane_dom_end, *lane_dom_next, *lane_dev_base, *n_lanes_out;
+  const u64 *n_lanes;  // total of the first scan
+  int64_t bound;       // lanes <= bound
+};
+struct LaneCodeIn {
+  LaneRows t;
+  __device__ u64 operator()(int64_t c) const { return t.lane_start[c] >= 0 ? 1ull : 0ull; }
+};
+struct LaneCodeOut {
+  LaneRows t;
+  __device__ void operator()(int64_t c, u64 l, u64 v) const {
+    if (!v || (int64_t)l >= t.bound) return;
+    const int w = (int)(c >> t.tbits), r = (int)(c & ((1ll << t.tbits) - 1));
+    const u64 code = t.tt->sorted_code[r];
+    t.lane_window[l] = w;
+    t.lane_pid[l] = code_pid(code);
+    t.lane_stream[l] = code_stream(code);
+    t.lane_domain[l] = code_domain(code);
+    t.lane_off[l] = t.lane_start[c];
+    t.lane_code[l] = (int32_t)c;
+    t.lane_slot[l] = w * t.n_pids + t.tt->pid_rank[r];
+  }
+};
+struct LaneDomIn {  // element r = lane L - 1 - r
+  LaneRows t;
+  __device__ u64 operator()(int64_t r) const {
+    const int64_t L = (int64_t)*t.n_lanes, l = L - 1 - r;
+    return l >= 0 && l + 1 < L && t.lane_domain[l + 1] != t.lane_domain[l] ? (u64)(L - (l + 1)) : 0ull;
+  }
+};
+struct LaneDomOut {
+  LaneRows t;
+  __device__ void operator()(int64_t r, u64 excl, u64 v) const {
+    const int64_t L = (int64_t)*t.n_lanes, l = L - 1 - r;
+    if (r == 0) {
+      t.lane_off[L] = (int32_t)t.n_valid;
+      t.n_lanes_out[0] = (int32_t)L;
+    }
+    if (l < 0) return;
+    const u64 best = excl > v ? excl : v;
+    const int64_t m = best ? L - (int64_t)best : L;
+    t.lane_dom_end[l] = m < L ? t.lane_off[m] : (int32_t)t.n_valid;
+    t.lane_dom_next[l] = (int32_t)m;
+  }
+};
+struct LaneDevIn {
+  LaneRows t;
+  __device__ u64 operator()(int64_t l) const {
+    const int64_t L = (int64_t)*t.n_lanes;
+    if (l >= L || t.lane_domain[l] != 1) return 0;
+    return (u64)((l + 1 < L ? t.lane_off[l + 1] : (int32_t)t.n_valid) - t.lane_off[l]);
+  }
+};
+struct LaneDevOut {
+  LaneRows t;
+  __device__ void operator()(int64_t l, u64 excl, u64 v) const {
+    if (l < (int64_t)*t.n_lanes) t.lane_dev_base[l] = (int32_t)excl;
+    if (l == t.bound - 1) t.n_lanes_out[1] = (int32_t)(excl + v);
+  }
+};
+// codes up to which one CTA makes the table
+#define LT_ONE_CTA 4096
 
 // ---- packed keys: index of the record a key stands for -------------------------
 struct PackInfo {
@@ -401,7 +440,7 @@ ta_status ta_run_sort_timeline(ta_window *h) {
 
   // temporaries (released at the end of the call)
   size_t tmp_bytes = 2 * Carver::pad(n * 8) + Carver::pad(n * 4) + ta_sort_temp_bytes(n) +
-                     Carver::pad(n_codes * 4) + 512;
+                     Carver::pad(n_codes * 4) + 2 * scan_temp_bytes(lane_cap) + scan_temp_bytes(n_codes) + 512;
   void *tb = ta_dalloc(h, tmp_bytes);
   if (!tb) return TA_ERR_OOM;
   Carver ct(tb);
@@ -509,11 +548,28 @@ ta_status ta_run_sort_timeline(ta_window *h) {
       g.slot_min = h->d_slot_min; g.slot_max = h->d_slot_max; g.status = h->d_status;
       k_gather<<<TA_N nblk(n, 256), 256, 0, st>>>(g);
     }
-    k_lane_table<<<TA_N 1, 1024, 0, st>>>(lane_start, n_codes, h->tbits,
+    if (n_codes <= LT_ONE_CTA || n == 0) {
+      k_lane_table<<<TA_N 1, 1024, 0, st>>>(lane_start, n_codes, h->tbits,
                                      h->n_pids > 0 ? h->n_pids : 1, h->d_triples, h->n_valid,
                                      lane_window, lane_pid, lane_stream, lane_domain, lane_off,
                                      lane_code, lane_slot, lane_dom_end, lane_dom_next, lane_dev_base, n_lanes_dev,
                                      lane_cap, h->d_status);
+    } else {
+      LaneRows t{lane_start, h->tbits, h->n_pids > 0 ? h->n_pids : 1, h->d_triples, h->n_valid,
+                 lane_window, lane_pid, lane_stream, lane_domain, lane_off, lane_code, lane_slot,
+                 lane_dom_end, lane_dom_next, lane_dev_base, n_lanes_dev, nullptr, lane_cap - 1};
+      Carver cs(sort_tmp);  // the sort is done with its temporaries by the time the scans run
+      ScanTemp s1, s2, s3;
+      cs.off += scan_temp_carve(cs.base + cs.off, n_codes, &s1);
+      cs.off += scan_temp_carve(cs.base + cs.off, t.bound, &s2);
+      cs.off += scan_temp_carve(cs.base + cs.off, t.bound, &s3);
+      TA_CHECK_CUDA(h, cudaMemsetAsync(sort_tmp, 0, cs.off, st));
+      t.n_lanes = s1.total;
+      TA_CHECK_CUDA(h, cudaMemsetAsync(n_lanes_dev, 0, 8, st));
+      TA_TRY((launch_scan<OpAdd, LaneCodeIn, LaneCodeOut>(h, n_codes, LaneCodeIn{t}, LaneCodeOut{t}, OpAdd(), s1)));
+      TA_TRY((launch_scan<OpMax, LaneDomIn, LaneDomOut>(h, t.bound, LaneDomIn{t}, LaneDomOut{t}, OpMax(), s2)));
+      TA_TRY((launch_scan<OpAdd, LaneDevIn, LaneDevOut>(h, t.bound, LaneDevIn{t}, LaneDevOut{t}, OpAdd(), s3)));
+    }
     TA_CHECK_CUDA(h, cudaGetLastError());
     TA_TRY(ta_queue_d2h(h, n_lanes_host, n_lanes_dev, 2 * sizeof(int32_t)));
     TA_TRY(ta_queue_d2h(h, h->h_slot_min.data(), h->d_slot_min, n_slots * 8));
