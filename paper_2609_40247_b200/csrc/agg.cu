@@ -126,8 +126,9 @@ __global__ void __launch_bounds__(256) k_name_rank(const u64 *sorted, int64_t D,
   name_rank[(u32)x & (NT_SLOTS - 1)] = (u32)i;
   name_of[i] = (int32_t)((u32)(x >> 32) ^ 0x80000000u);
 }
+template <bool TABLE>
 __device__ __forceinline__ int64_t name_rank_of(const AggArgs &a, int32_t nm) {
-  if (!a.names) return (int64_t)nm - a.min_name;
+  if (!TABLE) return (int64_t)nm - a.min_name;
   const u64 e = (u64)((u32)nm ^ 0x80000000u) + 1;
   u32 slot = name_hash((u32)(e - 1));
   // every id of the window is in the table: a bounded probe all the same
@@ -141,8 +142,9 @@ __device__ __forceinline__ int64_t row_of(const AggArgs &a, int64_t g) {
 
 struct AggSmem {
   int32_t key[AG_SLOTS];
-  u32 cnt[AG_SLOTS];
-  u32 sum16[3][AG_SLOTS];  // the sum in 16-bit limbs: native 32-bit shared-memory atomics only
+  // the sum in limbs of 17 bits (the third takes the rest, modulo 2^32): native 32-bit shared-memory
+  // atomics only, and one of them for a value below 131 us; the count is the sum of the bins
+  u32 sum[3][AG_SLOTS];
   u64 minc[AG_SLOTS];
   u64 maxb[AG_SLOTS];
   uint16_t hist[AG_SLOTS][TA_NBINS];
@@ -160,8 +162,7 @@ __device__ __forceinline__ void agg_global_add(const AggArgs &a, int64_t g, u64 
 __device__ __forceinline__ void agg_clear(AggSmem &s) {
   for (int i = threadIdx.x; i < AG_SLOTS; i += AG_THREADS) {
     s.key[i] = -1;
-    s.cnt[i] = 0;
-    s.sum16[0][i] = s.sum16[1][i] = s.sum16[2][i] = 0;
+    s.sum[0][i] = s.sum[1][i] = s.sum[2][i] = 0;
     s.minc[i] = 0;
     s.maxb[i] = 0;
   }
@@ -176,8 +177,11 @@ __device__ __forceinline__ void agg_flush(const AggArgs &a, AggSmem &s) {
     if (k >= 0) {
       k = (int32_t)row_of(a, k);
       s.key[i] = k;  // the row, for the bins below
-      agg_global_add(a, k, s.cnt[i],
-                     (u64)s.sum16[0][i] + ((u64)s.sum16[1][i] << 16) + ((u64)s.sum16[2][i] << 32),
+      const u32 *hw = reinterpret_cast<const u32 *>(&s.hist[i][0]);
+      u32 cnt = 0;
+#pragma unroll
+      for (int b = 0; b < TA_NBINS / 2; b++) cnt += (hw[b] & 0xFFFFu) + (hw[b] >> 16);
+      agg_global_add(a, k, cnt, (u64)s.sum[0][i] + ((u64)s.sum[1][i] << 17) + ((u64)s.sum[2][i] << 34),
                      s.minc[i], s.maxb[i]);
     }
   }
@@ -268,6 +272,7 @@ __device__ __forceinline__ void agg_select(const AggArgs &a, int64_t p0, int64_t
 }
 
 // sets the bit of every cell that holds a selected record
+template <bool TABLE>
 __global__ void __launch_bounds__(AG_THREADS) k_agg_mark(AggArgs a) {
   if (ta_failed(a.status)) return;
   LaneWalker lw(a.lane_off, a.n_lanes, a.n_valid, a.n_valid);
@@ -288,13 +293,14 @@ __global__ void __launch_bounds__(AG_THREADS) k_agg_mark(AggArgs a) {
 #pragma unroll
     for (int j = 0; j < AG_ITEMS; j++) {
       if (!sel[j]) continue;
-      const int64_t g = (int64_t)a.lane_slot[lw.at(p0 + j)] * a.R + name_rank_of(a, nm[j]);
+      const int64_t g = (int64_t)a.lane_slot[lw.at(p0 + j)] * a.R + name_rank_of<TABLE>(a, nm[j]);
       // a stale word only costs a second atomic: popular cells are set once and then read from L1
       if (!((a.bits[g >> 5] >> (g & 31)) & 1u)) atomicOr(&a.bits[g >> 5], 1u << (g & 31));
     }
   }
 }
 
+template <bool TABLE>
 __global__ void __launch_bounds__(AG_THREADS, 6) k_agg(AggArgs a) {
   __shared__ AggSmem s;
   if (ta_failed(a.status)) return;
@@ -329,7 +335,7 @@ __global__ void __launch_bounds__(AG_THREADS, 6) k_agg(AggArgs a) {
       for (int j = 0; j < AG_ITEMS; j++) {
         if (!sel[j]) continue;
         const int lane = lw.at(p0 + j);
-        const int64_t g = (int64_t)a.lane_slot[lane] * a.R + name_rank_of(a, nm[j]);
+        const int64_t g = (int64_t)a.lane_slot[lane] * a.R + name_rank_of<TABLE>(a, nm[j]);
         const u64 vb = (u64)v[j] ^ (1ull << 63);
         const int bin = log2_bin(v[j]);
         u32 hsh = (u32)g * 2654435761u;
@@ -345,13 +351,11 @@ __global__ void __launch_bounds__(AG_THREADS, 6) k_agg(AggArgs a) {
           slot = (slot + 1) & (AG_SLOTS - 1);
         }
         if (placed) {
-          atomicAdd(&s.cnt[slot], 1u);
-          {  // values are durations (>= 0): 16 + 16 + 32 bit limbs, at most 32768 adds per flush
-            const u64 uv = (u64)v[j];
-            atomicAdd(&s.sum16[0][slot], (u32)(uv & 0xFFFF));
-            if (uv >> 16) atomicAdd(&s.sum16[1][slot], (u32)((uv >> 16) & 0xFFFF));
-            if (uv >> 32) atomicAdd(&s.sum16[2][slot], (u32)(uv >> 32));
-          }
+          // values are durations (>= 0), at most 32768 adds per flush: 2^15 x 2^17 fits a word
+          const u64 uv = (u64)v[j];
+          atomicAdd(&s.sum[0][slot], (u32)(uv & 0x1FFFF));
+          if (uv >> 17) atomicAdd(&s.sum[1][slot], (u32)((uv >> 17) & 0x1FFFF));
+          if (uv >> 34) atomicAdd(&s.sum[2][slot], (u32)(uv >> 34));
           // 64-bit min/max in shared memory are compare-and-swap loops: skip them unless the
           // value would actually move the extreme (rare once a slot has seen a few records)
           if (~vb > s.minc[slot]) atomicMax(&s.minc[slot], ~vb);
@@ -728,6 +732,11 @@ ta_status ta_run_aggregate(ta_window *h, uint32_t kind_mask, int value_sel, ta_a
   a.per = (a.n_items + a.spread - 1) / a.spread;
   const int64_t blocks = (int64_t)a.spread * a.per;
 
+  auto run_agg = [&]() {
+    if (table) k_agg<true><<<TA_N (unsigned)blocks, AG_THREADS, 0, st>>>(a);
+    else k_agg<false><<<TA_N (unsigned)blocks, AG_THREADS, 0, st>>>(a);
+  };
+
   AggRowOut ro;
   memset(&ro, 0, sizeof(ro));
   ro.tt = h->d_triples; ro.n_pids = n_pids; ro.R = R; ro.min_name = h->min_name;
@@ -765,7 +774,7 @@ ta_status ta_run_aggregate(ta_window *h, uint32_t kind_mask, int value_sel, ta_a
     a.d_hist = ct.take<u32>((size_t)G * TA_NBINS);
     ct.off += scan_temp_carve(ct.base + ct.off, G, &t);
     TA_CHECK_CUDA(h, cudaMemsetAsync(tmpb, 0, ct.off, st));
-    k_agg<<<TA_N (unsigned)blocks, AG_THREADS, 0, st>>>(a);
+    run_agg();
     // the rows are compacted without waiting for their count: it is bounded by cells and records
     carve_rows(G < h->n_valid ? G : h->n_valid);
     if (!outb) return TA_ERR_OOM;
@@ -783,7 +792,8 @@ ta_status ta_run_aggregate(ta_window *h, uint32_t kind_mask, int value_sel, ta_a
     ct.off += scan_temp_carve(ct.base + ct.off, words, &t);
     TA_CHECK_CUDA(h, cudaMemsetAsync(tmpb, 0, ct.off, st));
     u32 *rank = ct.take<u32>(words);
-    k_agg_mark<<<TA_N a.n_items, AG_THREADS, 0, st>>>(a);
+    if (table) k_agg_mark<true><<<TA_N a.n_items, AG_THREADS, 0, st>>>(a);
+    else k_agg_mark<false><<<TA_N a.n_items, AG_THREADS, 0, st>>>(a);
     AggBitsIn bi{a.bits};
     AggBitsOut bo{rank};
     TA_TRY((launch_scan<OpAdd, AggBitsIn, AggBitsOut>(h, words, bi, bo, OpAdd(), t)));
@@ -796,7 +806,7 @@ ta_status ta_run_aggregate(ta_window *h, uint32_t kind_mask, int value_sel, ta_a
       a.rank = rank;
       a.d_cnt = (u64 *)ro.g_count; a.d_sum = (u64 *)ro.g_sum; a.d_minc = (u64 *)ro.g_min; a.d_maxb = (u64 *)ro.g_max;
       a.d_hist = ro.g_hist;
-      k_agg<<<TA_N (unsigned)blocks, AG_THREADS, 0, st>>>(a);
+      run_agg();
       k_agg_marked_rows<<<TA_N (unsigned)((words + 255) / 256), 256, 0, st>>>(a.bits, rank, words, ro, h->d_status);
     }
   }
