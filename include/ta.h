@@ -600,7 +600,8 @@ ta_status ta_critical_path(ta_window *h, ta_critpath_result *out,
  * cudaMalloc / cudaFree inside its callbacks, or a latency-critical loop that
  * cannot afford the device-wide synchronisation an allocation or a free may
  * imply.  Every other entry point obtains its buffers through ta_env; this one
- * obtains nothing: it calls no cudaMalloc, cudaFree or any allocating routine.
+ * obtains no device memory: it calls no cudaMalloc, cudaFree or any routine that
+ * allocates on the device (its first call page-locks a hundred bytes of host memory).
  * Its scratch (tile descriptors of the scan, a counter, a status word: about
  * 16 KB) is a fixed array inside the library image, which every GPU that loads
  * the library holds until the process exits.
@@ -630,6 +631,12 @@ ta_status ta_critical_path(ta_window *h, ta_critpath_result *out,
 ta_status ta_lane_gaps_noalloc(const int64_t *ts_start, const int64_t *ts_end, int64_t n,
                                int64_t win_t0, int64_t win_t1, int64_t *gap_before,
                                ta_lane_gaps *lane_out, void *cuda_stream);
+/* The same, and the row in host memory too (host_row, caller-owned, may be null): it is there
+ * when the call returns, without a copy of its own. */
+ta_status ta_lane_gaps_noalloc_host(const int64_t *ts_start, const int64_t *ts_end, int64_t n,
+                                    int64_t win_t0, int64_t win_t1, int64_t *gap_before,
+                                    ta_lane_gaps *lane_out, ta_lane_gaps *host_row,
+                                    void *cuda_stream);
 
 /* Helpers that carry no work. */
 const char *ta_strerror(ta_status s);

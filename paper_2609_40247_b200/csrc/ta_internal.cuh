@@ -252,6 +252,20 @@ ta_status ta_read_status(ta_window *h, int32_t *host_words /*ST_WORDS*/);
 void ta_dfree_later(ta_window *h, void *p);
 
 
+// Waits until the volatile word `word` (page-locked, written last by the last kernel queued on
+// stream `st`) equals `want`: some microseconds less than a stream synchronisation.  The stream is
+// asked now and then, so a kernel that fails (or returns early and writes nothing) ends the wait:
+// on a CUDA error the enclosing function returns TA_ERR_CUDA; the caller compares once more.
+#define TA_WAIT_SEQ(word, want, st)                                             \
+  do {                                                                          \
+    for (unsigned polls__ = 1; (word) != (want); polls__++) {                   \
+      if (polls__ & 1023u) continue;                                            \
+      const cudaError_t e__ = cudaStreamQuery(st);                              \
+      if (e__ == cudaSuccess) break;                                            \
+      if (e__ != cudaErrorNotReady) { cudaGetLastError(); return TA_ERR_CUDA; } \
+    }                                                                           \
+  } while (0)
+
 // ---- instrumentation (no work: a launch counter and optional event pairs) ----
 extern std::atomic<long long> g_ta_launches;  // kernels launched by this library since load
 extern int g_ta_profile;          // 1 = record a CUDA event pair around each radix pass

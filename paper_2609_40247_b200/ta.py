@@ -12,6 +12,7 @@ CPU fallback: if the library is missing, loading fails with an error.
 """
 from __future__ import annotations
 
+import contextlib
 import ctypes
 import os
 
@@ -99,7 +100,7 @@ _CritpathResult = _ptr_struct("_CritpathResult", [
 EXPORTS = ["ta_load_window", "ta_sort_timeline", "ta_correlate_launches", "ta_attribute_operators",
            "ta_stream_gaps", "ta_aggregate_ops", "ta_match_collectives", "ta_free", "ta_strerror",
            "ta_version", "ta_launch_count", "ta_profile_enable", "ta_profile_radix",
-           "ta_lane_gaps_noalloc", "ta_device_overlap", "ta_blame_gaps",
+           "ta_lane_gaps_noalloc", "ta_lane_gaps_noalloc_host", "ta_device_overlap", "ta_blame_gaps",
            "ta_rollup_operators", "ta_critical_path", "ta_set_spin_limit",
            "ta_selftest_wait_timeout", "ta_inject_device_error", "ta_operator_sol"]
 NOALLOC_MAX_RECORDS = 1 << 22
@@ -157,6 +158,9 @@ def lib():
         L.ta_lane_gaps_noalloc.restype = ctypes.c_int
         L.ta_lane_gaps_noalloc.argtypes = [_vp, _vp, ctypes.c_int64, ctypes.c_int64, ctypes.c_int64,
                                            _vp, _vp, _vp]
+        L.ta_lane_gaps_noalloc_host.restype = ctypes.c_int
+        L.ta_lane_gaps_noalloc_host.argtypes = [_vp, _vp, ctypes.c_int64, ctypes.c_int64, ctypes.c_int64,
+                                                _vp, _vp, _vp, _vp]
         L.ta_launch_count.restype = ctypes.c_int64
         L.ta_set_spin_limit.restype = None
         L.ta_set_spin_limit.argtypes = [ctypes.c_int32]
@@ -197,12 +201,14 @@ def lane_gaps_noalloc(ts_start, ts_end, win_t0: int, win_t1: int, gap_before=Non
     if lane_out is None:
         lane_out = torch.empty(LANE_GAPS.itemsize, dtype=torch.uint8, device=dev)
     s = stream if stream is not None else torch.cuda.current_stream(dev)
-    with torch.cuda.device(dev):
-        st = L.ta_lane_gaps_noalloc(ts_start.data_ptr(), ts_end.data_ptr(), n, int(win_t0), int(win_t1),
-                                    gap_before.data_ptr(), lane_out.data_ptr(), s.cuda_stream)
+    row = np.empty(1, dtype=LANE_GAPS)
+    with contextlib.nullcontext() if torch.cuda.current_device() == dev.index else torch.cuda.device(dev):
+        st = L.ta_lane_gaps_noalloc_host(ts_start.data_ptr(), ts_end.data_ptr(), n, int(win_t0), int(win_t1),
+                                         gap_before.data_ptr(), lane_out.data_ptr(), row.ctypes.data,
+                                         s.cuda_stream)
     if st != 0:
         raise TaError(st, "ta_lane_gaps_noalloc")
-    return gap_before[:n], lane_out.cpu().numpy().view(LANE_GAPS)[0]
+    return gap_before[:n], row[0]
 
 
 def launch_count() -> int:
