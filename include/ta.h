@@ -638,6 +638,30 @@ ta_status ta_lane_gaps_noalloc_host(const int64_t *ts_start, const int64_t *ts_e
                                     ta_lane_gaps *lane_out, ta_lane_gaps *host_row,
                                     void *cuda_stream);
 
+/* ------------------------------------------------------------------------
+ * Helpers around the results and their memory.
+ *
+ * ta_fetch: copies `count` device regions of the handle's results to host memory
+ * (dst[i] <- src[i], bytes[i]) with one synchronisation of env.cuda_stream.
+ * Regions of up to 64 KB are gathered by one kernel.
+ * ta_block_of: the allocation a result pointer of this handle lies in.
+ * ta_chunk_*: an allocator for ta_env that hands out pieces of one block of device
+ * memory the caller has obtained, for callers whose own allocator is expensive
+ * to call (an analysis makes some thirty requests); a request that does not
+ * fit goes to the caller's alloc / release.  Use it as
+ *   env.alloc = ta_chunk_alloc; env.release = ta_chunk_release; env.ctx = ta_chunk_open(...);
+ * one chunk per handle, closed after ta_free; the block itself stays the caller's.
+ */
+ta_status ta_fetch(ta_window *h, int32_t count, void *const *dst, const void *const *src,
+                   const uint64_t *bytes);
+ta_status ta_block_of(ta_window *h, const void *p, void **base, uint64_t *bytes);
+typedef struct ta_chunk ta_chunk;
+ta_chunk *ta_chunk_open(void *base, uint64_t bytes, void *(*alloc)(size_t, void *),
+                        void (*release)(void *, void *), void *ctx);
+void ta_chunk_close(ta_chunk *c);
+void *ta_chunk_alloc(size_t bytes, void *chunk);
+void ta_chunk_release(void *ptr, void *chunk);
+
 /* Helpers that carry no work. */
 const char *ta_strerror(ta_status s);
 int32_t ta_version(void);

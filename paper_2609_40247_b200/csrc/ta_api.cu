@@ -134,7 +134,7 @@ void ta_dfree(ta_window *h, void *p) {
 
 // Page-locked staging blocks are expensive to create (a system call and a page-table update
 // each), so they are kept for the life of the process and handed from handle to handle.
-#define TA_PIN_BYTES (512u << 10)
+#define TA_PIN_BYTES (512u << 10)  // and 64 bytes behind them for the number of the last fetch
 static std::mutex g_pin_guard;
 static std::vector<unsigned char *> g_pin_free;
 static unsigned char *pin_take() {
@@ -147,7 +147,7 @@ static unsigned char *pin_take() {
     }
   }
   void *p = nullptr;
-  if (cudaHostAlloc(&p, TA_PIN_BYTES, cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
+  if (cudaHostAlloc(&p, TA_PIN_BYTES + 64, cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
     cudaGetLastError();
     return nullptr;  // the copies then go straight to their (pageable) destinations
   }
@@ -159,33 +159,54 @@ static void pin_put(unsigned char *p) {
   g_pin_free.push_back(p);
 }
 
-// Writes up to TA_FETCH_MAX small device regions into the mapped staging block: one launch in
-// place of one copy each (a copy costs some six microseconds of stream time, however small).
-#define TA_FETCH_MAX 8
-#define TA_FETCH_BYTES (16u << 10)
+// Writes up to TA_FETCH_MAX device regions into the mapped staging block: one launch in place of
+// one copy each (a copy costs some six microseconds of stream time, however small).  The last CTA
+// to finish writes the number of the fetch behind the data, which the host waits for (seq 0: the
+// fetch is not the last of its call and nobody waits).
+#define TA_FETCH_MAX 16
+#define TA_FETCH_BYTES (64u << 10)
+#define TA_FETCH_STRIPE (8u << 10)  // bytes per CTA
 struct FetchList {
   const void *src[TA_FETCH_MAX];
   unsigned off[TA_FETCH_MAX], bytes[TA_FETCH_MAX];
 };
-__global__ void __launch_bounds__(256) k_collect(FetchList f, unsigned char *pin_dev) {
-  const unsigned char *s = (const unsigned char *)f.src[blockIdx.x];
-  unsigned char *d = pin_dev + f.off[blockIdx.x];
-  const unsigned b = f.bytes[blockIdx.x];
-  if ((((uintptr_t)s | (uintptr_t)b) & 7u) == 0) {
-    for (unsigned i = threadIdx.x; i < b / 8; i += blockDim.x)
-      reinterpret_cast<u64 *>(d)[i] = reinterpret_cast<const u64 *>(s)[i];
-  } else {
-    for (unsigned i = threadIdx.x; i < b; i += blockDim.x) d[i] = s[i];
+__global__ void __launch_bounds__(256) k_collect(FetchList f, int m, unsigned char *pin_dev, u32 *ticket, u32 seq,
+                                                 volatile u32 *seq_word) {
+  const unsigned lo = blockIdx.x * TA_FETCH_STRIPE;
+  for (int e = 0; e < m; e++) {
+    const unsigned b = f.bytes[e];
+    if (lo >= b) continue;
+    const unsigned hi = min(b, lo + TA_FETCH_STRIPE);
+    const unsigned char *s = (const unsigned char *)f.src[e];
+    unsigned char *d = pin_dev + f.off[e];
+    if ((((uintptr_t)s | (uintptr_t)b) & 7u) == 0) {
+      for (unsigned i = lo / 8 + threadIdx.x; i < hi / 8; i += blockDim.x)
+        reinterpret_cast<u64 *>(d)[i] = reinterpret_cast<const u64 *>(s)[i];
+    } else {
+      for (unsigned i = lo + threadIdx.x; i < hi; i += blockDim.x) d[i] = s[i];
+    }
   }
+  if (!seq) return;
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  __threadfence_system();
+  if (gridDim.x > 1 && atomicInc(ticket, gridDim.x - 1) != gridDim.x - 1) return;  // (wraps back to 0)
+  __threadfence_system();
+  *seq_word = seq;
 }
-static ta_status flush_fetch(ta_window *h) {
+static ta_status flush_fetch(ta_window *h, u32 seq) {
   if (h->fetch.empty()) return TA_OK;
   FetchList f;
   memset(&f, 0, sizeof(f));
   const unsigned m = (unsigned)h->fetch.size();
-  for (unsigned i = 0; i < m; i++) { f.src[i] = h->fetch[i].src; f.off[i] = h->fetch[i].off; f.bytes[i] = h->fetch[i].bytes; }
+  unsigned most = 1;
+  for (unsigned i = 0; i < m; i++) {
+    f.src[i] = h->fetch[i].src; f.off[i] = h->fetch[i].off; f.bytes[i] = h->fetch[i].bytes;
+    most = f.bytes[i] > most ? f.bytes[i] : most;
+  }
   h->fetch.clear();
-  k_collect<<<TA_N m, 256, 0, h->stream>>>(f, h->pin_dev);
+  k_collect<<<TA_N (most + TA_FETCH_STRIPE - 1) / TA_FETCH_STRIPE, 256, 0, h->stream>>>(
+      f, (int)m, h->pin_dev, (u32 *)&h->d_status[ST_TICKET], seq, (volatile u32 *)(h->pin_dev + TA_PIN_BYTES));
   TA_CHECK_CUDA(h, cudaGetLastError());
   return TA_OK;
 }
@@ -194,7 +215,7 @@ ta_status ta_queue_d2h(ta_window *h, void *dst, const void *dev_src, size_t byte
   if (bytes == 0) return TA_OK;
   const size_t need = (bytes + 15) & ~(size_t)15;
   if (h->pin_dev && bytes <= TA_FETCH_BYTES && h->pin_used + need <= h->pin_bytes) {
-    if (h->fetch.size() == TA_FETCH_MAX) TA_TRY(flush_fetch(h));
+    if (h->fetch.size() == TA_FETCH_MAX) TA_TRY(flush_fetch(h, 0));
     h->fetch.push_back(ta_window::Fetch{dev_src, (unsigned)h->pin_used, (unsigned)bytes});
     h->pending.push_back(ta_window::Pending{dst, h->pin_used, bytes});
     h->pin_used += need;
@@ -208,20 +229,27 @@ ta_status ta_queue_d2h(ta_window *h, void *dst, const void *dev_src, size_t byte
   return TA_OK;
 }
 
-static void release_one(ta_window *h, void *p, size_t bytes);
-
+static ta_status wait_fetch(ta_window *h) {
+  if (h->fetch.empty()) {
+    TA_CHECK_CUDA(h, cudaStreamSynchronize(h->stream));
+    return TA_OK;
+  }
+  volatile u32 *word = (volatile u32 *)(h->pin + TA_PIN_BYTES);
+  const u32 seq = ++h->fetch_seq ? h->fetch_seq : ++h->fetch_seq;
+  *word = 0;
+  TA_TRY(flush_fetch(h, seq));
+  TA_WAIT_SEQ(*word, seq, h->stream);
+  if (*word != seq) TA_CHECK_CUDA(h, cudaStreamSynchronize(h->stream));
+  std::atomic_thread_fence(std::memory_order_acquire);
+  return *word == seq ? TA_OK : TA_ERR_CUDA;
+}
 ta_status ta_sync_fetch(ta_window *h) {
-  const ta_status fs = flush_fetch(h);
-  if (fs != TA_OK) { h->pending.clear(); h->pin_used = 0; return fs; }
-  const cudaError_t e = cudaStreamSynchronize(h->stream);
-  if (e == cudaSuccess)
+  const ta_status fs = wait_fetch(h);
+  if (fs == TA_OK)
     for (const ta_window::Pending &q : h->pending) memcpy(q.dst, h->pin + q.off, q.bytes);
   h->pending.clear();
   h->pin_used = 0;
-  if (e != cudaSuccess) {
-    h->last_cuda = e;
-    return TA_ERR_CUDA;
-  }
+  if (fs != TA_OK) return fs;
   for (void *p : h->deferred) ta_dfree(h, p);
   h->deferred.clear();
   return TA_OK;
@@ -506,6 +534,7 @@ ta_status ta_load_window(const ta_env *env, const ta_event *events, int64_t n,
     else cudaGetLastError();
   }
   h->pin_used = 0;
+  h->fetch_seq = 0;
   h->h_off.assign(win_off, win_off + W + 1);
   h->h_t0.assign(win_t0, win_t0 + W);
   h->h_t1.assign(win_t1, win_t1 + W);
@@ -611,6 +640,88 @@ ta_status ta_device_overlap(ta_window *h, ta_overlap_result *out) {
   if (!(h->stage & 2)) return TA_ERR_ORDER;
   TA_TRY(begin_call(h));
   return ta_run_overlap(h, out);
+}
+
+ta_status ta_fetch(ta_window *h, int32_t count, void *const *dst, const void *const *src, const uint64_t *bytes) {
+  if (!h || count < 0 || (count > 0 && (!dst || !src || !bytes))) return TA_ERR_INVALID_ARG;
+  TA_TRY(begin_call(h));
+  for (int32_t i = 0; i < count; i++) TA_TRY(ta_queue_d2h(h, dst[i], src[i], (size_t)bytes[i]));
+  return ta_sync_fetch(h);
+}
+
+ta_status ta_block_of(ta_window *h, const void *p, void **base, uint64_t *bytes) {
+  if (!h || !base || !bytes) return TA_ERR_INVALID_ARG;
+  for (size_t i = 0; i < h->allocs.size(); i++) {
+    const char *b = (const char *)h->allocs[i];
+    if ((const char *)p >= b && (const char *)p < b + h->alloc_bytes[i]) {
+      *base = h->allocs[i];
+      *bytes = h->alloc_bytes[i];
+      return TA_OK;
+    }
+  }
+  return TA_ERR_INVALID_ARG;
+}
+
+// ---- a chunk of the caller's memory handed out piece by piece ----
+struct ta_chunk {
+  char *base;
+  size_t bytes;
+  void *(*alloc)(size_t, void *);
+  void (*release)(void *, void *);
+  void *ctx;
+  struct Piece { size_t off, bytes; bool used; };
+  std::vector<Piece> pieces;  // in address order, covering the chunk; free neighbours are merged
+};
+ta_chunk *ta_chunk_open(void *base, uint64_t bytes, void *(*alloc)(size_t, void *), void (*release)(void *, void *),
+                        void *ctx) {
+  if (!base || !alloc || !release) return nullptr;
+  ta_chunk *c = new (std::nothrow) ta_chunk();
+  if (!c) return nullptr;
+  c->base = (char *)base;
+  c->bytes = (size_t)bytes;
+  c->alloc = alloc;
+  c->release = release;
+  c->ctx = ctx;
+  c->pieces.push_back(ta_chunk::Piece{0, (size_t)bytes & ~(size_t)255, false});
+  return c;
+}
+void ta_chunk_close(ta_chunk *c) { delete c; }
+void *ta_chunk_alloc(size_t bytes, void *chunk) {
+  ta_chunk *c = (ta_chunk *)chunk;
+  const size_t need = Carver::pad(bytes ? bytes : 1);
+  size_t best = c->pieces.size();
+  for (size_t i = 0; i < c->pieces.size(); i++)
+    if (!c->pieces[i].used && c->pieces[i].bytes >= need &&
+        (best == c->pieces.size() || c->pieces[i].bytes < c->pieces[best].bytes))
+      best = i;
+  if (best == c->pieces.size()) return c->alloc(bytes, c->ctx);
+  ta_chunk::Piece &p = c->pieces[best];
+  const size_t off = p.off, rest = p.bytes - need;
+  p.bytes = need;
+  p.used = true;
+  if (rest) c->pieces.insert(c->pieces.begin() + best + 1, ta_chunk::Piece{off + need, rest, false});
+  return c->base + off;
+}
+void ta_chunk_release(void *ptr, void *chunk) {
+  ta_chunk *c = (ta_chunk *)chunk;
+  if ((char *)ptr < c->base || (char *)ptr >= c->base + c->bytes) {
+    c->release(ptr, c->ctx);
+    return;
+  }
+  const size_t off = (size_t)((char *)ptr - c->base);
+  for (size_t i = 0; i < c->pieces.size(); i++) {
+    if (c->pieces[i].off != off || !c->pieces[i].used) continue;
+    c->pieces[i].used = false;
+    if (i + 1 < c->pieces.size() && !c->pieces[i + 1].used) {
+      c->pieces[i].bytes += c->pieces[i + 1].bytes;
+      c->pieces.erase(c->pieces.begin() + i + 1);
+    }
+    if (i > 0 && !c->pieces[i - 1].used) {
+      c->pieces[i - 1].bytes += c->pieces[i].bytes;
+      c->pieces.erase(c->pieces.begin() + i);
+    }
+    return;
+  }
 }
 
 void ta_free(ta_window *h) {

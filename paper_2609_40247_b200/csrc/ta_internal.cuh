@@ -29,8 +29,9 @@ typedef unsigned int u32;
 
 // device status word indices (h->d_status)
 // ST_SPIN: polls a device-side wait may make before it gives up (0 = TA_SPIN_LIMIT)
+// ST_TICKET: counts the CTAs of k_collect that are done (wraps back to 0 by itself)
 enum { ST_ERR = 0, ST_LONG_RUN = 1, ST_N_TRIPLES = 2, ST_N_PIDS = 3, ST_N_COMMS = 4, ST_SPIN = 5,
-       ST_WORDS = 16 };
+       ST_TICKET = 15, ST_WORDS = 16 };
 
 struct TripleTable {       // device-resident, filled by the discovery kernel
   u64 slots[TA_TRIPLE_SLOTS];          // biased code or EMPTY
@@ -103,6 +104,7 @@ struct ta_window {
   unsigned char *pin_dev;  // device address of `pin`, null when the block is not mapped
   struct Fetch { const void *src; unsigned off, bytes; };
   std::vector<Fetch> fetch;
+  u32 fetch_seq;  // number of the last fetch somebody waited for
 
   // load products
   int32_t *d_status;

@@ -102,7 +102,8 @@ EXPORTS = ["ta_load_window", "ta_sort_timeline", "ta_correlate_launches", "ta_at
            "ta_version", "ta_launch_count", "ta_profile_enable", "ta_profile_radix",
            "ta_lane_gaps_noalloc", "ta_lane_gaps_noalloc_host", "ta_device_overlap", "ta_blame_gaps",
            "ta_rollup_operators", "ta_critical_path", "ta_set_spin_limit",
-           "ta_selftest_wait_timeout", "ta_inject_device_error", "ta_operator_sol"]
+           "ta_selftest_wait_timeout", "ta_inject_device_error", "ta_operator_sol", "ta_fetch",
+           "ta_block_of", "ta_chunk_open", "ta_chunk_close", "ta_chunk_alloc", "ta_chunk_release"]
 NOALLOC_MAX_RECORDS = 1 << 22
 
 _lib = None
@@ -173,6 +174,16 @@ def lib():
         L.ta_profile_radix.restype = ctypes.c_int32
         L.ta_profile_radix.argtypes = [ctypes.POINTER(ctypes.c_int64), ctypes.POINTER(ctypes.c_double),
                                        ctypes.POINTER(ctypes.c_double)]
+        L.ta_fetch.restype = ctypes.c_int
+        L.ta_fetch.argtypes = [_vp, ctypes.c_int32, _vp, _vp, _vp]
+        L.ta_block_of.restype = ctypes.c_int
+        L.ta_block_of.argtypes = [_vp, _vp, ctypes.POINTER(_vp), ctypes.POINTER(ctypes.c_uint64)]
+        L.ta_chunk_open.restype = _vp
+        L.ta_chunk_open.argtypes = [_vp, ctypes.c_uint64, _ALLOC_T, _RELEASE_T, _vp]
+        L.ta_chunk_close.restype = None
+        L.ta_chunk_close.argtypes = [_vp]
+        L.chunk_alloc = ctypes.cast(L.ta_chunk_alloc, _ALLOC_T)
+        L.chunk_release = ctypes.cast(L.ta_chunk_release, _RELEASE_T)
         _lib = L
     return _lib
 
@@ -204,7 +215,7 @@ def lane_gaps_noalloc(ts_start, ts_end, win_t0: int, win_t1: int, gap_before=Non
     row = np.empty(1, dtype=LANE_GAPS)
     with contextlib.nullcontext() if torch.cuda.current_device() == dev.index else torch.cuda.device(dev):
         st = L.ta_lane_gaps_noalloc_host(ts_start.data_ptr(), ts_end.data_ptr(), n, int(win_t0), int(win_t1),
-                                         gap_before.data_ptr(), lane_out.data_ptr(), row.ctypes.data,
+                                         gap_before.data_ptr(), lane_out.data_ptr(), _addr(row),
                                          s.cuda_stream)
     if st != 0:
         raise TaError(st, "ta_lane_gaps_noalloc")
@@ -244,6 +255,75 @@ def profile_radix():
     return n.value, ms.value, nb.value
 
 
+def _addr(a):
+    """Address of a numpy array's data (a third of the time .ctypes.data takes)."""
+    return a.__array_interface__["data"][0]
+
+
+# torch's caching allocator behind the ta_env callbacks: one pair of callbacks for all windows, the
+# context says which device and stream
+_places: list = [None]
+_place_of: dict = {}
+
+
+@_ALLOC_T
+def _torch_alloc(size, ctx):
+    import torch
+    try:
+        return torch.cuda.caching_allocator_alloc(int(size), *_places[ctx])
+    except Exception:
+        return None
+
+
+@_RELEASE_T
+def _torch_release(ptr, ctx):
+    import torch
+    torch.cuda.caching_allocator_delete(ptr)
+
+
+def _place(device, stream_ptr):
+    key = (device, stream_ptr)
+    at = _place_of.get(key)
+    if at is None:
+        _places.append(key)
+        at = _place_of[key] = len(_places) - 1
+    return at
+
+
+# An analysis makes some thirty requests for memory, each a call from C into Python.  Windows of up
+# to CHUNK_RECORDS records take one block up front, sized for the results and temporaries of the
+# seven calls, and the library hands out pieces of it; what does not fit is requested as before.
+CHUNK_RECORDS = 1 << 24
+CHUNK_BYTES_PER_RECORD = 176
+CHUNK_BYTES_FIXED = 4 << 20
+
+
+class _Handle:
+    """The C handle, its memory, and what the library borrows: everything a result needs to stay
+    valid.  Windows, results and the tensors made from them refer to it; it refers to none of them."""
+
+    def __init__(self, L, device):
+        self.lib, self.device = L, device
+        self.ptr = _vp()
+        self.chunk = self.block = None
+        self.callbacks = None
+
+    def close(self):
+        if self.ptr:
+            self.lib.ta_free(self.ptr)
+            self.ptr = _vp()
+        if self.chunk:
+            self.lib.ta_chunk_close(self.chunk)
+            _torch_release(self.block, None)
+            self.chunk = self.block = None
+
+    def __del__(self):
+        try:
+            self.close()
+        except Exception:
+            pass
+
+
 class _DevView:
     """Exposes a raw device range to torch through __cuda_array_interface__."""
 
@@ -253,42 +333,101 @@ class _DevView:
                                          "data": (int(ptr), False), "version": 2}
 
 
+class _Blocks:
+    """Tensors over the allocations of a handle; results are slices of them (making a tensor from
+    an address takes three times as long as slicing one)."""
+
+    def __init__(self, handle):
+        self.handle = handle
+        self.known = []  # (first address, address behind, tensor)
+
+    def slice(self, ptr, nbytes):
+        for lo, hi, t in self.known:
+            if lo <= ptr and ptr + nbytes <= hi:
+                return t[ptr - lo:ptr - lo + nbytes]
+        import torch
+        h = self.handle
+        if h.block is not None and h.block <= ptr < h.block + h.block_bytes:
+            lo, size = h.block, h.block_bytes
+        else:
+            base, room = _vp(), ctypes.c_uint64()
+            if h.lib.ta_block_of(h.ptr, ptr, ctypes.byref(base), ctypes.byref(room)) != 0:
+                raise ValueError("not a result of an open window")
+            lo, size = base.value, room.value
+        t = torch.as_tensor(_DevView(lo, size, h), device=f"cuda:{h.device}")
+        self.known.append((lo, lo + size, t))
+        return t[ptr - lo:ptr - lo + nbytes]
+
+
 class _Result:
     """Device pointers owned by the window handle, with typed access."""
     _layout: dict = {}
+    _names: dict = {}
+    _table: dict = {}  # name -> (field of the C struct, numpy type, bytes per element, count)
+
+    def __init_subclass__(cls):
+        cls._table = {k: (k, np.dtype(dt), np.dtype(dt).itemsize, count) for k, (dt, count) in cls._layout.items()}
+        cls._table.update({alias: cls._table[k] for alias, k in cls._names.items()})
 
     def __init__(self, window, raw, extra=None):
-        self._w = window
+        self._handle = window._handle
+        self._blocks = window._blocks
         self._raw = raw
+        self._host = {}
         self.__dict__.update(extra or {})
-
-    def _spec(self, name):
-        dt, count = self._layout[name]
-        cnt = count(self) if callable(count) else count
-        return np.dtype(dt), int(cnt)
 
     def tensor(self, name):
         """Zero-copy torch view (uint8 for struct arrays) of a device result; valid while
         the window is open."""
-        import torch
-        dt, cnt = self._spec(name)
-        ptr = getattr(self._raw, name)
-        nbytes = cnt * dt.itemsize
+        field, _, size, count = self._table[name]
+        nbytes = count(self) * size
+        ptr = getattr(self._raw, field)
         if nbytes == 0 or not ptr:
-            return torch.empty(0, dtype=torch.uint8, device=f"cuda:{self._w.device}")
-        return torch.as_tensor(_DevView(ptr, nbytes, self._w), device=f"cuda:{self._w.device}")
+            import torch
+            return torch.empty(0, dtype=torch.uint8, device=f"cuda:{self._handle.device}")
+        return self._blocks.slice(ptr, nbytes)
+
+    # Tables are mostly read together: a request for one brings the other small ones of the result
+    # along (a round trip costs more than their bytes), up to these limits.
+    _FETCH_EACH, _FETCH_ALL, _FETCH_COUNT = 64 << 10, 256 << 10, 16
+
+    def _fetch(self, name):
+        names, sizes, total = [], [], 0
+        for k in (name, *self._layout):
+            field, _, size, count = self._table[k]
+            if k != name and (k == self._table[name][0] or k in self._host):
+                continue
+            b = count(self) * size
+            if k == name or (b <= self._FETCH_EACH and total + b <= self._FETCH_ALL and len(names) < self._FETCH_COUNT):
+                names.append(k)
+                sizes.append(b)
+                total += (b + 15) & ~15
+        buf = np.empty(total, dtype=np.uint8)
+        m, at, base = len(names), 0, _addr(buf)
+        dst, src, num = (ctypes.c_void_p * m)(), (ctypes.c_void_p * m)(), (ctypes.c_uint64 * m)()
+        for i, (k, b) in enumerate(zip(names, sizes)):
+            field, dt, _, _ = self._table[k]
+            dst[i], src[i], num[i] = base + at, getattr(self._raw, field), b
+            self._host[field] = buf[at:at + b].view(dt)
+            at += (b + 15) & ~15
+        st = self._handle.lib.ta_fetch(self._handle.ptr, m, dst, src, num)
+        if st != 0:
+            self._host.clear()
+            raise TaError(st, "ta_fetch")
 
     def numpy(self, name):
-        if name in self.__dict__ and isinstance(self.__dict__[name], np.ndarray):
-            return self.__dict__[name]
-        dt, cnt = self._spec(name)
-        if cnt == 0:
+        got = self.__dict__.get(name)
+        if isinstance(got, np.ndarray):
+            return got
+        field, dt, _, count = self._table[name]
+        if count(self) == 0 or not getattr(self._raw, field):
             out = np.empty(0, dtype=dt)
         else:
-            import torch
-            with torch.cuda.stream(self._w.torch_stream):
-                out = self.tensor(name).cpu().numpy().view(dt).copy()
-        if name.endswith("_hist"):
+            out = self._host.pop(field, None)
+            if out is None:
+                self._fetch(name)
+                out = self._host.pop(field)
+        if field.endswith("_hist"):
             out = out.reshape(-1, NBINS)
         return out
 
@@ -350,12 +489,6 @@ class CollResult(_Result):
                "r_max_wait": ("<i8", lambda r: r.n_ranks),
                "r_n_straggler": ("<i8", lambda r: r.n_ranks)}
 
-    def numpy(self, name):
-        return super().numpy(self._names.get(name, name))
-
-    def tensor(self, name):
-        return super().tensor(self._names.get(name, name))
-
 
 ROLLUP_SUM = np.dtype([(k, "<i8") for k in ("n_graph_launches", "n_graph_kernels",
                                             "max_kernels_per_launch")])
@@ -395,10 +528,7 @@ class CritpathResult(_Result):
             s = self.critpath_sum
             return np.concatenate([s["n_paths"][:, None], s["n_nodes"][:, None], s["ns"]],
                                   axis=1).astype(np.int64).reshape(-1)
-        return super().numpy(self._names.get(name, name))
-
-    def tensor(self, name):
-        return super().tensor(self._names.get(name, name))
+        return super().numpy(name)
 
 
 BLAME_SUM = np.dtype([("count", "<i8", (4,)), ("ns", "<i8", (4,))])
@@ -414,10 +544,7 @@ class BlameResult(_Result):
             return self.blame_sum["count"].astype(np.int64).reshape(-1, 4)
         if name == "b_win_ns":
             return self.blame_sum["ns"].astype(np.int64).reshape(-1, 4)
-        return super().numpy(self._names.get(name, name))
-
-    def tensor(self, name):
-        return super().tensor(self._names.get(name, name))
+        return super().numpy(name)
 
 
 SOL_SUM = np.dtype([("n_resolved", "<i8"), ("n_no_kernels", "<i8"), ("n_no_counts", "<i8"),
@@ -435,10 +562,7 @@ class SolResult(_Result):
     def numpy(self, name):
         if name == "sol_sum":
             return self.sol_sum
-        return super().numpy(self._names.get(name, name))
-
-    def tensor(self, name):
-        return super().tensor(self._names.get(name, name))
+        return super().numpy(name)
 
 
 class OverlapResult(_Result):
@@ -459,7 +583,6 @@ class Window:
         import torch
         L = lib()
         self._lib = L
-        self._h = _vp()
         on_device = hasattr(events, "is_cuda")
         if on_device:
             if not events.is_cuda or not events.is_contiguous():
@@ -470,7 +593,7 @@ class Window:
         else:
             events = np.ascontiguousarray(events)
             nbytes = events.nbytes
-            ev_ptr = events.ctypes.data
+            ev_ptr = _addr(events)
             device = torch.cuda.current_device() if device is None else device
         if nbytes % 40:
             raise ValueError("events must hold whole 40-byte records")
@@ -485,6 +608,30 @@ class Window:
         if len(self._off) != self.W + 1 or len(self._t1) != self.W:
             raise ValueError("win_off needs W+1 entries, win_t0 / win_t1 W entries")
         dev, sptr = self.device, self.torch_stream.cuda_stream
+        self._handle = h = _Handle(L, dev)
+        self._blocks = _Blocks(h)
+        env = _Env()
+        env.ctx = None
+        if use_torch_allocator:
+            if alloc_fn is not None or release_fn is not None:
+                self._caller_memory(env, alloc_fn, release_fn, dev, sptr)
+            else:
+                env.alloc, env.release, env.ctx = _torch_alloc, _torch_release, _place(dev, sptr)
+                if self.n <= CHUNK_RECORDS:
+                    self._take_chunk(env)
+        env.cuda_stream = sptr
+        env.device = dev
+        self.load_summary = np.zeros(self.W, dtype=LOAD_SUM)
+        st = L.ta_load_window(ctypes.byref(env), ev_ptr, self.n, 1 if on_device else 0,
+                              _addr(self._off), _addr(self._t0), _addr(self._t1),
+                              self.W, _addr(self.load_summary), ctypes.byref(h.ptr))
+        if st != 0:
+            self.close()
+            raise TaError(st, "ta_load_window")
+        self._sorted = None
+
+    def _caller_memory(self, env, alloc_fn, release_fn, dev, sptr):
+        import torch
 
         def _alloc(size, ctx):
             try:
@@ -500,47 +647,33 @@ class Window:
             else:
                 torch.cuda.caching_allocator_delete(ptr)
 
-        self._alloc_cb = _ALLOC_T(_alloc)
-        self._release_cb = _RELEASE_T(_release)
-        env = _Env()
-        if use_torch_allocator:
-            env.alloc, env.release = self._alloc_cb, self._release_cb
-        env.ctx = None
-        env.cuda_stream = sptr
-        env.device = dev
-        self._env = env
-        self.load_summary = np.zeros(self.W, dtype=LOAD_SUM)
-        st = L.ta_load_window(ctypes.byref(env), ev_ptr, self.n, 1 if on_device else 0,
-                              self._off.ctypes.data, self._t0.ctypes.data, self._t1.ctypes.data,
-                              self.W, self.load_summary.ctypes.data, ctypes.byref(self._h))
-        if st != 0:
-            self.close()
-            raise TaError(st, "ta_load_window")
-        self._sorted = None
+        self._handle.callbacks = env.alloc, env.release = _ALLOC_T(_alloc), _RELEASE_T(_release)
+
+    def _take_chunk(self, env):
+        h = self._handle
+        size = CHUNK_BYTES_FIXED + self.n * CHUNK_BYTES_PER_RECORD
+        block = _torch_alloc(size, env.ctx)
+        if not block:
+            return
+        h.chunk = h.lib.ta_chunk_open(block, size, _torch_alloc, _torch_release, env.ctx)
+        h.block, h.block_bytes = block, size
+        env.alloc, env.release, env.ctx = h.lib.chunk_alloc, h.lib.chunk_release, h.chunk
 
     def inject_device_error(self, code: int) -> None:
         """Test hook: marks the handle as failed, as a device-side wait that gave up would."""
-        st = self._lib.ta_inject_device_error(self._h, int(code))
+        st = self._lib.ta_inject_device_error(self._handle.ptr, int(code))
         if st != 0:
             raise TaError(st, "ta_inject_device_error")
 
     # -- context manager / lifetime
     def close(self):
-        if self._h:
-            self._lib.ta_free(self._h)
-            self._h = _vp()
+        self._handle.close()
 
     def __enter__(self):
         return self
 
     def __exit__(self, *exc):
         self.close()
-
-    def __del__(self):
-        try:
-            self.close()
-        except Exception:
-            pass
 
     def _dims(self):
         s = self._sorted
@@ -549,7 +682,7 @@ class Window:
     # -- the seven calls
     def sort_timeline(self) -> SortResult:
         raw = _SortResult()
-        st = self._lib.ta_sort_timeline(self._h, ctypes.byref(raw))
+        st = self._lib.ta_sort_timeline(self._handle.ptr, ctypes.byref(raw))
         if st != 0:
             raise TaError(st, "ta_sort_timeline")
         self._sorted = SortResult(self, raw, {"n": raw.n, "n_valid": raw.n_valid,
@@ -560,7 +693,7 @@ class Window:
     def correlate_launches(self) -> JoinResult:
         raw = _JoinResult()
         summ = np.zeros(self.W, dtype=JOIN_SUM)
-        st = self._lib.ta_correlate_launches(self._h, ctypes.byref(raw), summ.ctypes.data)
+        st = self._lib.ta_correlate_launches(self._handle.ptr, ctypes.byref(raw), _addr(summ))
         if st != 0:
             raise TaError(st, "ta_correlate_launches")
         return JoinResult(self, raw, dict(self._dims(), join_sum=summ))
@@ -570,21 +703,21 @@ class Window:
         (see .status); the summaries are valid, the other outputs unspecified."""
         raw = _AttrResult()
         summ = np.zeros(self.W, dtype=ATTR_SUM)
-        st = self._lib.ta_attribute_operators(self._h, ctypes.byref(raw), summ.ctypes.data)
+        st = self._lib.ta_attribute_operators(self._handle.ptr, ctypes.byref(raw), _addr(summ))
         if st != 0 and (check or st not in (TA_ERR_DEPTH, TA_ERR_BAD_NESTING)):
             raise TaError(st, "ta_attribute_operators")
         return AttrResult(self, raw, dict(self._dims(), attr_sum=summ, status=st))
 
     def stream_gaps(self, min_gap_ns: int) -> GapResult:
         raw = _GapResult()
-        st = self._lib.ta_stream_gaps(self._h, int(min_gap_ns), ctypes.byref(raw))
+        st = self._lib.ta_stream_gaps(self._handle.ptr, int(min_gap_ns), ctypes.byref(raw))
         if st != 0:
             raise TaError(st, "ta_stream_gaps")
         return GapResult(self, raw, dict(self._dims(), n_long_gaps=raw.n_long_gaps))
 
     def aggregate_ops(self, kind_mask: int, value_sel: int) -> AggResult:
         raw = _AggResult()
-        st = self._lib.ta_aggregate_ops(self._h, kind_mask, value_sel, ctypes.byref(raw))
+        st = self._lib.ta_aggregate_ops(self._handle.ptr, kind_mask, value_sel, ctypes.byref(raw))
         if st != 0:
             raise TaError(st, "ta_aggregate_ops")
         return AggResult(self, raw, dict(self._dims(), n_groups=raw.n_groups))
@@ -592,7 +725,7 @@ class Window:
     def rollup_operators(self) -> RollupResult:
         raw = _RollupResult()
         summ = np.zeros(self.W, dtype=ROLLUP_SUM)
-        st = self._lib.ta_rollup_operators(self._h, ctypes.byref(raw), summ.ctypes.data)
+        st = self._lib.ta_rollup_operators(self._handle.ptr, ctypes.byref(raw), _addr(summ))
         if st != 0:
             raise TaError(st, "ta_rollup_operators")
         return RollupResult(self, raw, dict(self._dims(), rollup_sum=summ))
@@ -600,7 +733,7 @@ class Window:
     def critical_path(self) -> CritpathResult:
         raw = _CritpathResult()
         summ = np.zeros(self.W, dtype=CRITPATH_SUM)
-        st = self._lib.ta_critical_path(self._h, ctypes.byref(raw), summ.ctypes.data)
+        st = self._lib.ta_critical_path(self._handle.ptr, ctypes.byref(raw), _addr(summ))
         if st != 0:
             raise TaError(st, "ta_critical_path")
         return CritpathResult(self, raw, dict(self._dims(), n_rows=raw.n_rows, critpath_sum=summ))
@@ -609,7 +742,7 @@ class Window:
         """gaps: the GapResult of an earlier stream_gaps() call on this window."""
         raw = _BlameResult()
         summ = np.zeros(self.W, dtype=BLAME_SUM)
-        st = self._lib.ta_blame_gaps(self._h, ctypes.byref(gaps._raw), ctypes.byref(raw), summ.ctypes.data)
+        st = self._lib.ta_blame_gaps(self._handle.ptr, ctypes.byref(gaps._raw), ctypes.byref(raw), _addr(summ))
         if st != 0:
             raise TaError(st, "ta_blame_gaps")
         return BlameResult(self, raw, dict(self._dims(), n_long_gaps=raw.n_long_gaps, blame_sum=summ))
@@ -629,18 +762,18 @@ class Window:
         else:
             flops = np.ascontiguousarray(flops, dtype=np.float64)
             nbytes = np.ascontiguousarray(nbytes, dtype=np.float64)
-            fp, bp, cnt = flops.ctypes.data, nbytes.ctypes.data, (len(flops), len(nbytes))
+            fp, bp, cnt = _addr(flops), _addr(nbytes), (len(flops), len(nbytes))
         if cnt != (self.n, self.n):
             raise ValueError("one operation count and one data volume per input record")
-        st = self._lib.ta_operator_sol(self._h, fp, bp, 1 if on_device else 0, float(peak_flops),
-                                       float(peak_bw), ctypes.byref(raw), summ.ctypes.data)
+        st = self._lib.ta_operator_sol(self._handle.ptr, fp, bp, 1 if on_device else 0, float(peak_flops),
+                                       float(peak_bw), ctypes.byref(raw), _addr(summ))
         if st != 0:
             raise TaError(st, "ta_operator_sol")
         return SolResult(self, raw, dict(self._dims(), sol_sum=summ))
 
     def device_overlap(self) -> OverlapResult:
         raw = _OverlapResult()
-        st = self._lib.ta_device_overlap(self._h, ctypes.byref(raw))
+        st = self._lib.ta_device_overlap(self._handle.ptr, ctypes.byref(raw))
         if st != 0:
             raise TaError(st, "ta_device_overlap")
         return OverlapResult(self, raw, dict(self._dims(), n_rows=raw.n_rows))
@@ -650,7 +783,7 @@ class Window:
         for i, (cid, nr) in enumerate(comm_sizes):
             arr[i] = (cid, nr, 0)
         raw = _CollResult()
-        st = self._lib.ta_match_collectives(self._h, arr.ctypes.data if len(arr) else None, len(arr),
+        st = self._lib.ta_match_collectives(self._handle.ptr, _addr(arr) if len(arr) else None, len(arr),
                                             ctypes.byref(raw))
         if st != 0:
             raise TaError(st, "ta_match_collectives")
