@@ -78,6 +78,7 @@ __device__ __forceinline__ u32 name_hash(u32 b) {
 }
 __global__ void __launch_bounds__(256) k_name_set(const int32_t *name, int64_t n_valid, u64 *names, u64 *n_names,
                                                   u64 *list, int32_t *status) {
+  TA_PDL();
   __shared__ u64 cache[2048];  // ids this CTA has seen already (direct mapped, one word each)
   if (ta_failed(status)) return;
   for (int i = threadIdx.x; i < 2048; i += 256) cache[i] = NT_EMPTY;
@@ -119,6 +120,7 @@ __global__ void __launch_bounds__(256) k_name_set(const int32_t *name, int64_t n
 }
 __global__ void __launch_bounds__(256) k_name_rank(const u64 *sorted, int64_t D, u32 *name_rank, int32_t *name_of,
                                                    const int32_t *status) {
+  TA_PDL();
   if (ta_failed(status)) return;
   const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
   if (i >= D) return;
@@ -274,6 +276,7 @@ __device__ __forceinline__ void agg_select(const AggArgs &a, int64_t p0, int64_t
 // sets the bit of every cell that holds a selected record
 template <bool TABLE>
 __global__ void __launch_bounds__(AG_THREADS) k_agg_mark(AggArgs a) {
+  TA_PDL();
   if (ta_failed(a.status)) return;
   LaneWalker lw(a.lane_off, a.n_lanes, a.n_valid, a.n_valid);
   const int64_t begin = (int64_t)blockIdx.x * a.chunk, end = min(begin + a.chunk, a.n_valid);
@@ -302,6 +305,7 @@ __global__ void __launch_bounds__(AG_THREADS) k_agg_mark(AggArgs a) {
 
 template <bool TABLE>
 __global__ void __launch_bounds__(AG_THREADS, 6) k_agg(AggArgs a) {
+  TA_PDL();
   __shared__ AggSmem s;
   if (ta_failed(a.status)) return;
   int since_flush = 0;
@@ -429,6 +433,7 @@ struct AggBitsOut {
 // in order-preserving codes with 0 as "nothing yet")
 __global__ void __launch_bounds__(256) k_agg_marked_rows(const u32 *bits, const u32 *rank, int64_t words,
                                                          AggRowOut o, const int32_t *status) {
+  TA_PDL();
   if (ta_failed(status)) return;
   const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
   if (i >= words) return;
@@ -521,6 +526,7 @@ struct AggSortedOut {
 };
 __global__ void __launch_bounds__(256) k_agg_sorted_rows(AggSortCtx c, const u64 *ks, const int32_t *gstart,
                                                         int64_t ng, AggSortedOut o) {
+  TA_PDL();
   if (ta_failed(c.status)) return;
   const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (g >= ng) return;
@@ -534,6 +540,7 @@ __global__ void __launch_bounds__(256) k_agg_sorted_rows(AggSortCtx c, const u64
 }
 __global__ void __launch_bounds__(256) k_agg_sorted_reduce(AggSortCtx c, const u32 *pos, const int32_t *gid,
                                                           int64_t m, AggSortedOut o) {
+  TA_PDL();
   if (ta_failed(c.status)) return;
   const int64_t j0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 8;
   if (j0 >= m) return;
@@ -636,8 +643,8 @@ static ta_status ta_run_aggregate_sorted(ta_window *h, uint32_t kind_mask, int v
   o.g_count = co.take<int64_t>(ng); o.g_sum = co.take<int64_t>(ng);
   o.g_min = co.take<int64_t>(ng); o.g_max = co.take<int64_t>(ng);
   o.g_hist = co.take<u32>((size_t)ng * TA_NBINS);
-  k_agg_sorted_rows<<<TA_N (unsigned)((ng + 255) / 256), 256, 0, st>>>(c, ks, gstart, ng, o);
-  k_agg_sorted_reduce<<<TA_N (unsigned)((m + 2047) / 2048), 256, 0, st>>>(c, vs, gid, m, o);
+  ta_launch(k_agg_sorted_rows, (unsigned)((ng + 255) / 256), 256, 0, st, c, ks, gstart, ng, o);
+  ta_launch(k_agg_sorted_reduce, (unsigned)((m + 2047) / 2048), 256, 0, st, c, vs, gid, m, o);
   TA_CHECK_CUDA(h, cudaGetLastError());
   int32_t words[ST_WORDS];
   TA_TRY(ta_read_status(h, words));
@@ -669,8 +676,7 @@ static ta_status build_names(ta_window *h) {
   h->d_name_rank = ck.take<u32>(NT_SLOTS);
   h->d_name_of = ck.take<int32_t>(NT_MAX);
   const int64_t want = (h->n_valid + 1023) / 1024;
-  k_name_set<<<TA_N (unsigned)(want < 148 * 8 ? want : 148 * 8), 256, 0, st>>>(h->sorted.name_id, h->n_valid,
-                                                                               h->d_names, count, list, h->d_status);
+  ta_launch(k_name_set, (unsigned)(want < 148 * 8 ? want : 148 * 8), 256, 0, st, h->sorted.name_id, h->n_valid, h->d_names, count, list, h->d_status);
   TA_CHECK_CUDA(h, cudaGetLastError());
   u64 D = 0;
   TA_TRY(ta_queue_d2h(h, &D, count, 8));
@@ -683,8 +689,7 @@ static ta_status build_names(ta_window *h) {
     Carver cs(sb);
     u64 *scr = cs.take<u64>(D), *sorted = cs.take<u64>(D);
     TA_TRY(ta_radix_sort_keys(h, list, scr, sorted, (int64_t)D, ta_make_plan(32, 64), nullptr, cs.base + cs.off, false));
-    k_name_rank<<<TA_N (unsigned)((D + 255) / 256), 256, 0, st>>>(sorted, (int64_t)D, h->d_name_rank, h->d_name_of,
-                                                                  h->d_status);
+    ta_launch(k_name_rank, (unsigned)((D + 255) / 256), 256, 0, st, sorted, (int64_t)D, h->d_name_rank, h->d_name_of, h->d_status);
     TA_CHECK_CUDA(h, cudaGetLastError());
     h->n_names = (int64_t)D;
     ta_dfree_later(h, sb);
@@ -733,8 +738,8 @@ ta_status ta_run_aggregate(ta_window *h, uint32_t kind_mask, int value_sel, ta_a
   const int64_t blocks = (int64_t)a.spread * a.per;
 
   auto run_agg = [&]() {
-    if (table) k_agg<true><<<TA_N (unsigned)blocks, AG_THREADS, 0, st>>>(a);
-    else k_agg<false><<<TA_N (unsigned)blocks, AG_THREADS, 0, st>>>(a);
+    if (table) ta_launch(k_agg<true>, (unsigned)blocks, AG_THREADS, 0, st, a);
+    else ta_launch(k_agg<false>, (unsigned)blocks, AG_THREADS, 0, st, a);
   };
 
   AggRowOut ro;
@@ -792,8 +797,8 @@ ta_status ta_run_aggregate(ta_window *h, uint32_t kind_mask, int value_sel, ta_a
     ct.off += scan_temp_carve(ct.base + ct.off, words, &t);
     TA_CHECK_CUDA(h, cudaMemsetAsync(tmpb, 0, ct.off, st));
     u32 *rank = ct.take<u32>(words);
-    if (table) k_agg_mark<true><<<TA_N a.n_items, AG_THREADS, 0, st>>>(a);
-    else k_agg_mark<false><<<TA_N a.n_items, AG_THREADS, 0, st>>>(a);
+    if (table) ta_launch(k_agg_mark<true>, a.n_items, AG_THREADS, 0, st, a);
+    else ta_launch(k_agg_mark<false>, a.n_items, AG_THREADS, 0, st, a);
     AggBitsIn bi{a.bits};
     AggBitsOut bo{rank};
     TA_TRY((launch_scan<OpAdd, AggBitsIn, AggBitsOut>(h, words, bi, bo, OpAdd(), t)));
@@ -807,7 +812,7 @@ ta_status ta_run_aggregate(ta_window *h, uint32_t kind_mask, int value_sel, ta_a
       a.d_cnt = (u64 *)ro.g_count; a.d_sum = (u64 *)ro.g_sum; a.d_minc = (u64 *)ro.g_min; a.d_maxb = (u64 *)ro.g_max;
       a.d_hist = ro.g_hist;
       run_agg();
-      k_agg_marked_rows<<<TA_N (unsigned)((words + 255) / 256), 256, 0, st>>>(a.bits, rank, words, ro, h->d_status);
+      ta_launch(k_agg_marked_rows, (unsigned)((words + 255) / 256), 256, 0, st, a.bits, rank, words, ro, h->d_status);
     }
   }
   TA_CHECK_CUDA(h, cudaGetLastError());

@@ -107,6 +107,7 @@ __device__ __forceinline__ void wstack_combine(const WStack &ear, WStack &acc, b
 
 // ---- kernel 1: the stack each tile leaves behind --------------------------------
 __global__ void __launch_bounds__(AT_THREADS) k_attr_agg(AttrArgs a) {
+  TA_PDL();
   __shared__ i64 wmax[AT_THREADS / 32];
   __shared__ i64 s_e[AT_CAP];
   __shared__ int32_t s_pos[AT_CAP];
@@ -257,6 +258,7 @@ __device__ __forceinline__ void stack_store(const StackArr &dst, int64_t t, cons
 // parent[j] = child[32j] (+) ... (+) child[32j + 31]
 __global__ void __launch_bounds__(128) k_attr_fold_up(StackArr child, int64_t n_child, StackArr parent,
                                                       int64_t n_parent, int32_t *status) {
+  TA_PDL();
   __shared__ StackStage st;
   if (ta_failed(status)) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -279,6 +281,7 @@ __global__ void __launch_bounds__(128) k_attr_fold_up(StackArr child, int64_t n_
 // one warp: start[i] = node[0] (+) ... (+) node[i - 1] for the few nodes of the top level
 __global__ void __launch_bounds__(32) k_attr_fold_top(StackArr node, int64_t n, StackArr start,
                                                       int leaf, int32_t *status) {
+  TA_PDL();
   if (ta_failed(status)) return;
   const int lane = threadIdx.x & 31;
   bool overflow = false;
@@ -297,6 +300,7 @@ __global__ void __launch_bounds__(32) k_attr_fold_top(StackArr node, int64_t n, 
 __global__ void __launch_bounds__(128) k_attr_fold_down(StackArr child, int64_t n_child,
                                                         StackArr parent_start, int64_t n_parent,
                                                         StackArr child_start, int leaf, int32_t *status) {
+  TA_PDL();
   __shared__ StackStage st;
   if (ta_failed(status)) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -330,6 +334,7 @@ struct __align__(16) AttrSmem {
 };
 
 __global__ void __launch_bounds__(AT_THREADS, AT_RES_MINB) k_attr_resolve(AttrArgs a) {
+  TA_PDL();
   __shared__ AttrSmem s;
   if (ta_failed(a.status)) return;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -616,6 +621,7 @@ __device__ __forceinline__ void attr_emit(ta_attr_summary *sm, const u64 *t) {
   if (t[2]) atomicAdd((u64 *)&sm->n_no_op, t[2]);
 }
 __global__ void __launch_bounds__(AT_THREADS, AT_OPS_MINB) k_attr_ops(AttrArgs a) {
+  TA_PDL();
   constexpr int IT = AT_OPS_ITEMS;
   __shared__ u64 red[3][AT_THREADS / 32];
   __shared__ int s_lane0, s_lane1;
@@ -735,6 +741,7 @@ __global__ void __launch_bounds__(AT_THREADS, AT_OPS_MINB) k_attr_ops(AttrArgs a
 #define AT_FIN_ITEMS 4
 #endif
 __global__ void __launch_bounds__(256) k_attr_finalize(AttrArgs a) {
+  TA_PDL();
   constexpr int IT = AT_FIN_ITEMS;
   const int err = ta_peek_err(a.status);
   const int64_t p0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * IT;
@@ -823,7 +830,7 @@ ta_status ta_run_attribute(ta_window *h, ta_attr_summary *out_summary) {
   a.launch_of = h->join.launch_of; a.kol = h->join.kernels_of_launch; a.op_of = op_of; a.op_n = op_n; a.op_first = op_first;
   a.op_last = op_last; a.op_ns = op_ns;
   if (n > 0) {
-    k_attr_agg<<<TA_N (unsigned)tiles, AT_THREADS, 0, st>>>(a);
+    ta_launch(k_attr_agg, (unsigned)tiles, AT_THREADS, 0, st, a);
     {
       // level 0 = tiles; fold upwards until at most AT_FAN stacks remain, scan those, unfold
       std::vector<StackArr> node(level_n.size()), start(level_n.size());
@@ -836,19 +843,15 @@ ta_status ta_run_attribute(ta_window *h, ta_attr_summary *out_summary) {
       }
       const size_t top = level_n.size() - 1;
       for (size_t k = 1; k <= top; k++)
-        k_attr_fold_up<<<TA_N (unsigned)((level_n[k] + 3) / 4), 128, 0, st>>>(
-            node[k - 1], level_n[k - 1], node[k], level_n[k], h->d_status);
-      k_attr_fold_top<<<TA_N 1, 32, 0, st>>>(node[top], level_n[top], start[top], top == 0 ? 1 : 0,
-                                            h->d_status);
+        ta_launch(k_attr_fold_up, (unsigned)((level_n[k] + 3) / 4), 128, 0, st, node[k - 1], level_n[k - 1], node[k], level_n[k], h->d_status);
+      ta_launch(k_attr_fold_top, 1, 32, 0, st, node[top], level_n[top], start[top], top == 0 ? 1 : 0, h->d_status);
       for (size_t k = top; k >= 1; k--)
-        k_attr_fold_down<<<TA_N (unsigned)((level_n[k] + 3) / 4), 128, 0, st>>>(
-            node[k - 1], level_n[k - 1], start[k], level_n[k], start[k - 1], k == 1 ? 1 : 0,
-            h->d_status);
+        ta_launch(k_attr_fold_down, (unsigned)((level_n[k] + 3) / 4), 128, 0, st, node[k - 1], level_n[k - 1], start[k], level_n[k], start[k - 1], k == 1 ? 1 : 0, h->d_status);
     }
-    k_attr_resolve<<<TA_N (unsigned)tiles, AT_THREADS, 0, st>>>(a);
-    k_attr_ops<<<TA_N (unsigned)((n + AT_OPS_TILE - 1) / AT_OPS_TILE), AT_THREADS, 0, st>>>(a);
+    ta_launch(k_attr_resolve, (unsigned)tiles, AT_THREADS, 0, st, a);
+    ta_launch(k_attr_ops, (unsigned)((n + AT_OPS_TILE - 1) / AT_OPS_TILE), AT_THREADS, 0, st, a);
     const int64_t fb = (h->n_valid + 256 * AT_FIN_ITEMS - 1) / (256 * AT_FIN_ITEMS);
-    k_attr_finalize<<<TA_N (unsigned)(fb > 0 ? fb : 1), 256, 0, st>>>(a);
+    ta_launch(k_attr_finalize, (unsigned)(fb > 0 ? fb : 1), 256, 0, st, a);
     TA_CHECK_CUDA(h, cudaGetLastError());
   }
   std::vector<ta_attr_summary> hs(W);

@@ -44,6 +44,7 @@ struct BlameArgs {
 };
 
 __global__ void __launch_bounds__(256) k_blame_classify(BlameArgs a) {
+  TA_PDL();
   if (ta_failed(a.status)) return;
   const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int lane = threadIdx.x & 31;
@@ -93,6 +94,7 @@ struct GapLenOut {
 
 // lane_first[l] = number of list entries whose lane is < l
 __global__ void __launch_bounds__(256) k_blame_lanes(BlameArgs a) {
+  TA_PDL();
   if (ta_failed(a.status)) return;
   const int l = blockIdx.x * blockDim.x + threadIdx.x;
   if (l > a.n_lanes) return;
@@ -135,6 +137,7 @@ __device__ __forceinline__ i64 gap_time_within(const BlameArgs &a, int64_t first
 }
 
 __global__ void __launch_bounds__(BL_THREADS) k_blame_ops(BlameArgs a) {
+  TA_PDL();
   __shared__ int s_lane0;
   if (ta_failed(a.status)) return;
   const int tid = threadIdx.x;
@@ -228,15 +231,15 @@ ta_status ta_run_blame(ta_window *h, const ta_gap_result *gaps, ta_blame_result 
   a.lane_domain = h->sorted.lane_domain;
   a.g_class = g_class; a.g_launch = g_launch; a.op_gap_ns = op_gap; a.status = h->d_status;
 
-  k_blame_classify<<<TA_N (unsigned)((m + 255) / 256), 256, 0, st>>>(a);
+  ta_launch(k_blame_classify, (unsigned)((m + 255) / 256), 256, 0, st, a);
   ScanTemp s1;
   TA_TRY(scan_temp_init(h, scan_mem, m, &s1));
   GapLenIn gi{a.list};
   GapLenOut go{a.pre};
   TA_TRY((launch_scan<OpAdd, GapLenIn, GapLenOut>(h, m, gi, go, OpAdd(), s1)));
-  k_blame_lanes<<<TA_N (unsigned)((L + 1 + 255) / 256), 256, 0, st>>>(a);
+  ta_launch(k_blame_lanes, (unsigned)((L + 1 + 255) / 256), 256, 0, st, a);
   const int64_t tiles = (h->n_valid + BL_TILE - 1) / BL_TILE;
-  k_blame_ops<<<TA_N (unsigned)tiles, BL_THREADS, 0, st>>>(a);
+  ta_launch(k_blame_ops, (unsigned)tiles, BL_THREADS, 0, st, a);
   TA_CHECK_CUDA(h, cudaGetLastError());
 
   std::vector<u64> hc((size_t)W * 4), hn((size_t)W * 4);

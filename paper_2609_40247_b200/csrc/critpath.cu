@@ -158,6 +158,7 @@ __device__ __forceinline__ int cp_tile_lane(const CpArgs &a, int64_t tile_start,
 
 // ---- keys of the device records ------------------------------------------------------
 __global__ void __launch_bounds__(CP_THREADS) k_cp_keys(CpArgs a) {
+  TA_PDL();
   if (ta_failed(a.status)) return;
   __shared__ int s_lane0;
   const int64_t tile_start = (int64_t)blockIdx.x * CP_TILE;
@@ -185,6 +186,7 @@ __global__ void __launch_bounds__(CP_THREADS) k_cp_keys(CpArgs a) {
 
 // ---- binding dependency of device records, waits of API records ------------------------
 __global__ void __launch_bounds__(CP_THREADS, 3) k_cp_classify(CpArgs a) {
+  TA_PDL();
   if (ta_failed(a.status)) return;
   __shared__ int s_lane0;
   const int64_t tile_start = (int64_t)blockIdx.x * CP_TILE;
@@ -293,6 +295,7 @@ __global__ void __launch_bounds__(CP_THREADS, 3) k_cp_classify(CpArgs a) {
 
 // ---- runs: previous host node, then run heads ------------------------------------------
 __global__ void __launch_bounds__(CP_THREADS) k_cp_runs(CpArgs a) {
+  TA_PDL();
   __shared__ u64 tmp[33];
   __shared__ u64 s_excl;
   __shared__ int s_tile, s_lane0, s_fail;
@@ -436,6 +439,7 @@ __device__ __forceinline__ int32_t cp_follow(const CpArgs &a, int32_t d, bool re
 }
 
 __global__ void __launch_bounds__(256) k_cp_succ(CpArgs a) {
+  TA_PDL();
   if (ta_failed(a.status)) return;
   const int64_t id = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (id >= a.n_list) return;
@@ -444,6 +448,7 @@ __global__ void __launch_bounds__(256) k_cp_succ(CpArgs a) {
 
 // one thread per (window, process): the sink and the hops from it to the first listed wait
 __global__ void __launch_bounds__(64) k_cp_start(CpArgs a) {
+  TA_PDL();
   if (ta_failed(a.status)) return;
   const int64_t slot = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (slot >= a.n_slots) return;
@@ -501,6 +506,7 @@ __global__ void __launch_bounds__(64) k_cp_start(CpArgs a) {
 // one round: what a marked wait reaches is marked (a wait marked during the round may pass its
 // mark on at once - everything it reaches is on the path as well), successors are squared
 __global__ void __launch_bounds__(256) k_cp_double(CpArgs a) {
+  TA_PDL();
   if (ta_failed(a.status)) return;
   const int64_t id = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (id >= a.n_list) return;
@@ -514,6 +520,7 @@ __global__ void __launch_bounds__(256) k_cp_double(CpArgs a) {
 }
 
 __global__ void __launch_bounds__(256) k_cp_enter(CpArgs a) {
+  TA_PDL();
   if (ta_failed(a.status)) return;
   const int64_t id = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (id >= a.n_list || !a.mark[id]) return;
@@ -522,6 +529,7 @@ __global__ void __launch_bounds__(256) k_cp_enter(CpArgs a) {
 
 // ---- membership and time classes ---------------------------------------------------------
 __global__ void __launch_bounds__(CP_THREADS) k_cp_mark(CpArgs a) {
+  TA_PDL();
   if (ta_failed(a.status)) return;
   __shared__ int s_lane0;
   const int lane = threadIdx.x & 31;
@@ -754,7 +762,7 @@ ta_status ta_run_critpath(ta_window *h, ta_critpath_result *out, ta_critpath_sum
       u32 *v_in = cs.take<u32>(mm), *v_scr = cs.take<u32>(mm), *v_fin = cs.take<u32>(mm);
       void *sort_tmp = cs.base + cs.off;
       a.keys = k_in; a.pos = v_in;
-      k_cp_keys<<<TA_N (unsigned)tiles, CP_THREADS, 0, st>>>(a);
+      ta_launch(k_cp_keys, (unsigned)tiles, CP_THREADS, 0, st, a);
       TA_CHECK_CUDA(h, cudaGetLastError());
       if (idxbits) {
         TA_TRY(ta_radix_sort_keys(h, k_in, k_scr, k_fin, m, ta_make_plan(idxbits, idxbits + tsbits + slot_bits),
@@ -767,8 +775,8 @@ ta_status ta_run_critpath(ta_window *h, ta_critpath_result *out, ta_critpath_sum
       }
       a.skeys = k_fin;
     }
-    k_cp_classify<<<TA_N (unsigned)tiles, CP_THREADS, 0, st>>>(a);
-    k_cp_runs<<<TA_N (unsigned)tiles, CP_THREADS, 0, st>>>(a);
+    ta_launch(k_cp_classify, (unsigned)tiles, CP_THREADS, 0, st, a);
+    ta_launch(k_cp_runs, (unsigned)tiles, CP_THREADS, 0, st, a);
     TA_CHECK_CUDA(h, cudaGetLastError());
     // the waits that head a host run: a list whose length decides the number of doubling rounds
     u32 words2[2] = {0, 0};
@@ -788,16 +796,16 @@ ta_status ta_run_critpath(ta_window *h, ta_critpath_result *out, ta_critpath_sum
   a.mark = cl.take<uint8_t>(nl);
   TA_CHECK_CUDA(h, cudaMemsetAsync(a.mark, 0, (size_t)nl, st));
   const unsigned lblocks = (unsigned)((nl + 255) / 256);
-  if (n_list) k_cp_succ<<<TA_N lblocks, 256, 0, st>>>(a);
-  k_cp_start<<<TA_N (unsigned)((n_slots + 63) / 64), 64, 0, st>>>(a);
+  if (n_list) ta_launch(k_cp_succ, lblocks, 256, 0, st, a);
+  ta_launch(k_cp_start, (unsigned)((n_slots + 63) / 64), 64, 0, st, a);
   if (n_list) {
     for (int r = ta_bit_len((uint64_t)n_list); r > 0; r--) {
-      k_cp_double<<<TA_N lblocks, 256, 0, st>>>(a);
+      ta_launch(k_cp_double, lblocks, 256, 0, st, a);
       int32_t *t = a.jump_in; a.jump_in = a.jump_out; a.jump_out = t;
     }
-    k_cp_enter<<<TA_N lblocks, 256, 0, st>>>(a);
+    ta_launch(k_cp_enter, lblocks, 256, 0, st, a);
   }
-  k_cp_mark<<<TA_N (unsigned)tiles, CP_THREADS, 0, st>>>(a);
+  ta_launch(k_cp_mark, (unsigned)tiles, CP_THREADS, 0, st, a);
   TA_CHECK_CUDA(h, cudaGetLastError());
 
   ro.acc = a.acc; ro.tt = h->d_triples; ro.te = a.te; ro.n_pids = n_pids;

@@ -58,6 +58,7 @@ struct GapArgs {
 
 
 __global__ void __launch_bounds__(GP_THREADS, GP_MINB) k_gaps(GapArgs a) {
+  TA_PDL();
   __shared__ u64 tmp[33];
   __shared__ u64 red[4][GP_THREADS / 32];
   __shared__ u64 s_excl_max;
@@ -323,6 +324,7 @@ struct GapBitsOut {
 __global__ void __launch_bounds__(256) k_gap_list_order(const ta_long_gap *src, const u32 *key, const u64 *bits,
                                                         const u32 *rank, int64_t m, ta_long_gap *dst,
                                                         const int32_t *status) {
+  TA_PDL();
   if (ta_failed(status)) return;
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= m) return;
@@ -390,7 +392,7 @@ ta_status ta_run_gaps(ta_window *h, int64_t min_gap, ta_gap_result *out) {
   // first without the scan (every lane is taken to end its records in ascending order, which the
   // kernel checks); if a lane does not, once more with the chained maximum scan
   for (a.local = 1; a.local >= 0; a.local--) {
-    if (tiles > 0) k_gaps<<<TA_N (unsigned)tiles, GP_THREADS, 0, st>>>(a);
+    if (tiles > 0) ta_launch(k_gaps, (unsigned)tiles, GP_THREADS, 0, st, a);
     TA_CHECK_CUDA(h, cudaGetLastError());
     u64 two[3] = {0, 0, 0};
     TA_TRY(ta_queue_d2h(h, two, scal, 24));
@@ -412,7 +414,7 @@ ta_status ta_run_gaps(ta_window *h, int64_t min_gap, ta_gap_result *out) {
     ukeys = cl2.take<u32>(cap);
     TA_CHECK_CUDA(h, cudaMemsetAsync(tb, 0, state_bytes, st));
     a.list = ulist; a.list_key = ukeys; a.list_cap = cap; a.list_only = 1;
-    k_gaps<<<TA_N (unsigned)tiles, GP_THREADS, 0, st>>>(a);
+    ta_launch(k_gaps, (unsigned)tiles, GP_THREADS, 0, st, a);
     TA_CHECK_CUDA(h, cudaGetLastError());
     TA_TRY(ta_read_status(h, words));
     if (words[ST_ERR]) return (ta_status)words[ST_ERR];
@@ -426,7 +428,7 @@ ta_status ta_run_gaps(ta_window *h, int64_t min_gap, ta_gap_result *out) {
     GapBitsIn bi{bits};
     GapBitsOut bo{rank};
     TA_TRY((launch_scan<OpAdd, GapBitsIn, GapBitsOut>(h, n_bits, bi, bo, OpAdd(), scan)));
-    k_gap_list_order<<<TA_N (unsigned)((m + 255) / 256), 256, 0, st>>>(ulist, ukeys, bits, rank, m, list, h->d_status);
+    ta_launch(k_gap_list_order, (unsigned)((m + 255) / 256), 256, 0, st, ulist, ukeys, bits, rank, m, list, h->d_status);
     TA_CHECK_CUDA(h, cudaGetLastError());
     // both kernels are still queued: their temporaries go back after the handle's next
     // synchronisation (the list itself is used in stream order like every other result)

@@ -49,6 +49,7 @@ __device__ __forceinline__ i64 unbias64(u64 v) { return (i64)(v ^ (1ull << 63));
 
 // ---- direct path: fill the table -------------------------------------------
 __global__ void __launch_bounds__(JN_THREADS) k_join_build(JoinArgs a) {
+  TA_PDL();
   __shared__ int s_lane0;
   if (ta_failed(a.status)) return;
   const int tid = threadIdx.x;
@@ -107,6 +108,7 @@ __device__ __forceinline__ void join_emit(ta_join_summary *sm, const u64 *t) {
 
 template <bool DIRECT>
 __global__ void __launch_bounds__(JP_THREADS, JP_MINB) k_join_probe(JoinArgs a) {
+  TA_PDL();
   __shared__ u64 red[7][JP_THREADS / 32];
   __shared__ int s_lane0, s_lane1;
   if (ta_failed(a.status)) return;
@@ -238,6 +240,7 @@ __device__ __forceinline__ void launch_emit(ta_join_summary *sm, const u64 *t) {
 
 template <bool DIRECT>
 __global__ void __launch_bounds__(JP_THREADS) k_join_launch_stats(JoinArgs a) {
+  TA_PDL();
   __shared__ u64 red[3][JP_THREADS / 32];
   __shared__ int s_lane0, s_lane1;
   if (ta_failed(a.status)) return;
@@ -328,6 +331,7 @@ __global__ void __launch_bounds__(JP_THREADS) k_join_launch_stats(JoinArgs a) {
 // ---- general path helpers -----------------------------------------------------
 __global__ void __launch_bounds__(256) k_join_key_corr(const u32 *pos, int64_t m, const int64_t *corr,
                                                        u64 *out, const int32_t *status) {
+  TA_PDL();
   if (ta_failed(status)) return;
   int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (j < m) out[j] = bias64(corr[pos[j]]);
@@ -336,6 +340,7 @@ __global__ void __launch_bounds__(256) k_join_key_slot(const u32 *pos, int64_t m
                                                        const int32_t *lane_off, int n_lanes,
                                                        const int32_t *lane_slot, u64 *out,
                                                        const int32_t *status) {
+  TA_PDL();
   if (ta_failed(status)) return;
   int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (j < m) out[j] = (u64)lane_slot[lane_of_pos(lane_off, n_lanes, pos[j])];
@@ -425,9 +430,9 @@ ta_status ta_run_correlate(ta_window *h, ta_join_summary *out_summary) {
       a.table = (u32 *)tmp_alloc;
       TA_CHECK_CUDA(h, cudaMemsetAsync(a.table, 0xFF, (size_t)(M > 0 ? M : 1) * 4, st));
       TA_CHECK_CUDA(h, cudaMemcpyAsync(slot_base, hbase.data(), n_slots * 8, cudaMemcpyHostToDevice, st));
-      k_join_build<<<TA_N grid, JN_THREADS, 0, st>>>(a);
-      k_join_probe<true><<<TA_N grid_probe, JP_THREADS, 0, st>>>(a);
-      k_join_launch_stats<true><<<TA_N grid8, JP_THREADS, 0, st>>>(a);
+      ta_launch(k_join_build, grid, JN_THREADS, 0, st, a);
+      ta_launch(k_join_probe<true>, grid_probe, JP_THREADS, 0, st, a);
+      ta_launch(k_join_launch_stats<true>, grid8, JP_THREADS, 0, st, a);
     } else {
       // general path: compact, sort by (slot, corr) with sorted position as the stable tie-break
       size_t tb = Carver::pad(nn * 4) * 3 + Carver::pad(nn * 8) * 3 + scan_temp_bytes(n) * 2 +
@@ -454,11 +459,10 @@ ta_status ta_run_correlate(ta_window *h, ta_join_summary *out_summary) {
       if (m > 0) {
         const int gb = (int)((m + 255) / 256);
         u32 *vscr = (u32 *)found;  // found is not needed before the sorts are done
-        k_join_key_corr<<<TA_N gb, 256, 0, st>>>(pos, m, a.corr, k_in, h->d_status);
+        ta_launch(k_join_key_corr, gb, 256, 0, st, pos, m, a.corr, k_in, h->d_status);
         TA_TRY(ta_radix_sort_pairs(h, k_in, pos, k_s, vscr, k_f, pos_s, m, ta_make_plan(0, 64), nullptr,
                                    sort_tmp));
-        k_join_key_slot<<<TA_N gb, 256, 0, st>>>(pos_s, m, a.lane_off, a.n_lanes, a.lane_slot, k_in,
-                                                 h->d_status);
+        ta_launch(k_join_key_slot, gb, 256, 0, st, pos_s, m, a.lane_off, a.n_lanes, a.lane_slot, k_in, h->d_status);
         int sb = bit_length64((uint64_t)(n_slots > 1 ? n_slots - 1 : 1));
         TA_TRY(ta_radix_sort_pairs(h, k_in, pos_s, k_s, vscr, k_f, pos, m, ta_make_plan(0, sb), nullptr,
                                    sort_tmp));
@@ -470,8 +474,8 @@ ta_status ta_run_correlate(ta_window *h, ta_join_summary *out_summary) {
         TA_TRY((launch_scan<OpMax, JoinHeadIn, JoinHeadOut>(h, m, hin, hout, OpMax(), t2)));
       }
       a.found = found;
-      k_join_probe<false><<<TA_N grid_probe, JP_THREADS, 0, st>>>(a);
-      k_join_launch_stats<false><<<TA_N grid8, JP_THREADS, 0, st>>>(a);
+      ta_launch(k_join_probe<false>, grid_probe, JP_THREADS, 0, st, a);
+      ta_launch(k_join_launch_stats<false>, grid8, JP_THREADS, 0, st, a);
     }
     TA_CHECK_CUDA(h, cudaGetLastError());
   }

@@ -47,6 +47,7 @@ __global__ void __launch_bounds__(256) k_discover(const ta_event *ev, int64_t n,
                                                   TripleTable *tt, CommTable *cm,
                                                   ta_load_summary *sum, int64_t *misc,
                                                   int32_t *status, u64 *prekey) {
+  TA_PDL();
   __shared__ u64 cache[256];  // (triple code << 13) | slot: one word, so a racing reader sees a pair
   __shared__ u64 ccache[64];
   cache[threadIdx.x] = TRIPLE_EMPTY;
@@ -151,6 +152,7 @@ __global__ void __launch_bounds__(PL_THREADS) k_plan(const ta_event *ev, int64_t
                                                      const int64_t *t0, const int64_t *t1, int W,
                                                      int sbits, int64_t max_span, int64_t max_win,
                                                      int64_t *misc) {
+  TA_PDL();
   __shared__ u64 code[PL_SLOTS];
   __shared__ u32 cnt[PL_SLOTS];
   __shared__ u32 s_max, s_valid;
@@ -267,6 +269,7 @@ struct __align__(128) DiscoverSmem {
 };
 
 __global__ void __launch_bounds__(DS_THREADS) k_discover_staged(DiscoverArgs a) {
+  TA_PDL();
   extern __shared__ __align__(128) unsigned char ds_raw[];
   DiscoverSmem &s = *reinterpret_cast<DiscoverSmem *>(ds_raw);
   const int tid = threadIdx.x, lane = tid & 31;
@@ -493,6 +496,7 @@ __device__ __forceinline__ void top_hist_add(const TopHistArgs &a, u32 *hist, u6
 }
 // one window: the lane sizes are the per-triple counts
 __global__ void __launch_bounds__(1024) k_top_hist(TopHistArgs a) {
+  TA_PDL();
   for (int sl = threadIdx.x; sl < TA_TRIPLE_SLOTS; sl += blockDim.x) {
     const u32 c = a.slot_cnt[sl];
     if (c) top_hist_add(a, a.hist, (u64)a.tt->rank_of_slot[sl], c);
@@ -506,6 +510,7 @@ __global__ void __launch_bounds__(1024) k_top_hist(TopHistArgs a) {
 }
 // several windows: one pass over the words (8 bytes per record)
 __global__ void __launch_bounds__(256) k_top_hist_words(TopHistArgs a) {
+  TA_PDL();
   __shared__ u32 sh[10 * 256];
   for (int i = threadIdx.x; i < a.plan.n_pass * 256; i += blockDim.x) sh[i] = 0;
   __syncthreads();
@@ -646,6 +651,7 @@ __device__ __forceinline__ void rank_comms(CommTable *cm, int32_t *status, u64 *
 // Both rankings in one launch: CTA 0 the triples, CTA 1 the communicator ids (they are
 // independent, and two single-CTA kernels one after the other cost a launch latency more).
 __global__ void __launch_bounds__(1024) k_rank(TripleTable *tt, CommTable *cm, int32_t *status) {
+  TA_PDL();
   extern __shared__ u64 rank_buf[];  // TA_TRIPLE_SLOTS
   if (blockIdx.x == 0) rank_triples(tt, status, rank_buf);
   else rank_comms(cm, status, rank_buf);
@@ -667,6 +673,7 @@ struct LoadArgs {
 
 // Pass 2 over the records: sort key and the digit histograms of all passes.
 __global__ void __launch_bounds__(256) k_load(LoadArgs a) {
+  TA_PDL();
   __shared__ u32 sh[10 * 256];
   for (int i = threadIdx.x; i < a.plan.n_pass * 256; i += blockDim.x) sh[i] = 0;
   __syncthreads();
@@ -722,6 +729,7 @@ __global__ void __launch_bounds__(256) k_load(LoadArgs a) {
 // The same from the words k_discover left in a.keys (rewritten in place): 8 B read + 8 B
 // written per record instead of another pass over the 40-byte records.
 __global__ void __launch_bounds__(256) k_load_pre(LoadArgs a) {
+  TA_PDL();
   __shared__ u32 sh[10 * 256];
   for (int i = threadIdx.x; i < a.plan.n_pass * 256; i += blockDim.x) sh[i] = 0;
   __syncthreads();
@@ -790,8 +798,7 @@ ta_status ta_launch_discover(ta_window *h) {
         max_win = max_win > h->h_off[w + 1] - h->h_off[w] ? max_win : h->h_off[w + 1] - h->h_off[w];
       }
       const int sbits = ta_bit_len((uint64_t)(max_span - 1));
-      k_plan<<<TA_N 1, PL_THREADS, 0, h->stream>>>(h->events, h->n, h->d_off, h->d_t0, h->d_t1, h->W, sbits,
-                                                  max_span, max_win, h->d_misc);
+      ta_launch(k_plan, 1, PL_THREADS, 0, h->stream, h->events, h->n, h->d_off, h->d_t0, h->d_t1, h->W, sbits, max_span, max_win, h->d_misc);
       DiscoverArgs a;
       a.ev = h->events; a.n = h->n; a.off = h->d_off; a.t0 = h->d_t0; a.t1 = h->d_t1; a.W = h->W;
       a.tt = h->d_triples; a.cm = h->d_comms; a.sum = h->d_load_sum; a.misc = h->d_misc;
@@ -805,18 +812,16 @@ ta_status ta_launch_discover(ta_window *h) {
 #define DS_CTAS_PER_SM 4
 #endif
       const int grid = (int)(tiles < 148 * DS_CTAS_PER_SM ? tiles : 148 * DS_CTAS_PER_SM);
-      k_discover_staged<<<TA_N grid, DS_THREADS, sizeof(DiscoverSmem), h->stream>>>(a);
+      ta_launch(k_discover_staged, grid, DS_THREADS, sizeof(DiscoverSmem), h->stream, a);
       h->tkeep = -1;  // read back with the other results of the pass
     } else {
-      k_discover<<<TA_N grid_for(h->n, 256, 8), 256, 0, h->stream>>>(
-          h->events, h->n, h->d_off, h->d_t0, h->d_t1, h->W, h->d_triples, h->d_comms, h->d_load_sum,
-          h->d_misc, h->d_status, h->d_keys);
+      ta_launch(k_discover, grid_for(h->n, 256, 8), 256, 0, h->stream, h->events, h->n, h->d_off, h->d_t0, h->d_t1, h->W, h->d_triples, h->d_comms, h->d_load_sum, h->d_misc, h->d_status, h->d_keys);
     }
     h->prekeys = 1;
   }
   TA_CHECK_CUDA(h, cudaFuncSetAttribute(k_rank, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         TA_TRIPLE_SLOTS * (int)sizeof(u64)));
-  k_rank<<<TA_N 2, 1024, TA_TRIPLE_SLOTS * sizeof(u64), h->stream>>>(h->d_triples, h->d_comms, h->d_status);
+  ta_launch(k_rank, 2, 1024, TA_TRIPLE_SLOTS * sizeof(u64), h->stream, h->d_triples, h->d_comms, h->d_status);
   TA_CHECK_CUDA(h, cudaGetLastError());
   return TA_OK;
 }
@@ -869,8 +874,8 @@ ta_status ta_launch_load(ta_window *h, bool allow_packed) {
       a.tbits = h->tbits; a.wbits = h->wbits; a.n_dropped = h->n - h->n_valid;
       a.tt = h->d_triples; a.slot_cnt = h->d_slot_cnt; a.hist = h->d_hist;
       a.prekey = h->d_keys; a.n = h->n; a.off = h->d_off; a.W = h->W;
-      if (h->W == 1) k_top_hist<<<TA_N 1, 1024, 0, h->stream>>>(a);
-      else k_top_hist_words<<<TA_N grid_for(h->n, 256, 8), 256, 0, h->stream>>>(a);
+      if (h->W == 1) ta_launch(k_top_hist, 1, 1024, 0, h->stream, a);
+      else ta_launch(k_top_hist_words, grid_for(h->n, 256, 8), 256, 0, h->stream, a);
       TA_CHECK_CUDA(h, cudaGetLastError());
       return TA_OK;  // the words stay in d_keys (h->prekeys stays set): a retry can still use them
     }
@@ -904,8 +909,8 @@ ta_status ta_launch_load(ta_window *h, bool allow_packed) {
   a.packed = h->packed; a.dshift = h->dshift; a.ibits = h->ibits; a.status = h->d_status;
   // the words of the discovery pass are there once; a later call (the fall back to full
   // resolution keys) goes back to the records
-  if (h->prekeys) k_load_pre<<<TA_N grid_for(h->n, 256, 8), 256, 0, h->stream>>>(a);
-  else k_load<<<TA_N grid_for(h->n, 256, 8), 256, 0, h->stream>>>(a);
+  if (h->prekeys) ta_launch(k_load_pre, grid_for(h->n, 256, 8), 256, 0, h->stream, a);
+  else ta_launch(k_load, grid_for(h->n, 256, 8), 256, 0, h->stream, a);
   h->prekeys = 0;
   TA_CHECK_CUDA(h, cudaGetLastError());
   return TA_OK;

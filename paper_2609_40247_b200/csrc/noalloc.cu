@@ -142,6 +142,7 @@ __global__ void __launch_bounds__(NA_THREADS) k_lane_gaps_ascending(const int64_
                                                                     i64 W0, i64 W1, int64_t *gap_before,
                                                                     ta_lane_gaps *out, NaScratch *sc, NaHost *host,
                                                                     u32 seq) {
+  TA_PDL();
   __shared__ u64 red[4][8];
   const int64_t p0 = (int64_t)blockIdx.x * NF_TILE + (int64_t)threadIdx.x * NF_ITEMS;
   NaTile<NF_ITEMS> t;
@@ -163,6 +164,7 @@ __global__ void __launch_bounds__(NA_THREADS) k_lane_gaps_noalloc(const int64_t 
                                                                    int64_t n, i64 W0, i64 W1,
                                                                    int64_t *gap_before, ta_lane_gaps *out,
                                                                    NaScratch *sc, NaHost *host, u32 seq) {
+  TA_PDL();
   __shared__ u64 tmp[33];
   __shared__ u64 red[4][8];
   __shared__ u64 s_excl;
@@ -247,11 +249,9 @@ extern "C" ta_status ta_lane_gaps_noalloc_host(const int64_t *ts_start, const in
     const int64_t tile = scan ? NA_TILE : NF_TILE;
     const unsigned tiles = (unsigned)((n + tile - 1) / tile);
     if (scan)
-      k_lane_gaps_noalloc<<<TA_N tiles, NA_THREADS, 0, st>>>(ts_start, ts_end, n, win_t0, win_t1, gap_before,
-                                                            lane_out, sc, d->host_dev, seq);
+      ta_launch(k_lane_gaps_noalloc, tiles, NA_THREADS, 0, st, ts_start, ts_end, n, win_t0, win_t1, gap_before, lane_out, sc, d->host_dev, seq);
     else
-      k_lane_gaps_ascending<<<TA_N tiles, NA_THREADS, 0, st>>>(ts_start, ts_end, n, win_t0, win_t1, gap_before,
-                                                              lane_out, sc, d->host_dev, seq);
+      ta_launch(k_lane_gaps_ascending, tiles, NA_THREADS, 0, st, ts_start, ts_end, n, win_t0, win_t1, gap_before, lane_out, sc, d->host_dev, seq);
     if (cudaGetLastError() != cudaSuccess) return TA_ERR_CUDA;
     const NaHost *h = d->host;
     TA_WAIT_SEQ(h->seq, seq, st);

@@ -41,6 +41,7 @@ struct OvKeyArgs {
 
 // one tile of 2048 sorted positions per CTA; tiles that hold host lanes only leave at once
 __global__ void __launch_bounds__(OV_THREADS) k_ov_keys(OvKeyArgs a) {
+  TA_PDL();
   __shared__ int s_lane0;
   if (ta_failed(a.status)) return;
   const int tid = threadIdx.x;
@@ -101,6 +102,7 @@ struct OvScanArgs {
 };
 
 __global__ void __launch_bounds__(OV_THREADS, 3) k_ov_scan(OvScanArgs a) {
+  TA_PDL();
   __shared__ u64 tmp[3][33];
   __shared__ u64 s_excl[3];
   __shared__ int s_tile, s_fail;
@@ -308,7 +310,7 @@ ta_status ta_run_overlap(ta_window *h, ta_overlap_result *out) {
   ka.lane_domain = h->sorted.lane_domain; ka.t0 = h->d_t0; ka.tsbits = tsbits; ka.idxbits = idxbits;
   ka.keys = k_in; ka.pos = v_in; ka.status = h->d_status;
   const int64_t key_tiles = (h->n_valid + OV_TILE - 1) / OV_TILE;
-  k_ov_keys<<<TA_N (unsigned)key_tiles, OV_THREADS, 0, st>>>(ka);
+  ta_launch(k_ov_keys, (unsigned)key_tiles, OV_THREADS, 0, st, ka);
   TA_CHECK_CUDA(h, cudaGetLastError());
   if (idxbits) {
     TA_TRY(ta_radix_sort_keys(h, k_in, k_scr, k_fin, m,
@@ -323,7 +325,7 @@ ta_status ta_run_overlap(ta_window *h, ta_overlap_result *out) {
   sa.m = m; sa.keys = k_fin; sa.idxbits = idxbits;
   sa.te = h->sorted.ts_end; sa.kind = h->sorted.kind; sa.t0 = h->d_t0; sa.t1 = h->d_t1;
   sa.tsbits = tsbits; sa.n_pids = n_pids; sa.status = h->d_status;
-  k_ov_scan<<<TA_N (unsigned)tiles, OV_THREADS, 0, st>>>(sa);
+  ta_launch(k_ov_scan, (unsigned)tiles, OV_THREADS, 0, st, sa);
   TA_CHECK_CUDA(h, cudaGetLastError());
 
   ro.acc = sa.acc; ro.tt = h->d_triples; ro.t0 = h->d_t0; ro.t1 = h->d_t1; ro.n_pids = n_pids;

@@ -58,6 +58,7 @@ __device__ __forceinline__ bool roll_tile(const RollArgs &a, int domain, int64_t
 }
 
 __global__ void __launch_bounds__(RO_THREADS) k_roll_ops(RollArgs a) {
+  TA_PDL();
   int64_t p0, tile_end;
   if (!roll_tile(a, 0, &p0, &tile_end)) return;
   int16_t kd[RO_ITEMS];
@@ -83,6 +84,7 @@ __global__ void __launch_bounds__(RO_THREADS) k_roll_ops(RollArgs a) {
 }
 
 __global__ void __launch_bounds__(RO_THREADS) k_roll_replays(RollArgs a) {
+  TA_PDL();
   int64_t p0, tile_end;
   if (!roll_tile(a, 1, &p0, &tile_end)) return;
   int16_t kd[RO_ITEMS];
@@ -105,6 +107,7 @@ __global__ void __launch_bounds__(RO_THREADS) k_roll_replays(RollArgs a) {
 }
 
 __global__ void __launch_bounds__(RO_THREADS) k_roll_finalize(RollArgs a) {
+  TA_PDL();
   int64_t p0, tile_end;
   if (!roll_tile(a, 0, &p0, &tile_end)) return;
   int16_t kd[RO_ITEMS];
@@ -182,9 +185,9 @@ ta_status ta_run_rollup(ta_window *h, ta_rollup_result *out, ta_rollup_summary *
   a.lane_off = h->sorted.lane_off; a.lane_window = h->sorted.lane_window;
   a.lane_dom_end = h->d_lane_dom_end; a.lane_domain = h->sorted.lane_domain; a.status = h->d_status;
   const unsigned tiles = (unsigned)((h->n_valid + RO_TILE - 1) / RO_TILE);
-  k_roll_ops<<<TA_N tiles, RO_THREADS, 0, st>>>(a);
-  k_roll_replays<<<TA_N tiles, RO_THREADS, 0, st>>>(a);
-  k_roll_finalize<<<TA_N tiles, RO_THREADS, 0, st>>>(a);
+  ta_launch(k_roll_ops, tiles, RO_THREADS, 0, st, a);
+  ta_launch(k_roll_replays, tiles, RO_THREADS, 0, st, a);
+  ta_launch(k_roll_finalize, tiles, RO_THREADS, 0, st, a);
   TA_CHECK_CUDA(h, cudaGetLastError());
   std::vector<u64> hs((size_t)W * 3);
   TA_TRY(ta_queue_d2h(h, hs.data(), a.win_sum, (size_t)W * 24));

@@ -39,6 +39,7 @@ static inline ta_status scan_temp_init(ta_window *h, void *mem, int64_t n, ScanT
 template <class Op, class In, class Out>
 __global__ void __launch_bounds__(SC_THREADS) k_scan(int64_t n, In in, Out out, Op op, ScanTemp t,
                                                      int32_t *status) {
+  TA_PDL();
   __shared__ u64 tmp[33];
   __shared__ u64 s_excl;
   __shared__ int s_tile, s_fail;
@@ -83,7 +84,7 @@ template <class Op, class In, class Out>
 static inline ta_status launch_scan(ta_window *h, int64_t n, In in, Out out, Op op, ScanTemp t) {
   if (n <= 0) return TA_OK;
   int64_t tiles = (n + SC_TILE - 1) / SC_TILE;
-  k_scan<Op, In, Out><<<TA_N (unsigned)tiles, SC_THREADS, 0, h->stream>>>(n, in, out, op, t, h->d_status);
+  ta_launch(k_scan<Op, In, Out>, (unsigned)tiles, SC_THREADS, 0, h->stream, n, in, out, op, t, h->d_status);
   TA_CHECK_CUDA(h, cudaGetLastError());
   return TA_OK;
 }
@@ -219,6 +220,7 @@ static __global__ void __launch_bounds__(CK_THREADS) k_compact_kind(const int16_
                                                              u32 kind_mask, u32 *pos_out, ScanTemp t,
                                                              int32_t *status, i64 *zero_col,
                                                              int64_t zero_n) {
+  TA_PDL();
   __shared__ u64 tmp[33];
   __shared__ u64 s_excl;
   __shared__ int s_tile, s_fail;
@@ -272,8 +274,7 @@ static inline ta_status launch_compact_kind(ta_window *h, const int16_t *kind, i
     TA_CHECK_CUDA(h, cudaMemsetAsync(zero_col + tiles * CK_TILE, 0, (size_t)(zero_n - tiles * CK_TILE) * 8,
                                      h->stream));
   if (n_valid <= 0) return TA_OK;
-  k_compact_kind<<<TA_N (unsigned)tiles, CK_THREADS, 0, h->stream>>>(kind, n_valid, kind_mask, pos_out, t,
-                                                                   h->d_status, zero_col, zero_n);
+  ta_launch(k_compact_kind, (unsigned)tiles, CK_THREADS, 0, h->stream, kind, n_valid, kind_mask, pos_out, t, h->d_status, zero_col, zero_n);
   TA_CHECK_CUDA(h, cudaGetLastError());
   return TA_OK;
 }

@@ -105,6 +105,7 @@ __device__ __forceinline__ void sol_flush(SolAcc &acc, ta_sol_summary *row, u64 
 
 // Persistent CTAs, each over a contiguous range of tiles.
 __global__ void __launch_bounds__(SO_THREADS) k_operator_sol(SolArgs a, int64_t n_tiles, int64_t tiles_per_cta) {
+  TA_PDL();
   __shared__ int s_lane0, s_lane1;
   __shared__ u64 red[7][SO_THREADS / 32];
   if (ta_failed(a.status)) return;
@@ -262,7 +263,7 @@ ta_status ta_run_sol(ta_window *h, const double *flops, const double *bytes, int
     const int64_t n_tiles = (n + SO_TILE - 1) / SO_TILE;
     const int64_t ctas = n_tiles < 148 * 8 ? n_tiles : 148 * 8;
     const int64_t per = (n_tiles + ctas - 1) / ctas;
-    k_operator_sol<<<TA_N (unsigned)((n_tiles + per - 1) / per), SO_THREADS, 0, st>>>(a, n_tiles, per);
+    ta_launch(k_operator_sol, (unsigned)((n_tiles + per - 1) / per), SO_THREADS, 0, st, a, n_tiles, per);
     TA_CHECK_CUDA(h, cudaGetLastError());
   }
   std::vector<ta_sol_summary> hs(W);

@@ -330,6 +330,7 @@ __device__ __forceinline__ void radix_tile(const RadixArgs &a, RadixSmem<THREADS
 
 template <int THREADS, int ITEMS, bool VALS, int BITS, bool STABLE, bool PREKEY>
 __global__ void __launch_bounds__(THREADS, VALS ? RSP_MINB : RSK_MINB) k_radix_pass(RadixArgs a) {
+  TA_PDL();
   constexpr int TILE = THREADS * ITEMS;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   RadixSmem<THREADS, ITEMS> &s = *reinterpret_cast<RadixSmem<THREADS, ITEMS> *>(smem_raw);
@@ -373,6 +374,7 @@ __global__ void __launch_bounds__(THREADS, VALS ? RSP_MINB : RSK_MINB) k_radix_p
 // digit histograms of every pass (used when the caller has none)
 __global__ void __launch_bounds__(256) k_radix_hist(const u64 *keys, int64_t n, SortPlan plan,
                                                     u32 *hist) {
+  TA_PDL();
   // no failure check: reads keys by position only, and the passes that use the histogram check
   __shared__ u32 sh[10 * RS_BINS];
   for (int i = threadIdx.x; i < plan.n_pass * RS_BINS; i += blockDim.x) sh[i] = 0;
@@ -390,6 +392,7 @@ __global__ void __launch_bounds__(256) k_radix_hist(const u64 *keys, int64_t n, 
 
 // exclusive scan of each pass's histogram: one CTA of 256 threads per pass
 __global__ void __launch_bounds__(256) k_radix_scan_hist(const u32 *hist, u32 *bin_offset) {
+  TA_PDL();
   __shared__ u64 tmp[33];
   u64 total;
   u32 v = hist[blockIdx.x * RS_BINS + threadIdx.x];
@@ -420,7 +423,7 @@ static cudaError_t launch_pass(const RadixArgs &a, int bits, unsigned tiles, cud
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,         \
                                          (int)sizeof(Smem));                                        \
     if (e != cudaSuccess) return e;                                                                 \
-    kern<<<TA_N tiles, THREADS, sizeof(Smem), st>>>(a);                                             \
+    ta_launch(kern, tiles, THREADS, sizeof(Smem), st, a);                                             \
     return cudaGetLastError();                                                                      \
   }
   switch (bits) {
@@ -456,10 +459,10 @@ static ta_status radix_sort(ta_window *h, const u64 *keys_in, const u32 *vals_in
     TA_CHECK_CUDA(h, cudaMemsetAsync(own_hist, 0, 10 * RS_BINS * sizeof(u32), st));
     int64_t want = (n + 255) / 256;
     int grid = (int)(want < 148 * 8 ? want : 148 * 8);
-    k_radix_hist<<<TA_N grid, 256, 0, st>>>(keys_in, n, plan, own_hist);
+    ta_launch(k_radix_hist, grid, 256, 0, st, keys_in, n, plan, own_hist);
     hist = own_hist;
   }
-  k_radix_scan_hist<<<TA_N plan.n_pass, 256, 0, st>>>(hist, bin_offset);
+  ta_launch(k_radix_scan_hist, plan.n_pass, 256, 0, st, hist, bin_offset);
   // one clearing for all passes of a pair sort (descriptors tagged with their pass); every pass
   // draws its tile tickets from a counter of its own (state and counters are neighbours)
   TA_CHECK_CUDA(h, cudaMemsetAsync(state, 0, (size_t)((char *)(counter + 16) - (char *)state), st));

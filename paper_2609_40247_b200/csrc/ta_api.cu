@@ -172,6 +172,7 @@ struct FetchList {
 };
 __global__ void __launch_bounds__(256) k_collect(FetchList f, int m, unsigned char *pin_dev, u32 *ticket, u32 seq,
                                                  volatile u32 *seq_word) {
+  TA_PDL();
   const unsigned lo = blockIdx.x * TA_FETCH_STRIPE;
   for (int e = 0; e < m; e++) {
     const unsigned b = f.bytes[e];
@@ -205,8 +206,7 @@ static ta_status flush_fetch(ta_window *h, u32 seq) {
     most = f.bytes[i] > most ? f.bytes[i] : most;
   }
   h->fetch.clear();
-  k_collect<<<TA_N (most + TA_FETCH_STRIPE - 1) / TA_FETCH_STRIPE, 256, 0, h->stream>>>(
-      f, (int)m, h->pin_dev, (u32 *)&h->d_status[ST_TICKET], seq, (volatile u32 *)(h->pin_dev + TA_PIN_BYTES));
+  ta_launch(k_collect, (most + TA_FETCH_STRIPE - 1) / TA_FETCH_STRIPE, 256, 0, h->stream,  f, (int)m, h->pin_dev, (u32 *)&h->d_status[ST_TICKET], seq, (volatile u32 *)(h->pin_dev + TA_PIN_BYTES));
   TA_CHECK_CUDA(h, cudaGetLastError());
   return TA_OK;
 }
@@ -283,6 +283,7 @@ static std::atomic<int> g_ta_spin_limit{0};  // 0 = TA_SPIN_LIMIT; copied into e
 
 // One warp looks back from tile 1 at a tile-0 descriptor that nothing publishes.
 __global__ void k_selftest_wait(u64 *state, int32_t *status) {
+  TA_PDL();
   bool failed;
   tile_lookback<OpAdd>(state, 1, 1ull, OpAdd(), status, &failed);
   if (threadIdx.x == 0) status[ST_LONG_RUN] = failed ? 1 : 0;
@@ -360,7 +361,7 @@ ta_status ta_selftest_wait_timeout(void *cuda_stream, int32_t polls) {
   cudaError_t e = cudaMemsetAsync(buf, 0, 512, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(status, words, sizeof(words), cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) {
-    k_selftest_wait<<<TA_N 1, 32, 0, st>>>(state, status);
+    ta_launch(k_selftest_wait, 1, 32, 0, st, state, status);
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) e = cudaMemcpyAsync(words, status, sizeof(words), cudaMemcpyDeviceToHost, st);

@@ -8,6 +8,7 @@
 #include <stdint.h>
 
 #include <atomic>
+#include <utility>
 #include <vector>
 
 #include "../../include/ta.h"
@@ -271,8 +272,32 @@ void ta_dfree_later(ta_window *h, void *p);
 // ---- instrumentation (no work: a launch counter and optional event pairs) ----
 extern std::atomic<long long> g_ta_launches;  // kernels launched by this library since load
 extern int g_ta_profile;          // 1 = record a CUDA event pair around each radix pass
-static inline unsigned ta_one() { ++g_ta_launches; return 1u; }
-#define TA_N ta_one() *           // used as kernel<<<TA_N grid, ...>>>: counts the launch
+#ifdef __CUDACC__
+// Launches a kernel (and counts it) so that it may be set up while the kernel in front of it in the
+// stream still runs: its CTAs are scheduled once all CTAs of that kernel have started, and wait at
+// TA_PDL() until it has completed.  A step of small kernels is a chain of launch latencies; this
+// hides about a microsecond of each.
+template <class... P, class... A>
+static inline cudaError_t ta_launch(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem,
+                                    cudaStream_t st, A &&...args) {
+  ++g_ta_launches;
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = &at;
+  // a grid of many waves gains nothing from an early first wave, and measured 1 % slower with it
+  cfg.numAttrs = grid <= 148 * 16 ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+}
+// First statement of every kernel: lets the next kernel be set up, then waits until the kernel in
+// front has completed and its writes are visible.  No thread may leave a kernel without passing it.
+#define TA_PDL() asm volatile("griddepcontrol.launch_dependents;\n\tgriddepcontrol.wait;" ::: "memory")
+#endif
 void ta_profile_mark(cudaStream_t st, int begin, double bytes);  // called around k_radix_pass when profiling
 
 // =================================================================== device

@@ -20,6 +20,7 @@
 // ---- pair path: equal-key runs -------------------------------------------
 __global__ void __launch_bounds__(256) k_fix_ties(const u64 *keys, u32 *perm, int64_t n_valid,
                                                   const ta_event *ev, int32_t *status) {
+  TA_PDL();
   if (ta_failed(status)) return;
   int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= n_valid || p + 1 >= n_valid) return;
@@ -56,6 +57,7 @@ __global__ void __launch_bounds__(256) k_fix_ties(const u64 *keys, u32 *perm, in
 // ---- fallback: duration as a least-significant key ------------------------
 __global__ void __launch_bounds__(256) k_duration_key(const ta_event *ev, int64_t n, const u64 *keys,
                                                       u64 dropped_bit, i64 max_dur, u64 *out) {
+  TA_PDL();
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   if (keys[i] & dropped_bit) { out[i] = 0; return; }
@@ -64,6 +66,7 @@ __global__ void __launch_bounds__(256) k_duration_key(const ta_event *ev, int64_
 }
 __global__ void __launch_bounds__(256) k_gather_u64(const u64 *src, const u32 *idx, int64_t n, u64 *dst,
                                                     const int32_t *status) {
+  TA_PDL();
   if (ta_failed(status)) return;
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) dst[i] = src[idx[i]];
@@ -74,6 +77,7 @@ __global__ void __launch_bounds__(256) k_gather_u64(const u64 *src, const u32 *i
 __global__ void __launch_bounds__(256) k_tail_key(const ta_event *ev, const u32 *idx, int64_t m,
                                                   int stage, const int64_t *off, int W, u64 *out,
                                                   const int32_t *status) {
+  TA_PDL();
   if (ta_failed(status)) return;
   int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= m) return;
@@ -115,6 +119,7 @@ __device__ __forceinline__ u32 gather_index(u64 k, const GatherArgs &a) {
 #define GT_MINB 8
 #endif
 __global__ void __launch_bounds__(256, GT_MINB) k_gather(GatherArgs a) {
+  TA_PDL();
   __shared__ int s_slot[8];
   __shared__ u64 s_mx[8], s_mn[8];
   if (ta_failed(a.status)) return;  // the sort gave up: the keys name no records
@@ -237,6 +242,7 @@ __global__ void __launch_bounds__(1024) k_lane_table(const int32_t *lane_start, 
                                                      int32_t *lane_dom_end, int32_t *lane_dom_next,
                                                      int32_t *lane_dev_base, int32_t *n_lanes_out,
                                                      int64_t cap, const int32_t *status) {
+  TA_PDL();
   __shared__ u64 tmp[33];
   __shared__ u64 base;
   if (ta_failed(status)) {  // no lanes: every later call then finds nothing to index
@@ -402,6 +408,7 @@ __device__ __forceinline__ u32 packed_index(u64 k, const PackInfo &pi) {
 }
 __global__ void __launch_bounds__(256) k_unpack_tail(const u64 *keys, int64_t n_valid, int64_t n,
                                                      PackInfo pi, u32 *perm, const int32_t *status) {
+  TA_PDL();
   if (ta_failed(status)) return;
   int64_t p = n_valid + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (p < n) perm[p] = packed_index(keys[p], pi);
@@ -472,8 +479,7 @@ ta_status ta_run_sort_timeline(ta_window *h) {
         TA_TRY(ta_radix_sort_keys(h, h->d_keys, kscr, skeys, n, h->plan, h->d_hist, sort_tmp, true,
                                   h->fast_keys ? &pre : nullptr));
         if (n > h->n_valid)
-          k_unpack_tail<<<TA_N nblk(n - h->n_valid, 256), 256, 0, st>>>(skeys, h->n_valid, n, pi, perm,
-                                                                            h->d_status);
+          ta_launch(k_unpack_tail, nblk(n - h->n_valid, 256), 256, 0, st, skeys, h->n_valid, n, pi, perm, h->d_status);
       }
       if (!h->packed) {
         // step 1: (key, input index) pairs; the last pass writes (skeys, perm)
@@ -481,8 +487,7 @@ ta_status ta_run_sort_timeline(ta_window *h) {
                                    h->d_hist, sort_tmp));
         // step 2: equal-key runs
         if (h->n_valid > 1)
-          k_fix_ties<<<TA_N nblk(h->n_valid, 256), 256, 0, st>>>(skeys, perm, h->n_valid, h->events,
-                                                            h->d_status);
+          ta_launch(k_fix_ties, nblk(h->n_valid, 256), 256, 0, st, skeys, perm, h->n_valid, h->events, h->d_status);
         TA_TRY(ta_read_status(h, words));
         if (words[ST_ERR]) return (ta_status)words[ST_ERR];
         if (words[ST_LONG_RUN]) {
@@ -495,14 +500,13 @@ ta_status ta_run_sort_timeline(ta_window *h) {
           u64 *dkeys = cx.take<u64>(n);
           u32 *dorder = cx.take<u32>(n);
           const u64 dropped_bit = h->has_dropped ? 1ull << (h->sbits + h->tbits + h->wbits) : 0ull;
-          k_duration_key<<<TA_N nblk(n, 256), 256, 0, st>>>(h->events, n, h->d_keys, dropped_bit,
-                                                       h->max_dur, dkeys);
+          ta_launch(k_duration_key, nblk(n, 256), 256, 0, st, h->events, n, h->d_keys, dropped_bit, h->max_dur, dkeys);
           int dbits = 1;
           while (dbits < 63 && (h->max_dur >> dbits) != 0) dbits++;
           SortPlan dplan = ta_make_plan(0, dbits);
           TA_TRY(ta_radix_sort_pairs(h, dkeys, nullptr, kscr, vscr, skeys, dorder, n, dplan, nullptr,
                                      sort_tmp));
-          k_gather_u64<<<TA_N nblk(n, 256), 256, 0, st>>>(h->d_keys, dorder, n, dkeys, h->d_status);
+          ta_launch(k_gather_u64, nblk(n, 256), 256, 0, st, h->d_keys, dorder, n, dkeys, h->d_status);
           TA_TRY(ta_radix_sort_pairs(h, dkeys, dorder, kscr, vscr, skeys, perm, n, h->plan, nullptr,
                                      sort_tmp));
           TA_TRY(ta_sync_fetch(h));
@@ -523,8 +527,7 @@ ta_status ta_run_sort_timeline(ta_window *h) {
         // dropped records of a window share one key, so the tail is put in input order first
         for (int stage = h->packed ? -1 : 0; stage < 4; stage++) {
           if (stage == 3 && h->W == 1) break;
-          k_tail_key<<<TA_N nblk(m, 256), 256, 0, st>>>(h->events, cur, m, stage, h->d_off, h->W, tk,
-                                                        h->d_status);
+          ta_launch(k_tail_key, nblk(m, 256), 256, 0, st, h->events, cur, m, stage, h->d_off, h->W, tk, h->d_status);
           int bits = stage == 2 ? 49 : stage == 3 ? (h->wbits > 0 ? h->wbits : 1) : stage < 0 ? 32 : 64;
           SortPlan tp = ta_make_plan(0, bits);
           TA_TRY(ta_radix_sort_pairs(h, tk, cur, kscr, vscr, tk2, nxt, m, tp, nullptr, sort_tmp));
@@ -546,14 +549,10 @@ ta_status ta_run_sort_timeline(ta_window *h) {
       g.stream = c_stream; g.kind = c_kind; g.lane_start = lane_start;
       g.tt = h->d_triples; g.tbits = h->tbits; g.n_pids = h->n_pids > 0 ? h->n_pids : 1;
       g.slot_min = h->d_slot_min; g.slot_max = h->d_slot_max; g.status = h->d_status;
-      k_gather<<<TA_N nblk(n, 256), 256, 0, st>>>(g);
+      ta_launch(k_gather, nblk(n, 256), 256, 0, st, g);
     }
     if (n_codes <= LT_ONE_CTA || n == 0) {
-      k_lane_table<<<TA_N 1, 1024, 0, st>>>(lane_start, n_codes, h->tbits,
-                                     h->n_pids > 0 ? h->n_pids : 1, h->d_triples, h->n_valid,
-                                     lane_window, lane_pid, lane_stream, lane_domain, lane_off,
-                                     lane_code, lane_slot, lane_dom_end, lane_dom_next, lane_dev_base, n_lanes_dev,
-                                     lane_cap, h->d_status);
+      ta_launch(k_lane_table, 1, 1024, 0, st, lane_start, n_codes, h->tbits, h->n_pids > 0 ? h->n_pids : 1, h->d_triples, h->n_valid, lane_window, lane_pid, lane_stream, lane_domain, lane_off, lane_code, lane_slot, lane_dom_end, lane_dom_next, lane_dev_base, n_lanes_dev, lane_cap, h->d_status);
     } else {
       LaneRows t{lane_start, h->tbits, h->n_pids > 0 ? h->n_pids : 1, h->d_triples, h->n_valid,
                  lane_window, lane_pid, lane_stream, lane_domain, lane_off, lane_code, lane_slot,
