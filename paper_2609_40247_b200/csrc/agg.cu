@@ -747,6 +747,7 @@ ta_status ta_run_aggregate(ta_window *h, uint32_t kind_mask, int value_sel, ta_a
   ro.tt = h->d_triples; ro.n_pids = n_pids; ro.R = R; ro.min_name = h->min_name;
   ro.name_of = table ? h->d_name_of : nullptr;
   u64 ng = 0;
+  int32_t status[ST_WORDS];
   void *tmpb = nullptr, *outb = nullptr;
   // the three row tables (window, pid, symbol), the four 64-bit columns and the histograms of `rows` rows
   auto carve_rows = [&](int64_t rows) -> size_t {
@@ -769,24 +770,25 @@ ta_status ta_run_aggregate(ta_window *h, uint32_t kind_mask, int value_sel, ta_a
   if (G * 232 <= 8 * h->n_valid + (64ll << 20)) {
     ScanTemp t;
     size_t tb = 4 * Carver::pad((size_t)G * 8) + Carver::pad((size_t)G * TA_NBINS * 4) + scan_temp_bytes(G) + 256;
-    tmpb = ta_dalloc(h, tb);
-    if (!tmpb) return TA_ERR_OOM;
+    ta_status zs;
+    tmpb = ta_zalloc(h, tb, &zs);
+    if (!tmpb) return zs;
     Carver ct(tmpb);
     a.d_cnt = ct.take<u64>(G);
     a.d_sum = ct.take<u64>(G);
     a.d_minc = ct.take<u64>(G);
     a.d_maxb = ct.take<u64>(G);
     a.d_hist = ct.take<u32>((size_t)G * TA_NBINS);
-    ct.off += scan_temp_carve(ct.base + ct.off, G, &t);
-    TA_CHECK_CUDA(h, cudaMemsetAsync(tmpb, 0, ct.off, st));
+    scan_temp_carve(ct.base + ct.off, G, &t);
     run_agg();
     // the rows are compacted without waiting for their count: it is bounded by cells and records
     carve_rows(G < h->n_valid ? G : h->n_valid);
     if (!outb) return TA_ERR_OOM;
     ro.cnt = a.d_cnt; ro.sum = a.d_sum; ro.minc = a.d_minc; ro.maxb = a.d_maxb; ro.hist = a.d_hist;
     AggRowIn ri{a.d_cnt};
-    TA_TRY((launch_scan<OpAdd, AggRowIn, AggRowOut>(h, G, ri, ro, OpAdd(), t)));
     TA_TRY(ta_queue_d2h(h, &ng, t.total, 8));
+    TA_TRY(ta_queue_d2h(h, status, h->d_status, sizeof(status)));
+    TA_TRY((launch_scan<OpAdd, AggRowIn, AggRowOut>(h, G, ri, ro, OpAdd(), t, true)));
   } else {
     const int64_t words = (G + 31) / 32;
     ScanTemp t;
@@ -814,12 +816,12 @@ ta_status ta_run_aggregate(ta_window *h, uint32_t kind_mask, int value_sel, ta_a
       run_agg();
       ta_launch(k_agg_marked_rows, (unsigned)((words + 255) / 256), 256, 0, st, a.bits, rank, words, ro, h->d_status);
     }
+    TA_TRY(ta_queue_d2h(h, status, h->d_status, sizeof(status)));
   }
   TA_CHECK_CUDA(h, cudaGetLastError());
-  int32_t words[ST_WORDS];
-  TA_TRY(ta_read_status(h, words));
+  TA_TRY(ta_sync_fetch(h));
   ta_dfree(h, tmpb);
-  if (words[ST_ERR]) return (ta_status)words[ST_ERR];
+  if (status[ST_ERR]) return (ta_status)status[ST_ERR];
   out->n_groups = (int64_t)ng;
   if (ng == 0) return TA_OK;
   out->g_window = ro.g_window; out->g_pid = ro.g_pid; out->g_name = ro.g_name;

@@ -740,8 +740,7 @@ __global__ void __launch_bounds__(AT_THREADS, AT_OPS_MINB) k_attr_ops(AttrArgs a
 #ifndef AT_FIN_ITEMS
 #define AT_FIN_ITEMS 4
 #endif
-__global__ void __launch_bounds__(256) k_attr_finalize(AttrArgs a) {
-  TA_PDL();
+__device__ __forceinline__ void attr_finalize(const AttrArgs &a) {
   constexpr int IT = AT_FIN_ITEMS;
   const int err = ta_peek_err(a.status);
   const int64_t p0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * IT;
@@ -779,26 +778,31 @@ __global__ void __launch_bounds__(256) k_attr_finalize(AttrArgs a) {
     }
 }
 
+__global__ void __launch_bounds__(256) k_attr_finalize(AttrArgs a, Tail tail) {
+  TA_PDL();
+  attr_finalize(a);
+  run_tail(tail);
+}
+
 ta_status ta_run_attribute(ta_window *h, ta_attr_summary *out_summary) {
   const int64_t n = h->n, nn = n > 0 ? n : 1;
   const int W = h->W;
   cudaStream_t st = h->stream;
   const int64_t tiles = (n + AT_TILE - 1) / AT_TILE;
-  size_t keep = 3 * Carver::pad(nn * 4) + Carver::pad(nn) + 3 * Carver::pad(nn * 8) +
-                Carver::pad((size_t)W * sizeof(ta_attr_summary)) + 256;
+  size_t keep = 2 * Carver::pad(nn * 4) + Carver::pad(nn) + 256;
   void *kb = ta_dalloc(h, keep);
   if (!kb) return TA_ERR_OOM;
   Carver ck(kb);
   int32_t *parent = ck.take<int32_t>(nn), *op_of = ck.take<int32_t>(nn);
   uint8_t *depth = ck.take<uint8_t>(nn);
-  char *zero_begin = ck.base + ck.off;
-  int32_t *op_n = ck.take<int32_t>(nn);
-  u64 *op_first = ck.take<u64>(nn), *op_last = ck.take<u64>(nn);
-  int64_t *op_ns = ck.take<int64_t>(nn);
-  char *zero_end = ck.base + ck.off;
-  ta_attr_summary *d_sum = ck.take<ta_attr_summary>(W);
-  TA_CHECK_CUDA(h, cudaMemsetAsync(zero_begin, 0, zero_end - zero_begin, st));
-  TA_CHECK_CUDA(h, cudaMemsetAsync(d_sum, 0, (size_t)W * sizeof(ta_attr_summary), st));
+  ta_status zs;
+  void *zb = ta_zalloc(h, Carver::pad(nn * 4) + 3 * Carver::pad(nn * 8) + Carver::pad((size_t)W * sizeof(ta_attr_summary)), &zs);
+  if (!zb) return zs;
+  Carver cz(zb);
+  int32_t *op_n = cz.take<int32_t>(nn);
+  u64 *op_first = cz.take<u64>(nn), *op_last = cz.take<u64>(nn);
+  int64_t *op_ns = cz.take<int64_t>(nn);
+  ta_attr_summary *d_sum = cz.take<ta_attr_summary>(W);
 
   const int64_t tt = tiles > 0 ? tiles : 1;
   size_t tb = 2 * Carver::pad(tt * 4) + 2 * Carver::pad(tt * AT_CAP * 8) + 2 * Carver::pad(tt * AT_CAP * 4) + 256;
@@ -815,12 +819,10 @@ ta_status ta_run_attribute(ta_window *h, ta_attr_summary *out_summary) {
   memset(&a, 0, sizeof(a));
   a.agg_meta = ct.take<int32_t>(tt);
   a.carry_cnt = ct.take<int32_t>(tt);
-  const size_t zero_bytes = ct.off;  // metas and carry counts start at zero; payloads need not
   a.agg_e = ct.take<i64>(tt * AT_CAP);
   a.carry_e = ct.take<i64>(tt * AT_CAP);
   a.agg_pos = ct.take<int32_t>(tt * AT_CAP);
   a.carry_pos = ct.take<int32_t>(tt * AT_CAP);
-  TA_CHECK_CUDA(h, cudaMemsetAsync(tmpb, 0, zero_bytes, st));
 
   a.n = n; a.n_valid = h->n_valid; a.n_lanes = h->sorted.n_lanes; a.n_tiles = tiles;
   a.kind = h->sorted.kind; a.ts = h->sorted.ts_start; a.te = h->sorted.ts_end;
@@ -829,6 +831,11 @@ ta_status ta_run_attribute(ta_window *h, ta_attr_summary *out_summary) {
   a.parent = parent; a.depth = depth; a.sum = d_sum; a.status = h->d_status;
   a.launch_of = h->join.launch_of; a.kol = h->join.kernels_of_launch; a.op_of = op_of; a.op_n = op_n; a.op_first = op_first;
   a.op_last = op_last; a.op_ns = op_ns;
+  int32_t words[ST_WORDS];
+  std::vector<ta_attr_summary> hs(W);
+  const bool small = W * sizeof(ta_attr_summary) <= 4096;  // (more is copied once the kernels are queued)
+  TA_TRY(ta_queue_d2h(h, words, h->d_status, sizeof(words)));
+  if (small) TA_TRY(ta_queue_d2h(h, hs.data(), d_sum, W * sizeof(ta_attr_summary)));
   if (n > 0) {
     ta_launch(k_attr_agg, (unsigned)tiles, AT_THREADS, 0, st, a);
     {
@@ -851,13 +858,11 @@ ta_status ta_run_attribute(ta_window *h, ta_attr_summary *out_summary) {
     ta_launch(k_attr_resolve, (unsigned)tiles, AT_THREADS, 0, st, a);
     ta_launch(k_attr_ops, (unsigned)((n + AT_OPS_TILE - 1) / AT_OPS_TILE), AT_THREADS, 0, st, a);
     const int64_t fb = (h->n_valid + 256 * AT_FIN_ITEMS - 1) / (256 * AT_FIN_ITEMS);
-    ta_launch(k_attr_finalize, (unsigned)(fb > 0 ? fb : 1), 256, 0, st, a);
+    ta_launch(k_attr_finalize, (unsigned)(fb > 0 ? fb : 1), 256, 0, st, a, ta_tail(h, fb));
     TA_CHECK_CUDA(h, cudaGetLastError());
   }
-  std::vector<ta_attr_summary> hs(W);
-  TA_TRY(ta_queue_d2h(h, hs.data(), d_sum, W * sizeof(ta_attr_summary)));
-  int32_t words[ST_WORDS];
-  TA_TRY(ta_read_status(h, words));
+  if (!small) TA_TRY(ta_queue_d2h(h, hs.data(), d_sum, W * sizeof(ta_attr_summary)));
+  TA_TRY(ta_sync_fetch(h));
   ta_dfree(h, tmpb);
   bool any_bad = false, any_deep = words[ST_ERR] == TA_ERR_DEPTH;
   if (words[ST_ERR] && words[ST_ERR] != TA_ERR_DEPTH) return (ta_status)words[ST_ERR];

@@ -50,7 +50,7 @@ __global__ void __launch_bounds__(256) k_coll_keys(CollCtx c, u64 *keys, int32_t
   // every communicator id was inserted while the records were loaded: a bounded probe all the same
   u32 s = hash_code(cc) & (TA_COMM_SLOTS - 1);
   int probes = 0;
-  while (c.cm->slots[s] != cc && ++probes < TA_COMM_SLOTS) s = (s + 1) & (TA_COMM_SLOTS - 1);
+  while (c.cm->slots[s] != ~cc && ++probes < TA_COMM_SLOTS) s = (s + 1) & (TA_COMM_SLOTS - 1);
   u64 rank = 0;
   if (probes < TA_COMM_SLOTS) rank = (u64)c.cm->rank_of_slot[s];
   else ta_set_err(status, TA_ERR_OVERFLOW);
@@ -278,7 +278,7 @@ ta_status ta_run_collectives(ta_window *h, const ta_comm_size *sizes, int32_t n_
 
   // 2. keys + sort; 3. heads
   size_t t2b = 3 * Carver::pad((size_t)m * 8) + 4 * Carver::pad((size_t)m * 4) + Carver::pad((size_t)(m + 1) * 4) +
-               Carver::pad((size_t)h->n_comms * 4) + 5 * Carver::pad((size_t)n_slots * 8) +
+               Carver::pad((size_t)h->n_comms * 4) +
                ta_sort_temp_bytes(m) + scan_temp_bytes(m) + scan_temp_bytes(n_slots) + 512;
   void *t2 = ta_dalloc(h, t2b);
   if (!t2) return TA_ERR_OOM;
@@ -288,10 +288,12 @@ ta_status ta_run_collectives(ta_window *h, const ta_comm_size *sizes, int32_t n_
   int32_t *slot_of = c2.take<int32_t>(m), *gid_of_c = c2.take<int32_t>(m);
   int32_t *gstart = c2.take<int32_t>(m + 1);
   int32_t *d_expected = c2.take<int32_t>(h->n_comms);
-  char *zb = c2.base + c2.off;
-  u64 *r_seen = c2.take<u64>(n_slots), *r_ncoll = c2.take<u64>(n_slots), *r_sum = c2.take<u64>(n_slots);
-  u64 *r_maxw = c2.take<u64>(n_slots), *r_nstrag = c2.take<u64>(n_slots);
-  TA_CHECK_CUDA(h, cudaMemsetAsync(zb, 0, (c2.base + c2.off) - zb, st));
+  ta_status zs;
+  void *zb = ta_zalloc(h, 5 * Carver::pad((size_t)n_slots * 8), &zs);
+  if (!zb) return zs;
+  Carver cz(zb);
+  u64 *r_seen = cz.take<u64>(n_slots), *r_ncoll = cz.take<u64>(n_slots), *r_sum = cz.take<u64>(n_slots);
+  u64 *r_maxw = cz.take<u64>(n_slots), *r_nstrag = cz.take<u64>(n_slots);
   void *sort_tmp = c2.base + c2.off; c2.off += ta_sort_temp_bytes(m);
   void *scan2 = c2.base + c2.off; c2.off += scan_temp_bytes(m);
   void *scan3 = c2.base + c2.off;
@@ -354,14 +356,16 @@ ta_status ta_run_collectives(ta_window *h, const ta_comm_size *sizes, int32_t n_
   ScanTemp s3;
   TA_TRY(scan_temp_init(h, scan3, n_slots, &s3));
   RankRowIn ri{r_seen};
-  TA_TRY((launch_scan<OpAdd, RankRowIn, RankRowOut>(h, n_slots, ri, ro, OpAdd(), s3)));
   u64 nr64 = 0;
+  int32_t words[ST_WORDS];
   TA_TRY(ta_queue_d2h(h, &nr64, s3.total, 8));
   if (bounded) TA_TRY(ta_queue_d2h(h, &ng64, s2.total, 8));
-  int32_t words[ST_WORDS];
-  TA_TRY(ta_read_status(h, words));
+  TA_TRY(ta_queue_d2h(h, words, h->d_status, sizeof(words)));
+  TA_TRY((launch_scan<OpAdd, RankRowIn, RankRowOut>(h, n_slots, ri, ro, OpAdd(), s3, true)));
+  TA_TRY(ta_sync_fetch(h));
   ta_dfree(h, t1);
   ta_dfree(h, t2);
+  ta_dfree(h, zb);
   if (words[ST_ERR]) return (ta_status)words[ST_ERR];
 
   out->n_groups = (int64_t)ng64;

@@ -812,13 +812,16 @@ ta_status ta_run_critpath(ta_window *h, ta_critpath_result *out, ta_critpath_sum
   ScanTemp s3;
   TA_TRY(scan_temp_init(h, scan_mem, n_slots, &s3));
   CpRowIn ri{a.acc};
-  TA_TRY((launch_scan<OpAdd, CpRowIn, CpRowOut>(h, n_slots, ri, ro, OpAdd(), s3)));
   u64 rows = 0;
-  std::vector<u64> hacc((size_t)n_slots * CP_ACC);
-  TA_TRY(ta_queue_d2h(h, &rows, s3.total, 8));
-  TA_TRY(ta_queue_d2h(h, hacc.data(), a.acc, hacc.size() * 8));
   int32_t words[ST_WORDS];
-  TA_TRY(ta_read_status(h, words));
+  std::vector<u64> hacc((size_t)n_slots * CP_ACC);
+  const bool small = hacc.size() * 8 <= 4096;  // (more is copied once the kernels are queued)
+  TA_TRY(ta_queue_d2h(h, &rows, s3.total, 8));
+  TA_TRY(ta_queue_d2h(h, words, h->d_status, sizeof(words)));
+  if (small) TA_TRY(ta_queue_d2h(h, hacc.data(), a.acc, hacc.size() * 8));
+  TA_TRY((launch_scan<OpAdd, CpRowIn, CpRowOut>(h, n_slots, ri, ro, OpAdd(), s3, true)));
+  if (!small) TA_TRY(ta_queue_d2h(h, hacc.data(), a.acc, hacc.size() * 8));
+  TA_TRY(ta_sync_fetch(h));
   ta_dfree(h, lb);
   if (sortb) ta_dfree(h, sortb);
   ta_dfree(h, tmpb);

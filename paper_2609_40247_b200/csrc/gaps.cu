@@ -57,8 +57,7 @@ struct GapArgs {
 };
 
 
-__global__ void __launch_bounds__(GP_THREADS, GP_MINB) k_gaps(GapArgs a) {
-  TA_PDL();
+__device__ __forceinline__ void gaps_tile(const GapArgs &a) {
   __shared__ u64 tmp[33];
   __shared__ u64 red[4][GP_THREADS / 32];
   __shared__ u64 s_excl_max;
@@ -312,6 +311,12 @@ __global__ void __launch_bounds__(GP_THREADS, GP_MINB) k_gaps(GapArgs a) {
   }
 }
 
+__global__ void __launch_bounds__(GP_THREADS, GP_MINB) k_gaps(GapArgs a, Tail tail) {
+  TA_PDL();
+  gaps_tile(a);
+  run_tail(tail);
+}
+
 struct GapBitsIn {
   const u64 *bits;
   __device__ u64 operator()(int64_t i) const { return (u64)__popcll(bits[i]); }
@@ -340,25 +345,24 @@ ta_status ta_run_gaps(ta_window *h, int64_t min_gap, ta_gap_result *out) {
   if (L >= (1 << 22) - 1) return TA_ERR_TOO_LARGE;
   const int64_t tiles = (n + GP_TILE - 1) / GP_TILE;
   int64_t cap = n / 8 > 65536 ? n / 8 : 65536;  // first guess; a longer list is rebuilt below
-  size_t bytes = Carver::pad((size_t)(n > 0 ? n : 1) * 8) + Carver::pad((size_t)(L + 1) * sizeof(ta_lane_gaps)) +
-                 Carver::pad((size_t)(L + 1) * TA_NBINS * 4) + Carver::pad((size_t)W * TA_NBINS * 4) +
-                 512;
+  const size_t bytes = Carver::pad((size_t)(L + 1) * sizeof(ta_lane_gaps)) +
+                       Carver::pad((size_t)(L + 1) * TA_NBINS * 4) + Carver::pad((size_t)W * TA_NBINS * 4);
   // temporary: look-back state, scalars, the bitmap of the list's order, its scan
   const int64_t n_bits = (n + 31) / 32;
   const size_t tmp_bytes = Carver::pad((size_t)(tiles + 1) * 8) + Carver::pad(64) + Carver::pad((size_t)n_bits * 8) +
                            scan_temp_bytes(n_bits) + Carver::pad((size_t)n_bits * 4) + 512;
-  void *b = ta_dalloc(h, bytes);
-  if (!b) return TA_ERR_OOM;
+  int64_t *gap_before = (int64_t *)ta_dalloc(h, (size_t)(n > 0 ? n : 1) * 8);
+  if (!gap_before) return TA_ERR_OOM;
+  ta_status zs;
+  void *b = ta_zalloc(h, bytes, &zs);
+  if (!b) return zs;
   Carver c(b);
-  int64_t *gap_before = c.take<int64_t>(n > 0 ? n : 1);
-  // everything that must start at zero sits in one contiguous range
-  char *zero_begin = c.base + c.off;
   ta_lane_gaps *lane_gaps = c.take<ta_lane_gaps>(L + 1);
   u32 *lane_hist = c.take<u32>((size_t)(L + 1) * TA_NBINS);
   u32 *win_hist = c.take<u32>((size_t)W * TA_NBINS);
-  char *zero_end = c.base + c.off;
-  TA_CHECK_CUDA(h, cudaMemsetAsync(zero_begin, 0, zero_end - zero_begin, st));
-  void *tb = ta_dalloc(h, tmp_bytes);
+  void *tb = ta_zpool(h, tmp_bytes);
+  const bool pooled = tb != nullptr;
+  if (!tb) tb = ta_dalloc(h, tmp_bytes);
   if (!tb) return TA_ERR_OOM;
   Carver ct(tb);
   u64 *st_max = ct.take<u64>(tiles + 1);
@@ -369,7 +373,7 @@ ta_status ta_run_gaps(ta_window *h, int64_t min_gap, ta_gap_result *out) {
   ct.off += scan_temp_carve(ct.base + ct.off, n_bits, &scan);
   const size_t tmp_zero = ct.off;
   u32 *rank = ct.take<u32>(n_bits);
-  TA_CHECK_CUDA(h, cudaMemsetAsync(tb, 0, tmp_zero, st));
+  if (!pooled) TA_CHECK_CUDA(h, cudaMemsetAsync(tb, 0, tmp_zero, st));
   // unordered list + keys (temporary)
   void *lt = ta_dalloc(h, Carver::pad((size_t)cap * sizeof(ta_long_gap)) + Carver::pad((size_t)cap * 4) + 256);
   if (!lt) return TA_ERR_OOM;
@@ -392,15 +396,16 @@ ta_status ta_run_gaps(ta_window *h, int64_t min_gap, ta_gap_result *out) {
   // first without the scan (every lane is taken to end its records in ascending order, which the
   // kernel checks); if a lane does not, once more with the chained maximum scan
   for (a.local = 1; a.local >= 0; a.local--) {
-    if (tiles > 0) ta_launch(k_gaps, (unsigned)tiles, GP_THREADS, 0, st, a);
-    TA_CHECK_CUDA(h, cudaGetLastError());
     u64 two[3] = {0, 0, 0};
     TA_TRY(ta_queue_d2h(h, two, scal, 24));
-    TA_TRY(ta_read_status(h, words));
+    TA_TRY(ta_queue_d2h(h, words, h->d_status, sizeof(words)));
+    if (tiles > 0) ta_launch(k_gaps, (unsigned)tiles, GP_THREADS, 0, st, a, ta_tail(h, tiles));
+    TA_CHECK_CUDA(h, cudaGetLastError());
+    TA_TRY(ta_sync_fetch(h));
     if (words[ST_ERR]) return (ta_status)words[ST_ERR];
     n_long = two[0];
     if (!a.local || !(u32)two[2]) break;
-    TA_CHECK_CUDA(h, cudaMemsetAsync(zero_begin, 0, zero_end - zero_begin, st));
+    TA_CHECK_CUDA(h, cudaMemsetAsync(b, 0, bytes, st));
     TA_CHECK_CUDA(h, cudaMemsetAsync(tb, 0, tmp_zero, st));
   }
   if ((int64_t)n_long > cap) {
@@ -414,7 +419,7 @@ ta_status ta_run_gaps(ta_window *h, int64_t min_gap, ta_gap_result *out) {
     ukeys = cl2.take<u32>(cap);
     TA_CHECK_CUDA(h, cudaMemsetAsync(tb, 0, state_bytes, st));
     a.list = ulist; a.list_key = ukeys; a.list_cap = cap; a.list_only = 1;
-    ta_launch(k_gaps, (unsigned)tiles, GP_THREADS, 0, st, a);
+    ta_launch(k_gaps, (unsigned)tiles, GP_THREADS, 0, st, a, ta_tail(h, tiles));
     TA_CHECK_CUDA(h, cudaGetLastError());
     TA_TRY(ta_read_status(h, words));
     if (words[ST_ERR]) return (ta_status)words[ST_ERR];

@@ -24,7 +24,7 @@
 #define JN_THREADS 512
 #define JN_ITEMS 4
 #define JN_TILE (JN_THREADS * JN_ITEMS)
-#define EMPTY_U32 0xFFFFFFFFu
+// entry of the direct table: complement of the smallest position, 0 = empty
 
 struct JoinArgs {
   int64_t n, n_valid;
@@ -45,7 +45,7 @@ struct JoinArgs {
 };
 
 __device__ __forceinline__ u64 bias64(i64 v) { return (u64)v ^ (1ull << 63); }
-__device__ __forceinline__ i64 unbias64(u64 v) { return (i64)(v ^ (1ull << 63)); }
+__host__ __device__ __forceinline__ i64 unbias64(u64 v) { return (i64)(v ^ (1ull << 63)); }
 
 // ---- direct path: fill the table -------------------------------------------
 __global__ void __launch_bounds__(JN_THREADS) k_join_build(JoinArgs a) {
@@ -77,7 +77,7 @@ __global__ void __launch_bounds__(JN_THREADS) k_join_build(JoinArgs a) {
     if (p < a.n_valid && kd[j] == TA_KIND_LAUNCH) {
       while (p >= next_off) { l++; next_off = a.lane_off[l + 1]; slot = a.lane_slot[l]; }
       const i64 idx = a.slot_base[slot] + (c[j] - a.slot_min[slot]);
-      atomicMin(&a.table[idx], (u32)p);
+      atomicMax(&a.table[idx], ~(u32)p);
     }
   }
 }
@@ -101,8 +101,9 @@ __device__ __forceinline__ void join_emit(ta_join_summary *sm, const u64 *t) {
   atomicAdd((u64 *)&sm->n_matched, t[1]);
   atomicAdd((u64 *)&sm->sum_latency, t[2]);
   atomicAdd((u64 *)&sm->sum_queue, t[3]);
-  atomicMax((i64 *)&sm->max_latency, unbias64(t[4]));
-  atomicMin((i64 *)&sm->min_latency, unbias64(~t[5]));
+  // (codes with 0 as "none"; the host turns them into times)
+  atomicMax((u64 *)&sm->max_latency, t[4]);
+  atomicMax((u64 *)&sm->min_latency, t[5]);
   atomicMax((i64 *)&sm->max_queue, (i64)t[6]);
 }
 
@@ -169,7 +170,7 @@ __global__ void __launch_bounds__(JP_THREADS, JP_MINB) k_join_probe(JoinArgs a) 
           const i64 base = a.slot_base[slot];
           if (base >= 0 && c[j] >= a.slot_min[slot] && c[j] <= a.slot_max[slot]) {
             const u32 v = a.table[base + (c[j] - a.slot_min[slot])];
-            lo[j] = v == EMPTY_U32 ? -1 : (int32_t)v;
+            lo[j] = v == 0 ? -1 : (int32_t)~v;
           }
         } else {
           lo[j] = a.found[p];
@@ -239,8 +240,7 @@ __device__ __forceinline__ void launch_emit(ta_join_summary *sm, const u64 *t) {
 }
 
 template <bool DIRECT>
-__global__ void __launch_bounds__(JP_THREADS) k_join_launch_stats(JoinArgs a) {
-  TA_PDL();
+__device__ __forceinline__ void join_launch_stats(const JoinArgs &a) {
   __shared__ u64 red[3][JP_THREADS / 32];
   __shared__ int s_lane0, s_lane1;
   if (ta_failed(a.status)) return;
@@ -296,7 +296,7 @@ __global__ void __launch_bounds__(JP_THREADS) k_join_launch_stats(JoinArgs a) {
         const i64 base = a.slot_base[slot];
         if (base >= 0 && cr[j] >= a.slot_min[slot] && cr[j] <= a.slot_max[slot]) {
           const u32 v = a.table[base + (cr[j] - a.slot_min[slot])];
-          win[j] = v == EMPTY_U32 ? -1 : (int32_t)v;
+          win[j] = v == 0 ? -1 : (int32_t)~v;
         }
       } else {
         win[j] = a.found[p];
@@ -326,6 +326,13 @@ __global__ void __launch_bounds__(JP_THREADS) k_join_launch_stats(JoinArgs a) {
   __syncthreads();
   fold_by_window<3, 0, JP_THREADS / 32>(acc, wm, a.lane_window[l0], a.lane_window[s_lane1], red,
                                         [&](int w, const u64 *t) { launch_emit(&a.sum[w], t); });
+}
+
+template <bool DIRECT>
+__global__ void __launch_bounds__(JP_THREADS) k_join_launch_stats(JoinArgs a, Tail tail) {
+  TA_PDL();
+  join_launch_stats<DIRECT>(a);
+  run_tail(tail);
 }
 
 // ---- general path helpers -----------------------------------------------------
@@ -377,27 +384,20 @@ ta_status ta_run_correlate(ta_window *h, ta_join_summary *out_summary) {
   const int n_slots = W * (h->n_pids > 0 ? h->n_pids : 1);
   cudaStream_t st = h->stream;
   const int64_t nn = n > 0 ? n : 1;
-  size_t keep = 2 * Carver::pad(nn * 4) + 2 * Carver::pad(nn * 8) + Carver::pad((size_t)n_slots * 8) +
-                Carver::pad((size_t)W * sizeof(ta_join_summary)) + 256;
+  size_t keep = Carver::pad(nn * 4) + 2 * Carver::pad(nn * 8) + 256;
   void *kb = ta_dalloc(h, keep);
   if (!kb) return TA_ERR_OOM;
   Carver ck(kb);
-  int32_t *launch_of = ck.take<int32_t>(nn), *kol = ck.take<int32_t>(nn);
+  int32_t *launch_of = ck.take<int32_t>(nn);
   int64_t *latency = ck.take<int64_t>(nn), *qdelay = ck.take<int64_t>(nn);
-  i64 *slot_min = h->d_slot_min, *slot_max = h->d_slot_max;  // filled while the records were gathered
-  i64 *slot_base = ck.take<i64>(n_slots);
-  ta_join_summary *d_sum = ck.take<ta_join_summary>(W);
-
+  ta_status zs;
+  void *zb = ta_zalloc(h, Carver::pad(nn * 4) + Carver::pad((size_t)W * sizeof(ta_join_summary)), &zs);
+  if (!zb) return zs;
+  Carver cz(zb);
+  int32_t *kol = cz.take<int32_t>(nn);
+  ta_join_summary *d_sum = cz.take<ta_join_summary>(W);
   std::vector<ta_join_summary> hs(W);
-  for (auto &s : hs) {
-    memset(&s, 0, sizeof(s));
-    s.min_latency = INT64_MAX;
-    s.max_latency = INT64_MIN;
-  }
-  std::vector<i64> hmin(h->h_slot_min.begin(), h->h_slot_min.end());
-  std::vector<i64> hmax(h->h_slot_max.begin(), h->h_slot_max.end()), hbase(n_slots, -1);
-  TA_CHECK_CUDA(h, cudaMemcpyAsync(d_sum, hs.data(), W * sizeof(ta_join_summary), cudaMemcpyHostToDevice, st));
-  TA_CHECK_CUDA(h, cudaMemsetAsync(kol, 0, nn * 4, st));
+  const std::vector<int64_t> &hmin = h->h_slot_min, &hmax = h->h_slot_max;
 
   JoinArgs a;
   memset(&a, 0, sizeof(a));
@@ -405,7 +405,7 @@ ta_status ta_run_correlate(ta_window *h, ta_join_summary *out_summary) {
   a.kind = h->sorted.kind; a.corr = h->sorted.corr_id; a.ts = h->sorted.ts_start; a.te = h->sorted.ts_end;
   a.lane_off = h->sorted.lane_off; a.lane_slot = h->d_lane_slot; a.lane_window = h->sorted.lane_window;
   a.lane_domain = h->sorted.lane_domain; a.lane_dom_end = h->d_lane_dom_end;
-  a.slot_min = slot_min; a.slot_max = slot_max; a.slot_base = slot_base;
+  a.slot_min = h->d_slot_min; a.slot_max = h->d_slot_max; a.slot_base = h->d_slot_base;  // filled by the sort
   a.launch_of = launch_of; a.kol = kol; a.latency = latency; a.qdelay = qdelay; a.sum = d_sum;
   a.status = h->d_status;
   const unsigned grid = (unsigned)((n + JN_TILE - 1) / JN_TILE);
@@ -413,26 +413,25 @@ ta_status ta_run_correlate(ta_window *h, ta_join_summary *out_summary) {
   const unsigned grid_probe = (unsigned)((n + JP_TILE - 1) / JP_TILE);
   void *tmp_alloc = nullptr;
   bool direct = true;
+  int32_t words[ST_WORDS];
+  const bool small = W * sizeof(ta_join_summary) <= 4096;  // (more is copied once the kernels are queued)
+  TA_TRY(ta_queue_d2h(h, words, h->d_status, sizeof(words)));
+  if (small) TA_TRY(ta_queue_d2h(h, hs.data(), d_sum, W * sizeof(ta_join_summary)));
   if (n > 0) {
     // table size if every slot is addressed directly
     unsigned __int128 total = 0;
     for (int s = 0; s < n_slots; s++)
-      if (hmin[s] <= hmax[s]) {
-        hbase[s] = (i64)total;
-        total += (unsigned __int128)((uint64_t)hmax[s] - (uint64_t)hmin[s]) + 1;
-      }
+      if (hmin[s] <= hmax[s]) total += (unsigned __int128)((uint64_t)hmax[s] - (uint64_t)hmin[s]) + 1;
     const uint64_t limit = (uint64_t)4 * (uint64_t)n + 65536;
     direct = total <= limit;
     if (direct) {
       uint64_t M = (uint64_t)total;
-      tmp_alloc = ta_dalloc(h, (size_t)(M > 0 ? M : 1) * 4);
-      if (!tmp_alloc) return TA_ERR_OOM;
+      tmp_alloc = ta_zalloc(h, (size_t)(M > 0 ? M : 1) * 4, &zs);
+      if (!tmp_alloc) return zs;
       a.table = (u32 *)tmp_alloc;
-      TA_CHECK_CUDA(h, cudaMemsetAsync(a.table, 0xFF, (size_t)(M > 0 ? M : 1) * 4, st));
-      TA_CHECK_CUDA(h, cudaMemcpyAsync(slot_base, hbase.data(), n_slots * 8, cudaMemcpyHostToDevice, st));
       ta_launch(k_join_build, grid, JN_THREADS, 0, st, a);
       ta_launch(k_join_probe<true>, grid_probe, JP_THREADS, 0, st, a);
-      ta_launch(k_join_launch_stats<true>, grid8, JP_THREADS, 0, st, a);
+      ta_launch(k_join_launch_stats<true>, grid8, JP_THREADS, 0, st, a, ta_tail(h, grid8));
     } else {
       // general path: compact, sort by (slot, corr) with sorted position as the stable tie-break
       size_t tb = Carver::pad(nn * 4) * 3 + Carver::pad(nn * 8) * 3 + scan_temp_bytes(n) * 2 +
@@ -454,6 +453,8 @@ ta_status ta_run_correlate(ta_window *h, ta_join_summary *out_summary) {
       u64 m64 = 0;
       TA_TRY(ta_queue_d2h(h, &m64, t1.total, 8));
       TA_TRY(ta_sync_fetch(h));
+      TA_TRY(ta_queue_d2h(h, words, h->d_status, sizeof(words)));
+      if (small) TA_TRY(ta_queue_d2h(h, hs.data(), d_sum, W * sizeof(ta_join_summary)));
       const int64_t m = (int64_t)m64;
       TA_CHECK_CUDA(h, cudaMemsetAsync(found, 0xFF, nn * 4, st));
       if (m > 0) {
@@ -475,19 +476,19 @@ ta_status ta_run_correlate(ta_window *h, ta_join_summary *out_summary) {
       }
       a.found = found;
       ta_launch(k_join_probe<false>, grid_probe, JP_THREADS, 0, st, a);
-      ta_launch(k_join_launch_stats<false>, grid8, JP_THREADS, 0, st, a);
+      ta_launch(k_join_launch_stats<false>, grid8, JP_THREADS, 0, st, a, ta_tail(h, grid8));
     }
     TA_CHECK_CUDA(h, cudaGetLastError());
   }
-  TA_TRY(ta_queue_d2h(h, hs.data(), d_sum, W * sizeof(ta_join_summary)));
-  int32_t words[ST_WORDS];
-  TA_TRY(ta_read_status(h, words));
+  if (!small) TA_TRY(ta_queue_d2h(h, hs.data(), d_sum, W * sizeof(ta_join_summary)));
+  TA_TRY(ta_sync_fetch(h));
   if (tmp_alloc) ta_dfree(h, tmp_alloc);
   if (words[ST_ERR]) return (ta_status)words[ST_ERR];
   for (int w = 0; w < W; w++) {
     ta_join_summary &s = hs[w];
     s.n_unmatched = s.n_probe - s.n_matched;
-    if (s.n_matched == 0) { s.min_latency = 0; s.max_latency = 0; }
+    s.max_latency = s.n_matched ? unbias64((u64)s.max_latency) : 0;
+    s.min_latency = s.n_matched ? unbias64(~(u64)s.min_latency) : 0;
     if (out_summary) out_summary[w] = s;
   }
   h->join.launch_of = launch_of;

@@ -12,8 +12,8 @@
 //                   takes the digit histograms of the radix passes over the time bits and
 //                   counts the records of every triple, so that the first radix pass can build
 //                   the keys itself and no separate key pass is needed;
-//   k_top_hist*     digit histograms of the passes over the (window, lane) bits, from the
-//                   per-triple counts (one window) or from the words (several);
+//   k_top_hist_words  digit histograms of the passes over the (window, lane) bits of several
+//                   windows (of one window they follow from the per-triple counts);
 //   k_rank_*        one CTA each: sort and rank the few triples / communicator ids;
 //   k_load_pre      turns those words into keys in place - [dropped][window][triple
 //                   rank][(ts_start - t0) >> dshift]{[index in window]} - and takes the
@@ -23,7 +23,7 @@
 #include "ta_internal.cuh"
 #include "records.cuh"
 
-#define TRIPLE_EMPTY (~0ull)
+#define TRIPLE_EMPTY (~0ull)  // in the per-CTA caches and the sampling table
 
 __device__ __forceinline__ i64 warp_min_i64(i64 v) {
 #pragma unroll
@@ -83,10 +83,10 @@ __global__ void __launch_bounds__(256) k_discover(const ta_event *ev, int64_t n,
         bool ok = false;
         for (int probe = 0; probe < TA_COMM_SLOTS; probe++) {
           u64 cur = ld_relaxed(&cm->slots[slot]);
-          if (cur == cc) { ok = true; break; }
-          if (cur == TRIPLE_EMPTY) {
-            u64 old = atomicCAS(&cm->slots[slot], TRIPLE_EMPTY, cc);
-            if (old == TRIPLE_EMPTY || old == cc) { ok = true; break; }
+          if (cur == ~cc) { ok = true; break; }
+          if (cur == 0) {
+            u64 old = atomicCAS(&cm->slots[slot], 0ull, ~cc);
+            if (old == 0 || old == ~cc) { ok = true; break; }
           }
           slot = (slot + 1) & (TA_COMM_SLOTS - 1);
         }
@@ -106,10 +106,10 @@ __global__ void __launch_bounds__(256) k_discover(const ta_event *ev, int64_t n,
     bool done = false;
     for (int probe = 0; probe < TA_TRIPLE_SLOTS; probe++) {
       u64 cur = ld_relaxed(&tt->slots[slot]);
-      if (cur == code) { done = true; break; }
-      if (cur == TRIPLE_EMPTY) {
-        u64 old = atomicCAS(&tt->slots[slot], TRIPLE_EMPTY, code);
-        if (old == TRIPLE_EMPTY || old == code) { done = true; break; }
+      if (cur == code + 1) { done = true; break; }
+      if (cur == 0) {
+        u64 old = atomicCAS(&tt->slots[slot], 0ull, code + 1);
+        if (old == 0 || old == code + 1) { done = true; break; }
       }
       slot = (slot + 1) & (TA_TRIPLE_SLOTS - 1);
     }
@@ -148,11 +148,24 @@ __global__ void __launch_bounds__(256) k_discover(const ta_event *ev, int64_t n,
 #define PL_THREADS 1024
 #define PL_PER_THREAD 4
 #define PL_SLOTS 2048
-__global__ void __launch_bounds__(PL_THREADS) k_plan(const ta_event *ev, int64_t n, const int64_t *off,
+// Before that it writes down what the other kernels of the call expect in memory: the bounds of the
+// windows when they came as arguments (a copy costs more than the kernel), and where the value
+// ranges start.
+struct PlanWindows {
+  int64_t v[3 * TA_PLAN_WINDOWS + 1];  // off, t0, t1 as they lie in memory
+  int n;                               // 0: the bounds were copied
+};
+__global__ void __launch_bounds__(PL_THREADS) k_plan(const ta_event *ev, int64_t n, int64_t *off,
                                                      const int64_t *t0, const int64_t *t1, int W,
                                                      int sbits, int64_t max_span, int64_t max_win,
-                                                     int64_t *misc) {
+                                                     int64_t *misc, PlanWindows pw, int sample) {
   TA_PDL();
+  if (threadIdx.x < pw.n) off[threadIdx.x] = pw.v[threadIdx.x];
+  if (threadIdx.x < 16) {  // [0] / [1] smallest / largest name, [3] / [4] sequence number, the rest 0
+    const int k = threadIdx.x;
+    misc[k] = k == 0 || k == 3 ? INT64_MAX : k == 1 || k == 4 ? INT64_MIN : 0;
+  }
+  if (!sample) return;
   __shared__ u64 code[PL_SLOTS];
   __shared__ u32 cnt[PL_SLOTS];
   __shared__ u32 s_max, s_valid;
@@ -378,10 +391,10 @@ __global__ void __launch_bounds__(DS_THREADS) k_discover_staged(DiscoverArgs a) 
               bool ok = false;
               for (int probe = 0; probe < TA_COMM_SLOTS; probe++) {
                 const u64 c2 = ld_relaxed(&a.cm->slots[slot]);
-                if (c2 == cc) { ok = true; break; }
-                if (c2 == TRIPLE_EMPTY) {
-                  const u64 old = atomicCAS(&a.cm->slots[slot], TRIPLE_EMPTY, cc);
-                  if (old == TRIPLE_EMPTY || old == cc) { ok = true; break; }
+                if (c2 == ~cc) { ok = true; break; }
+                if (c2 == 0) {
+                  const u64 old = atomicCAS(&a.cm->slots[slot], 0ull, ~cc);
+                  if (old == 0 || old == ~cc) { ok = true; break; }
                 }
                 slot = (slot + 1) & (TA_COMM_SLOTS - 1);
               }
@@ -400,10 +413,10 @@ __global__ void __launch_bounds__(DS_THREADS) k_discover_staged(DiscoverArgs a) 
             bool done = false;
             for (int probe = 0; probe < TA_TRIPLE_SLOTS; probe++) {
               const u64 c2 = ld_relaxed(&a.tt->slots[slot]);
-              if (c2 == code) { done = true; break; }
-              if (c2 == TRIPLE_EMPTY) {
-                const u64 old = atomicCAS(&a.tt->slots[slot], TRIPLE_EMPTY, code);
-                if (old == TRIPLE_EMPTY || old == code) { done = true; break; }
+              if (c2 == code + 1) { done = true; break; }
+              if (c2 == 0) {
+                const u64 old = atomicCAS(&a.tt->slots[slot], 0ull, code + 1);
+                if (old == 0 || old == code + 1) { done = true; break; }
               }
               slot = (slot + 1) & (TA_TRIPLE_SLOTS - 1);
             }
@@ -473,16 +486,14 @@ __global__ void __launch_bounds__(DS_THREADS) k_discover_staged(DiscoverArgs a) 
 }
 
 // ---- histograms of the passes over the (dropped, window, triple rank) bits ------------------
+// (of a single window they follow from the records counted per triple: k_radix_scan_hist)
 struct TopHistArgs {
   SortPlan plan;        // the whole plan; passes [n_time, n_pass) are the top passes
   int n_time;
   int top_lo;           // key bit where the top bits begin (index bits + time bits kept)
   int tbits, wbits;
-  int64_t n_dropped;
   const TripleTable *tt;
-  const u32 *slot_cnt;
   u32 *hist;            // [pass][256]
-  // several windows: from the words
   const u64 *prekey;
   int64_t n;
   const int64_t *off;
@@ -492,20 +503,6 @@ __device__ __forceinline__ void top_hist_add(const TopHistArgs &a, u32 *hist, u6
   for (int p = a.n_time; p < a.plan.n_pass; p++) {
     const u32 d = (u32)(c >> (a.plan.shift[p] - a.top_lo)) & ((1u << a.plan.bits[p]) - 1u);
     atomicAdd(&hist[p * 256 + d], count);
-  }
-}
-// one window: the lane sizes are the per-triple counts
-__global__ void __launch_bounds__(1024) k_top_hist(TopHistArgs a) {
-  TA_PDL();
-  for (int sl = threadIdx.x; sl < TA_TRIPLE_SLOTS; sl += blockDim.x) {
-    const u32 c = a.slot_cnt[sl];
-    if (c) top_hist_add(a, a.hist, (u64)a.tt->rank_of_slot[sl], c);
-  }
-  if (threadIdx.x == 0) {
-    if (a.n_dropped > 0) {
-      top_hist_add(a, a.hist, 1ull << (a.wbits + a.tbits), (u32)a.n_dropped);
-      for (int p = 0; p < a.n_time; p++) atomicAdd(&a.hist[p * 256], (u32)a.n_dropped);  // time digits 0
-    }
   }
 }
 // several windows: one pass over the words (8 bytes per record)
@@ -575,7 +572,8 @@ __device__ __forceinline__ void block_sort(u64 *buf, int n) {
 // of triples: the occupied slots are packed to the front in any order, as code << 13 | slot, so
 // that the sorted entry names its slot; the table is read once and only its occupied slots are
 // written (two passes over all slots in block-scan rounds and a serial pid walk took 20 us).
-__device__ __forceinline__ void rank_triples(TripleTable *tt, int32_t *status, u64 *buf /* TA_TRIPLE_SLOTS */) {
+__device__ __forceinline__ void rank_triples(TripleTable *tt, const u32 *slot_cnt, int32_t *status,
+                                             u64 *buf /* TA_TRIPLE_SLOTS */) {
   __shared__ u64 tmp[33];
   __shared__ int n_tr;
   const int tid = threadIdx.x;
@@ -583,7 +581,7 @@ __device__ __forceinline__ void rank_triples(TripleTable *tt, int32_t *status, u
   __syncthreads();
   for (int s = tid; s < TA_TRIPLE_SLOTS; s += blockDim.x) {
     const u64 v = tt->slots[s];
-    if (v != TRIPLE_EMPTY) buf[atomicAdd(&n_tr, 1)] = (v << 13) | (u64)s;
+    if (v) buf[atomicAdd(&n_tr, 1)] = ((v - 1) << 13) | (u64)s;
   }
   __syncthreads();
   block_sort(buf, n_tr);
@@ -604,6 +602,7 @@ __device__ __forceinline__ void rank_triples(TripleTable *tt, int32_t *status, u
       tt->sorted_code[i] = c;
       tt->rank_of_slot[(u32)buf[i] & (TA_TRIPLE_SLOTS - 1)] = i;
       tt->pid_rank[i] = pr;
+      tt->rank_cnt[i] = slot_cnt[(u32)buf[i] & (TA_TRIPLE_SLOTS - 1)];
       if (head) tt->pid_value[pr] = (int32_t)((u32)(c >> 17) ^ 0x80000000u);
     }
     pids += (int)total;
@@ -623,9 +622,9 @@ __device__ __forceinline__ void rank_comms(CommTable *cm, int32_t *status, u64 *
   __syncthreads();
   for (int s = tid; s < TA_COMM_SLOTS; s += blockDim.x) {
     const u64 v = cm->slots[s];
-    if (v != TRIPLE_EMPTY) {
+    if (v) {
       const int at = atomicAdd(&n_c, 1);
-      buf[at] = v;
+      buf[at] = ~v;
       slot_of[at] = (u32)s;
     }
   }
@@ -637,7 +636,7 @@ __device__ __forceinline__ void rank_comms(CommTable *cm, int32_t *status, u64 *
   if (n > TA_MAX_COMMS && tid == 0) ta_set_err(status, TA_ERR_TOO_LARGE);
   for (int i = tid; i < n && i < TA_MAX_COMMS; i += blockDim.x) cm->sorted_id[i] = buf[i];
   for (int i = tid; i < n; i += blockDim.x) {
-    const u64 c = cm->slots[slot_of[i]];
+    const u64 c = ~cm->slots[slot_of[i]];
     int lo = 0, hi = n - 1;
     while (lo < hi) {
       int mid = (lo + hi) >> 1;
@@ -650,11 +649,13 @@ __device__ __forceinline__ void rank_comms(CommTable *cm, int32_t *status, u64 *
 
 // Both rankings in one launch: CTA 0 the triples, CTA 1 the communicator ids (they are
 // independent, and two single-CTA kernels one after the other cost a launch latency more).
-__global__ void __launch_bounds__(1024) k_rank(TripleTable *tt, CommTable *cm, int32_t *status) {
+__global__ void __launch_bounds__(1024) k_rank(TripleTable *tt, CommTable *cm, const u32 *slot_cnt,
+                                               int32_t *status, Tail tail) {
   TA_PDL();
   extern __shared__ u64 rank_buf[];  // TA_TRIPLE_SLOTS
-  if (blockIdx.x == 0) rank_triples(tt, status, rank_buf);
+  if (blockIdx.x == 0) rank_triples(tt, slot_cnt, status, rank_buf);
   else rank_comms(cm, status, rank_buf);
+  run_tail(tail);
 }
 
 struct LoadArgs {
@@ -696,7 +697,7 @@ __global__ void __launch_bounds__(256) k_load(LoadArgs a) {
         // behind the library's back (the records are borrowed): bounded probe, error, rank 0
         u32 slot = hash_code(code) & (TA_TRIPLE_SLOTS - 1);
         int probes = 0;
-        while (__ldg(&a.tt->slots[slot]) != code && ++probes < TA_TRIPLE_SLOTS)
+        while (__ldg(&a.tt->slots[slot]) != code + 1 && ++probes < TA_TRIPLE_SLOTS)
           slot = (slot + 1) & (TA_TRIPLE_SLOTS - 1);
         u64 rank = 0;
         if (probes < TA_TRIPLE_SLOTS) rank = (u64)__ldg(&a.tt->rank_of_slot[slot]);
@@ -788,17 +789,27 @@ static int grid_for(int64_t n, int threads, int per_sm) {
 ta_status ta_launch_discover(ta_window *h) {
   h->tkeep = 0;
   h->fast_keys = 0;
+  int64_t max_span = 1, max_win = 1;
+  for (int w = 0; w < h->W; w++) {
+    max_span = max_span > h->h_t1[w] - h->h_t0[w] ? max_span : h->h_t1[w] - h->h_t0[w];
+    max_win = max_win > h->h_off[w + 1] - h->h_off[w] ? max_win : h->h_off[w + 1] - h->h_off[w];
+  }
+  const int sbits = ta_bit_len((uint64_t)(max_span - 1));
+  // 16-byte aligned records: plan the time resolution, then the staged pass that also takes
+  // the histograms of the time passes and the per-triple counts
+  const bool staged = h->n > 0 && ((uintptr_t)h->events & 15u) == 0;
+  PlanWindows pw;
+  memset(&pw, 0, sizeof(pw));
+  if (h->W <= TA_PLAN_WINDOWS) {
+    pw.n = 3 * h->W + 1;
+    memcpy(pw.v, h->h_off.data(), (size_t)(h->W + 1) * 8);
+    memcpy(pw.v + h->W + 1, h->h_t0.data(), (size_t)h->W * 8);
+    memcpy(pw.v + 2 * h->W + 1, h->h_t1.data(), (size_t)h->W * 8);
+  }
+  ta_launch(k_plan, 1, PL_THREADS, 0, h->stream, h->events, h->n, h->d_off, h->d_t0, h->d_t1, h->W, sbits, max_span,
+            max_win, h->d_misc, pw, staged ? 1 : 0);
   if (h->n > 0) {
-    if (((uintptr_t)h->events & 15u) == 0) {
-      // 16-byte aligned records: plan the time resolution, then the staged pass that also takes
-      // the histograms of the time passes and the per-triple counts
-      int64_t max_span = 1, max_win = 1;
-      for (int w = 0; w < h->W; w++) {
-        max_span = max_span > h->h_t1[w] - h->h_t0[w] ? max_span : h->h_t1[w] - h->h_t0[w];
-        max_win = max_win > h->h_off[w + 1] - h->h_off[w] ? max_win : h->h_off[w + 1] - h->h_off[w];
-      }
-      const int sbits = ta_bit_len((uint64_t)(max_span - 1));
-      ta_launch(k_plan, 1, PL_THREADS, 0, h->stream, h->events, h->n, h->d_off, h->d_t0, h->d_t1, h->W, sbits, max_span, max_win, h->d_misc);
+    if (staged) {
       DiscoverArgs a;
       a.ev = h->events; a.n = h->n; a.off = h->d_off; a.t0 = h->d_t0; a.t1 = h->d_t1; a.W = h->W;
       a.tt = h->d_triples; a.cm = h->d_comms; a.sum = h->d_load_sum; a.misc = h->d_misc;
@@ -821,7 +832,8 @@ ta_status ta_launch_discover(ta_window *h) {
   }
   TA_CHECK_CUDA(h, cudaFuncSetAttribute(k_rank, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         TA_TRIPLE_SLOTS * (int)sizeof(u64)));
-  ta_launch(k_rank, 2, 1024, TA_TRIPLE_SLOTS * sizeof(u64), h->stream, h->d_triples, h->d_comms, h->d_status);
+  ta_launch(k_rank, 2, 1024, TA_TRIPLE_SLOTS * sizeof(u64), h->stream, h->d_triples, h->d_comms, h->d_slot_cnt,
+            h->d_status, ta_tail(h, 2));
   TA_CHECK_CUDA(h, cudaGetLastError());
   return TA_OK;
 }
@@ -848,6 +860,7 @@ ta_status ta_launch_load(ta_window *h, bool allow_packed) {
   h->ibits = ta_bit_len((uint64_t)(max_win - 1));
   if (h->ibits < 1) h->ibits = 1;
   h->fast_keys = 0;
+  h->top.rank_cnt = nullptr;
   if (allow_packed && h->prekeys && h->tkeep > 0 && h->tkeep <= h->sbits) {
     // The staged discovery pass took the histograms of the passes over the time bits kept, and
     // the lane sizes give those of the passes above them: the first radix pass can build the
@@ -868,14 +881,18 @@ ta_status ta_launch_load(ta_window *h, bool allow_packed) {
       h->plan.n_pass = tp.n_pass + n_top;
       h->fast_keys = 1;
       if (h->n == 0) return TA_OK;
+      if (h->W == 1) {  // k_radix_scan_hist completes the histograms
+        TopHist &t = h->top;
+        t.plan = h->plan; t.n_time = tp.n_pass; t.top_lo = h->ibits + T; t.tbits = h->tbits; t.wbits = h->wbits;
+        t.n_triples = h->n_triples; t.n_dropped = (u32)(h->n - h->n_valid); t.rank_cnt = h->d_triples->rank_cnt;
+        return TA_OK;
+      }
       TopHistArgs a;
       memset(&a, 0, sizeof(a));
       a.plan = h->plan; a.n_time = tp.n_pass; a.top_lo = h->ibits + T;
-      a.tbits = h->tbits; a.wbits = h->wbits; a.n_dropped = h->n - h->n_valid;
-      a.tt = h->d_triples; a.slot_cnt = h->d_slot_cnt; a.hist = h->d_hist;
+      a.tbits = h->tbits; a.wbits = h->wbits; a.tt = h->d_triples; a.hist = h->d_hist;
       a.prekey = h->d_keys; a.n = h->n; a.off = h->d_off; a.W = h->W;
-      if (h->W == 1) ta_launch(k_top_hist, 1, 1024, 0, h->stream, a);
-      else ta_launch(k_top_hist_words, grid_for(h->n, 256, 8), 256, 0, h->stream, a);
+      ta_launch(k_top_hist_words, grid_for(h->n, 256, 8), 256, 0, h->stream, a);
       TA_CHECK_CUDA(h, cudaGetLastError());
       return TA_OK;  // the words stay in d_keys (h->prekeys stays set): a retry can still use them
     }

@@ -332,11 +332,12 @@ ta_status ta_run_overlap(ta_window *h, ta_overlap_result *out) {
   ScanTemp s3;
   TA_TRY(scan_temp_init(h, scan_mem, n_slots, &s3));
   OvRowIn ri{sa.acc};
-  TA_TRY((launch_scan<OpAdd, OvRowIn, OvRowOut>(h, n_slots, ri, ro, OpAdd(), s3)));
   u64 rows = 0;
-  TA_TRY(ta_queue_d2h(h, &rows, s3.total, 8));
   int32_t words[ST_WORDS];
-  TA_TRY(ta_read_status(h, words));
+  TA_TRY(ta_queue_d2h(h, &rows, s3.total, 8));
+  TA_TRY(ta_queue_d2h(h, words, h->d_status, sizeof(words)));
+  TA_TRY((launch_scan<OpAdd, OvRowIn, OvRowOut>(h, n_slots, ri, ro, OpAdd(), s3, true)));
+  TA_TRY(ta_sync_fetch(h));
   ta_dfree(h, tmpb);
   if (words[ST_ERR]) return (ta_status)words[ST_ERR];
   out->n_rows = (int64_t)rows;

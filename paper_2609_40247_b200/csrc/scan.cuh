@@ -29,17 +29,21 @@ static inline size_t scan_temp_carve(void *mem, int64_t n, ScanTemp *t) {
   t->total = sc;
   return c.off;
 }
-// carves and zeroes the temp (one memset)
+// carves the temp out of the handle's cleared pool, or out of `mem` and clears it
 static inline ta_status scan_temp_init(ta_window *h, void *mem, int64_t n, ScanTemp *t) {
+  void *zeroed = ta_zpool(h, scan_temp_bytes(n));
+  if (zeroed) {
+    scan_temp_carve(zeroed, n, t);
+    return TA_OK;
+  }
   TA_CHECK_CUDA(h, cudaMemsetAsync(mem, 0, scan_temp_carve(mem, n, t), h->stream));
   return TA_OK;
 }
 
 #ifdef __CUDACC__
 template <class Op, class In, class Out>
-__global__ void __launch_bounds__(SC_THREADS) k_scan(int64_t n, In in, Out out, Op op, ScanTemp t,
-                                                     int32_t *status) {
-  TA_PDL();
+__device__ __forceinline__ void scan_tile(int64_t n, const In &in, const Out &out, Op op, const ScanTemp &t,
+                                          int32_t *status) {
   __shared__ u64 tmp[33];
   __shared__ u64 s_excl;
   __shared__ int s_tile, s_fail;
@@ -81,10 +85,22 @@ __global__ void __launch_bounds__(SC_THREADS) k_scan(int64_t n, In in, Out out, 
 }
 
 template <class Op, class In, class Out>
-static inline ta_status launch_scan(ta_window *h, int64_t n, In in, Out out, Op op, ScanTemp t) {
+__global__ void __launch_bounds__(SC_THREADS) k_scan(int64_t n, In in, Out out, Op op, ScanTemp t,
+                                                     int32_t *status, Tail tail) {
+  TA_PDL();
+  scan_tile<Op, In, Out>(n, in, out, op, t, status);
+  run_tail(tail);
+}
+
+// last: the scan is the last kernel of its call, and what is queued for the host may ride on it
+template <class Op, class In, class Out>
+static inline ta_status launch_scan(ta_window *h, int64_t n, In in, Out out, Op op, ScanTemp t, bool last = false) {
   if (n <= 0) return TA_OK;
   int64_t tiles = (n + SC_TILE - 1) / SC_TILE;
-  ta_launch(k_scan<Op, In, Out>, (unsigned)tiles, SC_THREADS, 0, h->stream, n, in, out, op, t, h->d_status);
+  Tail tail;
+  tail.m = 0;
+  if (last) tail = ta_tail(h, tiles);
+  ta_launch(k_scan<Op, In, Out>, (unsigned)tiles, SC_THREADS, 0, h->stream, n, in, out, op, t, h->d_status, tail);
   TA_CHECK_CUDA(h, cudaGetLastError());
   return TA_OK;
 }

@@ -11,6 +11,8 @@
 // pass is instruction-bound on B200, so the kernel is specialised on the digit
 // width and on full tiles, and every key costs one population count, one
 // shared-memory atomic and as many warp votes as the digit has bits.
+#include <cstring>
+
 #include "ta_internal.cuh"
 
 #define RS_BINS 256
@@ -391,13 +393,31 @@ __global__ void __launch_bounds__(256) k_radix_hist(const u64 *keys, int64_t n, 
 }
 
 // exclusive scan of each pass's histogram: one CTA of 256 threads per pass
-__global__ void __launch_bounds__(256) k_radix_scan_hist(const u32 *hist, u32 *bin_offset) {
+__global__ void __launch_bounds__(256) k_radix_scan_hist(const u32 *hist, u32 *bin_offset, TopHist top) {
   TA_PDL();
   __shared__ u64 tmp[33];
+  __shared__ u32 sh[RS_BINS];
+  const int p = blockIdx.x, tid = threadIdx.x;
   u64 total;
-  u32 v = hist[blockIdx.x * RS_BINS + threadIdx.x];
+  u32 v;
+  if (top.rank_cnt && p >= top.n_time) {  // from the records counted per lane
+    sh[tid] = 0;
+    __syncthreads();
+    const int shift = top.plan.shift[p] - top.top_lo;
+    const u32 mask = (1u << top.plan.bits[p]) - 1u;
+    for (int r = tid; r < top.n_triples; r += 256) {
+      const u32 c = top.rank_cnt[r];
+      if (c) atomicAdd(&sh[(u32)((u64)r >> shift) & mask], c);
+    }
+    if (tid == 0 && top.n_dropped) atomicAdd(&sh[(u32)((1ull << (top.wbits + top.tbits)) >> shift) & mask], top.n_dropped);
+    __syncthreads();
+    v = sh[tid];
+  } else {
+    v = hist[p * RS_BINS + tid];
+    if (top.rank_cnt && tid == 0) v += top.n_dropped;  // their time digits are 0
+  }
   u64 ex = block_scan_exclusive<OpAdd>((u64)v, OpAdd(), tmp, &total);
-  bin_offset[blockIdx.x * RS_BINS + threadIdx.x] = (u32)ex;
+  bin_offset[p * RS_BINS + tid] = (u32)ex;
 }
 
 SortPlan ta_make_plan(int lo_bit, int hi_bit) { return ta_plan_bits(lo_bit, hi_bit); }
@@ -407,11 +427,16 @@ static size_t min_tile() {
   return a < b ? a : b;
 }
 
-size_t ta_sort_temp_bytes(int64_t n) {
+// Descriptors of all passes are cleared at once while that is little memory (keys-only passes: 1 KB
+// per tile and pass); for more records each keys-only pass has the one array cleared in front of it.
+#define RS_AT_ONCE (1ll << 20)
+static size_t state_bytes(int64_t n) {
   size_t tiles = (size_t)((n + (int64_t)min_tile() - 1) / (int64_t)min_tile());
   if (tiles == 0) tiles = 1;
-  return Carver::pad(tiles * RS_BINS * sizeof(u64)) + Carver::pad(16 * sizeof(u32)) +
-         2 * Carver::pad(10 * RS_BINS * sizeof(u32));
+  return Carver::pad(tiles * RS_BINS * sizeof(u64) * (n <= RS_AT_ONCE ? 5 : 1));
+}
+size_t ta_sort_temp_bytes(int64_t n) {
+  return state_bytes(n) + Carver::pad(16 * sizeof(u32)) + 2 * Carver::pad(10 * RS_BINS * sizeof(u32));
 }
 
 template <int THREADS, int ITEMS, bool VALS, bool STABLE, bool PREKEY = false>
@@ -442,30 +467,38 @@ template <bool VALS>
 static ta_status radix_sort(ta_window *h, const u64 *keys_in, const u32 *vals_in, u64 *keys_scratch,
                             u32 *vals_scratch, u64 *keys_final, u32 *vals_final, int64_t n,
                             const SortPlan &plan, const u32 *hist, void *temp,
-                            bool first_pass_unstable, const PrekeyInfo *prekey) {
+                            bool first_pass_unstable, const PrekeyInfo *prekey, const TopHist *top) {
   if (n <= 0) return TA_OK;
   constexpr int THREADS = VALS ? RSP_THREADS : RSK_THREADS;
   constexpr int ITEMS = VALS ? RSP_ITEMS : RSK_ITEMS;
   constexpr int TILE = THREADS * ITEMS;
   size_t tiles = (size_t)((n + TILE - 1) / TILE);
-  Carver c(temp);
-  size_t max_tiles = (size_t)((n + (int64_t)min_tile() - 1) / (int64_t)min_tile());
-  u64 *state = c.take<u64>(max_tiles * RS_BINS);
-  u32 *counter = c.take<u32>(16);
-  u32 *bin_offset = c.take<u32>(10 * RS_BINS);
-  u32 *own_hist = c.take<u32>(10 * RS_BINS);
+  // what the sort has to find cleared, in one piece: tile descriptors, ticket counters (one per
+  // pass) and the histograms if there are none yet
+  const bool at_once = n <= RS_AT_ONCE;
+  const size_t per_pass = tiles * (VALS ? RS_BINS : RS_BINS / 2);  // descriptors
+  const size_t arrays = VALS || !at_once ? 1 : (size_t)plan.n_pass;
+  const size_t zero = Carver::pad(per_pass * arrays * sizeof(u64)) + Carver::pad(16 * sizeof(u32)) +
+                      (hist ? 0 : Carver::pad(10 * RS_BINS * sizeof(u32)));
   cudaStream_t st = h->stream;
+  Carver c(temp);
+  u32 *bin_offset = c.take<u32>(10 * RS_BINS);
+  void *zeroed = ta_zpool(h, zero);
+  Carver cz(zeroed ? zeroed : (void *)(c.base + c.off));
+  u64 *state = cz.take<u64>(per_pass * arrays);
+  u32 *counter = cz.take<u32>(16);
+  if (!zeroed) TA_CHECK_CUDA(h, cudaMemsetAsync(state, 0, zero, st));
   if (!hist) {
-    TA_CHECK_CUDA(h, cudaMemsetAsync(own_hist, 0, 10 * RS_BINS * sizeof(u32), st));
+    u32 *own_hist = cz.take<u32>(10 * RS_BINS);
     int64_t want = (n + 255) / 256;
     int grid = (int)(want < 148 * 8 ? want : 148 * 8);
     ta_launch(k_radix_hist, grid, 256, 0, st, keys_in, n, plan, own_hist);
     hist = own_hist;
   }
-  ta_launch(k_radix_scan_hist, plan.n_pass, 256, 0, st, hist, bin_offset);
-  // one clearing for all passes of a pair sort (descriptors tagged with their pass); every pass
-  // draws its tile tickets from a counter of its own (state and counters are neighbours)
-  TA_CHECK_CUDA(h, cudaMemsetAsync(state, 0, (size_t)((char *)(counter + 16) - (char *)state), st));
+  TopHist th;
+  if (top) th = *top;
+  else memset(&th, 0, sizeof(th));
+  ta_launch(k_radix_scan_hist, plan.n_pass, 256, 0, st, hist, bin_offset, th);
   const u64 *kin = keys_in;
   const u32 *vin = vals_in;
   for (int p = 0; p < plan.n_pass; p++) {
@@ -475,9 +508,9 @@ static ta_status radix_sort(ta_window *h, const u64 *keys_in, const u32 *vals_in
     a.vals_in = vin; a.vals_out = to_final ? vals_final : vals_scratch;
     a.n = n; a.shift = plan.shift[p];
     a.bin_offset = bin_offset + p * RS_BINS;
-    if (!VALS && p > 0)  // untagged descriptors: cleared in front of every pass
-      TA_CHECK_CUDA(h, cudaMemsetAsync(state, 0, tiles * (RS_BINS / 2) * sizeof(u64), st));
-    a.tile_state = state; a.tile_counter = counter + p; a.status = h->d_status;
+    if (!VALS && p > 0 && !at_once)  // untagged descriptors: cleared in front of every pass
+      TA_CHECK_CUDA(h, cudaMemsetAsync(state, 0, per_pass * sizeof(u64), st));
+    a.tile_state = state + (at_once && !VALS ? (size_t)p * per_pass : 0); a.tile_counter = counter + p; a.status = h->d_status;
     a.gen = VALS ? (u32)(p + 1) : 0u;
     const bool timed = g_ta_profile && n == h->n;  // only the timeline sort (all records)
     if (timed) ta_profile_mark(st, 1, (VALS ? 24.0 : 16.0) * (double)n);
@@ -508,12 +541,12 @@ ta_status ta_radix_sort_pairs(ta_window *h, const u64 *keys_in, const u32 *vals_
                               u32 *vals_final, int64_t n, const SortPlan &plan, const u32 *hist,
                               void *temp) {
   return radix_sort<true>(h, keys_in, vals_in, keys_scratch, vals_scratch, keys_final, vals_final, n,
-                          plan, hist, temp, false, nullptr);
+                          plan, hist, temp, false, nullptr, nullptr);
 }
 
 ta_status ta_radix_sort_keys(ta_window *h, const u64 *keys_in, u64 *keys_scratch, u64 *keys_final,
                              int64_t n, const SortPlan &plan, const u32 *hist, void *temp,
-                             bool first_pass_unstable, const PrekeyInfo *prekey) {
+                             bool first_pass_unstable, const PrekeyInfo *prekey, const TopHist *top) {
   return radix_sort<false>(h, keys_in, nullptr, keys_scratch, nullptr, keys_final, nullptr, n, plan,
-                           hist, temp, first_pass_unstable, prekey);
+                           hist, temp, first_pass_unstable, prekey, top);
 }

@@ -2,6 +2,7 @@
 // through the caller's allocator, call-order bookkeeping.  All arithmetic lives
 // in the kernels of the other translation units.
 #include <atomic>
+#include <cstddef>
 #include <cstring>
 #include <mutex>
 #include <new>
@@ -106,6 +107,26 @@ void *ta_dalloc(ta_window *h, size_t bytes) {
   if (p) {
     h->allocs.push_back(p);
     h->alloc_bytes.push_back(bytes);
+  }
+  return p;
+}
+
+void *ta_zpool(ta_window *h, size_t bytes) {
+  const size_t need = Carver::pad(bytes ? bytes : 1);
+  if (h->zero_used + need > h->zero_bytes) return nullptr;
+  void *p = h->zero_pool + h->zero_used;
+  h->zero_used += need;
+  return p;
+}
+void *ta_zalloc(ta_window *h, size_t bytes, ta_status *st) {
+  *st = TA_OK;
+  void *p = ta_zpool(h, bytes);
+  if (p) return p;
+  p = ta_dalloc(h, bytes);
+  if (!p) *st = TA_ERR_OOM;
+  else if (cudaMemsetAsync(p, 0, bytes, h->stream) != cudaSuccess) {
+    h->last_cuda = cudaGetLastError();
+    *st = TA_ERR_CUDA;
   }
   return p;
 }
@@ -229,13 +250,45 @@ ta_status ta_queue_d2h(ta_window *h, void *dst, const void *dev_src, size_t byte
   return TA_OK;
 }
 
+static u32 next_seq(ta_window *h) { return ++h->fetch_seq ? h->fetch_seq : ++h->fetch_seq; }
+static volatile u32 *seq_word(unsigned char *pin) { return (volatile u32 *)(pin + TA_PIN_BYTES); }
+Tail ta_tail(ta_window *h, int64_t grid) {
+  Tail t;
+  memset(&t, 0, sizeof(t));
+  if (!h->pin_dev || h->fetch.empty() || h->fetch.size() > TA_TAIL_MAX || grid > 1024) return t;
+  for (const ta_window::Fetch &f : h->fetch)
+    if (f.bytes > 4096 || (f.bytes & 3u)) return t;
+  for (size_t i = 0; i < h->fetch.size(); i++) {
+    t.src[i] = h->fetch[i].src;
+    t.off[i] = h->fetch[i].off;
+    t.bytes[i] = h->fetch[i].bytes;
+  }
+  t.m = (int)h->fetch.size();
+  h->fetch.clear();
+  t.pin_dev = h->pin_dev;
+  t.ticket = (u32 *)&h->d_status[ST_TICKET];
+  t.seq = h->tail_seq = next_seq(h);
+  t.seq_word = seq_word(h->pin_dev);
+  *seq_word(h->pin) = 0;
+  return t;
+}
 static ta_status wait_fetch(ta_window *h) {
+  if (h->fetch.empty() && h->tail_seq) {
+    const u32 seq = h->tail_seq;
+    h->tail_seq = 0;
+    volatile u32 *word = seq_word(h->pin);
+    TA_WAIT_SEQ(*word, seq, h->stream);
+    if (*word != seq) TA_CHECK_CUDA(h, cudaStreamSynchronize(h->stream));
+    std::atomic_thread_fence(std::memory_order_acquire);
+    return *word == seq ? TA_OK : TA_ERR_CUDA;
+  }
+  h->tail_seq = 0;
   if (h->fetch.empty()) {
     TA_CHECK_CUDA(h, cudaStreamSynchronize(h->stream));
     return TA_OK;
   }
-  volatile u32 *word = (volatile u32 *)(h->pin + TA_PIN_BYTES);
-  const u32 seq = ++h->fetch_seq ? h->fetch_seq : ++h->fetch_seq;
+  volatile u32 *word = seq_word(h->pin);
+  const u32 seq = next_seq(h);
   *word = 0;
   TA_TRY(flush_fetch(h, seq));
   TA_WAIT_SEQ(*word, seq, h->stream);
@@ -270,6 +323,7 @@ void ta_dfree_later(ta_window *h, void *p) {
 static ta_status begin_call(ta_window *h) {
   h->pending.clear();
   h->fetch.clear();
+  h->tail_seq = 0;
   h->pin_used = 0;
   if (cudaSetDevice(h->device) != cudaSuccess) {
     h->last_cuda = cudaGetLastError();
@@ -396,14 +450,18 @@ static ta_status load_impl(ta_window *h, const ta_event *events, int32_t on_devi
   const int64_t n = h->n;
   const int W = h->W;
   cudaStream_t st = h->stream;
-  // one device block: [off | t0 | t1 | misc] filled by one copy, [status | load summaries |
-  // digit histograms] zeroed by one fill, [triple table | communicator table] emptied (all
-  // ones) by one fill
+  // one device block: [off | t0 | t1 | misc], filled by the planning kernel (by a copy when there
+  // are many windows), and everything that starts at zero, cleared by one fill: [status | load
+  // summaries | digit histograms | triple table | communicator table | pool for the later calls]
   const size_t up_words = (size_t)(W + 1) + 2 * (size_t)W + 16;
+  // the pool: results and counters of the later calls (34 bytes per record), tile descriptors,
+  // lane tables and a few aggregate tables
+  h->zero_used = 0;
+  h->zero_bytes = n <= TA_ZERO_POOL_RECORDS ? Carver::pad((size_t)n * 36 + (2u << 20)) : 0;
   size_t bytes = Carver::pad(up_words * 8) + Carver::pad(ST_WORDS * 4) +
                  Carver::pad(sizeof(TripleTable)) + Carver::pad(sizeof(CommTable)) +
                  Carver::pad(W * sizeof(ta_load_summary)) + Carver::pad(10 * 256 * 4) +
-                 Carver::pad(TA_TRIPLE_SLOTS * 4) + 256;
+                 Carver::pad(TA_TRIPLE_SLOTS * 4) + h->zero_bytes + 256;
   void *b = ta_dalloc(h, bytes);
   if (!b) return TA_ERR_OOM;
   Carver c(b);
@@ -412,15 +470,17 @@ static ta_status load_impl(ta_window *h, const ta_event *events, int32_t on_devi
   h->d_t0 = up + (W + 1);
   h->d_t1 = h->d_t0 + W;
   h->d_misc = h->d_t1 + W;
-  char *zero_begin = c.base + c.off;
+  h->d_triples = c.take<TripleTable>(1);  // (only its first part, the slots, has to be cleared)
+  char *zero_begin = (char *)h->d_triples->slots;
+  static_assert(offsetof(TripleTable, slots) + sizeof(h->d_triples->slots) == sizeof(TripleTable), "slots come last");
   h->d_status = c.take<int32_t>(ST_WORDS);
   h->d_load_sum = c.take<ta_load_summary>(W);
   h->d_hist = c.take<u32>(10 * 256);
   h->d_slot_cnt = c.take<u32>(TA_TRIPLE_SLOTS);
-  char *zero_end = c.base + c.off;
-  h->d_triples = c.take<TripleTable>(1);
+  h->zero_pool = c.take<char>(h->zero_bytes);
   h->d_comms = c.take<CommTable>(1);
-  char *ones_end = c.base + c.off;
+  char *zero_end = (char *)h->d_comms + sizeof(h->d_comms->slots);
+  static_assert(offsetof(CommTable, slots) == 0, "slots come first");
   h->d_keys = (u64 *)ta_dalloc(h, (size_t)(n > 0 ? n : 1) * 8);
   if (!h->d_keys) return TA_ERR_OOM;
 
@@ -434,35 +494,31 @@ static ta_status load_impl(ta_window *h, const ta_event *events, int32_t on_devi
   } else {
     h->events = events;
   }
-  {
-    std::vector<int64_t> host(up_words, 0);
-    memcpy(host.data(), h->h_off.data(), (size_t)(W + 1) * 8);
-    memcpy(host.data() + (W + 1), h->h_t0.data(), (size_t)W * 8);
-    memcpy(host.data() + (W + 1) + W, h->h_t1.data(), (size_t)W * 8);
-    int64_t *misc_init = host.data() + (W + 1) + 2 * (size_t)W;
-    misc_init[0] = INT64_MAX;  // min name
-    misc_init[1] = INT64_MIN;  // max name
-    misc_init[3] = INT64_MAX;  // min seq
-    misc_init[4] = INT64_MIN;  // max seq
+  if (W > TA_PLAN_WINDOWS) {
+    std::vector<int64_t> host(h->h_off);
+    host.insert(host.end(), h->h_t0.begin(), h->h_t0.end());
+    host.insert(host.end(), h->h_t1.begin(), h->h_t1.end());
     // a pageable source is staged by the runtime before the call returns
-    TA_CHECK_CUDA(h, cudaMemcpyAsync(up, host.data(), up_words * 8, cudaMemcpyHostToDevice, st));
+    TA_CHECK_CUDA(h, cudaMemcpyAsync(up, host.data(), host.size() * 8, cudaMemcpyHostToDevice, st));
   }
   TA_CHECK_CUDA(h, cudaMemsetAsync(zero_begin, 0, zero_end - zero_begin, st));
-  TA_CHECK_CUDA(h, cudaMemsetAsync(zero_end, 0xFF, ones_end - zero_end, st));
   const int32_t spin = g_ta_spin_limit.load();
   if (spin > 0)
     TA_CHECK_CUDA(h, cudaMemcpyAsync(h->d_status + ST_SPIN, &spin, sizeof(spin), cudaMemcpyHostToDevice, st));
 
-  TA_TRY(ta_launch_discover(h));
-
   int32_t words[ST_WORDS];
   int64_t misc[16];
   std::vector<ta_load_summary> sums(W);
-  h->h_comm_sorted.assign(TA_MAX_COMMS, 0);
+  h->h_comm_sorted.assign(TA_COMMS_AT_ONCE, 0);
   TA_TRY(ta_queue_d2h(h, misc, h->d_misc, sizeof(misc)));
-  TA_TRY(ta_queue_d2h(h, sums.data(), h->d_load_sum, W * sizeof(ta_load_summary)));
-  TA_TRY(ta_queue_d2h(h, h->h_comm_sorted.data(), h->d_comms->sorted_id, TA_MAX_COMMS * sizeof(u64)));
-  TA_TRY(ta_read_status(h, words));
+  TA_TRY(ta_queue_d2h(h, h->h_comm_sorted.data(), h->d_comms->sorted_id, TA_COMMS_AT_ONCE * sizeof(u64)));
+  TA_TRY(ta_queue_d2h(h, words, h->d_status, sizeof(words)));
+  // (summaries beyond the staging block are copied directly, once the kernels are queued)
+  const bool small = W * sizeof(ta_load_summary) <= 4096;
+  if (small) TA_TRY(ta_queue_d2h(h, sums.data(), h->d_load_sum, W * sizeof(ta_load_summary)));
+  TA_TRY(ta_launch_discover(h));
+  if (!small) TA_TRY(ta_queue_d2h(h, sums.data(), h->d_load_sum, W * sizeof(ta_load_summary)));
+  TA_TRY(ta_sync_fetch(h));
   if (words[ST_ERR]) return (ta_status)words[ST_ERR];
   h->n_triples = words[ST_N_TRIPLES];
   h->n_pids = words[ST_N_PIDS];
@@ -475,6 +531,10 @@ static ta_status load_impl(ta_window *h, const ta_event *events, int32_t on_devi
   if (h->tkeep < 0) h->tkeep = (int)misc[6];
   h->n_comms = words[ST_N_COMMS];
   h->h_comm_sorted.resize((size_t)h->n_comms);
+  if (h->n_comms > TA_COMMS_AT_ONCE) {  // rarely: the rest of the communicator ids
+    TA_TRY(ta_queue_d2h(h, h->h_comm_sorted.data(), h->d_comms->sorted_id, (size_t)h->n_comms * sizeof(u64)));
+    TA_TRY(ta_sync_fetch(h));
+  }
   h->n_valid = 0;
   for (int w = 0; w < W; w++) {
     ta_load_summary &s = sums[w];
@@ -526,6 +586,7 @@ ta_status ta_load_window(const ta_env *env, const ta_event *events, int64_t n,
   h->d_op_gap_ns = nullptr;
   h->d_on_path = nullptr;
   h->d_status = nullptr;
+  h->zero_bytes = h->zero_used = 0;
   h->pin = pin_take();
   h->pin_bytes = h->pin ? TA_PIN_BYTES : 0;
   h->pin_dev = nullptr;
@@ -536,6 +597,7 @@ ta_status ta_load_window(const ta_env *env, const ta_event *events, int64_t n,
   }
   h->pin_used = 0;
   h->fetch_seq = 0;
+  h->tail_seq = 0;
   h->h_off.assign(win_off, win_off + W + 1);
   h->h_t0.assign(win_t0, win_t0 + W);
   h->h_t1.assign(win_t1, win_t1 + W);

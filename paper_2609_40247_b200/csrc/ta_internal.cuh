@@ -35,18 +35,21 @@ enum { ST_ERR = 0, ST_LONG_RUN = 1, ST_N_TRIPLES = 2, ST_N_PIDS = 3, ST_N_COMMS 
        ST_TICKET = 15, ST_WORDS = 16 };
 
 struct TripleTable {       // device-resident, filled by the discovery kernel
-  u64 slots[TA_TRIPLE_SLOTS];          // biased code or EMPTY
   int32_t rank_of_slot[TA_TRIPLE_SLOTS];
   u64 sorted_code[TA_MAX_TRIPLES];     // ascending
   int32_t pid_rank[TA_MAX_TRIPLES];    // per triple rank
   int32_t pid_value[TA_MAX_TRIPLES];   // per pid rank
+  u32 rank_cnt[TA_MAX_TRIPLES];        // kept records per triple rank (a single window)
+  u64 slots[TA_TRIPLE_SLOTS];          // code + 1, 0 = empty
 };
 
-struct CommTable {         // communicator ids seen on COLL records (biased; all-ones = empty)
-  u64 slots[TA_COMM_SLOTS];
+struct CommTable {         // communicator ids seen on COLL records
+  u64 slots[TA_COMM_SLOTS];            // complement of the biased id, 0 = empty (INT64_MAX is reserved)
   int32_t rank_of_slot[TA_COMM_SLOTS];
   u64 sorted_id[TA_MAX_COMMS];         // ascending (biased)
 };
+#define TA_COMMS_AT_ONCE 32  // communicator ids fetched with the other results of the load
+#define TA_PLAN_WINDOWS 8    // windows whose bounds travel as kernel arguments
 
 struct SortPlan {
   int n_pass;
@@ -74,6 +77,15 @@ static inline SortPlan ta_plan_bits(int lo_bit, int hi_bit) {
   return p;
 }
 
+// What the scan of the digit histograms still has to add to them: the (window, lane) digits of a
+// single window from the records counted per triple, and the dropped records of every pass.
+struct TopHist {
+  SortPlan plan;        // passes [n_time, n_pass) are over the bits above top_lo
+  int n_time, top_lo, tbits, wbits, n_triples;
+  u32 n_dropped;
+  const u32 *rank_cnt;  // records per triple rank; null: the histograms are complete
+};
+
 // --------------------------------------------------------------- handle
 struct ta_window {
   ta_env env;
@@ -91,6 +103,8 @@ struct ta_window {
 
   std::vector<void *> allocs;  // everything obtained from env.alloc (or the library's own pool)
   std::vector<size_t> alloc_bytes;  // their sizes, same order
+  char *zero_pool;   // cleared when the window was loaded, handed out by ta_zalloc
+  size_t zero_bytes, zero_used;
   std::vector<void *> deferred;  // temporaries to release after the next synchronisation
 
   // device -> host results of the call in progress: copies are queued into one page-locked
@@ -106,6 +120,7 @@ struct ta_window {
   struct Fetch { const void *src; unsigned off, bytes; };
   std::vector<Fetch> fetch;
   u32 fetch_seq;  // number of the last fetch somebody waited for
+  u32 tail_seq;   // number of the fetch the last kernel of the call makes itself, 0 = none
 
   // load products
   int32_t *d_status;
@@ -129,6 +144,7 @@ struct ta_window {
   u32 *d_slot_cnt;             // kept records per triple slot (one window only), or null
   int64_t min_name, max_name, max_dur;
   SortPlan plan;
+  TopHist top;
 
   // sort products
   ta_sort_result sorted;
@@ -139,6 +155,7 @@ struct ta_window {
   int32_t *d_lane_dom_next;  // per lane: index of the first later lane of the other domain
   int64_t n_device;          // kept device records
   i64 *d_slot_min, *d_slot_max;               // per slot: corr_id range of its LAUNCH records
+  i64 *d_slot_base;                           // per slot: offset of its range when all ranges are laid end to end, -1 = empty
   std::vector<int64_t> h_slot_min, h_slot_max;  // host copies (INT64_MAX / INT64_MIN when none)
 
   // join / attribution products
@@ -165,6 +182,14 @@ static inline int ta_bit_len(uint64_t v) {
 // -------------------------------------------------------------- memory
 void *ta_dalloc(ta_window *h, size_t bytes);            // NULL on failure
 void ta_dfree(ta_window *h, void *p);                   // early release of one allocation
+// Memory that starts at zero.  Windows of up to TA_ZERO_POOL_RECORDS records clear one pool for all
+// their calls while they are loaded (a clearing is a launch: sixteen of the fifty operations of a
+// small window); what does not fit it, or comes after TA_ZERO_POOL is used up, is allocated and
+// cleared on its own.  A pointer into the pool may be given to ta_dfree like any other (nothing
+// happens: the pool lives as long as the handle).
+#define TA_ZERO_POOL_RECORDS (1ll << 20)
+void *ta_zalloc(ta_window *h, size_t bytes, ta_status *st);
+void *ta_zpool(ta_window *h, size_t bytes);  // from the pool or NULL
 // carve sub-buffers out of one allocation
 struct Carver {
   char *base;
@@ -209,8 +234,8 @@ struct PrekeyInfo {
 };
 ta_status ta_radix_sort_keys(ta_window *h, const u64 *keys_in, u64 *keys_scratch, u64 *keys_final,
                              int64_t n, const SortPlan &plan, const u32 *hist /*nullable*/,
-                             void *temp,
-                             bool first_pass_unstable, const PrekeyInfo *prekey = nullptr);
+                             void *temp, bool first_pass_unstable, const PrekeyInfo *prekey = nullptr,
+                             const TopHist *top = nullptr);
 SortPlan ta_make_plan(int lo_bit, int hi_bit);
 // load.cu
 ta_status ta_launch_discover(ta_window *h);
@@ -251,6 +276,21 @@ ta_status ta_queue_d2h(ta_window *h, void *dst, const void *dev_src, size_t byte
 ta_status ta_sync_fetch(ta_window *h);
 // The same, with the device status words.
 ta_status ta_read_status(ta_window *h, int32_t *host_words /*ST_WORDS*/);
+// The last kernel of a call can write the results the host waits for itself (its last CTA to finish
+// does), instead of a kernel of its own for it: some four microseconds per call.  ta_tail takes the
+// queued regions over if they are few and small and the grid is (one atomic per CTA on one word);
+// otherwise the tail is empty and ta_sync_fetch launches k_collect as ever.
+#define TA_TAIL_MAX 6
+struct Tail {
+  const void *src[TA_TAIL_MAX];
+  unsigned off[TA_TAIL_MAX], bytes[TA_TAIL_MAX];  // multiples of 4 bytes
+  int m;                                         // 0: nothing to do
+  unsigned char *pin_dev;
+  u32 *ticket;
+  u32 seq;
+  volatile u32 *seq_word;
+};
+Tail ta_tail(ta_window *h, int64_t grid);
 // Releases a temporary that queued work may still use: after the next synchronisation.
 void ta_dfree_later(ta_window *h, void *p);
 
@@ -357,6 +397,30 @@ __device__ __forceinline__ u64 td_wait(const u64 *p, int32_t *status, bool *time
     w = ld_relaxed(p);
   }
   return w;
+}
+
+// End of a kernel that carries a tail; all threads of every CTA come here.
+__device__ __forceinline__ void run_tail(const Tail &t) {
+  __shared__ int s_last;
+  if (t.m == 0) return;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    s_last = gridDim.x == 1 || atomicInc(t.ticket, gridDim.x - 1) == gridDim.x - 1;  // (wraps back to 0)
+  }
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  for (int e = 0; e < t.m; e++) {
+    const u32 *s = (const u32 *)t.src[e];
+    u32 *d = (u32 *)(t.pin_dev + t.off[e]);
+    for (unsigned i = threadIdx.x; i < t.bytes[e] / 4; i += blockDim.x) d[i] = __ldcg(s + i);
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence_system();
+    *t.seq_word = t.seq;
+  }
 }
 
 struct OpAdd {

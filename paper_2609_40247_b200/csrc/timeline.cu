@@ -102,11 +102,12 @@ struct GatherArgs {
   // corr_id range of the LAUNCH records per (window, pid) slot, for the join
   const TripleTable *tt;
   int tbits, n_pids;
-  i64 *slot_min, *slot_max;
+  u64 *slot_code;     // [slot] largest biased id, [n_slots + slot] largest complement of one; 0 = none
+  int64_t n_slots;
   i64 *ts_start, *ts_end, *corr;
   int32_t *pid, *name, *seq;
   int16_t *stream, *kind;
-  int32_t *lane_start;  // per lane code, -1 = empty
+  int32_t *lane_start;  // per lane code: first position + 1, 0 = empty
   int32_t *status;
 };
 __device__ __forceinline__ u32 gather_index(u64 k, const GatherArgs &a) {
@@ -183,7 +184,7 @@ __global__ void __launch_bounds__(256, GT_MINB) k_gather(GatherArgs a) {
   a.kind[dst] = r.kind;
   if (p < nv) {
     const u64 code = k >> a.sbits;
-    if (p == 0 || (kprev >> a.sbits) != code) a.lane_start[code] = (int32_t)p;
+    if (p == 0 || (kprev >> a.sbits) != code) a.lane_start[code] = (int32_t)p + 1;
     if (r.kind == TA_KIND_LAUNCH) {
       slot = (int)(code >> a.tbits) * a.n_pids + a.tt->pid_rank[code & ((1ull << a.tbits) - 1)];
       mx = (u64)r.corr ^ (1ull << 63);
@@ -202,8 +203,8 @@ __global__ void __launch_bounds__(256, GT_MINB) k_gather(GatherArgs a) {
       mn_inv = warp_reduce(mn_inv, OpMax());
     } else {  // mixed warp (lane boundary): every thread for itself
       if (slot >= 0) {
-        atomicMax(&a.slot_max[slot], (i64)(mx ^ (1ull << 63)));
-        atomicMin(&a.slot_min[slot], (i64)((~mn_inv) ^ (1ull << 63)));
+        atomicMax(&a.slot_code[slot], mx);
+        atomicMax(&a.slot_code[a.n_slots + slot], mn_inv);
       }
       wslot = -1;
     }
@@ -218,9 +219,8 @@ __global__ void __launch_bounds__(256, GT_MINB) k_gather(GatherArgs a) {
       if (sl == -1) continue;
       if (sl != cur) {
         if (cur >= 0) {
-          const i64 hi = (i64)(cmx ^ (1ull << 63)), lo = (i64)((~cmn) ^ (1ull << 63));
-          if (hi > a.slot_max[cur]) atomicMax(&a.slot_max[cur], hi);
-          if (lo < a.slot_min[cur]) atomicMin(&a.slot_min[cur], lo);
+          if (cmx > a.slot_code[cur]) atomicMax(&a.slot_code[cur], cmx);
+          if (cmn > a.slot_code[a.n_slots + cur]) atomicMax(&a.slot_code[a.n_slots + cur], cmn);
         }
         cur = sl;
         cmx = 0;
@@ -231,9 +231,42 @@ __global__ void __launch_bounds__(256, GT_MINB) k_gather(GatherArgs a) {
   }
 }
 
+// One CTA: the correlation-id range of every slot in plain numbers, and where each range begins
+// when all are laid end to end (the join's direct table; meaningless, and not used, when the ranges
+// add up to more than such a table may hold).
+struct SlotRanges {
+  const u64 *code;
+  int64_t n_slots;
+  i64 *slot_min, *slot_max, *slot_base;
+};
+__device__ __forceinline__ void slot_ranges(const SlotRanges &a, u64 *tmp) {
+  u64 base = 0;
+  for (int64_t s0 = 0; s0 < a.n_slots; s0 += blockDim.x) {
+    const int64_t s = s0 + threadIdx.x;
+    u64 size = 0;
+    if (s < a.n_slots) {
+      const u64 mx = a.code[s], mn_inv = a.code[a.n_slots + s];
+      const bool any = mx != 0 || mn_inv != 0;
+      a.slot_max[s] = any ? (i64)(mx ^ (1ull << 63)) : INT64_MIN;
+      a.slot_min[s] = any ? (i64)((~mn_inv) ^ (1ull << 63)) : INT64_MAX;
+      if (any) size = min(mx - ~mn_inv, (1ull << 38) - 1) + 1;
+    }
+    u64 total;
+    const u64 ex = block_scan_exclusive<OpAdd>(size, OpAdd(), tmp, &total);
+    if (s < a.n_slots) a.slot_base[s] = size ? (i64)(base + ex) : -1;
+    base += total;
+  }
+}
+__global__ void __launch_bounds__(1024) k_slot_ranges(SlotRanges a, const int32_t *status, Tail tail) {
+  TA_PDL();
+  __shared__ u64 tmp[33];
+  if (!ta_failed(status)) slot_ranges(a, tmp);
+  run_tail(tail);
+}
+
 // One CTA: compacts the non-empty lane codes into the lane table (code order is
 // canonical order).  For few codes; k_scan with the functors below does the same for many.
-__global__ void __launch_bounds__(1024) k_lane_table(const int32_t *lane_start, int64_t n_codes,
+__device__ __forceinline__ void lane_table(const int32_t *lane_start, int64_t n_codes,
                                                      int tbits, int n_pids, const TripleTable *tt,
                                                      int64_t n_valid, int32_t *lane_window,
                                                      int32_t *lane_pid, int16_t *lane_stream,
@@ -241,9 +274,7 @@ __global__ void __launch_bounds__(1024) k_lane_table(const int32_t *lane_start, 
                                                      int32_t *lane_code, int32_t *lane_slot,
                                                      int32_t *lane_dom_end, int32_t *lane_dom_next,
                                                      int32_t *lane_dev_base, int32_t *n_lanes_out,
-                                                     int64_t cap, const int32_t *status) {
-  TA_PDL();
-  __shared__ u64 tmp[33];
+                                                     int64_t cap, const int32_t *status, u64 *tmp) {
   __shared__ u64 base;
   if (ta_failed(status)) {  // no lanes: every later call then finds nothing to index
     if (threadIdx.x == 0) { n_lanes_out[0] = 0; n_lanes_out[1] = 0; }
@@ -253,7 +284,7 @@ __global__ void __launch_bounds__(1024) k_lane_table(const int32_t *lane_start, 
   __syncthreads();
   for (int64_t c0 = 0; c0 < n_codes; c0 += blockDim.x) {
     int64_t c = c0 + threadIdx.x;
-    int32_t st = c < n_codes ? lane_start[c] : -1;
+    int32_t st = c < n_codes ? lane_start[c] - 1 : -1;
     u64 total;
     u64 ex = block_scan_exclusive<OpAdd>(st >= 0 ? 1ull : 0ull, OpAdd(), tmp, &total);
     if (st >= 0) {
@@ -324,6 +355,22 @@ __global__ void __launch_bounds__(1024) k_lane_table(const int32_t *lane_start, 
   }
   if (threadIdx.x == 0) n_lanes_out[1] = (int32_t)base;
 }
+__global__ void __launch_bounds__(1024) k_lane_table(const int32_t *lane_start, int64_t n_codes,
+                                                     int tbits, int n_pids, const TripleTable *tt,
+                                                     int64_t n_valid, int32_t *lane_window,
+                                                     int32_t *lane_pid, int16_t *lane_stream,
+                                                     int16_t *lane_domain, int32_t *lane_off,
+                                                     int32_t *lane_code, int32_t *lane_slot,
+                                                     int32_t *lane_dom_end, int32_t *lane_dom_next,
+                                                     int32_t *lane_dev_base, int32_t *n_lanes_out,
+                                                     int64_t cap, const int32_t *status,
+                                                     SlotRanges ranges, Tail tail) {
+  TA_PDL();
+  __shared__ u64 tmp[33];
+  lane_table(lane_start, n_codes, tbits, n_pids, tt, n_valid, lane_window, lane_pid, lane_stream, lane_domain, lane_off, lane_code, lane_slot, lane_dom_end, lane_dom_next, lane_dev_base, n_lanes_out, cap, status, tmp);
+  if (!ta_failed(status)) slot_ranges(ranges, tmp);
+  run_tail(tail);
+}
 
 // The same for many codes (a batch of 512 windows has 65 k of them, and one CTA was bound by the
 // scattered writes it has to make alone: 165 us): three scans over as many CTAs as it takes.
@@ -340,7 +387,7 @@ struct LaneRows {
 };
 struct LaneCodeIn {
   LaneRows t;
-  __device__ u64 operator()(int64_t c) const { return t.lane_start[c] >= 0 ? 1ull : 0ull; }
+  __device__ u64 operator()(int64_t c) const { return t.lane_start[c] > 0 ? 1ull : 0ull; }
 };
 struct LaneCodeOut {
   LaneRows t;
@@ -352,7 +399,7 @@ struct LaneCodeOut {
     t.lane_pid[l] = code_pid(code);
     t.lane_stream[l] = code_stream(code);
     t.lane_domain[l] = code_domain(code);
-    t.lane_off[l] = t.lane_start[c];
+    t.lane_off[l] = t.lane_start[c] - 1;
     t.lane_code[l] = (int32_t)c;
     t.lane_slot[l] = w * t.n_pids + t.tt->pid_rank[r];
   }
@@ -426,7 +473,7 @@ ta_status ta_run_sort_timeline(ta_window *h) {
   // result buffers (kept until ta_free)
   size_t keep = Carver::pad(n * 4) + 3 * Carver::pad(n * 8) + 3 * Carver::pad(n * 4) +
                 2 * Carver::pad(n * 2) + 7 * Carver::pad(lane_cap * 4) + 2 * Carver::pad(lane_cap * 2) +
-                Carver::pad((lane_cap + 1) * 4) + Carver::pad((size_t)n_slots * 16) + 512;
+                Carver::pad((lane_cap + 1) * 4) + Carver::pad((size_t)n_slots * 24) + 512;
   void *kb = ta_dalloc(h, keep);
   if (!kb) return TA_ERR_OOM;
   Carver ck(kb);
@@ -442,18 +489,26 @@ ta_status ta_run_sort_timeline(ta_window *h) {
   int32_t *lane_dev_base = ck.take<int32_t>(lane_cap);
   int32_t *lane_dom_next = ck.take<int32_t>(lane_cap);
   int32_t *n_lanes_dev = ck.take<int32_t>(2);  // [0] lanes, [1] device records
-  h->d_slot_min = ck.take<i64>(2 * n_slots);  // minima, then maxima, contiguous
+  h->d_slot_min = ck.take<i64>(3 * n_slots);
   h->d_slot_max = h->d_slot_min + n_slots;
+  h->d_slot_base = h->d_slot_max + n_slots;
 
   // temporaries (released at the end of the call)
   size_t tmp_bytes = 2 * Carver::pad(n * 8) + Carver::pad(n * 4) + ta_sort_temp_bytes(n) +
-                     Carver::pad(n_codes * 4) + 2 * scan_temp_bytes(lane_cap) + scan_temp_bytes(n_codes) + 512;
+                     2 * scan_temp_bytes(lane_cap) + scan_temp_bytes(n_codes) + 512;
   void *tb = ta_dalloc(h, tmp_bytes);
   if (!tb) return TA_ERR_OOM;
   Carver ct(tb);
   u64 *kscr = ct.take<u64>(n), *skeys = ct.take<u64>(n);
   u32 *vscr = ct.take<u32>(n);
-  int32_t *lane_start = ct.take<int32_t>(n_codes);
+  ta_status zs;
+  // cleared: first positions per lane code, correlation-id ranges per slot
+  const size_t zero_bytes = Carver::pad((size_t)n_codes * 4) + Carver::pad((size_t)n_slots * 16);
+  void *zb = ta_zalloc(h, zero_bytes, &zs);
+  if (!zb) return zs;
+  Carver cz(zb);
+  int32_t *lane_start = cz.take<int32_t>(n_codes);
+  u64 *slot_code = cz.take<u64>(2 * n_slots);
   void *sort_tmp = ct.base + ct.off;
 
   int32_t n_lanes_host[2] = {0, 0};
@@ -462,14 +517,9 @@ ta_status ta_run_sort_timeline(ta_window *h) {
   // second attempt sorts (key, index) pairs at full time resolution.
   for (int attempt = 0; attempt < 2; attempt++) {
     int32_t words[ST_WORDS];
-    h->h_slot_min.assign((size_t)n_slots, INT64_MAX);
-    h->h_slot_max.assign((size_t)n_slots, INT64_MIN);
-    {  // the two ranges sit side by side on the device: one copy
-      std::vector<int64_t> init(h->h_slot_min);
-      init.insert(init.end(), h->h_slot_max.begin(), h->h_slot_max.end());
-      TA_CHECK_CUDA(h, cudaMemcpyAsync(h->d_slot_min, init.data(), 2 * n_slots * 8, cudaMemcpyHostToDevice, st));
-    }
-    TA_CHECK_CUDA(h, cudaMemsetAsync(lane_start, 0xFF, n_codes * sizeof(int32_t), st));
+    h->h_slot_min.resize((size_t)n_slots);
+    h->h_slot_max.resize((size_t)n_slots);
+    if (attempt) TA_CHECK_CUDA(h, cudaMemsetAsync(zb, 0, zero_bytes, st));
     if (n > 0) {
       if (h->packed) {
         // keys carry the index: 8-byte elements, fewer bytes per pass
@@ -477,7 +527,7 @@ ta_status ta_run_sort_timeline(ta_window *h) {
         PrekeyInfo pre{h->d_off, h->W, h->d_triples->rank_of_slot, h->tbits, h->wbits,
                        h->sbits - h->dshift, h->dshift, h->ibits};
         TA_TRY(ta_radix_sort_keys(h, h->d_keys, kscr, skeys, n, h->plan, h->d_hist, sort_tmp, true,
-                                  h->fast_keys ? &pre : nullptr));
+                                  h->fast_keys ? &pre : nullptr, &h->top));
         if (n > h->n_valid)
           ta_launch(k_unpack_tail, nblk(n - h->n_valid, 256), 256, 0, st, skeys, h->n_valid, n, pi, perm, h->d_status);
       }
@@ -548,11 +598,19 @@ ta_status ta_run_sort_timeline(ta_window *h) {
       g.ts_start = c_ts; g.ts_end = c_te; g.corr = c_corr; g.pid = c_pid; g.name = c_name; g.seq = c_seq;
       g.stream = c_stream; g.kind = c_kind; g.lane_start = lane_start;
       g.tt = h->d_triples; g.tbits = h->tbits; g.n_pids = h->n_pids > 0 ? h->n_pids : 1;
-      g.slot_min = h->d_slot_min; g.slot_max = h->d_slot_max; g.status = h->d_status;
+      g.slot_code = slot_code; g.n_slots = n_slots; g.status = h->d_status;
       ta_launch(k_gather, nblk(n, 256), 256, 0, st, g);
     }
+    TA_TRY(ta_queue_d2h(h, n_lanes_host, n_lanes_dev, 2 * sizeof(int32_t)));
+    TA_TRY(ta_queue_d2h(h, words, h->d_status, sizeof(words)));
+    const bool small = n_slots * 8 <= 4096;  // (larger ranges are copied once the kernels are queued)
+    for (int q = 0; small && q < 2; q++)
+      TA_TRY(ta_queue_d2h(h, q ? h->h_slot_max.data() : h->h_slot_min.data(), q ? h->d_slot_max : h->d_slot_min, n_slots * 8));
+    const SlotRanges ranges{slot_code, n_slots, h->d_slot_min, h->d_slot_max, h->d_slot_base};
     if (n_codes <= LT_ONE_CTA || n == 0) {
-      ta_launch(k_lane_table, 1, 1024, 0, st, lane_start, n_codes, h->tbits, h->n_pids > 0 ? h->n_pids : 1, h->d_triples, h->n_valid, lane_window, lane_pid, lane_stream, lane_domain, lane_off, lane_code, lane_slot, lane_dom_end, lane_dom_next, lane_dev_base, n_lanes_dev, lane_cap, h->d_status);
+      ta_launch(k_lane_table, 1, 1024, 0, st, lane_start, n_codes, h->tbits, h->n_pids > 0 ? h->n_pids : 1, h->d_triples,
+                h->n_valid, lane_window, lane_pid, lane_stream, lane_domain, lane_off, lane_code, lane_slot,
+                lane_dom_end, lane_dom_next, lane_dev_base, n_lanes_dev, lane_cap, h->d_status, ranges, ta_tail(h, 1));
     } else {
       LaneRows t{lane_start, h->tbits, h->n_pids > 0 ? h->n_pids : 1, h->d_triples, h->n_valid,
                  lane_window, lane_pid, lane_stream, lane_domain, lane_off, lane_code, lane_slot,
@@ -568,12 +626,12 @@ ta_status ta_run_sort_timeline(ta_window *h) {
       TA_TRY((launch_scan<OpAdd, LaneCodeIn, LaneCodeOut>(h, n_codes, LaneCodeIn{t}, LaneCodeOut{t}, OpAdd(), s1)));
       TA_TRY((launch_scan<OpMax, LaneDomIn, LaneDomOut>(h, t.bound, LaneDomIn{t}, LaneDomOut{t}, OpMax(), s2)));
       TA_TRY((launch_scan<OpAdd, LaneDevIn, LaneDevOut>(h, t.bound, LaneDevIn{t}, LaneDevOut{t}, OpAdd(), s3)));
+      ta_launch(k_slot_ranges, 1, 1024, 0, st, ranges, h->d_status, ta_tail(h, 1));
     }
     TA_CHECK_CUDA(h, cudaGetLastError());
-    TA_TRY(ta_queue_d2h(h, n_lanes_host, n_lanes_dev, 2 * sizeof(int32_t)));
-    TA_TRY(ta_queue_d2h(h, h->h_slot_min.data(), h->d_slot_min, n_slots * 8));
-    TA_TRY(ta_queue_d2h(h, h->h_slot_max.data(), h->d_slot_max, n_slots * 8));
-    TA_TRY(ta_read_status(h, words));
+    for (int q = 0; !small && q < 2; q++)
+      TA_TRY(ta_queue_d2h(h, q ? h->h_slot_max.data() : h->h_slot_min.data(), q ? h->d_slot_max : h->d_slot_min, n_slots * 8));
+    TA_TRY(ta_sync_fetch(h));
     if (words[ST_ERR]) return (ta_status)words[ST_ERR];
     if (!words[ST_LONG_RUN]) break;
     if (!h->packed) return TA_ERR_OVERFLOW;  // cannot happen: the pair path resolves long runs itself
@@ -581,6 +639,7 @@ ta_status ta_run_sort_timeline(ta_window *h) {
     TA_TRY(ta_launch_load(h, false));
   }
   ta_dfree(h, tb);
+  ta_dfree(h, zb);
   ta_dfree(h, h->d_keys);
   h->d_keys = nullptr;
 
