@@ -110,90 +110,102 @@ struct GatherArgs {
   int32_t *lane_start;  // per lane code: first position + 1, 0 = empty
   int32_t *status;
 };
+template <bool ONE>  // one window: its records begin at 0
 __device__ __forceinline__ u32 gather_index(u64 k, const GatherArgs &a) {
+  const u32 i = (u32)(k & ((1ull << a.ibits) - 1));
+  if (ONE) return i;
   const int w = a.wbits ? (int)((k >> a.wshift) & ((1ull << a.wbits) - 1)) : 0;
-  return (u32)(a.off[w] + (int64_t)(k & ((1ull << a.ibits) - 1)));
+  return (u32)a.off[w] + i;
 }
 
-// eight CTAs per SM (32 registers): the kernel lives on occupancy, 42 or 51 registers measured slower
+// eight CTAs per SM (32 registers): the kernel lives on occupancy, 42 or 51 registers measured slower.
+// It is bound by instruction issue as much as by its scattered reads, so the members of a run of
+// equal coarse keys are counted by bit operations on one vote (loops over neighbouring keys, with a
+// fifth of the records in runs, made every warp diverge: 410 instructions per warp), and no warp
+// waits for the others at the end.
 #ifndef GT_MINB
 #define GT_MINB 8
 #endif
+template <bool PACKED, bool ONE>
 __global__ void __launch_bounds__(256, GT_MINB) k_gather(GatherArgs a) {
   TA_PDL();
   __shared__ int s_slot[8];
   __shared__ u64 s_mx[8], s_mn[8];
-  if (ta_failed(a.status)) return;  // the sort gave up: the keys name no records
+  __shared__ u32 s_done;
+  const bool failed = ta_failed(a.status);  // the sort gave up: the keys name no records
+  if (threadIdx.x == 0) s_done = 0;
+  __syncthreads();
+  if (failed) return;
   // positions fit 32 bits (n < 2^31): 32-bit indices keep the address arithmetic of the nine
   // column stores and of the neighbour reads short
   const u32 p = blockIdx.x * blockDim.x + threadIdx.x;
   const u32 n = (u32)a.n, nv = (u32)a.n_valid;
-  int slot = -1;
-  u64 mx = 0, mn_inv = 0;
-  if (p < n) {
-  u32 idx;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const u64 k = p < nv ? a.keys[p] : 0;
+  u64 kprev = __shfl_up_sync(0xffffffffu, k, 1);
+  if (lane == 0 && p > 0 && p < nv) kprev = a.keys[p - 1];
+  u32 idx = 0;
+  if (p < n) idx = PACKED && p < nv ? gather_index<ONE>(k, a) : a.perm[p];
+  Rec r;
+  if (p < n) r = load_rec(a.ev, idx);
   u32 dst = p;  // where the record goes: p, or its place inside a run of equal coarse keys
-  int before = 0, after = 0;
-  // the record's key and the key in front of it: both are needed twice below
-  u64 k = 0, kprev = 0;
-  if (p < nv) {
-    k = a.keys[p];
-    if (p > 0) kprev = a.keys[p - 1];
-  }
-  if (a.packed && p < nv) {
-    idx = gather_index(k, a);
+  if (PACKED) {
     // packed keys order the records down to a coarse time only: members of a run of equal
     // (lane, coarse time) sit in no particular order (the first radix pass is not stable) and
     // are ranked here by (ts_start, -ts_end, input index)
     const u64 hk = k >> a.ibits;
-    if (p > 0 && (kprev >> a.ibits) == hk) {
-      before = 1;
-      while (before <= TA_TIE_RUN_MAX && p - before > 0 && (a.keys[p - before - 1] >> a.ibits) == hk)
-        before++;
-    }
-    while (after <= TA_TIE_RUN_MAX && p + after + 1 < nv && (a.keys[p + after + 1] >> a.ibits) == hk)
-      after++;
-    if (before + after + 1 > TA_TIE_RUN_MAX) {
-      a.status[ST_LONG_RUN] = 1;  // the caller starts over with full-resolution keys
-      before = after = 0;
-    }
-  } else {
-    idx = a.perm[p];
-  }
-  Rec r = load_rec(a.ev, idx);
-  if (before + after > 0) {
-    int rank = 0;
-    for (int q = -before; q <= after; q++) {
-      if (q == 0) continue;
-      const u32 oi = gather_index(a.keys[p + q], a);
-      const i64 *o = reinterpret_cast<const i64 *>(a.ev) + (u64)oi * 5;
-      const i64 os = o[0], oe = o[1];
-      const bool first = os < r.ts_start || (os == r.ts_start && (oe > r.ts_end || (oe == r.ts_end && oi < idx)));
-      rank += first ? 1 : 0;
-    }
-    dst = p - before + rank;
-  }
-  if (a.packed && p < nv) a.perm[dst] = idx;
-  a.ts_start[dst] = r.ts_start;
-  a.ts_end[dst] = r.ts_end;
-  a.corr[dst] = r.corr;
-  a.pid[dst] = r.pid;
-  a.name[dst] = r.name;
-  a.seq[dst] = r.seq;
-  a.stream[dst] = r.stream;
-  a.kind[dst] = r.kind;
-  if (p < nv) {
-    const u64 code = k >> a.sbits;
-    if (p == 0 || (kprev >> a.sbits) != code) a.lane_start[code] = (int32_t)p + 1;
-    if (r.kind == TA_KIND_LAUNCH) {
-      slot = (int)(code >> a.tbits) * a.n_pids + a.tt->pid_rank[code & ((1ull << a.tbits) - 1)];
-      mx = (u64)r.corr ^ (1ull << 63);
-      mn_inv = ~mx;
+    const u32 eq = __ballot_sync(0xffffffffu, p < nv && p > 0 && (kprev >> a.ibits) == hk);
+    if (eq || lane == 31) {
+      // equal keys in front of the record and behind it, as far as the warp reaches; further only
+      // where a run meets the warp's edge
+      int before = __clz((int)~(eq << (31 - lane)));
+      int after = lane < 31 ? __ffs((int)~(eq >> (lane + 1))) - 1 : 0;
+      if (before == lane + 1)
+        while (before <= TA_TIE_RUN_MAX && p > (u32)before && (a.keys[p - before - 1] >> a.ibits) == hk) before++;
+      if (lane + after == 31 && p < nv)
+        while (after <= TA_TIE_RUN_MAX && p + after + 1 < nv && (a.keys[p + after + 1] >> a.ibits) == hk) after++;
+      if (before + after + 1 > TA_TIE_RUN_MAX) {
+        a.status[ST_LONG_RUN] = 1;  // the caller starts over with full-resolution keys
+        before = after = 0;
+      }
+      if (before + after > 0) {
+        int rank = 0;
+        for (int q = -before; q <= after; q++) {
+          if (q == 0) continue;
+          const u32 oi = gather_index<ONE>(a.keys[p + q], a);
+          const i64 *o = reinterpret_cast<const i64 *>(a.ev) + (u64)oi * 5;
+          const i64 os = o[0], oe = o[1];
+          const bool first = os < r.ts_start || (os == r.ts_start && (oe > r.ts_end || (oe == r.ts_end && oi < idx)));
+          rank += first ? 1 : 0;
+        }
+        dst = p - before + rank;
+      }
     }
   }
-  }  // p < n
-  // fold the range per CTA (a CTA almost always sits inside one lane)
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int slot = -1;
+  u64 mx = 0, mn_inv = 0;
+  if (p < n) {
+    if (PACKED && p < nv) a.perm[dst] = idx;
+    a.ts_start[dst] = r.ts_start;
+    a.ts_end[dst] = r.ts_end;
+    a.corr[dst] = r.corr;
+    a.pid[dst] = r.pid;
+    a.name[dst] = r.name;
+    a.seq[dst] = r.seq;
+    a.stream[dst] = r.stream;
+    a.kind[dst] = r.kind;
+    if (p < nv) {
+      const u64 code = k >> a.sbits;
+      if (p == 0 || (kprev >> a.sbits) != code) a.lane_start[code] = (int32_t)p + 1;
+      if (r.kind == TA_KIND_LAUNCH) {
+        slot = (int)(code >> a.tbits) * a.n_pids + a.tt->pid_rank[code & ((1ull << a.tbits) - 1)];
+        mx = (u64)r.corr ^ (1ull << 63);
+        mn_inv = ~mx;
+      }
+    }
+  }
+  // fold the range per CTA (a CTA almost always sits inside one lane); the last warp to get here
+  // adds the CTA's share
   const u32 has = __ballot_sync(0xffffffffu, slot >= 0);
   int wslot = -1;
   if (has) {
@@ -209,24 +221,27 @@ __global__ void __launch_bounds__(256, GT_MINB) k_gather(GatherArgs a) {
       wslot = -1;
     }
   }
-  if (lane == 0) { s_slot[warp] = wslot; s_mx[warp] = mx; s_mn[warp] = mn_inv; }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int cur = -1;
-    u64 cmx = 0, cmn = 0;
-    for (int w = 0; w <= 8; w++) {
-      const int sl = w < 8 ? s_slot[w] : -2;
-      if (sl == -1) continue;
-      if (sl != cur) {
-        if (cur >= 0) {
-          if (cmx > a.slot_code[cur]) atomicMax(&a.slot_code[cur], cmx);
-          if (cmn > a.slot_code[a.n_slots + cur]) atomicMax(&a.slot_code[a.n_slots + cur], cmn);
+  if (lane == 0) {
+    s_slot[warp] = wslot; s_mx[warp] = mx; s_mn[warp] = mn_inv;
+    __threadfence_block();
+    if (atomicAdd(&s_done, 1u) == 7u) {
+      __threadfence_block();
+      int cur = -1;
+      u64 cmx = 0, cmn = 0;
+      for (int w = 0; w <= 8; w++) {
+        const int sl = w < 8 ? ((volatile int *)s_slot)[w] : -2;
+        if (sl == -1) continue;
+        if (sl != cur) {
+          if (cur >= 0) {
+            if (cmx > a.slot_code[cur]) atomicMax(&a.slot_code[cur], cmx);
+            if (cmn > a.slot_code[a.n_slots + cur]) atomicMax(&a.slot_code[a.n_slots + cur], cmn);
+          }
+          cur = sl;
+          cmx = 0;
+          cmn = 0;
         }
-        cur = sl;
-        cmx = 0;
-        cmn = 0;
+        if (w < 8) { cmx = max(cmx, ((volatile u64 *)s_mx)[w]); cmn = max(cmn, ((volatile u64 *)s_mn)[w]); }
       }
-      if (w < 8) { cmx = max(cmx, s_mx[w]); cmn = max(cmn, s_mn[w]); }
     }
   }
 }
@@ -599,7 +614,8 @@ ta_status ta_run_sort_timeline(ta_window *h) {
       g.stream = c_stream; g.kind = c_kind; g.lane_start = lane_start;
       g.tt = h->d_triples; g.tbits = h->tbits; g.n_pids = h->n_pids > 0 ? h->n_pids : 1;
       g.slot_code = slot_code; g.n_slots = n_slots; g.status = h->d_status;
-      ta_launch(k_gather, nblk(n, 256), 256, 0, st, g);
+      auto gather = h->packed ? (h->W == 1 ? k_gather<true, true> : k_gather<true, false>) : k_gather<false, false>;
+      ta_launch(gather, nblk(n, 256), 256, 0, st, g);
     }
     TA_TRY(ta_queue_d2h(h, n_lanes_host, n_lanes_dev, 2 * sizeof(int32_t)));
     TA_TRY(ta_queue_d2h(h, words, h->d_status, sizeof(words)));
