@@ -643,7 +643,7 @@ ta_status ta_lane_gaps_noalloc_host(const int64_t *ts_start, const int64_t *ts_e
  *
  * ta_fetch: copies `count` device regions of the handle's results to host memory
  * (dst[i] <- src[i], bytes[i]) with one synchronisation of env.cuda_stream.
- * Regions of up to 64 KB are gathered by one kernel.
+ * Regions of up to 128 KB are gathered by one kernel.
  * ta_block_of: the allocation a result pointer of this handle lies in.
  * ta_chunk_*: an allocator for ta_env that hands out pieces of one block of device
  * memory the caller has obtained, for callers whose own allocator is expensive

@@ -248,8 +248,8 @@ ta_status ta_run_sol(ta_window *h, const double *flops, const double *bytes, int
     if (!tmp) return TA_ERR_OOM;
     Carver ct(tmp);
     double *df = ct.take<double>(n), *db = ct.take<double>(n);
-    TA_CHECK_CUDA(h, cudaMemcpyAsync(df, flops, (size_t)n * 8, cudaMemcpyHostToDevice, st));
-    TA_CHECK_CUDA(h, cudaMemcpyAsync(db, bytes, (size_t)n * 8, cudaMemcpyHostToDevice, st));
+    TA_TRY(ta_upload(h, df, flops, (size_t)n * 8));
+    TA_TRY(ta_upload(h, db, bytes, (size_t)n * 8));
     flops = df;
     bytes = db;
   }

@@ -1,0 +1,149 @@
+// Host records to the device.  Page-locked memory is copied as it is.  Pageable memory (a file mapped
+// or read by the caller, a numpy array) the driver copies through a staging buffer of its own with one
+// thread, at 11 to 20 GB/s; here several threads copy pieces into a ring of page-locked buffers, each
+// of which is on its way to the device as soon as it is full.  Bound by the host's memory
+// bandwidth or the link (55 GB/s), whichever is less.
+#include <algorithm>
+#include <cstring>
+#include <mutex>
+#include <thread>
+
+#include "ta_internal.cuh"
+
+#define UP_PIECE (1u << 20)
+#define UP_PIECES 24
+#define UP_THREADS 8
+#define UP_MIN (4u << 20)  // below this the threads cost more than they save
+
+namespace {
+struct Ring {
+  unsigned char *buf;
+  cudaEvent_t ev[UP_PIECES];
+  bool used[UP_PIECES];  // an event of an earlier upload is recorded
+  int device;
+  unsigned long long last_used;  // number of the handle that used it last
+};
+std::mutex g_ring_guard;
+std::vector<Ring *> g_rings;  // idle ones; an upload takes one out and puts it back
+unsigned long long g_handles = 0;
+
+void ring_free(Ring *r) {
+  for (int i = 0; i < UP_PIECES; i++)
+    if (r->ev[i]) cudaEventDestroy(r->ev[i]);
+  if (r->buf) cudaFreeHost(r->buf);
+  delete r;
+}
+Ring *ring_take(int device) {
+  {
+    std::lock_guard<std::mutex> lock(g_ring_guard);
+    for (size_t i = 0; i < g_rings.size(); i++)
+      if (g_rings[i]->device == device) {
+        Ring *r = g_rings[i];
+        g_rings.erase(g_rings.begin() + i);
+        return r;
+      }
+  }
+  Ring *r = new (std::nothrow) Ring();
+  if (!r) return nullptr;
+  memset(r, 0, sizeof(*r));
+  r->device = device;
+  void *p = nullptr;
+  if (cudaHostAlloc(&p, (size_t)UP_PIECE * UP_PIECES, cudaHostAllocPortable) != cudaSuccess) {
+    cudaGetLastError();
+    delete r;
+    return nullptr;
+  }
+  r->buf = (unsigned char *)p;
+  for (int i = 0; i < UP_PIECES; i++)
+    if (cudaEventCreateWithFlags(&r->ev[i], cudaEventDisableTiming) != cudaSuccess) {
+      cudaGetLastError();
+      r->ev[i] = nullptr;
+      ring_free(r);
+      return nullptr;
+    }
+  return r;
+}
+}  // namespace
+
+// Rings no upload has asked for during the lifetime of the last two handles are given back.
+void ta_upload_age() {
+  std::vector<Ring *> out;
+  {
+    std::lock_guard<std::mutex> lock(g_ring_guard);
+    g_handles++;
+    for (size_t i = 0; i < g_rings.size();)
+      if (g_rings[i]->last_used + 2 < g_handles) {
+        out.push_back(g_rings[i]);
+        g_rings.erase(g_rings.begin() + i);
+      } else {
+        i++;
+      }
+  }
+  for (Ring *r : out) ring_free(r);
+}
+
+ta_status ta_upload(ta_window *h, void *dst, const void *src, size_t bytes) {
+  cudaPointerAttributes at;
+  memset(&at, 0, sizeof(at));
+  const bool known = cudaPointerGetAttributes(&at, src) == cudaSuccess;
+  if (!known) cudaGetLastError();
+  Ring *r = nullptr;
+  if (bytes >= UP_MIN && known && at.type == cudaMemoryTypeUnregistered) r = ring_take(h->device);
+  if (!r) {
+    TA_CHECK_CUDA(h, cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, h->stream));
+    return TA_OK;
+  }
+  const size_t pieces = (bytes + UP_PIECE - 1) / UP_PIECE;
+  std::atomic<size_t> next{0};
+  std::atomic<int> failed{0};
+  std::atomic<size_t> issued[UP_PIECES];  // 1 + last piece sent from the buffer
+  for (int i = 0; i < UP_PIECES; i++) issued[i].store(0);
+  auto work = [&]() {
+    if (cudaSetDevice(h->device) != cudaSuccess) { failed.store(1); return; }
+    for (;;) {
+      const size_t c = next.fetch_add(1);
+      if (c >= pieces || failed.load()) return;
+      const int b = (int)(c % UP_PIECES);
+      // the buffer's piece before has been sent off (pieces are drawn in order, so some thread is at
+      // it or done with it), and has arrived
+      while (c >= UP_PIECES && issued[b].load(std::memory_order_acquire) != c - UP_PIECES + 1)
+        if (failed.load()) return;
+      if ((c >= UP_PIECES || r->used[b]) && cudaEventSynchronize(r->ev[b]) != cudaSuccess) { failed.store(1); return; }
+      const size_t off = c * (size_t)UP_PIECE, len = std::min((size_t)UP_PIECE, bytes - off);
+      unsigned char *buf = r->buf + (size_t)b * UP_PIECE;
+      memcpy(buf, (const unsigned char *)src + off, len);
+      if (cudaMemcpyAsync((unsigned char *)dst + off, buf, len, cudaMemcpyHostToDevice, h->stream) != cudaSuccess ||
+          cudaEventRecord(r->ev[b], h->stream) != cudaSuccess) {
+        failed.store(1);
+        return;
+      }
+      issued[b].store(c + 1, std::memory_order_release);
+    }
+  };
+  {
+    // half of the host's cores at most, a thread per four pieces at most
+    size_t threads = std::max<size_t>(1, std::min<size_t>(UP_THREADS, std::thread::hardware_concurrency() / 2));
+    threads = std::min(threads, (pieces + 3) / 4);
+    std::vector<std::thread> others;
+    for (size_t t = 1; t < threads; t++) {
+      try {
+        others.emplace_back(work);
+      } catch (...) {  // no more threads: those there are do the work
+        break;
+      }
+    }
+    work();
+    for (std::thread &t : others) t.join();
+  }
+  for (int i = 0; i < UP_PIECES; i++) r->used[i] = r->used[i] || issued[i].load() != 0;
+  {
+    std::lock_guard<std::mutex> lock(g_ring_guard);
+    r->last_used = g_handles;
+    g_rings.push_back(r);
+  }
+  if (failed.load()) {
+    h->last_cuda = cudaGetLastError();
+    return TA_ERR_CUDA;
+  }
+  return TA_OK;
+}

@@ -389,7 +389,7 @@ class _Result:
 
     # Tables are mostly read together: a request for one brings the other small ones of the result
     # along (a round trip costs more than their bytes), up to these limits.
-    _FETCH_EACH, _FETCH_ALL, _FETCH_COUNT = 64 << 10, 256 << 10, 16
+    _FETCH_EACH, _FETCH_ALL, _FETCH_COUNT = 128 << 10, 448 << 10, 16
 
     def _fetch(self, name):
         names, sizes, total = [], [], 0
