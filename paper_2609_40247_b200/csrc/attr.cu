@@ -18,11 +18,15 @@
 //                  fan-out-32 tree, leaves every tile the stack open at its start;
 //   k_attr_resolve per record: a backward look over the thread's own records,
 //                  else one descent of a max-tree over the threads' largest OP
-//                  end times in shared memory, else the carried stack.
+//                  end times in shared memory, else the carried stack.  The kernels of
+//                  every operator are added up on the way, from the launches inside it,
+//                  and all columns of the operator are written once, with the zeros of
+//                  all other rows;
+//   k_attr_spill   what a tile owes to operators of earlier tiles is added to their rows.
 // Partial overlap is detected on the way: that nearest running OP must also
 // cover i's end.
-// HBM-bound: 18 B read per host record + 5 B written per record, plus the
-// per-operator atomics of the device records.
+// HBM-bound by design: 26 B read per host record, 16 B per kernel (nearly sequential), 33 B
+// written per record.
 #include <climits>
 #include <cstring>
 #include <vector>
@@ -65,12 +69,17 @@ struct AttrArgs {
   i64 *agg_e, *carry_e;           // [tile][AT_CAP]
   int32_t *agg_pos, *carry_pos;
   int32_t *status;
-  const int32_t *kol;  // kernels of each launch (from the join)
-  // k_attr_ops
+  const int32_t *kol;        // kernels of each launch (from the join)
+  const int32_t *kernel_of;  // the kernel of each launch that has exactly one
   const int32_t *launch_of;
   int32_t *op_of, *op_n;
-  u64 *op_first, *op_last;
-  int64_t *op_ns;
+  i64 *op_first, *op_last, *op_ns;
+  struct AttrSpill *spill;   // what tiles owe to operators of earlier tiles
+  u32 *n_spill;
+};
+struct AttrSpill {
+  int32_t pos, cnt;
+  i64 first, last, ns;
 };
 
 // A stack of open operators, one entry per lane of a warp (bottom = lane 0).
@@ -330,8 +339,43 @@ struct __align__(16) AttrSmem {
   uint8_t kcarry[AT_TILE];
   i64 carry_e[AT_CAP];
   int32_t carry_pos[AT_CAP];
+  // kernels of the operators: one row per record of the tile, then one per carried operator
+  i64 k_first[AT_TILE + AT_CAP], k_last[AT_TILE + AT_CAP];
+  u64 k_ns[AT_TILE + AT_CAP];
+  int32_t k_cnt[AT_TILE + AT_CAP];  // bit 31: more may be added by other CTAs (the row keeps its identities)
   int lane0, lane1, dmax;
 };
+#define AT_MORE 0x80000000u
+// adds a run of kernels to an operator's row
+__device__ __forceinline__ void attr_add(AttrSmem &s, int row, int cnt, i64 first, i64 last, u64 ns) {
+  atomicAdd(&s.k_cnt[row], cnt);
+  atomicAdd(&s.k_ns[row], ns);
+  if (first < s.k_first[row]) atomicMin(&s.k_first[row], first);
+  if (last > s.k_last[row]) atomicMax(&s.k_last[row], last);
+}
+// the four columns of the thread's records
+template <bool ZERO>
+__device__ __forceinline__ void attr_store_ops(const AttrArgs &a, const AttrSmem &s, int64_t p0, int x0) {
+  int32_t c[AT_ITEMS];
+  i64 f[AT_ITEMS], l[AT_ITEMS], ns[AT_ITEMS];
+#pragma unroll
+  for (int j = 0; j < AT_ITEMS; j++) {
+    c[j] = 0;
+    f[j] = l[j] = ns[j] = 0;
+    if (ZERO) continue;
+    const u32 cnt = (u32)s.k_cnt[x0 + j];
+    c[j] = (int32_t)(cnt & ~AT_MORE);
+    if (cnt) {
+      f[j] = s.k_first[x0 + j];
+      l[j] = s.k_last[x0 + j];
+      ns[j] = (i64)s.k_ns[x0 + j];
+    }
+  }
+  storen_i32<AT_ITEMS>(a.op_n, p0, a.n, c);
+  storen_i64<AT_ITEMS>((int64_t *)a.op_first, p0, a.n, f);
+  storen_i64<AT_ITEMS>((int64_t *)a.op_last, p0, a.n, l);
+  storen_i64<AT_ITEMS>((int64_t *)a.op_ns, p0, a.n, ns);
+}
 
 __global__ void __launch_bounds__(AT_THREADS, AT_RES_MINB) k_attr_resolve(AttrArgs a) {
   TA_PDL();
@@ -368,8 +412,18 @@ __global__ void __launch_bounds__(AT_THREADS, AT_RES_MINB) k_attr_resolve(AttrAr
       for (int j = 0; j < AT_ITEMS; j++)
         if (p0 + j < a.n) { a.parent[p0 + j] = -1; a.depth[p0 + j] = 0; }
     }
+    attr_store_ops<true>(a, s, p0, x0);
     return;
   }
+  for (int i = tid; i < AT_TILE + AT_CAP; i += AT_THREADS) {
+    s.k_first[i] = INT64_MAX;
+    s.k_last[i] = INT64_MIN;
+    s.k_ns[i] = 0;
+    s.k_cnt[i] = 0;
+  }
+  // operators still open at the tile's end: later tiles may add to their rows
+  const int open_cnt = a.agg_meta[tile] & 0xFF;
+  const int open_pos = tid < open_cnt ? (int)(a.agg_pos[(size_t)tile * AT_CAP + tid] - tile_start) : -1;
   // kinds and both times of the thread's records are requested together (the tile holds a host
   // lane, so nearly every record needs its times)
   int16_t kd[AT_ITEMS];
@@ -378,15 +432,21 @@ __global__ void __launch_bounds__(AT_THREADS, AT_RES_MINB) k_attr_resolve(AttrAr
   loadn_i64<AT_ITEMS>(a.ts, p0, a.n, st);
   loadn_i64<AT_ITEMS>(a.te, p0, a.n, en);
   int32_t nk[AT_ITEMS];  // kernels of the thread's launches (0 elsewhere)
+  int32_t kp[AT_ITEMS];  // the kernel of those that have exactly one
   if (full) {
 #pragma unroll
     for (int q = 0; q < AT_ITEMS / 4; q++) {
       const int4 x = *reinterpret_cast<const int4 *>(a.kol + p0 + 4 * q);
+      const int4 y = *reinterpret_cast<const int4 *>(a.kernel_of + p0 + 4 * q);
       nk[4 * q] = x.x; nk[4 * q + 1] = x.y; nk[4 * q + 2] = x.z; nk[4 * q + 3] = x.w;
+      kp[4 * q] = y.x; kp[4 * q + 1] = y.y; kp[4 * q + 2] = y.z; kp[4 * q + 3] = y.w;
     }
   } else {
 #pragma unroll
-    for (int j = 0; j < AT_ITEMS; j++) nk[j] = p0 + j < a.n ? a.kol[p0 + j] : 0;
+    for (int j = 0; j < AT_ITEMS; j++) {
+      nk[j] = p0 + j < a.n ? a.kol[p0 + j] : 0;
+      kp[j] = p0 + j < a.n ? a.kernel_of[p0 + j] : 0;
+    }
   }
   unsigned hostmask = 0;
 #pragma unroll
@@ -423,6 +483,15 @@ __global__ void __launch_bounds__(AT_THREADS, AT_RES_MINB) k_attr_resolve(AttrAr
     }
   }
   s.T[AT_THREADS + tid] = m8;
+  // the times of those kernels: consecutive launches have consecutive kernels of a few streams, so the
+  // gathers of a warp mostly share their sectors
+  i64 ks[AT_ITEMS], ke[AT_ITEMS];
+#pragma unroll
+  for (int j = 0; j < AT_ITEMS; j++) {
+    ks[j] = ke[j] = 0;
+    if (!(hostmask & (1u << j)) || kd[j] != TA_KIND_LAUNCH) nk[j] = 0;
+    if (nk[j] == 1) { ks[j] = a.ts[kp[j]]; ke[j] = a.te[kp[j]]; }
+  }
   __syncwarp();
   // tree levels inside the warp's subtree: 16, 8, 4, 2, 1 nodes
 #pragma unroll
@@ -521,24 +590,40 @@ __global__ void __launch_bounds__(AT_THREADS, AT_RES_MINB) k_attr_resolve(AttrAr
     }
     plv[j] = (int16_t)pl;
   }
-  // Kernels per operator: an operator owns the kernels of the launches directly inside it, and
-  // the join has counted the kernels of every launch, so the counts are added up here, from
-  // the launch side - consecutive launches mostly share their operator, and one add serves a
-  // run of them - instead of one atomic per kernel from the device side.
+  // Kernels per operator: an operator owns the kernels of the launches directly inside it.  They are
+  // added up here, from the launch side, in shared memory - consecutive launches mostly share their
+  // operator, and one addition serves a run of them; three atomics per kernel on the operator's row
+  // in memory, from the device side, and the clearing and decoding passes around them took 1.2 ms
+  // of 66.8 M records.  The kernels of a launch that has several (a graph replay) are left to
+  // k_attr_ops, which meets them one by one.
   {
-    int32_t run_par = -1, run_cnt = 0;
+    int run_row = -1, run_cnt = 0;
+    i64 run_f = 0, run_l = 0;
+    u64 run_ns = 0;
 #pragma unroll
     for (int j = 0; j < AT_ITEMS; j++) {
-      if (!(hostmask & (1u << j)) || kd[j] != TA_KIND_LAUNCH || par_abs[j] < 0 || nk[j] <= 0) continue;
-      if (par_abs[j] != run_par) {
-        if (run_cnt) atomicAdd(&a.op_n[run_par], run_cnt);
-        run_par = par_abs[j];
-        run_cnt = 0;
+      if (nk[j] <= 0 || par_abs[j] < 0) continue;
+      const int row = plv[j] >= 0 ? plv[j] : AT_TILE + kc[j] - 1;
+      if (nk[j] > 1) {
+        if (row < AT_TILE) atomicOr(&s.k_cnt[row], (int)AT_MORE);
+        continue;
       }
-      run_cnt += nk[j];
+      if (row != run_row) {
+        if (run_row >= 0) attr_add(s, run_row, run_cnt, run_f, run_l, run_ns);
+        run_row = row;
+        run_cnt = 0;
+        run_f = INT64_MAX;
+        run_l = INT64_MIN;
+        run_ns = 0;
+      }
+      run_cnt++;
+      run_f = min(run_f, ks[j]);
+      run_l = max(run_l, ke[j]);
+      run_ns += (u64)(ke[j] - ks[j]);
     }
-    if (run_cnt) atomicAdd(&a.op_n[run_par], run_cnt);
+    if (run_row >= 0) attr_add(s, run_row, run_cnt, run_f, run_l, run_ns);
   }
+  if (open_pos >= 0) atomicOr(&s.k_cnt[open_pos], (int)AT_MORE);
 #pragma unroll
   for (int q = 0; q < AT_ITEMS / 2; q++)
     *reinterpret_cast<u32 *>(&s.parent_local[x0 + 2 * q]) =
@@ -593,6 +678,12 @@ __global__ void __launch_bounds__(AT_THREADS, AT_RES_MINB) k_attr_resolve(AttrAr
     for (int j = 0; j < AT_ITEMS; j++)
       if (p0 + j < a.n) { a.parent[p0 + j] = par_abs[j]; a.depth[p0 + j] = dep[j]; }
   }
+  attr_store_ops<false>(a, s, p0, x0);
+  // what the carried operators are owed
+  if (tid < ccnt && s.k_cnt[AT_TILE + tid]) {
+    const int r = AT_TILE + tid;
+    a.spill[atomicAdd(a.n_spill, 1u)] = AttrSpill{s.carry_pos[tid], s.k_cnt[r], s.k_first[r], s.k_last[r], (i64)s.k_ns[r]};
+  }
   // per-window maximum depth (a tile rarely meets more than one window)
   const int lane_last = s.lane1;
   const int w_first = l0 >= 0 ? a.lane_window[l0] : 0;
@@ -614,12 +705,31 @@ __global__ void __launch_bounds__(AT_THREADS, AT_RES_MINB) k_attr_resolve(AttrAr
 #define AT_OPS_ITEMS 4
 #endif
 #define AT_OPS_TILE (AT_THREADS * AT_OPS_ITEMS)
+// adds kernels to an operator's row in memory (whose first / last are identities while it has none)
+__device__ __forceinline__ void attr_row_add(const AttrArgs &a, int32_t r, int cnt, i64 first, i64 last, i64 ns) {
+  atomicAdd(&a.op_n[r], cnt);
+  atomicAdd((u64 *)&a.op_ns[r], (u64)ns);
+  atomicMin(&a.op_first[r], first);
+  atomicMax(&a.op_last[r], last);
+}
+__global__ void __launch_bounds__(256) k_attr_spill(AttrArgs a) {
+  TA_PDL();
+  if (ta_failed(a.status)) return;
+  const u32 m = *a.n_spill;
+  for (u32 i = blockIdx.x * 256 + threadIdx.x; i < m; i += gridDim.x * 256) {
+    const AttrSpill x = a.spill[i];
+    attr_row_add(a, x.pos, x.cnt, x.first, x.last, x.ns);
+  }
+}
+
 // adds a group of device records to the row of their window
 __device__ __forceinline__ void attr_emit(ta_attr_summary *sm, const u64 *t) {
   if (t[0]) atomicAdd((u64 *)&sm->n_attributed, t[0]);
   if (t[1]) atomicAdd((u64 *)&sm->n_no_launch, t[1]);
   if (t[2]) atomicAdd((u64 *)&sm->n_no_op, t[2]);
 }
+// MULTI: some launch has more than one kernel; those kernels are added to their operator here.
+template <bool MULTI>
 __global__ void __launch_bounds__(AT_THREADS, AT_OPS_MINB) k_attr_ops(AttrArgs a) {
   TA_PDL();
   constexpr int IT = AT_OPS_ITEMS;
@@ -649,33 +759,24 @@ __global__ void __launch_bounds__(AT_THREADS, AT_OPS_MINB) k_attr_ops(AttrArgs a
     }
     return;
   }
-  // kinds, launches and times of the thread's records are requested together (launch_of is -1
-  // wherever the record is no matched kernel or copy, so the gather below needs no kind), then
-  // the parents of the launches: two rounds of memory latency instead of three
+  // kinds and launches of the thread's records are requested together (launch_of is -1 wherever
+  // the record is no matched kernel or copy, so the gather below needs no kind), then the parents
+  // of the launches: two rounds of memory latency instead of three
   int16_t kd[IT];
   loadn_i16<IT>(a.kind, p0, a.n, 0, kd);
   int32_t lo[IT], op[IT];
-  i64 st[IT], en[IT];
 #pragma unroll
-  for (int j = 0; j < IT; j++) { lo[j] = -1; op[j] = -1; st[j] = en[j] = 0; }
+  for (int j = 0; j < IT; j++) { lo[j] = -1; op[j] = -1; }
   if (p0 + IT <= a.n) {
 #pragma unroll
     for (int q = 0; q < IT / 4; q++) {
       const int4 x = *reinterpret_cast<const int4 *>(a.launch_of + p0 + 4 * q);
       lo[4 * q] = x.x; lo[4 * q + 1] = x.y; lo[4 * q + 2] = x.z; lo[4 * q + 3] = x.w;
     }
-    const longlong2 *ps = reinterpret_cast<const longlong2 *>(a.ts + p0);
-    const longlong2 *pe = reinterpret_cast<const longlong2 *>(a.te + p0);
-#pragma unroll
-    for (int q = 0; q < IT / 2; q++) {
-      const longlong2 x = ps[q], y = pe[q];
-      st[2 * q] = x.x; st[2 * q + 1] = x.y;
-      en[2 * q] = y.x; en[2 * q + 1] = y.y;
-    }
   } else {
 #pragma unroll
     for (int j = 0; j < IT; j++)
-      if (p0 + j < a.n) { lo[j] = a.launch_of[p0 + j]; st[j] = a.ts[p0 + j]; en[j] = a.te[p0 + j]; }
+      if (p0 + j < a.n) lo[j] = a.launch_of[p0 + j];
   }
 #pragma unroll
   for (int j = 0; j < IT; j++)
@@ -698,12 +799,9 @@ __global__ void __launch_bounds__(AT_THREADS, AT_OPS_MINB) k_attr_ops(AttrArgs a
         do { l++; next_off = a.lane_off[l + 1]; } while (p >= next_off);
         win = a.lane_window[l];
       }
-      if (lo[j] >= 0 && op[j] >= 0) {
-        const int32_t r = op[j];
-        // (the kernel count of the operator is accumulated from the launch side, in k_attr_resolve)
-        atomicAdd((u64 *)&a.op_ns[r], (u64)(en[j] - st[j]));
-        atomicMax(&a.op_first[r], ~((u64)st[j] ^ (1ull << 63)));
-        atomicMax(&a.op_last[r], (u64)en[j] ^ (1ull << 63));
+      if (MULTI && lo[j] >= 0 && op[j] >= 0 && a.kol[lo[j]] > 1) {
+        const i64 s = a.ts[p], e = a.te[p];
+        attr_row_add(a, op[j], 1, s, e, e - s);
       }
       if (wm < 0) wm = win;
       if (win == wm) {
@@ -736,48 +834,17 @@ __global__ void __launch_bounds__(AT_THREADS, AT_OPS_MINB) k_attr_ops(AttrArgs a
                                         [&](int w, const u64 *t) { attr_emit(&a.sum[w], t); });
 }
 
-// first/last were accumulated in an order-preserving unsigned encoding (0 = untouched)
-#ifndef AT_FIN_ITEMS
-#define AT_FIN_ITEMS 4
-#endif
+// operators that were open at the end of their tile and got no kernels from anywhere: no identities
+// are left behind
 __device__ __forceinline__ void attr_finalize(const AttrArgs &a) {
-  constexpr int IT = AT_FIN_ITEMS;
-  const int err = ta_peek_err(a.status);
-  const int64_t p0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * IT;
-  if (p0 >= a.n_valid) return;
-  // A kernel count above zero only ever sits at the position of an operator that owns kernels
-  // (the counts are accumulated on operator rows alone), so the kinds need not be read: the
-  // counts of all the thread's positions in vector loads, then both times of those operators -
-  // two rounds of memory latency, the thread's misses overlapping
-  int32_t cnt[IT];
-  if (p0 + IT <= a.n) {
-#pragma unroll
-    for (int q = 0; q < IT / 4; q++) {
-      const int4 x = *reinterpret_cast<const int4 *>(a.op_n + p0 + 4 * q);
-      cnt[4 * q] = x.x; cnt[4 * q + 1] = x.y; cnt[4 * q + 2] = x.z; cnt[4 * q + 3] = x.w;
-    }
-  } else {
-#pragma unroll
-    for (int j = 0; j < IT; j++) cnt[j] = p0 + j < a.n ? a.op_n[p0 + j] : 0;
-  }
-  if (ta_is_failure(err)) return;
-  unsigned m = 0;
-#pragma unroll
-  for (int j = 0; j < IT; j++)
-    if (p0 + j < a.n_valid && cnt[j] > 0) m |= 1u << j;
-  if (!m) return;
-  u64 f[IT], l[IT];
-#pragma unroll
-  for (int j = 0; j < IT; j++)
-    if (m & (1u << j)) { f[j] = a.op_first[p0 + j]; l[j] = a.op_last[p0 + j]; }
-#pragma unroll
-  for (int j = 0; j < IT; j++)
-    if (m & (1u << j)) {
-      a.op_first[p0 + j] = (~f[j]) ^ (1ull << 63);
-      a.op_last[p0 + j] = l[j] ^ (1ull << 63);
-    }
+  if (ta_failed(a.status)) return;
+  const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
+  const int64_t tile = i / AT_CAP;
+  const int k = (int)(i - tile * AT_CAP);
+  if (tile >= a.n_tiles || k >= (a.agg_meta[tile] & 0xFF)) return;
+  const int32_t r = a.agg_pos[i];
+  if (a.op_n[r] == 0) { a.op_first[r] = 0; a.op_last[r] = 0; }
 }
-
 __global__ void __launch_bounds__(256) k_attr_finalize(AttrArgs a, Tail tail) {
   TA_PDL();
   attr_finalize(a);
@@ -789,23 +856,23 @@ ta_status ta_run_attribute(ta_window *h, ta_attr_summary *out_summary) {
   const int W = h->W;
   cudaStream_t st = h->stream;
   const int64_t tiles = (n + AT_TILE - 1) / AT_TILE;
-  size_t keep = 2 * Carver::pad(nn * 4) + Carver::pad(nn) + 256;
+  size_t keep = 3 * Carver::pad(nn * 4) + Carver::pad(nn) + 3 * Carver::pad(nn * 8) + 256;
   void *kb = ta_dalloc(h, keep);
   if (!kb) return TA_ERR_OOM;
   Carver ck(kb);
   int32_t *parent = ck.take<int32_t>(nn), *op_of = ck.take<int32_t>(nn);
   uint8_t *depth = ck.take<uint8_t>(nn);
+  int32_t *op_n = ck.take<int32_t>(nn);
+  i64 *op_first = ck.take<i64>(nn), *op_last = ck.take<i64>(nn), *op_ns = ck.take<i64>(nn);
   ta_status zs;
-  void *zb = ta_zalloc(h, Carver::pad(nn * 4) + 3 * Carver::pad(nn * 8) + Carver::pad((size_t)W * sizeof(ta_attr_summary)), &zs);
+  void *zb = ta_zalloc(h, Carver::pad((size_t)W * sizeof(ta_attr_summary)) + 256, &zs);
   if (!zb) return zs;
   Carver cz(zb);
-  int32_t *op_n = cz.take<int32_t>(nn);
-  u64 *op_first = cz.take<u64>(nn), *op_last = cz.take<u64>(nn);
-  int64_t *op_ns = cz.take<int64_t>(nn);
   ta_attr_summary *d_sum = cz.take<ta_attr_summary>(W);
+  u32 *n_spill = cz.take<u32>(1);
 
   const int64_t tt = tiles > 0 ? tiles : 1;
-  size_t tb = 2 * Carver::pad(tt * 4) + 2 * Carver::pad(tt * AT_CAP * 8) + 2 * Carver::pad(tt * AT_CAP * 4) + 256;
+  size_t tb = Carver::pad(tt * AT_CAP * sizeof(AttrSpill)) + 2 * Carver::pad(tt * 4) + 2 * Carver::pad(tt * AT_CAP * 8) + 2 * Carver::pad(tt * AT_CAP * 4) + 256;
   // upper levels of the stack scan: node and start stacks per level
   std::vector<int64_t> level_n(1, tt);
   while (level_n.back() > AT_FAN) level_n.push_back((level_n.back() + AT_FAN - 1) / AT_FAN);
@@ -823,13 +890,15 @@ ta_status ta_run_attribute(ta_window *h, ta_attr_summary *out_summary) {
   a.carry_e = ct.take<i64>(tt * AT_CAP);
   a.agg_pos = ct.take<int32_t>(tt * AT_CAP);
   a.carry_pos = ct.take<int32_t>(tt * AT_CAP);
+  a.spill = ct.take<AttrSpill>(tt * AT_CAP);
+  a.n_spill = n_spill;
 
   a.n = n; a.n_valid = h->n_valid; a.n_lanes = h->sorted.n_lanes; a.n_tiles = tiles;
   a.kind = h->sorted.kind; a.ts = h->sorted.ts_start; a.te = h->sorted.ts_end;
   a.lane_off = h->sorted.lane_off; a.lane_window = h->sorted.lane_window;
   a.lane_domain = h->sorted.lane_domain; a.lane_dom_end = h->d_lane_dom_end;
   a.parent = parent; a.depth = depth; a.sum = d_sum; a.status = h->d_status;
-  a.launch_of = h->join.launch_of; a.kol = h->join.kernels_of_launch; a.op_of = op_of; a.op_n = op_n; a.op_first = op_first;
+  a.launch_of = h->join.launch_of; a.kol = h->join.kernels_of_launch; a.kernel_of = h->d_kernel_of; a.op_of = op_of; a.op_n = op_n; a.op_first = op_first;
   a.op_last = op_last; a.op_ns = op_ns;
   int32_t words[ST_WORDS];
   std::vector<ta_attr_summary> hs(W);
@@ -856,9 +925,13 @@ ta_status ta_run_attribute(ta_window *h, ta_attr_summary *out_summary) {
         ta_launch(k_attr_fold_down, (unsigned)((level_n[k] + 3) / 4), 128, 0, st, node[k - 1], level_n[k - 1], start[k], level_n[k], start[k - 1], k == 1 ? 1 : 0, h->d_status);
     }
     ta_launch(k_attr_resolve, (unsigned)tiles, AT_THREADS, 0, st, a);
-    ta_launch(k_attr_ops, (unsigned)((n + AT_OPS_TILE - 1) / AT_OPS_TILE), AT_THREADS, 0, st, a);
-    const int64_t fb = (h->n_valid + 256 * AT_FIN_ITEMS - 1) / (256 * AT_FIN_ITEMS);
-    ta_launch(k_attr_finalize, (unsigned)(fb > 0 ? fb : 1), 256, 0, st, a, ta_tail(h, fb));
+    const int64_t sb = (tiles * 4 + 255) / 256;
+    ta_launch(k_attr_spill, (unsigned)(sb < 148 * 4 ? sb : 148 * 4), 256, 0, st, a);
+    const unsigned ob = (unsigned)((n + AT_OPS_TILE - 1) / AT_OPS_TILE);
+    if (h->multi_launch) ta_launch(k_attr_ops<true>, ob, AT_THREADS, 0, st, a);
+    else ta_launch(k_attr_ops<false>, ob, AT_THREADS, 0, st, a);
+    const int64_t fb = (tiles * AT_CAP + 255) / 256;
+    ta_launch(k_attr_finalize, (unsigned)fb, 256, 0, st, a, ta_tail(h, fb));
     TA_CHECK_CUDA(h, cudaGetLastError());
   }
   if (!small) TA_TRY(ta_queue_d2h(h, hs.data(), d_sum, W * sizeof(ta_attr_summary)));
@@ -878,7 +951,7 @@ ta_status ta_run_attribute(ta_window *h, ta_attr_summary *out_summary) {
   h->attr.op_of = op_of;
   h->attr.op_first_start = (const int64_t *)op_first;
   h->attr.op_last_end = (const int64_t *)op_last;
-  h->attr.op_kernel_ns = op_ns;
+  h->attr.op_kernel_ns = (const int64_t *)op_ns;
   h->attr.op_n_kernels = op_n;
   if (any_bad) return TA_ERR_BAD_NESTING;
   if (any_deep) return TA_ERR_DEPTH;
