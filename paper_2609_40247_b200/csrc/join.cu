@@ -4,16 +4,17 @@
 // (window, pid, corr_id); the smallest sorted position among equal LAUNCH keys
 // wins.
 //
-// Two paths, same results:
+// One table of sorted positions, two ways to address it:
 //   direct   when the correlation ids of each (window, pid) span a compact
-//            range (they count up per process in real traces): a table of
-//            sorted positions indexed by corr_id - min, filled with atomicMin.
-//            Launches and kernels are time-ordered, so the table is touched
-//            nearly sequentially.
-//   general  any 64-bit ids: launches and probes are compacted, stably sorted
-//            by (slot, corr_id) with the pair sorter, and each probe takes the
-//            head of its run if that head is a LAUNCH.
-// HBM-bound: streams kind/corr/ts columns, writes three outputs per record.
+//            range (they count up per process in real traces): the entry of
+//            corr_id - min.  Launches and kernels are time-ordered, so the
+//            table is touched nearly sequentially.
+//   hashed   any 64-bit ids: open addressing, twice as many entries as launches.
+//            An entry holds nothing but a position; whether it is the wanted key
+//            is read off the corr_id column and off the range of positions its
+//            (window, pid) occupies.
+// Equal keys share an entry and an atomic maximum over complements leaves the smallest
+// position.  HBM-bound: streams kind/corr/ts columns, writes three outputs per record.
 #include <climits>
 #include <cstring>
 #include <vector>
@@ -24,7 +25,6 @@
 #define JN_THREADS 512
 #define JN_ITEMS 4
 #define JN_TILE (JN_THREADS * JN_ITEMS)
-// entry of the direct table: complement of the smallest position, 0 = empty
 
 struct JoinArgs {
   int64_t n, n_valid;
@@ -35,10 +35,13 @@ struct JoinArgs {
   const int16_t *lane_domain;
   // per slot (window * n_pids + pid rank)
   i64 *slot_min, *slot_max;       // corr range of LAUNCH records
-  const i64 *slot_base;           // direct path: table offset of the slot, -1 = no launches
-  u32 *table;                     // direct path
-  const int32_t *found;           // general path: winner launch per launch/probe position
+  const i64 *slot_base;           // direct: table offset of the slot, -1 = no launches
+  const int32_t *slot_pos;        // hashed: first position of the slot (n_slots + 1 entries)
+  u32 table_size;                 // hashed: entries
+  u32 *table;                     // complement of the smallest position, 0 = empty
   int32_t *launch_of, *kol;
+  int32_t *kernel_of;             // per launch with exactly one kernel: its position
+  u32 *multi;                     // set when a launch has more than one
   int64_t *latency, *qdelay;
   ta_join_summary *sum;           // device, per window
   const int32_t *status;
@@ -47,7 +50,38 @@ struct JoinArgs {
 __device__ __forceinline__ u64 bias64(i64 v) { return (u64)v ^ (1ull << 63); }
 __host__ __device__ __forceinline__ i64 unbias64(u64 v) { return (i64)(v ^ (1ull << 63)); }
 
-// ---- direct path: fill the table -------------------------------------------
+// ---- hashed addressing -------------------------------------------------------
+__device__ __forceinline__ u32 join_hash(const JoinArgs &a, int slot, i64 c) {
+  u64 x = (u64)c * 0x9E3779B97F4A7C15ull ^ (u64)(u32)slot * 0xC2B2AE3D27D4EB4Full;
+  x ^= x >> 32;
+  x *= 0xD6E8FEB86659FD93ull;
+  return __umulhi((u32)(x >> 32), a.table_size);
+}
+__device__ __forceinline__ bool join_same(const JoinArgs &a, u32 pos, int slot, i64 c) {
+  return a.corr[pos] == c && (i64)pos >= a.slot_pos[slot] && (i64)pos < a.slot_pos[slot + 1];
+}
+// entry of the key or the empty entry that ends its chain, from entry i on; v = what it holds.  Half
+// of the table is empty, so the walk ends (bounded by the table all the same).
+__device__ __forceinline__ u32 join_find(const JoinArgs &a, u32 i, u32 v, int slot, i64 c) {
+  for (u32 step = 0; v != 0 && !join_same(a, ~v, slot, c) && step < a.table_size; step++) {
+    i = i + 1 == a.table_size ? 0 : i + 1;
+    v = a.table[i];
+  }
+  return v;
+}
+// first position of every slot
+__global__ void __launch_bounds__(256) k_join_slot_pos(const int32_t *lane_off, const int32_t *lane_slot, int n_lanes,
+                                                       int n_slots, int32_t *slot_pos, const int32_t *status) {
+  TA_PDL();
+  if (ta_failed(status)) return;
+  const int l = blockIdx.x * blockDim.x + threadIdx.x;
+  if (l > n_lanes) return;
+  const int lo = l == 0 ? 0 : lane_slot[l - 1] + 1, hi = l == n_lanes ? n_slots : lane_slot[l];
+  for (int s = lo; s <= hi; s++) slot_pos[s] = lane_off[l];  // lane_off[n_lanes] = records
+}
+
+// ---- fill the table -------------------------------------------------------------
+template <bool DIRECT>
 __global__ void __launch_bounds__(JN_THREADS) k_join_build(JoinArgs a) {
   TA_PDL();
   __shared__ int s_lane0;
@@ -76,8 +110,21 @@ __global__ void __launch_bounds__(JN_THREADS) k_join_build(JoinArgs a) {
     const int64_t p = p0 + j;
     if (p < a.n_valid && kd[j] == TA_KIND_LAUNCH) {
       while (p >= next_off) { l++; next_off = a.lane_off[l + 1]; slot = a.lane_slot[l]; }
-      const i64 idx = a.slot_base[slot] + (c[j] - a.slot_min[slot]);
-      atomicMax(&a.table[idx], ~(u32)p);
+      if (DIRECT) {
+        const i64 idx = a.slot_base[slot] + (c[j] - a.slot_min[slot]);
+        atomicMax(&a.table[idx], ~(u32)p);
+      } else {
+        u32 i = join_hash(a, slot, c[j]);
+        for (u32 step = 0; step < a.table_size; step++) {
+          const u32 old = atomicCAS(&a.table[i], 0u, ~(u32)p);
+          if (old == 0) break;
+          if (join_same(a, ~old, slot, c[j])) {
+            atomicMax(&a.table[i], ~(u32)p);
+            break;
+          }
+          i = i + 1 == a.table_size ? 0 : i + 1;
+        }
+      }
     }
   }
 }
@@ -150,6 +197,8 @@ __global__ void __launch_bounds__(JP_THREADS, JP_MINB) k_join_probe(JoinArgs a) 
   int32_t lo[IT];
   int wn[IT];  // window of the probe
   {
+    u32 at[DIRECT ? 1 : IT];
+    int sl[DIRECT ? 1 : IT];
     int l = l0;
     int64_t next_off = l >= 0 ? (int64_t)a.lane_off[l + 1] : LLONG_MAX;
     int slot = l >= 0 ? a.lane_slot[l] : 0;
@@ -173,8 +222,25 @@ __global__ void __launch_bounds__(JP_THREADS, JP_MINB) k_join_probe(JoinArgs a) 
             lo[j] = v == 0 ? -1 : (int32_t)~v;
           }
         } else {
-          lo[j] = a.found[p];
+          sl[DIRECT ? 0 : j] = slot;
+          at[DIRECT ? 0 : j] = join_hash(a, slot, c[j]);
         }
+      }
+    }
+    if (!DIRECT) {  // the first entries of all the thread's keys together, then the ids they name, then the chains
+      u32 v[IT];
+#pragma unroll
+      for (int j = 0; j < IT; j++) v[j] = pm & (1u << j) ? a.table[at[DIRECT ? 0 : j]] : 0u;
+      i64 cq[IT];
+#pragma unroll
+      for (int j = 0; j < IT; j++) cq[j] = v[j] ? a.corr[~v[j]] : 0;
+#pragma unroll
+      for (int j = 0; j < IT; j++) {
+        if (v[j] == 0) continue;
+        const int32_t q = (int32_t)~v[j];
+        if (cq[j] != c[j] || q < a.slot_pos[sl[DIRECT ? 0 : j]] || q >= a.slot_pos[sl[DIRECT ? 0 : j] + 1])
+          v[j] = join_find(a, at[DIRECT ? 0 : j], v[j], sl[DIRECT ? 0 : j], c[j]);
+        lo[j] = v[j] == 0 ? -1 : (int32_t)~v[j];
       }
     }
     const int64_t plast = min(tile_start + JP_TILE, a.n_valid) - 1;
@@ -204,6 +270,7 @@ __global__ void __launch_bounds__(JP_THREADS, JP_MINB) k_join_probe(JoinArgs a) 
       const i64 d = s[j] - le[j];
       q[j] = d > 0 ? d : 0;
       atomicAdd(&a.kol[lo[j]], 1);
+      a.kernel_of[lo[j]] = (int32_t)(p0 + j);
     }
     if (wm < 0) wm = wn[j];
     if (wn[j] == wm) {
@@ -291,22 +358,24 @@ __device__ __forceinline__ void join_launch_stats(const JoinArgs &a) {
       const int64_t p = p0 + j;
       while (p >= next_off) { l++; next_off = a.lane_off[l + 1]; }
       wn[j] = a.lane_window[l];
+      const int slot = a.lane_slot[l];
+      u32 v = 0;
       if (DIRECT) {
-        const int slot = a.lane_slot[l];
         const i64 base = a.slot_base[slot];
-        if (base >= 0 && cr[j] >= a.slot_min[slot] && cr[j] <= a.slot_max[slot]) {
-          const u32 v = a.table[base + (cr[j] - a.slot_min[slot])];
-          win[j] = v == 0 ? -1 : (int32_t)~v;
-        }
+        if (base >= 0 && cr[j] >= a.slot_min[slot] && cr[j] <= a.slot_max[slot])
+          v = a.table[base + (cr[j] - a.slot_min[slot])];
       } else {
-        win[j] = a.found[p];
+        const u32 i = join_hash(a, slot, cr[j]);
+        v = join_find(a, i, a.table[i], slot, cr[j]);
       }
+      win[j] = v == 0 ? -1 : (int32_t)~v;
     }
 #pragma unroll
     for (int j = 0; j < 8; j++) {
       if (!(lmask & (1u << j))) continue;
       const bool dup = win[j] != (int32_t)(p0 + j);
       const bool orphan = !dup && nk[j] == 0;
+      if (nk[j] > 1) *a.multi = 1u;
       if (wm < 0) wm = wn[j];
       if (wn[j] == wm) {
         acc[0]++;
@@ -335,60 +404,18 @@ __global__ void __launch_bounds__(JP_THREADS) k_join_launch_stats(JoinArgs a, Ta
   run_tail(tail);
 }
 
-// ---- general path helpers -----------------------------------------------------
-__global__ void __launch_bounds__(256) k_join_key_corr(const u32 *pos, int64_t m, const int64_t *corr,
-                                                       u64 *out, const int32_t *status) {
-  TA_PDL();
-  if (ta_failed(status)) return;
-  int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (j < m) out[j] = bias64(corr[pos[j]]);
-}
-__global__ void __launch_bounds__(256) k_join_key_slot(const u32 *pos, int64_t m,
-                                                       const int32_t *lane_off, int n_lanes,
-                                                       const int32_t *lane_slot, u64 *out,
-                                                       const int32_t *status) {
-  TA_PDL();
-  if (ta_failed(status)) return;
-  int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (j < m) out[j] = (u64)lane_slot[lane_of_pos(lane_off, n_lanes, pos[j])];
-}
-struct JoinHeadIn {
-  const u64 *slot_key;
-  const u32 *pos;
-  const int64_t *corr;
-  __device__ u64 operator()(int64_t j) const {
-    bool head = j == 0 || slot_key[j] != slot_key[j - 1] || corr[pos[j]] != corr[pos[j - 1]];
-    return head ? (u64)(j + 1) : 0ull;
-  }
-};
-struct JoinHeadOut {
-  const u32 *pos;
-  const int16_t *kind;
-  int32_t *found;
-  __device__ void operator()(int64_t j, u64 excl, u64 v) const {
-    u64 hd = (excl > v ? excl : v) - 1;  // index of the head of j's run
-    u32 hp = pos[hd];
-    found[pos[j]] = kind[hp] == TA_KIND_LAUNCH ? (int32_t)hp : -1;
-  }
-};
-
-static int bit_length64(uint64_t v) {
-  int b = 0;
-  while (v) { b++; v >>= 1; }
-  return b;
-}
-
 ta_status ta_run_correlate(ta_window *h, ta_join_summary *out_summary) {
   const int64_t n = h->n;
   const int W = h->W;
   const int n_slots = W * (h->n_pids > 0 ? h->n_pids : 1);
   cudaStream_t st = h->stream;
   const int64_t nn = n > 0 ? n : 1;
-  size_t keep = Carver::pad(nn * 4) + 2 * Carver::pad(nn * 8) + 256;
+  size_t keep = 2 * Carver::pad(nn * 4) + 2 * Carver::pad(nn * 8) + 256;
   void *kb = ta_dalloc(h, keep);
   if (!kb) return TA_ERR_OOM;
   Carver ck(kb);
   int32_t *launch_of = ck.take<int32_t>(nn);
+  h->d_kernel_of = ck.take<int32_t>(nn);
   int64_t *latency = ck.take<int64_t>(nn), *qdelay = ck.take<int64_t>(nn);
   ta_status zs;
   void *zb = ta_zalloc(h, Carver::pad(nn * 4) + Carver::pad((size_t)W * sizeof(ta_join_summary)), &zs);
@@ -406,7 +433,7 @@ ta_status ta_run_correlate(ta_window *h, ta_join_summary *out_summary) {
   a.lane_off = h->sorted.lane_off; a.lane_slot = h->d_lane_slot; a.lane_window = h->sorted.lane_window;
   a.lane_domain = h->sorted.lane_domain; a.lane_dom_end = h->d_lane_dom_end;
   a.slot_min = h->d_slot_min; a.slot_max = h->d_slot_max; a.slot_base = h->d_slot_base;  // filled by the sort
-  a.launch_of = launch_of; a.kol = kol; a.latency = latency; a.qdelay = qdelay; a.sum = d_sum;
+  a.launch_of = launch_of; a.kol = kol; a.kernel_of = h->d_kernel_of; a.multi = (u32 *)&h->d_status[ST_MULTI]; a.latency = latency; a.qdelay = qdelay; a.sum = d_sum;
   a.status = h->d_status;
   const unsigned grid = (unsigned)((n + JN_TILE - 1) / JN_TILE);
   const unsigned grid8 = (unsigned)((n + JS_TILE - 1) / JS_TILE);
@@ -424,57 +451,26 @@ ta_status ta_run_correlate(ta_window *h, ta_join_summary *out_summary) {
       if (hmin[s] <= hmax[s]) total += (unsigned __int128)((uint64_t)hmax[s] - (uint64_t)hmin[s]) + 1;
     const uint64_t limit = (uint64_t)4 * (uint64_t)n + 65536;
     direct = total <= limit;
+    // entries of the table: the span of all ids, or twice the launches
+    const uint64_t M = direct ? (uint64_t)total : 2 * (uint64_t)h->n_launch + 1;
+    if (!direct) {
+      const size_t sb = Carver::pad((size_t)(n_slots + 1) * 4);
+      void *sp = ta_dalloc(h, sb);
+      if (!sp) return TA_ERR_OOM;
+      a.slot_pos = (int32_t *)sp;
+      a.table_size = (u32)M;
+      ta_launch(k_join_slot_pos, (unsigned)((a.n_lanes + 256) / 256), 256, 0, st, a.lane_off, a.lane_slot, a.n_lanes,
+                n_slots, (int32_t *)sp, h->d_status);
+    }
+    tmp_alloc = ta_zalloc(h, (size_t)(M > 0 ? M : 1) * 4, &zs);
+    if (!tmp_alloc) return zs;
+    a.table = (u32 *)tmp_alloc;
     if (direct) {
-      uint64_t M = (uint64_t)total;
-      tmp_alloc = ta_zalloc(h, (size_t)(M > 0 ? M : 1) * 4, &zs);
-      if (!tmp_alloc) return zs;
-      a.table = (u32 *)tmp_alloc;
-      ta_launch(k_join_build, grid, JN_THREADS, 0, st, a);
+      ta_launch(k_join_build<true>, grid, JN_THREADS, 0, st, a);
       ta_launch(k_join_probe<true>, grid_probe, JP_THREADS, 0, st, a);
       ta_launch(k_join_launch_stats<true>, grid8, JP_THREADS, 0, st, a, ta_tail(h, grid8));
     } else {
-      // general path: compact, sort by (slot, corr) with sorted position as the stable tie-break
-      size_t tb = Carver::pad(nn * 4) * 3 + Carver::pad(nn * 8) * 3 + scan_temp_bytes(n) * 2 +
-                  ta_sort_temp_bytes(n) + 512;
-      tmp_alloc = ta_dalloc(h, tb);
-      if (!tmp_alloc) return TA_ERR_OOM;
-      Carver ct(tmp_alloc);
-      u32 *pos = ct.take<u32>(nn), *pos_s = ct.take<u32>(nn);
-      int32_t *found = ct.take<int32_t>(nn);
-      u64 *k_in = ct.take<u64>(nn), *k_s = ct.take<u64>(nn), *k_f = ct.take<u64>(nn);
-      void *scan_mem1 = ct.base + ct.off; ct.off += scan_temp_bytes(n);
-      void *scan_mem2 = ct.base + ct.off; ct.off += scan_temp_bytes(n);
-      void *sort_tmp = ct.base + ct.off;
-      ScanTemp t1;
-      TA_TRY(scan_temp_init(h, scan_mem1, n, &t1));
-      TA_TRY(launch_compact_kind(h, a.kind, h->n_valid,
-                                 (1u << TA_KIND_LAUNCH) | (1u << TA_KIND_KERNEL) | (1u << TA_KIND_MEMCPY),
-                                 pos, t1));
-      u64 m64 = 0;
-      TA_TRY(ta_queue_d2h(h, &m64, t1.total, 8));
-      TA_TRY(ta_sync_fetch(h));
-      TA_TRY(ta_queue_d2h(h, words, h->d_status, sizeof(words)));
-      if (small) TA_TRY(ta_queue_d2h(h, hs.data(), d_sum, W * sizeof(ta_join_summary)));
-      const int64_t m = (int64_t)m64;
-      TA_CHECK_CUDA(h, cudaMemsetAsync(found, 0xFF, nn * 4, st));
-      if (m > 0) {
-        const int gb = (int)((m + 255) / 256);
-        u32 *vscr = (u32 *)found;  // found is not needed before the sorts are done
-        ta_launch(k_join_key_corr, gb, 256, 0, st, pos, m, a.corr, k_in, h->d_status);
-        TA_TRY(ta_radix_sort_pairs(h, k_in, pos, k_s, vscr, k_f, pos_s, m, ta_make_plan(0, 64), nullptr,
-                                   sort_tmp));
-        ta_launch(k_join_key_slot, gb, 256, 0, st, pos_s, m, a.lane_off, a.n_lanes, a.lane_slot, k_in, h->d_status);
-        int sb = bit_length64((uint64_t)(n_slots > 1 ? n_slots - 1 : 1));
-        TA_TRY(ta_radix_sort_pairs(h, k_in, pos_s, k_s, vscr, k_f, pos, m, ta_make_plan(0, sb), nullptr,
-                                   sort_tmp));
-        TA_CHECK_CUDA(h, cudaMemsetAsync(found, 0xFF, nn * 4, st));
-        ScanTemp t2;
-        TA_TRY(scan_temp_init(h, scan_mem2, m, &t2));
-        JoinHeadIn hin{k_f, pos, a.corr};
-        JoinHeadOut hout{pos, a.kind, found};
-        TA_TRY((launch_scan<OpMax, JoinHeadIn, JoinHeadOut>(h, m, hin, hout, OpMax(), t2)));
-      }
-      a.found = found;
+      ta_launch(k_join_build<false>, grid, JN_THREADS, 0, st, a);
       ta_launch(k_join_probe<false>, grid_probe, JP_THREADS, 0, st, a);
       ta_launch(k_join_launch_stats<false>, grid8, JP_THREADS, 0, st, a, ta_tail(h, grid8));
     }
@@ -483,6 +479,7 @@ ta_status ta_run_correlate(ta_window *h, ta_join_summary *out_summary) {
   if (!small) TA_TRY(ta_queue_d2h(h, hs.data(), d_sum, W * sizeof(ta_join_summary)));
   TA_TRY(ta_sync_fetch(h));
   if (tmp_alloc) ta_dfree(h, tmp_alloc);
+  if (a.slot_pos) ta_dfree(h, (void *)a.slot_pos);
   if (words[ST_ERR]) return (ta_status)words[ST_ERR];
   for (int w = 0; w < W; w++) {
     ta_join_summary &s = hs[w];
@@ -491,6 +488,7 @@ ta_status ta_run_correlate(ta_window *h, ta_join_summary *out_summary) {
     s.min_latency = s.n_matched ? unbias64(~(u64)s.min_latency) : 0;
     if (out_summary) out_summary[w] = s;
   }
+  h->multi_launch = words[ST_MULTI];
   h->join.launch_of = launch_of;
   h->join.launch_latency = latency;
   h->join.queue_delay = qdelay;

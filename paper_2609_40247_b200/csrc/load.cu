@@ -55,6 +55,7 @@ __global__ void __launch_bounds__(256) k_discover(const ta_event *ev, int64_t n,
   __syncthreads();
   i64 mn = INT64_MAX, mx = INT64_MIN, md = 0, qmn = INT64_MAX, qmx = INT64_MIN;
   u64 n_coll = 0;  // kept COLL records: sizes the collective matching without a count round trip
+  u64 n_launch = 0;  // kept LAUNCH records: sizes the join's hash table
   WindowWalker ww(off, W);
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
@@ -71,6 +72,7 @@ __global__ void __launch_bounds__(256) k_discover(const ta_event *ev, int64_t n,
     mn = min(mn, (i64)r.name);
     mx = max(mx, (i64)r.name);
     md = max(md, r.ts_end - r.ts_start);
+    n_launch += r.kind == TA_KIND_LAUNCH;
     if (r.kind == TA_KIND_COLL) {  // communicator set and sequence range
       n_coll++;
       qmn = min(qmn, (i64)r.seq);
@@ -123,6 +125,8 @@ __global__ void __launch_bounds__(256) k_discover(const ta_event *ev, int64_t n,
   qmn = warp_min_i64(qmn);
   qmx = warp_max_i64(qmx);
   n_coll = warp_reduce(n_coll, OpAdd());
+  n_launch = warp_reduce(n_launch, OpAdd());
+  if ((threadIdx.x & 31) == 0 && n_launch) atomicAdd((u64 *)&misc[8], n_launch);
   if ((threadIdx.x & 31) == 0 && qmn != INT64_MAX) {
     atomicMin((i64 *)&misc[3], qmn);
     atomicMax((i64 *)&misc[4], qmx);
@@ -312,7 +316,7 @@ __global__ void __launch_bounds__(DS_THREADS) k_discover_staged(DiscoverArgs a) 
   // name and sequence ranges in 32 bits (the fields are int32), folded to 64 at the end
   int32_t mn = INT32_MAX, mx = INT32_MIN, qmn = INT32_MAX, qmx = INT32_MIN;
   i64 md = 0;
-  u32 n_coll = 0;
+  u32 n_coll = 0, n_launch = 0;
   WindowWalker ww(a.off, a.W);
   int cw = -1;  // window whose bounds are in registers
   i64 ct0 = 0, ct1 = 0;
@@ -379,6 +383,7 @@ __global__ void __launch_bounds__(DS_THREADS) k_discover_staged(DiscoverArgs a) 
           mn = min(mn, r.name);
           mx = max(mx, r.name);
           md = max(md, r.ts_end - r.ts_start);
+          n_launch += r.kind == TA_KIND_LAUNCH;
           if (r.kind == TA_KIND_COLL) {  // communicator set and sequence range
             n_coll++;
             qmn = min(qmn, r.seq);
@@ -470,6 +475,8 @@ __global__ void __launch_bounds__(DS_THREADS) k_discover_staged(DiscoverArgs a) 
   qmn = __reduce_min_sync(0xffffffffu, qmn);
   qmx = __reduce_max_sync(0xffffffffu, qmx);
   n_coll = __reduce_add_sync(0xffffffffu, n_coll);
+  n_launch = __reduce_add_sync(0xffffffffu, n_launch);
+  if (lane == 0 && n_launch) atomicAdd((u64 *)&a.misc[8], (u64)n_launch);
   md = warp_max_i64(md);
   if (lane == 0 && n_coll) {
     atomicMin((i64 *)&a.misc[3], (i64)qmn);

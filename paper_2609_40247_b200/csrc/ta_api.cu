@@ -185,7 +185,7 @@ static void pin_put(unsigned char *p) {
 // to finish writes the number of the fetch behind the data, which the host waits for (seq 0: the
 // fetch is not the last of its call and nobody waits).
 #define TA_FETCH_MAX 16
-#define TA_FETCH_BYTES (64u << 10)
+#define TA_FETCH_BYTES (128u << 10)
 #define TA_FETCH_STRIPE (8u << 10)  // bytes per CTA
 struct FetchList {
   const void *src[TA_FETCH_MAX];
@@ -488,8 +488,7 @@ static ta_status load_impl(ta_window *h, const ta_event *events, int32_t on_devi
     h->events_copy = ta_dalloc(h, (size_t)(n > 0 ? n : 1) * sizeof(ta_event));
     if (!h->events_copy) return TA_ERR_OOM;
     if (n > 0)
-      TA_CHECK_CUDA(h, cudaMemcpyAsync(h->events_copy, events, (size_t)n * sizeof(ta_event),
-                                       cudaMemcpyHostToDevice, st));
+      TA_TRY(ta_upload(h, h->events_copy, events, (size_t)n * sizeof(ta_event)));
     h->events = (const ta_event *)h->events_copy;
   } else {
     h->events = events;
@@ -528,6 +527,7 @@ static ta_status load_impl(ta_window *h, const ta_event *events, int32_t on_devi
   h->min_seq = misc[3];
   h->max_seq = misc[4];
   h->n_coll = misc[5];
+  h->n_launch = misc[8];
   if (h->tkeep < 0) h->tkeep = (int)misc[6];
   h->n_comms = words[ST_N_COMMS];
   h->h_comm_sorted.resize((size_t)h->n_comms);
@@ -798,6 +798,7 @@ void ta_free(ta_window *h) {
   const bool own = !h->env.alloc;
   delete h;
   if (own) cache_age();
+  ta_upload_age();
 }
 
 }  // extern "C"

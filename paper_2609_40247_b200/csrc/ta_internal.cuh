@@ -30,9 +30,10 @@ typedef unsigned int u32;
 
 // device status word indices (h->d_status)
 // ST_SPIN: polls a device-side wait may make before it gives up (0 = TA_SPIN_LIMIT)
+// ST_MULTI: some launch has more than one kernel
 // ST_TICKET: counts the CTAs of k_collect that are done (wraps back to 0 by itself)
 enum { ST_ERR = 0, ST_LONG_RUN = 1, ST_N_TRIPLES = 2, ST_N_PIDS = 3, ST_N_COMMS = 4, ST_SPIN = 5,
-       ST_TICKET = 15, ST_WORDS = 16 };
+       ST_MULTI = 6, ST_TICKET = 15, ST_WORDS = 16 };
 
 struct TripleTable {       // device-resident, filled by the discovery kernel
   int32_t rank_of_slot[TA_TRIPLE_SLOTS];
@@ -126,11 +127,11 @@ struct ta_window {
   int32_t *d_status;
   TripleTable *d_triples;
   int64_t *d_misc;           // [0]=min name,[1]=max name,[2]=max duration,[3]=min seq,[4]=max seq,
-                             // [5]=kept COLL records
+                             // [5]=kept COLL records,[8]=kept LAUNCH records
   CommTable *d_comms;
   int n_comms;
   std::vector<u64> h_comm_sorted;  // host copy of the ranked communicator ids (biased)
-  int64_t min_seq, max_seq, n_coll;
+  int64_t min_seq, max_seq, n_coll, n_launch;
   ta_load_summary *d_load_sum;
   u64 *d_keys;
   int prekeys;               // d_keys holds the words of the discovery pass, not keys yet
@@ -160,6 +161,8 @@ struct ta_window {
 
   // join / attribution products
   ta_join_result join;
+  int32_t *d_kernel_of;      // per launch with exactly one kernel or copy: its sorted position
+  int multi_launch;          // some launch has more than one
   ta_attr_result attr;
   const int64_t *d_op_gap_ns;  // per sorted position, set by the gap blame (null before)
   const uint8_t *d_on_path;    // per sorted position, set by the critical path (null before)
@@ -237,6 +240,9 @@ ta_status ta_radix_sort_keys(ta_window *h, const u64 *keys_in, u64 *keys_scratch
                              void *temp, bool first_pass_unstable, const PrekeyInfo *prekey = nullptr,
                              const TopHist *top = nullptr);
 SortPlan ta_make_plan(int lo_bit, int hi_bit);
+// upload.cu
+ta_status ta_upload(ta_window *h, void *dst, const void *host_src, size_t bytes);  // host -> device on the handle's stream
+void ta_upload_age();  // a handle has gone away
 // load.cu
 ta_status ta_launch_discover(ta_window *h);
 ta_status ta_launch_rank_triples(ta_window *h);

@@ -33,3 +33,57 @@ def test_aggregate_row_paths(scale, distinct, spread):
     ev["name_id"] = ids[pick].astype(np.int32)
     o, g = both(ev, wl.win_off, wl.win_t0, wl.win_t1, comm_sizes=wl.comm_sizes, agg_masks=(DEVICE_MASK, 1 << 2, 63))
     assert len(o["agg2_g_count"]) >= min(distinct, len(ev)) // 2
+
+
+@pytest.mark.parametrize("scale,dup,multi", [(0.004, 0.0, 0.0), (0.02, 0.2, 0.0), (0.02, 0.0, 0.3), (0.1, 0.05, 0.05)])
+@pytest.mark.parametrize("hashed", [False, True])
+def test_join_with_any_ids_and_several_kernels_per_launch(scale, dup, multi, hashed):
+    """Both ways to address the join's table, with launch ids used twice and with launches that own
+    several kernels (graph replays: their kernels reach the operators from the device side)."""
+    wl = synth.make_workload("c3", scale, truth=False)
+    ev = wl.events.copy()
+    rng = np.random.default_rng(int(1000 * scale + 10 * dup + 100 * multi))
+    joins = np.isin(ev["kind"], (2, 3, 4))
+    if hashed:
+        with np.errstate(over="ignore"):
+            ev["corr_id"][joins] *= np.int64(-7046029254386353131)
+        ev["corr_id"][np.nonzero(joins)[0][:2]] = (-2**63, 2**63 - 1)
+    for kinds, frac in (((2,), dup), ((3, 4), multi)):
+        at = np.nonzero(np.isin(ev["kind"], kinds))[0]
+        take = rng.choice(at, size=int(len(at) * frac), replace=False)
+        for pid in np.unique(ev["pid"]):
+            mine = take[ev["pid"][take] == pid]
+            pool = at[ev["pid"][at] == pid]
+            if len(mine):
+                ev["corr_id"][mine] = ev["corr_id"][rng.choice(pool, size=len(mine))]
+    o, g = both(ev, wl.win_off, wl.win_t0, wl.win_t1, comm_sizes=wl.comm_sizes)
+    if multi:
+        assert int(o["kernels_of_launch"].max()) > 1 and int(o["op_n_kernels"].sum()) > 1000
+    if dup:
+        assert int(o["join_sum"]["n_dup_launch"].sum()) > 0
+
+
+@pytest.mark.parametrize("bad", [1, 2, 255, 257, 4097, 16384, 16385])
+def test_dropped_tail_ranked_by_counting_and_by_sorting(bad):
+    """Dropped records around the size where the tail's order is no longer found by counting, with
+    equal tuples among them, in two windows."""
+    wl = synth.make_workload("c4", 0.05, truth=False, n_windows=2)
+    ev = wl.events.copy()
+    rng = np.random.default_rng(bad)
+    at = rng.choice(len(ev), size=bad, replace=False)
+    ev[at] = ev[rng.choice(at, size=bad)]  # equal records
+    ev["kind"][at] = rng.choice((9, -1, 6), size=bad)
+    both(ev, wl.win_off, wl.win_t0, wl.win_t1, comm_sizes=wl.comm_sizes)
+
+
+@pytest.mark.parametrize("n", [104_857, 104_858, 700_001])
+def test_pageable_records_around_the_threshold_of_the_staged_upload(n):
+    """Host records just below and above four megabytes and over several rings of buffers, twice."""
+    from runners import assert_same, run_gpu
+    wl = synth.make_workload("c2", 0.05, truth=False)
+    ev = np.ascontiguousarray(wl.events[:n])
+    assert len(ev) == n
+    off = [0, n]
+    a = run_gpu(ev, off, wl.win_t0, wl.win_t1, on_device=True)
+    for _ in range(2):
+        assert_same(a, run_gpu(ev, off, wl.win_t0, wl.win_t1, on_device=False))
