@@ -383,11 +383,6 @@ __global__ void __launch_bounds__(AG_THREADS, 6) k_agg(AggArgs a) {
   agg_flush(a, s);
 }
 
-// compaction of the non-empty rows in dense (= key) order
-struct AggRowIn {
-  const u64 *cnt;
-  __device__ u64 operator()(int64_t g) const { return cnt[g] ? 1ull : 0ull; }
-};
 struct AggRowOut {
   const u64 *cnt, *sum, *minc, *maxb;
   const u32 *hist;
@@ -398,27 +393,63 @@ struct AggRowOut {
   int32_t *g_window, *g_pid, *g_name;
   int64_t *g_count, *g_sum, *g_min, *g_max;
   u32 *g_hist;
-  __device__ void operator()(int64_t g, u64 row, u64 v) const {
-    if (!v) return;
-    int64_t slot = g / R;
-    g_window[row] = (int32_t)(slot / n_pids);
-    g_pid[row] = tt->pid_value[slot % n_pids];
-    g_name[row] = name_of ? name_of[g % R] : (int32_t)(min_name + g % R);
-    g_count[row] = (int64_t)cnt[g];
-    g_sum[row] = (int64_t)sum[g];
-    g_min[row] = (int64_t)((~minc[g]) ^ (1ull << 63));
-    g_max[row] = (int64_t)(maxb[g] ^ (1ull << 63));
-    // the 40 bins as ten 16-byte loads issued together, then ten stores (rows are 160 B apart,
-    // both tables 16-byte aligned)
-    const uint4 *src = reinterpret_cast<const uint4 *>(hist + (size_t)g * TA_NBINS);
-    uint4 *dst = reinterpret_cast<uint4 *>(g_hist + row * TA_NBINS);
-    uint4 q[TA_NBINS / 4];
-#pragma unroll
-    for (int b = 0; b < TA_NBINS / 4; b++) q[b] = src[b];
-#pragma unroll
-    for (int b = 0; b < TA_NBINS / 4; b++) dst[b] = q[b];
-  }
 };
+
+// Dense cells: compaction of the non-empty ones in cell (= key) order, 256 cells per CTA, chained over
+// the CTAs.  The histograms (160 of a row's 200 bytes) are copied by the CTA together, 16 bytes per
+// thread, rows side by side: one thread per row copying its own took 36 us for the 4096 cells of a
+// prefill window, most of it waiting.
+#define AC_THREADS 256
+__global__ void __launch_bounds__(AC_THREADS) k_agg_rows(int64_t G, AggRowOut o, u64 *state, u64 *total,
+                                                         u32 *ticket, int32_t *status, Tail tail) {
+  TA_PDL();
+  __shared__ u64 tmp[33];
+  __shared__ u64 s_excl;
+  __shared__ u32 s_cell[AC_THREADS];
+  __shared__ int s_fail, s_tile;
+  const int tid = threadIdx.x;
+  if (tid == 0) s_tile = (int)atomicAdd(ticket, 1u);
+  __syncthreads();
+  const int tile = s_tile;
+  const int64_t g = (int64_t)tile * AC_THREADS + tid;
+  const bool failed = ta_failed(status);
+  const u64 c = !failed && g < G ? o.cnt[g] : 0;
+  u64 rows;
+  const u64 ex = block_scan_exclusive<OpAdd>(c ? 1ull : 0ull, OpAdd(), tmp, &rows);
+  if (tid < 32) {
+    bool gave_up = false;
+    const u64 e = failed ? 0 : tile_lookback<OpAdd>(state, tile, rows, OpAdd(), status, &gave_up);
+    if (tid == 0) {
+      s_excl = e;
+      s_fail = failed || gave_up;
+      if (!s_fail && tile == (int)gridDim.x - 1) *total = e + rows;
+    }
+  }
+  if (c) s_cell[ex] = (u32)tid;
+  __syncthreads();
+  if (!s_fail) {
+    const u64 first = s_excl;
+    if (c) {
+      const u64 row = first + ex;
+      const int64_t slot = g / o.R, r = g - slot * o.R;
+      o.g_window[row] = (int32_t)(slot / o.n_pids);
+      o.g_pid[row] = o.tt->pid_value[slot % o.n_pids];
+      o.g_name[row] = o.name_of ? o.name_of[r] : (int32_t)(o.min_name + r);
+      o.g_count[row] = (int64_t)c;
+      o.g_sum[row] = (int64_t)o.sum[g];
+      o.g_min[row] = (int64_t)((~o.minc[g]) ^ (1ull << 63));
+      o.g_max[row] = (int64_t)(o.maxb[g] ^ (1ull << 63));
+    }
+    const uint4 *src = reinterpret_cast<const uint4 *>(o.hist) + (size_t)tile * AC_THREADS * (TA_NBINS / 4);
+    uint4 *dst = reinterpret_cast<uint4 *>(o.g_hist) + first * (TA_NBINS / 4);
+    const int words = (int)rows * (TA_NBINS / 4);
+    for (int i = tid; i < words; i += AC_THREADS) {
+      const int r = i / (TA_NBINS / 4);
+      dst[i] = src[s_cell[r] * (TA_NBINS / 4) + (i - r * (TA_NBINS / 4))];
+    }
+  }
+  run_tail(tail);
+}
 
 // ---- marked cells: numbering, and what is left to write of a row -----------------------------
 struct AggBitsIn {
@@ -768,8 +799,8 @@ ta_status ta_run_aggregate(ta_window *h, uint32_t kind_mask, int value_sel, ta_a
   // (pass, scan, round trip) are worth.  512 windows of 65 k records have 33 M cells, one in
   // twenty of them occupied: 1.85 ms per call dense.
   if (G * 232 <= 8 * h->n_valid + (64ll << 20)) {
-    ScanTemp t;
-    size_t tb = 4 * Carver::pad((size_t)G * 8) + Carver::pad((size_t)G * TA_NBINS * 4) + scan_temp_bytes(G) + 256;
+    const int64_t tiles = (G + AC_THREADS - 1) / AC_THREADS;
+    size_t tb = 4 * Carver::pad((size_t)G * 8) + Carver::pad((size_t)G * TA_NBINS * 4) + Carver::pad((size_t)(tiles + 2) * 8);
     ta_status zs;
     tmpb = ta_zalloc(h, tb, &zs);
     if (!tmpb) return zs;
@@ -779,16 +810,16 @@ ta_status ta_run_aggregate(ta_window *h, uint32_t kind_mask, int value_sel, ta_a
     a.d_minc = ct.take<u64>(G);
     a.d_maxb = ct.take<u64>(G);
     a.d_hist = ct.take<u32>((size_t)G * TA_NBINS);
-    scan_temp_carve(ct.base + ct.off, G, &t);
+    u64 *state = ct.take<u64>(tiles + 2), *total = state + tiles;
     run_agg();
     // the rows are compacted without waiting for their count: it is bounded by cells and records
     carve_rows(G < h->n_valid ? G : h->n_valid);
     if (!outb) return TA_ERR_OOM;
     ro.cnt = a.d_cnt; ro.sum = a.d_sum; ro.minc = a.d_minc; ro.maxb = a.d_maxb; ro.hist = a.d_hist;
-    AggRowIn ri{a.d_cnt};
-    TA_TRY(ta_queue_d2h(h, &ng, t.total, 8));
+    TA_TRY(ta_queue_d2h(h, &ng, total, 8));
     TA_TRY(ta_queue_d2h(h, status, h->d_status, sizeof(status)));
-    TA_TRY((launch_scan<OpAdd, AggRowIn, AggRowOut>(h, G, ri, ro, OpAdd(), t, true)));
+    ta_launch(k_agg_rows, (unsigned)tiles, AC_THREADS, 0, st, G, ro, state, total, (u32 *)(total + 1),
+              h->d_status, ta_tail(h, tiles));
   } else {
     const int64_t words = (G + 31) / 32;
     ScanTemp t;
