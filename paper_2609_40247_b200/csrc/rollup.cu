@@ -106,8 +106,7 @@ __global__ void __launch_bounds__(RO_THREADS) k_roll_replays(RollArgs a) {
   }
 }
 
-__global__ void __launch_bounds__(RO_THREADS) k_roll_finalize(RollArgs a) {
-  TA_PDL();
+__device__ __forceinline__ void roll_finalize(const RollArgs &a) {
   int64_t p0, tile_end;
   if (!roll_tile(a, 0, &p0, &tile_end)) return;
   int16_t kd[RO_ITEMS];
@@ -152,6 +151,12 @@ __global__ void __launch_bounds__(RO_THREADS) k_roll_finalize(RollArgs a) {
   }
 }
 
+__global__ void __launch_bounds__(RO_THREADS) k_roll_finalize(RollArgs a, Tail tail) {
+  TA_PDL();
+  roll_finalize(a);
+  run_tail(tail);
+}
+
 ta_status ta_run_rollup(ta_window *h, ta_rollup_result *out, ta_rollup_summary *out_summary) {
   cudaStream_t st = h->stream;
   memset(out, 0, sizeof(*out));
@@ -186,13 +191,15 @@ ta_status ta_run_rollup(ta_window *h, ta_rollup_result *out, ta_rollup_summary *
   a.lane_dom_end = h->d_lane_dom_end; a.lane_domain = h->sorted.lane_domain; a.status = h->d_status;
   const unsigned tiles = (unsigned)((h->n_valid + RO_TILE - 1) / RO_TILE);
   ta_launch(k_roll_ops, tiles, RO_THREADS, 0, st, a);
-  ta_launch(k_roll_replays, tiles, RO_THREADS, 0, st, a);
-  ta_launch(k_roll_finalize, tiles, RO_THREADS, 0, st, a);
-  TA_CHECK_CUDA(h, cudaGetLastError());
+  if (h->multi_launch) ta_launch(k_roll_replays, tiles, RO_THREADS, 0, st, a);  // (the join knows whether there are any)
   std::vector<u64> hs((size_t)W * 3);
-  TA_TRY(ta_queue_d2h(h, hs.data(), a.win_sum, (size_t)W * 24));
   int32_t words[ST_WORDS];
-  TA_TRY(ta_read_status(h, words));
+  TA_TRY(ta_queue_d2h(h, hs.data(), a.win_sum, (size_t)W * 24));
+  TA_TRY(ta_queue_d2h(h, words, h->d_status, sizeof(words)));
+  const Tail tail = W * 24 <= 4096 ? ta_tail(h, tiles) : Tail();
+  ta_launch(k_roll_finalize, tiles, RO_THREADS, 0, st, a, tail);
+  TA_CHECK_CUDA(h, cudaGetLastError());
+  TA_TRY(ta_sync_fetch(h));
   if (words[ST_ERR]) return (ta_status)words[ST_ERR];
   for (int w = 0; w < W; w++) {
     out_summary[w].n_graph_launches = (int64_t)hs[(size_t)w * 3];

@@ -98,7 +98,6 @@ static inline ta_status launch_scan(ta_window *h, int64_t n, In in, Out out, Op 
   if (n <= 0) return TA_OK;
   int64_t tiles = (n + SC_TILE - 1) / SC_TILE;
   Tail tail;
-  tail.m = 0;
   if (last) tail = ta_tail(h, tiles);
   ta_launch(k_scan<Op, In, Out>, (unsigned)tiles, SC_THREADS, 0, h->stream, n, in, out, op, t, h->d_status, tail);
   TA_CHECK_CUDA(h, cudaGetLastError());

@@ -104,8 +104,7 @@ __device__ __forceinline__ void sol_flush(SolAcc &acc, ta_sol_summary *row, u64 
 }
 
 // Persistent CTAs, each over a contiguous range of tiles.
-__global__ void __launch_bounds__(SO_THREADS) k_operator_sol(SolArgs a, int64_t n_tiles, int64_t tiles_per_cta) {
-  TA_PDL();
+__device__ __forceinline__ void operator_sol(const SolArgs &a, int64_t n_tiles, int64_t tiles_per_cta) {
   __shared__ int s_lane0, s_lane1;
   __shared__ u64 red[7][SO_THREADS / 32];
   if (ta_failed(a.status)) return;
@@ -226,13 +225,19 @@ __global__ void __launch_bounds__(SO_THREADS) k_operator_sol(SolArgs a, int64_t 
   if (cw >= 0) sol_flush(acc, &a.sum[cw], red);
 }
 
+__global__ void __launch_bounds__(SO_THREADS) k_operator_sol(SolArgs a, int64_t n_tiles, int64_t tiles_per_cta,
+                                                             Tail tail) {
+  TA_PDL();
+  operator_sol(a, n_tiles, tiles_per_cta);
+  run_tail(tail);
+}
+
 ta_status ta_run_sol(ta_window *h, const double *flops, const double *bytes, int on_device,
                      double peak_flops, double peak_bw, ta_sol_result *out, ta_sol_summary *out_summary) {
   const int64_t n = h->n, nn = n > 0 ? n : 1;
   const int W = h->W;
   cudaStream_t st = h->stream;
-  size_t keep = 3 * Carver::pad((size_t)nn * 8) + Carver::pad((size_t)nn) +
-                Carver::pad((size_t)W * sizeof(ta_sol_summary)) + 256;
+  size_t keep = 3 * Carver::pad((size_t)nn * 8) + Carver::pad((size_t)nn) + 256;
   void *kb = ta_dalloc(h, keep);
   if (!kb) return TA_ERR_OOM;
   Carver ck(kb);
@@ -240,8 +245,9 @@ ta_status ta_run_sol(ta_window *h, const double *flops, const double *bytes, int
   memset(&a, 0, sizeof(a));
   a.mfu = ck.take<double>(nn); a.mbu = ck.take<double>(nn); a.sol = ck.take<double>(nn);
   a.state = ck.take<uint8_t>(nn);
-  a.sum = ck.take<ta_sol_summary>(W);
-  TA_CHECK_CUDA(h, cudaMemsetAsync(a.sum, 0, (size_t)W * sizeof(ta_sol_summary), st));
+  ta_status zs;
+  a.sum = (ta_sol_summary *)ta_zalloc(h, (size_t)W * sizeof(ta_sol_summary), &zs);
+  if (!a.sum) return zs;
   void *tmp = nullptr;
   if (!on_device && n > 0) {
     tmp = ta_dalloc(h, 2 * Carver::pad((size_t)n * 8));
@@ -259,17 +265,20 @@ ta_status ta_run_sol(ta_window *h, const double *flops, const double *bytes, int
   a.flops = flops; a.bytes = bytes; a.peak_flops = peak_flops; a.peak_bw = peak_bw;
   a.lane_off = h->sorted.lane_off; a.lane_window = h->sorted.lane_window; a.status = h->d_status;
   a.lane_domain = h->sorted.lane_domain; a.lane_dom_end = h->d_lane_dom_end;
+  std::vector<ta_sol_summary> hs(W);
+  int32_t words[ST_WORDS];
+  TA_TRY(ta_queue_d2h(h, hs.data(), a.sum, (size_t)W * sizeof(ta_sol_summary)));
+  TA_TRY(ta_queue_d2h(h, words, h->d_status, sizeof(words)));
   if (n > 0) {
     const int64_t n_tiles = (n + SO_TILE - 1) / SO_TILE;
     const int64_t ctas = n_tiles < 148 * 8 ? n_tiles : 148 * 8;
     const int64_t per = (n_tiles + ctas - 1) / ctas;
-    ta_launch(k_operator_sol, (unsigned)((n_tiles + per - 1) / per), SO_THREADS, 0, st, a, n_tiles, per);
+    const int64_t grid = (n_tiles + per - 1) / per;
+    const Tail tail = W * sizeof(ta_sol_summary) <= 4096 ? ta_tail(h, grid) : Tail();
+    ta_launch(k_operator_sol, (unsigned)grid, SO_THREADS, 0, st, a, n_tiles, per, tail);
     TA_CHECK_CUDA(h, cudaGetLastError());
   }
-  std::vector<ta_sol_summary> hs(W);
-  TA_TRY(ta_queue_d2h(h, hs.data(), a.sum, (size_t)W * sizeof(ta_sol_summary)));
-  int32_t words[ST_WORDS];
-  TA_TRY(ta_read_status(h, words));
+  TA_TRY(ta_sync_fetch(h));
   if (tmp) ta_dfree(h, tmp);
   if (words[ST_ERR]) return (ta_status)words[ST_ERR];
   for (int w = 0; w < W; w++) out_summary[w] = hs[w];

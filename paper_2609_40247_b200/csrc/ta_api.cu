@@ -254,7 +254,6 @@ static u32 next_seq(ta_window *h) { return ++h->fetch_seq ? h->fetch_seq : ++h->
 static volatile u32 *seq_word(unsigned char *pin) { return (volatile u32 *)(pin + TA_PIN_BYTES); }
 Tail ta_tail(ta_window *h, int64_t grid) {
   Tail t;
-  memset(&t, 0, sizeof(t));
   if (!h->pin_dev || h->fetch.empty() || h->fetch.size() > TA_TAIL_MAX || grid > 1024) return t;
   for (const ta_window::Fetch &f : h->fetch)
     if (f.bytes > 4096 || (f.bytes & 3u)) return t;

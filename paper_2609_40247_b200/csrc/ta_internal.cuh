@@ -290,7 +290,7 @@ ta_status ta_read_status(ta_window *h, int32_t *host_words /*ST_WORDS*/);
 struct Tail {
   const void *src[TA_TAIL_MAX];
   unsigned off[TA_TAIL_MAX], bytes[TA_TAIL_MAX];  // multiples of 4 bytes
-  int m;                                         // 0: nothing to do
+  int m = 0;                                     // 0: nothing to do
   unsigned char *pin_dev;
   u32 *ticket;
   u32 seq;

@@ -340,9 +340,11 @@ class _Blocks:
     def __init__(self, handle):
         self.handle = handle
         self.known = []  # (first address, address behind, tensor)
+        self.last = (0, 0, None)
 
     def slice(self, ptr, nbytes):
-        for lo, hi, t in self.known:
+        for self.last in self.known:
+            lo, hi, t = self.last
             if lo <= ptr and ptr + nbytes <= hi:
                 return t[ptr - lo:ptr - lo + nbytes]
         import torch
@@ -355,7 +357,8 @@ class _Blocks:
                 raise ValueError("not a result of an open window")
             lo, size = base.value, room.value
         t = torch.as_tensor(_DevView(lo, size, h), device=f"cuda:{h.device}")
-        self.known.append((lo, lo + size, t))
+        self.last = (lo, lo + size, t)
+        self.known.append(self.last)
         return t[ptr - lo:ptr - lo + nbytes]
 
 
@@ -385,6 +388,9 @@ class _Result:
         if nbytes == 0 or not ptr:
             import torch
             return torch.empty(0, dtype=torch.uint8, device=f"cuda:{self._handle.device}")
+        lo, hi, t = self._blocks.last
+        if lo <= ptr and ptr + nbytes <= hi:
+            return t[ptr - lo:ptr - lo + nbytes]
         return self._blocks.slice(ptr, nbytes)
 
     # Tables are mostly read together: a request for one brings the other small ones of the result
