@@ -89,6 +89,7 @@ struct CpArgs {
   int32_t *jump_in, *jump_out;  // per listed wait: the wait 2^round steps down the path, or -1
   uint8_t *mark;        // per listed wait: on a path
   int64_t n_list;
+  const u32 *gate;      // k_cp_mark: run only if this word is set (null: run)
   u64 *acc;             // [slot][CP_ACC]
   uint8_t *on_path;
   int32_t *status;
@@ -125,6 +126,42 @@ __device__ __forceinline__ int32_t cp_last_ended(const CpArgs &a, int first_dev_
       const i64 e = a.te[lo - 1];
       if (best < 0 || e >= best_e) { best = (int32_t)(lo - 1); best_e = e; }
     }
+  }
+  return best;
+}
+
+// The same for the process of host position p and ends before `limit`, by the lanes of a warp together
+// (act: the lanes that are here), one stream per lane and round.
+__device__ __forceinline__ int32_t cp_last_ended_warp(const CpArgs &a, u32 act, int64_t p, i64 limit) {
+  const int l = lane_of_pos(a.lane_off, a.n_lanes, p);
+  const int slot = a.lane_slot[l], n_act = __popc(act);
+  const int rank = __popc(act & ((1u << (threadIdx.x & 31)) - 1u));
+  int32_t best = -1;
+  i64 best_e = 0;
+  for (int d0 = a.lane_dom_next[l];; d0 += n_act) {
+    const int dl = d0 + rank;
+    const bool mine = dl < a.n_lanes && a.lane_slot[dl] == slot && a.lane_domain[dl] == 1;
+    if (mine) {
+      int64_t lo = a.lane_off[dl], hi = a.lane_off[dl + 1];
+      const int64_t begin = lo;
+      while (lo < hi) {
+        const int64_t mid = (lo + hi) >> 1;
+        if (a.te[mid] < limit) lo = mid + 1;
+        else hi = mid;
+      }
+      if (lo > begin) {
+        const i64 e = a.te[lo - 1];
+        if (best < 0 || e >= best_e) { best = (int32_t)(lo - 1); best_e = e; }
+      }
+    }
+    if (!__all_sync(act, mine)) break;  // the lanes of a process are neighbours: there are no more
+  }
+  // greatest end, then highest position
+  for (u32 m = __ballot_sync(act, best >= 0); m; m &= m - 1) {
+    const int src = __ffs((int)m) - 1;
+    const int32_t ob = __shfl_sync(act, best, src);
+    const i64 oe = __shfl_sync(act, best_e, src);
+    if (best < 0 || oe > best_e || (oe == best_e && ob > best)) { best = ob; best_e = oe; }
   }
   return best;
 }
@@ -232,6 +269,7 @@ __global__ void __launch_bounds__(CP_THREADS, 3) k_cp_classify(CpArgs a) {
   CpLane ln(a, l0);
   const int sh = a.tsbits + a.idxbits;
   u64 links = 0;
+  unsigned api = 0;  // the thread's API records
   int run_slot = -1;
   u64 run_max = 0;
 #pragma unroll
@@ -255,33 +293,52 @@ __global__ void __launch_bounds__(CP_THREADS, 3) k_cp_classify(CpArgs a) {
       }
       run_max = max(run_max, cp_code(e[j]));
       if (kd[j] == TA_KIND_API) {
-        // last element of the sorted (slot, ts_end) keys below (slot, this call's ts_end)
-        int32_t d = -1;
         if (!a.use_sort) {
-          d = cp_last_ended(a, a.lane_dom_next[ln.l], slot, e[j], false);
-          if (d >= 0 && a.te[d] < s[j]) d = -1;
-        } else if (a.m > 0) {
-          const u64 want = ((u64)slot << a.tsbits) | (u64)(e[j] - a.t0[a.lane_window[ln.l]]);
-          int64_t lo_i = 0, hi_i = a.m;
-          while (lo_i < hi_i) {
-            const int64_t mid = (lo_i + hi_i) >> 1;
-            if ((a.skeys[mid] >> a.idxbits) < want) lo_i = mid + 1;
-            else hi_i = mid;
+          api |= 1u << j;  // searched below, by the warp together
+        } else {
+          // last element of the sorted (slot, ts_end) keys below (slot, this call's ts_end)
+          int32_t d = -1;
+          if (a.m > 0) {
+            const u64 want = ((u64)slot << a.tsbits) | (u64)(e[j] - a.t0[a.lane_window[ln.l]]);
+            int64_t lo_i = 0, hi_i = a.m;
+            while (lo_i < hi_i) {
+              const int64_t mid = (lo_i + hi_i) >> 1;
+              if ((a.skeys[mid] >> a.idxbits) < want) lo_i = mid + 1;
+              else hi_i = mid;
+            }
+            if (lo_i > 0 && (int)(a.skeys[lo_i - 1] >> sh) == slot) {
+              d = cp_pos_of(a, lo_i - 1);
+              if (a.te[d] < s[j]) d = -1;  // finished before the call began: the call did not wait for it
+            }
           }
-          if (lo_i > 0 && (int)(a.skeys[lo_i - 1] >> sh) == slot) {
-            d = cp_pos_of(a, lo_i - 1);
-            if (a.te[d] < s[j]) d = -1;  // finished before the call began: the call did not wait for it
-          }
+          a.cross[p] = d;
         }
-        a.cross[p] = d;
       }
     }
   }
   if (p0 + CP_ITEMS <= a.n) *reinterpret_cast<u64 *>(a.link + p0) = links;
   else
     for (int j = 0; j < CP_ITEMS && p0 + j < a.n; j++) a.link[p0 + j] = (uint8_t)(links >> (8 * j));
-  // the thread's last slot: one atomic per warp when the whole warp is here and sits in that slot
+  // lanes that are here: they left together, at the tile's end, so the mask is the same for all of them
   const u32 act = __activemask();
+  // The waits: each is one binary search per stream of its process, and one thread going through
+  // eight streams for each of its calls is a chain of a hundred dependent reads (54 us for a prefill
+  // window of 250 k records).  The calls of a warp (few) are taken one by one, a lane per stream.
+  if (!a.use_sort) {
+#pragma unroll
+    for (int j = 0; j < CP_ITEMS; j++) {
+      u32 todo = __ballot_sync(act, (api >> j) & 1u);
+      while (todo) {
+        const int src = __ffs((int)todo) - 1;
+        todo &= todo - 1;
+        const int64_t p = __shfl_sync(act, p0 + j, src);
+        const i64 cs = __shfl_sync(act, s[j], src), ce = __shfl_sync(act, e[j], src);
+        const int32_t d = cp_last_ended_warp(a, act, p, ce);
+        if ((threadIdx.x & 31) == src) a.cross[p] = d >= 0 && a.te[d] < cs ? -1 : d;
+      }
+    }
+  }
+  // the thread's last slot: one atomic per warp when the whole warp is here and sits in that slot
   const u32 has = __ballot_sync(act, run_slot >= 0);
   if (!has) return;
   const int s0 = __shfl_sync(act, run_slot, __ffs(has) - 1);
@@ -446,12 +503,9 @@ __global__ void __launch_bounds__(256) k_cp_succ(CpArgs a) {
   a.jump_in[id] = cp_follow(a, a.cross[a.eff_pos[id]], false);
 }
 
-// one thread per (window, process): the sink and the hops from it to the first listed wait
-__global__ void __launch_bounds__(64) k_cp_start(CpArgs a) {
-  TA_PDL();
-  if (ta_failed(a.status)) return;
-  const int64_t slot = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (slot >= a.n_slots) return;
+// one (window, process): the sink and the hops from it to the first listed wait, whose list index it
+// returns (-1: the path meets none)
+__device__ __forceinline__ int32_t cp_start_slot(const CpArgs &a, int64_t slot) {
   const int sh = a.tsbits + a.idxbits;
   // last device record of the slot in (ts_end, position) order
   int32_t dsink = -1;
@@ -475,7 +529,7 @@ __global__ void __launch_bounds__(64) k_cp_start(CpArgs a) {
   }
   const int32_t hsink = a.slot_host_te[slot] ? a.slot_host_pos[slot] : -1;
   int32_t sink;
-  if (dsink < 0 && hsink < 0) return;
+  if (dsink < 0 && hsink < 0) return -1;
   if (dsink >= 0 && hsink >= 0) sink = a.te[dsink] >= a.te[hsink] ? dsink : hsink;  // device positions are the higher ones
   else sink = dsink >= 0 ? dsink : hsink;
   u64 *acc = a.acc + (size_t)slot * CP_ACC;
@@ -500,6 +554,14 @@ __global__ void __launch_bounds__(64) k_cp_start(CpArgs a) {
       }
     }
   }
+  return first;
+}
+__global__ void __launch_bounds__(64) k_cp_start(CpArgs a) {
+  TA_PDL();
+  if (ta_failed(a.status)) return;
+  const int64_t slot = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (slot >= a.n_slots) return;
+  const int32_t first = cp_start_slot(a, slot);
   if (first >= 0) a.mark[first] = 1;
 }
 
@@ -527,10 +589,48 @@ __global__ void __launch_bounds__(256) k_cp_enter(CpArgs a) {
   cp_follow(a, a.cross[a.eff_pos[id]], true);
 }
 
+// The whole chain in one CTA when the list is short: every step above for all of it, a block barrier
+// where the launches of the many-CTA form are (twelve rounds of doubling are twelve launches, and the
+// list's length would have to be fetched before them).  Reports through *chained whether it did.
+#define CP_CHAIN_MAX 8192    // waits listed: 72 KB of shared memory, and eight per thread and round
+#define CP_CHAIN_SLOTS 1024  // processes, one thread each
+__global__ void __launch_bounds__(1024) k_cp_chain(CpArgs a, u32 *chained) {
+  TA_PDL();
+  extern __shared__ int32_t cp_smem[];  // successors, twice; marks
+  int32_t *jump[2] = {cp_smem, cp_smem + CP_CHAIN_MAX};
+  volatile uint8_t *mark = reinterpret_cast<uint8_t *>(cp_smem + 2 * CP_CHAIN_MAX);
+  const u32 m = *a.n_eff;
+  if (ta_failed(a.status) || m > CP_CHAIN_MAX || *a.not_ascending) return;
+  const int tid = threadIdx.x;
+  for (u32 i = tid; i < m; i += blockDim.x) {
+    jump[0][i] = cp_follow(a, a.cross[a.eff_pos[i]], false);
+    mark[i] = 0;
+  }
+  __syncthreads();
+  for (int64_t slot = tid; slot < a.n_slots; slot += blockDim.x) {
+    const int32_t first = cp_start_slot(a, slot);
+    if (first >= 0) mark[first] = 1;
+  }
+  __syncthreads();
+  int cur = 0;
+  for (u32 reach = 1; reach <= m; reach <<= 1) {
+    for (u32 i = tid; i < m; i += blockDim.x) {
+      const int32_t j = jump[cur][i];
+      if (j >= 0 && mark[i]) mark[j] = 1;
+      jump[cur ^ 1][i] = j >= 0 ? jump[cur][j] : -1;
+    }
+    cur ^= 1;
+    __syncthreads();
+  }
+  for (u32 i = tid; i < m; i += blockDim.x)
+    if (mark[i]) cp_follow(a, a.cross[a.eff_pos[i]], true);
+  if (tid == 0) *chained = 1u;
+}
+
 // ---- membership and time classes ---------------------------------------------------------
 __global__ void __launch_bounds__(CP_THREADS) k_cp_mark(CpArgs a) {
   TA_PDL();
-  if (ta_failed(a.status)) return;
+  if (ta_failed(a.status) || (a.gate && !*a.gate)) return;
   __shared__ int s_lane0;
   const int lane = threadIdx.x & 31;
   const int64_t tile_start = (int64_t)blockIdx.x * CP_TILE;
@@ -681,13 +781,13 @@ ta_status ta_run_critpath(ta_window *h, ta_critpath_result *out, ta_critpath_sum
   if (tsbits + slot_bits + idxbits > 64) idxbits = 0;
 
   // results (kept)
-  size_t kb = Carver::pad((size_t)nn) + 5 * Carver::pad((size_t)n_slots * 4) + 2 * Carver::pad((size_t)n_slots * 8) +
+  size_t kb = 5 * Carver::pad((size_t)n_slots * 4) + 2 * Carver::pad((size_t)n_slots * 8) +
               Carver::pad((size_t)n_slots * 64) + 256;
+  uint8_t *on_path = (uint8_t *)ta_dalloc(h, (size_t)nn);  // (the aggregates read it later)
   void *keep = ta_dalloc(h, kb);
-  if (!keep) return TA_ERR_OOM;
+  if (!on_path || !keep) return TA_ERR_OOM;
   Carver ck(keep);
   CpRowOut ro;
-  uint8_t *on_path = ck.take<uint8_t>(nn);
   ro.p_window = ck.take<int32_t>(n_slots); ro.p_pid = ck.take<int32_t>(n_slots);
   ro.p_sink = ck.take<int32_t>(n_slots); ro.p_n_nodes = ck.take<int32_t>(n_slots);
   ro.p_reason = ck.take<int32_t>(n_slots);
@@ -750,6 +850,30 @@ ta_status ta_run_critpath(ta_window *h, ta_critpath_result *out, ta_critpath_sum
   // second attempt sorts the device records by (process slot, ts_end) and searches there.
   void *sortb = nullptr;
   u32 n_list = 0;
+  bool done = false;
+  u32 *chained = a.counter + 4;   // set by k_cp_chain
+  u32 words3[3] = {0, 0, 0};      // length of the list, not ascending, chained
+  u64 rows = 0;
+  int32_t words[ST_WORDS] = {0};
+  std::vector<u64> hacc((size_t)n_slots * CP_ACC);
+  // membership, time classes and rows, and everything the host wants to know of them
+  auto cp_rows = [&](bool assumed) -> ta_status {
+    a.gate = assumed ? chained : nullptr;
+    ta_launch(k_cp_mark, (unsigned)tiles, CP_THREADS, 0, st, a);
+    TA_CHECK_CUDA(h, cudaGetLastError());
+    ro.acc = a.acc; ro.tt = h->d_triples; ro.te = a.te; ro.n_pids = n_pids;
+    ScanTemp s3;
+    TA_TRY(scan_temp_init(h, scan_mem, n_slots, &s3));
+    CpRowIn ri{a.acc};
+    const bool small = hacc.size() * 8 <= 4096;  // (more is copied once the kernels are queued)
+    TA_TRY(ta_queue_d2h(h, &rows, s3.total, 8));
+    TA_TRY(ta_queue_d2h(h, words, h->d_status, sizeof(words)));
+    if (assumed) TA_TRY(ta_queue_d2h(h, words3, a.n_eff, 12));
+    if (small) TA_TRY(ta_queue_d2h(h, hacc.data(), a.acc, hacc.size() * 8));
+    TA_TRY((launch_scan<OpAdd, CpRowIn, CpRowOut>(h, n_slots, ri, ro, OpAdd(), s3, true)));
+    if (!small) TA_TRY(ta_queue_d2h(h, hacc.data(), a.acc, hacc.size() * 8));
+    return ta_sync_fetch(h);
+  };
   for (int attempt = 0; attempt < 2; attempt++) {
     a.use_sort = attempt;
     TA_CHECK_CUDA(h, cudaMemsetAsync(zb, 0, zbytes, st));
@@ -778,51 +902,50 @@ ta_status ta_run_critpath(ta_window *h, ta_critpath_result *out, ta_critpath_sum
     ta_launch(k_cp_classify, (unsigned)tiles, CP_THREADS, 0, st, a);
     ta_launch(k_cp_runs, (unsigned)tiles, CP_THREADS, 0, st, a);
     TA_CHECK_CUDA(h, cudaGetLastError());
+    // First on the assumption that the list of waits is short: everything is queued up to the rows, and
+    // one round trip tells whether the assumptions (ascending ends, short list) held.
+    if (!a.use_sort && n_slots <= CP_CHAIN_SLOTS) {
+      constexpr int smem = CP_CHAIN_MAX * 9;
+      TA_CHECK_CUDA(h, cudaFuncSetAttribute(k_cp_chain, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+      ta_launch(k_cp_chain, 1, 1024, smem, st, a, chained);
+      TA_TRY(cp_rows(true));
+      if (words[ST_ERR]) break;
+      if (words3[2]) { done = true; break; }
+      if (words3[1]) continue;
+      n_list = words3[0];  // a long list
+      break;
+    }
     // the waits that head a host run: a list whose length decides the number of doubling rounds
-    u32 words2[2] = {0, 0};
-    TA_TRY(ta_queue_d2h(h, words2, a.n_eff, 8));
+    TA_TRY(ta_queue_d2h(h, words3, a.n_eff, 8));
     TA_TRY(ta_sync_fetch(h));
-    n_list = words2[0];
-    if (!a.use_sort && words2[1]) continue;
+    n_list = words3[0];
+    if (!a.use_sort && words3[1]) continue;
     break;
   }
-  a.n_list = (int64_t)n_list;
-  const int64_t nl = n_list > 0 ? n_list : 1;
-  void *lb = ta_dalloc(h, 2 * Carver::pad((size_t)nl * 4) + Carver::pad((size_t)nl) + 256);
-  if (!lb) return TA_ERR_OOM;
-  Carver cl(lb);
-  a.jump_in = cl.take<int32_t>(nl);
-  a.jump_out = cl.take<int32_t>(nl);
-  a.mark = cl.take<uint8_t>(nl);
-  TA_CHECK_CUDA(h, cudaMemsetAsync(a.mark, 0, (size_t)nl, st));
-  const unsigned lblocks = (unsigned)((nl + 255) / 256);
-  if (n_list) ta_launch(k_cp_succ, lblocks, 256, 0, st, a);
-  ta_launch(k_cp_start, (unsigned)((n_slots + 63) / 64), 64, 0, st, a);
-  if (n_list) {
-    for (int r = ta_bit_len((uint64_t)n_list); r > 0; r--) {
-      ta_launch(k_cp_double, lblocks, 256, 0, st, a);
-      int32_t *t = a.jump_in; a.jump_in = a.jump_out; a.jump_out = t;
+  void *lb = nullptr;
+  if (!done && !words[ST_ERR]) {
+    a.n_list = (int64_t)n_list;
+    const int64_t nl = n_list > 0 ? n_list : 1;
+    lb = ta_dalloc(h, 2 * Carver::pad((size_t)nl * 4) + Carver::pad((size_t)nl) + 256);
+    if (!lb) return TA_ERR_OOM;
+    Carver cl(lb);
+    a.jump_in = cl.take<int32_t>(nl);
+    a.jump_out = cl.take<int32_t>(nl);
+    a.mark = cl.take<uint8_t>(nl);
+    TA_CHECK_CUDA(h, cudaMemsetAsync(a.mark, 0, (size_t)nl, st));
+    const unsigned lblocks = (unsigned)((nl + 255) / 256);
+    if (n_list) ta_launch(k_cp_succ, lblocks, 256, 0, st, a);
+    ta_launch(k_cp_start, (unsigned)((n_slots + 63) / 64), 64, 0, st, a);
+    if (n_list) {
+      for (int r = ta_bit_len((uint64_t)n_list); r > 0; r--) {
+        ta_launch(k_cp_double, lblocks, 256, 0, st, a);
+        int32_t *t = a.jump_in; a.jump_in = a.jump_out; a.jump_out = t;
+      }
+      ta_launch(k_cp_enter, lblocks, 256, 0, st, a);
     }
-    ta_launch(k_cp_enter, lblocks, 256, 0, st, a);
+    TA_TRY(cp_rows(false));
   }
-  ta_launch(k_cp_mark, (unsigned)tiles, CP_THREADS, 0, st, a);
-  TA_CHECK_CUDA(h, cudaGetLastError());
-
-  ro.acc = a.acc; ro.tt = h->d_triples; ro.te = a.te; ro.n_pids = n_pids;
-  ScanTemp s3;
-  TA_TRY(scan_temp_init(h, scan_mem, n_slots, &s3));
-  CpRowIn ri{a.acc};
-  u64 rows = 0;
-  int32_t words[ST_WORDS];
-  std::vector<u64> hacc((size_t)n_slots * CP_ACC);
-  const bool small = hacc.size() * 8 <= 4096;  // (more is copied once the kernels are queued)
-  TA_TRY(ta_queue_d2h(h, &rows, s3.total, 8));
-  TA_TRY(ta_queue_d2h(h, words, h->d_status, sizeof(words)));
-  if (small) TA_TRY(ta_queue_d2h(h, hacc.data(), a.acc, hacc.size() * 8));
-  TA_TRY((launch_scan<OpAdd, CpRowIn, CpRowOut>(h, n_slots, ri, ro, OpAdd(), s3, true)));
-  if (!small) TA_TRY(ta_queue_d2h(h, hacc.data(), a.acc, hacc.size() * 8));
-  TA_TRY(ta_sync_fetch(h));
-  ta_dfree(h, lb);
+  if (lb) ta_dfree(h, lb);
   if (sortb) ta_dfree(h, sortb);
   ta_dfree(h, tmpb);
   if (words[ST_ERR]) return (ta_status)words[ST_ERR];
