@@ -52,9 +52,9 @@ __host__ __device__ __forceinline__ i64 unbias64(u64 v) { return (i64)(v ^ (1ull
 
 // ---- hashed addressing -------------------------------------------------------
 __device__ __forceinline__ u32 join_hash(const JoinArgs &a, int slot, i64 c) {
-  u64 x = (u64)c * 0x9E3779B97F4A7C15ull ^ (u64)(u32)slot * 0xC2B2AE3D27D4EB4Full;
-  x ^= x >> 32;
-  x *= 0xD6E8FEB86659FD93ull;
+  // multiplicative hashing (the golden ratio in 64 bits), twice so that low bits reach the top word
+  u64 x = ((u64)c ^ ((u64)(u32)slot << 40)) * 0x9E3779B97F4A7C15ull;
+  x = (x ^ (x >> 32)) * 0x9E3779B97F4A7C15ull;
   return __umulhi((u32)(x >> 32), a.table_size);
 }
 __device__ __forceinline__ bool join_same(const JoinArgs &a, u32 pos, int slot, i64 c) {

@@ -15,6 +15,7 @@ from __future__ import annotations
 import contextlib
 import ctypes
 import os
+import threading
 
 import numpy as np
 
@@ -264,6 +265,7 @@ def _addr(a):
 # context says which device and stream
 _places: list = [None]
 _place_of: dict = {}
+_place_guard = threading.Lock()
 
 
 @_ALLOC_T
@@ -285,8 +287,11 @@ def _place(device, stream_ptr):
     key = (device, stream_ptr)
     at = _place_of.get(key)
     if at is None:
-        _places.append(key)
-        at = _place_of[key] = len(_places) - 1
+        with _place_guard:
+            at = _place_of.get(key)
+            if at is None:
+                _places.append(key)
+                at = _place_of[key] = len(_places) - 1
     return at
 
 
