@@ -4,16 +4,16 @@
 // of every radix pass.
 //   k_plan          one CTA samples the records and decides how many time bits the packed
 //                   sort key keeps (before anything is known about the lanes);
-//   k_discover      one pass over the 40-byte records: defect counters, the triple and
-//                   communicator sets, value ranges, and one 64-bit word per record
-//                   (dropped flag | triple slot | ts_start - t0);
-//   k_discover_staged  the same for 16-byte aligned input, tiles of records brought to shared
-//                   memory by bulk asynchronous copies (two tiles in flight per CTA); it also
-//                   takes the digit histograms of the radix passes over the time bits and
-//                   counts the records of every triple, so that the first radix pass can build
-//                   the keys itself and no separate key pass is needed;
-//   k_top_hist_words  digit histograms of the passes over the (window, lane) bits of several
-//                   windows (of one window they follow from the per-triple counts);
+//   k_discover_staged  one pass over the 40-byte records, tiles of them brought to shared memory
+//                   by bulk asynchronous copies (two tiles in flight per CTA): defect counters,
+//                   the triple and communicator sets, value ranges, and one 64-bit word per
+//                   record (dropped flag | triple slot | ts_start - t0); it also takes the
+//                   digit histograms of the radix passes over the time bits and counts the
+//                   records of every triple, so that the first radix pass can build the keys
+//                   itself and no separate key pass is needed;
+//   k_top_hist_*    digit histograms of the passes over the (window, lane) bits of several windows,
+//                   from the records counted per window and triple, or from the words when there
+//                   are too many windows for that (of one window: see k_radix_scan_hist);
 //   k_rank_*        one CTA each: sort and rank the few triples / communicator ids;
 //   k_load_pre      turns those words into keys in place - [dropped][window][triple
 //                   rank][(ts_start - t0) >> dshift]{[index in window]} - and takes the
@@ -36,110 +36,11 @@ __device__ __forceinline__ i64 warp_max_i64(i64 v) {
   return v;
 }
 
-// Pass 1 over the records: defect counters, the set of lane triples, the range
-// of name ids and the longest duration.  It also leaves one 64-bit word per record with
-// all the key pass needs - bit 63 for a dropped record, else the triple's slot in the hash
-// table (13 bits) and ts_start - t0 (40 bits) - so that the 40-byte records are read once.
+// The discovery pass leaves one 64-bit word per record with all the sort needs - bit 63 for a dropped
+// record, else the triple's slot in the hash table (13 bits) and ts_start - t0 (40 bits) - so that
+// the 40-byte records are read once.
 #define PRE_DROPPED (1ull << 63)
 #define PRE_TS_BITS 40
-__global__ void __launch_bounds__(256) k_discover(const ta_event *ev, int64_t n, const int64_t *off,
-                                                  const int64_t *t0, const int64_t *t1, int W,
-                                                  TripleTable *tt, CommTable *cm,
-                                                  ta_load_summary *sum, int64_t *misc,
-                                                  int32_t *status, u64 *prekey) {
-  TA_PDL();
-  __shared__ u64 cache[256];  // (triple code << 13) | slot: one word, so a racing reader sees a pair
-  __shared__ u64 ccache[64];
-  cache[threadIdx.x] = TRIPLE_EMPTY;
-  if (threadIdx.x < 64) ccache[threadIdx.x] = TRIPLE_EMPTY;
-  __syncthreads();
-  i64 mn = INT64_MAX, mx = INT64_MIN, md = 0, qmn = INT64_MAX, qmx = INT64_MIN;
-  u64 n_coll = 0;  // kept COLL records: sizes the collective matching without a count round trip
-  u64 n_launch = 0;  // kept LAUNCH records: sizes the join's hash table
-  WindowWalker ww(off, W);
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    Rec r = load_rec(ev, i);
-    int w = ww.at(i);
-    int def = defect_of(r, t0[w], t1[w]);
-    if (def) {
-      int64_t *f = def == 1 ? &sum[w].n_bad_kind
-                            : def == 2 ? &sum[w].n_bad_interval : &sum[w].n_out_of_window;
-      atomicAdd((u64 *)f, 1ull);
-      prekey[i] = PRE_DROPPED;
-      continue;
-    }
-    mn = min(mn, (i64)r.name);
-    mx = max(mx, (i64)r.name);
-    md = max(md, r.ts_end - r.ts_start);
-    n_launch += r.kind == TA_KIND_LAUNCH;
-    if (r.kind == TA_KIND_COLL) {  // communicator set and sequence range
-      n_coll++;
-      qmn = min(qmn, (i64)r.seq);
-      qmx = max(qmx, (i64)r.seq);
-      u64 cc = (u64)r.corr ^ (1ull << 63);
-      u32 ch = hash_code(cc);
-      if (cc == TRIPLE_EMPTY) ta_set_err(status, TA_ERR_INVALID_ARG);  // reserved id
-      else if (ccache[ch & 63] != cc) {
-        u32 slot = ch & (TA_COMM_SLOTS - 1);
-        bool ok = false;
-        for (int probe = 0; probe < TA_COMM_SLOTS; probe++) {
-          u64 cur = ld_relaxed(&cm->slots[slot]);
-          if (cur == ~cc) { ok = true; break; }
-          if (cur == 0) {
-            u64 old = atomicCAS(&cm->slots[slot], 0ull, ~cc);
-            if (old == 0 || old == ~cc) { ok = true; break; }
-          }
-          slot = (slot + 1) & (TA_COMM_SLOTS - 1);
-        }
-        if (!ok) ta_set_err(status, TA_ERR_TOO_LARGE);
-        ccache[ch & 63] = cc;
-      }
-    }
-    u64 code = triple_code(r.pid, r.kind, r.stream);
-    u32 hsh = hash_code(code);
-    const u64 ts_rel = (u64)(r.ts_start - t0[w]);
-    const u64 hit = cache[hsh & 255];
-    if ((hit >> 13) == code) {  // a stale miss only costs a probe
-      prekey[i] = ((hit & (TA_TRIPLE_SLOTS - 1)) << PRE_TS_BITS) | ts_rel;
-      continue;
-    }
-    u32 slot = hsh & (TA_TRIPLE_SLOTS - 1);
-    bool done = false;
-    for (int probe = 0; probe < TA_TRIPLE_SLOTS; probe++) {
-      u64 cur = ld_relaxed(&tt->slots[slot]);
-      if (cur == code + 1) { done = true; break; }
-      if (cur == 0) {
-        u64 old = atomicCAS(&tt->slots[slot], 0ull, code + 1);
-        if (old == 0 || old == code + 1) { done = true; break; }
-      }
-      slot = (slot + 1) & (TA_TRIPLE_SLOTS - 1);
-    }
-    if (!done) ta_set_err(status, TA_ERR_TOO_LARGE);
-    cache[hsh & 255] = (code << 13) | slot;
-    prekey[i] = ((u64)slot << PRE_TS_BITS) | ts_rel;
-  }
-  mn = warp_min_i64(mn);
-  mx = warp_max_i64(mx);
-  md = warp_max_i64(md);
-  qmn = warp_min_i64(qmn);
-  qmx = warp_max_i64(qmx);
-  n_coll = warp_reduce(n_coll, OpAdd());
-  n_launch = warp_reduce(n_launch, OpAdd());
-  if ((threadIdx.x & 31) == 0 && n_launch) atomicAdd((u64 *)&misc[8], n_launch);
-  if ((threadIdx.x & 31) == 0 && qmn != INT64_MAX) {
-    atomicMin((i64 *)&misc[3], qmn);
-    atomicMax((i64 *)&misc[4], qmx);
-    atomicAdd((u64 *)&misc[5], n_coll);
-  }
-  if ((threadIdx.x & 31) == 0) {
-    if (mn != INT64_MAX) {
-      atomicMin((i64 *)&misc[0], mn);
-      atomicMax((i64 *)&misc[1], mx);
-    }
-    if (md > 0) atomicMax((i64 *)&misc[2], md);
-  }
-}
 
 // ---- planning: how many time bits the packed key keeps -----------------------------------
 // The sort settles the order down to cells of 2^d ns; records of one lane that share a cell
@@ -162,14 +63,13 @@ struct PlanWindows {
 __global__ void __launch_bounds__(PL_THREADS) k_plan(const ta_event *ev, int64_t n, int64_t *off,
                                                      const int64_t *t0, const int64_t *t1, int W,
                                                      int sbits, int64_t max_span, int64_t max_win,
-                                                     int64_t *misc, PlanWindows pw, int sample) {
+                                                     int64_t *misc, PlanWindows pw) {
   TA_PDL();
   if (threadIdx.x < pw.n) off[threadIdx.x] = pw.v[threadIdx.x];
   if (threadIdx.x < 16) {  // [0] / [1] smallest / largest name, [3] / [4] sequence number, the rest 0
     const int k = threadIdx.x;
     misc[k] = k == 0 || k == 3 ? INT64_MAX : k == 1 || k == 4 ? INT64_MIN : 0;
   }
-  if (!sample) return;
   __shared__ u64 code[PL_SLOTS];
   __shared__ u32 cnt[PL_SLOTS];
   __shared__ u32 s_max, s_valid;
@@ -229,6 +129,8 @@ __global__ void __launch_bounds__(PL_THREADS) k_plan(const ta_event *ev, int64_t
 #endif
 #define DS_TILE (DS_THREADS * DS_RPT)     // 512 records = 20480 bytes
 #define DS_TILE_BYTES (DS_TILE * 40)
+#define DS_CACHE 512
+#define DS_PROBES 4
 #define DS_WAIT_POLLS (1 << 18)  // a tile arrives within microseconds; each poll may itself wait a little
 
 __device__ __forceinline__ u32 smem_addr(const void *p) { return (u32)__cvta_generic_to_shared(p); }
@@ -272,14 +174,15 @@ struct DiscoverArgs {
   int32_t *status;
   u64 *prekey;
   u32 *hist;      // [pass][256]: digit histograms of the passes over time bits
-  u32 *slot_cnt;  // [TA_TRIPLE_SLOTS] kept records per triple slot, or null (several windows)
+  u32 *slot_cnt;  // [window][TA_TRIPLE_SLOTS] kept records per triple slot, or null (too many windows)
   int sbits, ibits;
 };
 
 struct __align__(128) DiscoverSmem {
-  unsigned char buf[2][DS_TILE_BYTES];
+  unsigned char buf[2][DS_TILE_BYTES + 16];  // records that begin at an odd eight bytes: copied from the eight before on
   u64 bar[2];
-  u64 cache[256];
+  u64 cache[DS_CACHE];  // (triple code << 13) | slot of the triples this CTA has met; an entry, once taken, stays
+  u32 count[DS_CACHE];  // records of that triple, in the window w_cnt, not yet added to the global counters
   u64 ccache[64];
   u32 hist[5][256];
   int fail;
@@ -290,7 +193,7 @@ __global__ void __launch_bounds__(DS_THREADS) k_discover_staged(DiscoverArgs a) 
   extern __shared__ __align__(128) unsigned char ds_raw[];
   DiscoverSmem &s = *reinterpret_cast<DiscoverSmem *>(ds_raw);
   const int tid = threadIdx.x, lane = tid & 31;
-  for (int i = tid; i < 256; i += DS_THREADS) s.cache[i] = TRIPLE_EMPTY;
+  for (int i = tid; i < DS_CACHE; i += DS_THREADS) { s.cache[i] = TRIPLE_EMPTY; s.count[i] = 0; }
   if (tid < 64) s.ccache[tid] = TRIPLE_EMPTY;
   for (int i = tid; i < 5 * 256; i += DS_THREADS) (&s.hist[0][0])[i] = 0;
   if (tid == 0) {
@@ -317,40 +220,68 @@ __global__ void __launch_bounds__(DS_THREADS) k_discover_staged(DiscoverArgs a) 
   int32_t mn = INT32_MAX, mx = INT32_MIN, qmn = INT32_MAX, qmx = INT32_MIN;
   i64 md = 0;
   u32 n_coll = 0, n_launch = 0;
-  WindowWalker ww(a.off, a.W);
+  WindowWalker ww(a.off, a.W), wt(a.off, a.W);
   int cw = -1;  // window whose bounds are in registers
+  int w_cnt = 0;  // window the CTA's counts are of: that of the tile's first record
+  auto flush_counts = [&]() {
+    for (int i = tid; i < DS_CACHE; i += DS_THREADS)
+      if (s.count[i]) {
+        atomicAdd(&a.slot_cnt[w_cnt * TA_TRIPLE_SLOTS + (int)(s.cache[i] & (TA_TRIPLE_SLOTS - 1))], s.count[i]);
+        s.count[i] = 0;
+      }
+  };
   i64 ct0 = 0, ct1 = 0;
   int64_t tile = blockIdx.x;
   auto tile_bytes = [&](int64_t t) -> u32 {
     const int64_t cntr = min((int64_t)DS_TILE, a.n - t * DS_TILE);
     return (u32)(cntr * 40);
   };
-  // a tile whose size is no multiple of 16 bytes (an odd number of records, the last tile only)
-  // is copied with plain loads instead
-  if (tid == 0 && tile < n_tiles && (tile_bytes(tile) & 15u) == 0)
-    bulk_load(s.buf[0], reinterpret_cast<const unsigned char *>(a.ev) + tile * DS_TILE_BYTES, tile_bytes(tile),
-              &s.bar[0]);
+  // A bulk copy starts and ends on 16 bytes.  Records at an odd eight bytes (mis = 8) are copied with
+  // the eight bytes in front of them and behind them; the first and the last tile, where those are not
+  // the caller's, with plain loads, as is a tile whose size is no multiple of 16 bytes (the last).
+  const u32 mis = (u32)((uintptr_t)a.ev & 15u);
+  auto bulk_tile = [&](int64_t t) -> bool {
+    return mis ? t > 0 && t + 1 < n_tiles : (tile_bytes(t) & 15u) == 0;
+  };
+  auto load_tile = [&](int64_t t, int b) {
+    bulk_load(s.buf[b], reinterpret_cast<const unsigned char *>(a.ev) + t * DS_TILE_BYTES - mis,
+              tile_bytes(t) + 2 * mis, &s.bar[b]);
+  };
+  if (tid == 0 && tile < n_tiles && bulk_tile(tile)) load_tile(tile, 0);
+  u32 phase[2] = {0, 0};  // copies waited for so far, per buffer
   for (int it = 0; tile < n_tiles; tile += gridDim.x, it++) {
     const int cur = it & 1;
     const int64_t nxt = tile + gridDim.x;
-    if (tid == 0 && nxt < n_tiles && (tile_bytes(nxt) & 15u) == 0)
-      bulk_load(s.buf[cur ^ 1], reinterpret_cast<const unsigned char *>(a.ev) + nxt * DS_TILE_BYTES,
-                tile_bytes(nxt), &s.bar[cur ^ 1]);
+    if (tid == 0 && nxt < n_tiles && bulk_tile(nxt)) load_tile(nxt, cur ^ 1);
     const u32 bytes = tile_bytes(tile);
     const int count = (int)(bytes / 40);
-    if ((bytes & 15u) == 0) {
+    if (bulk_tile(tile)) {
       // one thread polls the barrier; the others sleep at the block barrier below instead of
       // spending issue slots on polls
-      if (tid == 0 && !mbar_wait(&s.bar[cur], (u32)((it >> 1) & 1))) s.fail = 1;
+      if (tid == 0 && !mbar_wait(&s.bar[cur], cur ? phase[1] & 1u : phase[0] & 1u)) s.fail = 1;
+      if (cur) phase[1]++; else phase[0]++;
     } else {
       const u64 *src = reinterpret_cast<const u64 *>(a.ev) + tile * (DS_TILE * 5);
-      u64 *dst = reinterpret_cast<u64 *>(s.buf[cur]);
+      u64 *dst = reinterpret_cast<u64 *>(s.buf[cur] + mis);
       for (int k = tid; k < count * 5; k += DS_THREADS) dst[k] = __ldg(src + k);
+      // a later bulk copy writes the same buffer
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
     __syncthreads();
-    if (s.fail) {  // the copy never arrived: report and leave (nothing this CTA holds is pending use)
-      if (tid == 0) ta_set_err(a.status, TA_ERR_TIMEOUT);
+    if (s.fail) {  // the copy never arrived: report, wait for the one behind it (bounded as well) and leave
+      if (tid == 0) {
+        ta_set_err(a.status, TA_ERR_TIMEOUT);
+        if (nxt < n_tiles && bulk_tile(nxt)) mbar_wait(&s.bar[cur ^ 1], cur ? phase[0] & 1u : phase[1] & 1u);
+      }
       return;
+    }
+    if (a.W > 1) {  // the same in every thread; the barrier above is behind the counts of the tile before
+      const int w = wt.at(tile * DS_TILE);
+      if (w != w_cnt) {
+        if (a.slot_cnt) flush_counts();
+        w_cnt = w;
+        __syncthreads();
+      }
     }
 #pragma unroll
     for (int j = 0; j < DS_RPT; j++) {
@@ -358,9 +289,10 @@ __global__ void __launch_bounds__(DS_THREADS) k_discover_staged(DiscoverArgs a) 
       const bool in = rl < count;
       const int64_t i = tile * DS_TILE + rl;
       int slot_mine = -1;  // triple slot of a kept record
+      int entry = -1;      // its entry in the CTA's table
       u64 trel = 0;
       if (in) {
-        const u64 *q = reinterpret_cast<const u64 *>(s.buf[cur] + (size_t)rl * 40);
+        const u64 *q = reinterpret_cast<const u64 *>(s.buf[cur] + mis + (size_t)rl * 40);
         Rec r;
         r.ts_start = (i64)q[0];
         r.ts_end = (i64)q[1];
@@ -410,9 +342,16 @@ __global__ void __launch_bounds__(DS_THREADS) k_discover_staged(DiscoverArgs a) 
           const u64 code = triple_code(r.pid, r.kind, r.stream);
           const u32 hsh = hash_code(code);
           trel = (u64)(r.ts_start - ct0);
-          const u64 hit = s.cache[hsh & 255];
-          if ((hit >> 13) == code) {  // a stale miss only costs a probe
+          // the CTA's own table first: an entry or an empty one within a few steps
+          int at = (int)(hsh & (DS_CACHE - 1));
+          u64 hit = s.cache[at];
+          for (int probe = 1; probe < DS_PROBES && (hit >> 13) != code && hit != TRIPLE_EMPTY; probe++) {
+            at = (at + 1) & (DS_CACHE - 1);
+            hit = s.cache[at];
+          }
+          if ((hit >> 13) == code) {
             slot_mine = (int)(hit & (TA_TRIPLE_SLOTS - 1));
+            entry = at;
           } else {
             u32 slot = hsh & (TA_TRIPLE_SLOTS - 1);
             bool done = false;
@@ -426,9 +365,14 @@ __global__ void __launch_bounds__(DS_THREADS) k_discover_staged(DiscoverArgs a) 
               slot = (slot + 1) & (TA_TRIPLE_SLOTS - 1);
             }
             if (!done) ta_set_err(a.status, TA_ERR_TOO_LARGE);
-            s.cache[hsh & 255] = (code << 13) | slot;
             slot_mine = (int)slot;
+            const u64 mine = (code << 13) | slot;
+            if (hit == TRIPLE_EMPTY) {
+              const u64 old = atomicCAS(&s.cache[at], TRIPLE_EMPTY, mine);
+              if (old == TRIPLE_EMPTY || old == mine) entry = at;
+            }
           }
+          if (w != w_cnt) entry = -1;  // counts of another window than the tile's first
           a.prekey[i] = ((u64)slot_mine << PRE_TS_BITS) | trel;
         }
       }
@@ -451,21 +395,24 @@ __global__ void __launch_bounds__(DS_THREADS) k_discover_staged(DiscoverArgs a) 
           }
           if (slot_mine >= 0) atomicAdd(&s.hist[p][d], 1u);
         }
-        // records per triple slot: one add per distinct slot of the warp
+        // records per triple: in the CTA's table (neighbouring records mostly share their triple:
+        // one add for all of them; input in no order at all takes an add each, on chip - adding
+        // to the global counters per distinct triple of a warp took 70 us of 1.2 M shuffled records)
         if (a.slot_cnt) {
-          u32 left = kept;
-          while (left) {
-            const int ld = __ffs(left) - 1;
-            const int sv = __shfl_sync(0xffffffffu, slot_mine, ld);
-            const u32 same = __ballot_sync(0xffffffffu, slot_mine == sv) & left;
-            if (lane == ld) atomicAdd(&a.slot_cnt[sv], (u32)__popc(same));
-            left &= ~same;
+          const int e0 = __shfl_sync(0xffffffffu, entry, leader);
+          if (__all_sync(0xffffffffu, slot_mine < 0 || entry == e0) && e0 >= 0) {
+            if (lane == leader) atomicAdd(&s.count[e0], (u32)__popc(kept));
+          } else if (entry >= 0) {
+            atomicAdd(&s.count[entry], 1u);
+          } else if (slot_mine >= 0) {
+            atomicAdd(&a.slot_cnt[cw * TA_TRIPLE_SLOTS + slot_mine], 1u);  // (cw: the record's window)
           }
         }
       }
     }
     __syncthreads();  // every thread is done with buf[cur] before the next copy into it is issued
   }
+  if (a.slot_cnt) flush_counts();
   for (int i = tid; i < n_tp * 256; i += DS_THREADS) {
     const u32 c = (&s.hist[0][0])[i];
     if (c) atomicAdd(&a.hist[i], c);
@@ -512,7 +459,34 @@ __device__ __forceinline__ void top_hist_add(const TopHistArgs &a, u32 *hist, u6
     atomicAdd(&hist[p * 256 + d], count);
   }
 }
-// several windows: one pass over the words (8 bytes per record)
+// several windows, counted by window and slot: from the counts
+__global__ void __launch_bounds__(256) k_top_hist_counts(TopHistArgs a, const u32 *slot_cnt, const ta_load_summary *sum) {
+  TA_PDL();
+  __shared__ u32 sh[10 * 256];
+  for (int i = threadIdx.x; i < a.plan.n_pass * 256; i += blockDim.x) sh[i] = 0;
+  __syncthreads();
+  const int64_t cells = (int64_t)a.W * TA_TRIPLE_SLOTS;
+  for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 4; i < cells;
+       i += (int64_t)gridDim.x * blockDim.x * 4) {
+    const uint4 q = *reinterpret_cast<const uint4 *>(slot_cnt + i);
+    const u32 c[4] = {q.x, q.y, q.z, q.w};
+    const u64 w = (u64)(i / TA_TRIPLE_SLOTS);
+#pragma unroll
+    for (int j = 0; j < 4; j++)
+      if (c[j])
+        top_hist_add(a, sh, (w << a.tbits) | (u64)a.tt->rank_of_slot[(int)(i + j) & (TA_TRIPLE_SLOTS - 1)], c[j]);
+  }
+  for (int w = blockIdx.x * blockDim.x + threadIdx.x; w < a.W; w += gridDim.x * blockDim.x) {
+    const u32 nd = (u32)(sum[w].n_bad_kind + sum[w].n_bad_interval + sum[w].n_out_of_window);
+    if (!nd) continue;
+    top_hist_add(a, sh, (1ull << (a.wbits + a.tbits)) | ((u64)w << a.tbits), nd);
+    for (int p = 0; p < a.n_time; p++) atomicAdd(&sh[p * 256], nd);  // time digits 0
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < a.plan.n_pass * 256; i += blockDim.x)
+    if (sh[i]) atomicAdd(&a.hist[i], sh[i]);
+}
+// more windows: one pass over the words (8 bytes per record)
 __global__ void __launch_bounds__(256) k_top_hist_words(TopHistArgs a) {
   TA_PDL();
   __shared__ u32 sh[10 * 256];
@@ -734,7 +708,7 @@ __global__ void __launch_bounds__(256) k_load(LoadArgs a) {
     if (sh[i]) atomicAdd(&a.hist[i], sh[i]);
 }
 
-// The same from the words k_discover left in a.keys (rewritten in place): 8 B read + 8 B
+// The same from the words k_discover_staged left in a.keys (rewritten in place): 8 B read + 8 B
 // written per record instead of another pass over the 40-byte records.
 __global__ void __launch_bounds__(256) k_load_pre(LoadArgs a) {
   TA_PDL();
@@ -802,9 +776,6 @@ ta_status ta_launch_discover(ta_window *h) {
     max_win = max_win > h->h_off[w + 1] - h->h_off[w] ? max_win : h->h_off[w + 1] - h->h_off[w];
   }
   const int sbits = ta_bit_len((uint64_t)(max_span - 1));
-  // 16-byte aligned records: plan the time resolution, then the staged pass that also takes
-  // the histograms of the time passes and the per-triple counts
-  const bool staged = h->n > 0 && ((uintptr_t)h->events & 15u) == 0;
   PlanWindows pw;
   memset(&pw, 0, sizeof(pw));
   if (h->W <= TA_PLAN_WINDOWS) {
@@ -814,27 +785,25 @@ ta_status ta_launch_discover(ta_window *h) {
     memcpy(pw.v + 2 * h->W + 1, h->h_t1.data(), (size_t)h->W * 8);
   }
   ta_launch(k_plan, 1, PL_THREADS, 0, h->stream, h->events, h->n, h->d_off, h->d_t0, h->d_t1, h->W, sbits, max_span,
-            max_win, h->d_misc, pw, staged ? 1 : 0);
+            max_win, h->d_misc, pw);
   if (h->n > 0) {
-    if (staged) {
-      DiscoverArgs a;
-      a.ev = h->events; a.n = h->n; a.off = h->d_off; a.t0 = h->d_t0; a.t1 = h->d_t1; a.W = h->W;
-      a.tt = h->d_triples; a.cm = h->d_comms; a.sum = h->d_load_sum; a.misc = h->d_misc;
-      a.status = h->d_status; a.prekey = h->d_keys; a.hist = h->d_hist;
-      a.slot_cnt = h->W == 1 ? h->d_slot_cnt : nullptr;
-      a.sbits = sbits; a.ibits = 0;
-      TA_CHECK_CUDA(h, cudaFuncSetAttribute(k_discover_staged, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                            (int)sizeof(DiscoverSmem)));
-      const int64_t tiles = (h->n + DS_TILE - 1) / DS_TILE;
+    // plan the time resolution (above), then the pass over the records, which also takes the histograms of
+    // the time passes and counts the records per triple
+    DiscoverArgs a;
+    a.ev = h->events; a.n = h->n; a.off = h->d_off; a.t0 = h->d_t0; a.t1 = h->d_t1; a.W = h->W;
+    a.tt = h->d_triples; a.cm = h->d_comms; a.sum = h->d_load_sum; a.misc = h->d_misc;
+    a.status = h->d_status; a.prekey = h->d_keys; a.hist = h->d_hist;
+    a.slot_cnt = h->cnt_windows ? h->d_slot_cnt : nullptr;
+    a.sbits = sbits; a.ibits = 0;
+    TA_CHECK_CUDA(h, cudaFuncSetAttribute(k_discover_staged, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          (int)sizeof(DiscoverSmem)));
+    const int64_t tiles = (h->n + DS_TILE - 1) / DS_TILE;
 #ifndef DS_CTAS_PER_SM
 #define DS_CTAS_PER_SM 4
 #endif
-      const int grid = (int)(tiles < 148 * DS_CTAS_PER_SM ? tiles : 148 * DS_CTAS_PER_SM);
-      ta_launch(k_discover_staged, grid, DS_THREADS, sizeof(DiscoverSmem), h->stream, a);
-      h->tkeep = -1;  // read back with the other results of the pass
-    } else {
-      ta_launch(k_discover, grid_for(h->n, 256, 8), 256, 0, h->stream, h->events, h->n, h->d_off, h->d_t0, h->d_t1, h->W, h->d_triples, h->d_comms, h->d_load_sum, h->d_misc, h->d_status, h->d_keys);
-    }
+    const int grid = (int)(tiles < 148 * DS_CTAS_PER_SM ? tiles : 148 * DS_CTAS_PER_SM);
+    ta_launch(k_discover_staged, grid, DS_THREADS, sizeof(DiscoverSmem), h->stream, a);
+    h->tkeep = -1;  // read back with the other results of the pass
     h->prekeys = 1;
   }
   TA_CHECK_CUDA(h, cudaFuncSetAttribute(k_rank, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -899,7 +868,11 @@ ta_status ta_launch_load(ta_window *h, bool allow_packed) {
       a.plan = h->plan; a.n_time = tp.n_pass; a.top_lo = h->ibits + T;
       a.tbits = h->tbits; a.wbits = h->wbits; a.tt = h->d_triples; a.hist = h->d_hist;
       a.prekey = h->d_keys; a.n = h->n; a.off = h->d_off; a.W = h->W;
-      ta_launch(k_top_hist_words, grid_for(h->n, 256, 8), 256, 0, h->stream, a);
+      // (512 windows of 65 k records: 211 us from the words)
+      if (h->cnt_windows)
+        ta_launch(k_top_hist_counts, grid_for((int64_t)h->W * TA_TRIPLE_SLOTS, 1024, 4), 256, 0, h->stream, a,
+                  h->d_slot_cnt, h->d_load_sum);
+      else ta_launch(k_top_hist_words, grid_for(h->n, 256, 8), 256, 0, h->stream, a);
       TA_CHECK_CUDA(h, cudaGetLastError());
       return TA_OK;  // the words stay in d_keys (h->prekeys stays set): a retry can still use them
     }

@@ -455,12 +455,15 @@ static ta_status load_impl(ta_window *h, const ta_event *events, int32_t on_devi
   const size_t up_words = (size_t)(W + 1) + 2 * (size_t)W + 16;
   // the pool: results and counters of the later calls (34 bytes per record), tile descriptors,
   // lane tables and a few aggregate tables
+  // records per window and triple slot, as long as a window's counters (32 KB) are small beside its words
+  h->cnt_windows = W == 1 || (W <= 1024 && n / W >= 8192) ? W : 0;
+  const size_t cnt_bytes = (size_t)(h->cnt_windows ? h->cnt_windows : 1) * TA_TRIPLE_SLOTS * 4;
   h->zero_used = 0;
   h->zero_bytes = n <= TA_ZERO_POOL_RECORDS ? Carver::pad((size_t)n * 36 + (2u << 20)) : 0;
   size_t bytes = Carver::pad(up_words * 8) + Carver::pad(ST_WORDS * 4) +
                  Carver::pad(sizeof(TripleTable)) + Carver::pad(sizeof(CommTable)) +
                  Carver::pad(W * sizeof(ta_load_summary)) + Carver::pad(10 * 256 * 4) +
-                 Carver::pad(TA_TRIPLE_SLOTS * 4) + h->zero_bytes + 256;
+                 Carver::pad(cnt_bytes) + h->zero_bytes + 256;
   void *b = ta_dalloc(h, bytes);
   if (!b) return TA_ERR_OOM;
   Carver c(b);
@@ -475,7 +478,7 @@ static ta_status load_impl(ta_window *h, const ta_event *events, int32_t on_devi
   h->d_status = c.take<int32_t>(ST_WORDS);
   h->d_load_sum = c.take<ta_load_summary>(W);
   h->d_hist = c.take<u32>(10 * 256);
-  h->d_slot_cnt = c.take<u32>(TA_TRIPLE_SLOTS);
+  h->d_slot_cnt = c.take<u32>(cnt_bytes / 4);
   h->zero_pool = c.take<char>(h->zero_bytes);
   h->d_comms = c.take<CommTable>(1);
   char *zero_end = (char *)h->d_comms + sizeof(h->d_comms->slots);

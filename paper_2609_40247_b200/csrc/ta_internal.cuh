@@ -142,7 +142,8 @@ struct ta_window {
   int packed, dshift, ibits;   // packed keys: low ibits = index inside the window, dshift low time bits dropped
   int tkeep;                   // time bits the planning kernel decided to keep (0 = it did not run)
   int fast_keys;               // the first radix pass builds the keys from the discovery words itself
-  u32 *d_slot_cnt;             // kept records per triple slot (one window only), or null
+  u32 *d_slot_cnt;             // kept records per (window, triple slot) of the first cnt_windows windows
+  int cnt_windows;             // W, or 0 when there are too many windows to count by window and slot
   int64_t min_name, max_name, max_dur;
   SortPlan plan;
   TopHist top;

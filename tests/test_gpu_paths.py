@@ -87,3 +87,43 @@ def test_pageable_records_around_the_threshold_of_the_staged_upload(n):
     a = run_gpu(ev, off, wl.win_t0, wl.win_t1, on_device=True)
     for _ in range(2):
         assert_same(a, run_gpu(ev, off, wl.win_t0, wl.win_t1, on_device=False))
+
+
+@pytest.mark.parametrize("scale,gap", [(0.02, 4_990_000), (0.12, 4_990_000)])
+def test_critical_path_with_a_short_and_a_long_list_of_waits(scale, gap):
+    """Prefill windows wait once per step: some three thousand waits (walked by one CTA) and some
+    twenty thousand (pointer doubling over many)."""
+    wl = synth.make_workload("c2", scale, truth=False)
+    both(wl.events, wl.win_off, wl.win_t0, wl.win_t1, min_gap=gap)
+    assert ((wl.events["kind"] == 1).sum() > 16_384) == (scale > 0.1)
+
+
+@pytest.mark.parametrize("windows,per", [(2, 20_000), (9, 38_460), (40, 20_000)])
+def test_many_windows_counted_by_window_and_lane(windows, per):
+    """Batches whose lane histograms come from counts per window and lane, some records dropped."""
+    wl = synth.make_workload("c4", per * 512 / (1 << 28), truth=False, n_windows=windows)
+    ev = wl.events.copy()
+    ev["kind"][::97] = 8
+    assert len(ev) // windows >= 8192
+    both(ev, wl.win_off, wl.win_t0, wl.win_t1, comm_sizes=wl.comm_sizes)
+
+
+@pytest.mark.parametrize("n", [1, 511, 512, 513, 1023, 1024, 1025, 1536, 60_001])
+def test_records_at_an_odd_eight_bytes(n, monkeypatch):
+    """A device buffer that begins at eight bytes past a multiple of sixteen, around the size of the
+    tiles that are copied in bulk."""
+    import torch
+    from paper_2609_40247_b200 import ta
+
+    class Shifted(ta.Window):
+        def __init__(self, events, *args, **kw):
+            room = torch.zeros(events.numel() + 40, dtype=torch.uint8, device="cuda")
+            room[8:8 + events.numel()] = events
+            assert room.data_ptr() % 16 == 0
+            super().__init__(room[8:8 + events.numel()], *args, **kw)
+
+    monkeypatch.setattr(ta, "Window", Shifted)
+    wl = synth.make_workload("c3", 0.002, truth=False)
+    ev = np.ascontiguousarray(wl.events[:n])
+    assert len(ev) == n
+    both(ev, [0, n], wl.win_t0, wl.win_t1, comm_sizes=wl.comm_sizes)
