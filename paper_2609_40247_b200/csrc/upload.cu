@@ -2,7 +2,10 @@
 // or read by the caller, a numpy array) the driver copies through a staging buffer of its own with one
 // thread, at 11 to 20 GB/s; here several threads copy pieces into a ring of page-locked buffers, each
 // of which is on its way to the device as soon as it is full.  Bound by the host's memory
-// bandwidth or the link (55 GB/s), whichever is less.
+// bandwidth or the link (52 GB/s), whichever is less: 42 MB take 3.9 ms through the driver, 2.0 ms
+// with memcpy into the buffers, 1.06 ms with streaming stores (0.77 from page-locked memory).
+#include <emmintrin.h>
+
 #include <algorithm>
 #include <cstring>
 #include <mutex>
@@ -12,7 +15,7 @@
 
 #define UP_PIECE (1u << 20)
 #define UP_PIECES 24
-#define UP_THREADS 8
+#define UP_THREADS 6
 #define UP_MIN (4u << 20)  // below this the threads cost more than they save
 
 namespace {
@@ -65,14 +68,30 @@ Ring *ring_take(int device) {
 }
 }  // namespace
 
-// Rings no upload has asked for during the lifetime of the last two handles are given back.
+// Copies a piece past the caches: the device then reads it from memory.  Lines that are still dirty in
+// some core's cache have to be snooped out of it one by one, which held the link at half its rate.
+static void copy_piece(unsigned char *dst /* 64-byte aligned */, const unsigned char *src, size_t len) {
+  size_t i = 0;
+  for (; i + 64 <= len; i += 64) {
+    const __m128i a = _mm_loadu_si128((const __m128i *)(src + i)), b = _mm_loadu_si128((const __m128i *)(src + i + 16));
+    const __m128i c = _mm_loadu_si128((const __m128i *)(src + i + 32)), d = _mm_loadu_si128((const __m128i *)(src + i + 48));
+    _mm_stream_si128((__m128i *)(dst + i), a);
+    _mm_stream_si128((__m128i *)(dst + i + 16), b);
+    _mm_stream_si128((__m128i *)(dst + i + 32), c);
+    _mm_stream_si128((__m128i *)(dst + i + 48), d);
+  }
+  if (i < len) memcpy(dst + i, src + i, len - i);
+  _mm_sfence();
+}
+
+// Rings no upload has asked for during the lifetime of the last 64 handles are given back.
 void ta_upload_age() {
   std::vector<Ring *> out;
   {
     std::lock_guard<std::mutex> lock(g_ring_guard);
     g_handles++;
     for (size_t i = 0; i < g_rings.size();)
-      if (g_rings[i]->last_used + 2 < g_handles) {
+      if (g_rings[i]->last_used + 64 < g_handles) {
         out.push_back(g_rings[i]);
         g_rings.erase(g_rings.begin() + i);
       } else {
@@ -111,7 +130,7 @@ ta_status ta_upload(ta_window *h, void *dst, const void *src, size_t bytes) {
       if ((c >= UP_PIECES || r->used[b]) && cudaEventSynchronize(r->ev[b]) != cudaSuccess) { failed.store(1); return; }
       const size_t off = c * (size_t)UP_PIECE, len = std::min((size_t)UP_PIECE, bytes - off);
       unsigned char *buf = r->buf + (size_t)b * UP_PIECE;
-      memcpy(buf, (const unsigned char *)src + off, len);
+      copy_piece(buf, (const unsigned char *)src + off, len);
       if (cudaMemcpyAsync((unsigned char *)dst + off, buf, len, cudaMemcpyHostToDevice, h->stream) != cudaSuccess ||
           cudaEventRecord(r->ev[b], h->stream) != cudaSuccess) {
         failed.store(1);
