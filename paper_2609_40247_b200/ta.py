@@ -329,30 +329,36 @@ class _Handle:
             pass
 
 
-class _DevView:
-    """Exposes a raw device range to torch through __cuda_array_interface__."""
+def _views():
+    """(wrap, part) of csrc/views.cpp; like the library it has to be built."""
+    global _wrap, _part
+    if _part is None:
+        import torch  # noqa: F401  (its libraries have to be there first)
+        try:
+            from . import _views as native
+        except ImportError as e:
+            raise RuntimeError("_views.so is missing or was built against another torch: build it with "
+                               "`python -m paper_2609_40247_b200.build`") from e
+        _wrap, _part = native.wrap, native.part
+    return _wrap, _part
 
-    def __init__(self, ptr, nbytes, owner):
-        self.owner = owner
-        self.__cuda_array_interface__ = {"shape": (nbytes,), "typestr": "|u1",
-                                         "data": (int(ptr), False), "version": 2}
+
+_wrap = _part = None
 
 
 class _Blocks:
-    """Tensors over the allocations of a handle; results are slices of them (making a tensor from
-    an address takes three times as long as slicing one)."""
+    """Tensors over the allocations of a handle; the columns are parts of them."""
 
     def __init__(self, handle):
         self.handle = handle
         self.known = []  # (first address, address behind, tensor)
         self.last = (0, 0, None)
 
-    def slice(self, ptr, nbytes):
+    def part(self, ptr, nbytes):
         for self.last in self.known:
             lo, hi, t = self.last
             if lo <= ptr and ptr + nbytes <= hi:
-                return t[ptr - lo:ptr - lo + nbytes]
-        import torch
+                return _part(t, ptr - lo, nbytes)
         h = self.handle
         if h.block is not None and h.block <= ptr < h.block + h.block_bytes:
             lo, size = h.block, h.block_bytes
@@ -361,10 +367,10 @@ class _Blocks:
             if h.lib.ta_block_of(h.ptr, ptr, ctypes.byref(base), ctypes.byref(room)) != 0:
                 raise ValueError("not a result of an open window")
             lo, size = base.value, room.value
-        t = torch.as_tensor(_DevView(lo, size, h), device=f"cuda:{h.device}")
-        self.last = (lo, lo + size, t)
+        wrap, part = _views()
+        self.last = (lo, lo + size, wrap(lo, size, h.device, h))
         self.known.append(self.last)
-        return t[ptr - lo:ptr - lo + nbytes]
+        return part(self.last[2], ptr - lo, nbytes)
 
 
 class _Result:
@@ -395,8 +401,8 @@ class _Result:
             return torch.empty(0, dtype=torch.uint8, device=f"cuda:{self._handle.device}")
         lo, hi, t = self._blocks.last
         if lo <= ptr and ptr + nbytes <= hi:
-            return t[ptr - lo:ptr - lo + nbytes]
-        return self._blocks.slice(ptr, nbytes)
+            return _part(t, ptr - lo, nbytes)
+        return self._blocks.part(ptr, nbytes)
 
     # Tables are mostly read together: a request for one brings the other small ones of the result
     # along (a round trip costs more than their bytes), up to these limits.
