@@ -5,9 +5,8 @@
 //
 // In canonical order (ts_start ascending, ts_end descending) a properly nested
 // host lane has a simple structure: the innermost encloser of record i is the
-// nearest earlier OP that is still running when i starts.  Tiles of 2048
-// records (256 threads x 8 consecutive records), three kernels, no kernel ever
-// waits for another CTA:
+// nearest earlier OP that is still running when i starts.  Tiles of 1024 records
+// (256 of a small window), no kernel ever waits for another CTA:
 //   k_attr_agg     per tile, the stack of OPs that are still undominated at the
 //                  tile's end (at most TA_MAX_DEPTH + 1 entries when nesting is
 //                  legal);
@@ -16,10 +15,8 @@
 //                  later tile's outermost surviving OP are dropped; a tile whose
 //                  last lane starts inside it cuts off what came before), as a
 //                  fan-out-32 tree, leaves every tile the stack open at its start;
-//   k_attr_resolve per record: a backward look over the thread's own records,
-//                  else one descent of a max-tree over the threads' largest OP
-//                  end times in shared memory, else the carried stack.  The kernels of
-//                  every operator are added up on the way, from the launches inside it,
+//   k_attr_resolve parent and level of every record, 32 at a time.  The kernels of every
+//                  operator are added up on the way, from the launches inside it,
 //                  and all columns of the operator are written once, with the zeros of
 //                  all other rows;
 //   k_attr_spill   what a tile owes to operators of earlier tiles is added to their rows.
@@ -35,23 +32,15 @@
 #include "ta_internal.cuh"
 
 #define AT_THREADS 256
-// 4 or 8 records per thread in the stack and resolve kernels: with four the resolve kernel fits
-// 64 registers and 16 KB of shared memory, four CTAs per SM (eight and three: 0.12 ms slower)
-#ifndef AT_ITEMS
-#define AT_ITEMS 4
-#endif
-#define AT_TILE (AT_THREADS * AT_ITEMS)
 #define AT_CAP 16
-#ifndef AT_RES_MINB
-#define AT_RES_MINB 4
+#ifndef AS_MINB
+#define AS_MINB 4
 #endif
 // k_attr_ops: four records per thread keep it at 64 registers, four CTAs per SM (eight records and
 // three CTAs measured 0.12 ms slower on the 66.8 M record window: the kernel waits on gathers)
 #ifndef AT_OPS_MINB
 #define AT_OPS_MINB 4
 #endif
-#define AT_NONE (-1)
-#define AT_UNRESOLVED (-2)
 
 struct AttrArgs {
   int64_t n, n_valid;
@@ -59,7 +48,7 @@ struct AttrArgs {
   int64_t n_tiles;
   const int16_t *kind;
   const int64_t *ts, *te;
-  const int32_t *lane_off, *lane_window, *lane_dom_end;
+  const int32_t *lane_off, *lane_window, *lane_dom_end, *lane_dom_next;
   const int16_t *lane_domain;
   int32_t *parent;
   uint8_t *depth;
@@ -115,8 +104,10 @@ __device__ __forceinline__ void wstack_combine(const WStack &ear, WStack &acc, b
 
 
 // ---- kernel 1: the stack each tile leaves behind --------------------------------
+template <int ITEMS>  // records per thread
 __global__ void __launch_bounds__(AT_THREADS) k_attr_agg(AttrArgs a) {
   TA_PDL();
+  constexpr int TILE = AT_THREADS * ITEMS;
   __shared__ i64 wmax[AT_THREADS / 32];
   __shared__ i64 s_e[AT_CAP];
   __shared__ int32_t s_pos[AT_CAP];
@@ -124,17 +115,17 @@ __global__ void __launch_bounds__(AT_THREADS) k_attr_agg(AttrArgs a) {
   if (ta_failed(a.status)) return;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int tile = blockIdx.x;
-  const int64_t tile_start = (int64_t)tile * AT_TILE;
-  const int64_t p0 = tile_start + (int64_t)tid * AT_ITEMS;
-  const int64_t plast = min(tile_start + AT_TILE, a.n_valid) - 1;
+  const int64_t tile_start = (int64_t)tile * TILE;
+  const int64_t p0 = tile_start + (int64_t)tid * ITEMS;
+  const int64_t plast = min(tile_start + TILE, a.n_valid) - 1;
   if (tid == 0) s_raw = 0;
   if (warp == 0) {
     int l = -1;
     if (plast >= tile_start) l = tile_lane_search(a.lane_off, a.n_lanes, plast);
     if (lane == 0) s_lane1 = l;
   }
-  int16_t kd[AT_ITEMS];
-  loadn_i16<AT_ITEMS>(a.kind, p0, a.n, 9, kd);
+  int16_t kd[ITEMS];
+  loadn_i16<ITEMS>(a.kind, p0, a.n, 9, kd);
   __syncthreads();
   const int lane1 = s_lane1;
   if (lane1 < 0 || a.lane_domain[lane1] != 0) {
@@ -144,17 +135,17 @@ __global__ void __launch_bounds__(AT_THREADS) k_attr_agg(AttrArgs a) {
   const int64_t seg_begin = a.lane_off[lane1];  // first record of the tile's last lane
   unsigned opmask = 0;
 #pragma unroll
-  for (int j = 0; j < AT_ITEMS; j++)
+  for (int j = 0; j < ITEMS; j++)
     if (kd[j] == TA_KIND_OP && p0 + j <= plast && p0 + j >= seg_begin) opmask |= 1u << j;
-  i64 en[AT_ITEMS];
+  i64 en[ITEMS];
 #pragma unroll
-  for (int j = 0; j < AT_ITEMS; j++) en[j] = INT64_MIN;
+  for (int j = 0; j < ITEMS; j++) en[j] = INT64_MIN;
   i64 m8 = INT64_MIN;
   if (opmask) {
-    i64 t[AT_ITEMS];
-    loadn_i64<AT_ITEMS>(a.te, p0, a.n, t);
+    i64 t[ITEMS];
+    loadn_i64<ITEMS>(a.te, p0, a.n, t);
 #pragma unroll
-    for (int j = 0; j < AT_ITEMS; j++)
+    for (int j = 0; j < ITEMS; j++)
       if (opmask & (1u << j)) { en[j] = t[j]; m8 = m8 > t[j] ? m8 : t[j]; }
   }
   // largest OP end among the threads after this one
@@ -174,7 +165,7 @@ __global__ void __launch_bounds__(AT_THREADS) k_attr_agg(AttrArgs a) {
   }
   i64 sfx = after;
 #pragma unroll
-  for (int j = AT_ITEMS - 1; j >= 0; j--) {
+  for (int j = ITEMS - 1; j >= 0; j--) {
     if (opmask & (1u << j)) {
       if (en[j] >= sfx) {  // equal ends nest: the earlier OP encloses the later one
         int o = atomicAdd(&s_raw, 1);
@@ -328,376 +319,257 @@ __global__ void __launch_bounds__(128) k_attr_fold_down(StackArr child, int64_t 
   if (overflow && lane == 0) ta_set_err(status, TA_ERR_DEPTH);
 }
 
-// ---- kernel 3: parent and depth of every host record -----------------------------
-// a thread's eight leaves are followed by one pad entry: the threads of a warp then touch
-// distinct banks when each walks its own records
-#define AT_LX(x) ((x) + ((x) >> 3))
-struct __align__(16) AttrSmem {
-  i64 leaf[AT_TILE + AT_TILE / 8];  // OP end time, INT64_MIN elsewhere; index through AT_LX
-  i64 T[2 * AT_THREADS];          // max-tree over the threads' maxima, leaves at [AT_THREADS, 2*AT_THREADS)
-  int16_t parent_local[AT_TILE];
-  uint8_t kcarry[AT_TILE];
-  i64 carry_e[AT_CAP];
-  int32_t carry_pos[AT_CAP];
-  // kernels of the operators: one row per record of the tile, then one per carried operator
-  i64 k_first[AT_TILE + AT_CAP], k_last[AT_TILE + AT_CAP];
-  u64 k_ns[AT_TILE + AT_CAP];
-  int32_t k_cnt[AT_TILE + AT_CAP];  // bit 31: more may be added by other CTAs (the row keeps its identities)
-  int lane0, lane1, dmax;
+// ---- kernel 3: parent and depth of every host record, kernels of every operator ---------
+// A warp takes a tile row by row, 32 records of ONE lane per row and one record per thread, and keeps
+// the stack of operators open in front of the row in shared memory.  The innermost operator around a
+// record is the nearest one in front of it that ends at or after the record's threshold: every thread
+// starts from the operator just in front of its record and, while that has ended, jumps to that
+// operator's own candidate (what lies between an operator and its candidate has ended for the
+// operator, so also for whoever jumps over it); all 32 move at the same time, so a row takes the
+// logarithm of its nesting in rounds of three shuffles.  What a row does not answer, the stack does.
+// The kernels of the launches are added up on the way: an operator owns those of the launches
+// directly inside it, so every one arrives while its operator is in the row or on the stack.
+// (Four consecutive records per thread, each searched by a walk over a max-tree in shared memory and
+// added to shared-memory rows by 64-bit atomics, took 660 warp instructions per 32 records, 1.33 ms
+// of 66.8 M records; three atomics per kernel in memory, before that, 1.2 ms more.)
+#define AS_LEVELS 64   // open operators a warp keeps; more than TA_MAX_DEPTH is an error anyway
+#define AS_WARPS 8
+#define AS_MORE 0x80000000u
+struct AttrStack {
+  i64 e[AS_LEVELS];      // end times, none above is greater than one below
+  i64 first[AS_LEVELS], last[AS_LEVELS];
+  u64 ns[AS_LEVELS];
+  int32_t pos[AS_LEVELS];
+  u32 cnt[AS_LEVELS];    // kernels; bit 31: k_attr_ops may add more, the row keeps its identities
 };
-#define AT_MORE 0x80000000u
-// adds a run of kernels to an operator's row
-__device__ __forceinline__ void attr_add(AttrSmem &s, int row, int cnt, i64 first, i64 last, u64 ns) {
-  atomicAdd(&s.k_cnt[row], cnt);
-  atomicAdd(&s.k_ns[row], ns);
-  if (first < s.k_first[row]) atomicMin(&s.k_first[row], first);
-  if (last > s.k_last[row]) atomicMax(&s.k_last[row], last);
-}
-// the four columns of the thread's records
-template <bool ZERO>
-__device__ __forceinline__ void attr_store_ops(const AttrArgs &a, const AttrSmem &s, int64_t p0, int x0) {
-  int32_t c[AT_ITEMS];
-  i64 f[AT_ITEMS], l[AT_ITEMS], ns[AT_ITEMS];
-#pragma unroll
-  for (int j = 0; j < AT_ITEMS; j++) {
-    c[j] = 0;
-    f[j] = l[j] = ns[j] = 0;
-    if (ZERO) continue;
-    const u32 cnt = (u32)s.k_cnt[x0 + j];
-    c[j] = (int32_t)(cnt & ~AT_MORE);
-    if (cnt) {
-      f[j] = s.k_first[x0 + j];
-      l[j] = s.k_last[x0 + j];
-      ns[j] = (i64)s.k_ns[x0 + j];
-    }
-  }
-  storen_i32<AT_ITEMS>(a.op_n, p0, a.n, c);
-  storen_i64<AT_ITEMS>((int64_t *)a.op_first, p0, a.n, f);
-  storen_i64<AT_ITEMS>((int64_t *)a.op_last, p0, a.n, l);
-  storen_i64<AT_ITEMS>((int64_t *)a.op_ns, p0, a.n, ns);
-}
+__device__ __forceinline__ i64 shfl_i64(i64 v, int src) { return __shfl_sync(0xffffffffu, v, src); }
 
-__global__ void __launch_bounds__(AT_THREADS, AT_RES_MINB) k_attr_resolve(AttrArgs a) {
-  TA_PDL();
-  __shared__ AttrSmem s;
-  if (ta_failed(a.status)) return;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int tile = blockIdx.x;
-  const int64_t tile_start = (int64_t)tile * AT_TILE;
-  const int x0 = tid * AT_ITEMS;
-  const int64_t p0 = tile_start + x0;
-  const bool full = p0 + AT_ITEMS <= a.n;
-  if (tid == 0) { s.lane1 = -1; s.dmax = 0; s.lane0 = -1; }
-  __syncthreads();
-  if (warp == 0 && tile_start < a.n_valid && a.n_lanes > 0) {
-    int l = tile_lane_search(a.lane_off, a.n_lanes, tile_start);
-    if (lane == 0) s.lane0 = l;
+// rows of positions without a host record
+__device__ __forceinline__ void attr_fill(const AttrArgs &a, int64_t from, int64_t to) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll 2
+  for (int64_t p = from + lane; p < to; p += 32) {
+    a.parent[p] = -1;
+    a.depth[p] = 0;
+    a.op_n[p] = 0;
+    a.op_first[p] = 0;
+    a.op_last[p] = 0;
+    a.op_ns[p] = 0;
   }
-  const int ccnt = a.carry_cnt[tile];
-  if (tid < ccnt) {
-    s.carry_e[tid] = a.carry_e[(size_t)tile * AT_CAP + tid];
-    s.carry_pos[tid] = a.carry_pos[(size_t)tile * AT_CAP + tid];
-  }
-  __syncthreads();
-  const int l0 = s.lane0;
-  // A tile of device lanes holds no host record: parent -1, depth 0 throughout, nothing read.
-  if (l0 < 0 || span_outside_domain(a.lane_domain, a.lane_dom_end, l0, min(tile_start + AT_TILE, a.n_valid), 0)) {
-    if (full) {
-#pragma unroll
-      for (int q = 0; q < AT_ITEMS / 4; q++) {
-        *reinterpret_cast<int4 *>(a.parent + p0 + 4 * q) = make_int4(-1, -1, -1, -1);
-        *reinterpret_cast<u32 *>(a.depth + p0 + 4 * q) = 0u;
-      }
-    } else {
-      for (int j = 0; j < AT_ITEMS; j++)
-        if (p0 + j < a.n) { a.parent[p0 + j] = -1; a.depth[p0 + j] = 0; }
+}
+// levels [from, to) leave the stack: what they own is written, or noted for the rows of earlier tiles
+// (the lowest `carried` levels).  open: later tiles may add to them.
+__device__ __forceinline__ void attr_pop(const AttrArgs &a, const AttrStack &st, int from, int to, int carried, bool open) {
+  const int lane = threadIdx.x & 31;
+  for (int k = from + lane; k < to; k += 32) {
+    const u32 c = st.cnt[k];
+    const int32_t r = st.pos[k];
+    if (k < carried) {
+      if (c & ~AS_MORE)
+        a.spill[atomicAdd(a.n_spill, 1u)] = AttrSpill{r, (int32_t)(c & ~AS_MORE), st.first[k], st.last[k], (i64)st.ns[k]};
+    } else if (c || open) {
+      a.op_n[r] = (int32_t)(c & ~AS_MORE);
+      a.op_first[r] = st.first[k];
+      a.op_last[r] = st.last[k];
+      a.op_ns[r] = (i64)st.ns[k];
     }
-    attr_store_ops<true>(a, s, p0, x0);
-    return;
-  }
-  for (int i = tid; i < AT_TILE + AT_CAP; i += AT_THREADS) {
-    s.k_first[i] = INT64_MAX;
-    s.k_last[i] = INT64_MIN;
-    s.k_ns[i] = 0;
-    s.k_cnt[i] = 0;
-  }
-  // operators still open at the tile's end: later tiles may add to their rows
-  const int open_cnt = a.agg_meta[tile] & 0xFF;
-  const int open_pos = tid < open_cnt ? (int)(a.agg_pos[(size_t)tile * AT_CAP + tid] - tile_start) : -1;
-  // kinds and both times of the thread's records are requested together (the tile holds a host
-  // lane, so nearly every record needs its times)
-  int16_t kd[AT_ITEMS];
-  i64 st[AT_ITEMS], en[AT_ITEMS];
-  loadn_i16<AT_ITEMS>(a.kind, p0, a.n, 9, kd);
-  loadn_i64<AT_ITEMS>(a.ts, p0, a.n, st);
-  loadn_i64<AT_ITEMS>(a.te, p0, a.n, en);
-  int32_t nk[AT_ITEMS];  // kernels of the thread's launches (0 elsewhere)
-  int32_t kp[AT_ITEMS];  // the kernel of those that have exactly one
-  if (full) {
-#pragma unroll
-    for (int q = 0; q < AT_ITEMS / 4; q++) {
-      const int4 x = *reinterpret_cast<const int4 *>(a.kol + p0 + 4 * q);
-      const int4 y = *reinterpret_cast<const int4 *>(a.kernel_of + p0 + 4 * q);
-      nk[4 * q] = x.x; nk[4 * q + 1] = x.y; nk[4 * q + 2] = x.z; nk[4 * q + 3] = x.w;
-      kp[4 * q] = y.x; kp[4 * q + 1] = y.y; kp[4 * q + 2] = y.z; kp[4 * q + 3] = y.w;
-    }
-  } else {
-#pragma unroll
-    for (int j = 0; j < AT_ITEMS; j++) {
-      nk[j] = p0 + j < a.n ? a.kol[p0 + j] : 0;
-      kp[j] = p0 + j < a.n ? a.kernel_of[p0 + j] : 0;
-    }
-  }
-  unsigned hostmask = 0;
-#pragma unroll
-  for (int j = 0; j < AT_ITEMS; j++)
-    if (p0 + j < a.n_valid && kd[j] <= TA_KIND_LAUNCH) hostmask |= 1u << j;
-  // lanes, leaves, the thread's maximum
-  int ln[AT_ITEMS];
-  int lo_local[AT_ITEMS];  // first tile-local index of the record's lane (-1: the lane began earlier)
-  i64 m8 = INT64_MIN;
-  unsigned opmask = 0;  // the thread's own OP records (its leaves are their en[])
-  {
-    int l = l0;
-    int64_t next_off = l >= 0 ? (int64_t)a.lane_off[l + 1] : LLONG_MAX;
-    int64_t cur_off = l >= 0 ? (int64_t)a.lane_off[l] : 0;
-#pragma unroll
-    for (int j = 0; j < AT_ITEMS; j++) {
-      const int64_t p = p0 + j;
-      ln[j] = -1;
-      lo_local[j] = 0;
-      i64 leaf = INT64_MIN;
-      if (hostmask & (1u << j)) {
-        while (p >= next_off) { l++; cur_off = next_off; next_off = a.lane_off[l + 1]; }
-        ln[j] = l;
-        lo_local[j] = cur_off < tile_start ? -1 : (int)(cur_off - tile_start);
-        if (kd[j] == TA_KIND_OP) { leaf = en[j]; opmask |= 1u << j; }
-      }
-      s.leaf[AT_LX(x0 + j)] = leaf;
-      m8 = leaf > m8 ? leaf : m8;
-    }
-    const int64_t plast = min(tile_start + AT_TILE, a.n_valid) - 1;
-    if (plast >= p0 && plast < p0 + AT_ITEMS) {
-      while (plast >= next_off) { l++; next_off = a.lane_off[l + 1]; }
-      s.lane1 = l;
-    }
-  }
-  s.T[AT_THREADS + tid] = m8;
-  // the times of those kernels: consecutive launches have consecutive kernels of a few streams, so the
-  // gathers of a warp mostly share their sectors
-  i64 ks[AT_ITEMS], ke[AT_ITEMS];
-#pragma unroll
-  for (int j = 0; j < AT_ITEMS; j++) {
-    ks[j] = ke[j] = 0;
-    if (!(hostmask & (1u << j)) || kd[j] != TA_KIND_LAUNCH) nk[j] = 0;
-    if (nk[j] == 1) { ks[j] = a.ts[kp[j]]; ke[j] = a.te[kp[j]]; }
   }
   __syncwarp();
-  // tree levels inside the warp's subtree: 16, 8, 4, 2, 1 nodes
-#pragma unroll
-  for (int lv = 4; lv >= 0; lv--) {
-    const int cntl = 1 << lv;
-    const int base = (AT_THREADS >> (5 - lv)) + warp * cntl;  // first node of this warp on the level
-    if (lane < cntl) {
-      const int i = base + lane;
-      i64 x = s.T[2 * i], y = s.T[2 * i + 1];
-      s.T[i] = x > y ? x : y;
+}
+
+template <int TILE>
+__global__ void __launch_bounds__(AS_WARPS * 32, AS_MINB) k_attr_resolve(AttrArgs a) {
+  TA_PDL();
+  __shared__ AttrStack s_stack[AS_WARPS];
+  if (ta_failed(a.status)) return;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const u32 lt = (1u << lane) - 1u;
+  const int64_t tile = (int64_t)blockIdx.x * AS_WARPS + warp;
+  if (tile >= a.n_tiles) return;
+  AttrStack &st = s_stack[warp];
+  const int64_t tile_start = tile * TILE, tile_end = min(tile_start + TILE, a.n), vend = min(tile_end, a.n_valid);
+  if (tile_start >= vend) {
+    attr_fill(a, tile_start, tile_end);
+    return;
+  }
+  int l = tile_lane_search(a.lane_off, a.n_lanes, tile_start);
+  int64_t pos = tile_start;
+  int depth = 0, carried = 0;  // levels on the stack; of these, the lowest ones come from earlier tiles
+  if (a.lane_domain[l] == 0 && (int64_t)a.lane_off[l] < tile_start) {
+    depth = carried = a.carry_cnt[tile];
+    if (lane < depth) {
+      st.e[lane] = a.carry_e[(size_t)tile * AT_CAP + lane];
+      st.pos[lane] = a.carry_pos[(size_t)tile * AT_CAP + lane];
+      st.first[lane] = INT64_MAX; st.last[lane] = INT64_MIN; st.ns[lane] = 0; st.cnt[lane] = 0;
     }
     __syncwarp();
   }
-  __syncthreads();
-  if (warp == 0) {
-#pragma unroll
-    for (int lv = 2; lv >= 0; lv--) {
-      const int cntl = 1 << lv;
-      if (lane < cntl) {
-        const int i = cntl + lane;
-        i64 x = s.T[2 * i], y = s.T[2 * i + 1];
-        s.T[i] = x > y ? x : y;
-      }
-      __syncwarp();
+  while (pos < vend) {
+    if (a.lane_domain[l] != 0) {
+      const int64_t stop = min((int64_t)a.lane_dom_end[l], vend);
+      attr_fill(a, pos, stop);
+      pos = stop;
+      l = a.lane_dom_next[l];
+      continue;
     }
-  }
-  __syncthreads();
-
-  // nearest earlier OP that is still running when the record starts.  Consecutive records
-  // mostly share it: when the threshold t did not go down since the previous record, nothing
-  // between the previous answer and that record can qualify, so the previous answer (or the
-  // fact that the tile holds none) is reused and the tree is only walked when it has ended.
-  unsigned bad = 0;
-  int32_t par_abs[AT_ITEMS];
-  int16_t plv[AT_ITEMS];
-  uint8_t kc[AT_ITEMS];
-  bool have = false;  // (tq, yq, yeq): threshold and answer of the previous search outside the thread
-  i64 tq = 0, yeq = 0;
-  int yq = -1;
-#pragma unroll
-  for (int j = 0; j < AT_ITEMS; j++) {
-    const int x = x0 + j;
-    int pl = AT_NONE;
-    par_abs[j] = -1;
-    kc[j] = 0;
-    if (hostmask & (1u << j)) {
-      const i64 t = en[j] > st[j] ? st[j] + 1 : en[j];
-      int y = -1;
-      i64 ye = 0;  // end time of y
-#pragma unroll
-      for (int jj = AT_ITEMS - 1; jj >= 0; jj--)
-        if (jj < j && y < 0 && (opmask & (1u << jj)) && en[jj] >= t) { y = x0 + jj; ye = en[jj]; }
-      if (y < 0) {
-        if (have && t >= tq && (yq < 0 || yeq >= t)) {
-          y = yq;
-          ye = yeq;
-        } else {
-          int pos = AT_THREADS + tid;
-          while (pos > 1) {
-            if ((pos & 1) && s.T[pos - 1] >= t) {
-              pos = pos - 1;
-              while (pos < AT_THREADS) pos = s.T[2 * pos + 1] >= t ? 2 * pos + 1 : 2 * pos;
-              const int tb = (pos - AT_THREADS) * AT_ITEMS;
-              for (int k = tb + AT_ITEMS - 1; k >= tb; k--) {
-                ye = s.leaf[AT_LX(k)];
-                if (ye >= t) { y = k; break; }
-              }
-              break;
-            }
-            pos >>= 1;
-          }
-          have = true;
-          yq = y;
-          yeq = ye;
-        }
-        tq = t;
+    const int64_t lane_end = a.lane_off[l + 1], seg_end = min(lane_end, vend);
+    int dmax = 0;
+    bool bad = false;
+    // a row's columns are requested while the row in front of it is worked on
+    int kd = 9, nk = 0, kp = 0;
+    i64 ts = 0, en = 0;
+    auto load = [&](int64_t p) {
+      kd = 9;
+      if (p < seg_end) { kd = a.kind[p]; ts = a.ts[p]; en = a.te[p]; nk = a.kol[p]; kp = a.kernel_of[p]; }
+    };
+    load(pos + lane);
+    for (; pos < seg_end; pos += 32) {
+      const int64_t p = pos + lane;
+      const bool in = p < seg_end, op = kd == TA_KIND_OP;
+      const i64 e = en, t = e > ts ? ts + 1 : e;
+      const int n_k = kd == TA_KIND_LAUNCH ? nk : 0;
+      i64 ks = 0, ke = 0;
+      if (n_k == 1) { ks = a.ts[kp]; ke = a.te[kp]; }
+      load(p + 32);
+      const u32 ops = __ballot_sync(0xffffffffu, op);
+      // nearest operator of the row
+      int q = (ops & lt) ? 31 - __clz((int)(ops & lt)) : -1;
+      i64 pe = 0;  // its end
+      for (;;) {
+        const int src = q < 0 ? 0 : q;
+        pe = shfl_i64(e, src);
+        const int up = __shfl_sync(0xffffffffu, q, src);
+        const bool ended = in && q >= 0 && pe < t;
+        if (!__any_sync(0xffffffffu, ended)) break;
+        if (ended) q = up;
       }
-      const int lo = lo_local[j];
-      if (y >= 0 && y >= lo) {
-        pl = y;
-        par_abs[j] = (int32_t)(tile_start + y);
-        if (ye < en[j]) bad |= 1u << j;
-      } else if (lo >= 0) {
-        pl = AT_NONE;
-      } else {  // the encloser, if any, lies before the tile: the carried stack has it
-        pl = AT_UNRESOLVED;
-        int k = 0;
-        while (k < ccnt && s.carry_e[k] >= t) k++;
-        s.kcarry[x] = (uint8_t)k;
-        kc[j] = (uint8_t)k;
-        if (k > 0) {
-          par_abs[j] = s.carry_pos[k - 1];
-          if (s.carry_e[k - 1] < en[j]) bad |= 1u << j;
-        }
+      // else the stack, from the top
+      int par = q;  // 0..31: record of the row, 32 + k: level k, -1: none
+      bool ask = in && q < 0;
+      for (int k = depth - 1; k >= 0; k--) {
+        if (!__any_sync(0xffffffffu, ask)) break;
+        const i64 ek = st.e[k];
+        if (ask && ek >= t) { par = 32 + k; pe = ek; ask = false; }
       }
-    }
-    plv[j] = (int16_t)pl;
-  }
-  // Kernels per operator: an operator owns the kernels of the launches directly inside it.  They are
-  // added up here, from the launch side, in shared memory - consecutive launches mostly share their
-  // operator, and one addition serves a run of them; three atomics per kernel on the operator's row
-  // in memory, from the device side, and the clearing and decoding passes around them took 1.2 ms
-  // of 66.8 M records.  The kernels of a launch that has several (a graph replay) are left to
-  // k_attr_ops, which meets them one by one.
-  {
-    int run_row = -1, run_cnt = 0;
-    i64 run_f = 0, run_l = 0;
-    u64 run_ns = 0;
-#pragma unroll
-    for (int j = 0; j < AT_ITEMS; j++) {
-      if (nk[j] <= 0 || par_abs[j] < 0) continue;
-      const int row = plv[j] >= 0 ? plv[j] : AT_TILE + kc[j] - 1;
-      if (nk[j] > 1) {
-        if (row < AT_TILE) atomicOr(&s.k_cnt[row], (int)AT_MORE);
-        continue;
-      }
-      if (row != run_row) {
-        if (run_row >= 0) attr_add(s, run_row, run_cnt, run_f, run_l, run_ns);
-        run_row = row;
-        run_cnt = 0;
-        run_f = INT64_MAX;
-        run_l = INT64_MIN;
-        run_ns = 0;
-      }
-      run_cnt++;
-      run_f = min(run_f, ks[j]);
-      run_l = max(run_l, ke[j]);
-      run_ns += (u64)(ke[j] - ks[j]);
-    }
-    if (run_row >= 0) attr_add(s, run_row, run_cnt, run_f, run_l, run_ns);
-  }
-  if (open_pos >= 0) atomicOr(&s.k_cnt[open_pos], (int)AT_MORE);
-#pragma unroll
-  for (int q = 0; q < AT_ITEMS / 2; q++)
-    *reinterpret_cast<u32 *>(&s.parent_local[x0 + 2 * q]) =
-        (u32)(uint16_t)plv[2 * q] | ((u32)(uint16_t)plv[2 * q + 1] << 16);
-  __syncthreads();
-  // depth = level in the parent forest; the chain is only followed through shared memory when
-  // the parent is another thread's record and differs from the previous record's parent
-  int dmax = 0;
-  uint8_t dep[AT_ITEMS];
-#pragma unroll
-  for (int j = 0; j < AT_ITEMS; j++) {
-    int d = 0;
-    if (hostmask & (1u << j)) {
-      const int pl = plv[j];
-      if (pl == AT_UNRESOLVED) {
-        d = kc[j];
-      } else if (pl >= x0) {  // one of the thread's own earlier records
-#pragma unroll
-        for (int jj = 0; jj < AT_ITEMS; jj++)
-          if (jj < j && pl == x0 + jj) d = dep[jj] + 1;
-      } else if (pl >= 0) {
-        if (j > 0 && (hostmask & (1u << (j > 0 ? j - 1 : 0))) && plv[j > 0 ? j - 1 : 0] == pl) {
-          d = dep[j > 0 ? j - 1 : 0];
-        } else {
-          d = 1;
-          int c = pl;
-          for (int it = 0; it < 300; it++) {
-            const int q = s.parent_local[c];
-            if (q == AT_NONE) break;
-            if (q == AT_UNRESOLVED) { d += s.kcarry[c]; break; }
-            d++;
-            c = q;
-          }
-        }
+      bad |= in && par >= 0 && pe < e;
+      // level in the forest: distances to an ancestor, doubled until it is one whose level is known
+      int d = par >= 32 ? par - 31 : par >= 0 ? 1 : 0, anc = q;
+      if (!in) anc = -1;
+      while (__any_sync(0xffffffffu, anc >= 0)) {
+        const int src = anc < 0 ? 0 : anc;
+        const int d2 = __shfl_sync(0xffffffffu, d, src), a2 = __shfl_sync(0xffffffffu, anc, src);
+        if (anc >= 0) { d += d2; anc = a2; }
       }
       if (d > 255) d = 255;
-      dmax = max(dmax, d);
-      if (bad & (1u << j)) atomicOr(&a.sum[a.lane_window[ln[j]]].bad_nesting, 1);
+      if (in) dmax = max(dmax, d);
+      // kernels, operator by operator (a row has a handful of operators that own launches)
+      u32 cnt = 0;
+      i64 first = INT64_MAX, last = INT64_MIN;
+      u64 ns = 0;
+      u32 left = __ballot_sync(0xffffffffu, n_k == 1 && par >= 0);
+      if (left) {
+        const i64 base = shfl_i64(ks, __ffs((int)left) - 1);
+        const i64 rs = ks - base, re = ke - base, dur = ke - ks;
+        const bool mine = left >> lane & 1u;
+        // times within half a second of the row's first kernel and kernels below 67 ms: 32-bit reductions
+        const bool near = rs > -(1ll << 30) && re < (1ll << 30) && dur < (1ll << 26);
+        if (__all_sync(0xffffffffu, !mine || near)) {
+          while (left) {
+            const int key = __shfl_sync(0xffffffffu, par, __ffs((int)left) - 1);
+            const bool same = mine && par == key;
+            const u32 who = __ballot_sync(0xffffffffu, same);
+            const i64 f = base + __reduce_min_sync(0xffffffffu, same ? (int)rs : INT_MAX);
+            const i64 g = base + __reduce_max_sync(0xffffffffu, same ? (int)re : INT_MIN);
+            const u32 du = __reduce_add_sync(0xffffffffu, same ? (u32)dur : 0u);
+            left &= ~who;
+            if (key < 32) {
+              if (lane == key) { cnt = (u32)__popc(who); first = f; last = g; ns = du; }
+            } else if (lane == 0) {
+              const int k = key - 32;
+              st.cnt[k] += (u32)__popc(who);
+              st.first[k] = min(st.first[k], f);
+              st.last[k] = max(st.last[k], g);
+              st.ns[k] += du;
+            }
+          }
+        } else {
+          for (; left; left &= left - 1) {
+            const int src = __ffs((int)left) - 1;
+            const int key = __shfl_sync(0xffffffffu, par, src);
+            const i64 f = shfl_i64(ks, src), g = shfl_i64(ke, src);
+            if (key < 32) {
+              if (lane == key) { cnt++; first = min(first, f); last = max(last, g); ns += (u64)(g - f); }
+            } else if (lane == 0) {
+              const int k = key - 32;
+              st.cnt[k]++;
+              st.first[k] = min(st.first[k], f);
+              st.last[k] = max(st.last[k], g);
+              st.ns[k] += (u64)(g - f);
+            }
+          }
+        }
+      }
+      // launches with several kernels (graph replays): k_attr_ops meets their kernels one by one
+      for (u32 many = __ballot_sync(0xffffffffu, n_k > 1 && par >= 0); many; many &= many - 1) {
+        const int key = __shfl_sync(0xffffffffu, par, __ffs((int)many) - 1);
+        if (key < 32) { if (lane == key) cnt |= AS_MORE; }
+        else if (lane == 0) st.cnt[key - 32] |= AS_MORE;
+      }
+      __syncwarp();
+      if (in) {
+        a.parent[p] = par >= 32 ? st.pos[par - 32] : par >= 0 ? (int32_t)(pos + par) : -1;
+        a.depth[p] = (uint8_t)d;
+        a.op_n[p] = (int32_t)(cnt & ~AS_MORE);
+        a.op_first[p] = cnt ? first : 0;
+        a.op_last[p] = cnt ? last : 0;
+        a.op_ns[p] = (i64)ns;
+      }
+      if (ops) {
+        // the stack behind the row: the last operator and those around it, on what is left of the levels
+        u32 open = 0;
+        int c = 31 - __clz((int)ops);
+        while (c >= 0 && c < 32) {
+          open |= 1u << c;
+          c = __shfl_sync(0xffffffffu, par, c);
+        }
+        const int keep = c >= 32 ? c - 31 : 0;
+        __syncwarp();  // (the row's zeros and parents are out before levels are written to or replaced)
+        attr_pop(a, st, keep, depth, carried, false);
+        if (carried > keep) carried = keep;
+        const int at = keep + __popc(open & lt);
+        if ((open >> lane & 1u) && at < AS_LEVELS) {
+          st.e[at] = e;
+          st.pos[at] = (int32_t)p;
+          st.first[at] = first;
+          st.last[at] = last;
+          st.ns[at] = ns;
+          st.cnt[at] = cnt;
+        }
+        depth = keep + __popc(open);
+        if (depth > AS_LEVELS) {
+          depth = AS_LEVELS;
+          if (lane == 0) ta_set_err(a.status, TA_ERR_DEPTH);
+        }
+        __syncwarp();
+      }
     }
-    dep[j] = (uint8_t)d;
-  }
-  if (full) {
-#pragma unroll
-    for (int q = 0; q < AT_ITEMS / 4; q++) {
-      *reinterpret_cast<int4 *>(a.parent + p0 + 4 * q) =
-          make_int4(par_abs[4 * q], par_abs[4 * q + 1], par_abs[4 * q + 2], par_abs[4 * q + 3]);
-      *reinterpret_cast<u32 *>(a.depth + p0 + 4 * q) =
-          dep[4 * q] | (dep[4 * q + 1] << 8) | (dep[4 * q + 2] << 16) | ((u32)dep[4 * q + 3] << 24);
+    pos = seg_end;
+    // the window's deepest record and partial overlap
+    dmax = __reduce_max_sync(0xffffffffu, dmax);
+    bad = __any_sync(0xffffffffu, bad);
+    if (lane == 0) {
+      ta_attr_summary *row = &a.sum[a.lane_window[l]];
+      if (dmax > *(volatile int32_t *)&row->max_depth) atomicMax(&row->max_depth, dmax);
+      if (bad) atomicOr(&row->bad_nesting, 1);
     }
-  } else {
-#pragma unroll
-    for (int j = 0; j < AT_ITEMS; j++)
-      if (p0 + j < a.n) { a.parent[p0 + j] = par_abs[j]; a.depth[p0 + j] = dep[j]; }
+    if (lane_end <= vend) {  // the lane is over: nothing stays open
+      attr_pop(a, st, 0, depth, carried, false);
+      depth = carried = 0;
+      l++;
+    }
   }
-  attr_store_ops<false>(a, s, p0, x0);
-  // what the carried operators are owed
-  if (tid < ccnt && s.k_cnt[AT_TILE + tid]) {
-    const int r = AT_TILE + tid;
-    a.spill[atomicAdd(a.n_spill, 1u)] = AttrSpill{s.carry_pos[tid], s.k_cnt[r], s.k_first[r], s.k_last[r], (i64)s.k_ns[r]};
-  }
-  // per-window maximum depth (a tile rarely meets more than one window)
-  const int lane_last = s.lane1;
-  const int w_first = l0 >= 0 ? a.lane_window[l0] : 0;
-  const int w_last = lane_last >= 0 ? a.lane_window[lane_last] : w_first;
-  if (w_first == w_last) {
-    dmax = (int)warp_reduce((u64)dmax, OpMax());
-    if (lane == 0 && dmax > 0) atomicMax(&s.dmax, dmax);
-    __syncthreads();
-    if (tid == 0 && s.dmax > 0) atomicMax(&a.sum[w_first].max_depth, s.dmax);
-  } else {
-#pragma unroll
-    for (int j = 0; j < AT_ITEMS; j++)
-      if ((hostmask & (1u << j)) && dep[j]) atomicMax(&a.sum[a.lane_window[ln[j]]].max_depth, (int)dep[j]);
-  }
+  attr_pop(a, st, 0, depth, carried, true);
+  if (vend < tile_end) attr_fill(a, vend, tile_end);
 }
 
 // ---- device records inherit the operator of their launch ------------------------
@@ -855,7 +727,10 @@ ta_status ta_run_attribute(ta_window *h, ta_attr_summary *out_summary) {
   const int64_t n = h->n, nn = n > 0 ? n : 1;
   const int W = h->W;
   cudaStream_t st = h->stream;
-  const int64_t tiles = (n + AT_TILE - 1) / AT_TILE;
+  // Tiles of 1024 records; of 256 while their stacks are folded in two levels, so that a window of some
+  // ten thousand records has work for more than a few SMs (a warp takes a tile).
+  const int per_tile = n <= 256ll * AT_FAN * AT_FAN ? 256 : 1024;
+  const int64_t tiles = (n + per_tile - 1) / per_tile;
   size_t keep = 3 * Carver::pad(nn * 4) + Carver::pad(nn) + 3 * Carver::pad(nn * 8) + 256;
   void *kb = ta_dalloc(h, keep);
   if (!kb) return TA_ERR_OOM;
@@ -896,7 +771,7 @@ ta_status ta_run_attribute(ta_window *h, ta_attr_summary *out_summary) {
   a.n = n; a.n_valid = h->n_valid; a.n_lanes = h->sorted.n_lanes; a.n_tiles = tiles;
   a.kind = h->sorted.kind; a.ts = h->sorted.ts_start; a.te = h->sorted.ts_end;
   a.lane_off = h->sorted.lane_off; a.lane_window = h->sorted.lane_window;
-  a.lane_domain = h->sorted.lane_domain; a.lane_dom_end = h->d_lane_dom_end;
+  a.lane_domain = h->sorted.lane_domain; a.lane_dom_end = h->d_lane_dom_end; a.lane_dom_next = h->d_lane_dom_next;
   a.parent = parent; a.depth = depth; a.sum = d_sum; a.status = h->d_status;
   a.launch_of = h->join.launch_of; a.kol = h->join.kernels_of_launch; a.kernel_of = h->d_kernel_of; a.op_of = op_of; a.op_n = op_n; a.op_first = op_first;
   a.op_last = op_last; a.op_ns = op_ns;
@@ -906,7 +781,7 @@ ta_status ta_run_attribute(ta_window *h, ta_attr_summary *out_summary) {
   TA_TRY(ta_queue_d2h(h, words, h->d_status, sizeof(words)));
   if (small) TA_TRY(ta_queue_d2h(h, hs.data(), d_sum, W * sizeof(ta_attr_summary)));
   if (n > 0) {
-    ta_launch(k_attr_agg, (unsigned)tiles, AT_THREADS, 0, st, a);
+    ta_launch(per_tile == 256 ? k_attr_agg<1> : k_attr_agg<4>, (unsigned)tiles, AT_THREADS, 0, st, a);
     {
       // level 0 = tiles; fold upwards until at most AT_FAN stacks remain, scan those, unfold
       std::vector<StackArr> node(level_n.size()), start(level_n.size());
@@ -924,7 +799,8 @@ ta_status ta_run_attribute(ta_window *h, ta_attr_summary *out_summary) {
       for (size_t k = top; k >= 1; k--)
         ta_launch(k_attr_fold_down, (unsigned)((level_n[k] + 3) / 4), 128, 0, st, node[k - 1], level_n[k - 1], start[k], level_n[k], start[k - 1], k == 1 ? 1 : 0, h->d_status);
     }
-    ta_launch(k_attr_resolve, (unsigned)tiles, AT_THREADS, 0, st, a);
+    ta_launch(per_tile == 256 ? k_attr_resolve<256> : k_attr_resolve<1024>, (unsigned)((tiles + AS_WARPS - 1) / AS_WARPS),
+              AS_WARPS * 32, 0, st, a);
     const int64_t sb = (tiles * 4 + 255) / 256;
     ta_launch(k_attr_spill, (unsigned)(sb < 148 * 4 ? sb : 148 * 4), 256, 0, st, a);
     const unsigned ob = (unsigned)((n + AT_OPS_TILE - 1) / AT_OPS_TILE);

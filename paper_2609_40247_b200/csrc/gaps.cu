@@ -3,14 +3,15 @@
 // the busy union, idle time, a log2 gap histogram and the list of long gaps.
 // Idle time of a stream = what none of its activity records covers (Sec. 9.1).
 //
-// One pass over the sorted ts_start / ts_end / kind columns.  The scan is made
-// lane-aware without segment flags: the scanned value is (lane + 1) << 40 |
+// One pass over the sorted ts_start / ts_end columns, k_gaps_rows, where every lane ends its
+// records in ascending order; a chained scan, k_gaps, where some lane does not.  The scan is
+// made lane-aware without segment flags: the scanned value is (lane + 1) << 40 |
 // (clipped end - window start), which grows from lane to lane, so a prefix
 // that belongs to an earlier lane is recognised by its upper bits.  Long gaps
 // are rare: they are appended to a list with an atomic cursor, each sets the bit of its
 // place in the order (two per record: the gap in front of it, the tail gap behind it) in
 // a bitmap, and a scan over the bitmap's words tells every entry its rank.
-// HBM-bound: 18 B read + 8 B written per device record.
+// HBM-bound: 16 B read + 8 B written per device record.
 #include <climits>
 
 #include "scan.cuh"
@@ -24,6 +25,12 @@
 #define GP_MINB 4
 #endif
 #define GP_TILE (GP_THREADS * GP_ITEMS)
+#ifndef GR_MINB
+#define GR_MINB 6
+#endif
+#ifndef GR_ROWS
+#define GR_ROWS 32
+#endif
 // lanes of a tile whose statistics are folded on chip: in a batch of many windows a lane is a
 // thousand records or so and a tile meets several (a batch of 512 windows of 65 k records: 395 us
 // with two lanes folded and the rest by global atomics per record)
@@ -37,12 +44,11 @@ struct GapArgs {
   const int16_t *kind;
   const int32_t *lane_off, *lane_window;
   const int16_t *lane_domain;
-  const int32_t *lane_dom_end;
+  const int32_t *lane_dom_end, *lane_dom_next;
   const int64_t *t0, *t1;
   i64 min_gap;
   int list_only;  // second run: only (re)write the long-gap list
-  int local;      // 1: take the end of the record in front as the running maximum (and check that it is)
-  u32 *not_ascending;  // set in local mode when some lane does not end its records in ascending order
+  u32 *not_ascending;  // set by k_gaps_rows when some lane does not end its records in ascending order
   int64_t *gap_before;
   ta_lane_gaps *lane_gaps;
   u32 *lane_hist, *win_hist;
@@ -56,6 +62,15 @@ struct GapArgs {
   u64 *n_long;        // append cursor
 };
 
+
+// entry `o` of the long-gap list; key: its place in the order
+__device__ __forceinline__ void gap_append(const GapArgs &a, i64 o, const ta_long_gap &g, u32 key) {
+  if (o < a.list_cap) {
+    a.list[o] = g;
+    a.list_key[o] = key;
+  }
+  atomicOr(&a.bits[key >> 6], 1ull << (key & 63u));
+}
 
 __device__ __forceinline__ void gaps_tile(const GapArgs &a) {
   __shared__ u64 tmp[33];
@@ -98,8 +113,7 @@ __device__ __forceinline__ void gaps_tile(const GapArgs &a) {
     }
     return;
   }
-  // kinds, start and end times of the thread's records and, for the scan-free mode, the end of
-  // the record in front of the thread's first one: all requested together (the tile holds a
+  // kinds, start and end times of the thread's records, all requested together (the tile holds a
   // device lane, so nearly every record needs its times anyway)
   int16_t kd[GP_ITEMS];
   loadn_i16<GP_ITEMS>(a.kind, p0, a.n, 0, kd);
@@ -120,7 +134,6 @@ __device__ __forceinline__ void gaps_tile(const GapArgs &a) {
     for (int j = 0; j < GP_ITEMS; j++)
       if (p0 + j < a.n) { s[j] = a.ts[p0 + j]; ce[j] = a.te[p0 + j]; }
   }
-  const i64 e_before = (a.local && p0 > 0 && p0 <= a.n) ? a.te[p0 - 1] : 0;
 #pragma unroll
   for (int j = 0; j < GP_ITEMS; j++)
     if (p0 + j >= a.n_valid) kd[j] = 0;
@@ -155,30 +168,16 @@ __device__ __forceinline__ void gaps_tile(const GapArgs &a) {
       s_lane1 = l;
     }
   }
-  u64 pre = 0;
-  if (a.local) {
-    // in-order streams end their records in ascending order: the running maximum in front of a
-    // record is the (clipped) end of its neighbour, no scan and no look-back; the loop below
-    // checks the order and reports the first lane that breaks it
-    const int l = ln[0];
-    if (l >= 0 && p0 > (int64_t)a.lane_off[l]) {
-      const int w = a.lane_window[l];
-      const i64 w0 = a.t0[w], w1 = a.t1[w], e = e_before;
-      pre = ((u64)(l + 1) << 40) | (u64)((e < w1 ? e : w1) - w0);
-    }
-    __syncthreads();  // s_lane1 and the zeroed histograms are read below
-  } else {
-    u64 tile_max;
-    u64 thread_excl = block_scan_exclusive<OpMax>(run, OpMax(), tmp, &tile_max);
-    if (tid < 32) {
-      bool failed;
-      u64 ex = tile_lookback<OpMax>(a.st_max, tile, tile_max, OpMax(), a.status, &failed);
-      if (tid == 0) { s_excl_max = ex; s_fail = failed ? 1 : 0; }
-    }
-    __syncthreads();
-    if (s_fail) return;
-    pre = s_excl_max > thread_excl ? s_excl_max : thread_excl;
+  u64 tile_max;
+  u64 thread_excl = block_scan_exclusive<OpMax>(run, OpMax(), tmp, &tile_max);
+  if (tid < 32) {
+    bool failed;
+    u64 ex = tile_lookback<OpMax>(a.st_max, tile, tile_max, OpMax(), a.status, &failed);
+    if (tid == 0) { s_excl_max = ex; s_fail = failed ? 1 : 0; }
   }
+  __syncthreads();
+  if (s_fail) return;
+  u64 pre = s_excl_max > thread_excl ? s_excl_max : thread_excl;
 
   // gaps; statistics of the thread's first lane stay in registers, anything else is rare
   i64 gap[GP_ITEMS];
@@ -196,7 +195,6 @@ __device__ __forceinline__ void gaps_tile(const GapArgs &a) {
       if (l >= 0) {
         if (wl != l) { int w = a.lane_window[l]; w0 = a.t0[w]; w1 = a.t1[w]; wl = l; }
         Pi = ((pre >> 40) == (u64)(l + 1)) ? w0 + (i64)(pre & GP_LOW) : w0;
-        if (a.local && (pre >> 40) == (u64)(l + 1) && ce[j] < Pi) *a.not_ascending = 1u;
         g = s[j] > Pi ? s[j] - Pi : 0;
         const i64 from = s[j] > Pi ? s[j] : Pi;
         bz = ce[j] > from ? ce[j] - from : 0;
@@ -217,22 +215,10 @@ __device__ __forceinline__ void gaps_tile(const GapArgs &a) {
           u64 base = 0;
           if (wlane == 0) base = atomicAdd(a.n_long, (u64)(__popc(m_g) + __popc(m_t)));
           base = __shfl_sync(0xffffffffu, base, 0);
-          if (lg) {
-            const i64 o = (i64)base + __popc(m_g & below);
-            if (o < a.list_cap) {
-              a.list[o] = ta_long_gap{l, (int32_t)(p0 + j), Pi, g};
-              a.list_key[o] = (u32)(p0 + j) << 1;
-            }
-            atomicOr(&a.bits[(p0 + j) >> 5], 1ull << (((u32)(p0 + j) & 31u) << 1));
-          }
-          if (lt) {
-            const i64 o = (i64)base + __popc(m_g) + __popc(m_t & below);
-            if (o < a.list_cap) {
-              a.list[o] = ta_long_gap{l, -1, w1 - tl, tl};
-              a.list_key[o] = (u32)(p0 + j) << 1 | 1u;
-            }
-            atomicOr(&a.bits[(p0 + j) >> 5], 2ull << (((u32)(p0 + j) & 31u) << 1));
-          }
+          if (lg) gap_append(a, (i64)base + __popc(m_g & below), ta_long_gap{l, (int32_t)(p0 + j), Pi, g}, (u32)(p0 + j) << 1);
+          if (lt)
+            gap_append(a, (i64)base + __popc(m_g) + __popc(m_t & below), ta_long_gap{l, -1, w1 - tl, tl},
+                       (u32)(p0 + j) << 1 | 1u);
         }
       }
       if (l < 0) continue;
@@ -317,6 +303,160 @@ __global__ void __launch_bounds__(GP_THREADS, GP_MINB) k_gaps(GapArgs a, Tail ta
   run_tail(tail);
 }
 
+// The same for streams that end their records in ascending order, as in-order streams do: the running
+// maximum in front of a record is the clipped end of its neighbour, no scan and no tile waits for
+// another.  Checked on the way; one record that ends before the one in front of it sends the call
+// through k_gaps.
+// A warp takes `rows` x 32 consecutive positions, 32 records of ONE lane at a time: lane, window and
+// bounds are then the same for the whole warp and the neighbour's end is a shuffle away (a thread
+// with eight consecutive records, each with its own lane walk, took 270 warp instructions per 32
+// records and bound the kernel: 480 us for 66.8 M records).  Statistics of the CTA's first GR_LANES
+// lanes are folded on chip.
+#define GR_LANES 4
+__device__ __forceinline__ void gaps_rows(const GapArgs &a, int rows) {
+  __shared__ u64 s_sum[GR_LANES][3];  // busy, idle, gaps
+  __shared__ i64 s_max[GR_LANES];
+  __shared__ u32 s_hist[GR_LANES][TA_NBINS];
+  __shared__ int s_lane0;
+  if (ta_failed(a.status)) return;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  for (int i = tid; i < GR_LANES * TA_NBINS; i += GP_THREADS) (&s_hist[0][0])[i] = 0;
+  if (tid < GR_LANES * 3) (&s_sum[0][0])[tid] = 0;
+  if (tid < GR_LANES) s_max[tid] = 0;
+  const int64_t span = (int64_t)rows * 32;
+  const int64_t begin = ((int64_t)blockIdx.x * (GP_THREADS / 32) + warp) * span;
+  const int64_t end = min(begin + span, a.n), vend = min(end, a.n_valid);
+  int l = begin < vend ? tile_lane_search(a.lane_off, a.n_lanes, begin) : 0;
+  if (tid == 0) s_lane0 = l;
+  __syncthreads();
+  const int l0 = s_lane0;
+  int64_t pos = begin;
+  while (pos < vend) {
+    if (a.lane_domain[l] != 1) {  // host lanes: no gaps
+      const int64_t stop = min((int64_t)a.lane_dom_end[l], vend);
+      for (int64_t p = pos + lane; p < stop; p += 32) a.gap_before[p] = 0;
+      pos = stop;
+      l = a.lane_dom_next[l];
+      continue;
+    }
+    const int64_t off = a.lane_off[l], lane_end = a.lane_off[l + 1], seg_end = min(lane_end, vend);
+    const int w = a.lane_window[l];
+    const i64 w0 = a.t0[w], w1 = a.t1[w];
+    const int li = l - l0;
+    u32 *hist = li < GR_LANES ? s_hist[li] : nullptr;
+    i64 s = 0, e = 0;
+    if (pos + lane < seg_end) { s = a.ts[pos + lane]; e = a.te[pos + lane]; }
+    i64 carry = pos > off ? min((i64)a.te[pos - 1], w1) : w0;  // P of the row's first record
+    u64 sb = 0, si = 0;
+    i64 mg = 0;
+    u32 ng = 0;
+    for (; pos < seg_end; pos += 32) {
+      const int64_t p = pos + lane;
+      const bool in = p < seg_end;
+      const i64 ce = min(e, w1), cs = s;
+      if (p + 32 < seg_end) { s = a.ts[p + 32]; e = a.te[p + 32]; }  // the next row's, while this one is worked on
+      i64 P = __shfl_up_sync(0xffffffffu, ce, 1);
+      if (lane == 0) P = carry;
+      carry = __shfl_sync(0xffffffffu, ce, 31);
+      const i64 g = in && cs > P ? cs - P : 0;
+      bool lt = false;
+      i64 tl = 0;
+      if (in) {
+        if (p > off && ce < P) *a.not_ascending = 1u;
+        const i64 from = cs > P ? cs : P;
+        sb += (u64)(ce > from ? ce - from : 0);
+        si += (u64)g;
+        if (g > 0) {
+          ng++;
+          mg = max(mg, g);
+          if (hist) {
+            atomicAdd(&hist[log2_bin(g)], 1u);
+          } else {
+            atomicAdd(&a.lane_hist[(size_t)l * TA_NBINS + log2_bin(g)], 1u);
+            atomicAdd(&a.win_hist[(size_t)w * TA_NBINS + log2_bin(g)], 1u);
+          }
+        }
+        a.gap_before[p] = g;
+        if (p == off) a.lane_gaps[l].first_start = cs;
+        if (p + 1 == lane_end) {
+          tl = w1 - max(P, ce);
+          if (tl > 0) {
+            ng++;
+            mg = max(mg, tl);
+            si += (u64)tl;
+            if (hist) {
+              atomicAdd(&hist[log2_bin(tl)], 1u);
+            } else {
+              atomicAdd(&a.lane_hist[(size_t)l * TA_NBINS + log2_bin(tl)], 1u);
+              atomicAdd(&a.win_hist[(size_t)w * TA_NBINS + log2_bin(tl)], 1u);
+            }
+            lt = tl >= a.min_gap;
+          }
+          a.lane_gaps[l].last_end = w1 - tl;
+          a.lane_gaps[l].n_events = lane_end - off;
+        }
+      }
+      // long-gap list: the warp reserves its entries with one add on the cursor (they are put in
+      // order afterwards)
+      const bool lg = g > 0 && g >= a.min_gap;
+      if (__any_sync(0xffffffffu, lg || lt)) {
+        const u32 m_g = __ballot_sync(0xffffffffu, lg), m_t = __ballot_sync(0xffffffffu, lt);
+        const u32 below = (1u << lane) - 1u;
+        u64 base = 0;
+        if (lane == 0) base = atomicAdd(a.n_long, (u64)(__popc(m_g) + __popc(m_t)));
+        base = __shfl_sync(0xffffffffu, base, 0);
+        if (lg) gap_append(a, (i64)base + __popc(m_g & below), ta_long_gap{l, (int32_t)p, P, g}, (u32)p << 1);
+        if (lt) gap_append(a, (i64)base + __popc(m_g) + __popc(m_t & below), ta_long_gap{l, -1, w1 - tl, tl}, (u32)p << 1 | 1u);
+      }
+    }
+    pos = seg_end;
+    // the lane's share of this warp
+    sb = warp_reduce(sb, OpAdd());
+    si = warp_reduce(si, OpAdd());
+    ng = __reduce_add_sync(0xffffffffu, ng);
+    mg = (i64)warp_reduce((u64)mg, OpMax());
+    if (lane == 0) {
+      if (hist) {
+        if (sb) atomicAdd(&s_sum[li][0], sb);
+        if (si) atomicAdd(&s_sum[li][1], si);
+        if (ng) atomicAdd(&s_sum[li][2], (u64)ng);
+        if (mg > s_max[li]) atomicMax(&s_max[li], mg);
+      } else {
+        ta_lane_gaps *gl = &a.lane_gaps[l];
+        if (sb) atomicAdd((u64 *)&gl->busy, sb);
+        if (si) atomicAdd((u64 *)&gl->idle, si);
+        if (ng) atomicAdd((u64 *)&gl->n_gaps, (u64)ng);
+        if (mg) atomicMax((i64 *)&gl->max_gap, mg);
+      }
+    }
+    if (lane_end <= vend) l++;
+  }
+  for (int64_t p = max(begin, vend) + lane; p < end; p += 32) a.gap_before[p] = 0;  // dropped records
+  __syncthreads();
+  for (int i = tid; i < GR_LANES * (TA_NBINS + 4); i += GP_THREADS) {
+    const int li = i / (TA_NBINS + 4), k = i - li * (TA_NBINS + 4), ll = l0 + li;
+    if (ll >= a.n_lanes) continue;
+    ta_lane_gaps *gl = &a.lane_gaps[ll];
+    if (k < TA_NBINS) {
+      const u32 c = s_hist[li][k];
+      if (c) {
+        atomicAdd(&a.lane_hist[(size_t)ll * TA_NBINS + k], c);
+        atomicAdd(&a.win_hist[(size_t)a.lane_window[ll] * TA_NBINS + k], c);
+      }
+    } else if (k < TA_NBINS + 3) {
+      const u64 v = s_sum[li][k - TA_NBINS];
+      if (v) atomicAdd(k == TA_NBINS ? (u64 *)&gl->busy : k == TA_NBINS + 1 ? (u64 *)&gl->idle : (u64 *)&gl->n_gaps, v);
+    } else if (s_max[li]) {
+      atomicMax((i64 *)&gl->max_gap, s_max[li]);
+    }
+  }
+}
+__global__ void __launch_bounds__(GP_THREADS, GR_MINB) k_gaps_rows(GapArgs a, int rows, Tail tail) {
+  TA_PDL();
+  gaps_rows(a, rows);
+  run_tail(tail);
+}
+
 struct GapBitsIn {
   const u64 *bits;
   __device__ u64 operator()(int64_t i) const { return (u64)__popcll(bits[i]); }
@@ -385,7 +525,7 @@ ta_status ta_run_gaps(ta_window *h, int64_t min_gap, ta_gap_result *out) {
   a.n = n; a.n_valid = h->n_valid; a.n_lanes = L;
   a.ts = h->sorted.ts_start; a.te = h->sorted.ts_end; a.kind = h->sorted.kind;
   a.lane_off = h->sorted.lane_off; a.lane_window = h->sorted.lane_window;
-  a.lane_domain = h->sorted.lane_domain; a.lane_dom_end = h->d_lane_dom_end; a.t0 = h->d_t0; a.t1 = h->d_t1;
+  a.lane_domain = h->sorted.lane_domain; a.lane_dom_end = h->d_lane_dom_end; a.lane_dom_next = h->d_lane_dom_next; a.t0 = h->d_t0; a.t1 = h->d_t1;
   a.min_gap = min_gap; a.list_only = 0;
   a.gap_before = gap_before; a.lane_gaps = lane_gaps; a.lane_hist = lane_hist; a.win_hist = win_hist;
   a.list = ulist; a.list_key = ukeys; a.list_cap = cap; a.st_max = st_max; a.bits = bits;
@@ -395,16 +535,25 @@ ta_status ta_run_gaps(ta_window *h, int64_t min_gap, ta_gap_result *out) {
   int32_t words[ST_WORDS];
   // first without the scan (every lane is taken to end its records in ascending order, which the
   // kernel checks); if a lane does not, once more with the chained maximum scan
-  for (a.local = 1; a.local >= 0; a.local--) {
-    u64 two[3] = {0, 0, 0};
-    TA_TRY(ta_queue_d2h(h, two, scal, 24));
+  for (int scan = 0; scan < 2; scan++) {
+    u64 three[3] = {0, 0, 0};
+    TA_TRY(ta_queue_d2h(h, three, scal, 24));
     TA_TRY(ta_queue_d2h(h, words, h->d_status, sizeof(words)));
-    if (tiles > 0) ta_launch(k_gaps, (unsigned)tiles, GP_THREADS, 0, st, a, ta_tail(h, tiles));
+    if (tiles > 0 && scan) {
+      ta_launch(k_gaps, (unsigned)tiles, GP_THREADS, 0, st, a, ta_tail(h, tiles));
+    } else if (tiles > 0) {
+      // rows per warp: 32 (a thousand records share a warp's set-up and its flush), fewer while that
+      // would leave SMs without work
+      int64_t rows = n / 32 / (148 * 16);
+      rows = rows < 4 ? 4 : rows > GR_ROWS ? GR_ROWS : rows;
+      const int64_t per_cta = rows * GP_THREADS, grid = (n + per_cta - 1) / per_cta;
+      ta_launch(k_gaps_rows, (unsigned)grid, GP_THREADS, 0, st, a, (int)rows, ta_tail(h, grid));
+    }
     TA_CHECK_CUDA(h, cudaGetLastError());
     TA_TRY(ta_sync_fetch(h));
     if (words[ST_ERR]) return (ta_status)words[ST_ERR];
-    n_long = two[0];
-    if (!a.local || !(u32)two[2]) break;
+    n_long = three[0];
+    if (scan || !(u32)three[2]) break;
     TA_CHECK_CUDA(h, cudaMemsetAsync(b, 0, bytes, st));
     TA_CHECK_CUDA(h, cudaMemsetAsync(tb, 0, tmp_zero, st));
   }

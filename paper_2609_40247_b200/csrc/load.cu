@@ -188,7 +188,7 @@ struct __align__(128) DiscoverSmem {
   int fail;
 };
 
-__global__ void __launch_bounds__(DS_THREADS) k_discover_staged(DiscoverArgs a) {
+__global__ void __launch_bounds__(DS_THREADS, 4) k_discover_staged(DiscoverArgs a) {
   TA_PDL();
   extern __shared__ __align__(128) unsigned char ds_raw[];
   DiscoverSmem &s = *reinterpret_cast<DiscoverSmem *>(ds_raw);

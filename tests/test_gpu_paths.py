@@ -127,3 +127,20 @@ def test_records_at_an_odd_eight_bytes(n, monkeypatch):
     ev = np.ascontiguousarray(wl.events[:n])
     assert len(ev) == n
     both(ev, [0, n], wl.win_t0, wl.win_t1, comm_sizes=wl.comm_sizes)
+
+
+@pytest.mark.parametrize("name,scale", [("c2", 0.004), ("c2", 0.03), ("c3", 0.01)])
+def test_operators_with_kernels_far_apart(name, scale):
+    """Kernels that start up to seconds after their launch or run for up to seconds: the row's kernel
+    times do not fit the 32-bit reductions of the attribution, nor do the lanes end in ascending order."""
+    wl = synth.make_workload(name, scale, truth=False)
+    ev = wl.events.copy()
+    rng = np.random.default_rng(5)
+    k = np.nonzero(ev["kind"] == 3)[0]
+    late = rng.choice(k, size=len(k) // 50, replace=False)
+    shift = rng.integers(0, 3_000_000_000, size=len(late))
+    ev["ts_start"][late] += shift
+    ev["ts_end"][late] += shift
+    long = rng.choice(k, size=len(k) // 50, replace=False)
+    ev["ts_end"][long] += rng.integers(0, 1 << 33, size=len(long))
+    both(ev, wl.win_off, wl.win_t0, np.asarray(wl.win_t1) + 4_000_000_000, comm_sizes=wl.comm_sizes)
