@@ -395,23 +395,24 @@ struct AggRowOut {
   u32 *g_hist;
 };
 
-// Dense cells: compaction of the non-empty ones in cell (= key) order, 256 cells per CTA, chained over
-// the CTAs.  The histograms (160 of a row's 200 bytes) are copied by the CTA together, 16 bytes per
+// Dense cells: compaction of the non-empty ones in cell (= key) order, AC_CELLS cells per CTA (few, so
+// that the thousands of cells of a window spread over many SMs), chained over the CTAs.  The histograms (160 of a row's 200 bytes) are copied by the CTA together, 16 bytes per
 // thread, rows side by side: one thread per row copying its own took 36 us for the 4096 cells of a
 // prefill window, most of it waiting.
 #define AC_THREADS 256
+#define AC_CELLS 64
 __global__ void __launch_bounds__(AC_THREADS) k_agg_rows(int64_t G, AggRowOut o, u64 *state, u64 *total,
                                                          u32 *ticket, int32_t *status, Tail tail) {
   TA_PDL();
   __shared__ u64 tmp[33];
   __shared__ u64 s_excl;
-  __shared__ u32 s_cell[AC_THREADS];
+  __shared__ u32 s_cell[AC_CELLS];
   __shared__ int s_fail, s_tile;
   const int tid = threadIdx.x;
   if (tid == 0) s_tile = (int)atomicAdd(ticket, 1u);
   __syncthreads();
   const int tile = s_tile;
-  const int64_t g = (int64_t)tile * AC_THREADS + tid;
+  const int64_t g = tid < AC_CELLS ? (int64_t)tile * AC_CELLS + tid : G;
   const bool failed = ta_failed(status);
   const u64 c = !failed && g < G ? o.cnt[g] : 0;
   u64 rows;
@@ -440,7 +441,7 @@ __global__ void __launch_bounds__(AC_THREADS) k_agg_rows(int64_t G, AggRowOut o,
       o.g_min[row] = (int64_t)((~o.minc[g]) ^ (1ull << 63));
       o.g_max[row] = (int64_t)(o.maxb[g] ^ (1ull << 63));
     }
-    const uint4 *src = reinterpret_cast<const uint4 *>(o.hist) + (size_t)tile * AC_THREADS * (TA_NBINS / 4);
+    const uint4 *src = reinterpret_cast<const uint4 *>(o.hist) + (size_t)tile * AC_CELLS * (TA_NBINS / 4);
     uint4 *dst = reinterpret_cast<uint4 *>(o.g_hist) + first * (TA_NBINS / 4);
     const int words = (int)rows * (TA_NBINS / 4);
     for (int i = tid; i < words; i += AC_THREADS) {
@@ -799,7 +800,7 @@ ta_status ta_run_aggregate(ta_window *h, uint32_t kind_mask, int value_sel, ta_a
   // (pass, scan, round trip) are worth.  512 windows of 65 k records have 33 M cells, one in
   // twenty of them occupied: 1.85 ms per call dense.
   if (G * 232 <= 8 * h->n_valid + (64ll << 20)) {
-    const int64_t tiles = (G + AC_THREADS - 1) / AC_THREADS;
+    const int64_t tiles = (G + AC_CELLS - 1) / AC_CELLS;
     size_t tb = 4 * Carver::pad((size_t)G * 8) + Carver::pad((size_t)G * TA_NBINS * 4) + Carver::pad((size_t)(tiles + 2) * 8);
     ta_status zs;
     tmpb = ta_zalloc(h, tb, &zs);

@@ -278,18 +278,21 @@ __global__ void __launch_bounds__(128) k_attr_fold_up(StackArr child, int64_t n_
   if (overflow && lane == 0) ta_set_err(status, TA_ERR_DEPTH);
 }
 
-// one warp: start[i] = node[0] (+) ... (+) node[i - 1] for the few nodes of the top level
+// one warp: start[i] = node[0] (+) ... (+) node[i - 1] for the few (at most AT_FAN) nodes of the top
+// level, staged first (a chain of loads from memory took 18 us for 31 of them)
 __global__ void __launch_bounds__(32) k_attr_fold_top(StackArr node, int64_t n, StackArr start,
                                                       int leaf, int32_t *status) {
   TA_PDL();
+  __shared__ StackStage st;
   if (ta_failed(status)) return;
   const int lane = threadIdx.x & 31;
+  stack_stage(node, 0, n, st, 0, lane);
   bool overflow = false;
   WStack acc;
   acc.cnt = 0; acc.reset = 0; acc.e = 0; acc.pos = 0;
-  for (int64_t i = 0; i < n; i++) {
+  for (int i = 0; i < (int)n; i++) {
     stack_store(start, i, acc, lane, leaf != 0);
-    WStack nxt = stack_load(node, i, lane);
+    WStack nxt = stack_staged(st, 0, i, lane);
     wstack_combine(acc, nxt, &overflow);
     acc = nxt;
   }
@@ -341,6 +344,10 @@ struct AttrStack {
   u64 ns[AS_LEVELS];
   int32_t pos[AS_LEVELS];
   u32 cnt[AS_LEVELS];    // kernels; bit 31: k_attr_ops may add more, the row keeps its identities
+  // what the launches of one row add: to the operators of the row (0..31), to the levels (32 + k);
+  // times relative to the row's first kernel
+  int32_t r_first[32 + AS_LEVELS], r_last[32 + AS_LEVELS];
+  u32 r_ns[32 + AS_LEVELS], r_cnt[32 + AS_LEVELS];
 };
 __device__ __forceinline__ i64 shfl_i64(i64 v, int src) { return __shfl_sync(0xffffffffu, v, src); }
 
@@ -377,6 +384,14 @@ __device__ __forceinline__ void attr_pop(const AttrArgs &a, const AttrStack &st,
   __syncwarp();
 }
 
+// kernels of an operator on the stack (one thread)
+__device__ __forceinline__ void attr_level_add(AttrStack &st, int k, u32 cnt, i64 first, i64 last, u64 ns) {
+  st.cnt[k] += cnt;
+  st.first[k] = min(st.first[k], first);
+  st.last[k] = max(st.last[k], last);
+  st.ns[k] += ns;
+}
+
 template <int TILE>
 __global__ void __launch_bounds__(AS_WARPS * 32, AS_MINB) k_attr_resolve(AttrArgs a) {
   TA_PDL();
@@ -392,6 +407,10 @@ __global__ void __launch_bounds__(AS_WARPS * 32, AS_MINB) k_attr_resolve(AttrArg
     attr_fill(a, tile_start, tile_end);
     return;
   }
+  for (int i = lane; i < 32 + AS_LEVELS; i += 32) {
+    st.r_first[i] = INT_MAX; st.r_last[i] = INT_MIN; st.r_ns[i] = 0; st.r_cnt[i] = 0;
+  }
+  __syncwarp();
   int l = tile_lane_search(a.lane_off, a.n_lanes, tile_start);
   int64_t pos = tile_start;
   int depth = 0, carried = 0;  // levels on the stack; of these, the lowest ones come from earlier tiles
@@ -415,23 +434,33 @@ __global__ void __launch_bounds__(AS_WARPS * 32, AS_MINB) k_attr_resolve(AttrArg
     const int64_t lane_end = a.lane_off[l + 1], seg_end = min(lane_end, vend);
     int dmax = 0;
     bool bad = false;
-    // a row's columns are requested while the row in front of it is worked on
-    int kd = 9, nk = 0, kp = 0;
-    i64 ts = 0, en = 0;
-    auto load = [&](int64_t p) {
-      kd = 9;
-      if (p < seg_end) { kd = a.kind[p]; ts = a.ts[p]; en = a.te[p]; nk = a.kol[p]; kp = a.kernel_of[p]; }
+    // A row's columns are requested while the row in front of it is worked on, and so are the times of
+    // its launches' kernels, whose positions come from one row further ahead.  (The join counts
+    // kernels at launches only.)
+    int kd1 = 9, nk1 = 0, nk2 = 0, kp2 = 0;
+    i64 ts1 = 0, en1 = 0, ks1 = 0, ke1 = 0;
+    auto ahead2 = [&](int64_t p) {
+      nk2 = kp2 = 0;
+      if (p < seg_end) { nk2 = a.kol[p]; kp2 = a.kernel_of[p]; }
     };
-    load(pos + lane);
+    auto ahead1 = [&](int64_t p) {
+      kd1 = 9;
+      if (p < seg_end) { kd1 = a.kind[p]; ts1 = a.ts[p]; en1 = a.te[p]; }
+      nk1 = nk2;
+      if (nk1 == 1) { ks1 = a.ts[kp2]; ke1 = a.te[kp2]; }
+    };
+    ahead2(pos + lane);
+    ahead1(pos + lane);
+    ahead2(pos + 32 + lane);
     for (; pos < seg_end; pos += 32) {
       const int64_t p = pos + lane;
-      const bool in = p < seg_end, op = kd == TA_KIND_OP;
-      const i64 e = en, t = e > ts ? ts + 1 : e;
-      const int n_k = kd == TA_KIND_LAUNCH ? nk : 0;
-      i64 ks = 0, ke = 0;
-      if (n_k == 1) { ks = a.ts[kp]; ke = a.te[kp]; }
-      load(p + 32);
-      const u32 ops = __ballot_sync(0xffffffffu, op);
+      const bool in = p < seg_end, op = kd1 == TA_KIND_OP;
+      const bool empty = !(en1 > ts1);
+      const i64 e = en1, t = empty ? e : ts1 + 1, ks = ks1, ke = ke1;
+      const int n_k = nk1;
+      ahead1(p + 32);
+      ahead2(p + 64);
+      const u32 ops = __ballot_sync(0xffffffffu, op), empty_ops = __ballot_sync(0xffffffffu, op && empty);
       // nearest operator of the row
       int q = (ops & lt) ? 31 - __clz((int)(ops & lt)) : -1;
       i64 pe = 0;  // its end
@@ -443,13 +472,16 @@ __global__ void __launch_bounds__(AS_WARPS * 32, AS_MINB) k_attr_resolve(AttrArg
         if (!__any_sync(0xffffffffu, ended)) break;
         if (ended) q = up;
       }
-      // else the stack, from the top
+      // else the stack: the highest of the levels that end at or after the threshold
       int par = q;  // 0..31: record of the row, 32 + k: level k, -1: none
-      bool ask = in && q < 0;
-      for (int k = depth - 1; k >= 0; k--) {
-        if (!__any_sync(0xffffffffu, ask)) break;
-        const i64 ek = st.e[k];
-        if (ask && ek >= t) { par = 32 + k; pe = ek; ask = false; }
+      if (__any_sync(0xffffffffu, in && q < 0) && depth > 0) {
+        int lo = 0, hi = depth;  // levels known to qualify / not known not to
+        while (lo < hi) {
+          const int mid = (lo + hi) >> 1;
+          if (st.e[mid] >= t) lo = mid + 1;
+          else hi = mid;
+        }
+        if (q < 0 && lo > 0) { par = 31 + lo; pe = st.e[lo - 1]; }
       }
       bad |= in && par >= 0 && pe < e;
       // level in the forest: distances to an ancestor, doubled until it is one whose level is known
@@ -462,7 +494,8 @@ __global__ void __launch_bounds__(AS_WARPS * 32, AS_MINB) k_attr_resolve(AttrArg
       }
       if (d > 255) d = 255;
       if (in) dmax = max(dmax, d);
-      // kernels, operator by operator (a row has a handful of operators that own launches)
+      // kernels of the operators: 32-bit atomics on chip, a few operators' worth of neighbours at a
+      // time (a vote and three warp reductions per operator took half of the kernel's instructions)
       u32 cnt = 0;
       i64 first = INT64_MAX, last = INT64_MIN;
       u64 ns = 0;
@@ -471,26 +504,28 @@ __global__ void __launch_bounds__(AS_WARPS * 32, AS_MINB) k_attr_resolve(AttrArg
         const i64 base = shfl_i64(ks, __ffs((int)left) - 1);
         const i64 rs = ks - base, re = ke - base, dur = ke - ks;
         const bool mine = left >> lane & 1u;
-        // times within half a second of the row's first kernel and kernels below 67 ms: 32-bit reductions
+        // times within a second of the row's first kernel and kernels below 67 ms
         const bool near = rs > -(1ll << 30) && re < (1ll << 30) && dur < (1ll << 26);
         if (__all_sync(0xffffffffu, !mine || near)) {
-          while (left) {
-            const int key = __shfl_sync(0xffffffffu, par, __ffs((int)left) - 1);
-            const bool same = mine && par == key;
-            const u32 who = __ballot_sync(0xffffffffu, same);
-            const i64 f = base + __reduce_min_sync(0xffffffffu, same ? (int)rs : INT_MAX);
-            const i64 g = base + __reduce_max_sync(0xffffffffu, same ? (int)re : INT_MIN);
-            const u32 du = __reduce_add_sync(0xffffffffu, same ? (u32)dur : 0u);
-            left &= ~who;
-            if (key < 32) {
-              if (lane == key) { cnt = (u32)__popc(who); first = f; last = g; ns = du; }
-            } else if (lane == 0) {
-              const int k = key - 32;
-              st.cnt[k] += (u32)__popc(who);
-              st.first[k] = min(st.first[k], f);
-              st.last[k] = max(st.last[k], g);
-              st.ns[k] += du;
-            }
+          if (mine) {
+            atomicMin(&st.r_first[par], (int)rs);
+            atomicMax(&st.r_last[par], (int)re);
+            atomicAdd(&st.r_ns[par], (u32)dur);
+            atomicAdd(&st.r_cnt[par], 1u);
+          }
+          __syncwarp();
+          cnt = st.r_cnt[lane];
+          if (cnt) {
+            first = base + st.r_first[lane];
+            last = base + st.r_last[lane];
+            ns = st.r_ns[lane];
+            st.r_first[lane] = INT_MAX; st.r_last[lane] = INT_MIN; st.r_ns[lane] = 0; st.r_cnt[lane] = 0;
+          }
+          for (int k = lane; k < depth; k += 32) {
+            const u32 c = st.r_cnt[32 + k];
+            if (!c) continue;
+            attr_level_add(st, k, c, base + st.r_first[32 + k], base + st.r_last[32 + k], st.r_ns[32 + k]);
+            st.r_first[32 + k] = INT_MAX; st.r_last[32 + k] = INT_MIN; st.r_ns[32 + k] = 0; st.r_cnt[32 + k] = 0;
           }
         } else {
           for (; left; left &= left - 1) {
@@ -500,14 +535,11 @@ __global__ void __launch_bounds__(AS_WARPS * 32, AS_MINB) k_attr_resolve(AttrArg
             if (key < 32) {
               if (lane == key) { cnt++; first = min(first, f); last = max(last, g); ns += (u64)(g - f); }
             } else if (lane == 0) {
-              const int k = key - 32;
-              st.cnt[k]++;
-              st.first[k] = min(st.first[k], f);
-              st.last[k] = max(st.last[k], g);
-              st.ns[k] += (u64)(g - f);
+              attr_level_add(st, key - 32, 1u, f, g, (u64)(g - f));
             }
           }
         }
+        __syncwarp();
       }
       // launches with several kernels (graph replays): k_attr_ops meets their kernels one by one
       for (u32 many = __ballot_sync(0xffffffffu, n_k > 1 && par >= 0); many; many &= many - 1) {
@@ -526,15 +558,26 @@ __global__ void __launch_bounds__(AS_WARPS * 32, AS_MINB) k_attr_resolve(AttrArg
       }
       if (ops) {
         // the stack behind the row: the last operator and those around it, on what is left of the levels
-        u32 open = 0;
         int c = 31 - __clz((int)ops);
-        while (c >= 0 && c < 32) {
-          open |= 1u << c;
-          c = __shfl_sync(0xffffffffu, par, c);
+        const i64 tc = shfl_i64(t, c);
+        u32 open;
+        int keep = 0;
+        if (empty_ops >> c & 1u) {
+          // it is empty: what ends at that instant may lie beside it, not around it; up the chain instead
+          open = 0;
+          while (c >= 0 && c < 32) {
+            open |= 1u << c;
+            c = __shfl_sync(0xffffffffu, par, c);
+          }
+          keep = c >= 32 ? c - 31 : 0;
+        } else {
+          // what still runs when it has begun is around it
+          open = __ballot_sync(0xffffffffu, op && (lane == c || e >= tc));
+          for (int k = lane; k < depth; k += 32) keep += st.e[k] >= tc;
+          keep = depth <= 32 ? __popc(__ballot_sync(0xffffffffu, keep)) : (int)__reduce_add_sync(0xffffffffu, (u32)keep);
         }
-        const int keep = c >= 32 ? c - 31 : 0;
         __syncwarp();  // (the row's zeros and parents are out before levels are written to or replaced)
-        attr_pop(a, st, keep, depth, carried, false);
+        if (keep < depth) attr_pop(a, st, keep, depth, carried, false);
         if (carried > keep) carried = keep;
         const int at = keep + __popc(open & lt);
         if ((open >> lane & 1u) && at < AS_LEVELS) {
@@ -729,7 +772,10 @@ ta_status ta_run_attribute(ta_window *h, ta_attr_summary *out_summary) {
   cudaStream_t st = h->stream;
   // Tiles of 1024 records; of 256 while their stacks are folded in two levels, so that a window of some
   // ten thousand records has work for more than a few SMs (a warp takes a tile).
-  const int per_tile = n <= 256ll * AT_FAN * AT_FAN ? 256 : 1024;
+#ifndef AT_BIG
+#define AT_BIG 1024
+#endif
+  const int per_tile = n <= 256ll * AT_FAN * AT_FAN ? 256 : AT_BIG;
   const int64_t tiles = (n + per_tile - 1) / per_tile;
   size_t keep = 3 * Carver::pad(nn * 4) + Carver::pad(nn) + 3 * Carver::pad(nn * 8) + 256;
   void *kb = ta_dalloc(h, keep);
@@ -781,7 +827,7 @@ ta_status ta_run_attribute(ta_window *h, ta_attr_summary *out_summary) {
   TA_TRY(ta_queue_d2h(h, words, h->d_status, sizeof(words)));
   if (small) TA_TRY(ta_queue_d2h(h, hs.data(), d_sum, W * sizeof(ta_attr_summary)));
   if (n > 0) {
-    ta_launch(per_tile == 256 ? k_attr_agg<1> : k_attr_agg<4>, (unsigned)tiles, AT_THREADS, 0, st, a);
+    ta_launch(per_tile == 256 ? k_attr_agg<1> : k_attr_agg<AT_BIG / 256>, (unsigned)tiles, AT_THREADS, 0, st, a);
     {
       // level 0 = tiles; fold upwards until at most AT_FAN stacks remain, scan those, unfold
       std::vector<StackArr> node(level_n.size()), start(level_n.size());
@@ -799,7 +845,7 @@ ta_status ta_run_attribute(ta_window *h, ta_attr_summary *out_summary) {
       for (size_t k = top; k >= 1; k--)
         ta_launch(k_attr_fold_down, (unsigned)((level_n[k] + 3) / 4), 128, 0, st, node[k - 1], level_n[k - 1], start[k], level_n[k], start[k - 1], k == 1 ? 1 : 0, h->d_status);
     }
-    ta_launch(per_tile == 256 ? k_attr_resolve<256> : k_attr_resolve<1024>, (unsigned)((tiles + AS_WARPS - 1) / AS_WARPS),
+    ta_launch(per_tile == 256 ? k_attr_resolve<256> : k_attr_resolve<AT_BIG>, (unsigned)((tiles + AS_WARPS - 1) / AS_WARPS),
               AS_WARPS * 32, 0, st, a);
     const int64_t sb = (tiles * 4 + 255) / 256;
     ta_launch(k_attr_spill, (unsigned)(sb < 148 * 4 ? sb : 148 * 4), 256, 0, st, a);

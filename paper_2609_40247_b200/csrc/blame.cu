@@ -24,6 +24,7 @@
 
 #define BL_THREADS 256
 #define BL_TILE (BL_THREADS * 4)
+#define BL_LANES 64
 
 struct BlameArgs {
   int64_t n, n_valid, m;  // m = long gaps
@@ -146,19 +147,23 @@ __device__ __forceinline__ void blame_ops(const BlameArgs &a) {
   __shared__ uint16_t s_op[BL_TILE];
   __shared__ int32_t s_dlo[BL_TILE];
   __shared__ uint16_t s_dn[BL_TILE];
+  __shared__ int s_d0;                       // first device lane of the tile's operators, -1: there are several processes
+  __shared__ i64 s_from, s_to;               // earliest start, latest end among them
+  __shared__ int32_t s_lo[BL_LANES], s_hi[BL_LANES];  // per stream: the gaps that can matter to them
   if (ta_failed(a.status)) return;
   const int tid = threadIdx.x;
   const int64_t tile_start = (int64_t)blockIdx.x * BL_TILE;
   if (tile_start >= a.n_valid) return;
   if (tid < 32) {
     const int l = tile_lane_search(a.lane_off, a.n_lanes, tile_start);
-    if (tid == 0) { s_lane0 = l; s_n = 0; s_most = 0; }
+    if (tid == 0) { s_lane0 = l; s_n = 0; s_most = 0; s_d0 = -2; s_from = INT64_MAX; s_to = INT64_MIN; }
   }
   __syncthreads();
   const int l0 = s_lane0;
   const int64_t tile_end = min(tile_start + BL_TILE, a.n_valid);
   if (span_outside_domain(a.lane_domain, a.lane_dom_end, l0, tile_end, 0)) return;
   int l = l0, cur = -1, dlo = 0, dn = 0;
+  i64 from = INT64_MAX, to = INT64_MIN;
   int64_t next_off = a.lane_off[l + 1];
 #pragma unroll
   for (int k = 0; k < BL_TILE / BL_THREADS; k++) {
@@ -181,13 +186,29 @@ __device__ __forceinline__ void blame_ops(const BlameArgs &a) {
     s_dn[i] = (uint16_t)dn;
     s_sum[i] = 0;
     if (dn > s_most) atomicMax(&s_most, dn);
+    if (s_d0 != dlo && atomicCAS(&s_d0, -2, dlo) != -2 && s_d0 != dlo) s_d0 = -1;
+    from = min(from, (i64)a.ts[p]);
+    to = max(to, (i64)a.te[p]);
   }
+  from = (i64)(~warp_reduce(~((u64)from ^ (1ull << 63)), OpMax()) ^ (1ull << 63));
+  to = (i64)(warp_reduce((u64)to ^ (1ull << 63), OpMax()) ^ (1ull << 63));
+  if ((tid & 31) == 0 && from <= to) { atomicMin(&s_from, from); atomicMax(&s_to, to); }
   __syncthreads();
   const int ops = s_n, most = s_most;
+  // Operators of one tile lie close together in time: with one search per stream for all of them, each
+  // has to look among a few gaps only.
+  const bool one = s_d0 >= 0 && most <= BL_LANES;
+  if (one && tid < most) {
+    const int64_t first = a.lane_first[s_d0 + tid], last = a.lane_first[s_d0 + tid + 1];
+    const int64_t lo = gaps_started_before(a, first, last, s_from);
+    s_lo[tid] = (int32_t)(lo > first ? lo - 1 : first);
+    s_hi[tid] = (int32_t)gaps_started_before(a, lo, last, s_to);
+  }
+  if (one) __syncthreads();
   for (int q = tid; q < ops * most; q += BL_THREADS) {
     const int i = q / most, d = q - i * most;  // (a tile nearly always lies in one process: all pairs exist)
     if (d >= s_dn[i]) continue;
-    const int64_t first = a.lane_first[s_dlo[i] + d], last = a.lane_first[s_dlo[i] + d + 1];
+    const int64_t first = one ? s_lo[d] : a.lane_first[s_dlo[i] + d], last = one ? s_hi[d] : a.lane_first[s_dlo[i] + d + 1];
     if (first == last) continue;
     const int64_t p = tile_start + s_op[i];
     const i64 t = gap_time_within(a, first, last, a.ts[p], a.te[p]);

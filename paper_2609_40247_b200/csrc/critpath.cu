@@ -116,10 +116,11 @@ __device__ __forceinline__ int32_t cp_last_ended(const CpArgs &a, int first_dev_
   for (int dl = first_dev_lane; dl >= 0 && dl < a.n_lanes && a.lane_slot[dl] == slot && a.lane_domain[dl] == 1; dl++) {
     int64_t lo = a.lane_off[dl], hi = a.lane_off[dl + 1];  // first position of the lane that ends at / after the limit
     const int64_t begin = lo;
+    if (inclusive) lo = hi;  // no limit: the lane's last record
     while (lo < hi) {
       const int64_t mid = (lo + hi) >> 1;
       const i64 e = a.te[mid];
-      if (inclusive ? e <= limit : e < limit) lo = mid + 1;
+      if (e < limit) lo = mid + 1;
       else hi = mid;
     }
     if (lo > begin) {
@@ -499,7 +500,8 @@ __global__ void __launch_bounds__(256) k_cp_succ(CpArgs a) {
   TA_PDL();
   if (ta_failed(a.status)) return;
   const int64_t id = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (id >= a.n_list) return;
+  if (id >= (a.n_list < 0 ? (int64_t)*a.n_eff : a.n_list)) return;
+  if (a.n_list < 0 && *a.not_ascending) return;  // (the successors would be those of a wrong search)
   a.jump_in[id] = cp_follow(a, a.cross[a.eff_pos[id]], false);
 }
 
@@ -585,13 +587,14 @@ __global__ void __launch_bounds__(256) k_cp_enter(CpArgs a) {
   TA_PDL();
   if (ta_failed(a.status)) return;
   const int64_t id = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (id >= a.n_list || !a.mark[id]) return;
+  if (a.gate && !*a.gate) return;
+  if (id >= (a.n_list < 0 ? (int64_t)*a.n_eff : a.n_list) || !a.mark[id]) return;
   cp_follow(a, a.cross[a.eff_pos[id]], true);
 }
 
-// The whole chain in one CTA when the list is short: every step above for all of it, a block barrier
-// where the launches of the many-CTA form are (twelve rounds of doubling are twelve launches, and the
-// list's length would have to be fetched before them).  Reports through *chained whether it did.
+// The doubling in one CTA when the list is short: a block barrier where the launches of the many-CTA
+// form are (twelve rounds are twelve launches, and the list's length would have to be fetched before
+// them).  Reports through *chained whether it did.
 #define CP_CHAIN_MAX 8192    // waits listed: 72 KB of shared memory, and eight per thread and round
 #define CP_CHAIN_SLOTS 1024  // processes, one thread each
 __global__ void __launch_bounds__(1024) k_cp_chain(CpArgs a, u32 *chained) {
@@ -603,7 +606,7 @@ __global__ void __launch_bounds__(1024) k_cp_chain(CpArgs a, u32 *chained) {
   if (ta_failed(a.status) || m > CP_CHAIN_MAX || *a.not_ascending) return;
   const int tid = threadIdx.x;
   for (u32 i = tid; i < m; i += blockDim.x) {
-    jump[0][i] = cp_follow(a, a.cross[a.eff_pos[i]], false);
+    jump[0][i] = a.jump_in[i];
     mark[i] = 0;
   }
   __syncthreads();
@@ -622,8 +625,7 @@ __global__ void __launch_bounds__(1024) k_cp_chain(CpArgs a, u32 *chained) {
     cur ^= 1;
     __syncthreads();
   }
-  for (u32 i = tid; i < m; i += blockDim.x)
-    if (mark[i]) cp_follow(a, a.cross[a.eff_pos[i]], true);
+  for (u32 i = tid; i < m; i += blockDim.x) a.mark[i] = mark[i];
   if (tid == 0) *chained = 1u;
 }
 
@@ -805,7 +807,7 @@ ta_status ta_run_critpath(ta_window *h, ta_critpath_result *out, ta_critpath_sum
   size_t tb = Carver::pad((size_t)nn) + 6 * Carver::pad((size_t)nn * 4) + Carver::pad((size_t)(n_lanes + 1) * 4) +
               2 * Carver::pad((size_t)tiles * 8) + Carver::pad(64) + Carver::pad((size_t)n_slots * 8) +
               Carver::pad((size_t)n_slots * 4) + Carver::pad((size_t)n_slots * CP_ACC * 8) +
-              scan_temp_bytes(n_slots) + 1024;
+              scan_temp_bytes(n_slots) + CP_CHAIN_MAX * 5 + 1024;
   void *tmpb = ta_dalloc(h, tb);
   if (!tmpb) return TA_ERR_OOM;
   Carver ct(tmpb);
@@ -816,6 +818,8 @@ ta_status ta_run_critpath(ta_window *h, ta_critpath_result *out, ta_critpath_sum
   a.prev_node = ct.take<int32_t>(nn);
   a.head = ct.take<int32_t>(nn);
   a.eff_pos = ct.take<u32>(nn);
+  int32_t *list_jump = ct.take<int32_t>(CP_CHAIN_MAX);
+  uint8_t *list_mark = ct.take<uint8_t>(CP_CHAIN_MAX);
   // zeroed block
   char *zb = ct.base + ct.off;
   a.st_a = ct.take<u64>(tiles); a.st_b = ct.take<u64>(tiles);
@@ -907,7 +911,13 @@ ta_status ta_run_critpath(ta_window *h, ta_critpath_result *out, ta_critpath_sum
     if (!a.use_sort && n_slots <= CP_CHAIN_SLOTS) {
       constexpr int smem = CP_CHAIN_MAX * 9;
       TA_CHECK_CUDA(h, cudaFuncSetAttribute(k_cp_chain, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+      a.n_list = -1;  // (not known yet)
+      a.jump_in = list_jump;
+      a.mark = list_mark;
+      a.gate = chained;
+      ta_launch(k_cp_succ, CP_CHAIN_MAX / 256, 256, 0, st, a);
       ta_launch(k_cp_chain, 1, 1024, smem, st, a, chained);
+      ta_launch(k_cp_enter, CP_CHAIN_MAX / 256, 256, 0, st, a);
       TA_TRY(cp_rows(true));
       if (words[ST_ERR]) break;
       if (words3[2]) { done = true; break; }
@@ -925,6 +935,7 @@ ta_status ta_run_critpath(ta_window *h, ta_critpath_result *out, ta_critpath_sum
   void *lb = nullptr;
   if (!done && !words[ST_ERR]) {
     a.n_list = (int64_t)n_list;
+    a.gate = nullptr;
     const int64_t nl = n_list > 0 ? n_list : 1;
     lb = ta_dalloc(h, 2 * Carver::pad((size_t)nl * 4) + Carver::pad((size_t)nl) + 256);
     if (!lb) return TA_ERR_OOM;

@@ -26,10 +26,10 @@
 #endif
 #define GP_TILE (GP_THREADS * GP_ITEMS)
 #ifndef GR_MINB
-#define GR_MINB 6
+#define GR_MINB 5
 #endif
 #ifndef GR_ROWS
-#define GR_ROWS 32
+#define GR_ROWS 12
 #endif
 // lanes of a tile whose statistics are folded on chip: in a batch of many windows a lane is a
 // thousand records or so and a tile meets several (a batch of 512 windows of 65 k records: 395 us
@@ -542,8 +542,8 @@ ta_status ta_run_gaps(ta_window *h, int64_t min_gap, ta_gap_result *out) {
     if (tiles > 0 && scan) {
       ta_launch(k_gaps, (unsigned)tiles, GP_THREADS, 0, st, a, ta_tail(h, tiles));
     } else if (tiles > 0) {
-      // rows per warp: 32 (a thousand records share a warp's set-up and its flush), fewer while that
-      // would leave SMs without work
+      // rows per warp: 12 (66.8 M records: 292 us; 32: 383, 8: 319), fewer while that would leave SMs
+      // without work
       int64_t rows = n / 32 / (148 * 16);
       rows = rows < 4 ? 4 : rows > GR_ROWS ? GR_ROWS : rows;
       const int64_t per_cta = rows * GP_THREADS, grid = (n + per_cta - 1) / per_cta;

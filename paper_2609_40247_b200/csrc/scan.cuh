@@ -173,7 +173,10 @@ __device__ __forceinline__ void store8_i32(int32_t *col, int64_t p0, int64_t n, 
 template <int IT>
 __device__ __forceinline__ void loadn_i16(const int16_t *col, int64_t p0, int64_t n, int16_t fill, int16_t *v) {
   if (IT == 8) { load8_i16(col, p0, n, fill, v); return; }
-  if (IT == 1) { v[0] = p0 < n ? col[p0] : fill; return; }
+  if (IT <= 2) {
+    for (int j = 0; j < IT; j++) v[j] = p0 + j < n ? col[p0 + j] : fill;
+    return;
+  }
   if (p0 + IT <= n) {
     const uint2 q = *reinterpret_cast<const uint2 *>(col + p0);
     const int16_t *hq = reinterpret_cast<const int16_t *>(&q);
@@ -186,7 +189,10 @@ __device__ __forceinline__ void loadn_i16(const int16_t *col, int64_t p0, int64_
 }
 template <int IT>
 __device__ __forceinline__ void loadn_i64(const int64_t *col, int64_t p0, int64_t n, i64 *v) {
-  if (IT == 1) { v[0] = p0 < n ? col[p0] : 0; return; }
+  if (IT <= 2) {
+    for (int j = 0; j < IT; j++) v[j] = p0 + j < n ? col[p0 + j] : 0;
+    return;
+  }
   if (p0 + IT <= n) {
     const longlong2 *ps = reinterpret_cast<const longlong2 *>(col + p0);
 #pragma unroll
