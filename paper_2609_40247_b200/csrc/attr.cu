@@ -5,8 +5,7 @@
 //
 // In canonical order (ts_start ascending, ts_end descending) a properly nested
 // host lane has a simple structure: the innermost encloser of record i is the
-// nearest earlier OP that is still running when i starts.  Tiles of 1024 records
-// (256 of a small window), no kernel ever waits for another CTA:
+// nearest earlier OP that is still running when i starts.  Tiles of 256 to 1024 records, no kernel ever waits for another CTA:
 //   k_attr_agg     per tile, the stack of OPs that are still undominated at the
 //                  tile's end (at most TA_MAX_DEPTH + 1 entries when nesting is
 //                  legal);
@@ -19,7 +18,8 @@
 //                  operator are added up on the way, from the launches inside it,
 //                  and all columns of the operator are written once, with the zeros of
 //                  all other rows;
-//   k_attr_spill   what a tile owes to operators of earlier tiles is added to their rows.
+//   k_attr_ops     device records inherit the operator of their launch; what a tile owes to
+//                  operators of earlier tiles is added to their rows.
 // Partial overlap is detected on the way: that nearest running OP must also
 // cover i's end.
 // HBM-bound by design: 26 B read per host record, 16 B per kernel (nearly sequential), 33 B
@@ -65,6 +65,7 @@ struct AttrArgs {
   i64 *op_first, *op_last, *op_ns;
   struct AttrSpill *spill;   // what tiles owe to operators of earlier tiles
   u32 *n_spill;
+  unsigned spill_blocks;     // k_attr_ops: so many CTAs in front work through that list
 };
 struct AttrSpill {
   int32_t pos, cnt;
@@ -104,92 +105,60 @@ __device__ __forceinline__ void wstack_combine(const WStack &ear, WStack &acc, b
 
 
 // ---- kernel 1: the stack each tile leaves behind --------------------------------
-template <int ITEMS>  // records per thread
+// The operators of the tile's last lane that end no earlier than every later one.  A warp takes a
+// tile, from its last row of 32 records to its first; nearly every row but the last is behind what
+// later rows have raised the bar to, and costs its loads and one vote.  (A CTA per tile, with block
+// barriers around its suffix maximum, took 170 us of 66.8 M records.)
+template <int TILE>
 __global__ void __launch_bounds__(AT_THREADS) k_attr_agg(AttrArgs a) {
   TA_PDL();
-  constexpr int TILE = AT_THREADS * ITEMS;
-  __shared__ i64 wmax[AT_THREADS / 32];
-  __shared__ i64 s_e[AT_CAP];
-  __shared__ int32_t s_pos[AT_CAP];
-  __shared__ int s_raw, s_lane1;
   if (ta_failed(a.status)) return;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int tile = blockIdx.x;
-  const int64_t tile_start = (int64_t)tile * TILE;
-  const int64_t p0 = tile_start + (int64_t)tid * ITEMS;
-  const int64_t plast = min(tile_start + TILE, a.n_valid) - 1;
-  if (tid == 0) s_raw = 0;
-  if (warp == 0) {
-    int l = -1;
-    if (plast >= tile_start) l = tile_lane_search(a.lane_off, a.n_lanes, plast);
-    if (lane == 0) s_lane1 = l;
-  }
-  int16_t kd[ITEMS];
-  loadn_i16<ITEMS>(a.kind, p0, a.n, 9, kd);
-  __syncthreads();
-  const int lane1 = s_lane1;
-  if (lane1 < 0 || a.lane_domain[lane1] != 0) {
-    if (tid == 0) a.agg_meta[tile] = 1 << 8;  // nothing carried past a device lane
+  const int lane = threadIdx.x & 31;
+  const int64_t tile = (int64_t)blockIdx.x * (AT_THREADS / 32) + (threadIdx.x >> 5);
+  if (tile >= a.n_tiles) return;
+  const int64_t tile_start = tile * TILE, vend = min(tile_start + TILE, a.n_valid);
+  const int l = vend > tile_start ? tile_lane_search(a.lane_off, a.n_lanes, vend - 1) : -1;
+  if (l < 0 || a.lane_domain[l] != 0) {
+    if (lane == 0) a.agg_meta[tile] = 1 << 8;  // nothing carried past a device lane
     return;
   }
-  const int64_t seg_begin = a.lane_off[lane1];  // first record of the tile's last lane
-  unsigned opmask = 0;
+  const int64_t seg = a.lane_off[l], from = max(seg, tile_start);
+  i64 bar = INT64_MIN;  // latest end so far
+  int cnt = 0;
+  i64 my_e = 0;         // entry `lane` of the stack, innermost first
+  int32_t my_pos = 0;
+  constexpr int AHEAD = 4;  // rows whose columns are in flight
+  for (int64_t hi = vend; hi > from; hi -= 32 * AHEAD) {
+    i64 e[AHEAD];
 #pragma unroll
-  for (int j = 0; j < ITEMS; j++)
-    if (kd[j] == TA_KIND_OP && p0 + j <= plast && p0 + j >= seg_begin) opmask |= 1u << j;
-  i64 en[ITEMS];
-#pragma unroll
-  for (int j = 0; j < ITEMS; j++) en[j] = INT64_MIN;
-  i64 m8 = INT64_MIN;
-  if (opmask) {
-    i64 t[ITEMS];
-    loadn_i64<ITEMS>(a.te, p0, a.n, t);
-#pragma unroll
-    for (int j = 0; j < ITEMS; j++)
-      if (opmask & (1u << j)) { en[j] = t[j]; m8 = m8 > t[j] ? m8 : t[j]; }
-  }
-  // largest OP end among the threads after this one
-  i64 after = INT64_MIN;
-  {
-    i64 v = m8;  // inclusive suffix max inside the warp
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      i64 t = __shfl_down_sync(0xffffffffu, v, o);
-      if (lane + o < 32) v = v > t ? v : t;
+    for (int r = 0; r < AHEAD; r++) {
+      const int64_t p = hi - 32 * (r + 1) + lane;
+      e[r] = p >= from && a.kind[p] == TA_KIND_OP ? (i64)a.te[p] : INT64_MIN;
     }
-    if (lane == 0) wmax[warp] = v;
-    i64 nxt = __shfl_down_sync(0xffffffffu, v, 1);
-    after = lane < 31 ? nxt : INT64_MIN;
-    __syncthreads();
-    for (int w = warp + 1; w < AT_THREADS / 32; w++) after = after > wmax[w] ? after : wmax[w];
-  }
-  i64 sfx = after;
 #pragma unroll
-  for (int j = ITEMS - 1; j >= 0; j--) {
-    if (opmask & (1u << j)) {
-      if (en[j] >= sfx) {  // equal ends nest: the earlier OP encloses the later one
-        int o = atomicAdd(&s_raw, 1);
-        if (o < AT_CAP) { s_e[o] = en[j]; s_pos[o] = (int32_t)(p0 + j); }
+    for (int r = 0; r < AHEAD; r++) {
+      // equal ends nest: the earlier operator encloses the later one
+      u32 m = __ballot_sync(0xffffffffu, e[r] >= bar && e[r] != INT64_MIN);
+      while (m) {
+        const int src = 31 - __clz((int)m);
+        m &= ~(1u << src);
+        const i64 es = __shfl_sync(0xffffffffu, e[r], src);
+        if (es < bar) continue;
+        bar = es;
+        if (lane == cnt) { my_e = es; my_pos = (int32_t)(hi - 32 * (r + 1) + src); }
+        cnt++;
       }
-      sfx = sfx > en[j] ? sfx : en[j];
     }
   }
-  __syncthreads();
-  if (warp == 0) {
-    const int raw = s_raw;
-    const int cnt = raw > AT_CAP ? AT_CAP : raw;
-    if (raw > AT_CAP && lane == 0) ta_set_err(a.status, TA_ERR_DEPTH);
-    // survivors were appended in arbitrary order: rank them by position
-    const i64 me = lane < cnt ? s_e[lane] : 0;
-    const int32_t mp = lane < cnt ? s_pos[lane] : INT_MAX;
-    int rank = 0;
-    for (int k = 0; k < cnt; k++) rank += __shfl_sync(0xffffffffu, mp, k) < mp ? 1 : 0;
-    if (lane < cnt) {
-      a.agg_e[(size_t)tile * AT_CAP + rank] = me;
-      a.agg_pos[(size_t)tile * AT_CAP + rank] = mp;
-    }
-    if (lane == 0) a.agg_meta[tile] = cnt | ((seg_begin >= tile_start ? 1 : 0) << 8);
+  if (cnt > AT_CAP) {  // the outermost ones are lost: nesting this deep is reported anyway
+    if (lane == 0) ta_set_err(a.status, TA_ERR_DEPTH);
+    cnt = AT_CAP;
   }
+  if (lane < cnt) {
+    a.agg_e[(size_t)tile * AT_CAP + (cnt - 1 - lane)] = my_e;
+    a.agg_pos[(size_t)tile * AT_CAP + (cnt - 1 - lane)] = my_pos;
+  }
+  if (lane == 0) a.agg_meta[tile] = cnt | ((seg >= tile_start ? 1 : 0) << 8);
 }
 
 // ---- kernel 2: the stack open at the start of every tile --------------------------
@@ -627,11 +596,9 @@ __device__ __forceinline__ void attr_row_add(const AttrArgs &a, int32_t r, int c
   atomicMin(&a.op_first[r], first);
   atomicMax(&a.op_last[r], last);
 }
-__global__ void __launch_bounds__(256) k_attr_spill(AttrArgs a) {
-  TA_PDL();
-  if (ta_failed(a.status)) return;
+__device__ __forceinline__ void attr_spill(const AttrArgs &a) {
   const u32 m = *a.n_spill;
-  for (u32 i = blockIdx.x * 256 + threadIdx.x; i < m; i += gridDim.x * 256) {
+  for (u32 i = blockIdx.x * AT_THREADS + threadIdx.x; i < m; i += a.spill_blocks * AT_THREADS) {
     const AttrSpill x = a.spill[i];
     attr_row_add(a, x.pos, x.cnt, x.first, x.last, x.ns);
   }
@@ -651,8 +618,12 @@ __global__ void __launch_bounds__(AT_THREADS, AT_OPS_MINB) k_attr_ops(AttrArgs a
   __shared__ u64 red[3][AT_THREADS / 32];
   __shared__ int s_lane0, s_lane1;
   if (ta_failed(a.status)) return;
+  if (blockIdx.x < a.spill_blocks) {
+    attr_spill(a);
+    return;
+  }
   const int tid = threadIdx.x, lane = tid & 31;
-  const int64_t tile_start = (int64_t)blockIdx.x * AT_OPS_TILE;
+  const int64_t tile_start = (int64_t)(blockIdx.x - a.spill_blocks) * AT_OPS_TILE;
   const int64_t p0 = tile_start + (int64_t)tid * IT;
   if (tid == 0) { s_lane0 = -1; s_lane1 = -1; }
   __syncthreads();
@@ -770,12 +741,11 @@ ta_status ta_run_attribute(ta_window *h, ta_attr_summary *out_summary) {
   const int64_t n = h->n, nn = n > 0 ? n : 1;
   const int W = h->W;
   cudaStream_t st = h->stream;
-  // Tiles of 1024 records; of 256 while their stacks are folded in two levels, so that a window of some
-  // ten thousand records has work for more than a few SMs (a warp takes a tile).
-#ifndef AT_BIG
-#define AT_BIG 1024
-#endif
-  const int per_tile = n <= 256ll * AT_FAN * AT_FAN ? 256 : AT_BIG;
+  // A warp takes a tile.  256 records while the stacks are folded in two levels, so that a window of some
+  // ten thousand records has work for more than a few SMs; 1024 from ten rounds of the 148 * 32 warps
+  // k_attr_resolve keeps on the chip (66.8 M records: 750 us instead of 782, and half the stacks); 512
+  // between, where the last round's slowest warps show (16.8 M: 263 us instead of 342).
+  const int per_tile = n <= 256ll * AT_FAN * AT_FAN ? 256 : n <= 10ll * 148 * 32 * 1024 ? 512 : 1024;
   const int64_t tiles = (n + per_tile - 1) / per_tile;
   size_t keep = 3 * Carver::pad(nn * 4) + Carver::pad(nn) + 3 * Carver::pad(nn * 8) + 256;
   void *kb = ta_dalloc(h, keep);
@@ -827,7 +797,8 @@ ta_status ta_run_attribute(ta_window *h, ta_attr_summary *out_summary) {
   TA_TRY(ta_queue_d2h(h, words, h->d_status, sizeof(words)));
   if (small) TA_TRY(ta_queue_d2h(h, hs.data(), d_sum, W * sizeof(ta_attr_summary)));
   if (n > 0) {
-    ta_launch(per_tile == 256 ? k_attr_agg<1> : k_attr_agg<AT_BIG / 256>, (unsigned)tiles, AT_THREADS, 0, st, a);
+    const unsigned wblocks = (unsigned)((tiles + AS_WARPS - 1) / AS_WARPS);
+    ta_launch(per_tile == 256 ? k_attr_agg<256> : per_tile == 512 ? k_attr_agg<512> : k_attr_agg<1024>, wblocks, AT_THREADS, 0, st, a);
     {
       // level 0 = tiles; fold upwards until at most AT_FAN stacks remain, scan those, unfold
       std::vector<StackArr> node(level_n.size()), start(level_n.size());
@@ -845,11 +816,11 @@ ta_status ta_run_attribute(ta_window *h, ta_attr_summary *out_summary) {
       for (size_t k = top; k >= 1; k--)
         ta_launch(k_attr_fold_down, (unsigned)((level_n[k] + 3) / 4), 128, 0, st, node[k - 1], level_n[k - 1], start[k], level_n[k], start[k - 1], k == 1 ? 1 : 0, h->d_status);
     }
-    ta_launch(per_tile == 256 ? k_attr_resolve<256> : k_attr_resolve<AT_BIG>, (unsigned)((tiles + AS_WARPS - 1) / AS_WARPS),
-              AS_WARPS * 32, 0, st, a);
-    const int64_t sb = (tiles * 4 + 255) / 256;
-    ta_launch(k_attr_spill, (unsigned)(sb < 148 * 4 ? sb : 148 * 4), 256, 0, st, a);
-    const unsigned ob = (unsigned)((n + AT_OPS_TILE - 1) / AT_OPS_TILE);
+    ta_launch(per_tile == 256 ? k_attr_resolve<256> : per_tile == 512 ? k_attr_resolve<512> : k_attr_resolve<1024>, wblocks, AS_WARPS * 32, 0, st, a);
+    // (a tile owes something to few operators of earlier ones, as a rule)
+    const int64_t sb = (tiles * 2 + AT_THREADS - 1) / AT_THREADS;
+    a.spill_blocks = (unsigned)(sb < 148 * 2 ? sb : 148 * 2);
+    const unsigned ob = a.spill_blocks + (unsigned)((n + AT_OPS_TILE - 1) / AT_OPS_TILE);
     if (h->multi_launch) ta_launch(k_attr_ops<true>, ob, AT_THREADS, 0, st, a);
     else ta_launch(k_attr_ops<false>, ob, AT_THREADS, 0, st, a);
     const int64_t fb = (tiles * AT_CAP + 255) / 256;

@@ -103,8 +103,10 @@ __device__ __forceinline__ void sol_flush(SolAcc &acc, ta_sol_summary *row, u64 
   acc.clear();
 }
 
-// Persistent CTAs, each over a contiguous range of tiles.
-__device__ __forceinline__ void operator_sol(const SolArgs &a, int64_t n_tiles, int64_t tiles_per_cta) {
+// Persistent CTAs.  stride 1: each over a contiguous range of tiles (windows follow each other); else
+// every stride-th tile (one window: host and device lanes, whose tiles cost very different amounts,
+// are then spread evenly).
+__device__ __forceinline__ void operator_sol(const SolArgs &a, int64_t n_tiles, int64_t tiles_per_cta, int64_t stride) {
   __shared__ int s_lane0, s_lane1;
   __shared__ u64 red[7][SO_THREADS / 32];
   if (ta_failed(a.status)) return;
@@ -112,9 +114,9 @@ __device__ __forceinline__ void operator_sol(const SolArgs &a, int64_t n_tiles, 
   SolAcc acc;
   acc.clear();
   int cw = -1;  // window the registers hold sums of (the same in every thread)
-  const int64_t t_begin = (int64_t)blockIdx.x * tiles_per_cta;
-  const int64_t t_end = min(t_begin + tiles_per_cta, n_tiles);
-  for (int64_t tile = t_begin; tile < t_end; tile++) {
+  const int64_t t_begin = stride > 1 ? (int64_t)blockIdx.x : (int64_t)blockIdx.x * tiles_per_cta;
+  const int64_t t_end = stride > 1 ? n_tiles : min(t_begin + tiles_per_cta, n_tiles);
+  for (int64_t tile = t_begin; tile < t_end; tile += stride) {
     const int64_t tile_start = tile * SO_TILE;
     const int64_t p0 = tile_start + (int64_t)tid * SO_ITEMS;
     const int64_t valid_end = min(tile_start + SO_TILE, a.n_valid);
@@ -226,9 +228,9 @@ __device__ __forceinline__ void operator_sol(const SolArgs &a, int64_t n_tiles, 
 }
 
 __global__ void __launch_bounds__(SO_THREADS) k_operator_sol(SolArgs a, int64_t n_tiles, int64_t tiles_per_cta,
-                                                             Tail tail) {
+                                                             int64_t stride, Tail tail) {
   TA_PDL();
-  operator_sol(a, n_tiles, tiles_per_cta);
+  operator_sol(a, n_tiles, tiles_per_cta, stride);
   run_tail(tail);
 }
 
@@ -275,7 +277,8 @@ ta_status ta_run_sol(ta_window *h, const double *flops, const double *bytes, int
     const int64_t per = (n_tiles + ctas - 1) / ctas;
     const int64_t grid = (n_tiles + per - 1) / per;
     const Tail tail = W * sizeof(ta_sol_summary) <= 4096 ? ta_tail(h, grid) : Tail();
-    ta_launch(k_operator_sol, (unsigned)grid, SO_THREADS, 0, st, a, n_tiles, per, tail);
+    ta_launch(k_operator_sol, (unsigned)grid, SO_THREADS, 0, st, a, n_tiles, per,
+              W == 1 ? grid : (int64_t)1, tail);
     TA_CHECK_CUDA(h, cudaGetLastError());
   }
   TA_TRY(ta_sync_fetch(h));

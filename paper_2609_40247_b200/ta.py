@@ -319,7 +319,6 @@ class _Handle:
             self.ptr = _vp()
         if self.chunk:
             self.lib.ta_chunk_close(self.chunk)
-            _torch_release(self.block, None)
             self.chunk = self.block = None
 
     def __del__(self):
@@ -360,13 +359,10 @@ class _Blocks:
             if lo <= ptr and ptr + nbytes <= hi:
                 return _part(t, ptr - lo, nbytes)
         h = self.handle
-        if h.block is not None and h.block <= ptr < h.block + h.block_bytes:
-            lo, size = h.block, h.block_bytes
-        else:
-            base, room = _vp(), ctypes.c_uint64()
-            if h.lib.ta_block_of(h.ptr, ptr, ctypes.byref(base), ctypes.byref(room)) != 0:
-                raise ValueError("not a result of an open window")
-            lo, size = base.value, room.value
+        base, room = _vp(), ctypes.c_uint64()
+        if h.lib.ta_block_of(h.ptr, ptr, ctypes.byref(base), ctypes.byref(room)) != 0:
+            raise ValueError("not a result of an open window")
+        lo, size = base.value, room.value
         wrap, part = _views()
         self.last = (lo, lo + size, wrap(lo, size, h.device, h))
         self.known.append(self.last)
@@ -667,13 +663,23 @@ class Window:
         self._handle.callbacks = env.alloc, env.release = _ALLOC_T(_alloc), _RELEASE_T(_release)
 
     def _take_chunk(self, env):
+        import torch
+        _views()
         h = self._handle
         size = CHUNK_BYTES_FIXED + self.n * CHUNK_BYTES_PER_RECORD
-        block = _torch_alloc(size, env.ctx)
-        if not block:
-            return
-        h.chunk = h.lib.ta_chunk_open(block, size, _torch_alloc, _torch_release, env.ctx)
-        h.block, h.block_bytes = block, size
+        try:
+            if torch.cuda.current_device() == h.device and torch.cuda.current_stream() == self.torch_stream:
+                t = torch.empty(size, dtype=torch.uint8, device="cuda")
+            else:
+                with torch.cuda.stream(self.torch_stream):
+                    t = torch.empty(size, dtype=torch.uint8, device=f"cuda:{h.device}")
+        except torch.cuda.OutOfMemoryError:
+            return  # piece by piece, as far as it goes
+        base = t.data_ptr()
+        h.chunk = h.lib.ta_chunk_open(base, size, _torch_alloc, _torch_release, env.ctx)
+        h.block = t
+        self._blocks.last = (base, base + size, t)
+        self._blocks.known.append(self._blocks.last)
         env.alloc, env.release, env.ctx = h.lib.chunk_alloc, h.lib.chunk_release, h.chunk
 
     def inject_device_error(self, code: int) -> None:
