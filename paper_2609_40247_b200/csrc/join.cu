@@ -31,7 +31,7 @@ struct JoinArgs {
   int n_lanes;
   const int16_t *kind;
   const int64_t *corr, *ts, *te;
-  const int32_t *lane_off, *lane_slot, *lane_window, *lane_dom_end;
+  const int32_t *lane_off, *lane_slot, *lane_window, *lane_dom_end, *lane_dom_next;
   const int16_t *lane_domain;
   // per slot (window * n_pids + pid rank)
   i64 *slot_min, *slot_max;       // corr range of LAUNCH records
@@ -130,17 +130,18 @@ __global__ void __launch_bounds__(JN_THREADS) k_join_build(JoinArgs a) {
 }
 
 // ---- pass 2: probes ----------------------------------------------------------
-// 256 threads x JP_ITEMS consecutive positions; every output column is written once.  The kernel waits
-// on its gathers: four records per thread and four CTAs per SM (64 registers, no spills) hide more of
-// that than eight and three (66.8 M records: 1.06 -> 1.00 ms).
+// A warp takes so many rows of 32 records, every row of ONE lane: window, process and table range are
+// the same for the whole row, and no warp waits for another.  The kernel waits on its gathers, a
+// chain of three (columns, table, launch times), so a warp works on JP_ROWS rows at a time and has the
+// columns of the next JP_ROWS on their way meanwhile.  (A CTA per 1024 records, lanes walked by every
+// thread, two block barriers at the start: 1035 us of 66.8 M records, half of it in those waits.)
 #define JP_THREADS 256
 #ifndef JP_MINB
-#define JP_MINB 4
+#define JP_MINB 3
 #endif
-#ifndef JP_ITEMS
-#define JP_ITEMS 4
+#ifndef JP_ROWS
+#define JP_ROWS 3
 #endif
-#define JP_TILE (JP_THREADS * JP_ITEMS)
 
 // adds a group of probes to the row of their window
 __device__ __forceinline__ void join_emit(ta_join_summary *sm, const u64 *t) {
@@ -156,147 +157,166 @@ __device__ __forceinline__ void join_emit(ta_join_summary *sm, const u64 *t) {
   atomicMax((i64 *)&sm->max_queue, (i64)t[6]);
 }
 
+struct ProbeRow {
+  i64 c, s;
+  bool probe;
+};
+__device__ __forceinline__ void probe_row(const JoinArgs &a, u32 q, u32 end, ProbeRow &x) {
+  x.probe = false;
+  x.c = x.s = 0;
+  if (q < end) {
+    // all three requested together: one round of memory latency less than loading the ids only where the kinds ask for them
+    const int kd = a.kind[q];
+    x.c = a.corr[q];
+    x.s = a.ts[q];
+    x.probe = kd == TA_KIND_KERNEL || kd == TA_KIND_MEMCPY;
+  }
+}
+
 template <bool DIRECT>
-__global__ void __launch_bounds__(JP_THREADS, JP_MINB) k_join_probe(JoinArgs a) {
+__global__ void __launch_bounds__(JP_THREADS, JP_MINB) k_join_probe(JoinArgs a, int rows) {
   TA_PDL();
   __shared__ u64 red[7][JP_THREADS / 32];
-  __shared__ int s_lane0, s_lane1;
+  __shared__ int red_w[JP_THREADS / 32];
   if (ta_failed(a.status)) return;
-  const int tid = threadIdx.x, lane = tid & 31;
-  const int64_t tile_start = (int64_t)blockIdx.x * JP_TILE;
-  constexpr int IT = JP_ITEMS;
-  const int64_t p0 = tile_start + (int64_t)tid * IT;
-  if (tid == 0) { s_lane0 = -1; s_lane1 = -1; }
-  __syncthreads();
-  if (tid < 32 && tile_start < a.n_valid && a.n_lanes > 0) {
-    int l = tile_lane_search(a.lane_off, a.n_lanes, tile_start);
-    if (lane == 0) s_lane0 = l;
-  }
-  __syncthreads();
-  const int l0 = s_lane0;
-  // A tile of host lanes holds no probe: nothing to read, the three outputs are -1 / 0 / 0.
-  if (l0 >= 0 && span_outside_domain(a.lane_domain, a.lane_dom_end, l0, min(tile_start + JP_TILE, a.n_valid), 1)) {
-    int32_t lo0[IT];
-    i64 z[IT];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const u32 n = (u32)a.n, nv = (u32)a.n_valid;
+  const u64 first = ((u64)blockIdx.x * (JP_THREADS / 32) + warp) * (u32)rows * 32;
+  const u32 begin = (u32)min(first, (u64)n), end = (u32)min(first + (u32)rows * 32, (u64)n), vend = min(end, nv);
+  // probes and matches; latencies and delays summed; largest latency, largest complement, largest delay
+  u32 n_probe = 0, n_match = 0;
+  u64 acc[5] = {0, 0, 0, 0, 0};
+  int cur = -1;  // window they are of
+  auto fold = [&](u64 *t) {
+    t[0] = __reduce_add_sync(0xffffffffu, n_probe);
+    t[1] = __reduce_add_sync(0xffffffffu, n_match);
+    t[2] = warp_reduce(acc[0], OpAdd());
+    t[3] = warp_reduce(acc[1], OpAdd());
 #pragma unroll
-    for (int j = 0; j < IT; j++) { lo0[j] = -1; z[j] = 0; }
-    storen_i32<IT>(a.launch_of, p0, a.n, lo0);
-    storen_i64<IT>(a.latency, p0, a.n, z);
-    storen_i64<IT>(a.qdelay, p0, a.n, z);
-    return;
-  }
-  // kinds, correlation ids and start times are requested together: one round of memory
-  // latency less than loading the ids only where the kinds ask for them
-  int16_t kd[IT];
-  i64 c[IT], s[IT];
-  loadn_i16<IT>(a.kind, p0, a.n, 0, kd);
-  loadn_i64<IT>(a.corr, p0, a.n, c);
-  loadn_i64<IT>(a.ts, p0, a.n, s);
-  unsigned pm = 0;  // probes among the thread's records
+    for (int k = 4; k < 7; k++) t[k] = warp_reduce(acc[k - 2], OpMax());
+  };
+  int l = begin < vend ? tile_lane_search(a.lane_off, a.n_lanes, begin) : 0;
+  for (u32 p = begin; p < vend;) {
+    if (a.lane_domain[l] != 1) {  // host lanes hold no probe: the three outputs are -1 / 0 / 0
+      const u32 e = min((u32)a.lane_dom_end[l], vend);
+      for (u32 q = p + lane; q < e; q += 32) {
+        a.launch_of[q] = -1;
+        a.latency[q] = 0;
+        a.qdelay[q] = 0;
+      }
+      p = e;
+      if (p >= vend) break;
+      l = a.lane_dom_next[l];
+    }
+    const u32 lane_end = (u32)a.lane_off[l + 1], e = min(lane_end, vend);
+    const int slot = a.lane_slot[l], win = a.lane_window[l];
+    if (win != cur) {
+      if (cur >= 0) {
+        u64 t[7];
+        fold(t);
+        if (lane == 0) join_emit(&a.sum[cur], t);
+        n_probe = n_match = 0;
 #pragma unroll
-  for (int j = 0; j < IT; j++)
-    if (p0 + j < a.n_valid && (kd[j] == TA_KIND_KERNEL || kd[j] == TA_KIND_MEMCPY)) pm |= 1u << j;
-  int32_t lo[IT];
-  int wn[IT];  // window of the probe
-  {
-    u32 at[DIRECT ? 1 : IT];
-    int sl[DIRECT ? 1 : IT];
-    int l = l0;
-    int64_t next_off = l >= 0 ? (int64_t)a.lane_off[l + 1] : LLONG_MAX;
-    int slot = l >= 0 ? a.lane_slot[l] : 0;
-    int win = l >= 0 ? a.lane_window[l] : 0;
+        for (int k = 0; k < 5; k++) acc[k] = 0;
+      }
+      cur = win;
+    }
+    const i64 base = DIRECT ? a.slot_base[slot] : 0;
+    // direct: ids of the slot; hashed: positions of the slot
+    const i64 lo_id = DIRECT ? a.slot_min[slot] : a.slot_pos[slot], hi_id = DIRECT ? (base >= 0 ? a.slot_max[slot] : INT64_MIN) : a.slot_pos[slot + 1];
+    ProbeRow x[JP_ROWS];
 #pragma unroll
-    for (int j = 0; j < IT; j++) {
-      lo[j] = -1;
-      wn[j] = -1;
-      if (pm & (1u << j)) {
-        const int64_t p = p0 + j;
-        if (p >= next_off) {
-          do { l++; next_off = a.lane_off[l + 1]; } while (p >= next_off);
-          slot = a.lane_slot[l];
-          win = a.lane_window[l];
-        }
-        wn[j] = win;
+    for (int r = 0; r < JP_ROWS; r++) probe_row(a, p + 32 * r + lane, e, x[r]);
+    for (u32 q0 = p + lane;; q0 += 32 * JP_ROWS) {
+      u32 v[JP_ROWS], at[JP_ROWS];  // what the table holds, 0 = nothing
+#pragma unroll
+      for (int r = 0; r < JP_ROWS; r++) {
+        v[r] = at[r] = 0;
         if (DIRECT) {
-          const i64 base = a.slot_base[slot];
-          if (base >= 0 && c[j] >= a.slot_min[slot] && c[j] <= a.slot_max[slot]) {
-            const u32 v = a.table[base + (c[j] - a.slot_min[slot])];
-            lo[j] = v == 0 ? -1 : (int32_t)~v;
-          }
-        } else {
-          sl[DIRECT ? 0 : j] = slot;
-          at[DIRECT ? 0 : j] = join_hash(a, slot, c[j]);
+          if (x[r].probe && x[r].c >= lo_id && x[r].c <= hi_id) v[r] = a.table[base + (x[r].c - lo_id)];
+        } else if (x[r].probe) {
+          at[r] = join_hash(a, slot, x[r].c);
+          v[r] = a.table[at[r]];
         }
       }
-    }
-    if (!DIRECT) {  // the first entries of all the thread's keys together, then the ids they name, then the chains
-      u32 v[IT];
+      ProbeRow nx[JP_ROWS];
+      const u32 q1 = q0 + 32 * JP_ROWS;
 #pragma unroll
-      for (int j = 0; j < IT; j++) v[j] = pm & (1u << j) ? a.table[at[DIRECT ? 0 : j]] : 0u;
-      i64 cq[IT];
+      for (int r = 0; r < JP_ROWS; r++) probe_row(a, q1 + 32 * r, e, nx[r]);
+      if (!DIRECT) {  // the ids the first entries name, then the chains
+        i64 cq[JP_ROWS];
 #pragma unroll
-      for (int j = 0; j < IT; j++) cq[j] = v[j] ? a.corr[~v[j]] : 0;
+        for (int r = 0; r < JP_ROWS; r++) cq[r] = v[r] ? a.corr[~v[r]] : 0;
 #pragma unroll
-      for (int j = 0; j < IT; j++) {
-        if (v[j] == 0) continue;
-        const int32_t q = (int32_t)~v[j];
-        if (cq[j] != c[j] || q < a.slot_pos[sl[DIRECT ? 0 : j]] || q >= a.slot_pos[sl[DIRECT ? 0 : j] + 1])
-          v[j] = join_find(a, at[DIRECT ? 0 : j], v[j], sl[DIRECT ? 0 : j], c[j]);
-        lo[j] = v[j] == 0 ? -1 : (int32_t)~v[j];
+        for (int r = 0; r < JP_ROWS; r++)
+          if (v[r] && (cq[r] != x[r].c || (i64)~v[r] < lo_id || (i64)~v[r] >= hi_id))
+            v[r] = join_find(a, at[r], v[r], slot, x[r].c);
       }
-    }
-    const int64_t plast = min(tile_start + JP_TILE, a.n_valid) - 1;
-    if (plast >= p0 && plast < p0 + IT) {
-      while (plast >= next_off) { l++; next_off = a.lane_off[l + 1]; }
-      s_lane1 = l;
-    }
-  }
-  // launch times of the matched probes (independent gathers, issued together)
-  i64 ls[IT], le[IT];
+      // launch times of the matched probes (independent gathers, issued together)
+      i64 ls[JP_ROWS], le[JP_ROWS];
 #pragma unroll
-  for (int j = 0; j < IT; j++) {
-    ls[j] = le[j] = 0;
-    if (lo[j] >= 0) { ls[j] = a.ts[lo[j]]; le[j] = a.te[lo[j]]; }
-  }
-  i64 lat[IT], q[IT];
-  // probes, matches, latencies and delays summed; largest latency, largest complement, largest delay
-  u64 acc[7] = {0, 0, 0, 0, 0, 0, 0};
-  int wm = -1;
-#pragma unroll
-  for (int j = 0; j < IT; j++) {
-    lat[j] = q[j] = 0;
-    if (!(pm & (1u << j))) continue;
-    const bool matched = lo[j] >= 0;
-    if (matched) {
-      lat[j] = s[j] - ls[j];
-      const i64 d = s[j] - le[j];
-      q[j] = d > 0 ? d : 0;
-      atomicAdd(&a.kol[lo[j]], 1);
-      a.kernel_of[lo[j]] = (int32_t)(p0 + j);
-    }
-    if (wm < 0) wm = wn[j];
-    if (wn[j] == wm) {
-      acc[0]++;
-      if (matched) {
-        acc[1]++;
-        acc[2] += (u64)lat[j];
-        acc[3] += (u64)q[j];
-        acc[4] = max(acc[4], bias64(lat[j]));
-        acc[5] = max(acc[5], ~bias64(lat[j]));
-        acc[6] = max(acc[6], (u64)q[j]);
+      for (int r = 0; r < JP_ROWS; r++) {
+        ls[r] = le[r] = 0;
+        if (v[r]) { ls[r] = a.ts[~v[r]]; le[r] = a.te[~v[r]]; }
       }
-    } else {  // a thread that straddles a window boundary
-      const u64 one[7] = {1, matched ? 1ull : 0ull, (u64)lat[j], (u64)q[j], bias64(lat[j]), ~bias64(lat[j]), (u64)q[j]};
-      join_emit(&a.sum[wn[j]], one);
+#pragma unroll
+      for (int r = 0; r < JP_ROWS; r++) {
+        const u32 q = q0 + 32 * r;
+        if (q < e) {
+          i64 lat = 0, delay = 0;
+          if (v[r]) {
+            lat = x[r].s - ls[r];
+            delay = max(x[r].s - le[r], (i64)0);
+            atomicAdd(&a.kol[~v[r]], 1);
+            a.kernel_of[~v[r]] = (int32_t)q;
+            n_match++;
+            acc[0] += (u64)lat;
+            acc[1] += (u64)delay;
+            acc[2] = max(acc[2], bias64(lat));
+            acc[3] = max(acc[3], ~bias64(lat));
+            acc[4] = max(acc[4], (u64)delay);
+          }
+          n_probe += x[r].probe;
+          a.launch_of[q] = v[r] ? (int32_t)~v[r] : -1;
+          a.latency[q] = lat;
+          a.qdelay[q] = delay;
+        }
+        x[r] = nx[r];
+      }
+      if (q1 - lane >= e) break;
     }
+    p = e;
+    if (lane_end == e) l++;
   }
-  storen_i32<IT>(a.launch_of, p0, a.n, lo);
-  storen_i64<IT>(a.latency, p0, a.n, lat);
-  storen_i64<IT>(a.qdelay, p0, a.n, q);
+  for (u32 q = max(begin, vend) + lane; q < end; q += 32) {  // dropped records
+    a.launch_of[q] = -1;
+    a.latency[q] = 0;
+    a.qdelay[q] = 0;
+  }
+  u64 t[7] = {0, 0, 0, 0, 0, 0, 0};
+  if (cur >= 0) fold(t);
+  if (lane == 0) {
+    red_w[warp] = cur;
+#pragma unroll
+    for (int k = 0; k < 7; k++) red[k][warp] = t[k];
+  }
   __syncthreads();
-  if (l0 < 0) return;
-  fold_by_window<4, 3, JP_THREADS / 32>(acc, wm, a.lane_window[l0], a.lane_window[s_lane1], red,
-                                        [&](int w, const u64 *t) { join_emit(&a.sum[w], t); });
+  if (warp > 0) return;
+  const int w = lane < JP_THREADS / 32 ? red_w[lane] : -1;
+  const u32 has = __ballot_sync(0xffffffffu, w >= 0);
+  if (has == 0) return;
+#pragma unroll
+  for (int k = 0; k < 7; k++) t[k] = w >= 0 ? red[k][lane] : 0;
+  const int w0 = __shfl_sync(0xffffffffu, w, __ffs(has) - 1);
+  if (__all_sync(0xffffffffu, w < 0 || w == w0)) {
+#pragma unroll
+    for (int k = 0; k < 4; k++) t[k] = warp_reduce(t[k], OpAdd());
+#pragma unroll
+    for (int k = 4; k < 7; k++) t[k] = warp_reduce(t[k], OpMax());
+    if (lane == 0) join_emit(&a.sum[w0], t);
+  } else if (w >= 0) {
+    join_emit(&a.sum[w], t);
+  }
 }
 
 // ---- pass 3: launch statistics (duplicates, orphans) ---------------------------
@@ -433,13 +453,19 @@ ta_status ta_run_correlate(ta_window *h, ta_join_summary *out_summary) {
   a.n = n; a.n_valid = h->n_valid; a.n_lanes = h->sorted.n_lanes;
   a.kind = h->sorted.kind; a.corr = h->sorted.corr_id; a.ts = h->sorted.ts_start; a.te = h->sorted.ts_end;
   a.lane_off = h->sorted.lane_off; a.lane_slot = h->d_lane_slot; a.lane_window = h->sorted.lane_window;
-  a.lane_domain = h->sorted.lane_domain; a.lane_dom_end = h->d_lane_dom_end;
+  a.lane_domain = h->sorted.lane_domain; a.lane_dom_end = h->d_lane_dom_end; a.lane_dom_next = h->d_lane_dom_next;
   a.slot_min = h->d_slot_min; a.slot_max = h->d_slot_max; a.slot_base = h->d_slot_base;  // filled by the sort
   a.launch_of = launch_of; a.kol = kol; a.kernel_of = h->d_kernel_of; a.multi = (u32 *)&h->d_status[ST_MULTI]; a.latency = latency; a.qdelay = qdelay; a.sum = d_sum;
   a.status = h->d_status;
   const unsigned grid = (unsigned)((n + JN_TILE - 1) / JN_TILE);
   const unsigned grid8 = (unsigned)((n + JS_TILE - 1) / JS_TILE);
-  const unsigned grid_probe = (unsigned)((n + JP_TILE - 1) / JP_TILE);
+  // Rows per warp: 12, fewer where that would be less than a round of the 148 * 24 warps on the chip
+  // (1.2 M records: 101 us with 12, 90 with 8), 24 where it leaves twenty rounds and more (66.8 M: 730 us
+  // with 12, 690 with 24; 16.8 M: 182 with 12, 233 with 32, whose last warps run long).
+  int64_t rows = n / 32 / (148 * 32);
+  rows = rows < JP_ROWS ? JP_ROWS : rows > 12 ? 12 : rows / JP_ROWS * JP_ROWS;
+  if (n > (int64_t)20 * 148 * 24 * 24 * 32) rows = 24;
+  const unsigned grid_probe = (unsigned)((n + rows * JP_THREADS - 1) / (rows * JP_THREADS));
   void *tmp_alloc = nullptr;
   bool direct = true;
   int32_t words[ST_WORDS];
@@ -469,11 +495,11 @@ ta_status ta_run_correlate(ta_window *h, ta_join_summary *out_summary) {
     a.table = (u32 *)tmp_alloc;
     if (direct) {
       ta_launch(k_join_build<true>, grid, JN_THREADS, 0, st, a);
-      ta_launch(k_join_probe<true>, grid_probe, JP_THREADS, 0, st, a);
+      ta_launch(k_join_probe<true>, grid_probe, JP_THREADS, 0, st, a, (int)rows);
       ta_launch(k_join_launch_stats<true>, grid8, JP_THREADS, 0, st, a, ta_tail(h, grid8));
     } else {
       ta_launch(k_join_build<false>, grid, JN_THREADS, 0, st, a);
-      ta_launch(k_join_probe<false>, grid_probe, JP_THREADS, 0, st, a);
+      ta_launch(k_join_probe<false>, grid_probe, JP_THREADS, 0, st, a, (int)rows);
       ta_launch(k_join_launch_stats<false>, grid8, JP_THREADS, 0, st, a, ta_tail(h, grid8));
     }
     TA_CHECK_CUDA(h, cudaGetLastError());
