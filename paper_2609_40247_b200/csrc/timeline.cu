@@ -197,6 +197,7 @@ __global__ void __launch_bounds__(256, GT_MINB) k_gather(GatherArgs a) {
   const u64 k = p < nv ? a.keys[p] : 0;
   u64 kprev = __shfl_up_sync(0xffffffffu, k, 1);
   if (lane == 0 && p > 0 && p < nv) kprev = a.keys[p - 1];
+  const u64 knext = PACKED && lane == 31 && p + 1 < nv ? a.keys[p + 1] : 0;
   u32 idx = 0;
   if (p < n) idx = PACKED && p < nv ? gather_index<ONE>(k, a) : a.perm[p];
   Rec r;
@@ -208,21 +209,39 @@ __global__ void __launch_bounds__(256, GT_MINB) k_gather(GatherArgs a) {
     // are ranked here by (ts_start, -ts_end, input index)
     const u64 hk = k >> a.ibits;
     const u32 eq = __ballot_sync(0xffffffffu, p < nv && p > 0 && (kprev >> a.ibits) == hk);
-    if (eq || lane == 31) {
-      // equal keys in front of the record and behind it, as far as the warp reaches; further only
-      // where a run meets the warp's edge
+    const bool next = __any_sync(0xffffffffu, lane == 31 && p + 1 < nv && (knext >> a.ibits) == hk);
+    if (eq || next) {
+      // equal keys in front of the record and behind it, as far as the warp reaches
       int before = __clz((int)~(eq << (31 - lane)));
       int after = lane < 31 ? __ffs((int)~(eq >> (lane + 1))) - 1 : 0;
-      if (before == lane + 1)
-        while (before <= TA_TIE_RUN_MAX && p > (u32)before && (a.keys[p - before - 1] >> a.ibits) == hk) before++;
-      if (lane + after == 31 && p < nv)
-        while (after <= TA_TIE_RUN_MAX && p + after + 1 < nv && (a.keys[p + after + 1] >> a.ibits) == hk) after++;
-      if (before + after + 1 > TA_TIE_RUN_MAX) {
-        a.status[ST_LONG_RUN] = 1;  // the caller starts over with full-resolution keys
-        before = after = 0;
+      // a run that meets the warp's edge goes on in memory
+      const bool open = p < nv && (before == lane + 1 || (lane + after == 31 && next));
+      int rank = 0;
+      // the others: every member is compared with the one d places in front of it, and what it
+      // learns holds the other way round for that one
+      for (int d = 1;; d++) {
+        const bool me = !open && before >= d;
+        const u32 m = __ballot_sync(0xffffffffu, me);
+        if (m == 0) break;
+        const i64 os = __shfl_up_sync(0xffffffffu, r.ts_start, d);
+        bool first = os < r.ts_start;
+        if (__any_sync(0xffffffffu, me && os == r.ts_start)) {
+          const i64 oe = __shfl_up_sync(0xffffffffu, r.ts_end, d);
+          const u32 oi = __shfl_up_sync(0xffffffffu, idx, d);
+          first = first || (os == r.ts_start && (oe > r.ts_end || (oe == r.ts_end && oi < idx)));
+        }
+        const u32 b = __ballot_sync(0xffffffffu, me && first);
+        rank += (me && first ? 1 : 0) + (int)(((m & ~b) >> d) >> lane & 1u);
       }
-      if (before + after > 0) {
-        int rank = 0;
+      if (open) {
+        if (before == lane + 1)
+          while (before <= TA_TIE_RUN_MAX && p > (u32)before && (a.keys[p - before - 1] >> a.ibits) == hk) before++;
+        if (lane + after == 31)
+          while (after <= TA_TIE_RUN_MAX && p + after + 1 < nv && (a.keys[p + after + 1] >> a.ibits) == hk) after++;
+        if (before + after + 1 > TA_TIE_RUN_MAX) {
+          a.status[ST_LONG_RUN] = 1;  // the caller starts over with full-resolution keys
+          before = after = 0;
+        }
         for (int q = -before; q <= after; q++) {
           if (q == 0) continue;
           const u32 oi = gather_index<ONE>(a.keys[p + q], a);
@@ -231,8 +250,8 @@ __global__ void __launch_bounds__(256, GT_MINB) k_gather(GatherArgs a) {
           const bool first = os < r.ts_start || (os == r.ts_start && (oe > r.ts_end || (oe == r.ts_end && oi < idx)));
           rank += first ? 1 : 0;
         }
-        dst = p - before + rank;
       }
+      if (p < nv) dst = p - before + rank;
     }
   }
   int slot = -1;
