@@ -129,7 +129,8 @@ __global__ void __launch_bounds__(PL_THREADS) k_plan(const ta_event *ev, int64_t
 #endif
 #define DS_TILE (DS_THREADS * DS_RPT)     // 512 records = 20480 bytes
 #define DS_TILE_BYTES (DS_TILE * 40)
-#define DS_CACHE 512
+#define DS_CACHE_BITS 9
+#define DS_CACHE (1 << DS_CACHE_BITS)
 #define DS_PROBES 4
 #define DS_WAIT_POLLS (1 << 18)  // a tile arrives within microseconds; each poll may itself wait a little
 
@@ -203,7 +204,7 @@ __global__ void __launch_bounds__(DS_THREADS, 4) k_discover_staged(DiscoverArgs 
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
-  // passes over the time bits kept (decided by k_plan): digit p = (ts_rel >> sh[p]) & mk[p]
+  // passes over the time bits kept (decided by k_plan): digit p = (ts_rel >> dshift >> sh[p]) & mk[p]
   const int keep = (int)a.misc[6];
   const int dshift = a.sbits - keep;
   const SortPlan tp = ta_plan_bits(0, keep);
@@ -212,7 +213,7 @@ __global__ void __launch_bounds__(DS_THREADS, 4) k_discover_staged(DiscoverArgs 
   u32 mk[5];
 #pragma unroll
   for (int p = 0; p < 5; p++) {
-    sh[p] = dshift + tp.shift[p];
+    sh[p] = tp.shift[p];
     mk[p] = (1u << tp.bits[p]) - 1u;
   }
   const int64_t n_tiles = (a.n + DS_TILE - 1) / DS_TILE;
@@ -321,10 +322,10 @@ __global__ void __launch_bounds__(DS_THREADS, 4) k_discover_staged(DiscoverArgs 
             qmn = min(qmn, r.seq);
             qmx = max(qmx, r.seq);
             const u64 cc = (u64)r.corr ^ (1ull << 63);
-            const u32 ch = hash_code(cc);
+            const u32 ch = (((u32)cc ^ (u32)(cc >> 32)) * 0x9E3779B1u) >> 26;
             if (cc == TRIPLE_EMPTY) ta_set_err(a.status, TA_ERR_INVALID_ARG);  // reserved id
-            else if (s.ccache[ch & 63] != cc) {
-              u32 slot = ch & (TA_COMM_SLOTS - 1);
+            else if (s.ccache[ch] != cc) {
+              u32 slot = hash_code(cc) & (TA_COMM_SLOTS - 1);
               bool ok = false;
               for (int probe = 0; probe < TA_COMM_SLOTS; probe++) {
                 const u64 c2 = ld_relaxed(&a.cm->slots[slot]);
@@ -336,14 +337,13 @@ __global__ void __launch_bounds__(DS_THREADS, 4) k_discover_staged(DiscoverArgs 
                 slot = (slot + 1) & (TA_COMM_SLOTS - 1);
               }
               if (!ok) ta_set_err(a.status, TA_ERR_TOO_LARGE);
-              s.ccache[ch & 63] = cc;
+              s.ccache[ch] = cc;
             }
           }
           const u64 code = triple_code(r.pid, r.kind, r.stream);
-          const u32 hsh = hash_code(code);
           trel = (u64)(r.ts_start - ct0);
           // the CTA's own table first: an entry or an empty one within a few steps
-          int at = (int)(hsh & (DS_CACHE - 1));
+          int at = (int)(((u32)code * 0x9E3779B1u + (u32)(code >> 32) * 0x85EBCA77u) >> (32 - DS_CACHE_BITS));
           u64 hit = s.cache[at];
           for (int probe = 1; probe < DS_PROBES && (hit >> 13) != code && hit != TRIPLE_EMPTY; probe++) {
             at = (at + 1) & (DS_CACHE - 1);
@@ -353,7 +353,7 @@ __global__ void __launch_bounds__(DS_THREADS, 4) k_discover_staged(DiscoverArgs 
             slot_mine = (int)(hit & (TA_TRIPLE_SLOTS - 1));
             entry = at;
           } else {
-            u32 slot = hsh & (TA_TRIPLE_SLOTS - 1);
+            u32 slot = hash_code(code) & (TA_TRIPLE_SLOTS - 1);
             bool done = false;
             for (int probe = 0; probe < TA_TRIPLE_SLOTS; probe++) {
               const u64 c2 = ld_relaxed(&a.tt->slots[slot]);
@@ -382,10 +382,11 @@ __global__ void __launch_bounds__(DS_THREADS, 4) k_discover_staged(DiscoverArgs 
       const u32 kept = __ballot_sync(0xffffffffu, slot_mine >= 0);
       if (kept) {
         const int leader = __ffs(kept) - 1;
+        const u64 tk = trel >> dshift;  // (digits are at most 8 bits wide: the first four begin below bit 32)
 #pragma unroll
         for (int p = 0; p < 5; p++) {
           if (p >= n_tp) break;
-          const u32 d = (u32)(trel >> sh[p]) & mk[p];
+          const u32 d = (p < 4 ? __funnelshift_r((u32)tk, (u32)(tk >> 32), sh[p]) : (u32)(tk >> sh[p])) & mk[p];
           if (p >= 1) {
             const u32 d0 = __shfl_sync(0xffffffffu, d, leader);
             if (__all_sync(0xffffffffu, slot_mine < 0 || d == d0)) {
