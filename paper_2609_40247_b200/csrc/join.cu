@@ -22,10 +22,6 @@
 #include "scan.cuh"
 #include "ta_internal.cuh"
 
-#define JN_THREADS 512
-#define JN_ITEMS 4
-#define JN_TILE (JN_THREADS * JN_ITEMS)
-
 struct JoinArgs {
   int64_t n, n_valid;
   int n_lanes;
@@ -80,53 +76,147 @@ __global__ void __launch_bounds__(256) k_join_slot_pos(const int32_t *lane_off, 
   for (int s = lo; s <= hi; s++) slot_pos[s] = lane_off[l];  // lane_off[n_lanes] = records
 }
 
-// ---- fill the table -------------------------------------------------------------
-template <bool DIRECT>
-__global__ void __launch_bounds__(JN_THREADS) k_join_build(JoinArgs a) {
-  TA_PDL();
-  __shared__ int s_lane0;
-  if (ta_failed(a.status)) return;
-  const int tid = threadIdx.x;
-  const int64_t tile_start = (int64_t)blockIdx.x * JN_TILE;
-  if (tile_start >= a.n_valid) return;
-  if (tid < 32) {
-    const int l = tile_lane_search(a.lane_off, a.n_lanes, tile_start);
-    if (tid == 0) s_lane0 = l;
+#define JN_THREADS 256
+#define JN_WARPS (JN_THREADS / 32)
+
+// The span of records a warp works on: so many rows of 32.
+struct JoinSpan {
+  u32 begin, end, vend;  // vend: end of the kept records in it
+};
+__device__ __forceinline__ JoinSpan join_span(const JoinArgs &a, int rows) {
+  const u64 first = ((u64)blockIdx.x * JN_WARPS + (threadIdx.x >> 5)) * (u32)rows * 32;
+  JoinSpan x;
+  x.begin = (u32)min(first, (u64)a.n);
+  x.end = (u32)min(first + (u32)rows * 32, (u64)a.n);
+  x.vend = min(x.end, (u32)a.n_valid);
+  return x;
+}
+// Adds the figures of a CTA's warps (t: the same in every lane of a warp; cur: their window, -1 = none)
+// to the rows of their windows.  Called by all threads.
+template <int NS, int NM, class Emit>
+__device__ __forceinline__ void join_fold(u64 (&t)[NS + NM], int cur, Emit emit) {
+  __shared__ u64 red[NS + NM][JN_WARPS];
+  __shared__ int red_w[JN_WARPS];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (lane == 0) {
+    red_w[warp] = cur;
+#pragma unroll
+    for (int k = 0; k < NS + NM; k++) red[k][warp] = t[k];
   }
   __syncthreads();
-  const int l0 = s_lane0;
-  // launches live in host lanes: a tile of device lanes has none
-  if (span_outside_domain(a.lane_domain, a.lane_dom_end, l0, min(tile_start + JN_TILE, a.n_valid), 0)) return;
-  const int64_t p0 = tile_start + (int64_t)tid * JN_ITEMS;
-  int16_t kd[JN_ITEMS];
-  i64 c[JN_ITEMS];
-  loadn_i16<JN_ITEMS>(a.kind, p0, a.n, 9, kd);
-  loadn_i64<JN_ITEMS>(a.corr, p0, a.n, c);
-  int l = l0;
-  int64_t next_off = a.lane_off[l + 1];
-  int slot = a.lane_slot[l];
+  if (warp > 0) return;
+  const int w = lane < JN_WARPS ? red_w[lane] : -1;
+  const u32 has = __ballot_sync(0xffffffffu, w >= 0);
+  if (has == 0) return;
 #pragma unroll
-  for (int j = 0; j < JN_ITEMS; j++) {
-    const int64_t p = p0 + j;
-    if (p < a.n_valid && kd[j] == TA_KIND_LAUNCH) {
-      while (p >= next_off) { l++; next_off = a.lane_off[l + 1]; slot = a.lane_slot[l]; }
-      if (DIRECT) {
-        const i64 idx = a.slot_base[slot] + (c[j] - a.slot_min[slot]);
-        atomicMax(&a.table[idx], ~(u32)p);
-      } else {
-        u32 i = join_hash(a, slot, c[j]);
-        for (u32 step = 0; step < a.table_size; step++) {
-          const u32 old = atomicCAS(&a.table[i], 0u, ~(u32)p);
-          if (old == 0) break;
-          if (join_same(a, ~old, slot, c[j])) {
-            atomicMax(&a.table[i], ~(u32)p);
-            break;
+  for (int k = 0; k < NS + NM; k++) t[k] = w >= 0 ? red[k][lane] : 0;
+  const int w0 = __shfl_sync(0xffffffffu, w, __ffs(has) - 1);
+  if (__all_sync(0xffffffffu, w < 0 || w == w0)) {
+#pragma unroll
+    for (int k = 0; k < NS; k++) t[k] = warp_reduce(t[k], OpAdd());
+#pragma unroll
+    for (int k = NS; k < NS + NM; k++) t[k] = warp_reduce(t[k], OpMax());
+    if (lane == 0) emit(w0, t);
+  } else if (w >= 0) {
+    emit(w, t);
+  }
+}
+
+// ---- fill the table -------------------------------------------------------------
+// A warp takes rows of 32 records of one host lane, JB_ROWS at a time, with the kinds and ids of the
+// next JB_ROWS on their way.  What an entry held before tells a first launch of its id from a repeated
+// one, so that launches, duplicates and ids are counted here and no later pass has to look them up.
+#ifndef JB_ROWS
+#define JB_ROWS 2
+#endif
+// adds a group of launches to the row of their window; k_join_probe takes the ids with a kernel off the orphans again
+__device__ __forceinline__ void launch_emit(ta_join_summary *sm, const u64 *t) {
+  if (t[0] == 0) return;
+  atomicAdd((u64 *)&sm->n_launch, t[0]);
+  if (t[1]) atomicAdd((u64 *)&sm->n_dup_launch, t[1]);
+  atomicAdd((u64 *)&sm->n_orphan_launch, t[0] - t[1]);
+}
+struct LaunchRow {
+  i64 c;
+  bool launch;
+};
+__device__ __forceinline__ void launch_row(const JoinArgs &a, u32 q, u32 end, LaunchRow &x) {
+  x.launch = false;
+  x.c = 0;
+  if (q < end) {
+    x.launch = a.kind[q] == TA_KIND_LAUNCH;
+    x.c = a.corr[q];
+  }
+}
+template <bool DIRECT>
+__global__ void __launch_bounds__(JN_THREADS) k_join_build(JoinArgs a, int rows) {
+  TA_PDL();
+  if (ta_failed(a.status)) return;
+  const int lane = threadIdx.x & 31;
+  const JoinSpan sp = join_span(a, rows);
+  u32 n_launch = 0, n_dup = 0;
+  int cur = -1;  // window they are of
+  int l = sp.begin < sp.vend ? tile_lane_search(a.lane_off, a.n_lanes, sp.begin) : 0;
+  for (u32 p = sp.begin; p < sp.vend;) {
+    if (a.lane_domain[l] != 0) {  // launches live in host lanes
+      p = min((u32)a.lane_dom_end[l], sp.vend);
+      if (p >= sp.vend) break;
+      l = a.lane_dom_next[l];
+    }
+    const u32 lane_end = (u32)a.lane_off[l + 1], e = min(lane_end, sp.vend);
+    const int slot = a.lane_slot[l], win = a.lane_window[l];
+    if (win != cur) {
+      if (cur >= 0) {
+        const u64 t[2] = {__reduce_add_sync(0xffffffffu, n_launch), __reduce_add_sync(0xffffffffu, n_dup)};
+        if (lane == 0) launch_emit(&a.sum[cur], t);
+        n_launch = n_dup = 0;
+      }
+      cur = win;
+    }
+    const i64 base = DIRECT ? a.slot_base[slot] - a.slot_min[slot] : 0;
+    LaunchRow x[JB_ROWS];
+#pragma unroll
+    for (int r = 0; r < JB_ROWS; r++) launch_row(a, p + 32 * r + lane, e, x[r]);
+    for (u32 q0 = p + lane;; q0 += 32 * JB_ROWS) {
+      LaunchRow nx[JB_ROWS];
+      const u32 q1 = q0 + 32 * JB_ROWS;
+#pragma unroll
+      for (int r = 0; r < JB_ROWS; r++) launch_row(a, q1 + 32 * r, e, nx[r]);
+      u32 old[JB_ROWS];
+#pragma unroll
+      for (int r = 0; r < JB_ROWS; r++) {
+        const u32 q = q0 + 32 * r;
+        old[r] = 0;
+        if (!x[r].launch) continue;
+        if (DIRECT) {
+          old[r] = atomicMax(&a.table[base + x[r].c], ~q);
+        } else {
+          u32 i = join_hash(a, slot, x[r].c);
+          for (u32 step = 0; step < a.table_size; step++) {
+            const u32 was = atomicCAS(&a.table[i], 0u, ~q);
+            if (was == 0) break;
+            if (join_same(a, ~was, slot, x[r].c)) {
+              atomicMax(&a.table[i], ~q);
+              old[r] = was;
+              break;
+            }
+            i = i + 1 == a.table_size ? 0 : i + 1;
           }
-          i = i + 1 == a.table_size ? 0 : i + 1;
         }
       }
+#pragma unroll
+      for (int r = 0; r < JB_ROWS; r++) {
+        n_launch += x[r].launch;
+        n_dup += old[r] != 0;
+        x[r] = nx[r];
+      }
+      if (q1 - lane >= e) break;
     }
+    p = e;
+    if (lane_end == e) l++;
   }
+  u64 t[2] = {__reduce_add_sync(0xffffffffu, n_launch), __reduce_add_sync(0xffffffffu, n_dup)};
+  join_fold<2, 0>(t, cur, [&](int w, const u64 *v) { launch_emit(&a.sum[w], v); });
 }
 
 // ---- pass 2: probes ----------------------------------------------------------
@@ -135,7 +225,6 @@ __global__ void __launch_bounds__(JN_THREADS) k_join_build(JoinArgs a) {
 // chain of three (columns, table, launch times), so a warp works on JP_ROWS rows at a time and has the
 // columns of the next JP_ROWS on their way meanwhile.  (A CTA per 1024 records, lanes walked by every
 // thread, two block barriers at the start: 1035 us of 66.8 M records, half of it in those waits.)
-#define JP_THREADS 256
 #ifndef JP_MINB
 #define JP_MINB 3
 #endif
@@ -152,9 +241,10 @@ __device__ __forceinline__ void join_emit(ta_join_summary *sm, const u64 *t) {
   atomicAdd((u64 *)&sm->sum_latency, t[2]);
   atomicAdd((u64 *)&sm->sum_queue, t[3]);
   // (codes with 0 as "none"; the host turns them into times)
-  atomicMax((u64 *)&sm->max_latency, t[4]);
-  atomicMax((u64 *)&sm->min_latency, t[5]);
-  atomicMax((i64 *)&sm->max_queue, (i64)t[6]);
+  atomicMax((u64 *)&sm->max_latency, t[5]);
+  atomicMax((u64 *)&sm->min_latency, t[6]);
+  atomicMax((u64 *)&sm->max_queue, t[7]);
+  if (t[4]) atomicAdd((u64 *)&sm->n_orphan_launch, 0ull - t[4]);
 }
 
 struct ProbeRow {
@@ -174,26 +264,36 @@ __device__ __forceinline__ void probe_row(const JoinArgs &a, u32 q, u32 end, Pro
 }
 
 template <bool DIRECT>
-__global__ void __launch_bounds__(JP_THREADS, JP_MINB) k_join_probe(JoinArgs a, int rows) {
-  TA_PDL();
-  __shared__ u64 red[7][JP_THREADS / 32];
-  __shared__ int red_w[JP_THREADS / 32];
+__device__ __forceinline__ void join_probe(const JoinArgs &a, int rows) {
   if (ta_failed(a.status)) return;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const u32 n = (u32)a.n, nv = (u32)a.n_valid;
-  const u64 first = ((u64)blockIdx.x * (JP_THREADS / 32) + warp) * (u32)rows * 32;
-  const u32 begin = (u32)min(first, (u64)n), end = (u32)min(first + (u32)rows * 32, (u64)n), vend = min(end, nv);
-  // probes and matches; latencies and delays summed; largest latency, largest complement, largest delay
-  u32 n_probe = 0, n_match = 0;
+  const int lane = threadIdx.x & 31;
+  const JoinSpan sp = join_span(a, rows);
+  const u32 begin = sp.begin, end = sp.end, vend = sp.vend;
+  // probes, matches, launches met for the first time; latencies and delays summed; largest latency, largest complement, largest delay
+  u32 n_probe = 0, n_match = 0, n_first = 0;
+  bool multi = false;
   u64 acc[5] = {0, 0, 0, 0, 0};
   int cur = -1;  // window they are of
+  int had[JP_ROWS];  // kernels a matched launch had before this warp's last rows; -1 = none matched
+#pragma unroll
+  for (int r = 0; r < JP_ROWS; r++) had[r] = -1;
+  auto count_had = [&]() {
+#pragma unroll
+    for (int r = 0; r < JP_ROWS; r++) {
+      n_first += had[r] == 0;
+      multi |= had[r] > 0;
+      had[r] = -1;
+    }
+  };
   auto fold = [&](u64 *t) {
+    count_had();
     t[0] = __reduce_add_sync(0xffffffffu, n_probe);
     t[1] = __reduce_add_sync(0xffffffffu, n_match);
     t[2] = warp_reduce(acc[0], OpAdd());
     t[3] = warp_reduce(acc[1], OpAdd());
+    t[4] = __reduce_add_sync(0xffffffffu, n_first);
 #pragma unroll
-    for (int k = 4; k < 7; k++) t[k] = warp_reduce(acc[k - 2], OpMax());
+    for (int k = 5; k < 8; k++) t[k] = warp_reduce(acc[k - 3], OpMax());
   };
   int l = begin < vend ? tile_lane_search(a.lane_off, a.n_lanes, begin) : 0;
   for (u32 p = begin; p < vend;) {
@@ -212,10 +312,10 @@ __global__ void __launch_bounds__(JP_THREADS, JP_MINB) k_join_probe(JoinArgs a, 
     const int slot = a.lane_slot[l], win = a.lane_window[l];
     if (win != cur) {
       if (cur >= 0) {
-        u64 t[7];
+        u64 t[8];
         fold(t);
         if (lane == 0) join_emit(&a.sum[cur], t);
-        n_probe = n_match = 0;
+        n_probe = n_match = n_first = 0;
 #pragma unroll
         for (int k = 0; k < 5; k++) acc[k] = 0;
       }
@@ -252,6 +352,7 @@ __global__ void __launch_bounds__(JP_THREADS, JP_MINB) k_join_probe(JoinArgs a, 
           if (v[r] && (cq[r] != x[r].c || (i64)~v[r] < lo_id || (i64)~v[r] >= hi_id))
             v[r] = join_find(a, at[r], v[r], slot, x[r].c);
       }
+      count_had();  // (asked for a round of rows ago: nothing waits here)
       // launch times of the matched probes (independent gathers, issued together)
       i64 ls[JP_ROWS], le[JP_ROWS];
 #pragma unroll
@@ -267,7 +368,7 @@ __global__ void __launch_bounds__(JP_THREADS, JP_MINB) k_join_probe(JoinArgs a, 
           if (v[r]) {
             lat = x[r].s - ls[r];
             delay = max(x[r].s - le[r], (i64)0);
-            atomicAdd(&a.kol[~v[r]], 1);
+            had[r] = atomicAdd(&a.kol[~v[r]], 1);
             a.kernel_of[~v[r]] = (int32_t)q;
             n_match++;
             acc[0] += (u64)lat;
@@ -293,136 +394,16 @@ __global__ void __launch_bounds__(JP_THREADS, JP_MINB) k_join_probe(JoinArgs a, 
     a.latency[q] = 0;
     a.qdelay[q] = 0;
   }
-  u64 t[7] = {0, 0, 0, 0, 0, 0, 0};
+  u64 t[8] = {0, 0, 0, 0, 0, 0, 0, 0};
   if (cur >= 0) fold(t);
-  if (lane == 0) {
-    red_w[warp] = cur;
-#pragma unroll
-    for (int k = 0; k < 7; k++) red[k][warp] = t[k];
-  }
-  __syncthreads();
-  if (warp > 0) return;
-  const int w = lane < JP_THREADS / 32 ? red_w[lane] : -1;
-  const u32 has = __ballot_sync(0xffffffffu, w >= 0);
-  if (has == 0) return;
-#pragma unroll
-  for (int k = 0; k < 7; k++) t[k] = w >= 0 ? red[k][lane] : 0;
-  const int w0 = __shfl_sync(0xffffffffu, w, __ffs(has) - 1);
-  if (__all_sync(0xffffffffu, w < 0 || w == w0)) {
-#pragma unroll
-    for (int k = 0; k < 4; k++) t[k] = warp_reduce(t[k], OpAdd());
-#pragma unroll
-    for (int k = 4; k < 7; k++) t[k] = warp_reduce(t[k], OpMax());
-    if (lane == 0) join_emit(&a.sum[w0], t);
-  } else if (w >= 0) {
-    join_emit(&a.sum[w], t);
-  }
-}
-
-// ---- pass 3: launch statistics (duplicates, orphans) ---------------------------
-#define JS_TILE (JP_THREADS * 8)
-// adds a group of launches to the row of their window
-__device__ __forceinline__ void launch_emit(ta_join_summary *sm, const u64 *t) {
-  if (t[0]) atomicAdd((u64 *)&sm->n_launch, t[0]);
-  if (t[1]) atomicAdd((u64 *)&sm->n_dup_launch, t[1]);
-  if (t[2]) atomicAdd((u64 *)&sm->n_orphan_launch, t[2]);
+  if (multi) *a.multi = 1u;
+  join_fold<5, 3>(t, cur, [&](int w, const u64 *v) { join_emit(&a.sum[w], v); });
 }
 
 template <bool DIRECT>
-__device__ __forceinline__ void join_launch_stats(const JoinArgs &a) {
-  __shared__ u64 red[3][JP_THREADS / 32];
-  __shared__ int s_lane0, s_lane1;
-  if (ta_failed(a.status)) return;
-  const int tid = threadIdx.x, lane = tid & 31;
-  const int64_t tile_start = (int64_t)blockIdx.x * JS_TILE;
-  const int64_t p0 = tile_start + (int64_t)tid * 8;
-  if (tid == 0) { s_lane0 = -1; s_lane1 = -1; }
-  __syncthreads();
-  if (tid < 32 && tile_start < a.n_valid && a.n_lanes > 0) {
-    int l = tile_lane_search(a.lane_off, a.n_lanes, tile_start);
-    if (lane == 0) s_lane0 = l;
-  }
-  __syncthreads();
-  const int l0 = s_lane0;
-  // launches live in host lanes: a tile of device lanes has none
-  if (l0 < 0 || span_outside_domain(a.lane_domain, a.lane_dom_end, l0, min(tile_start + JS_TILE, a.n_valid), 0))
-    return;
-  // kinds, correlation ids and kernel counts of the thread's records together, then the table
-  // entries of its launches together: two rounds of memory latency
-  int16_t kd[8];
-  i64 cr[8];
-  int32_t nk[8];
-  load8_i16(a.kind, p0, a.n, 0, kd);
-  load8_i64(a.corr, p0, a.n, cr);
-  if (p0 + 8 <= a.n) {
-    const int4 x = *reinterpret_cast<const int4 *>(a.kol + p0), y = *reinterpret_cast<const int4 *>(a.kol + p0 + 4);
-    nk[0] = x.x; nk[1] = x.y; nk[2] = x.z; nk[3] = x.w; nk[4] = y.x; nk[5] = y.y; nk[6] = y.z; nk[7] = y.w;
-  } else {
-#pragma unroll
-    for (int j = 0; j < 8; j++) nk[j] = p0 + j < a.n ? a.kol[p0 + j] : 0;
-  }
-  unsigned lmask = 0;
-#pragma unroll
-  for (int j = 0; j < 8; j++)
-    if (p0 + j < a.n_valid && kd[j] == TA_KIND_LAUNCH) lmask |= 1u << j;
-  u64 acc[3] = {0, 0, 0};  // launches, duplicates, orphans of the thread's first window
-  int wm = -1;
-  {
-    int l = l0;
-    int64_t next_off = (int64_t)a.lane_off[l + 1];
-    int wn[8];
-    int32_t win[8];
-#pragma unroll
-    for (int j = 0; j < 8; j++) {
-      wn[j] = -1;
-      win[j] = -1;
-      if (!(lmask & (1u << j))) continue;
-      const int64_t p = p0 + j;
-      while (p >= next_off) { l++; next_off = a.lane_off[l + 1]; }
-      wn[j] = a.lane_window[l];
-      const int slot = a.lane_slot[l];
-      u32 v = 0;
-      if (DIRECT) {
-        const i64 base = a.slot_base[slot];
-        if (base >= 0 && cr[j] >= a.slot_min[slot] && cr[j] <= a.slot_max[slot])
-          v = a.table[base + (cr[j] - a.slot_min[slot])];
-      } else {
-        const u32 i = join_hash(a, slot, cr[j]);
-        v = join_find(a, i, a.table[i], slot, cr[j]);
-      }
-      win[j] = v == 0 ? -1 : (int32_t)~v;
-    }
-#pragma unroll
-    for (int j = 0; j < 8; j++) {
-      if (!(lmask & (1u << j))) continue;
-      const bool dup = win[j] != (int32_t)(p0 + j);
-      const bool orphan = !dup && nk[j] == 0;
-      if (nk[j] > 1) *a.multi = 1u;
-      if (wm < 0) wm = wn[j];
-      if (wn[j] == wm) {
-        acc[0]++;
-        acc[1] += dup;
-        acc[2] += orphan;
-      } else {
-        const u64 one[3] = {1, dup, orphan};
-        launch_emit(&a.sum[wn[j]], one);
-      }
-    }
-    const int64_t plast = min(tile_start + JS_TILE, a.n_valid) - 1;
-    if (plast >= p0 && plast < p0 + 8) {
-      while (plast >= next_off) { l++; next_off = a.lane_off[l + 1]; }
-      s_lane1 = l;
-    }
-  }
-  __syncthreads();
-  fold_by_window<3, 0, JP_THREADS / 32>(acc, wm, a.lane_window[l0], a.lane_window[s_lane1], red,
-                                        [&](int w, const u64 *t) { launch_emit(&a.sum[w], t); });
-}
-
-template <bool DIRECT>
-__global__ void __launch_bounds__(JP_THREADS) k_join_launch_stats(JoinArgs a, Tail tail) {
+__global__ void __launch_bounds__(JN_THREADS, JP_MINB) k_join_probe(JoinArgs a, int rows, Tail tail) {
   TA_PDL();
-  join_launch_stats<DIRECT>(a);
+  join_probe<DIRECT>(a, rows);
   run_tail(tail);
 }
 
@@ -457,15 +438,16 @@ ta_status ta_run_correlate(ta_window *h, ta_join_summary *out_summary) {
   a.slot_min = h->d_slot_min; a.slot_max = h->d_slot_max; a.slot_base = h->d_slot_base;  // filled by the sort
   a.launch_of = launch_of; a.kol = kol; a.kernel_of = h->d_kernel_of; a.multi = (u32 *)&h->d_status[ST_MULTI]; a.latency = latency; a.qdelay = qdelay; a.sum = d_sum;
   a.status = h->d_status;
-  const unsigned grid = (unsigned)((n + JN_TILE - 1) / JN_TILE);
-  const unsigned grid8 = (unsigned)((n + JS_TILE - 1) / JS_TILE);
   // Rows per warp: 12, fewer where that would be less than a round of the 148 * 24 warps on the chip
   // (1.2 M records: 101 us with 12, 90 with 8), 24 where it leaves twenty rounds and more (66.8 M: 730 us
   // with 12, 690 with 24; 16.8 M: 182 with 12, 233 with 32, whose last warps run long).
   int64_t rows = n / 32 / (148 * 32);
   rows = rows < JP_ROWS ? JP_ROWS : rows > 12 ? 12 : rows / JP_ROWS * JP_ROWS;
   if (n > (int64_t)20 * 148 * 24 * 24 * 32) rows = 24;
-  const unsigned grid_probe = (unsigned)((n + rows * JP_THREADS - 1) / (rows * JP_THREADS));
+  const unsigned grid = (unsigned)((n + rows * JN_THREADS - 1) / (rows * JN_THREADS));
+  int64_t brows = n / 32 / (148 * 32);  // (of k_join_build, the same way)
+  brows = brows < JB_ROWS ? JB_ROWS : brows > 16 ? 16 : brows / JB_ROWS * JB_ROWS;
+  const unsigned bgrid = (unsigned)((n + brows * JN_THREADS - 1) / (brows * JN_THREADS));
   void *tmp_alloc = nullptr;
   bool direct = true;
   int32_t words[ST_WORDS];
@@ -494,13 +476,11 @@ ta_status ta_run_correlate(ta_window *h, ta_join_summary *out_summary) {
     if (!tmp_alloc) return zs;
     a.table = (u32 *)tmp_alloc;
     if (direct) {
-      ta_launch(k_join_build<true>, grid, JN_THREADS, 0, st, a);
-      ta_launch(k_join_probe<true>, grid_probe, JP_THREADS, 0, st, a, (int)rows);
-      ta_launch(k_join_launch_stats<true>, grid8, JP_THREADS, 0, st, a, ta_tail(h, grid8));
+      ta_launch(k_join_build<true>, bgrid, JN_THREADS, 0, st, a, (int)brows);
+      ta_launch(k_join_probe<true>, grid, JN_THREADS, 0, st, a, (int)rows, ta_tail(h, grid));
     } else {
-      ta_launch(k_join_build<false>, grid, JN_THREADS, 0, st, a);
-      ta_launch(k_join_probe<false>, grid_probe, JP_THREADS, 0, st, a, (int)rows);
-      ta_launch(k_join_launch_stats<false>, grid8, JP_THREADS, 0, st, a, ta_tail(h, grid8));
+      ta_launch(k_join_build<false>, bgrid, JN_THREADS, 0, st, a, (int)brows);
+      ta_launch(k_join_probe<false>, grid, JN_THREADS, 0, st, a, (int)rows, ta_tail(h, grid));
     }
     TA_CHECK_CUDA(h, cudaGetLastError());
   }

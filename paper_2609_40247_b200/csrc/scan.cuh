@@ -231,10 +231,10 @@ __device__ __forceinline__ void storen_i32(int32_t *col, int64_t p0, int64_t n, 
   }
 }
 
-// Ordered compaction of the sorted positions whose kind is in `kind_mask`: 256 threads x 16
+// Ordered compaction of the sorted positions whose kind is in `kind_mask`: 256 threads x 32
 // positions per tile, vector loads of the kind column, one tile scan.
 #define CK_THREADS 256
-#define CK_ITEMS 16
+#define CK_ITEMS 32  // (16: 200 us of 66.8 M records instead of 172)
 #define CK_TILE (CK_THREADS * CK_ITEMS)
 // zero_col (may be null): an n-sized 64-bit column the caller needs cleared; the kernel reads two
 // bytes per record and has the bandwidth to write it on the way (positions below zero_n that its
@@ -265,8 +265,8 @@ static __global__ void __launch_bounds__(CK_THREADS) k_compact_kind(const int16_
     }
   }
   int16_t kd[CK_ITEMS];
-  load8_i16(kind, p0, n_valid, -1, kd);
-  load8_i16(kind, p0 + 8, n_valid, -1, kd + 8);
+#pragma unroll
+  for (int j = 0; j < CK_ITEMS; j += 8) load8_i16(kind, p0 + j, n_valid, -1, kd + j);
   u32 sel = 0;
 #pragma unroll
   for (int j = 0; j < CK_ITEMS; j++)
