@@ -186,6 +186,10 @@ struct __align__(128) DiscoverSmem {
   u32 count[DS_CACHE];  // records of that triple, in the window w_cnt, not yet added to the global counters
   u64 ccache[64];
   u32 hist[5][256];
+  // ranges and counts of the CTA's warps
+  int32_t mn, mx, qmn, qmx;
+  u32 n_coll, n_launch;
+  i64 md;
   int fail;
 };
 
@@ -201,6 +205,10 @@ __global__ void __launch_bounds__(DS_THREADS, 4) k_discover_staged(DiscoverArgs 
     mbar_init(&s.bar[0], 1);
     mbar_init(&s.bar[1], 1);
     s.fail = 0;
+    s.mn = s.qmn = INT32_MAX;
+    s.mx = s.qmx = INT32_MIN;
+    s.n_coll = s.n_launch = 0;
+    s.md = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
@@ -418,25 +426,37 @@ __global__ void __launch_bounds__(DS_THREADS, 4) k_discover_staged(DiscoverArgs 
     const u32 c = (&s.hist[0][0])[i];
     if (c) atomicAdd(&a.hist[i], c);
   }
+  // ranges and counts: on chip first, one thread's atomics per CTA (from every warp they queued up in
+  // one memory sector at the kernel's end)
   mn = __reduce_min_sync(0xffffffffu, mn);
   mx = __reduce_max_sync(0xffffffffu, mx);
   qmn = __reduce_min_sync(0xffffffffu, qmn);
   qmx = __reduce_max_sync(0xffffffffu, qmx);
   n_coll = __reduce_add_sync(0xffffffffu, n_coll);
   n_launch = __reduce_add_sync(0xffffffffu, n_launch);
-  if (lane == 0 && n_launch) atomicAdd((u64 *)&a.misc[8], (u64)n_launch);
   md = warp_max_i64(md);
-  if (lane == 0 && n_coll) {
-    atomicMin((i64 *)&a.misc[3], (i64)qmn);
-    atomicMax((i64 *)&a.misc[4], (i64)qmx);
-    atomicAdd((u64 *)&a.misc[5], (u64)n_coll);
-  }
   if (lane == 0) {
-    if (mn <= mx) {
-      atomicMin((i64 *)&a.misc[0], (i64)mn);
-      atomicMax((i64 *)&a.misc[1], (i64)mx);
+    atomicMin(&s.mn, mn);
+    atomicMax(&s.mx, mx);
+    atomicMin(&s.qmn, qmn);
+    atomicMax(&s.qmx, qmx);
+    if (n_coll) atomicAdd(&s.n_coll, n_coll);
+    if (n_launch) atomicAdd(&s.n_launch, n_launch);
+    if (md > 0) atomicMax(&s.md, md);
+  }
+  __syncthreads();
+  if (tid == 0) {
+    if (s.n_launch) atomicAdd((u64 *)&a.misc[8], (u64)s.n_launch);
+    if (s.n_coll) {
+      atomicMin((i64 *)&a.misc[3], (i64)s.qmn);
+      atomicMax((i64 *)&a.misc[4], (i64)s.qmx);
+      atomicAdd((u64 *)&a.misc[5], (u64)s.n_coll);
     }
-    if (md > 0) atomicMax((i64 *)&a.misc[2], md);
+    if (s.mn <= s.mx) {
+      atomicMin((i64 *)&a.misc[0], (i64)s.mn);
+      atomicMax((i64 *)&a.misc[1], (i64)s.mx);
+    }
+    if (s.md > 0) atomicMax((i64 *)&a.misc[2], s.md);
   }
 }
 
