@@ -36,23 +36,28 @@ static PyObject *wrap(PyObject *, PyObject *const *args, Py_ssize_t n) {
   }
 }
 
-// part(tensor, offset, length): the bytes [offset, offset + length) of a uint8 tensor made by wrap
+// part((first address, address behind, tensor made by wrap), address, nbytes): those bytes of the
+// tensor as one of its own, None if they are not its
 static PyObject *part(PyObject *, PyObject *const *args, Py_ssize_t n) {
-  if (n != 3 || !THPVariable_Check(args[0])) {
-    PyErr_SetString(PyExc_TypeError, "part(tensor, offset, length)");
+  if (n != 3 || !PyTuple_Check(args[0]) || PyTuple_GET_SIZE(args[0]) != 3) {
+    PyErr_SetString(PyExc_TypeError, "part((first, behind, tensor), address, nbytes)");
     return nullptr;
   }
-  const long long off = PyLong_AsLongLong(args[1]), len = PyLong_AsLongLong(args[2]);
+  const unsigned long long lo = PyLong_AsUnsignedLongLong(PyTuple_GET_ITEM(args[0], 0)),
+                           hi = PyLong_AsUnsignedLongLong(PyTuple_GET_ITEM(args[0], 1)),
+                           at = PyLong_AsUnsignedLongLong(args[1]), len = PyLong_AsUnsignedLongLong(args[2]);
   if (PyErr_Occurred()) return nullptr;
-  const at::Tensor &t = THPVariable_Unpack(args[0]);
-  if (off < 0 || len < 0 || t.dim() != 1 || off + len > t.numel()) {
-    PyErr_SetString(PyExc_IndexError, "part: outside the tensor");
+  PyObject *base = PyTuple_GET_ITEM(args[0], 2);
+  if (at < lo || at > hi || len > hi - at || !THPVariable_Check(base)) Py_RETURN_NONE;
+  const at::Tensor &t = THPVariable_Unpack(base);
+  if (t.dim() != 1 || (unsigned long long)t.numel() != hi - lo) {
+    PyErr_SetString(PyExc_ValueError, "part: not a tensor of these bytes");
     return nullptr;
   }
   at::Tensor r = at::detail::make_tensor<c10::TensorImpl>(c10::TensorImpl::VIEW, c10::Storage(t.storage()),
                                                           t.key_set(), t.dtype());
   c10::TensorImpl *impl = r.unsafeGetTensorImpl();
-  impl->set_storage_offset(t.storage_offset() + off);
+  impl->set_storage_offset(t.storage_offset() + (int64_t)(at - lo));
   impl->set_sizes_contiguous(at::IntArrayRef{(int64_t)len});
   return THPVariable_Wrap(std::move(r));
 }

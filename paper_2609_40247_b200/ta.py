@@ -261,6 +261,13 @@ def _addr(a):
     return a.__array_interface__["data"][0]
 
 
+def _rows(n, dtype):
+    """A zeroed table of n rows and its address (the array interface of a structured array describes
+    every field first)."""
+    raw = np.zeros(n * dtype.itemsize, dtype=np.uint8)
+    return raw.view(dtype), _addr(raw)
+
+
 # torch's caching allocator behind the ta_env callbacks: one pair of callbacks for all windows, the
 # context says which device and stream
 _places: list = [None]
@@ -352,21 +359,35 @@ class _Blocks:
         self.handle = handle
         self.known = []  # (first address, address behind, tensor)
         self.last = (0, 0, None)
+        self.none = None
 
     def part(self, ptr, nbytes):
+        wrap, part = _views()
         for self.last in self.known:
-            lo, hi, t = self.last
-            if lo <= ptr and ptr + nbytes <= hi:
-                return _part(t, ptr - lo, nbytes)
+            t = part(self.last, ptr, nbytes)
+            if t is not None:
+                return t
         h = self.handle
         base, room = _vp(), ctypes.c_uint64()
         if h.lib.ta_block_of(h.ptr, ptr, ctypes.byref(base), ctypes.byref(room)) != 0:
             raise ValueError("not a result of an open window")
         lo, size = base.value, room.value
-        wrap, part = _views()
         self.last = (lo, lo + size, wrap(lo, size, h.device, h))
         self.known.append(self.last)
-        return part(self.last[2], ptr - lo, nbytes)
+        return part(self.last, ptr, nbytes)
+
+    def drop(self):
+        """The window is closed: its memory goes back once no column made so far is in use."""
+        self.known.clear()
+        self.last = (0, 0, None)
+
+    def empty(self):
+        """A tensor of no bytes, a part of what is there as every result is."""
+        if self.none is None:
+            import torch
+            _views()
+            self.none = (0, 0, torch.empty(0, dtype=torch.uint8, device=f"cuda:{self.handle.device}"))
+        return _part(self.none, 0, 0)
 
 
 class _Result:
@@ -393,12 +414,9 @@ class _Result:
         nbytes = count(self) * size
         ptr = getattr(self._raw, field)
         if nbytes == 0 or not ptr:
-            import torch
-            return torch.empty(0, dtype=torch.uint8, device=f"cuda:{self._handle.device}")
-        lo, hi, t = self._blocks.last
-        if lo <= ptr and ptr + nbytes <= hi:
-            return _part(t, ptr - lo, nbytes)
-        return self._blocks.part(ptr, nbytes)
+            return self._blocks.empty()
+        t = _part(self._blocks.last, ptr, nbytes) if _part else None
+        return self._blocks.part(ptr, nbytes) if t is None else t
 
     # Tables are mostly read together: a request for one brings the other small ones of the result
     # along (a round trip costs more than their bytes), up to these limits.
@@ -631,13 +649,13 @@ class Window:
             else:
                 env.alloc, env.release, env.ctx = _torch_alloc, _torch_release, _place(dev, sptr)
                 if self.n <= CHUNK_RECORDS:
-                    self._take_chunk(env)
+                    self._take_chunk(env, stream)
         env.cuda_stream = sptr
         env.device = dev
-        self.load_summary = np.zeros(self.W, dtype=LOAD_SUM)
+        self.load_summary, summary_at = _rows(self.W, LOAD_SUM)
         st = L.ta_load_window(ctypes.byref(env), ev_ptr, self.n, 1 if on_device else 0,
                               _addr(self._off), _addr(self._t0), _addr(self._t1),
-                              self.W, _addr(self.load_summary), ctypes.byref(h.ptr))
+                              self.W, summary_at, ctypes.byref(h.ptr))
         if st != 0:
             self.close()
             raise TaError(st, "ta_load_window")
@@ -662,17 +680,15 @@ class Window:
 
         self._handle.callbacks = env.alloc, env.release = _ALLOC_T(_alloc), _RELEASE_T(_release)
 
-    def _take_chunk(self, env):
+    def _take_chunk(self, env, stream):
         import torch
         _views()
         h = self._handle
         size = CHUNK_BYTES_FIXED + self.n * CHUNK_BYTES_PER_RECORD
         try:
-            if torch.cuda.current_device() == h.device and torch.cuda.current_stream() == self.torch_stream:
-                t = torch.empty(size, dtype=torch.uint8, device="cuda")
-            else:
-                with torch.cuda.stream(self.torch_stream):
-                    t = torch.empty(size, dtype=torch.uint8, device=f"cuda:{h.device}")
+            # (without a stream of the caller's choice the window is on the device's current one)
+            with contextlib.nullcontext() if stream is None else torch.cuda.stream(stream):
+                t = torch.empty(size, dtype=torch.uint8, device=torch.device("cuda", h.device))
         except torch.cuda.OutOfMemoryError:
             return  # piece by piece, as far as it goes
         base = t.data_ptr()
@@ -691,6 +707,7 @@ class Window:
     # -- context manager / lifetime
     def close(self):
         self._handle.close()
+        self._blocks.drop()
 
     def __enter__(self):
         return self
@@ -715,8 +732,8 @@ class Window:
 
     def correlate_launches(self) -> JoinResult:
         raw = _JoinResult()
-        summ = np.zeros(self.W, dtype=JOIN_SUM)
-        st = self._lib.ta_correlate_launches(self._handle.ptr, ctypes.byref(raw), _addr(summ))
+        summ, at = _rows(self.W, JOIN_SUM)
+        st = self._lib.ta_correlate_launches(self._handle.ptr, ctypes.byref(raw), at)
         if st != 0:
             raise TaError(st, "ta_correlate_launches")
         return JoinResult(self, raw, dict(self._dims(), join_sum=summ))
@@ -725,8 +742,8 @@ class Window:
         """check=False returns the result even for TA_ERR_DEPTH / TA_ERR_BAD_NESTING
         (see .status); the summaries are valid, the other outputs unspecified."""
         raw = _AttrResult()
-        summ = np.zeros(self.W, dtype=ATTR_SUM)
-        st = self._lib.ta_attribute_operators(self._handle.ptr, ctypes.byref(raw), _addr(summ))
+        summ, at = _rows(self.W, ATTR_SUM)
+        st = self._lib.ta_attribute_operators(self._handle.ptr, ctypes.byref(raw), at)
         if st != 0 and (check or st not in (TA_ERR_DEPTH, TA_ERR_BAD_NESTING)):
             raise TaError(st, "ta_attribute_operators")
         return AttrResult(self, raw, dict(self._dims(), attr_sum=summ, status=st))
@@ -747,16 +764,16 @@ class Window:
 
     def rollup_operators(self) -> RollupResult:
         raw = _RollupResult()
-        summ = np.zeros(self.W, dtype=ROLLUP_SUM)
-        st = self._lib.ta_rollup_operators(self._handle.ptr, ctypes.byref(raw), _addr(summ))
+        summ, at = _rows(self.W, ROLLUP_SUM)
+        st = self._lib.ta_rollup_operators(self._handle.ptr, ctypes.byref(raw), at)
         if st != 0:
             raise TaError(st, "ta_rollup_operators")
         return RollupResult(self, raw, dict(self._dims(), rollup_sum=summ))
 
     def critical_path(self) -> CritpathResult:
         raw = _CritpathResult()
-        summ = np.zeros(self.W, dtype=CRITPATH_SUM)
-        st = self._lib.ta_critical_path(self._handle.ptr, ctypes.byref(raw), _addr(summ))
+        summ, at = _rows(self.W, CRITPATH_SUM)
+        st = self._lib.ta_critical_path(self._handle.ptr, ctypes.byref(raw), at)
         if st != 0:
             raise TaError(st, "ta_critical_path")
         return CritpathResult(self, raw, dict(self._dims(), n_rows=raw.n_rows, critpath_sum=summ))
@@ -764,8 +781,8 @@ class Window:
     def blame_gaps(self, gaps) -> BlameResult:
         """gaps: the GapResult of an earlier stream_gaps() call on this window."""
         raw = _BlameResult()
-        summ = np.zeros(self.W, dtype=BLAME_SUM)
-        st = self._lib.ta_blame_gaps(self._handle.ptr, ctypes.byref(gaps._raw), ctypes.byref(raw), _addr(summ))
+        summ, at = _rows(self.W, BLAME_SUM)
+        st = self._lib.ta_blame_gaps(self._handle.ptr, ctypes.byref(gaps._raw), ctypes.byref(raw), at)
         if st != 0:
             raise TaError(st, "ta_blame_gaps")
         return BlameResult(self, raw, dict(self._dims(), n_long_gaps=raw.n_long_gaps, blame_sum=summ))
@@ -774,7 +791,7 @@ class Window:
         """flops / nbytes: float64 per INPUT record (numpy arrays, or CUDA tensors on this
         window's device); negative or NaN = not known."""
         raw = _SolResult()
-        summ = np.zeros(self.W, dtype=SOL_SUM)
+        summ, at = _rows(self.W, SOL_SUM)
         on_device = hasattr(flops, "is_cuda")
         if on_device:
             import torch
@@ -789,7 +806,7 @@ class Window:
         if cnt != (self.n, self.n):
             raise ValueError("one operation count and one data volume per input record")
         st = self._lib.ta_operator_sol(self._handle.ptr, fp, bp, 1 if on_device else 0, float(peak_flops),
-                                       float(peak_bw), ctypes.byref(raw), _addr(summ))
+                                       float(peak_bw), ctypes.byref(raw), at)
         if st != 0:
             raise TaError(st, "ta_operator_sol")
         return SolResult(self, raw, dict(self._dims(), sol_sum=summ))
