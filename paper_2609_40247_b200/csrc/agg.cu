@@ -304,8 +304,7 @@ __global__ void __launch_bounds__(AG_THREADS) k_agg_mark(AggArgs a) {
 }
 
 template <bool TABLE>
-__global__ void __launch_bounds__(AG_THREADS, 6) k_agg(AggArgs a) {
-  TA_PDL();
+__device__ __forceinline__ void agg_chunk(const AggArgs &a) {
   __shared__ AggSmem s;
   if (ta_failed(a.status)) return;
   int since_flush = 0;
@@ -450,6 +449,49 @@ __global__ void __launch_bounds__(AC_THREADS) k_agg_rows(int64_t G, AggRowOut o,
     }
   }
   run_tail(tail);
+}
+
+// The same for a few cells, by the last CTA of k_agg.
+#define AG_ROWS_HERE AG_THREADS
+__device__ __forceinline__ void agg_rows_here(int G, const AggRowOut &o, u64 *total) {
+  __shared__ u64 tmp[33];
+  __shared__ u32 s_cell[AG_ROWS_HERE];
+  const int g = threadIdx.x;
+  const u64 c = g < G ? __ldcg(&o.cnt[g]) : 0;
+  u64 rows;
+  const u64 row = block_scan_exclusive<OpAdd>(c ? 1ull : 0ull, OpAdd(), tmp, &rows);
+  if (c) {
+    s_cell[row] = (u32)g;
+    const int slot = g / (int)o.R, r = g - slot * (int)o.R;
+    o.g_window[row] = slot / o.n_pids;
+    o.g_pid[row] = o.tt->pid_value[slot % o.n_pids];
+    o.g_name[row] = o.name_of ? o.name_of[r] : (int32_t)(o.min_name + r);
+    o.g_count[row] = (int64_t)c;
+    o.g_sum[row] = (int64_t)__ldcg(&o.sum[g]);
+    o.g_min[row] = (int64_t)((~__ldcg(&o.minc[g])) ^ (1ull << 63));
+    o.g_max[row] = (int64_t)(__ldcg(&o.maxb[g]) ^ (1ull << 63));
+  }
+  if (g == 0) {
+    *total = rows;
+    __threadfence();
+  }
+  __syncthreads();
+  const uint4 *src = reinterpret_cast<const uint4 *>(o.hist);
+  uint4 *dst = reinterpret_cast<uint4 *>(o.g_hist);
+  for (int i = g; i < (int)rows * (TA_NBINS / 4); i += AG_THREADS) {
+    const int r = i / (TA_NBINS / 4);
+    dst[i] = __ldcg(src + s_cell[r] * (TA_NBINS / 4) + (i - r * (TA_NBINS / 4)));
+  }
+}
+
+// rows_here: cells whose rows the last CTA compacts, 0 = none (k_agg_rows does, or there is nothing to compact)
+template <bool TABLE>
+__global__ void __launch_bounds__(AG_THREADS, 6) k_agg(AggArgs a, int rows_here, AggRowOut o, u64 *total, Tail tail) {
+  TA_PDL();
+  agg_chunk<TABLE>(a);
+  run_tail(tail, [&] {
+    if (rows_here && !ta_failed(a.status)) agg_rows_here(rows_here, o, total);
+  });
 }
 
 // ---- marked cells: numbering, and what is left to write of a row -----------------------------
@@ -771,16 +813,16 @@ ta_status ta_run_aggregate(ta_window *h, uint32_t kind_mask, int value_sel, ta_a
   a.per = (a.n_items + a.spread - 1) / a.spread;
   const int64_t blocks = (int64_t)a.spread * a.per;
 
-  auto run_agg = [&]() {
-    if (table) ta_launch(k_agg<true>, (unsigned)blocks, AG_THREADS, 0, st, a);
-    else ta_launch(k_agg<false>, (unsigned)blocks, AG_THREADS, 0, st, a);
-  };
 
   AggRowOut ro;
   memset(&ro, 0, sizeof(ro));
   ro.tt = h->d_triples; ro.n_pids = n_pids; ro.R = R; ro.min_name = h->min_name;
   ro.name_of = table ? h->d_name_of : nullptr;
   u64 ng = 0;
+  auto run_agg = [&](int rows_here, u64 *total, Tail tail) {
+    if (table) ta_launch(k_agg<true>, (unsigned)blocks, AG_THREADS, 0, st, a, rows_here, ro, total, tail);
+    else ta_launch(k_agg<false>, (unsigned)blocks, AG_THREADS, 0, st, a, rows_here, ro, total, tail);
+  };
   int32_t status[ST_WORDS];
   void *tmpb = nullptr, *outb = nullptr;
   // the three row tables (window, pid, symbol), the four 64-bit columns and the histograms of `rows` rows
@@ -814,14 +856,16 @@ ta_status ta_run_aggregate(ta_window *h, uint32_t kind_mask, int value_sel, ta_a
     a.d_maxb = ct.take<u64>(G);
     a.d_hist = ct.take<u32>((size_t)G * TA_NBINS);
     u64 *state = ct.take<u64>(tiles + 2), *total = state + tiles;
-    run_agg();
     // the rows are compacted without waiting for their count: it is bounded by cells and records
     carve_rows(G < h->n_valid ? G : h->n_valid);
     if (!outb) return TA_ERR_OOM;
     ro.cnt = a.d_cnt; ro.sum = a.d_sum; ro.minc = a.d_minc; ro.maxb = a.d_maxb; ro.hist = a.d_hist;
     TA_TRY(ta_queue_d2h(h, &ng, total, 8));
     TA_TRY(ta_queue_d2h(h, status, h->d_status, sizeof(status)));
-    ta_launch(k_agg_rows, (unsigned)tiles, AC_THREADS, 0, st, G, ro, state, total, (u32 *)(total + 1),
+    Tail here;
+    if (G <= AG_ROWS_HERE) here = ta_tail(h, blocks);
+    run_agg(here.m ? (int)G : 0, total, here);
+    if (here.m == 0) ta_launch(k_agg_rows, (unsigned)tiles, AC_THREADS, 0, st, G, ro, state, total, (u32 *)(total + 1),
               h->d_status, ta_tail(h, tiles));
   } else {
     const int64_t words = (G + 31) / 32;
@@ -847,7 +891,7 @@ ta_status ta_run_aggregate(ta_window *h, uint32_t kind_mask, int value_sel, ta_a
       a.rank = rank;
       a.d_cnt = (u64 *)ro.g_count; a.d_sum = (u64 *)ro.g_sum; a.d_minc = (u64 *)ro.g_min; a.d_maxb = (u64 *)ro.g_max;
       a.d_hist = ro.g_hist;
-      run_agg();
+      run_agg(0, nullptr, Tail());
       ta_launch(k_agg_marked_rows, (unsigned)((words + 255) / 256), 256, 0, st, a.bits, rank, words, ro, h->d_status);
     }
     TA_TRY(ta_queue_d2h(h, status, h->d_status, sizeof(status)));

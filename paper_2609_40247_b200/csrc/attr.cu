@@ -66,6 +66,10 @@ struct AttrArgs {
   struct AttrSpill *spill;   // what tiles owe to operators of earlier tiles
   u32 *n_spill;
   unsigned spill_blocks;     // k_attr_ops: so many CTAs in front work through that list
+  int fold_here;             // k_attr_resolve folds the stacks in front of a tile itself: tiles ...
+  const int32_t *group_meta; // ... and, of more than 32, groups of 32 tiles
+  const i64 *group_e;
+  const int32_t *group_pos;
 };
 struct AttrSpill {
   int32_t pos, cnt;
@@ -353,6 +357,44 @@ __device__ __forceinline__ void attr_pop(const AttrArgs &a, const AttrStack &st,
   __syncwarp();
 }
 
+// The stack open at the start of `tile`, whose lane begins in tile `from`: the stacks in between folded by
+// the warp that needs them, whole groups of 32 at a time.  At most 31 groups and 31 tiles, the next
+// one's entries on their way while one is combined: up to 1024 tiles this takes less than the two
+// launches (k_attr_fold_top, k_attr_fold_down) it stands for.
+__device__ __forceinline__ WStack attr_open(const AttrArgs &a, int64_t from, int64_t tile) {
+  const int lane = threadIdx.x & 31;
+  WStack acc;
+  acc.cnt = 0; acc.reset = 0; acc.e = 0; acc.pos = 0;
+  bool overflow = false;
+  auto take = [&](const int32_t *meta, const i64 *es, const int32_t *ps, int64_t b, int64_t e) {
+    int m1 = 0;
+    i64 e1 = 0;
+    int32_t p1 = 0;
+    auto ask = [&](int64_t t) {
+      m1 = meta[t];
+      if (lane < AT_CAP) { e1 = es[(size_t)t * AT_CAP + lane]; p1 = ps[(size_t)t * AT_CAP + lane]; }
+    };
+    if (b < e) ask(b);
+    for (int64_t t = b; t < e; t++) {
+      WStack x;
+      x.cnt = m1 & 0xFF;
+      x.reset = (m1 >> 8) & 1;
+      x.e = lane < x.cnt ? e1 : 0;
+      x.pos = lane < x.cnt ? p1 : 0;
+      if (t + 1 < e) ask(t + 1);
+      wstack_combine(acc, x, &overflow);
+      acc = x;
+    }
+  };
+  if ((from >> 5) < (tile >> 5)) {
+    take(a.group_meta, a.group_e, a.group_pos, from >> 5, tile >> 5);
+    from = tile & ~(int64_t)31;
+  }
+  take(a.agg_meta, a.agg_e, a.agg_pos, from, tile);
+  if (overflow && lane == 0) ta_set_err(a.status, TA_ERR_DEPTH);
+  return acc;
+}
+
 // kernels of an operator on the stack (one thread)
 __device__ __forceinline__ void attr_level_add(AttrStack &st, int k, u32 cnt, i64 first, i64 last, u64 ns) {
   st.cnt[k] += cnt;
@@ -384,10 +426,23 @@ __global__ void __launch_bounds__(AS_WARPS * 32, AS_MINB) k_attr_resolve(AttrArg
   int64_t pos = tile_start;
   int depth = 0, carried = 0;  // levels on the stack; of these, the lowest ones come from earlier tiles
   if (a.lane_domain[l] == 0 && (int64_t)a.lane_off[l] < tile_start) {
-    depth = carried = a.carry_cnt[tile];
+    i64 open_e = 0;
+    int32_t open_pos = 0;
+    if (a.fold_here) {
+      const WStack open = attr_open(a, (int64_t)a.lane_off[l] / TILE, tile);
+      depth = carried = open.cnt;
+      open_e = open.e;
+      open_pos = open.pos;
+    } else {
+      depth = carried = a.carry_cnt[tile];
+      if (lane < depth) {
+        open_e = a.carry_e[(size_t)tile * AT_CAP + lane];
+        open_pos = a.carry_pos[(size_t)tile * AT_CAP + lane];
+      }
+    }
     if (lane < depth) {
-      st.e[lane] = a.carry_e[(size_t)tile * AT_CAP + lane];
-      st.pos[lane] = a.carry_pos[(size_t)tile * AT_CAP + lane];
+      st.e[lane] = open_e;
+      st.pos[lane] = open_pos;
       st.first[lane] = INT64_MAX; st.last[lane] = INT64_MIN; st.ns[lane] = 0; st.cnt[lane] = 0;
     }
     __syncwarp();
@@ -612,8 +667,7 @@ __device__ __forceinline__ void attr_emit(ta_attr_summary *sm, const u64 *t) {
 }
 // MULTI: some launch has more than one kernel; those kernels are added to their operator here.
 template <bool MULTI>
-__global__ void __launch_bounds__(AT_THREADS, AT_OPS_MINB) k_attr_ops(AttrArgs a) {
-  TA_PDL();
+__device__ __forceinline__ void attr_ops(const AttrArgs &a) {
   constexpr int IT = AT_OPS_ITEMS;
   __shared__ u64 red[3][AT_THREADS / 32];
   __shared__ int s_lane0, s_lane1;
@@ -722,19 +776,27 @@ __global__ void __launch_bounds__(AT_THREADS, AT_OPS_MINB) k_attr_ops(AttrArgs a
 
 // operators that were open at the end of their tile and got no kernels from anywhere: no identities
 // are left behind
-__device__ __forceinline__ void attr_finalize(const AttrArgs &a) {
-  if (ta_failed(a.status)) return;
-  const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
+__device__ __forceinline__ void attr_finalize(const AttrArgs &a, int64_t i) {
   const int64_t tile = i / AT_CAP;
   const int k = (int)(i - tile * AT_CAP);
   if (tile >= a.n_tiles || k >= (a.agg_meta[tile] & 0xFF)) return;
   const int32_t r = a.agg_pos[i];
-  if (a.op_n[r] == 0) { a.op_first[r] = 0; a.op_last[r] = 0; }
+  if (__ldcg(&a.op_n[r]) == 0) { a.op_first[r] = 0; a.op_last[r] = 0; }
 }
 __global__ void __launch_bounds__(256) k_attr_finalize(AttrArgs a, Tail tail) {
   TA_PDL();
-  attr_finalize(a);
+  if (!ta_failed(a.status)) attr_finalize(a, (int64_t)blockIdx.x * 256 + threadIdx.x);
   run_tail(tail);
+}
+// With a tail the last CTA does the work of k_attr_finalize (of a few tiles).
+template <bool MULTI>
+__global__ void __launch_bounds__(AT_THREADS, AT_OPS_MINB) k_attr_ops(AttrArgs a, Tail tail) {
+  TA_PDL();
+  attr_ops<MULTI>(a);
+  run_tail(tail, [&] {
+    if (ta_failed(a.status)) return;
+    for (int64_t i = threadIdx.x; i < a.n_tiles * AT_CAP; i += AT_THREADS) attr_finalize(a, i);
+  });
 }
 
 ta_status ta_run_attribute(ta_window *h, ta_attr_summary *out_summary) {
@@ -810,10 +872,13 @@ ta_status ta_run_attribute(ta_window *h, ta_attr_summary *out_summary) {
         start[k] = StackArr{ct.take<int32_t>(c), ct.take<i64>(c * AT_CAP), ct.take<int32_t>(c * AT_CAP)};
       }
       const size_t top = level_n.size() - 1;
+      a.fold_here = top <= 1;
+      if (top == 1) { a.group_meta = node[1].meta; a.group_e = node[1].e; a.group_pos = node[1].pos; }
       for (size_t k = 1; k <= top; k++)
         ta_launch(k_attr_fold_up, (unsigned)((level_n[k] + 3) / 4), 128, 0, st, node[k - 1], level_n[k - 1], node[k], level_n[k], h->d_status);
-      ta_launch(k_attr_fold_top, 1, 32, 0, st, node[top], level_n[top], start[top], top == 0 ? 1 : 0, h->d_status);
-      for (size_t k = top; k >= 1; k--)
+      if (!a.fold_here)
+        ta_launch(k_attr_fold_top, 1, 32, 0, st, node[top], level_n[top], start[top], 0, h->d_status);
+      for (size_t k = top; k >= 1 && !a.fold_here; k--)
         ta_launch(k_attr_fold_down, (unsigned)((level_n[k] + 3) / 4), 128, 0, st, node[k - 1], level_n[k - 1], start[k], level_n[k], start[k - 1], k == 1 ? 1 : 0, h->d_status);
     }
     ta_launch(per_tile == 256 ? k_attr_resolve<256> : per_tile == 512 ? k_attr_resolve<512> : k_attr_resolve<1024>, wblocks, AS_WARPS * 32, 0, st, a);
@@ -821,10 +886,16 @@ ta_status ta_run_attribute(ta_window *h, ta_attr_summary *out_summary) {
     const int64_t sb = (tiles * 2 + AT_THREADS - 1) / AT_THREADS;
     a.spill_blocks = (unsigned)(sb < 148 * 2 ? sb : 148 * 2);
     const unsigned ob = a.spill_blocks + (unsigned)((n + AT_OPS_TILE - 1) / AT_OPS_TILE);
-    if (h->multi_launch) ta_launch(k_attr_ops<true>, ob, AT_THREADS, 0, st, a);
-    else ta_launch(k_attr_ops<false>, ob, AT_THREADS, 0, st, a);
-    const int64_t fb = (tiles * AT_CAP + 255) / 256;
-    ta_launch(k_attr_finalize, (unsigned)fb, 256, 0, st, a, ta_tail(h, fb));
+    // the last step in the last CTA of this one (16 entries per tile, so many a thread takes one by one)
+    const int64_t entries = tiles * AT_CAP;
+    Tail tail;
+    if (entries <= 16 * AT_THREADS) tail = ta_tail(h, ob);
+    if (h->multi_launch) ta_launch(k_attr_ops<true>, ob, AT_THREADS, 0, st, a, tail);
+    else ta_launch(k_attr_ops<false>, ob, AT_THREADS, 0, st, a, tail);
+    if (tail.m == 0) {
+      const int64_t fb = (entries + 255) / 256;
+      ta_launch(k_attr_finalize, (unsigned)fb, 256, 0, st, a, ta_tail(h, fb));
+    }
     TA_CHECK_CUDA(h, cudaGetLastError());
   }
   if (!small) TA_TRY(ta_queue_d2h(h, hs.data(), d_sum, W * sizeof(ta_attr_summary)));

@@ -406,8 +406,11 @@ __device__ __forceinline__ u64 td_wait(const u64 *p, int32_t *status, bool *time
   return w;
 }
 
-// End of a kernel that carries a tail; all threads of every CTA come here.
-__device__ __forceinline__ void run_tail(const Tail &t) {
+// End of a kernel that carries a tail; all threads of every CTA come here.  The last CTA to do so runs
+// `before` first: what is left to do once all others are through, where that is too little for a
+// launch of its own (it reads what they wrote with __ldcg).
+template <class Before>
+__device__ __forceinline__ void run_tail(const Tail &t, Before before) {
   __shared__ int s_last;
   if (t.m == 0) return;
   __syncthreads();
@@ -418,6 +421,7 @@ __device__ __forceinline__ void run_tail(const Tail &t) {
   __syncthreads();
   if (!s_last) return;
   __threadfence();
+  before();
   for (int e = 0; e < t.m; e++) {
     const u32 *s = (const u32 *)t.src[e];
     u32 *d = (u32 *)(t.pin_dev + t.off[e]);
@@ -428,6 +432,9 @@ __device__ __forceinline__ void run_tail(const Tail &t) {
     __threadfence_system();
     *t.seq_word = t.seq;
   }
+}
+__device__ __forceinline__ void run_tail(const Tail &t) {
+  run_tail(t, [] {});
 }
 
 struct OpAdd {

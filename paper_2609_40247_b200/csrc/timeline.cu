@@ -707,7 +707,8 @@ ta_status ta_run_sort_timeline(ta_window *h) {
       TA_TRY(ta_queue_d2h(h, q ? h->h_slot_max.data() : h->h_slot_min.data(), q ? h->d_slot_max : h->d_slot_min, n_slots * 8));
     const SlotRanges ranges{slot_code, n_slots, h->d_slot_min, h->d_slot_max, h->d_slot_base};
     if (n_codes <= LT_ONE_CTA || n == 0) {
-      ta_launch(k_lane_table, 1, 1024, 0, st, lane_start, n_codes, h->tbits, h->n_pids > 0 ? h->n_pids : 1, h->d_triples,
+      // (few codes: fewer warps to wait for at each of its barriers)
+      ta_launch(k_lane_table, 1, n_codes <= 256 && n_slots <= 256 ? 256 : 1024, 0, st, lane_start, n_codes, h->tbits, h->n_pids > 0 ? h->n_pids : 1, h->d_triples,
                 h->n_valid, lane_window, lane_pid, lane_stream, lane_domain, lane_off, lane_code, lane_slot,
                 lane_dom_end, lane_dom_next, lane_dev_base, n_lanes_dev, lane_cap, h->d_status, ranges, ta_tail(h, 1));
     } else {

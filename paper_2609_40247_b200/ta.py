@@ -407,6 +407,10 @@ class _Result:
         self._host = {}
         self.__dict__.update(extra or {})
 
+    def _spec(self, name):
+        _, dt, _, count = self._table[name]
+        return dt, int(count(self))
+
     def tensor(self, name):
         """Zero-copy torch view (uint8 for struct arrays) of a device result; valid while
         the window is open."""

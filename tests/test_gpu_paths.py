@@ -144,3 +144,51 @@ def test_operators_with_kernels_far_apart(name, scale):
     long = rng.choice(k, size=len(k) // 50, replace=False)
     ev["ts_end"][long] += rng.integers(0, 1 << 33, size=len(long))
     both(ev, wl.win_off, wl.win_t0, np.asarray(wl.win_t1) + 4_000_000_000, comm_sizes=wl.comm_sizes)
+
+
+@pytest.mark.parametrize("n", [255, 8_191, 8_192, 8_193, 16_385, 65_536, 65_537, 262_144, 262_145, 524_289])
+def test_one_deep_host_lane_of_many_tiles(n):
+    """A single host lane whose operators stay open across hundreds of tiles, around the sizes where
+    the stacks in front of a tile are folded by the tile itself, where the attribution's last step
+    moves into the operators' launch, and where tiles grow."""
+    rng = np.random.default_rng(n)
+    ev = np.zeros(n, dtype=synth.EVENT_DTYPE)
+    ev["pid"], ev["kind"] = 7, 0
+    ev["name_id"] = rng.integers(0, 5, size=n)
+    t0, span = 1_000_000, 4 * n + 64
+    ev["ts_start"] = t0 + 32 + 4 * np.arange(n)
+    ev["ts_end"] = ev["ts_start"] + 1
+    enc = 5  # nested operators around everything else
+    for d in range(enc):
+        ev["ts_start"][d], ev["ts_end"][d] = t0 + d, t0 + span - d
+    middle = [enc + (d + 1) * n // 5 for d in range(3)]
+    for k in middle:  # and around a seventh of the rest
+        ev["ts_end"][k] = ev["ts_start"][min(n - 1, k + n // 7)] - 1
+    launch = enc + 1 + np.arange((n - enc - 1) // 3) * 3
+    launch = launch[~np.isin(launch, middle)]
+    ev["kind"][launch] = 2
+    ev["corr_id"][launch] = np.arange(len(launch)) + 5
+    dev = launch[rng.random(len(launch)) < 0.5] + 1
+    dev = dev[(dev < n) & ~np.isin(dev, middle)]
+    ev["kind"][dev], ev["stream"][dev], ev["corr_id"][dev] = 3, 4, ev["corr_id"][dev - 1]
+    ev = ev[rng.permutation(n)]
+    o, _ = both(ev, np.array([0, n]), np.array([t0]), np.array([t0 + span + 1]))
+    assert o["attr_status"] == 0 and int(o["attr_sum"]["max_depth"].max()) >= 6
+
+
+@pytest.mark.parametrize("run", [1, 2, 3, 31, 32, 33, 47, 48, 49])
+@pytest.mark.parametrize("shift", [0, 5])
+def test_runs_of_one_coarse_time(run, shift):
+    """Records of one lane that begin at the same instant or a few ns apart, in runs inside a warp,
+    across its edge and beyond the length that is ranked in place."""
+    n = 20_000
+    rng = np.random.default_rng(run * 8 + shift)
+    ev = np.zeros(n, dtype=synth.EVENT_DTYPE)
+    ev["pid"], ev["kind"], ev["stream"] = 3, 3, 1 + (np.arange(n) < shift)
+    group = np.arange(n) // run
+    ev["ts_start"] = 500 + group * 1_500_000 + rng.integers(0, 3, size=n)
+    ev["ts_end"] = ev["ts_start"] + rng.integers(0, 3, size=n)
+    ev["corr_id"] = rng.integers(0, 50, size=n)
+    ev["name_id"] = rng.integers(0, 9, size=n)
+    ev = ev[rng.permutation(n)]
+    both(ev, np.array([0, n]), np.array([0]), np.array([int(ev["ts_end"].max()) + 1]))
