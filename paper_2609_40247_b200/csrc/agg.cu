@@ -394,12 +394,13 @@ struct AggRowOut {
   u32 *g_hist;
 };
 
-// Dense cells: compaction of the non-empty ones in cell (= key) order, AC_CELLS cells per CTA (few, so
-// that the thousands of cells of a window spread over many SMs), chained over the CTAs.  The histograms (160 of a row's 200 bytes) are copied by the CTA together, 16 bytes per
+// Dense cells: compaction of the non-empty ones in cell (= key) order, chained over the CTAs.  The histograms (160 of a row's 200 bytes) are copied by the CTA together, 16 bytes per
 // thread, rows side by side: one thread per row copying its own took 36 us for the 4096 cells of a
 // prefill window, most of it waiting.
 #define AC_THREADS 256
-#define AC_CELLS 64
+// Cells per CTA: 64 while a window has a few thousand; 256 beyond 4096, where all CTAs look back at once and
+// the length of the chain is what counts (62 k cells: 20 us with 977 CTAs).
+template <int AC_CELLS>
 __global__ void __launch_bounds__(AC_THREADS) k_agg_rows(int64_t G, AggRowOut o, u64 *state, u64 *total,
                                                          u32 *ticket, int32_t *status, Tail tail) {
   TA_PDL();
@@ -413,7 +414,12 @@ __global__ void __launch_bounds__(AC_THREADS) k_agg_rows(int64_t G, AggRowOut o,
   const int tile = s_tile;
   const int64_t g = tid < AC_CELLS ? (int64_t)tile * AC_CELLS + tid : G;
   const bool failed = ta_failed(status);
-  const u64 c = !failed && g < G ? o.cnt[g] : 0;
+  // everything a row takes is asked for before the CTAs in front are looked back at
+  const bool in = !failed && g < G;
+  const u64 c = in ? o.cnt[g] : 0, sum = in ? o.sum[g] : 0, minc = in ? o.minc[g] : 0, maxb = in ? o.maxb[g] : 0;
+  const int64_t slot = in ? g / o.R : 0, r = in ? g - slot * o.R : 0;
+  const int32_t pid = in ? o.tt->pid_value[slot % o.n_pids] : 0;
+  const int32_t name = in && o.name_of ? o.name_of[r] : (int32_t)(o.min_name + r);
   u64 rows;
   const u64 ex = block_scan_exclusive<OpAdd>(c ? 1ull : 0ull, OpAdd(), tmp, &rows);
   if (tid < 32) {
@@ -431,21 +437,28 @@ __global__ void __launch_bounds__(AC_THREADS) k_agg_rows(int64_t G, AggRowOut o,
     const u64 first = s_excl;
     if (c) {
       const u64 row = first + ex;
-      const int64_t slot = g / o.R, r = g - slot * o.R;
       o.g_window[row] = (int32_t)(slot / o.n_pids);
-      o.g_pid[row] = o.tt->pid_value[slot % o.n_pids];
-      o.g_name[row] = o.name_of ? o.name_of[r] : (int32_t)(o.min_name + r);
+      o.g_pid[row] = pid;
+      o.g_name[row] = name;
       o.g_count[row] = (int64_t)c;
-      o.g_sum[row] = (int64_t)o.sum[g];
-      o.g_min[row] = (int64_t)((~o.minc[g]) ^ (1ull << 63));
-      o.g_max[row] = (int64_t)(o.maxb[g] ^ (1ull << 63));
+      o.g_sum[row] = (int64_t)sum;
+      o.g_min[row] = (int64_t)((~minc) ^ (1ull << 63));
+      o.g_max[row] = (int64_t)(maxb ^ (1ull << 63));
     }
     const uint4 *src = reinterpret_cast<const uint4 *>(o.hist) + (size_t)tile * AC_CELLS * (TA_NBINS / 4);
     uint4 *dst = reinterpret_cast<uint4 *>(o.g_hist) + first * (TA_NBINS / 4);
     const int words = (int)rows * (TA_NBINS / 4);
-    for (int i = tid; i < words; i += AC_THREADS) {
-      const int r = i / (TA_NBINS / 4);
-      dst[i] = src[s_cell[r] * (TA_NBINS / 4) + (i - r * (TA_NBINS / 4))];
+    constexpr int BATCH = 5;
+    for (int i0 = tid; i0 < words; i0 += AC_THREADS * BATCH) {
+      uint4 v[BATCH];
+#pragma unroll
+      for (int k = 0; k < BATCH; k++) {
+        const int i = i0 + k * AC_THREADS, row = i / (TA_NBINS / 4);
+        if (i < words) v[k] = src[s_cell[row] * (TA_NBINS / 4) + (i - row * (TA_NBINS / 4))];
+      }
+#pragma unroll
+      for (int k = 0; k < BATCH; k++)
+        if (i0 + k * AC_THREADS < words) dst[i0 + k * AC_THREADS] = v[k];
     }
   }
   run_tail(tail);
@@ -844,7 +857,8 @@ ta_status ta_run_aggregate(ta_window *h, uint32_t kind_mask, int value_sel, ta_a
   // (pass, scan, round trip) are worth.  512 windows of 65 k records have 33 M cells, one in
   // twenty of them occupied: 1.85 ms per call dense.
   if (G * 232 <= 8 * h->n_valid + (64ll << 20)) {
-    const int64_t tiles = (G + AC_CELLS - 1) / AC_CELLS;
+    const int cells = G <= 4096 ? 64 : 256;
+    const int64_t tiles = (G + cells - 1) / cells;
     size_t tb = 4 * Carver::pad((size_t)G * 8) + Carver::pad((size_t)G * TA_NBINS * 4) + Carver::pad((size_t)(tiles + 2) * 8);
     ta_status zs;
     tmpb = ta_zalloc(h, tb, &zs);
@@ -865,7 +879,7 @@ ta_status ta_run_aggregate(ta_window *h, uint32_t kind_mask, int value_sel, ta_a
     Tail here;
     if (G <= AG_ROWS_HERE) here = ta_tail(h, blocks);
     run_agg(here.m ? (int)G : 0, total, here);
-    if (here.m == 0) ta_launch(k_agg_rows, (unsigned)tiles, AC_THREADS, 0, st, G, ro, state, total, (u32 *)(total + 1),
+    if (here.m == 0) ta_launch(cells == 64 ? k_agg_rows<64> : k_agg_rows<256>, (unsigned)tiles, AC_THREADS, 0, st, G, ro, state, total, (u32 *)(total + 1),
               h->d_status, ta_tail(h, tiles));
   } else {
     const int64_t words = (G + 31) / 32;

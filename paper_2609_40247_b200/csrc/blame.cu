@@ -25,6 +25,7 @@
 #define BL_THREADS 256
 #define BL_TILE (BL_THREADS * 4)
 #define BL_LANES 64
+#define BL_GAPS 768    // gaps staged on chip: 18 KB, five CTAs per SM
 
 struct BlameArgs {
   int64_t n, n_valid, m;  // m = long gaps
@@ -107,40 +108,71 @@ __global__ void __launch_bounds__(256) k_blame_lanes(BlameArgs a) {
   a.lane_first[l] = (int32_t)lo;
 }
 
-// number of gaps of list range [first, last) that start before time t
-__device__ __forceinline__ int64_t gaps_started_before(const BlameArgs &a, int64_t first, int64_t last,
-                                                       i64 t) {
+// Long gaps by index, in the list or in a part of it staged on chip.
+struct GapList {
+  const ta_long_gap *list;
+  const u64 *before;  // total length in front of an entry
+  __device__ __forceinline__ i64 start(int64_t i) const { return list[i].gap_start; }
+  __device__ __forceinline__ i64 len(int64_t i) const { return list[i].gap_len; }
+  __device__ __forceinline__ u64 pre(int64_t i) const { return before[i]; }
+};
+struct GapStage {
+  const i64 *starts, *lens;
+  const u64 *before;
+  __device__ __forceinline__ i64 start(int64_t i) const { return starts[i]; }
+  __device__ __forceinline__ i64 len(int64_t i) const { return lens[i]; }
+  __device__ __forceinline__ u64 pre(int64_t i) const { return before[i]; }
+};
+// number of gaps of the range [first, last) that start before time t
+template <class Gaps>
+__device__ __forceinline__ int64_t gaps_started_before(const Gaps &g, int64_t first, int64_t last, i64 t) {
   int64_t lo = first, hi = last;
   while (lo < hi) {
     const int64_t mid = (lo + hi) >> 1;
-    if (a.list[mid].gap_start < t) lo = mid + 1;
+    if (g.start(mid) < t) lo = mid + 1;
     else hi = mid;
   }
   return lo;
 }
+// the same by a warp, 32 gaps at a time
+template <class Gaps>
+__device__ __forceinline__ int64_t warp_gaps_started_before(const Gaps &g, int64_t first, int64_t last, i64 t) {
+  const int lane = threadIdx.x & 31;
+  int64_t lo = first, hi = last;
+  while (lo < hi) {
+    const int64_t step = (hi - lo + 31) >> 5, i = lo + lane * step;
+    const int c = __popc(__ballot_sync(0xffffffffu, i < hi && g.start(i) < t));
+    if (c == 0) break;
+    hi = min(hi, lo + c * step);
+    lo += (c - 1) * step + 1;
+  }
+  return lo;
+}
 // total long-gap length of the range that lies before time t, given i = gaps_started_before(t)
-__device__ __forceinline__ i64 gap_time_before(const BlameArgs &a, int64_t first, int64_t i, i64 t) {
+template <class Gaps>
+__device__ __forceinline__ i64 gap_time_before(const Gaps &g, int64_t first, int64_t i, i64 t) {
   if (i == first) return 0;
   const int64_t k = i - 1;
-  const i64 part = t - a.list[k].gap_start, len = a.list[k].gap_len;
-  return (i64)(a.pre[k] - a.pre[first]) + (part < len ? part : len);
+  const i64 part = t - g.start(k), len = g.len(k);
+  return (i64)(g.pre(k) - g.pre(first)) + (part < len ? part : len);
 }
 // length of [s, e) that lies inside the gaps of the range
-__device__ __forceinline__ i64 gap_time_within(const BlameArgs &a, int64_t first, int64_t last, i64 s,
-                                               i64 e) {
-  const int64_t ie = gaps_started_before(a, first, last, e);
+template <class Gaps>
+__device__ __forceinline__ i64 gap_time_within(const Gaps &g, int64_t first, int64_t last, i64 s, i64 e) {
+  const int64_t ie = gaps_started_before(g, first, last, e);
   if (ie == first) return 0;  // every gap starts at or after e
-  const ta_long_gap g = a.list[ie - 1];
-  if (g.gap_start < s && g.gap_start + g.gap_len <= s) return 0;  // the last gap before e ends before s
-  const int64_t is = g.gap_start < s ? ie : gaps_started_before(a, first, ie, s);
-  return gap_time_before(a, first, ie, e) - gap_time_before(a, first, is, s);
+  const i64 start = g.start(ie - 1);
+  if (start < s && start + g.len(ie - 1) <= s) return 0;  // the last gap before e ends before s
+  const int64_t is = start < s ? ie : gaps_started_before(g, first, ie, s);
+  return gap_time_before(g, first, ie, e) - gap_time_before(g, first, is, s);
 }
 
 // One tile of 1024 positions per CTA.  An operator's charge is two binary searches in each of its
 // process's streams, a chain of some thirty dependent reads per stream; the operators of the tile are
 // listed first and the (operator, stream) pairs are dealt out over the threads, so that no lane idles
 // beside a launch record and no thread walks eight streams one after the other (one thread per eight
-// records: 120 us for a prefill window of 250 k records, 195 us for 8 M decode records).
+// records: 120 us for a prefill window of 250 k records, 195 us for 8 M decode records).  The gaps
+// that can matter to the tile are few, as a rule, and are searched on chip.
 __device__ __forceinline__ void blame_ops(const BlameArgs &a) {
   __shared__ int s_lane0, s_n, s_most;
   __shared__ u64 s_sum[BL_TILE];
@@ -150,6 +182,9 @@ __device__ __forceinline__ void blame_ops(const BlameArgs &a) {
   __shared__ int s_d0;                       // first device lane of the tile's operators, -1: there are several processes
   __shared__ i64 s_from, s_to;               // earliest start, latest end among them
   __shared__ int32_t s_lo[BL_LANES], s_hi[BL_LANES];  // per stream: the gaps that can matter to them
+  __shared__ int32_t s_at[BL_LANES + 1];              // and where they are staged
+  __shared__ i64 s_start[BL_GAPS], s_len[BL_GAPS];
+  __shared__ u64 s_pre[BL_GAPS];
   if (ta_failed(a.status)) return;
   const int tid = threadIdx.x;
   const int64_t tile_start = (int64_t)blockIdx.x * BL_TILE;
@@ -165,30 +200,51 @@ __device__ __forceinline__ void blame_ops(const BlameArgs &a) {
   int l = l0, cur = -1, dlo = 0, dn = 0;
   i64 from = INT64_MAX, to = INT64_MIN;
   int64_t next_off = a.lane_off[l + 1];
+  constexpr int PER = BL_TILE / BL_THREADS;
+  bool op[PER];
 #pragma unroll
-  for (int k = 0; k < BL_TILE / BL_THREADS; k++) {
+  for (int k = 0; k < PER; k++) {
+    const int64_t p = tile_start + k * BL_THREADS + tid;
+    op[k] = p < tile_end && a.kind[p] == TA_KIND_OP;
+  }
+  i64 ps[PER], pe[PER];
+#pragma unroll
+  for (int k = 0; k < PER; k++) {
+    const int64_t p = tile_start + k * BL_THREADS + tid;
+    ps[k] = op[k] ? (i64)a.ts[p] : INT64_MAX;
+    pe[k] = op[k] ? (i64)a.te[p] : INT64_MIN;
+  }
+#pragma unroll
+  for (int k = 0; k < PER; k++) {
     const int x = k * BL_THREADS + tid;
     const int64_t p = tile_start + x;
-    if (p >= tile_end || a.kind[p] != TA_KIND_OP) continue;
-    while (p >= next_off) { l++; next_off = a.lane_off[l + 1]; }
-    if (l != cur) {  // device lanes of the record's (window, process)
-      cur = l;
-      dlo = a.lane_dom_next[l];
-      int dhi = dlo;
-      const int slot = a.lane_slot[l];
-      while (dhi < a.n_lanes && a.lane_domain[dhi] == 1 && a.lane_slot[dhi] == slot) dhi++;
-      dn = dhi - dlo;
+    if (op[k]) {
+      while (p >= next_off) { l++; next_off = a.lane_off[l + 1]; }
+      if (l != cur) {  // device lanes of the record's (window, process)
+        cur = l;
+        dlo = a.lane_dom_next[l];
+        int dhi = dlo;
+        const int slot = a.lane_slot[l];
+        while (dhi < a.n_lanes && a.lane_domain[dhi] == 1 && a.lane_slot[dhi] == slot) dhi++;
+        dn = dhi - dlo;
+      }
     }
-    if (dn == 0) continue;
-    const int i = atomicAdd(&s_n, 1);
+    // the warp's operators take their places with one add
+    const bool take = op[k] && dn > 0;
+    const u32 m = __ballot_sync(0xffffffffu, take);
+    if (m == 0) continue;
+    int base = 0;
+    if ((tid & 31) == 0) base = atomicAdd(&s_n, __popc(m));
+    const int i = __shfl_sync(0xffffffffu, base, 0) + __popc(m & ((1u << (tid & 31)) - 1u));
+    if (!take) continue;
     s_op[i] = (uint16_t)x;
     s_dlo[i] = dlo;
     s_dn[i] = (uint16_t)dn;
     s_sum[i] = 0;
     if (dn > s_most) atomicMax(&s_most, dn);
     if (s_d0 != dlo && atomicCAS(&s_d0, -2, dlo) != -2 && s_d0 != dlo) s_d0 = -1;
-    from = min(from, (i64)a.ts[p]);
-    to = max(to, (i64)a.te[p]);
+    from = min(from, ps[k]);
+    to = max(to, pe[k]);
   }
   from = (i64)(~warp_reduce(~((u64)from ^ (1ull << 63)), OpMax()) ^ (1ull << 63));
   to = (i64)(warp_reduce((u64)to ^ (1ull << 63), OpMax()) ^ (1ull << 63));
@@ -198,20 +254,53 @@ __device__ __forceinline__ void blame_ops(const BlameArgs &a) {
   // Operators of one tile lie close together in time: with one search per stream for all of them, each
   // has to look among a few gaps only.
   const bool one = s_d0 >= 0 && most <= BL_LANES;
-  if (one && tid < most) {
-    const int64_t first = a.lane_first[s_d0 + tid], last = a.lane_first[s_d0 + tid + 1];
-    const int64_t lo = gaps_started_before(a, first, last, s_from);
-    s_lo[tid] = (int32_t)(lo > first ? lo - 1 : first);
-    s_hi[tid] = (int32_t)gaps_started_before(a, lo, last, s_to);
-  }
+  const GapList list{a.list, a.pre};
+  if (one)
+    for (int d = tid >> 5; d < most; d += BL_THREADS / 32) {  // a warp per stream
+      const int64_t first = a.lane_first[s_d0 + d], last = a.lane_first[s_d0 + d + 1];
+      const int64_t lo = warp_gaps_started_before(list, first, last, s_from);
+      const int64_t hi = warp_gaps_started_before(list, lo, last, s_to);
+      if ((tid & 31) == 0) {
+        s_lo[d] = (int32_t)(lo > first ? lo - 1 : first);
+        s_hi[d] = (int32_t)hi;
+      }
+    }
   if (one) __syncthreads();
+  bool staged = false;
+  if (one) {
+    if (tid == 0) {
+      int at = 0;
+      for (int d = 0; d < most; d++) {
+        s_at[d] = at;
+        at += s_hi[d] - s_lo[d];
+      }
+      s_at[most] = at;
+    }
+    __syncthreads();
+    staged = s_at[most] <= BL_GAPS;
+    if (staged) {
+      for (int d = tid >> 5; d < most; d += BL_THREADS / 32)
+        for (int k = tid & 31; k < s_hi[d] - s_lo[d]; k += 32) {
+          const int64_t g = s_lo[d] + k;
+          s_start[s_at[d] + k] = list.start(g);
+          s_len[s_at[d] + k] = list.len(g);
+          s_pre[s_at[d] + k] = list.pre(g);
+        }
+      __syncthreads();
+    }
+  }
+  const GapStage stage{s_start, s_len, s_pre};
   for (int q = tid; q < ops * most; q += BL_THREADS) {
     const int i = q / most, d = q - i * most;  // (a tile nearly always lies in one process: all pairs exist)
     if (d >= s_dn[i]) continue;
-    const int64_t first = one ? s_lo[d] : a.lane_first[s_dlo[i] + d], last = one ? s_hi[d] : a.lane_first[s_dlo[i] + d + 1];
-    if (first == last) continue;
     const int64_t p = tile_start + s_op[i];
-    const i64 t = gap_time_within(a, first, last, a.ts[p], a.te[p]);
+    i64 t = 0;
+    if (staged) {
+      if (s_at[d] < s_at[d + 1]) t = gap_time_within(stage, s_at[d], s_at[d + 1], a.ts[p], a.te[p]);
+    } else {
+      const int64_t first = one ? s_lo[d] : a.lane_first[s_dlo[i] + d], last = one ? s_hi[d] : a.lane_first[s_dlo[i] + d + 1];
+      if (first < last) t = gap_time_within(list, first, last, a.ts[p], a.te[p]);
+    }
     if (t) atomicAdd(&s_sum[i], (u64)t);
   }
   __syncthreads();

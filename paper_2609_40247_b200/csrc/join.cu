@@ -9,7 +9,7 @@
 //            range (they count up per process in real traces): the entry of
 //            corr_id - min.  Launches and kernels are time-ordered, so the
 //            table is touched nearly sequentially.
-//   hashed   any 64-bit ids: open addressing, twice as many entries as launches.
+//   hashed   any 64-bit ids: open addressing, two to four times as many entries as launches.
 //            An entry holds nothing but a position; whether it is the wanted key
 //            is read off the corr_id column and off the range of positions its
 //            (window, pid) occupies.
@@ -57,7 +57,7 @@ __device__ __forceinline__ bool join_same(const JoinArgs &a, u32 pos, int slot, 
   return a.corr[pos] == c && (i64)pos >= a.slot_pos[slot] && (i64)pos < a.slot_pos[slot + 1];
 }
 // entry of the key or the empty entry that ends its chain, from entry i on; v = what it holds.  Half
-// of the table is empty, so the walk ends (bounded by the table all the same).
+// of the table at least is empty, so the walk ends (bounded by the table all the same).
 __device__ __forceinline__ u32 join_find(const JoinArgs &a, u32 i, u32 v, int slot, i64 c) {
   for (u32 step = 0; v != 0 && !join_same(a, ~v, slot, c) && step < a.table_size; step++) {
     i = i + 1 == a.table_size ? 0 : i + 1;
@@ -182,25 +182,35 @@ __global__ void __launch_bounds__(JN_THREADS) k_join_build(JoinArgs a, int rows)
       const u32 q1 = q0 + 32 * JB_ROWS;
 #pragma unroll
       for (int r = 0; r < JB_ROWS; r++) launch_row(a, q1 + 32 * r, e, nx[r]);
-      u32 old[JB_ROWS];
+      u32 old[JB_ROWS], at[JB_ROWS];
 #pragma unroll
       for (int r = 0; r < JB_ROWS; r++) {
         const u32 q = q0 + 32 * r;
-        old[r] = 0;
+        old[r] = at[r] = 0;
         if (!x[r].launch) continue;
         if (DIRECT) {
           old[r] = atomicMax(&a.table[base + x[r].c], ~q);
-        } else {
-          u32 i = join_hash(a, slot, x[r].c);
-          for (u32 step = 0; step < a.table_size; step++) {
-            const u32 was = atomicCAS(&a.table[i], 0u, ~q);
-            if (was == 0) break;
-            if (join_same(a, ~was, slot, x[r].c)) {
-              atomicMax(&a.table[i], ~q);
-              old[r] = was;
+        } else {  // (the first entries of all rows together)
+          at[r] = join_hash(a, slot, x[r].c);
+          old[r] = atomicCAS(&a.table[at[r]], 0u, ~q);
+        }
+      }
+      if (!DIRECT) {
+        i64 cq[JB_ROWS];
+#pragma unroll
+        for (int r = 0; r < JB_ROWS; r++) cq[r] = old[r] ? a.corr[~old[r]] : 0;
+#pragma unroll
+        for (int r = 0; r < JB_ROWS; r++) {
+          const u32 q = q0 + 32 * r;
+          bool same = cq[r] == x[r].c;
+          for (u32 step = 0; old[r] && step < a.table_size; step++) {
+            if (same && (i64)~old[r] >= a.slot_pos[slot] && (i64)~old[r] < a.slot_pos[slot + 1]) {
+              atomicMax(&a.table[at[r]], ~q);
               break;
             }
-            i = i + 1 == a.table_size ? 0 : i + 1;
+            at[r] = at[r] + 1 == a.table_size ? 0 : at[r] + 1;
+            old[r] = atomicCAS(&a.table[at[r]], 0u, ~q);
+            same = old[r] && a.corr[~old[r]] == x[r].c;
           }
         }
       }
@@ -445,7 +455,7 @@ ta_status ta_run_correlate(ta_window *h, ta_join_summary *out_summary) {
   rows = rows < JP_ROWS ? JP_ROWS : rows > 12 ? 12 : rows / JP_ROWS * JP_ROWS;
   if (n > (int64_t)20 * 148 * 24 * 24 * 32) rows = 24;
   const unsigned grid = (unsigned)((n + rows * JN_THREADS - 1) / (rows * JN_THREADS));
-  int64_t brows = n / 32 / (148 * 32);  // (of k_join_build, the same way)
+  int64_t brows = n / 32 / (148 * 64);  // (of k_join_build, the same way)
   brows = brows < JB_ROWS ? JB_ROWS : brows > 16 ? 16 : brows / JB_ROWS * JB_ROWS;
   const unsigned bgrid = (unsigned)((n + brows * JN_THREADS - 1) / (brows * JN_THREADS));
   void *tmp_alloc = nullptr;
@@ -461,8 +471,9 @@ ta_status ta_run_correlate(ta_window *h, ta_join_summary *out_summary) {
       if (hmin[s] <= hmax[s]) total += (unsigned __int128)((uint64_t)hmax[s] - (uint64_t)hmin[s]) + 1;
     const uint64_t limit = (uint64_t)4 * (uint64_t)n + 65536;
     direct = total <= limit;
-    // entries of the table: the span of all ids, or twice the launches
-    const uint64_t M = direct ? (uint64_t)total : 2 * (uint64_t)h->n_launch + 1;
+    // entries of the table: the span of all ids, or twice the launches and more
+    // (four times while the table stays in the caches: shorter chains, and they are what the inserts wait for)
+    const uint64_t M = direct ? (uint64_t)total : (h->n_launch < (1 << 21) ? 4 : 2) * (uint64_t)h->n_launch + 1;
     if (!direct) {
       const size_t sb = Carver::pad((size_t)(n_slots + 1) * 4);
       void *sp = ta_dalloc(h, sb);
