@@ -357,40 +357,71 @@ __device__ __forceinline__ void attr_pop(const AttrArgs &a, const AttrStack &st,
   __syncwarp();
 }
 
-// The stack open at the start of `tile`, whose lane begins in tile `from`: the stacks in between folded by
-// the warp that needs them, whole groups of 32 at a time.  At most 31 groups and 31 tiles, the next
-// one's entries on their way while one is combined: up to 1024 tiles this takes less than the two
-// launches (k_attr_fold_top, k_attr_fold_down) it stands for.
-__device__ __forceinline__ WStack attr_open(const AttrArgs &a, int64_t from, int64_t tile) {
+// With fold_here the stacks in front of a tile are folded by the CTA that resolves it: the groups of 32
+// tiles in front of its own and the tiles of the group in front of its first, at most 31 and 24, are
+// dealt out over its warps, which leave eight partial folds on chip; every warp adds its CTA's tiles in
+// front of its own.  Up to 1024 tiles this takes less than the two launches (k_attr_fold_top,
+// k_attr_fold_down) it stands for.
+struct StackPart {
+  i64 e[AT_CAP];
+  int32_t pos[AT_CAP];
+  int cnt, reset;
+};
+// acc = acc (+) stacks [b, e) of an array, the next one's entries on their way while one is combined
+__device__ __forceinline__ void attr_take(WStack &acc, const int32_t *meta, const i64 *es, const int32_t *ps,
+                                          int64_t b, int64_t e, bool *overflow) {
+  const int lane = threadIdx.x & 31;
+  int m1 = 0;
+  i64 e1 = 0;
+  int32_t p1 = 0;
+  auto ask = [&](int64_t t) {
+    m1 = meta[t];
+    if (lane < AT_CAP) { e1 = es[(size_t)t * AT_CAP + lane]; p1 = ps[(size_t)t * AT_CAP + lane]; }
+  };
+  if (b < e) ask(b);
+  for (int64_t t = b; t < e; t++) {
+    WStack x;
+    x.cnt = m1 & 0xFF;
+    x.reset = (m1 >> 8) & 1;
+    x.e = lane < x.cnt ? e1 : 0;
+    x.pos = lane < x.cnt ? p1 : 0;
+    if (t + 1 < e) ask(t + 1);
+    wstack_combine(acc, x, overflow);
+    acc = x;
+  }
+}
+__device__ __forceinline__ void attr_parts(const AttrArgs &a, int64_t tile0, StackPart *part) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int groups = (int)(tile0 >> 5), m = groups + (int)(tile0 & 31);
+  const int b = warp * m / AS_WARPS, e = (warp + 1) * m / AS_WARPS;
+  WStack acc;
+  acc.cnt = 0; acc.reset = 0; acc.e = 0; acc.pos = 0;
+  bool overflow = false;
+  attr_take(acc, a.group_meta, a.group_e, a.group_pos, min(b, groups), min(e, groups), &overflow);
+  const int64_t first = (int64_t)groups * 32 - groups;  // tile of element i behind the groups: first + i
+  attr_take(acc, a.agg_meta, a.agg_e, a.agg_pos, first + max(b, groups), first + max(e, groups), &overflow);
+  if (lane < AT_CAP) { part[warp].e[lane] = acc.e; part[warp].pos[lane] = acc.pos; }
+  if (lane == 0) {
+    part[warp].cnt = acc.cnt;
+    part[warp].reset = acc.reset;
+    if (overflow) ta_set_err(a.status, TA_ERR_DEPTH);
+  }
+}
+__device__ __forceinline__ WStack attr_open(const AttrArgs &a, const StackPart *part, int64_t tile0, int64_t tile) {
   const int lane = threadIdx.x & 31;
   WStack acc;
   acc.cnt = 0; acc.reset = 0; acc.e = 0; acc.pos = 0;
   bool overflow = false;
-  auto take = [&](const int32_t *meta, const i64 *es, const int32_t *ps, int64_t b, int64_t e) {
-    int m1 = 0;
-    i64 e1 = 0;
-    int32_t p1 = 0;
-    auto ask = [&](int64_t t) {
-      m1 = meta[t];
-      if (lane < AT_CAP) { e1 = es[(size_t)t * AT_CAP + lane]; p1 = ps[(size_t)t * AT_CAP + lane]; }
-    };
-    if (b < e) ask(b);
-    for (int64_t t = b; t < e; t++) {
-      WStack x;
-      x.cnt = m1 & 0xFF;
-      x.reset = (m1 >> 8) & 1;
-      x.e = lane < x.cnt ? e1 : 0;
-      x.pos = lane < x.cnt ? p1 : 0;
-      if (t + 1 < e) ask(t + 1);
-      wstack_combine(acc, x, &overflow);
-      acc = x;
-    }
-  };
-  if ((from >> 5) < (tile >> 5)) {
-    take(a.group_meta, a.group_e, a.group_pos, from >> 5, tile >> 5);
-    from = tile & ~(int64_t)31;
+  for (int w = 0; w < AS_WARPS; w++) {
+    WStack x;
+    x.cnt = part[w].cnt;
+    x.reset = part[w].reset;
+    x.e = lane < x.cnt ? part[w].e[lane] : 0;
+    x.pos = lane < x.cnt ? part[w].pos[lane] : 0;
+    wstack_combine(acc, x, &overflow);
+    acc = x;
   }
-  take(a.agg_meta, a.agg_e, a.agg_pos, from, tile);
+  attr_take(acc, a.agg_meta, a.agg_e, a.agg_pos, tile0, tile, &overflow);
   if (overflow && lane == 0) ta_set_err(a.status, TA_ERR_DEPTH);
   return acc;
 }
@@ -407,10 +438,15 @@ template <int TILE>
 __global__ void __launch_bounds__(AS_WARPS * 32, AS_MINB) k_attr_resolve(AttrArgs a) {
   TA_PDL();
   __shared__ AttrStack s_stack[AS_WARPS];
+  __shared__ StackPart s_part[AS_WARPS];
   if (ta_failed(a.status)) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const u32 lt = (1u << lane) - 1u;
-  const int64_t tile = (int64_t)blockIdx.x * AS_WARPS + warp;
+  const int64_t tile0 = (int64_t)blockIdx.x * AS_WARPS, tile = tile0 + warp;
+  if (a.fold_here) {
+    attr_parts(a, tile0, s_part);
+    __syncthreads();
+  }
   if (tile >= a.n_tiles) return;
   AttrStack &st = s_stack[warp];
   const int64_t tile_start = tile * TILE, tile_end = min(tile_start + TILE, a.n), vend = min(tile_end, a.n_valid);
@@ -429,7 +465,7 @@ __global__ void __launch_bounds__(AS_WARPS * 32, AS_MINB) k_attr_resolve(AttrArg
     i64 open_e = 0;
     int32_t open_pos = 0;
     if (a.fold_here) {
-      const WStack open = attr_open(a, (int64_t)a.lane_off[l] / TILE, tile);
+      const WStack open = attr_open(a, s_part, tile0, tile);
       depth = carried = open.cnt;
       open_e = open.e;
       open_pos = open.pos;
