@@ -498,11 +498,11 @@ __device__ __forceinline__ void agg_rows_here(int G, const AggRowOut &o, u64 *to
 }
 
 // rows_here: cells whose rows the last CTA compacts, 0 = none (k_agg_rows does, or there is nothing to compact)
-template <bool TABLE>
+template <bool TABLE, bool TAIL>
 __global__ void __launch_bounds__(AG_THREADS, 6) k_agg(AggArgs a, int rows_here, AggRowOut o, u64 *total, Tail tail) {
   TA_PDL();
   agg_chunk<TABLE>(a);
-  run_tail(tail, [&] {
+  if (TAIL) run_tail(tail, [&] {
     if (rows_here && !ta_failed(a.status)) agg_rows_here(rows_here, o, total);
   });
 }
@@ -833,8 +833,8 @@ ta_status ta_run_aggregate(ta_window *h, uint32_t kind_mask, int value_sel, ta_a
   ro.name_of = table ? h->d_name_of : nullptr;
   u64 ng = 0;
   auto run_agg = [&](int rows_here, u64 *total, Tail tail) {
-    if (table) ta_launch(k_agg<true>, (unsigned)blocks, AG_THREADS, 0, st, a, rows_here, ro, total, tail);
-    else ta_launch(k_agg<false>, (unsigned)blocks, AG_THREADS, 0, st, a, rows_here, ro, total, tail);
+    auto kernel = table ? (tail.m ? k_agg<true, true> : k_agg<true, false>) : (tail.m ? k_agg<false, true> : k_agg<false, false>);
+    ta_launch(kernel, (unsigned)blocks, AG_THREADS, 0, st, a, rows_here, ro, total, tail);
   };
   int32_t status[ST_WORDS];
   void *tmpb = nullptr, *outb = nullptr;

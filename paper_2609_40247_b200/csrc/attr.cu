@@ -825,11 +825,11 @@ __global__ void __launch_bounds__(256) k_attr_finalize(AttrArgs a, Tail tail) {
   run_tail(tail);
 }
 // With a tail the last CTA does the work of k_attr_finalize (of a few tiles).
-template <bool MULTI>
+template <bool MULTI, bool TAIL>
 __global__ void __launch_bounds__(AT_THREADS, AT_OPS_MINB) k_attr_ops(AttrArgs a, Tail tail) {
   TA_PDL();
   attr_ops<MULTI>(a);
-  run_tail(tail, [&] {
+  if (TAIL) run_tail(tail, [&] {
     if (ta_failed(a.status)) return;
     for (int64_t i = threadIdx.x; i < a.n_tiles * AT_CAP; i += AT_THREADS) attr_finalize(a, i);
   });
@@ -926,8 +926,9 @@ ta_status ta_run_attribute(ta_window *h, ta_attr_summary *out_summary) {
     const int64_t entries = tiles * AT_CAP;
     Tail tail;
     if (entries <= 16 * AT_THREADS) tail = ta_tail(h, ob);
-    if (h->multi_launch) ta_launch(k_attr_ops<true>, ob, AT_THREADS, 0, st, a, tail);
-    else ta_launch(k_attr_ops<false>, ob, AT_THREADS, 0, st, a, tail);
+    auto ops = h->multi_launch ? (tail.m ? k_attr_ops<true, true> : k_attr_ops<true, false>)
+                               : (tail.m ? k_attr_ops<false, true> : k_attr_ops<false, false>);
+    ta_launch(ops, ob, AT_THREADS, 0, st, a, tail);
     if (tail.m == 0) {
       const int64_t fb = (entries + 255) / 256;
       ta_launch(k_attr_finalize, (unsigned)fb, 256, 0, st, a, ta_tail(h, fb));

@@ -307,10 +307,11 @@ __device__ __forceinline__ void blame_ops(const BlameArgs &a) {
   for (int i = tid; i < ops; i += BL_THREADS)
     if (s_sum[i]) a.op_gap_ns[tile_start + s_op[i]] = (i64)s_sum[i];
 }
+template <bool TAIL>
 __global__ void __launch_bounds__(BL_THREADS) k_blame_ops(BlameArgs a, Tail tail) {
   TA_PDL();
   blame_ops(a);
-  run_tail(tail);
+  if (TAIL) run_tail(tail);
 }
 
 ta_status ta_run_blame(ta_window *h, const ta_gap_result *gaps, ta_blame_result *out,
@@ -369,7 +370,7 @@ ta_status ta_run_blame(ta_window *h, const ta_gap_result *gaps, ta_blame_result 
   TA_TRY(ta_queue_d2h(h, hn.data(), a.win_ns, (size_t)W * 32));
   TA_TRY(ta_queue_d2h(h, words, h->d_status, sizeof(words)));
   const Tail tail = W * 32 <= 4096 ? ta_tail(h, tiles) : Tail();
-  ta_launch(k_blame_ops, (unsigned)tiles, BL_THREADS, 0, st, a, tail);
+  ta_launch(tail.m ? k_blame_ops<true> : k_blame_ops<false>, (unsigned)tiles, BL_THREADS, 0, st, a, tail);
   TA_CHECK_CUDA(h, cudaGetLastError());
   TA_TRY(ta_sync_fetch(h));
   ta_dfree(h, tmpb);

@@ -451,10 +451,11 @@ __device__ __forceinline__ void gaps_rows(const GapArgs &a, int rows) {
     }
   }
 }
+template <bool TAIL>
 __global__ void __launch_bounds__(GP_THREADS, GR_MINB) k_gaps_rows(GapArgs a, int rows, Tail tail) {
   TA_PDL();
   gaps_rows(a, rows);
-  run_tail(tail);
+  if (TAIL) run_tail(tail);
 }
 
 struct GapBitsIn {
@@ -547,7 +548,8 @@ ta_status ta_run_gaps(ta_window *h, int64_t min_gap, ta_gap_result *out) {
       int64_t rows = n / 32 / (148 * 16);
       rows = rows < 4 ? 4 : rows > GR_ROWS ? GR_ROWS : rows;
       const int64_t per_cta = rows * GP_THREADS, grid = (n + per_cta - 1) / per_cta;
-      ta_launch(k_gaps_rows, (unsigned)grid, GP_THREADS, 0, st, a, (int)rows, ta_tail(h, grid));
+      const Tail tail = ta_tail(h, grid);
+      ta_launch(tail.m ? k_gaps_rows<true> : k_gaps_rows<false>, (unsigned)grid, GP_THREADS, 0, st, a, (int)rows, tail);
     }
     TA_CHECK_CUDA(h, cudaGetLastError());
     TA_TRY(ta_sync_fetch(h));

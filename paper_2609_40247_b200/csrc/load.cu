@@ -72,23 +72,31 @@ __global__ void __launch_bounds__(PL_THREADS) k_plan(const ta_event *ev, int64_t
   }
   __shared__ u64 code[PL_SLOTS];
   __shared__ u32 cnt[PL_SLOTS];
-  __shared__ u32 s_max, s_valid;
+  __shared__ u32 s_max;
   for (int i = threadIdx.x; i < PL_SLOTS; i += PL_THREADS) { code[i] = TRIPLE_EMPTY; cnt[i] = 0; }
-  if (threadIdx.x == 0) { s_max = 0; s_valid = 0; }
+  if (threadIdx.x == 0) s_max = 0;
   __syncthreads();
   const int64_t S = n < (int64_t)PL_THREADS * PL_PER_THREAD ? n : (int64_t)PL_THREADS * PL_PER_THREAD;
+  // the thread's samples together, then the table (one sample after the other was a chain of four
+  // cold reads, window searches in between)
+  u64 mine[PL_PER_THREAD];
+#pragma unroll
   for (int j = 0; j < PL_PER_THREAD; j++) {
     const int64_t k = (int64_t)j * PL_THREADS + threadIdx.x;
-    if (k >= S) break;
+    mine[j] = TRIPLE_EMPTY;
+    if (k >= S) continue;
     const int64_t i = k * (n / S);  // S <= n: evenly spread, in range
     const Rec r = load_rec(ev, i);
     const int w = window_of(off, W, i);
-    if (defect_of(r, t0[w], t1[w])) continue;
-    atomicAdd(&s_valid, 1u);
     // lanes are per window: the window is part of the sampled code
-    const u64 c = triple_code(r.pid, r.kind, r.stream) ^ ((u64)w * 0x9E3779B97F4A7C15ull);
+    if (!defect_of(r, t0[w], t1[w]))
+      mine[j] = triple_code(r.pid, r.kind, r.stream) ^ ((u64)w * 0x9E3779B97F4A7C15ull);
+  }
+  for (int j = 0; j < PL_PER_THREAD; j++) {
+    const u64 c = mine[j];
+    if (c == TRIPLE_EMPTY) continue;
     u32 slot = hash_code(c) & (PL_SLOTS - 1);
-    for (int probe = 0; probe < 64; probe++) {  // a table that fills up only loses samples
+    for (int probe = 0; probe < 16; probe++) {  // a table that fills up only loses samples
       const u64 cur = code[slot];
       if (cur == c) { atomicAdd(&cnt[slot], 1u); break; }
       if (cur == TRIPLE_EMPTY) {

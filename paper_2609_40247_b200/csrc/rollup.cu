@@ -151,10 +151,11 @@ __device__ __forceinline__ void roll_finalize(const RollArgs &a) {
   }
 }
 
+template <bool TAIL>
 __global__ void __launch_bounds__(RO_THREADS) k_roll_finalize(RollArgs a, Tail tail) {
   TA_PDL();
   roll_finalize(a);
-  run_tail(tail);
+  if (TAIL) run_tail(tail);
 }
 
 ta_status ta_run_rollup(ta_window *h, ta_rollup_result *out, ta_rollup_summary *out_summary) {
@@ -197,7 +198,7 @@ ta_status ta_run_rollup(ta_window *h, ta_rollup_result *out, ta_rollup_summary *
   TA_TRY(ta_queue_d2h(h, hs.data(), a.win_sum, (size_t)W * 24));
   TA_TRY(ta_queue_d2h(h, words, h->d_status, sizeof(words)));
   const Tail tail = W * 24 <= 4096 ? ta_tail(h, tiles) : Tail();
-  ta_launch(k_roll_finalize, tiles, RO_THREADS, 0, st, a, tail);
+  ta_launch(tail.m ? k_roll_finalize<true> : k_roll_finalize<false>, tiles, RO_THREADS, 0, st, a, tail);
   TA_CHECK_CUDA(h, cudaGetLastError());
   TA_TRY(ta_sync_fetch(h));
   if (words[ST_ERR]) return (ta_status)words[ST_ERR];

@@ -227,11 +227,12 @@ __device__ __forceinline__ void operator_sol(const SolArgs &a, int64_t n_tiles, 
   if (cw >= 0) sol_flush(acc, &a.sum[cw], red);
 }
 
+template <bool TAIL>
 __global__ void __launch_bounds__(SO_THREADS) k_operator_sol(SolArgs a, int64_t n_tiles, int64_t tiles_per_cta,
                                                              int64_t stride, Tail tail) {
   TA_PDL();
   operator_sol(a, n_tiles, tiles_per_cta, stride);
-  run_tail(tail);
+  if (TAIL) run_tail(tail);
 }
 
 ta_status ta_run_sol(ta_window *h, const double *flops, const double *bytes, int on_device,
@@ -277,7 +278,7 @@ ta_status ta_run_sol(ta_window *h, const double *flops, const double *bytes, int
     const int64_t per = (n_tiles + ctas - 1) / ctas;
     const int64_t grid = (n_tiles + per - 1) / per;
     const Tail tail = W * sizeof(ta_sol_summary) <= 4096 ? ta_tail(h, grid) : Tail();
-    ta_launch(k_operator_sol, (unsigned)grid, SO_THREADS, 0, st, a, n_tiles, per,
+    ta_launch(tail.m ? k_operator_sol<true> : k_operator_sol<false>, (unsigned)grid, SO_THREADS, 0, st, a, n_tiles, per,
               W == 1 ? grid : (int64_t)1, tail);
     TA_CHECK_CUDA(h, cudaGetLastError());
   }

@@ -408,7 +408,9 @@ __device__ __forceinline__ u64 td_wait(const u64 *p, int32_t *status, bool *time
 
 // End of a kernel that carries a tail; all threads of every CTA come here.  The last CTA to do so runs
 // `before` first: what is left to do once all others are through, where that is too little for a
-// launch of its own (it reads what they wrote with __ldcg).
+// launch of its own (it reads what they wrote with __ldcg).  Large grids carry no tail, and their kernels
+// are compiled without one: code behind the body costs its early returns (k_join_probe on 512 windows
+// of 52 k records took 354 us with it, 279 without).
 template <class Before>
 __device__ __forceinline__ void run_tail(const Tail &t, Before before) {
   __shared__ int s_last;
