@@ -429,7 +429,7 @@ static size_t min_tile() {
 
 // Descriptors of all passes are cleared at once while that is little memory (keys-only passes: 1 KB
 // per tile and pass); for more records each keys-only pass has the one array cleared in front of it.
-#define RS_AT_ONCE (1ll << 20)
+#define RS_AT_ONCE (1ll << 24)
 static size_t state_bytes(int64_t n) {
   size_t tiles = (size_t)((n + (int64_t)min_tile() - 1) / (int64_t)min_tile());
   if (tiles == 0) tiles = 1;

@@ -453,13 +453,13 @@ static ta_status load_impl(ta_window *h, const ta_event *events, int32_t on_devi
   // are many windows), and everything that starts at zero, cleared by one fill: [status | load
   // summaries | digit histograms | triple table | communicator table | pool for the later calls]
   const size_t up_words = (size_t)(W + 1) + 2 * (size_t)W + 16;
-  // the pool: results and counters of the later calls (34 bytes per record), tile descriptors,
-  // lane tables and a few aggregate tables
+  // the pool: kernel counts (4 bytes per record), the join's table (some 2), the sort's descriptors (1.3),
+  // bitmaps, lane tables and a few aggregate tables; what does not fit is cleared by itself
   // records per window and triple slot, as long as a window's counters (32 KB) are small beside its words
   h->cnt_windows = W == 1 || (W <= 1024 && n / W >= 8192) ? W : 0;
   const size_t cnt_bytes = (size_t)(h->cnt_windows ? h->cnt_windows : 1) * TA_TRIPLE_SLOTS * 4;
   h->zero_used = 0;
-  h->zero_bytes = n <= TA_ZERO_POOL_RECORDS ? Carver::pad((size_t)n * 36 + (2u << 20)) : 0;
+  h->zero_bytes = n <= TA_ZERO_POOL_RECORDS ? Carver::pad((size_t)n * 16 + (3u << 20)) : 0;
   size_t bytes = Carver::pad(up_words * 8) + Carver::pad(ST_WORDS * 4) +
                  Carver::pad(sizeof(TripleTable)) + Carver::pad(sizeof(CommTable)) +
                  Carver::pad(W * sizeof(ta_load_summary)) + Carver::pad(10 * 256 * 4) +
