@@ -5,7 +5,7 @@
 //
 // In canonical order (ts_start ascending, ts_end descending) a properly nested
 // host lane has a simple structure: the innermost encloser of record i is the
-// nearest earlier OP that is still running when i starts.  Tiles of 256 to 1024 records, no kernel ever waits for another CTA:
+// nearest earlier OP that is still running when i starts.  Tiles of 128 to 1024 records, no kernel ever waits for another CTA:
 //   k_attr_agg     per tile, the stack of OPs that are still undominated at the
 //                  tile's end (at most TA_MAX_DEPTH + 1 entries when nesting is
 //                  legal);
@@ -839,11 +839,12 @@ ta_status ta_run_attribute(ta_window *h, ta_attr_summary *out_summary) {
   const int64_t n = h->n, nn = n > 0 ? n : 1;
   const int W = h->W;
   cudaStream_t st = h->stream;
-  // A warp takes a tile.  256 records while the stacks are folded in two levels, so that a window of some
-  // ten thousand records has work for more than a few SMs; 1024 from ten rounds of the 148 * 32 warps
-  // k_attr_resolve keeps on the chip (66.8 M records: 750 us instead of 782, and half the stacks); 512
-  // between, where the last round's slowest warps show (16.8 M: 263 us instead of 342).
-  const int per_tile = n <= 256ll * AT_FAN * AT_FAN ? 256 : n <= 10ll * 148 * 32 * 1024 ? 512 : 1024;
+  // A warp takes a tile.  Small tiles keep a warp's chain of rows short: 128 records while the CTA folds the
+  // stacks in front of its tiles itself (60 k records 400 us with 256, 387 with 128), 256 up to some
+  // three million (1.2 M: 833 with 512, 822), 1024 from ten rounds of the 148 * 32 warps
+  // k_attr_resolve keeps on the chip (66.8 M: 782 us of the kernel with 512, 750, and half the stacks); 512
+  // between, where the last round's slowest warps show (16.8 M: 342 us of the kernel with 1024, 263).
+  const int per_tile = n <= 128ll * AT_FAN * AT_FAN ? 128 : n <= (3 << 20) ? 256 : n <= 10ll * 148 * 32 * 1024 ? 512 : 1024;
   const int64_t tiles = (n + per_tile - 1) / per_tile;
   size_t keep = 3 * Carver::pad(nn * 4) + Carver::pad(nn) + 3 * Carver::pad(nn * 8) + 256;
   void *kb = ta_dalloc(h, keep);
@@ -896,7 +897,7 @@ ta_status ta_run_attribute(ta_window *h, ta_attr_summary *out_summary) {
   if (small) TA_TRY(ta_queue_d2h(h, hs.data(), d_sum, W * sizeof(ta_attr_summary)));
   if (n > 0) {
     const unsigned wblocks = (unsigned)((tiles + AS_WARPS - 1) / AS_WARPS);
-    ta_launch(per_tile == 256 ? k_attr_agg<256> : per_tile == 512 ? k_attr_agg<512> : k_attr_agg<1024>, wblocks, AT_THREADS, 0, st, a);
+    ta_launch(per_tile == 128 ? k_attr_agg<128> : per_tile == 256 ? k_attr_agg<256> : per_tile == 512 ? k_attr_agg<512> : k_attr_agg<1024>, wblocks, AT_THREADS, 0, st, a);
     {
       // level 0 = tiles; fold upwards until at most AT_FAN stacks remain, scan those, unfold
       std::vector<StackArr> node(level_n.size()), start(level_n.size());
@@ -917,15 +918,15 @@ ta_status ta_run_attribute(ta_window *h, ta_attr_summary *out_summary) {
       for (size_t k = top; k >= 1 && !a.fold_here; k--)
         ta_launch(k_attr_fold_down, (unsigned)((level_n[k] + 3) / 4), 128, 0, st, node[k - 1], level_n[k - 1], start[k], level_n[k], start[k - 1], k == 1 ? 1 : 0, h->d_status);
     }
-    ta_launch(per_tile == 256 ? k_attr_resolve<256> : per_tile == 512 ? k_attr_resolve<512> : k_attr_resolve<1024>, wblocks, AS_WARPS * 32, 0, st, a);
+    ta_launch(per_tile == 128 ? k_attr_resolve<128> : per_tile == 256 ? k_attr_resolve<256> : per_tile == 512 ? k_attr_resolve<512> : k_attr_resolve<1024>, wblocks, AS_WARPS * 32, 0, st, a);
     // (a tile owes something to few operators of earlier ones, as a rule)
     const int64_t sb = (tiles * 2 + AT_THREADS - 1) / AT_THREADS;
     a.spill_blocks = (unsigned)(sb < 148 * 2 ? sb : 148 * 2);
     const unsigned ob = a.spill_blocks + (unsigned)((n + AT_OPS_TILE - 1) / AT_OPS_TILE);
-    // the last step in the last CTA of this one (16 entries per tile, so many a thread takes one by one)
+    // the last step in the last CTA of this one, for a few tiles (16 entries each)
     const int64_t entries = tiles * AT_CAP;
     Tail tail;
-    if (entries <= 16 * AT_THREADS) tail = ta_tail(h, ob);
+    if (entries <= 4 * AT_THREADS) tail = ta_tail(h, ob);
     auto ops = h->multi_launch ? (tail.m ? k_attr_ops<true, true> : k_attr_ops<true, false>)
                                : (tail.m ? k_attr_ops<false, true> : k_attr_ops<false, false>);
     ta_launch(ops, ob, AT_THREADS, 0, st, a, tail);

@@ -146,7 +146,7 @@ def test_operators_with_kernels_far_apart(name, scale):
     both(ev, wl.win_off, wl.win_t0, np.asarray(wl.win_t1) + 4_000_000_000, comm_sizes=wl.comm_sizes)
 
 
-@pytest.mark.parametrize("n", [255, 8_191, 8_192, 8_193, 16_385, 65_536, 65_537, 262_144, 262_145, 524_289])
+@pytest.mark.parametrize("n", [255, 4_096, 4_097, 8_191, 8_192, 8_193, 16_385, 65_536, 65_537, 131_072, 131_073, 524_289])
 def test_one_deep_host_lane_of_many_tiles(n):
     """A single host lane whose operators stay open across hundreds of tiles, around the sizes where
     the stacks in front of a tile are folded by the tile itself, where the attribution's last step
