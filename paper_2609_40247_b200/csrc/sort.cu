@@ -372,6 +372,13 @@ __global__ void __launch_bounds__(THREADS, VALS ? RSP_MINB : RSK_MINB) k_radix_p
 #ifndef RSK_ITEMS
 #define RSK_ITEMS 16
 #endif
+// Up to RS_SMALL keys a pass waits for its one round of CTAs, not for the chip: half the keys per thread
+// (60 k records 384 -> 377 us for the whole analysis, 500 k 587 -> 575, 1.2 M 818 -> 810; a quarter
+// of them makes the look back longer than it saves).
+#define RSK_ITEMS_SMALL 8
+#ifndef RS_SMALL
+#define RS_SMALL (2ll << 20)
+#endif
 
 // digit histograms of every pass (used when the caller has none)
 __global__ void __launch_bounds__(256) k_radix_hist(const u64 *keys, int64_t n, SortPlan plan,
@@ -422,8 +429,8 @@ __global__ void __launch_bounds__(256) k_radix_scan_hist(const u32 *hist, u32 *b
 
 SortPlan ta_make_plan(int lo_bit, int hi_bit) { return ta_plan_bits(lo_bit, hi_bit); }
 
-static size_t min_tile() {
-  size_t a = (size_t)RSP_THREADS * RSP_ITEMS, b = (size_t)RSK_THREADS * RSK_ITEMS;
+static size_t min_tile(int64_t n) {
+  size_t a = (size_t)RSP_THREADS * RSP_ITEMS, b = (size_t)RSK_THREADS * (n <= RS_SMALL ? RSK_ITEMS_SMALL : RSK_ITEMS);
   return a < b ? a : b;
 }
 
@@ -431,7 +438,8 @@ static size_t min_tile() {
 // per tile and pass); for more records each keys-only pass has the one array cleared in front of it.
 #define RS_AT_ONCE (1ll << 24)
 static size_t state_bytes(int64_t n) {
-  size_t tiles = (size_t)((n + (int64_t)min_tile() - 1) / (int64_t)min_tile());
+  const int64_t tile = (int64_t)min_tile(n);
+  size_t tiles = (size_t)((n + tile - 1) / tile);
   if (tiles == 0) tiles = 1;
   return Carver::pad(tiles * RS_BINS * sizeof(u64) * (n <= RS_AT_ONCE ? 5 : 1));
 }
@@ -463,14 +471,13 @@ static cudaError_t launch_pass(const RadixArgs &a, int bits, unsigned tiles, cud
 // writes the final ones; keys_in / vals_in are only read (pairs with vals_in null:
 // the value of element i is i).  keys_in must not alias scratch or final.
 // `hist` = precomputed [pass][256] digit histograms, or null.
-template <bool VALS>
+template <bool VALS, int ITEMS>
 static ta_status radix_sort(ta_window *h, const u64 *keys_in, const u32 *vals_in, u64 *keys_scratch,
                             u32 *vals_scratch, u64 *keys_final, u32 *vals_final, int64_t n,
                             const SortPlan &plan, const u32 *hist, void *temp,
                             bool first_pass_unstable, const PrekeyInfo *prekey, const TopHist *top) {
   if (n <= 0) return TA_OK;
   constexpr int THREADS = VALS ? RSP_THREADS : RSK_THREADS;
-  constexpr int ITEMS = VALS ? RSP_ITEMS : RSK_ITEMS;
   constexpr int TILE = THREADS * ITEMS;
   size_t tiles = (size_t)((n + TILE - 1) / TILE);
   // what the sort has to find cleared, in one piece: tile descriptors, ticket counters (one per
@@ -540,13 +547,14 @@ ta_status ta_radix_sort_pairs(ta_window *h, const u64 *keys_in, const u32 *vals_
                               u64 *keys_scratch, u32 *vals_scratch, u64 *keys_final,
                               u32 *vals_final, int64_t n, const SortPlan &plan, const u32 *hist,
                               void *temp) {
-  return radix_sort<true>(h, keys_in, vals_in, keys_scratch, vals_scratch, keys_final, vals_final, n,
+  return radix_sort<true, RSP_ITEMS>(h, keys_in, vals_in, keys_scratch, vals_scratch, keys_final, vals_final, n,
                           plan, hist, temp, false, nullptr, nullptr);
 }
 
 ta_status ta_radix_sort_keys(ta_window *h, const u64 *keys_in, u64 *keys_scratch, u64 *keys_final,
                              int64_t n, const SortPlan &plan, const u32 *hist, void *temp,
                              bool first_pass_unstable, const PrekeyInfo *prekey, const TopHist *top) {
-  return radix_sort<false>(h, keys_in, nullptr, keys_scratch, nullptr, keys_final, nullptr, n, plan,
-                           hist, temp, first_pass_unstable, prekey, top);
+  auto sort = n <= RS_SMALL ? radix_sort<false, RSK_ITEMS_SMALL> : radix_sort<false, RSK_ITEMS>;
+  return sort(h, keys_in, nullptr, keys_scratch, nullptr, keys_final, nullptr, n, plan, hist, temp,
+              first_pass_unstable, prekey, top);
 }

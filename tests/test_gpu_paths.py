@@ -192,3 +192,11 @@ def test_runs_of_one_coarse_time(run, shift):
     ev["name_id"] = rng.integers(0, 9, size=n)
     ev = ev[rng.permutation(n)]
     both(ev, np.array([0, n]), np.array([0]), np.array([int(ev["ts_end"].max()) + 1]))
+
+
+@pytest.mark.parametrize("n", [2_047, 2_048, 2_049, 4_097, 2_097_152, 2_097_153])
+def test_sort_around_its_tiles_and_where_they_grow(n):
+    wl = synth.make_workload("c1", max(0.002, 1.03 * n / 4_194_304), truth=False)
+    ev = np.ascontiguousarray(wl.events[:n])
+    assert len(ev) == n
+    both(ev, [0, n], wl.win_t0, wl.win_t1, comm_sizes=wl.comm_sizes)
