@@ -376,6 +376,7 @@ __global__ void __launch_bounds__(THREADS, VALS ? RSP_MINB : RSK_MINB) k_radix_p
 // (60 k records 384 -> 377 us for the whole analysis, 500 k 587 -> 575, 1.2 M 818 -> 810; a quarter
 // of them makes the look back longer than it saves).
 #define RSK_ITEMS_SMALL 8
+#define RSP_ITEMS_SMALL 6  // pairs (100 k expert records, 8 k collectives: 628 -> 596 us)
 #ifndef RS_SMALL
 #define RS_SMALL (2ll << 20)
 #endif
@@ -430,7 +431,7 @@ __global__ void __launch_bounds__(256) k_radix_scan_hist(const u32 *hist, u32 *b
 SortPlan ta_make_plan(int lo_bit, int hi_bit) { return ta_plan_bits(lo_bit, hi_bit); }
 
 static size_t min_tile(int64_t n) {
-  size_t a = (size_t)RSP_THREADS * RSP_ITEMS, b = (size_t)RSK_THREADS * (n <= RS_SMALL ? RSK_ITEMS_SMALL : RSK_ITEMS);
+  size_t a = (size_t)RSP_THREADS * (n <= RS_SMALL ? RSP_ITEMS_SMALL : RSP_ITEMS), b = (size_t)RSK_THREADS * (n <= RS_SMALL ? RSK_ITEMS_SMALL : RSK_ITEMS);
   return a < b ? a : b;
 }
 
@@ -547,8 +548,9 @@ ta_status ta_radix_sort_pairs(ta_window *h, const u64 *keys_in, const u32 *vals_
                               u64 *keys_scratch, u32 *vals_scratch, u64 *keys_final,
                               u32 *vals_final, int64_t n, const SortPlan &plan, const u32 *hist,
                               void *temp) {
-  return radix_sort<true, RSP_ITEMS>(h, keys_in, vals_in, keys_scratch, vals_scratch, keys_final, vals_final, n,
-                          plan, hist, temp, false, nullptr, nullptr);
+  auto sort = n <= RS_SMALL ? radix_sort<true, RSP_ITEMS_SMALL> : radix_sort<true, RSP_ITEMS>;
+  return sort(h, keys_in, vals_in, keys_scratch, vals_scratch, keys_final, vals_final, n, plan, hist, temp, false,
+              nullptr, nullptr);
 }
 
 ta_status ta_radix_sort_keys(ta_window *h, const u64 *keys_in, u64 *keys_scratch, u64 *keys_final,
