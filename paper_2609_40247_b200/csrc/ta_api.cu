@@ -240,12 +240,16 @@ ta_status ta_queue_d2h(ta_window *h, void *dst, const void *dev_src, size_t byte
     h->fetch.push_back(ta_window::Fetch{dev_src, (unsigned)h->pin_used, (unsigned)bytes});
     h->pending.push_back(ta_window::Pending{dst, h->pin_used, bytes});
     h->pin_used += need;
-  } else if (h->pin && h->pin_used + need <= h->pin_bytes) {
-    TA_CHECK_CUDA(h, cudaMemcpyAsync(h->pin + h->pin_used, dev_src, bytes, cudaMemcpyDeviceToHost, h->stream));
-    h->pending.push_back(ta_window::Pending{dst, h->pin_used, bytes});
-    h->pin_used += need;
   } else {
-    TA_CHECK_CUDA(h, cudaMemcpyAsync(dst, dev_src, bytes, cudaMemcpyDeviceToHost, h->stream));
+    // a real copy: it is done when the stream is, not when the word of a tail taken in front of it appears
+    h->tail_seq = 0;
+    if (h->pin && h->pin_used + need <= h->pin_bytes) {
+      TA_CHECK_CUDA(h, cudaMemcpyAsync(h->pin + h->pin_used, dev_src, bytes, cudaMemcpyDeviceToHost, h->stream));
+      h->pending.push_back(ta_window::Pending{dst, h->pin_used, bytes});
+      h->pin_used += need;
+    } else {
+      TA_CHECK_CUDA(h, cudaMemcpyAsync(dst, dev_src, bytes, cudaMemcpyDeviceToHost, h->stream));
+    }
   }
   return TA_OK;
 }

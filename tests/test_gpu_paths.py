@@ -200,3 +200,40 @@ def test_sort_around_its_tiles_and_where_they_grow(n):
     ev = np.ascontiguousarray(wl.events[:n])
     assert len(ev) == n
     both(ev, [0, n], wl.win_t0, wl.win_t1, comm_sizes=wl.comm_sizes)
+
+
+def _many_small_windows(windows, pids, rng):
+    """A few records per process and window: an operator, a launch of two kernels (one of them in
+    a third of the windows), a wait, a collective and now and then a damaged record."""
+    rows = np.zeros((windows, pids, 6), dtype=synth.EVENT_DTYPE)
+    span = 5_000
+    t0 = 1_000_000 + span * np.arange(windows, dtype=np.int64)
+    at = t0[:, None] + rng.integers(0, 900, size=(windows, pids))
+    rows["pid"] = np.arange(pids)[None, :, None]
+    rows["name_id"] = rng.integers(0, 7, size=rows.shape)
+    for k, (kind, stream, begin, length) in enumerate((
+            (0, 0, 0, 2_000), (2, 0, 20, 30), (3, 1, 200, 300), (3, 1, 700, 250), (1, 0, 400, 1_200), (5, 1, 1_100, 100))):
+        e = rows[:, :, k]
+        e["kind"], e["stream"] = kind, stream
+        e["ts_start"] = at + begin + rng.integers(0, 15, size=at.shape)
+        e["ts_end"] = e["ts_start"] + length + rng.integers(0, 50, size=at.shape)
+    rows["corr_id"][:, :, 1:4] = 5 + rng.integers(0, 3, size=(windows, pids, 1))
+    rows["corr_id"][::3, :, 3] = -1
+    rows["corr_id"][:, :, 5], rows["seq"][:, :, 5] = 77, rng.integers(0, 2, size=(windows, 1))
+    rows["kind"][::5, 0, 4] = 9
+    ev = rows.reshape(windows, -1)
+    ev = ev[np.arange(windows)[:, None], rng.permuted(np.tile(np.arange(pids * 6), (windows, 1)), axis=1)]
+    off = pids * 6 * np.arange(windows + 1, dtype=np.int64)
+    return np.ascontiguousarray(ev).reshape(-1), off, t0, t0 + span, [(77, pids)]
+
+
+@pytest.mark.parametrize("windows,pids", [(86, 16), (1_100, 16), (1_600, 1), (3_500, 1), (5_600, 1)])
+def test_summaries_too_large_for_the_staging_kernel(windows, pids):
+    """Tables of more than 128 KB come back by real copies, behind the call's last kernel: the path
+    figures of 1376 processes, the id ranges of 17 600, and the summaries of thousands of windows."""
+    from runners import assert_same, run_gpu, run_oracle
+    ev, off, t0, t1, sizes = _many_small_windows(windows, pids, np.random.default_rng(windows))
+    o = run_oracle(ev, off, t0, t1, min_gap=100, comm_sizes=sizes)
+    g = run_gpu(ev, off, t0, t1, min_gap=100, comm_sizes=sizes)
+    assert o["attr_status"] == 0 and int(o["join_sum"]["n_matched"].min()) > 0
+    assert_same(o, g, skip=("roll_sum",))
