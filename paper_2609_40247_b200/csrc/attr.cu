@@ -892,9 +892,8 @@ ta_status ta_run_attribute(ta_window *h, ta_attr_summary *out_summary) {
   a.op_last = op_last; a.op_ns = op_ns;
   int32_t words[ST_WORDS];
   std::vector<ta_attr_summary> hs(W);
-  const bool small = W * sizeof(ta_attr_summary) <= 4096;  // (more is copied once the kernels are queued)
   TA_TRY(ta_queue_d2h(h, words, h->d_status, sizeof(words)));
-  if (small) TA_TRY(ta_queue_d2h(h, hs.data(), d_sum, W * sizeof(ta_attr_summary)));
+  TA_TRY(ta_queue_d2h(h, hs.data(), d_sum, W * sizeof(ta_attr_summary)));
   if (n > 0) {
     const unsigned wblocks = (unsigned)((tiles + AS_WARPS - 1) / AS_WARPS);
     ta_launch(per_tile == 128 ? k_attr_agg<128> : per_tile == 256 ? k_attr_agg<256> : per_tile == 512 ? k_attr_agg<512> : k_attr_agg<1024>, wblocks, AT_THREADS, 0, st, a);
@@ -936,7 +935,6 @@ ta_status ta_run_attribute(ta_window *h, ta_attr_summary *out_summary) {
     }
     TA_CHECK_CUDA(h, cudaGetLastError());
   }
-  if (!small) TA_TRY(ta_queue_d2h(h, hs.data(), d_sum, W * sizeof(ta_attr_summary)));
   TA_TRY(ta_sync_fetch(h));
   ta_dfree(h, tmpb);
   bool any_bad = false, any_deep = words[ST_ERR] == TA_ERR_DEPTH;

@@ -369,7 +369,7 @@ ta_status ta_run_blame(ta_window *h, const ta_gap_result *gaps, ta_blame_result 
   TA_TRY(ta_queue_d2h(h, hc.data(), a.win_count, (size_t)W * 32));
   TA_TRY(ta_queue_d2h(h, hn.data(), a.win_ns, (size_t)W * 32));
   TA_TRY(ta_queue_d2h(h, words, h->d_status, sizeof(words)));
-  const Tail tail = W * 32 <= 4096 ? ta_tail(h, tiles) : Tail();
+  const Tail tail = ta_tail(h, tiles);
   ta_launch(tail.m ? k_blame_ops<true> : k_blame_ops<false>, (unsigned)tiles, BL_THREADS, 0, st, a, tail);
   TA_CHECK_CUDA(h, cudaGetLastError());
   TA_TRY(ta_sync_fetch(h));

@@ -869,13 +869,11 @@ ta_status ta_run_critpath(ta_window *h, ta_critpath_result *out, ta_critpath_sum
     ScanTemp s3;
     TA_TRY(scan_temp_init(h, scan_mem, n_slots, &s3));
     CpRowIn ri{a.acc};
-    const bool small = hacc.size() * 8 <= 4096;  // (more is copied once the kernels are queued)
     TA_TRY(ta_queue_d2h(h, &rows, s3.total, 8));
     TA_TRY(ta_queue_d2h(h, words, h->d_status, sizeof(words)));
     if (assumed) TA_TRY(ta_queue_d2h(h, words3, a.n_eff, 12));
-    if (small) TA_TRY(ta_queue_d2h(h, hacc.data(), a.acc, hacc.size() * 8));
+    TA_TRY(ta_queue_d2h(h, hacc.data(), a.acc, hacc.size() * 8));
     TA_TRY((launch_scan<OpAdd, CpRowIn, CpRowOut>(h, n_slots, ri, ro, OpAdd(), s3, true)));
-    if (!small) TA_TRY(ta_queue_d2h(h, hacc.data(), a.acc, hacc.size() * 8));
     return ta_sync_fetch(h);
   };
   for (int attempt = 0; attempt < 2; attempt++) {

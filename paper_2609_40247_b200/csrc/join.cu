@@ -511,9 +511,8 @@ ta_status ta_run_correlate(ta_window *h, ta_join_summary *out_summary) {
   void *tmp_alloc = nullptr;
   bool direct = true;
   int32_t words[ST_WORDS];
-  const bool small = W * sizeof(ta_join_summary) <= 4096;  // (more is copied once the kernels are queued)
   TA_TRY(ta_queue_d2h(h, words, h->d_status, sizeof(words)));
-  if (small) TA_TRY(ta_queue_d2h(h, hs.data(), d_sum, W * sizeof(ta_join_summary)));
+  TA_TRY(ta_queue_d2h(h, hs.data(), d_sum, W * sizeof(ta_join_summary)));
   if (n > 0) {
     // table size if every slot is addressed directly
     unsigned __int128 total = 0;
@@ -553,7 +552,6 @@ ta_status ta_run_correlate(ta_window *h, ta_join_summary *out_summary) {
     }
     TA_CHECK_CUDA(h, cudaGetLastError());
   }
-  if (!small) TA_TRY(ta_queue_d2h(h, hs.data(), d_sum, W * sizeof(ta_join_summary)));
   TA_TRY(ta_sync_fetch(h));
   if (tmp_alloc) ta_dfree(h, tmp_alloc);
   if (a.slot_pos) ta_dfree(h, (void *)a.slot_pos);

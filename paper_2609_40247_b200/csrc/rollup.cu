@@ -197,7 +197,7 @@ ta_status ta_run_rollup(ta_window *h, ta_rollup_result *out, ta_rollup_summary *
   int32_t words[ST_WORDS];
   TA_TRY(ta_queue_d2h(h, hs.data(), a.win_sum, (size_t)W * 24));
   TA_TRY(ta_queue_d2h(h, words, h->d_status, sizeof(words)));
-  const Tail tail = W * 24 <= 4096 ? ta_tail(h, tiles) : Tail();
+  const Tail tail = ta_tail(h, tiles);
   ta_launch(tail.m ? k_roll_finalize<true> : k_roll_finalize<false>, tiles, RO_THREADS, 0, st, a, tail);
   TA_CHECK_CUDA(h, cudaGetLastError());
   TA_TRY(ta_sync_fetch(h));

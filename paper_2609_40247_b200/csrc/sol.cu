@@ -277,7 +277,7 @@ ta_status ta_run_sol(ta_window *h, const double *flops, const double *bytes, int
     const int64_t ctas = n_tiles < 148 * 8 ? n_tiles : 148 * 8;
     const int64_t per = (n_tiles + ctas - 1) / ctas;
     const int64_t grid = (n_tiles + per - 1) / per;
-    const Tail tail = W * sizeof(ta_sol_summary) <= 4096 ? ta_tail(h, grid) : Tail();
+    const Tail tail = ta_tail(h, grid);
     ta_launch(tail.m ? k_operator_sol<true> : k_operator_sol<false>, (unsigned)grid, SO_THREADS, 0, st, a, n_tiles, per,
               W == 1 ? grid : (int64_t)1, tail);
     TA_CHECK_CUDA(h, cudaGetLastError());

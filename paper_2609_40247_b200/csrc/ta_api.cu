@@ -216,18 +216,23 @@ __global__ void __launch_bounds__(256) k_collect(FetchList f, int m, unsigned ch
   __threadfence_system();
   *seq_word = seq;
 }
+// (at most TA_FETCH_MAX regions a launch; the last launch writes the number)
 static ta_status flush_fetch(ta_window *h, u32 seq) {
-  if (h->fetch.empty()) return TA_OK;
-  FetchList f;
-  memset(&f, 0, sizeof(f));
-  const unsigned m = (unsigned)h->fetch.size();
-  unsigned most = 1;
-  for (unsigned i = 0; i < m; i++) {
-    f.src[i] = h->fetch[i].src; f.off[i] = h->fetch[i].off; f.bytes[i] = h->fetch[i].bytes;
-    most = f.bytes[i] > most ? f.bytes[i] : most;
+  for (size_t first = 0; first < h->fetch.size(); first += TA_FETCH_MAX) {
+    FetchList f;
+    memset(&f, 0, sizeof(f));
+    const bool last = h->fetch.size() - first <= TA_FETCH_MAX;
+    const unsigned m = last ? (unsigned)(h->fetch.size() - first) : TA_FETCH_MAX;
+    unsigned most = 1;
+    for (unsigned i = 0; i < m; i++) {
+      const ta_window::Fetch &q = h->fetch[first + i];
+      f.src[i] = q.src; f.off[i] = q.off; f.bytes[i] = q.bytes;
+      most = q.bytes > most ? q.bytes : most;
+    }
+    ta_launch(k_collect, (most + TA_FETCH_STRIPE - 1) / TA_FETCH_STRIPE, 256, 0, h->stream, f, (int)m, h->pin_dev,
+              (u32 *)&h->d_status[ST_TICKET], last ? seq : 0u, (volatile u32 *)(h->pin_dev + TA_PIN_BYTES));
   }
   h->fetch.clear();
-  ta_launch(k_collect, (most + TA_FETCH_STRIPE - 1) / TA_FETCH_STRIPE, 256, 0, h->stream,  f, (int)m, h->pin_dev, (u32 *)&h->d_status[ST_TICKET], seq, (volatile u32 *)(h->pin_dev + TA_PIN_BYTES));
   TA_CHECK_CUDA(h, cudaGetLastError());
   return TA_OK;
 }
@@ -235,22 +240,16 @@ static ta_status flush_fetch(ta_window *h, u32 seq) {
 ta_status ta_queue_d2h(ta_window *h, void *dst, const void *dev_src, size_t bytes) {
   if (bytes == 0) return TA_OK;
   const size_t need = (bytes + 15) & ~(size_t)15;
-  if (h->pin_dev && bytes <= TA_FETCH_BYTES && h->pin_used + need <= h->pin_bytes) {
-    if (h->fetch.size() == TA_FETCH_MAX) TA_TRY(flush_fetch(h, 0));
-    h->fetch.push_back(ta_window::Fetch{dev_src, (unsigned)h->pin_used, (unsigned)bytes});
-    h->pending.push_back(ta_window::Pending{dst, h->pin_used, bytes});
-    h->pin_used += need;
-  } else {
-    // a real copy: it is done when the stream is, not when the word of a tail taken in front of it appears
-    h->tail_seq = 0;
-    if (h->pin && h->pin_used + need <= h->pin_bytes) {
-      TA_CHECK_CUDA(h, cudaMemcpyAsync(h->pin + h->pin_used, dev_src, bytes, cudaMemcpyDeviceToHost, h->stream));
-      h->pending.push_back(ta_window::Pending{dst, h->pin_used, bytes});
-      h->pin_used += need;
-    } else {
-      TA_CHECK_CUDA(h, cudaMemcpyAsync(dst, dev_src, bytes, cudaMemcpyDeviceToHost, h->stream));
-    }
+  if (!h->pin || h->pin_used + need > h->pin_bytes) {
+    h->copies.push_back(ta_window::Copy{dst, dev_src, bytes});
+    return TA_OK;
   }
+  if (h->pin_dev && bytes <= TA_FETCH_BYTES)
+    h->fetch.push_back(ta_window::Fetch{dev_src, (unsigned)h->pin_used, (unsigned)bytes});
+  else
+    h->copies.push_back(ta_window::Copy{h->pin + h->pin_used, dev_src, bytes});
+  h->pending.push_back(ta_window::Pending{dst, h->pin_used, bytes});
+  h->pin_used += need;
   return TA_OK;
 }
 
@@ -258,7 +257,7 @@ static u32 next_seq(ta_window *h) { return ++h->fetch_seq ? h->fetch_seq : ++h->
 static volatile u32 *seq_word(unsigned char *pin) { return (volatile u32 *)(pin + TA_PIN_BYTES); }
 Tail ta_tail(ta_window *h, int64_t grid) {
   Tail t;
-  if (!h->pin_dev || h->fetch.empty() || h->fetch.size() > TA_TAIL_MAX || grid > 1024) return t;
+  if (!h->pin_dev || h->fetch.empty() || h->fetch.size() > TA_TAIL_MAX || !h->copies.empty() || grid > 1024) return t;
   for (const ta_window::Fetch &f : h->fetch)
     if (f.bytes > 4096 || (f.bytes & 3u)) return t;
   for (size_t i = 0; i < h->fetch.size(); i++) {
@@ -276,6 +275,11 @@ Tail ta_tail(ta_window *h, int64_t grid) {
   return t;
 }
 static ta_status wait_fetch(ta_window *h) {
+  // real copies are done when the stream is, not when a kernel's word appears
+  if (!h->copies.empty()) h->tail_seq = 0;
+  for (const ta_window::Copy &c : h->copies)
+    TA_CHECK_CUDA(h, cudaMemcpyAsync(c.dst, c.src, c.bytes, cudaMemcpyDeviceToHost, h->stream));
+  h->copies.clear();
   if (h->fetch.empty() && h->tail_seq) {
     const u32 seq = h->tail_seq;
     h->tail_seq = 0;
@@ -326,6 +330,7 @@ void ta_dfree_later(ta_window *h, void *p) {
 static ta_status begin_call(ta_window *h) {
   h->pending.clear();
   h->fetch.clear();
+  h->copies.clear();
   h->tail_seq = 0;
   h->pin_used = 0;
   if (cudaSetDevice(h->device) != cudaSuccess) {
@@ -518,11 +523,8 @@ static ta_status load_impl(ta_window *h, const ta_event *events, int32_t on_devi
   TA_TRY(ta_queue_d2h(h, misc, h->d_misc, sizeof(misc)));
   TA_TRY(ta_queue_d2h(h, h->h_comm_sorted.data(), h->d_comms->sorted_id, TA_COMMS_AT_ONCE * sizeof(u64)));
   TA_TRY(ta_queue_d2h(h, words, h->d_status, sizeof(words)));
-  // (summaries beyond the staging block are copied directly, once the kernels are queued)
-  const bool small = W * sizeof(ta_load_summary) <= 4096;
-  if (small) TA_TRY(ta_queue_d2h(h, sums.data(), h->d_load_sum, W * sizeof(ta_load_summary)));
+  TA_TRY(ta_queue_d2h(h, sums.data(), h->d_load_sum, W * sizeof(ta_load_summary)));
   TA_TRY(ta_launch_discover(h));
-  if (!small) TA_TRY(ta_queue_d2h(h, sums.data(), h->d_load_sum, W * sizeof(ta_load_summary)));
   TA_TRY(ta_sync_fetch(h));
   if (words[ST_ERR]) return (ta_status)words[ST_ERR];
   h->n_triples = words[ST_N_TRIPLES];

@@ -120,6 +120,9 @@ struct ta_window {
   unsigned char *pin_dev;  // device address of `pin`, null when the block is not mapped
   struct Fetch { const void *src; unsigned off, bytes; };
   std::vector<Fetch> fetch;
+  // results too large for that kernel (or all of them, without a mapped block): copied at the end of the call
+  struct Copy { void *dst; const void *src; size_t bytes; };
+  std::vector<Copy> copies;
   u32 fetch_seq;  // number of the last fetch somebody waited for
   u32 tail_seq;   // number of the fetch the last kernel of the call makes itself, 0 = none
 
@@ -276,8 +279,9 @@ ta_status ta_run_blame(ta_window *h, const ta_gap_result *gaps, ta_blame_result 
 // critpath.cu
 ta_status ta_run_critpath(ta_window *h, ta_critpath_result *out, ta_critpath_summary *out_summary);
 
-// Queues a device -> host copy of the call in progress; *dst is valid after the next
-// ta_read_status / ta_sync_fetch.
+// Notes a device -> host copy of the call in progress; *dst is valid after the next
+// ta_read_status / ta_sync_fetch, and holds what *dev_src holds once all kernels launched before
+// that have run, whatever was launched before or after this.
 ta_status ta_queue_d2h(ta_window *h, void *dst, const void *dev_src, size_t bytes);
 // One stream synchronisation: delivers the queued copies and releases deferred temporaries.
 ta_status ta_sync_fetch(ta_window *h);

@@ -702,8 +702,7 @@ ta_status ta_run_sort_timeline(ta_window *h) {
     }
     TA_TRY(ta_queue_d2h(h, n_lanes_host, n_lanes_dev, 2 * sizeof(int32_t)));
     TA_TRY(ta_queue_d2h(h, words, h->d_status, sizeof(words)));
-    const bool small = n_slots * 8 <= 4096;  // (larger ranges are copied once the kernels are queued)
-    for (int q = 0; small && q < 2; q++)
+    for (int q = 0; q < 2; q++)
       TA_TRY(ta_queue_d2h(h, q ? h->h_slot_max.data() : h->h_slot_min.data(), q ? h->d_slot_max : h->d_slot_min, n_slots * 8));
     const SlotRanges ranges{slot_code, n_slots, h->d_slot_min, h->d_slot_max, h->d_slot_base};
     if (n_codes <= LT_ONE_CTA || n == 0) {
@@ -729,8 +728,6 @@ ta_status ta_run_sort_timeline(ta_window *h) {
       ta_launch(k_slot_ranges, 1, 1024, 0, st, ranges, h->d_status, ta_tail(h, 1));
     }
     TA_CHECK_CUDA(h, cudaGetLastError());
-    for (int q = 0; !small && q < 2; q++)
-      TA_TRY(ta_queue_d2h(h, q ? h->h_slot_max.data() : h->h_slot_min.data(), q ? h->d_slot_max : h->d_slot_min, n_slots * 8));
     TA_TRY(ta_sync_fetch(h));
     if (words[ST_ERR]) return (ta_status)words[ST_ERR];
     if (!words[ST_LONG_RUN]) break;

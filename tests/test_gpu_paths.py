@@ -227,13 +227,16 @@ def _many_small_windows(windows, pids, rng):
     return np.ascontiguousarray(ev).reshape(-1), off, t0, t0 + span, [(77, pids)]
 
 
-@pytest.mark.parametrize("windows,pids", [(86, 16), (1_100, 16), (1_600, 1), (3_500, 1), (5_600, 1)])
+@pytest.mark.parametrize("windows,pids", [(86, 16), (1_100, 16), (1_600, 1), (2_500, 1), (3_500, 1), (5_600, 1)])
 def test_summaries_too_large_for_the_staging_kernel(windows, pids):
     """Tables of more than 128 KB come back by real copies, behind the call's last kernel: the path
     figures of 1376 processes, the id ranges of 17 600, and the summaries of thousands of windows."""
     from runners import assert_same, run_gpu, run_oracle
-    ev, off, t0, t1, sizes = _many_small_windows(windows, pids, np.random.default_rng(windows))
-    o = run_oracle(ev, off, t0, t1, min_gap=100, comm_sizes=sizes)
-    g = run_gpu(ev, off, t0, t1, min_gap=100, comm_sizes=sizes)
+    rng = np.random.default_rng(windows)
+    ev, off, t0, t1, sizes = _many_small_windows(windows, pids, rng)
+    work = (rng.uniform(1e9, 1e12, len(ev)), rng.uniform(1e6, 1e9, len(ev)), synth.PEAK_FLOPS, synth.PEAK_BW)
+    o = run_oracle(ev, off, t0, t1, min_gap=100, comm_sizes=sizes, op_work=work)
+    g = run_gpu(ev, off, t0, t1, min_gap=100, comm_sizes=sizes, op_work=work)
     assert o["attr_status"] == 0 and int(o["join_sum"]["n_matched"].min()) > 0
-    assert_same(o, g, skip=("roll_sum",))
+    assert int(o["sol_sum"]["n_resolved"].min()) > 0 and int(o["roll_sum"].sum()) > 0
+    assert_same(o, g)
