@@ -404,7 +404,8 @@ class _Result:
         self._handle = window._handle
         self._blocks = window._blocks
         self._raw = raw
-        self._host = {}
+        self._host = {}      # tables fetched with another one and not asked for yet
+        self._shown = set()  # fields the caller has a tensor of and may write to: read when asked for
         self.__dict__.update(extra or {})
 
     def _spec(self, name):
@@ -419,18 +420,21 @@ class _Result:
         ptr = getattr(self._raw, field)
         if nbytes == 0 or not ptr:
             return self._blocks.empty()
+        self._shown.add(field)
+        self._host.pop(field, None)
         t = _part(self._blocks.last, ptr, nbytes) if _part else None
         return self._blocks.part(ptr, nbytes) if t is None else t
 
     # Tables are mostly read together: a request for one brings the other small ones of the result
-    # along (a round trip costs more than their bytes), up to these limits.
+    # along (a round trip costs more than their bytes), up to these limits.  Only tables nobody but
+    # the library can have written to since: none the caller holds a tensor of.
     _FETCH_EACH, _FETCH_ALL, _FETCH_COUNT = 128 << 10, 448 << 10, 16
 
     def _fetch(self, name):
         names, sizes, total = [], [], 0
         for k in (name, *self._layout):
             field, _, size, count = self._table[k]
-            if k != name and (k == self._table[name][0] or k in self._host):
+            if k != name and (k == self._table[name][0] or k in self._host or k in self._shown):
                 continue
             b = count(self) * size
             if k == name or (b <= self._FETCH_EACH and total + b <= self._FETCH_ALL and len(names) < self._FETCH_COUNT):
@@ -458,7 +462,7 @@ class _Result:
         if count(self) == 0 or not getattr(self._raw, field):
             out = np.empty(0, dtype=dt)
         else:
-            out = self._host.pop(field, None)
+            out = self._host.pop(field, None) if self._handle.ptr else None  # (none of a closed window)
             if out is None:
                 self._fetch(name)
                 out = self._host.pop(field)
