@@ -29,10 +29,13 @@
  *   - Call order: load -> sort -> { correlate -> attribute ; gaps ;
  *     aggregate(value_sel 0) ; collectives }.  aggregate(value_sel 1) needs
  *     attribute.  A call made too early returns TA_ERR_ORDER.
- *   - Threads: a handle is used by one thread at a time; different handles may
- *     be used from different threads and on different streams at the same time
- *     (the library keeps no state outside the handle except its memory pool, the
- *     launch counter and the benchmark instrumentation at the end of this file).
+ *   - Threads: a handle is used by one thread at a time, except that ta_fetch and
+ *     ta_block_of may be called by any thread, also while another is in a call on
+ *     the handle (not in ta_free); different handles may be used from different
+ *     threads and on different streams at the same time.  Outside the handles the
+ *     library keeps its memory pools, page-locked blocks (staging of results, rings
+ *     for uploads, the row of ta_lane_gaps_noalloc), the launch counter and the
+ *     benchmark instrumentation at the end of this file.
  */
 #ifndef TA_H
 #define TA_H

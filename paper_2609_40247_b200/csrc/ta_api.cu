@@ -105,6 +105,7 @@ void *ta_dalloc(ta_window *h, size_t bytes) {
     }
   }
   if (p) {
+    std::lock_guard<std::mutex> lock(h->alloc_guard);
     h->allocs.push_back(p);
     h->alloc_bytes.push_back(bytes);
   }
@@ -141,16 +142,19 @@ static void release_one(ta_window *h, void *p, size_t bytes) {
 
 void ta_dfree(ta_window *h, void *p) {
   if (!p) return;
-  for (size_t i = 0; i < h->allocs.size(); i++)
-    if (h->allocs[i] == p) {
-      const size_t bytes = h->alloc_bytes[i];
-      h->allocs[i] = h->allocs.back();
-      h->allocs.pop_back();
-      h->alloc_bytes[i] = h->alloc_bytes.back();
-      h->alloc_bytes.pop_back();
-      release_one(h, p, bytes);
-      return;
-    }
+  size_t bytes = 0;
+  {
+    std::lock_guard<std::mutex> lock(h->alloc_guard);
+    size_t i = 0;
+    while (i < h->allocs.size() && h->allocs[i] != p) i++;
+    if (i == h->allocs.size()) return;
+    bytes = h->alloc_bytes[i];
+    h->allocs[i] = h->allocs.back();
+    h->allocs.pop_back();
+    h->alloc_bytes[i] = h->alloc_bytes.back();
+    h->alloc_bytes.pop_back();
+  }
+  release_one(h, p, bytes);
 }
 
 // Page-locked staging blocks are expensive to create (a system call and a page-table update
@@ -216,100 +220,117 @@ __global__ void __launch_bounds__(256) k_collect(FetchList f, int m, unsigned ch
   __threadfence_system();
   *seq_word = seq;
 }
+static volatile u32 *seq_word(unsigned char *pin) { return (volatile u32 *)(pin + TA_PIN_BYTES); }
+static u32 next_seq(ResultStage &o) { return ++o.seq ? o.seq : ++o.seq; }
+static void stage_open(ResultStage &o) {
+  o.pin = pin_take();
+  o.pin_dev = nullptr;
+  if (o.pin) {
+    void *dp = nullptr;
+    if (cudaHostGetDevicePointer(&dp, o.pin, 0) == cudaSuccess) o.pin_dev = (unsigned char *)dp;
+    else cudaGetLastError();
+  }
+  o.used = 0;
+  o.seq = o.tail_seq = 0;
+}
+static void stage_clear(ResultStage &o) {
+  o.pending.clear();
+  o.fetch.clear();
+  o.copies.clear();
+  o.tail_seq = 0;
+  o.used = 0;
+}
+static void stage_queue(ResultStage &o, void *dst, const void *dev_src, size_t bytes) {
+  if (bytes == 0) return;
+  const size_t need = (bytes + 15) & ~(size_t)15;
+  if (!o.pin || o.used + need > TA_PIN_BYTES) {
+    o.copies.push_back(ResultStage::Copy{dst, dev_src, bytes});
+    return;
+  }
+  if (o.pin_dev && bytes <= TA_FETCH_BYTES)
+    o.fetch.push_back(ResultStage::Fetch{dev_src, (unsigned)o.used, (unsigned)bytes});
+  else
+    o.copies.push_back(ResultStage::Copy{o.pin + o.used, dev_src, bytes});
+  o.pending.push_back(ResultStage::Pending{dst, o.used, bytes});
+  o.used += need;
+}
 // (at most TA_FETCH_MAX regions a launch; the last launch writes the number)
-static ta_status flush_fetch(ta_window *h, u32 seq) {
-  for (size_t first = 0; first < h->fetch.size(); first += TA_FETCH_MAX) {
+static ta_status stage_collect(ta_window *h, ResultStage &o, u32 seq) {
+  for (size_t first = 0; first < o.fetch.size(); first += TA_FETCH_MAX) {
     FetchList f;
     memset(&f, 0, sizeof(f));
-    const bool last = h->fetch.size() - first <= TA_FETCH_MAX;
-    const unsigned m = last ? (unsigned)(h->fetch.size() - first) : TA_FETCH_MAX;
+    const bool last = o.fetch.size() - first <= TA_FETCH_MAX;
+    const unsigned m = last ? (unsigned)(o.fetch.size() - first) : TA_FETCH_MAX;
     unsigned most = 1;
     for (unsigned i = 0; i < m; i++) {
-      const ta_window::Fetch &q = h->fetch[first + i];
+      const ResultStage::Fetch &q = o.fetch[first + i];
       f.src[i] = q.src; f.off[i] = q.off; f.bytes[i] = q.bytes;
       most = q.bytes > most ? q.bytes : most;
     }
-    ta_launch(k_collect, (most + TA_FETCH_STRIPE - 1) / TA_FETCH_STRIPE, 256, 0, h->stream, f, (int)m, h->pin_dev,
-              (u32 *)&h->d_status[ST_TICKET], last ? seq : 0u, (volatile u32 *)(h->pin_dev + TA_PIN_BYTES));
+    ta_launch(k_collect, (most + TA_FETCH_STRIPE - 1) / TA_FETCH_STRIPE, 256, 0, h->stream, f, (int)m, o.pin_dev,
+              (u32 *)&h->d_status[ST_TICKET], last ? seq : 0u, seq_word(o.pin_dev));
   }
-  h->fetch.clear();
+  o.fetch.clear();
   TA_CHECK_CUDA(h, cudaGetLastError());
   return TA_OK;
 }
-
-ta_status ta_queue_d2h(ta_window *h, void *dst, const void *dev_src, size_t bytes) {
-  if (bytes == 0) return TA_OK;
-  const size_t need = (bytes + 15) & ~(size_t)15;
-  if (!h->pin || h->pin_used + need > h->pin_bytes) {
-    h->copies.push_back(ta_window::Copy{dst, dev_src, bytes});
-    return TA_OK;
-  }
-  if (h->pin_dev && bytes <= TA_FETCH_BYTES)
-    h->fetch.push_back(ta_window::Fetch{dev_src, (unsigned)h->pin_used, (unsigned)bytes});
-  else
-    h->copies.push_back(ta_window::Copy{h->pin + h->pin_used, dev_src, bytes});
-  h->pending.push_back(ta_window::Pending{dst, h->pin_used, bytes});
-  h->pin_used += need;
-  return TA_OK;
-}
-
-static u32 next_seq(ta_window *h) { return ++h->fetch_seq ? h->fetch_seq : ++h->fetch_seq; }
-static volatile u32 *seq_word(unsigned char *pin) { return (volatile u32 *)(pin + TA_PIN_BYTES); }
-Tail ta_tail(ta_window *h, int64_t grid) {
-  Tail t;
-  if (!h->pin_dev || h->fetch.empty() || h->fetch.size() > TA_TAIL_MAX || !h->copies.empty() || grid > 1024) return t;
-  for (const ta_window::Fetch &f : h->fetch)
-    if (f.bytes > 4096 || (f.bytes & 3u)) return t;
-  for (size_t i = 0; i < h->fetch.size(); i++) {
-    t.src[i] = h->fetch[i].src;
-    t.off[i] = h->fetch[i].off;
-    t.bytes[i] = h->fetch[i].bytes;
-  }
-  t.m = (int)h->fetch.size();
-  h->fetch.clear();
-  t.pin_dev = h->pin_dev;
-  t.ticket = (u32 *)&h->d_status[ST_TICKET];
-  t.seq = h->tail_seq = next_seq(h);
-  t.seq_word = seq_word(h->pin_dev);
-  *seq_word(h->pin) = 0;
-  return t;
-}
-static ta_status wait_fetch(ta_window *h) {
+static ta_status stage_wait(ta_window *h, ResultStage &o) {
   // real copies are done when the stream is, not when a kernel's word appears
-  if (!h->copies.empty()) h->tail_seq = 0;
-  for (const ta_window::Copy &c : h->copies)
+  if (!o.copies.empty()) o.tail_seq = 0;
+  for (const ResultStage::Copy &c : o.copies)
     TA_CHECK_CUDA(h, cudaMemcpyAsync(c.dst, c.src, c.bytes, cudaMemcpyDeviceToHost, h->stream));
-  h->copies.clear();
-  if (h->fetch.empty() && h->tail_seq) {
-    const u32 seq = h->tail_seq;
-    h->tail_seq = 0;
-    volatile u32 *word = seq_word(h->pin);
-    TA_WAIT_SEQ(*word, seq, h->stream);
-    if (*word != seq) TA_CHECK_CUDA(h, cudaStreamSynchronize(h->stream));
-    std::atomic_thread_fence(std::memory_order_acquire);
-    return *word == seq ? TA_OK : TA_ERR_CUDA;
-  }
-  h->tail_seq = 0;
-  if (h->fetch.empty()) {
+  o.copies.clear();
+  u32 seq = o.tail_seq;
+  o.tail_seq = 0;
+  if (!o.fetch.empty()) {
+    seq = next_seq(o);
+    *seq_word(o.pin) = 0;
+    TA_TRY(stage_collect(h, o, seq));
+  } else if (!seq) {
     TA_CHECK_CUDA(h, cudaStreamSynchronize(h->stream));
     return TA_OK;
   }
-  volatile u32 *word = seq_word(h->pin);
-  const u32 seq = next_seq(h);
-  *word = 0;
-  TA_TRY(flush_fetch(h, seq));
+  volatile u32 *word = seq_word(o.pin);
   TA_WAIT_SEQ(*word, seq, h->stream);
   if (*word != seq) TA_CHECK_CUDA(h, cudaStreamSynchronize(h->stream));
   std::atomic_thread_fence(std::memory_order_acquire);
   return *word == seq ? TA_OK : TA_ERR_CUDA;
 }
-ta_status ta_sync_fetch(ta_window *h) {
-  const ta_status fs = wait_fetch(h);
+// one wait, then everything to its destination
+static ta_status stage_deliver(ta_window *h, ResultStage &o) {
+  const ta_status fs = stage_wait(h, o);
   if (fs == TA_OK)
-    for (const ta_window::Pending &q : h->pending) memcpy(q.dst, h->pin + q.off, q.bytes);
-  h->pending.clear();
-  h->pin_used = 0;
-  if (fs != TA_OK) return fs;
+    for (const ResultStage::Pending &q : o.pending) memcpy(q.dst, o.pin + q.off, q.bytes);
+  stage_clear(o);
+  return fs;
+}
+
+ta_status ta_queue_d2h(ta_window *h, void *dst, const void *dev_src, size_t bytes) {
+  stage_queue(h->out, dst, dev_src, bytes);
+  return TA_OK;
+}
+Tail ta_tail(ta_window *h, int64_t grid) {
+  ResultStage &o = h->out;
+  Tail t;
+  if (!o.pin_dev || o.fetch.empty() || o.fetch.size() > TA_TAIL_MAX || !o.copies.empty() || grid > 1024) return t;
+  for (const ResultStage::Fetch &f : o.fetch)
+    if (f.bytes > 4096 || (f.bytes & 3u)) return t;
+  for (size_t i = 0; i < o.fetch.size(); i++) {
+    t.src[i] = o.fetch[i].src;
+    t.off[i] = o.fetch[i].off;
+    t.bytes[i] = o.fetch[i].bytes;
+  }
+  t.m = (int)o.fetch.size();
+  o.fetch.clear();
+  t.pin_dev = o.pin_dev;
+  t.ticket = (u32 *)&h->d_status[ST_TICKET];
+  t.seq = o.tail_seq = next_seq(o);
+  t.seq_word = seq_word(o.pin_dev);
+  *seq_word(o.pin) = 0;
+  return t;
+}
+ta_status ta_sync_fetch(ta_window *h) {
+  TA_TRY(stage_deliver(h, h->out));
   for (void *p : h->deferred) ta_dfree(h, p);
   h->deferred.clear();
   return TA_OK;
@@ -328,11 +349,7 @@ void ta_dfree_later(ta_window *h, void *p) {
 // early with an error) must not be delivered to destinations that no longer exist.
 // Also makes the handle's device current (it stays current when the call returns).
 static ta_status begin_call(ta_window *h) {
-  h->pending.clear();
-  h->fetch.clear();
-  h->copies.clear();
-  h->tail_seq = 0;
-  h->pin_used = 0;
+  stage_clear(h->out);
   if (cudaSetDevice(h->device) != cudaSuccess) {
     h->last_cuda = cudaGetLastError();
     return TA_ERR_CUDA;
@@ -595,17 +612,7 @@ ta_status ta_load_window(const ta_env *env, const ta_event *events, int64_t n,
   h->d_on_path = nullptr;
   h->d_status = nullptr;
   h->zero_bytes = h->zero_used = 0;
-  h->pin = pin_take();
-  h->pin_bytes = h->pin ? TA_PIN_BYTES : 0;
-  h->pin_dev = nullptr;
-  if (h->pin) {
-    void *dp = nullptr;
-    if (cudaHostGetDevicePointer(&dp, h->pin, 0) == cudaSuccess) h->pin_dev = (unsigned char *)dp;
-    else cudaGetLastError();
-  }
-  h->pin_used = 0;
-  h->fetch_seq = 0;
-  h->tail_seq = 0;
+  stage_open(h->out);
   h->h_off.assign(win_off, win_off + W + 1);
   h->h_t0.assign(win_t0, win_t0 + W);
   h->h_t1.assign(win_t1, win_t1 + W);
@@ -715,13 +722,23 @@ ta_status ta_device_overlap(ta_window *h, ta_overlap_result *out) {
 
 ta_status ta_fetch(ta_window *h, int32_t count, void *const *dst, const void *const *src, const uint64_t *bytes) {
   if (!h || count < 0 || (count > 0 && (!dst || !src || !bytes))) return TA_ERR_INVALID_ARG;
-  TA_TRY(begin_call(h));
-  for (int32_t i = 0; i < count; i++) TA_TRY(ta_queue_d2h(h, dst[i], src[i], (size_t)bytes[i]));
-  return ta_sync_fetch(h);
+  if (cudaSetDevice(h->device) != cudaSuccess) {
+    cudaGetLastError();
+    return TA_ERR_CUDA;
+  }
+  // a block of its own: results are read while another thread is in a call on the handle, or reads as well
+  ResultStage o;
+  stage_open(o);
+  for (int32_t i = 0; i < count; i++) stage_queue(o, dst[i], src[i], (size_t)bytes[i]);
+  const ta_status s = stage_deliver(h, o);
+  if (s != TA_OK) cudaStreamSynchronize(h->stream);  // nothing queued may write to the block any more
+  pin_put(o.pin);
+  return s;
 }
 
 ta_status ta_block_of(ta_window *h, const void *p, void **base, uint64_t *bytes) {
   if (!h || !base || !bytes) return TA_ERR_INVALID_ARG;
+  std::lock_guard<std::mutex> lock(h->alloc_guard);
   for (size_t i = 0; i < h->allocs.size(); i++) {
     const char *b = (const char *)h->allocs[i];
     if ((const char *)p >= b && (const char *)p < b + h->alloc_bytes[i]) {
@@ -802,7 +819,7 @@ void ta_free(ta_window *h) {
   for (size_t i = 0; i < h->allocs.size(); i++) release_one(h, h->allocs[i], h->alloc_bytes[i]);
   h->allocs.clear();
   h->alloc_bytes.clear();
-  pin_put(h->pin);
+  pin_put(h->out.pin);
   const bool own = !h->env.alloc;
   delete h;
   if (own) cache_age();

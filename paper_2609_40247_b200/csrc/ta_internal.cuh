@@ -8,6 +8,7 @@
 #include <stdint.h>
 
 #include <atomic>
+#include <mutex>
 #include <utility>
 #include <vector>
 
@@ -87,6 +88,25 @@ struct TopHist {
   const u32 *rank_cnt;  // records per triple rank; null: the histograms are complete
 };
 
+// Device -> host results on their way.  They go through a page-locked block and are handed to their
+// destinations after one wait (a copy into pageable memory would block until it is done).
+struct ResultStage {
+  unsigned char *pin;      // null: none to be had, the copies go straight to their destinations
+  unsigned char *pin_dev;  // its device address, null when the block is not mapped
+  size_t used;
+  struct Pending { void *dst; size_t off, bytes; };
+  std::vector<Pending> pending;
+  // small results (status words, per-window summaries) are not copied one by one: one kernel
+  // writes them all into the block through its device address
+  struct Fetch { const void *src; unsigned off, bytes; };
+  std::vector<Fetch> fetch;
+  // those too large for that kernel (or all of them, without a mapped block)
+  struct Copy { void *dst; const void *src; size_t bytes; };
+  std::vector<Copy> copies;
+  u32 seq;       // number of the last fetch somebody waited for
+  u32 tail_seq;  // number of the fetch the last kernel of the call makes itself, 0 = none
+};
+
 // --------------------------------------------------------------- handle
 struct ta_window {
   ta_env env;
@@ -102,29 +122,14 @@ struct ta_window {
   std::vector<int64_t> h_off, h_t0, h_t1;
   int64_t *d_off, *d_t0, *d_t1;
 
+  std::mutex alloc_guard;      // of the next two: results are located while a call is in progress
   std::vector<void *> allocs;  // everything obtained from env.alloc (or the library's own pool)
   std::vector<size_t> alloc_bytes;  // their sizes, same order
   char *zero_pool;   // cleared when the window was loaded, handed out by ta_zalloc
   size_t zero_bytes, zero_used;
   std::vector<void *> deferred;  // temporaries to release after the next synchronisation
 
-  // device -> host results of the call in progress: copies are queued into one page-locked
-  // staging block (truly asynchronous, unlike a copy into pageable memory, which blocks until
-  // it is done) and handed to their destinations after the call's one synchronisation
-  unsigned char *pin;
-  size_t pin_bytes, pin_used;
-  struct Pending { void *dst; size_t off, bytes; };
-  std::vector<Pending> pending;
-  // small results (status words, per-window summaries) are not copied one by one: one kernel
-  // at the end of the call writes them all into the staging block through its device alias
-  unsigned char *pin_dev;  // device address of `pin`, null when the block is not mapped
-  struct Fetch { const void *src; unsigned off, bytes; };
-  std::vector<Fetch> fetch;
-  // results too large for that kernel (or all of them, without a mapped block): copied at the end of the call
-  struct Copy { void *dst; const void *src; size_t bytes; };
-  std::vector<Copy> copies;
-  u32 fetch_seq;  // number of the last fetch somebody waited for
-  u32 tail_seq;   // number of the fetch the last kernel of the call makes itself, 0 = none
+  ResultStage out;  // results of the call in progress on their way to the host
 
   // load products
   int32_t *d_status;

@@ -363,18 +363,19 @@ class _Blocks:
 
     def part(self, ptr, nbytes):
         wrap, part = _views()
-        for self.last in self.known:
-            t = part(self.last, ptr, nbytes)
+        for at in self.known:
+            t = part(at, ptr, nbytes)
             if t is not None:
+                self.last = at
                 return t
         h = self.handle
         base, room = _vp(), ctypes.c_uint64()
         if h.lib.ta_block_of(h.ptr, ptr, ctypes.byref(base), ctypes.byref(room)) != 0:
             raise ValueError("not a result of an open window")
         lo, size = base.value, room.value
-        self.last = (lo, lo + size, wrap(lo, size, h.device, h))
-        self.known.append(self.last)
-        return part(self.last, ptr, nbytes)
+        at = self.last = (lo, lo + size, wrap(lo, size, h.device, h))
+        self.known.append(at)
+        return part(at, ptr, nbytes)
 
     def drop(self):
         """The window is closed: its memory goes back once no column made so far is in use."""
@@ -444,15 +445,20 @@ class _Result:
         buf = np.empty(total, dtype=np.uint8)
         m, at, base = len(names), 0, _addr(buf)
         dst, src, num = (ctypes.c_void_p * m)(), (ctypes.c_void_p * m)(), (ctypes.c_uint64 * m)()
+        arrays = []
         for i, (k, b) in enumerate(zip(names, sizes)):
             field, dt, _, _ = self._table[k]
             dst[i], src[i], num[i] = base + at, getattr(self._raw, field), b
-            self._host[field] = buf[at:at + b].view(dt)
+            arrays.append((field, buf[at:at + b].view(dt)))
             at += (b + 15) & ~15
         st = self._handle.lib.ta_fetch(self._handle.ptr, m, dst, src, num)
         if st != 0:
-            self._host.clear()
             raise TaError(st, "ta_fetch")
+        for field, array in arrays[1:]:
+            self._host[field] = array
+            if field in self._shown:  # a tensor was handed out meanwhile, by another thread
+                self._host.pop(field, None)
+        return arrays[0][1]
 
     def numpy(self, name):
         got = self.__dict__.get(name)
@@ -464,8 +470,7 @@ class _Result:
         else:
             out = self._host.pop(field, None) if self._handle.ptr else None  # (none of a closed window)
             if out is None:
-                self._fetch(name)
-                out = self._host.pop(field)
+                out = self._fetch(name)
         if field.endswith("_hist"):
             out = out.reshape(-1, NBINS)
         return out

@@ -42,3 +42,60 @@ def test_no_table_of_a_closed_window():
     for name in ("lane_pid", "lane_off", "lane_window"):
         with pytest.raises(ta.TaError):
             s.numpy(name)
+
+
+def test_threads_read_results_of_a_window_that_is_being_analysed():
+    """Three threads read every table and column of a window's results over and over, as arrays and
+    as tensors, while a fourth makes further calls on the window."""
+    import threading
+    import torch
+    from runners import AGG_KEYS, GAP_KEYS, SORT_KEYS
+    wl, buf = _window(0.05)
+    with ta.Window(buf, wl.win_off, wl.win_t0, wl.win_t1) as w:
+        s = w.sort_timeline()
+        g = w.stream_gaps(500_000)
+        k = w.aggregate_ops(ta.DEVICE_KINDS, 0)
+        tables = [(s, SORT_KEYS), (g, GAP_KEYS), (k, AGG_KEYS)]
+        want = [[r.numpy(n).copy() for n in names] for r, names in tables]
+        errors, stop = [], threading.Event()
+
+        def reader(seed):
+            try:
+                torch.cuda.set_device(buf.device)
+                rng = np.random.default_rng(seed)
+                for _ in range(60):
+                    i = rng.integers(len(tables))
+                    r, names = tables[i]
+                    for j in rng.permutation(len(names)):
+                        if rng.random() < 0.5:
+                            got = r.numpy(names[j])
+                        else:
+                            got = r.tensor(names[j]).cpu().numpy().view(want[i][j].dtype).reshape(want[i][j].shape)
+                        assert np.array_equal(got, want[i][j]), names[j]
+            except BaseException as e:  # reported in the main thread
+                errors.append(e)
+
+        def caller():
+            try:
+                torch.cuda.set_device(buf.device)
+                for _ in range(300):  # (what a call returns stays until the window is closed)
+                    if stop.is_set():
+                        break
+                    again = w.stream_gaps(500_000)
+                    assert np.array_equal(again.numpy("lane_gaps"), want[1][GAP_KEYS.index("lane_gaps")])
+                    del again
+                    assert w.aggregate_ops(ta.DEVICE_KINDS, 0).n_groups == k.n_groups
+            except BaseException as e:
+                errors.append(e)
+
+        call = threading.Thread(target=caller)
+        readers = [threading.Thread(target=reader, args=(q,)) for q in range(3)]
+        call.start()
+        for t in readers:
+            t.start()
+        for t in readers:
+            t.join()
+        stop.set()
+        call.join()
+        if errors:
+            raise errors[0]
