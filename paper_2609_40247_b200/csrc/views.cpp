@@ -4,6 +4,7 @@
 #include <Python.h>
 
 #include <ATen/ops/from_blob.h>
+#include <c10/core/InferenceMode.h>
 #include <torch/csrc/autograd/python_variable.h>
 
 // wrap(address, nbytes, device index, owner): uint8 tensor that keeps `owner` alive
@@ -17,6 +18,7 @@ static PyObject *wrap(PyObject *, PyObject *const *args, Py_ssize_t n) {
   if (PyErr_Occurred()) return nullptr;
   PyObject *owner = args[3];
   try {
+    const c10::InferenceMode plain(false);  // usable outside the caller's inference mode as well
     const at::Device device(at::kCUDA, (c10::DeviceIndex)dev);
     Py_INCREF(owner);
     at::Tensor t = at::for_blob(p, {(int64_t)bytes})

@@ -352,6 +352,12 @@ def _views():
 _wrap = _part = None
 
 
+def _plain():
+    """Tensors made here outlive the caller's inference mode and are as usable outside of it."""
+    import torch
+    return torch.inference_mode(False) if torch.is_inference_mode_enabled() else contextlib.nullcontext()
+
+
 class _Blocks:
     """Tensors over the allocations of a handle; the columns are parts of them."""
 
@@ -387,7 +393,8 @@ class _Blocks:
         if self.none is None:
             import torch
             _views()
-            self.none = (0, 0, torch.empty(0, dtype=torch.uint8, device=f"cuda:{self.handle.device}"))
+            with _plain():
+                self.none = (0, 0, torch.empty(0, dtype=torch.uint8, device=f"cuda:{self.handle.device}"))
         return _part(self.none, 0, 0)
 
 
@@ -697,12 +704,14 @@ class Window:
         import torch
         _views()
         h = self._handle
+        if torch.are_deterministic_algorithms_enabled() and torch.utils.deterministic.fill_uninitialized_memory:
+            return  # (torch would write all of it first; the allocator the pieces come from does not)
         size = CHUNK_BYTES_FIXED + self.n * CHUNK_BYTES_PER_RECORD
         try:
             # (without a stream of the caller's choice the window is on the device's current one)
-            with contextlib.nullcontext() if stream is None else torch.cuda.stream(stream):
+            with _plain(), contextlib.nullcontext() if stream is None else torch.cuda.stream(stream):
                 t = torch.empty(size, dtype=torch.uint8, device=torch.device("cuda", h.device))
-        except torch.cuda.OutOfMemoryError:
+        except RuntimeError:  # out of memory, or whatever else the allocator in use has to say
             return  # piece by piece, as far as it goes
         base = t.data_ptr()
         h.chunk = h.lib.ta_chunk_open(base, size, _torch_alloc, _torch_release, env.ctx)

@@ -99,3 +99,51 @@ def test_threads_read_results_of_a_window_that_is_being_analysed():
         call.join()
         if errors:
             raise errors[0]
+
+
+@pytest.mark.parametrize("memory", ["torch", "pieces", "library"])
+def test_tensors_of_a_window_opened_in_inference_mode_are_ordinary(memory):
+    """They can be written to, and hold the results, outside of that mode and inside."""
+    import torch
+    wl, buf = _window()
+    kw = {"torch": {}, "library": {"use_torch_allocator": False},
+          "pieces": {"alloc_fn": lambda n: torch.cuda.caching_allocator_alloc(n, buf.device.index),
+                     "release_fn": torch.cuda.caching_allocator_delete}}[memory]
+    with torch.inference_mode():
+        w = ta.Window(buf, wl.win_off, wl.win_t0, wl.win_t1, **kw)
+        s = w.sort_timeline()
+        k = w.aggregate_ops(0, 0)
+        made = [s.tensor("perm"), k.tensor("g_name")]
+    with w:
+        made += [s.tensor("lane_off"), k.tensor("g_count")]
+        assert not any(t.is_inference() for t in made)
+        for t in made:
+            t.add_(0)
+        assert (s.numpy("perm") == made[0].view(torch.int32).cpu().numpy()).all()
+
+
+def test_no_block_up_front_where_torch_would_fill_it_or_cannot_give_it(monkeypatch):
+    """Deterministic mode writes to all fresh memory of a tensor; another allocator may refuse in
+    its own words.  The window then takes its memory in pieces."""
+    import torch
+    wl, buf = _window()
+
+    def lanes():
+        with ta.Window(buf, wl.win_off, wl.win_t0, wl.win_t1) as w:
+            return w._handle.chunk, w.sort_timeline().numpy("lane_off")
+
+    chunk, want = lanes()
+    assert chunk
+    torch.use_deterministic_algorithms(True)
+    try:
+        chunk, got = lanes()
+    finally:
+        torch.use_deterministic_algorithms(False)
+    assert not chunk and np.array_equal(got, want)
+
+    def refuse(*args, **kw):
+        raise RuntimeError("no")
+
+    monkeypatch.setattr(torch, "empty", refuse)
+    chunk, got = lanes()
+    assert not chunk and np.array_equal(got, want)
