@@ -315,15 +315,30 @@ void ta_dfree_later(ta_window *h, void *p);
 // stream `st`) equals `want`: some microseconds less than a stream synchronisation.  The stream is
 // asked now and then, so a kernel that fails (or returns early and writes nothing) ends the wait:
 // on a CUDA error the enclosing function returns TA_ERR_CUDA; the caller compares once more.
-#define TA_WAIT_SEQ(word, want, st)                                             \
-  do {                                                                          \
-    for (unsigned polls__ = 1; (word) != (want); polls__++) {                   \
-      if (polls__ & 1023u) continue;                                            \
-      const cudaError_t e__ = cudaStreamQuery(st);                              \
-      if (e__ == cudaSuccess) break;                                            \
-      if (e__ != cudaErrorNotReady) { cudaGetLastError(); return TA_ERR_CUDA; } \
-    }                                                                           \
+// A device whose host threads are to block or to yield while they wait (cudaDeviceScheduleBlockingSync,
+// cudaDeviceScheduleYield) gets a stream synchronisation, which does that.
+#define TA_WAIT_SEQ(word, want, st)                                               \
+  do {                                                                            \
+    unsigned flags__ = 0;                                                         \
+    if (cudaGetDeviceFlags(&flags__) != cudaSuccess) cudaGetLastError();          \
+    if (flags__ & (cudaDeviceScheduleBlockingSync | cudaDeviceScheduleYield)) {   \
+      if (cudaStreamSynchronize(st) != cudaSuccess) { cudaGetLastError(); return TA_ERR_CUDA; } \
+      break;                                                                      \
+    }                                                                             \
+    for (unsigned polls__ = 1; (word) != (want); polls__++) {                     \
+      ta_pause();                                                                 \
+      if (polls__ & 1023u) continue;                                              \
+      const cudaError_t e__ = cudaStreamQuery(st);                                \
+      if (e__ == cudaSuccess) break;                                              \
+      if (e__ != cudaErrorNotReady) { cudaGetLastError(); return TA_ERR_CUDA; }   \
+    }                                                                             \
   } while (0)
+// leaves the core to its other hardware thread for a moment
+static inline void ta_pause() {
+#if defined(__x86_64__)
+  __builtin_ia32_pause();
+#endif
+}
 
 // ---- instrumentation (no work: a launch counter and optional event pairs) ----
 extern std::atomic<long long> g_ta_launches;  // kernels launched by this library since load

@@ -147,3 +147,47 @@ def test_no_block_up_front_where_torch_would_fill_it_or_cannot_give_it(monkeypat
     monkeypatch.setattr(torch, "empty", refuse)
     chunk, got = lanes()
     assert not chunk and np.array_equal(got, want)
+
+
+_BLOCKING = """
+import ctypes, sys, time
+cuda = ctypes.CDLL("libcuda.so.1")
+assert cuda.cuInit(0) == 0
+assert cuda.cuDevicePrimaryCtxSetFlags_v2(0, 4) == 0  # CU_CTX_SCHED_BLOCKING_SYNC
+sys.path[:0] = [%r, %r]
+import numpy as np, torch
+from paper_2609_40247_b200 import synth, ta
+wl = synth.make_workload("c1", 0.02, truth=False)
+buf = torch.from_numpy(np.ascontiguousarray(wl.events).view(np.uint8).reshape(-1)).cuda()
+for _ in range(2):
+    with ta.Window(buf, wl.win_off, wl.win_t0, wl.win_t1) as w:
+        torch.cuda.synchronize()
+        torch.cuda._sleep(1_000_000_000)  # half a second of the stream's time in front of the call
+        wall, cpu = time.perf_counter(), time.thread_time()
+        s = w.sort_timeline()
+        wall, cpu = time.perf_counter() - wall, time.thread_time() - cpu
+        g = w.stream_gaps(1000)
+        l = int(np.nonzero(s.numpy("lane_domain") == 1)[0][0])
+        a, b = s.numpy("lane_off")[l:l + 2]
+        ts, te = (s.tensor(k).view(torch.int64)[a:b].contiguous() for k in ("ts_start", "ts_end"))
+        torch.cuda.synchronize()
+        torch.cuda._sleep(1_000_000_000)
+        wall2, cpu2 = time.perf_counter(), time.thread_time()
+        _, row = ta.lane_gaps_noalloc(ts, te, int(wl.win_t0[0]), int(wl.win_t1[0]))
+        wall2, cpu2 = time.perf_counter() - wall2, time.thread_time() - cpu2
+        assert row == g.numpy("lane_gaps")[l]
+print(wall, cpu, wall2, cpu2)
+assert wall > 0.2 and wall2 > 0.2, "nothing was waited for"
+assert cpu < 0.25 * wall and cpu2 < 0.25 * wall2, "the host thread was busy while it waited"
+"""
+
+
+def test_calls_block_where_the_device_is_set_to_blocking():
+    """A process that has asked the driver for blocking waits keeps its cores while a call waits."""
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", _BLOCKING % (root, os.path.join(root, "tests"))], capture_output=True,
+                       text=True, timeout=300)
+    assert r.returncode == 0, r.stdout + r.stderr
