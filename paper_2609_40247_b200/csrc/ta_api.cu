@@ -765,12 +765,14 @@ ta_chunk *ta_chunk_open(void *base, uint64_t bytes, void *(*alloc)(size_t, void 
   if (!base || !alloc || !release) return nullptr;
   ta_chunk *c = new (std::nothrow) ta_chunk();
   if (!c) return nullptr;
-  c->base = (char *)base;
-  c->bytes = (size_t)bytes;
+  // pieces are as aligned as ta_env asks for, whatever the block is
+  const size_t skip = (size_t)(-(uintptr_t)base & 255u);
+  c->base = (char *)base + skip;
+  c->bytes = bytes > skip ? (size_t)(bytes - skip) & ~(size_t)255 : 0;
   c->alloc = alloc;
   c->release = release;
   c->ctx = ctx;
-  c->pieces.push_back(ta_chunk::Piece{0, (size_t)bytes & ~(size_t)255, false});
+  c->pieces.push_back(ta_chunk::Piece{0, c->bytes, false});
   return c;
 }
 void ta_chunk_close(ta_chunk *c) { delete c; }
