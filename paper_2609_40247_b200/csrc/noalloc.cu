@@ -229,6 +229,8 @@ extern "C" ta_status ta_lane_gaps_noalloc_host(const int64_t *ts_start, const in
                                                ta_lane_gaps *lane_out, ta_lane_gaps *host_row, void *cuda_stream) {
   if (n < 0 || win_t0 >= win_t1 || !lane_out || (n > 0 && (!ts_start || !ts_end || !gap_before)))
     return TA_ERR_INVALID_ARG;
+  if (((uintptr_t)lane_out | (n > 0 ? (uintptr_t)ts_start | (uintptr_t)ts_end | (uintptr_t)gap_before : 0)) & 7u)
+    return TA_ERR_INVALID_ARG;  // 64-bit accesses
   if (n > NA_MAX_RECORDS) return TA_ERR_TOO_LARGE;  // the fixed scratch array covers no more
   if ((uint64_t)win_t1 - (uint64_t)win_t0 >= (1ull << 40)) return TA_ERR_TOO_LARGE;
   cudaStream_t st = (cudaStream_t)cuda_stream;

@@ -84,3 +84,14 @@ def test_arguments_are_rejected_before_any_device_work():
                       (L.ta_blame_gaps, 4)):
         raw = ctypes.CFUNCTYPE(ctypes.c_int, *([vp] * nargs))(ctypes.cast(fn, vp).value)
         assert raw(None, *([ctypes.addressof(out)] * (nargs - 1))) == 1
+
+
+def test_misaligned_columns_of_the_no_alloc_scan_are_rejected():
+    from paper_2609_40247_b200 import ta
+    L = ta.lib()
+    good = [1 << 40, (1 << 40) + (1 << 20), (1 << 40) + (2 << 20), (1 << 40) + (3 << 20)]  # never touched
+    for k in range(4):
+        for off in (1, 4, 7):
+            ts, te, gap, row = (a + (off if i == k else 0) for i, a in enumerate(good))
+            assert L.ta_lane_gaps_noalloc(ts, te, 10, 0, 100, gap, row, None) == 1
+            assert L.ta_lane_gaps_noalloc_host(ts, te, 10, 0, 100, gap, row, None, None) == 1
