@@ -65,33 +65,39 @@ static void *cache_take(int device, cudaStream_t stream, size_t bytes) {
   return nullptr;
 }
 static void cache_put(int device, cudaStream_t stream, void *p, size_t bytes) {
-  std::lock_guard<std::mutex> lock(g_cache_guard);
-  g_cache.push_back(CachedBlock{p, bytes, device, stream, g_cache_gen});
-}
-// Called when a handle goes away, after its stream has been synchronised.  Invariant: a block
-// enters the cache only once the stream it was used on is idle (ta_dfree and ta_free are only
-// reached behind a synchronisation), so handing it back to the pool below cannot race with work
-// still queued on that stream - cudaFree itself does not wait for a stream-ordered allocation.
-static void cache_age() {
-  std::vector<void *> out;
-  {
+  try {
     std::lock_guard<std::mutex> lock(g_cache_guard);
-    g_cache_gen++;
-    for (size_t i = 0; i < g_cache.size();) {
-      if (g_cache[i].gen + 2 < g_cache_gen) {
-        out.push_back(g_cache[i].p);
-        g_cache[i] = g_cache.back();
-        g_cache.pop_back();
-      } else {
-        i++;
-      }
-    }
+    g_cache.push_back(CachedBlock{p, bytes, device, stream, g_cache_gen});
+  } catch (...) {  // no host memory to remember it by
+    cudaFreeAsync(p, stream);
   }
-  for (void *p : out) cudaFree(p);  // the stream the block was used on may no longer exist
+}
+// Called when a handle goes away.  Invariant: a block enters the cache only once the work that used it
+// is done (ta_dfree is reached behind the wait that ends a call, and what it is given for later behind
+// the next one; ta_free synchronises the stream), so handing it back to the pool below cannot race with
+// a kernel of the stream it was used on - cudaFree itself does not wait for a stream-ordered allocation.
+static void cache_age() {
+  bool first = true;
+  for (void *p = nullptr;; cudaFree(p)) {  // the stream the block was used on may no longer exist
+    std::lock_guard<std::mutex> lock(g_cache_guard);
+    if (first) g_cache_gen++;
+    first = false;
+    size_t i = 0;
+    while (i < g_cache.size() && g_cache[i].gen + 2 >= g_cache_gen) i++;
+    if (i == g_cache.size()) return;
+    p = g_cache[i].p;
+    g_cache[i] = g_cache.back();
+    g_cache.pop_back();
+  }
 }
 
 void *ta_dalloc(ta_window *h, size_t bytes) {
   if (bytes == 0) bytes = 256;
+  if (h->allocs.size() == h->allocs.capacity()) {  // host memory first: a block must not be lost for want of it
+    std::lock_guard<std::mutex> lock(h->alloc_guard);
+    h->alloc_bytes.reserve(2 * h->allocs.size() + 32);
+    h->allocs.reserve(2 * h->allocs.size() + 32);
+  }
   void *p = nullptr;
   if (h->env.alloc) {
     p = h->env.alloc(bytes, h->env.ctx);
@@ -180,8 +186,12 @@ static unsigned char *pin_take() {
 }
 static void pin_put(unsigned char *p) {
   if (!p) return;
-  std::lock_guard<std::mutex> lock(g_pin_guard);
-  g_pin_free.push_back(p);
+  try {
+    std::lock_guard<std::mutex> lock(g_pin_guard);
+    g_pin_free.push_back(p);
+  } catch (...) {
+    cudaFreeHost(p);
+  }
 }
 
 // Writes up to TA_FETCH_MAX device regions into the mapped staging block: one launch in place of
@@ -383,6 +393,24 @@ void ta_profile_mark(cudaStream_t st, int begin, double bytes) {
     g_prof_events.push_back(e);
   }
   cudaEventRecord(g_prof_events[g_prof_used++], st);
+}
+
+// What the library throws are failed allocations of host memory (its tables grow with the windows); none
+// leaves an entry point.
+template <class F>
+static ta_status no_throw(F f) {
+  try {
+    return f();
+  } catch (...) {
+    return TA_ERR_OOM;
+  }
+}
+template <class F>
+static ta_status run_call(ta_window *h, F f) {
+  return no_throw([&]() -> ta_status {
+    TA_TRY(begin_call(h));
+    return f();
+  });
 }
 
 extern "C" {
@@ -612,52 +640,56 @@ ta_status ta_load_window(const ta_env *env, const ta_event *events, int64_t n,
   h->d_on_path = nullptr;
   h->d_status = nullptr;
   h->zero_bytes = h->zero_used = 0;
-  stage_open(h->out);
-  h->h_off.assign(win_off, win_off + W + 1);
-  h->h_t0.assign(win_t0, win_t0 + W);
-  h->h_t1.assign(win_t1, win_t1 + W);
   *handle = h;
-  TA_TRY(begin_call(h));
-  return load_impl(h, events, events_on_device, out_summary);
+  return no_throw([&]() -> ta_status {
+    stage_open(h->out);
+    h->h_off.assign(win_off, win_off + W + 1);
+    h->h_t0.assign(win_t0, win_t0 + W);
+    h->h_t1.assign(win_t1, win_t1 + W);
+    TA_TRY(begin_call(h));
+    return load_impl(h, events, events_on_device, out_summary);
+  });
 }
 
 ta_status ta_sort_timeline(ta_window *h, ta_sort_result *out) {
   if (!h || !out) return TA_ERR_INVALID_ARG;
   if (!(h->stage & 1) || (h->stage & 2)) return TA_ERR_ORDER;
-  TA_TRY(begin_call(h));
-  TA_TRY(ta_run_sort_timeline(h));
-  h->stage |= 2;
-  *out = h->sorted;
-  return TA_OK;
+  return run_call(h, [&]() -> ta_status {
+    TA_TRY(ta_run_sort_timeline(h));
+    h->stage |= 2;
+    *out = h->sorted;
+    return TA_OK;
+  });
 }
 
 ta_status ta_correlate_launches(ta_window *h, ta_join_result *out, ta_join_summary *out_summary) {
   if (!h || !out) return TA_ERR_INVALID_ARG;
   if (!(h->stage & 2) || (h->stage & 4)) return TA_ERR_ORDER;
-  TA_TRY(begin_call(h));
-  TA_TRY(ta_run_correlate(h, out_summary));
-  h->stage |= 4;
-  *out = h->join;
-  return TA_OK;
+  return run_call(h, [&]() -> ta_status {
+    TA_TRY(ta_run_correlate(h, out_summary));
+    h->stage |= 4;
+    *out = h->join;
+    return TA_OK;
+  });
 }
 
 ta_status ta_attribute_operators(ta_window *h, ta_attr_result *out, ta_attr_summary *out_summary) {
   if (!h || !out) return TA_ERR_INVALID_ARG;
   if (!(h->stage & 4) || (h->stage & 8)) return TA_ERR_ORDER;
-  TA_TRY(begin_call(h));
-  ta_status s = ta_run_attribute(h, out_summary);
-  if (s != TA_OK && s != TA_ERR_DEPTH && s != TA_ERR_BAD_NESTING) return s;
-  h->stage |= 8;
-  h->attr_status = (int)s;
-  *out = h->attr;
-  return s;
+  return run_call(h, [&]() -> ta_status {
+    ta_status s = ta_run_attribute(h, out_summary);
+    if (s != TA_OK && s != TA_ERR_DEPTH && s != TA_ERR_BAD_NESTING) return s;
+    h->stage |= 8;
+    h->attr_status = (int)s;
+    *out = h->attr;
+    return s;
+  });
 }
 
 ta_status ta_stream_gaps(ta_window *h, int64_t min_gap_ns, ta_gap_result *out) {
   if (!h || !out) return TA_ERR_INVALID_ARG;
   if (!(h->stage & 2)) return TA_ERR_ORDER;
-  TA_TRY(begin_call(h));
-  return ta_run_gaps(h, min_gap_ns, out);
+  return run_call(h, [&] { return ta_run_gaps(h, min_gap_ns, out); });
 }
 
 ta_status ta_aggregate_ops(ta_window *h, uint32_t kind_mask, int32_t value_sel, ta_agg_result *out) {
@@ -668,23 +700,20 @@ ta_status ta_aggregate_ops(ta_window *h, uint32_t kind_mask, int32_t value_sel, 
   if (value_sel == 1 && (!(h->stage & 8) || h->attr_status != 0)) return TA_ERR_ORDER;
   if (value_sel == 2 && !h->d_op_gap_ns) return TA_ERR_ORDER;
   if (value_sel == 3 && !h->d_on_path) return TA_ERR_ORDER;
-  TA_TRY(begin_call(h));
-  return ta_run_aggregate(h, kind_mask, value_sel, out);
+  return run_call(h, [&] { return ta_run_aggregate(h, kind_mask, value_sel, out); });
 }
 
 ta_status ta_match_collectives(ta_window *h, const ta_comm_size *sizes, int32_t n_comms,
                                ta_coll_result *out) {
   if (!h || !out || n_comms < 0 || (n_comms > 0 && !sizes)) return TA_ERR_INVALID_ARG;
   if (!(h->stage & 2)) return TA_ERR_ORDER;
-  TA_TRY(begin_call(h));
-  return ta_run_collectives(h, sizes, n_comms, out);
+  return run_call(h, [&] { return ta_run_collectives(h, sizes, n_comms, out); });
 }
 
 ta_status ta_rollup_operators(ta_window *h, ta_rollup_result *out, ta_rollup_summary *out_summary) {
   if (!h || !out || !out_summary) return TA_ERR_INVALID_ARG;
   if (!(h->stage & 8) || h->attr_status != 0) return TA_ERR_ORDER;
-  TA_TRY(begin_call(h));
-  return ta_run_rollup(h, out, out_summary);
+  return run_call(h, [&] { return ta_run_rollup(h, out, out_summary); });
 }
 
 ta_status ta_operator_sol(ta_window *h, const double *flops, const double *bytes,
@@ -693,8 +722,7 @@ ta_status ta_operator_sol(ta_window *h, const double *flops, const double *bytes
   if (!h || !out || !out_summary || (h->n > 0 && (!flops || !bytes))) return TA_ERR_INVALID_ARG;
   if (!(peak_flops > 0.0) || !(peak_bw > 0.0)) return TA_ERR_INVALID_ARG;
   if (!(h->stage & 8) || h->attr_status != 0) return TA_ERR_ORDER;
-  TA_TRY(begin_call(h));
-  return ta_run_sol(h, flops, bytes, counts_on_device, peak_flops, peak_bw, out, out_summary);
+  return run_call(h, [&] { return ta_run_sol(h, flops, bytes, counts_on_device, peak_flops, peak_bw, out, out_summary); });
 }
 
 ta_status ta_blame_gaps(ta_window *h, const ta_gap_result *gaps, ta_blame_result *out,
@@ -702,22 +730,19 @@ ta_status ta_blame_gaps(ta_window *h, const ta_gap_result *gaps, ta_blame_result
   if (!h || !gaps || !out || !out_summary) return TA_ERR_INVALID_ARG;
   if (gaps->n_long_gaps < 0 || (gaps->n_long_gaps > 0 && !gaps->long_gaps)) return TA_ERR_INVALID_ARG;
   if (!(h->stage & 4)) return TA_ERR_ORDER;
-  TA_TRY(begin_call(h));
-  return ta_run_blame(h, gaps, out, out_summary);
+  return run_call(h, [&] { return ta_run_blame(h, gaps, out, out_summary); });
 }
 
 ta_status ta_critical_path(ta_window *h, ta_critpath_result *out, ta_critpath_summary *out_summary) {
   if (!h || !out || !out_summary) return TA_ERR_INVALID_ARG;
   if (!(h->stage & 4)) return TA_ERR_ORDER;
-  TA_TRY(begin_call(h));
-  return ta_run_critpath(h, out, out_summary);
+  return run_call(h, [&] { return ta_run_critpath(h, out, out_summary); });
 }
 
 ta_status ta_device_overlap(ta_window *h, ta_overlap_result *out) {
   if (!h || !out) return TA_ERR_INVALID_ARG;
   if (!(h->stage & 2)) return TA_ERR_ORDER;
-  TA_TRY(begin_call(h));
-  return ta_run_overlap(h, out);
+  return run_call(h, [&] { return ta_run_overlap(h, out); });
 }
 
 ta_status ta_fetch(ta_window *h, int32_t count, void *const *dst, const void *const *src, const uint64_t *bytes) {
@@ -729,8 +754,10 @@ ta_status ta_fetch(ta_window *h, int32_t count, void *const *dst, const void *co
   // a block of its own: results are read while another thread is in a call on the handle, or reads as well
   ResultStage o;
   stage_open(o);
-  for (int32_t i = 0; i < count; i++) stage_queue(o, dst[i], src[i], (size_t)bytes[i]);
-  const ta_status s = stage_deliver(h, o);
+  const ta_status s = no_throw([&]() -> ta_status {
+    for (int32_t i = 0; i < count; i++) stage_queue(o, dst[i], src[i], (size_t)bytes[i]);
+    return stage_deliver(h, o);
+  });
   if (s != TA_OK) cudaStreamSynchronize(h->stream);  // nothing queued may write to the block any more
   pin_put(o.pin);
   return s;
@@ -772,7 +799,12 @@ ta_chunk *ta_chunk_open(void *base, uint64_t bytes, void *(*alloc)(size_t, void 
   c->alloc = alloc;
   c->release = release;
   c->ctx = ctx;
-  c->pieces.push_back(ta_chunk::Piece{0, c->bytes, false});
+  try {
+    c->pieces.push_back(ta_chunk::Piece{0, c->bytes, false});
+  } catch (...) {
+    delete c;
+    return nullptr;
+  }
   return c;
 }
 void ta_chunk_close(ta_chunk *c) { delete c; }
@@ -785,11 +817,16 @@ void *ta_chunk_alloc(size_t bytes, void *chunk) {
         (best == c->pieces.size() || c->pieces[i].bytes < c->pieces[best].bytes))
       best = i;
   if (best == c->pieces.size()) return c->alloc(bytes, c->ctx);
-  ta_chunk::Piece &p = c->pieces[best];
-  const size_t off = p.off, rest = p.bytes - need;
-  p.bytes = need;
-  p.used = true;
-  if (rest) c->pieces.insert(c->pieces.begin() + best + 1, ta_chunk::Piece{off + need, rest, false});
+  const size_t off = c->pieces[best].off, rest = c->pieces[best].bytes - need;
+  if (rest) {
+    try {
+      c->pieces.insert(c->pieces.begin() + best + 1, ta_chunk::Piece{off + need, rest, false});
+    } catch (...) {  // no host memory to write the split down: the chunk stays as it is
+      return c->alloc(bytes, c->ctx);
+    }
+  }
+  c->pieces[best].bytes = need;
+  c->pieces[best].used = true;
   return c->base + off;
 }
 void ta_chunk_release(void *ptr, void *chunk) {

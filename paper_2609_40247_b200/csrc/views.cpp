@@ -51,17 +51,22 @@ static PyObject *part(PyObject *, PyObject *const *args, Py_ssize_t n) {
   if (PyErr_Occurred()) return nullptr;
   PyObject *base = PyTuple_GET_ITEM(args[0], 2);
   if (at < lo || at > hi || len > hi - at || !THPVariable_Check(base)) Py_RETURN_NONE;
-  const at::Tensor &t = THPVariable_Unpack(base);
-  if (t.dim() != 1 || (unsigned long long)t.numel() != hi - lo) {
-    PyErr_SetString(PyExc_ValueError, "part: not a tensor of these bytes");
+  try {
+    const at::Tensor &t = THPVariable_Unpack(base);
+    if (t.dim() != 1 || (unsigned long long)t.numel() != hi - lo) {
+      PyErr_SetString(PyExc_ValueError, "part: not a tensor of these bytes");
+      return nullptr;
+    }
+    at::Tensor r = at::detail::make_tensor<c10::TensorImpl>(c10::TensorImpl::VIEW, c10::Storage(t.storage()),
+                                                            t.key_set(), t.dtype());
+    c10::TensorImpl *impl = r.unsafeGetTensorImpl();
+    impl->set_storage_offset(t.storage_offset() + (int64_t)(at - lo));
+    impl->set_sizes_contiguous(at::IntArrayRef{(int64_t)len});
+    return THPVariable_Wrap(std::move(r));
+  } catch (const std::exception &e) {
+    PyErr_SetString(PyExc_RuntimeError, e.what());
     return nullptr;
   }
-  at::Tensor r = at::detail::make_tensor<c10::TensorImpl>(c10::TensorImpl::VIEW, c10::Storage(t.storage()),
-                                                          t.key_set(), t.dtype());
-  c10::TensorImpl *impl = r.unsafeGetTensorImpl();
-  impl->set_storage_offset(t.storage_offset() + (int64_t)(at - lo));
-  impl->set_sizes_contiguous(at::IntArrayRef{(int64_t)len});
-  return THPVariable_Wrap(std::move(r));
 }
 
 static PyMethodDef methods[] = {

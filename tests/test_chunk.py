@@ -56,3 +56,32 @@ def test_pieces_are_aligned_and_inside_the_block(base, size):
     if room > 0:  # all of it is one piece again
         assert c.alloc(room) == base + -base % 256
     c.lib.ta_chunk_close(c.ptr)
+
+
+_NO_MEMORY = """
+import resource, sys
+sys.path[:0] = [%r, %r]
+from test_chunk import Chunk
+c = Chunk(1 << 40, 1 << 40)
+for _ in range(1000):  # whatever Python and the loader set up on first use
+    c.release(c.alloc(1))
+now = int(open("/proc/self/statm").read().split()[0]) * resource.getpagesize()
+resource.setrlimit(resource.RLIMIT_AS, (now + (3 << 20), now + (3 << 20)))
+alloc, ptr, i = c.lib.chunk_alloc, c.ptr, 0
+while i < 2000000 and not c.asked:
+    p = alloc(1, ptr)
+    i += 1
+assert c.asked == [1] and p == 0x7000 + 256 and i > 1000, (c.asked, i)
+print("ok", i)
+"""
+
+
+def test_a_list_that_cannot_grow_is_no_exception():
+    """The list of pieces needs host memory; without any more the request goes to the caller."""
+    import os
+    import subprocess
+    import sys
+    here = os.path.dirname(os.path.abspath(__file__))
+    r = subprocess.run([sys.executable, "-c", _NO_MEMORY % (os.path.dirname(here), here)], capture_output=True,
+                       text=True, timeout=120)
+    assert r.returncode == 0 and r.stdout.startswith("ok"), (r.returncode, r.stdout, r.stderr)
