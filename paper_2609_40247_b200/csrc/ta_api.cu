@@ -164,18 +164,16 @@ void ta_dfree(ta_window *h, void *p) {
 }
 
 // Page-locked staging blocks are expensive to create (a system call and a page-table update
-// each), so they are kept for the life of the process and handed from handle to handle.
+// each), so up to TA_PIN_KEEP of them are kept for the life of the process and handed from handle to handle.
+#define TA_PIN_KEEP 32
 #define TA_PIN_BYTES (512u << 10)  // and 64 bytes behind them for the number of the last fetch
 static std::mutex g_pin_guard;
-static std::vector<unsigned char *> g_pin_free;
+static unsigned char *g_pin_free[TA_PIN_KEEP];
+static int g_pins_idle = 0;
 static unsigned char *pin_take() {
   {
     std::lock_guard<std::mutex> lock(g_pin_guard);
-    if (!g_pin_free.empty()) {
-      unsigned char *p = g_pin_free.back();
-      g_pin_free.pop_back();
-      return p;
-    }
+    if (g_pins_idle > 0) return g_pin_free[--g_pins_idle];
   }
   void *p = nullptr;
   if (cudaHostAlloc(&p, TA_PIN_BYTES + 64, cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
@@ -186,12 +184,14 @@ static unsigned char *pin_take() {
 }
 static void pin_put(unsigned char *p) {
   if (!p) return;
-  try {
+  {
     std::lock_guard<std::mutex> lock(g_pin_guard);
-    g_pin_free.push_back(p);
-  } catch (...) {
-    cudaFreeHost(p);
+    if (g_pins_idle < TA_PIN_KEEP) {
+      g_pin_free[g_pins_idle++] = p;
+      return;
+    }
   }
+  cudaFreeHost(p);
 }
 
 // Writes up to TA_FETCH_MAX device regions into the mapped staging block: one launch in place of

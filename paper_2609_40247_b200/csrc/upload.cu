@@ -17,6 +17,8 @@
 #define UP_PIECES 24
 #define UP_THREADS 6
 #define UP_MIN (4u << 20)  // below this the threads cost more than they save
+#define UP_RINGS 4         // rings (24 MB each) per device at most: the link is shared by more uploads than that anyway
+#define UP_DEVICES 64
 
 namespace {
 struct Ring {
@@ -27,7 +29,8 @@ struct Ring {
   unsigned long long last_used;  // number of the handle that used it last
 };
 std::mutex g_ring_guard;
-std::vector<Ring *> g_rings;  // idle ones; an upload takes one out and puts it back
+Ring *g_idle[UP_DEVICES][UP_RINGS];  // an upload takes one out and puts it back
+int g_made[UP_DEVICES];              // idle ones and those in use
 unsigned long long g_handles = 0;
 
 void ring_free(Ring *r) {
@@ -36,35 +39,52 @@ void ring_free(Ring *r) {
   if (r->buf) cudaFreeHost(r->buf);
   delete r;
 }
-Ring *ring_take(int device) {
-  {
-    std::lock_guard<std::mutex> lock(g_ring_guard);
-    for (size_t i = 0; i < g_rings.size(); i++)
-      if (g_rings[i]->device == device) {
-        Ring *r = g_rings[i];
-        g_rings.erase(g_rings.begin() + i);
-        return r;
-      }
-  }
+Ring *ring_make(int device) {
   Ring *r = new (std::nothrow) Ring();
   if (!r) return nullptr;
-  memset(r, 0, sizeof(*r));
   r->device = device;
   void *p = nullptr;
-  if (cudaHostAlloc(&p, (size_t)UP_PIECE * UP_PIECES, cudaHostAllocPortable) != cudaSuccess) {
-    cudaGetLastError();
-    delete r;
-    return nullptr;
-  }
+  bool ok = cudaHostAlloc(&p, (size_t)UP_PIECE * UP_PIECES, cudaHostAllocPortable) == cudaSuccess;
   r->buf = (unsigned char *)p;
-  for (int i = 0; i < UP_PIECES; i++)
+  for (int i = 0; i < UP_PIECES && ok; i++)
     if (cudaEventCreateWithFlags(&r->ev[i], cudaEventDisableTiming) != cudaSuccess) {
-      cudaGetLastError();
       r->ev[i] = nullptr;
-      ring_free(r);
-      return nullptr;
+      ok = false;
     }
+  if (ok) return r;
+  cudaGetLastError();
+  ring_free(r);
+  return nullptr;
+}
+// null: as many as there may be are in use, or there is no memory for one
+Ring *ring_take(int device) {
+  if (device < 0 || device >= UP_DEVICES) return nullptr;
+  {
+    std::lock_guard<std::mutex> lock(g_ring_guard);
+    for (Ring *&idle : g_idle[device])
+      if (idle) {
+        Ring *r = idle;
+        idle = nullptr;
+        return r;
+      }
+    if (g_made[device] == UP_RINGS) return nullptr;
+    g_made[device]++;
+  }
+  Ring *r = ring_make(device);
+  if (!r) {
+    std::lock_guard<std::mutex> lock(g_ring_guard);
+    g_made[device]--;
+  }
   return r;
+}
+void ring_put(Ring *r) {
+  std::lock_guard<std::mutex> lock(g_ring_guard);
+  r->last_used = g_handles;
+  for (Ring *&idle : g_idle[r->device])
+    if (!idle) {
+      idle = r;
+      return;
+    }
 }
 }  // namespace
 
@@ -86,19 +106,20 @@ static void copy_piece(unsigned char *dst /* 64-byte aligned */, const unsigned 
 
 // Rings no upload has asked for during the lifetime of the last 64 handles are given back.
 void ta_upload_age() {
-  std::vector<Ring *> out;
+  Ring *out[UP_RINGS];
+  int n = 0;
   {
     std::lock_guard<std::mutex> lock(g_ring_guard);
     g_handles++;
-    for (size_t i = 0; i < g_rings.size();)
-      if (g_rings[i]->last_used + 64 < g_handles) {
-        out.push_back(g_rings[i]);
-        g_rings.erase(g_rings.begin() + i);
-      } else {
-        i++;
-      }
+    for (int d = 0; d < UP_DEVICES && n == 0; d++)  // (of one device at a time)
+      for (Ring *&idle : g_idle[d])
+        if (idle && idle->last_used + 64 < g_handles) {
+          out[n++] = idle;
+          idle = nullptr;
+          g_made[d]--;
+        }
   }
-  for (Ring *r : out) ring_free(r);
+  for (int i = 0; i < n; i++) ring_free(out[i]);
 }
 
 ta_status ta_upload(ta_window *h, void *dst, const void *src, size_t bytes) {
@@ -143,26 +164,23 @@ ta_status ta_upload(ta_window *h, void *dst, const void *src, size_t bytes) {
     // half of the host's cores at most, a thread per four pieces at most
     size_t threads = std::max<size_t>(1, std::min<size_t>(UP_THREADS, std::thread::hardware_concurrency() / 2));
     threads = std::min(threads, (pieces + 3) / 4);
-    std::vector<std::thread> others;
+    std::thread others[UP_THREADS];
     for (size_t t = 1; t < threads; t++) {
       try {
-        others.emplace_back(work);
+        others[t] = std::thread(work);
       } catch (...) {  // no more threads: those there are do the work
         break;
       }
     }
     work();
-    for (std::thread &t : others) t.join();
+    for (std::thread &t : others)
+      if (t.joinable()) t.join();
   }
   for (int i = 0; i < UP_PIECES; i++) r->used[i] = r->used[i] || issued[i].load() != 0;
-  {
-    std::lock_guard<std::mutex> lock(g_ring_guard);
-    r->last_used = g_handles;
-    g_rings.push_back(r);
-  }
   if (failed.load()) {
     h->last_cuda = cudaGetLastError();
-    return TA_ERR_CUDA;
+    cudaStreamSynchronize(h->stream);  // what has been sent off still reads the buffers
   }
-  return TA_OK;
+  ring_put(r);
+  return failed.load() ? TA_ERR_CUDA : TA_OK;
 }

@@ -52,3 +52,33 @@ def test_four_threads_analyse_different_windows_at_once(torch_alloc):
     args, sizes, want = work[0]
     assert_same(want, run_gpu(*args, comm_sizes=sizes, use_torch_allocator=torch_alloc))
     assert np.array_equal(want["perm"], run_gpu(*args, comm_sizes=sizes)["perm"])
+
+
+def test_more_uploads_at_once_than_there_are_rings_of_buffers():
+    """Nine threads hand over records in pageable memory together, again and again: some go through
+    the staged upload, the rest through the driver's own copy."""
+    import torch
+    wl = synth.make_workload("c2", 0.04, truth=False)
+    args = (np.ascontiguousarray(wl.events), wl.win_off, wl.win_t0, wl.win_t1)
+    assert args[0].nbytes > 24 << 20
+    want = run_gpu(*args, comm_sizes=wl.comm_sizes)
+    errors, start = [], threading.Barrier(9)
+
+    def worker():
+        try:
+            torch.cuda.set_device(0)
+            with torch.cuda.stream(torch.cuda.Stream()):
+                for _ in range(3):
+                    start.wait(120)
+                    assert_same(want, run_gpu(*args, comm_sizes=wl.comm_sizes, on_device=False))
+        except BaseException as exc:
+            errors.append(exc)
+            start.abort()
+
+    threads = [threading.Thread(target=worker) for _ in range(9)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    if errors:
+        raise errors[0]
