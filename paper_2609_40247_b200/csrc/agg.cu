@@ -688,8 +688,10 @@ static ta_status ta_run_aggregate_sorted(ta_window *h, uint32_t kind_mask, int v
   AggSelOut so{c, k_in, v_in};
   TA_TRY((launch_scan<OpAdd, AggSelIn, AggSelOut>(h, nv, si, so, OpAdd(), s1)));
   u64 m64 = 0;
+  int32_t words[ST_WORDS];
   TA_TRY(ta_queue_d2h(h, &m64, s1.total, 8));
-  TA_TRY(ta_sync_fetch(h));
+  TA_TRY(ta_read_status(h, words));
+  if (words[ST_ERR]) return (ta_status)words[ST_ERR];  // (nothing was selected then)
   const int64_t m = (int64_t)m64;
   if (m == 0) { ta_dfree(h, t1); return TA_OK; }
 
@@ -733,7 +735,6 @@ static ta_status ta_run_aggregate_sorted(ta_window *h, uint32_t kind_mask, int v
   ta_launch(k_agg_sorted_rows, (unsigned)((ng + 255) / 256), 256, 0, st, c, ks, gstart, ng, o);
   ta_launch(k_agg_sorted_reduce, (unsigned)((m + 2047) / 2048), 256, 0, st, c, vs, gid, m, o);
   TA_CHECK_CUDA(h, cudaGetLastError());
-  int32_t words[ST_WORDS];
   TA_TRY(ta_read_status(h, words));
   ta_dfree(h, t1);
   ta_dfree(h, t2);

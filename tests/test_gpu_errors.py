@@ -251,3 +251,20 @@ def test_allocation_failure_at_every_request():
     torch.cuda.synchronize()
     a = (wl.events, wl.win_off, wl.win_t0, wl.win_t1)
     assert_same(run_oracle(*a), run_gpu(*a))
+
+
+def test_a_failed_handle_fails_the_aggregate_of_symbols_spread_wide():
+    """Symbols are ranked through a table or grouped by sorting then; both notice the failure."""
+    import torch
+    wl = synth.make_workload("c1", 0.02, truth=False)
+    ev = wl.events.copy()
+    ev["name_id"] = (ev["name_id"].astype(np.int64) * 2654435761 % (1 << 31)).astype(np.int32)
+    buf = torch.from_numpy(np.ascontiguousarray(ev).view(np.uint8).reshape(-1)).cuda()
+    for ranked in (False, True):
+        with ta.Window(buf, wl.win_off, wl.win_t0, wl.win_t1) as w:
+            w.sort_timeline()
+            if ranked:
+                assert w.aggregate_ops(ta.DEVICE_KINDS, 0).n_groups > 0
+            w.inject_device_error(TA_ERR_TIMEOUT)
+            for mask in (ta.DEVICE_KINDS, 1, 63):
+                assert _status(lambda: w.aggregate_ops(mask, 0)) == TA_ERR_TIMEOUT
