@@ -48,8 +48,11 @@ __host__ __device__ __forceinline__ i64 unbias64(u64 v) { return (i64)(v ^ (1ull
 
 // ---- hashed addressing -------------------------------------------------------
 __device__ __forceinline__ u32 join_hash(const JoinArgs &a, int slot, i64 c) {
-  // multiplicative hashing (the golden ratio in 64 bits), twice so that low bits reach the top word
-  u64 x = ((u64)c ^ ((u64)(u32)slot << 40)) * 0x9E3779B97F4A7C15ull;
+  // multiplicative hashing (the golden ratio in 64 bits), twice so that low bits reach the top word; the
+  // slot enters with all 64 bits: shifted to the upper ones it met ids that carry a number there, and
+  // 64 processes with a rank or a thread in bits 40 and up shared every chain (8 M records 7.57 ms instead
+  // of 0.51)
+  u64 x = ((u64)c + (u64)(u32)slot * 0xD6E8FEB86659FD93ull) * 0x9E3779B97F4A7C15ull;
   x = (x ^ (x >> 32)) * 0x9E3779B97F4A7C15ull;
   return __umulhi((u32)(x >> 32), a.table_size);
 }

@@ -240,3 +240,37 @@ def test_summaries_too_large_for_the_staging_kernel(windows, pids):
     assert o["attr_status"] == 0 and int(o["join_sum"]["n_matched"].min()) > 0
     assert int(o["sol_sum"]["n_resolved"].min()) > 0 and int(o["roll_sum"].sum()) > 0
     assert_same(o, g)
+
+
+def test_hashed_ids_with_a_number_in_their_upper_bits_share_no_chains():
+    """Ids that carry a rank or a thread in bits 40 and up, on 64 processes of 32 threads: the join
+    takes about as long as with ids of no structure."""
+    import time
+    import torch
+    from paper_2609_40247_b200 import ta
+    P, T, per = 64, 32, 500
+    p, t, k = (x.astype(np.int64) for x in np.ogrid[:P, :T, :per])
+    ev = np.zeros((P, T, per, 2), dtype=synth.EVENT_DTYPE)
+    ev["pid"], ev["stream"] = p[..., None], t[..., None]
+    ev["kind"][..., 0], ev["kind"][..., 1] = 2, 3
+    ev["ts_start"] = 1_000 + k[..., None] * 1_000 + np.array([0, 400])
+    ev["ts_end"] = ev["ts_start"] + 300
+
+    def join(ids):
+        ev["corr_id"] = np.broadcast_to(ids, (P, T, per))[..., None]
+        flat = np.ascontiguousarray(ev).reshape(-1)
+        buf = torch.from_numpy(flat.view(np.uint8)).cuda()
+        best = 1e9
+        for _ in range(5):
+            with ta.Window(buf, [0, len(flat)], [0], [per * 1_000 + 5_000]) as w:
+                w.sort_timeline()
+                torch.cuda.synchronize()
+                at = time.perf_counter()
+                j = w.correlate_launches()
+                best = min(best, time.perf_counter() - at)
+                assert int(j.join_sum["n_matched"][0]) == P * T * per and int(j.join_sum["n_dup_launch"][0]) == 0
+        return best
+
+    mixed = join(((t << 40) | (p << 48) | k) * np.int64(-7046029254386353131))
+    assert join((t << 40) | k) < 4 * mixed
+    assert join((p << 40) | (t << 32) | k) < 4 * mixed
