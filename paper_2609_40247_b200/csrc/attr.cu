@@ -134,15 +134,17 @@ __global__ void __launch_bounds__(AT_THREADS) k_attr_agg(AttrArgs a) {
   constexpr int AHEAD = 4;  // rows whose columns are in flight
   for (int64_t hi = vend; hi > from; hi -= 32 * AHEAD) {
     i64 e[AHEAD];
+    bool op[AHEAD];
 #pragma unroll
     for (int r = 0; r < AHEAD; r++) {
       const int64_t p = hi - 32 * (r + 1) + lane;
-      e[r] = p >= from && a.kind[p] == TA_KIND_OP ? (i64)a.te[p] : INT64_MIN;
+      op[r] = p >= from && a.kind[p] == TA_KIND_OP;
+      e[r] = op[r] ? (i64)a.te[p] : 0;
     }
 #pragma unroll
     for (int r = 0; r < AHEAD; r++) {
       // equal ends nest: the earlier operator encloses the later one
-      u32 m = __ballot_sync(0xffffffffu, e[r] >= bar && e[r] != INT64_MIN);
+      u32 m = __ballot_sync(0xffffffffu, op[r] && e[r] >= bar);
       while (m) {
         const int src = 31 - __clz((int)m);
         m &= ~(1u << src);

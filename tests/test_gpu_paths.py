@@ -274,3 +274,29 @@ def test_hashed_ids_with_a_number_in_their_upper_bits_share_no_chains():
     mixed = join(((t << 40) | (p << 48) | k) * np.int64(-7046029254386353131))
     assert join((t << 40) | k) < 4 * mixed
     assert join((p << 40) | (t << 32) | k) < 4 * mixed
+
+
+@pytest.mark.parametrize("n", [40, 129, 700])
+def test_operators_at_the_first_instant_there_is(n):
+    """Records at the smallest time of all, over several tiles: an empty operator there encloses the
+    empty records behind it."""
+    import torch
+    from oracle.ta_oracle import Oracle
+    from paper_2609_40247_b200 import ta
+    first = -2**63
+    ev = np.zeros(n, dtype=synth.EVENT_DTYPE)
+    ev["ts_start"] = ev["ts_end"] = first
+    ev["kind"] = 1
+    ev["kind"][0] = 0
+    ev["ts_end"][1], ev["kind"][1] = first + 50, 0
+    o = Oracle(ev, [0, n], [first], [first + 1_000])
+    o.load(), o.sort(), o.correlate(), o.attribute()
+    assert (o.get("parent") >= 0).sum() == n - 1
+    buf = torch.from_numpy(ev.view(np.uint8)).cuda()
+    with ta.Window(buf, [0, n], [first], [first + 1_000]) as w:
+        s = w.sort_timeline()
+        w.correlate_launches()
+        a = w.attribute_operators()
+        assert np.array_equal(s.numpy("perm"), o.get("perm"))
+        for k in ("parent", "depth"):
+            assert np.array_equal(a.numpy(k), o.get(k)), k
