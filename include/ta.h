@@ -604,7 +604,9 @@ ta_status ta_critical_path(ta_window *h, ta_critpath_result *out,
  * cannot afford the device-wide synchronisation an allocation or a free may
  * imply.  Every other entry point obtains its buffers through ta_env; this one
  * obtains no device memory: it calls no cudaMalloc, cudaFree or any routine that
- * allocates on the device (its first call page-locks a hundred bytes of host memory).
+ * allocates on the device.  (Its first call on a device asks for a hundred bytes of
+ * page-locked host memory, which may synchronise the device, and does without if there
+ * are none.)
  * Its scratch (tile descriptors of the scan, a counter, a status word: about
  * 16 KB) is a fixed array inside the library image, which every GPU that loads
  * the library holds until the process exits.

@@ -31,16 +31,17 @@ struct NaSums {
   u32 counter;         // tile tickets of the scan
   u32 pad[3];
 };
-struct NaScratch {
-  NaSums sum;
-  u64 state[NA_MAX_TILES + 1];  // tile descriptors of the max-scan
-};
 // the result in page-locked host memory, next to the device row the caller asked for
 struct NaHost {
   ta_lane_gaps row;
   int32_t err;
   u32 not_ascending;
   volatile u32 seq;  // the call's number, written last
+};
+struct NaScratch {
+  NaSums sum;
+  u64 state[NA_MAX_TILES + 1];  // tile descriptors of the max-scan
+  NaHost host;                  // stands in where no memory could be page-locked, and is copied
 };
 
 // Every device that loads the library holds this array until the process exits.
@@ -209,15 +210,20 @@ static NaDevice *na_device(u32 *seq) {
   NaDevice &d = g_na_device[dev];
   if (!d.scratch) {
     void *p = nullptr, *hp = nullptr, *hd = nullptr;
-    if (cudaGetSymbolAddress(&p, g_na_scratch) != cudaSuccess || !p ||
-        cudaHostAlloc(&hp, sizeof(NaHost), cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess ||
-        cudaHostGetDevicePointer(&hd, hp, 0) != cudaSuccess) {
+    if (cudaGetSymbolAddress(&p, g_na_scratch) != cudaSuccess || !p) {
       cudaGetLastError();
       return nullptr;
     }
-    memset(hp, 0, sizeof(NaHost));
-    d.host = (NaHost *)hp;
-    d.host_dev = (NaHost *)hd;
+    if (cudaHostAlloc(&hp, sizeof(NaHost), cudaHostAllocPortable | cudaHostAllocMapped) == cudaSuccess &&
+        cudaHostGetDevicePointer(&hd, hp, 0) == cudaSuccess) {
+      memset(hp, 0, sizeof(NaHost));
+      d.host = (NaHost *)hp;
+      d.host_dev = (NaHost *)hd;
+    } else {
+      cudaGetLastError();
+      if (hp) cudaFreeHost(hp);
+      d.host_dev = &((NaScratch *)p)->host;
+    }
     d.scratch = (NaScratch *)p;
   }
   *seq = ++d.seq;
@@ -255,15 +261,22 @@ extern "C" ta_status ta_lane_gaps_noalloc_host(const int64_t *ts_start, const in
     else
       ta_launch(k_lane_gaps_ascending, tiles, NA_THREADS, 0, st, ts_start, ts_end, n, win_t0, win_t1, gap_before, lane_out, sc, d->host_dev, seq);
     if (cudaGetLastError() != cudaSuccess) return TA_ERR_CUDA;
-    const NaHost *h = d->host;
-    TA_WAIT_SEQ(h->seq, seq, st);
+    NaHost copy;
+    const NaHost *h = d->host ? d->host : &copy;
+    if (d->host) {
+      TA_WAIT_SEQ(h->seq, seq, st);
+    } else if (cudaMemcpyAsync(&copy, d->host_dev, sizeof(copy), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+               cudaStreamSynchronize(st) != cudaSuccess) {
+      cudaGetLastError();
+      return TA_ERR_CUDA;
+    }
     if (h->seq != seq) return TA_ERR_CUDA;  // two calls overlapped
     std::atomic_thread_fence(std::memory_order_acquire);
     if (h->err) return (ta_status)h->err;
     if (host_row) *host_row = h->row;
     if (!h->not_ascending) break;
     if (scan) break;
-    d->host->seq = seq - 1;  // the scan announces itself again
+    if (d->host) d->host->seq = seq - 1;  // the scan announces itself again
   }
   return TA_OK;
 }
