@@ -130,10 +130,13 @@ void *ta_zalloc(ta_window *h, size_t bytes, ta_status *st) {
   void *p = ta_zpool(h, bytes);
   if (p) return p;
   p = ta_dalloc(h, bytes);
-  if (!p) *st = TA_ERR_OOM;
-  else if (cudaMemsetAsync(p, 0, bytes, h->stream) != cudaSuccess) {
+  if (!p) {
+    *st = TA_ERR_OOM;
+  } else if (cudaMemsetAsync(p, 0, bytes, h->stream) != cudaSuccess) {
     h->last_cuda = cudaGetLastError();
     *st = TA_ERR_CUDA;
+    ta_dfree(h, p);
+    p = nullptr;
   }
   return p;
 }

@@ -196,11 +196,11 @@ void *ta_dalloc(ta_window *h, size_t bytes);            // NULL on failure
 void ta_dfree(ta_window *h, void *p);                   // early release of one allocation
 // Memory that starts at zero.  Windows of up to TA_ZERO_POOL_RECORDS records clear one pool for all
 // their calls while they are loaded (a clearing is a launch: sixteen of the fifty operations of a
-// small window); what does not fit it, or comes after TA_ZERO_POOL is used up, is allocated and
+// small window); what does not fit it, or comes after it is used up, is allocated and
 // cleared on its own.  A pointer into the pool may be given to ta_dfree like any other (nothing
 // happens: the pool lives as long as the handle).
 #define TA_ZERO_POOL_RECORDS (1ll << 23)  // (128 MB of pool; at 16.8 M records clearing what nobody takes costs 1 %)
-void *ta_zalloc(ta_window *h, size_t bytes, ta_status *st);
+void *ta_zalloc(ta_window *h, size_t bytes, ta_status *st);  // NULL: *st says why
 void *ta_zpool(ta_window *h, size_t bytes);  // from the pool or NULL
 // carve sub-buffers out of one allocation
 struct Carver {
