@@ -33,7 +33,7 @@
 #define AG_STEP (AG_THREADS * AG_ITEMS)
 #define AG_SLOTS 256
 #define AG_ITEM (8 * AG_STEP)    // positions per CTA at most
-#define AG_FLUSH_EVERY 32768  // records per CTA between flushes (keeps 16-bit bins safe)
+static_assert(AG_ITEM < (1 << 15), "a CTA's bins are 16 bits wide, the limbs of its sums 17 bits in a word");
 
 struct AggArgs {
   int64_t n_valid;
@@ -194,9 +194,6 @@ __device__ __forceinline__ void agg_flush(const AggArgs &a, AggSmem &s) {
     const u32 c = s.hist[sl][b];
     if (c) atomicAdd(&a.d_hist[(size_t)s.key[sl] * TA_NBINS + b], c);
   }
-  __syncthreads();
-  agg_clear(s);
-  __syncthreads();
 }
 
 // Which of the thread's four records are selected, their values and symbols (a caller that makes no
@@ -307,7 +304,6 @@ template <bool TABLE>
 __device__ __forceinline__ void agg_chunk(const AggArgs &a) {
   __shared__ AggSmem s;
   if (ta_failed(a.status)) return;
-  int since_flush = 0;
   LaneWalker lw(a.lane_off, a.n_lanes, a.n_valid, a.n_valid);
   {
     // CTA b -> chunk (b mod G) * S + b / G: CTAs that run together work far apart in the
@@ -354,7 +350,7 @@ __device__ __forceinline__ void agg_chunk(const AggArgs &a) {
           slot = (slot + 1) & (AG_SLOTS - 1);
         }
         if (placed) {
-          // values are durations (>= 0), at most 32768 adds per flush: 2^15 x 2^17 fits a word
+          // values are durations (>= 0), fewer than 2^15 adds per CTA: 2^15 x 2^17 fits a word
           const u64 uv = (u64)v[j];
           atomicAdd(&s.sum[0][slot], (u32)(uv & 0x1FFFF));
           if (uv >> 17) atomicAdd(&s.sum[1][slot], (u32)((uv >> 17) & 0x1FFFF));
@@ -371,11 +367,6 @@ __device__ __forceinline__ void agg_chunk(const AggArgs &a) {
           agg_global_add(a, row, 1, (u64)v[j], ~vb, vb);
           atomicAdd(&a.d_hist[(size_t)row * TA_NBINS + bin], 1u);
         }
-      }
-      since_flush += AG_STEP;
-      if (since_flush >= AG_FLUSH_EVERY) {
-        agg_flush(a, s);
-        since_flush = 0;
       }
     }
   }
