@@ -33,14 +33,10 @@
 
 #define AT_THREADS 256
 #define AT_CAP 16
-#ifndef AS_MINB
 #define AS_MINB 4
-#endif
 // k_attr_ops: four records per thread keep it at 64 registers, four CTAs per SM (eight records and
 // three CTAs measured 0.12 ms slower on the 66.8 M record window: the kernel waits on gathers)
-#ifndef AT_OPS_MINB
 #define AT_OPS_MINB 4
-#endif
 
 struct AttrArgs {
   int64_t n, n_valid;
@@ -678,9 +674,7 @@ __global__ void __launch_bounds__(AS_WARPS * 32, AS_MINB) k_attr_resolve(AttrArg
 }
 
 // ---- device records inherit the operator of their launch ------------------------
-#ifndef AT_OPS_ITEMS
 #define AT_OPS_ITEMS 4
-#endif
 #define AT_OPS_TILE (AT_THREADS * AT_OPS_ITEMS)
 // adds kernels to an operator's row in memory (whose first / last are identities while it has none)
 __device__ __forceinline__ void attr_row_add(const AttrArgs &a, int32_t r, int cnt, i64 first, i64 last, i64 ns) {

@@ -18,19 +18,11 @@
 #include "ta_internal.cuh"
 
 #define GP_THREADS 256
-#ifndef GP_ITEMS
 #define GP_ITEMS 8
-#endif
-#ifndef GP_MINB
 #define GP_MINB 4
-#endif
 #define GP_TILE (GP_THREADS * GP_ITEMS)
-#ifndef GR_MINB
 #define GR_MINB 5
-#endif
-#ifndef GR_ROWS
 #define GR_ROWS 12
-#endif
 // lanes of a tile whose statistics are folded on chip: in a batch of many windows a lane is a
 // thousand records or so and a tile meets several (a batch of 512 windows of 65 k records: 395 us
 // with two lanes folded and the rest by global atomics per record)

@@ -130,9 +130,7 @@ __device__ __forceinline__ void join_fold(u64 (&t)[NS + NM], int cur, Emit emit)
 // A warp takes rows of 32 records of one host lane, JB_ROWS at a time, with the kinds and ids of the
 // next JB_ROWS on their way.  What an entry held before tells a first launch of its id from a repeated
 // one, so that launches, duplicates and ids are counted here and no later pass has to look them up.
-#ifndef JB_ROWS
 #define JB_ROWS 2
-#endif
 // adds a group of launches to the row of their window; k_join_probe takes the ids with a kernel off the orphans again
 __device__ __forceinline__ void launch_emit(ta_join_summary *sm, const u64 *t) {
   if (t[0] == 0) return;
@@ -239,12 +237,8 @@ __global__ void __launch_bounds__(JN_THREADS) k_join_build(JoinArgs a, int rows)
 // chain of three (columns, table, launch times), so a warp works on JP_ROWS rows at a time and has the
 // columns of the next JP_ROWS on their way meanwhile.  (A CTA per 1024 records, lanes walked by every
 // thread, two block barriers at the start: 1035 us of 66.8 M records, half of it in those waits.)
-#ifndef JP_MINB
 #define JP_MINB 3
-#endif
-#ifndef JP_ROWS
 #define JP_ROWS 3
-#endif
 
 // adds a group of probes to the row of their window
 __device__ __forceinline__ void join_emit(ta_join_summary *sm, const u64 *t) {
@@ -571,8 +565,5 @@ ta_status ta_run_correlate(ta_window *h, ta_join_summary *out_summary) {
   h->join.launch_latency = latency;
   h->join.queue_delay = qdelay;
   h->join.kernels_of_launch = kol;
-  if (n == 0) {
-    // nothing was launched: outputs are single dummy entries
-  }
   return TA_OK;
 }

@@ -25,11 +25,6 @@
 
 #define TRIPLE_EMPTY (~0ull)  // in the per-CTA caches and the sampling table
 
-__device__ __forceinline__ i64 warp_min_i64(i64 v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = min(v, (i64)__shfl_xor_sync(0xffffffffu, v, o));
-  return v;
-}
 __device__ __forceinline__ i64 warp_max_i64(i64 v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v = max(v, (i64)__shfl_xor_sync(0xffffffffu, v, o));
@@ -129,12 +124,8 @@ __global__ void __launch_bounds__(PL_THREADS) k_plan(const ta_event *ev, int64_t
 }
 
 // ---- discovery with staged tiles -----------------------------------------------------------
-#ifndef DS_THREADS
 #define DS_THREADS 256
-#endif
-#ifndef DS_RPT
 #define DS_RPT 2                          // records per thread and tile
-#endif
 #define DS_TILE (DS_THREADS * DS_RPT)     // 512 records = 20480 bytes
 #define DS_TILE_BYTES (DS_TILE * 40)
 #define DS_CACHE_BITS 9
@@ -184,7 +175,7 @@ struct DiscoverArgs {
   u64 *prekey;
   u32 *hist;      // [pass][256]: digit histograms of the passes over time bits
   u32 *slot_cnt;  // [window][TA_TRIPLE_SLOTS] kept records per triple slot, or null (too many windows)
-  int sbits, ibits;
+  int sbits;
 };
 
 struct __align__(128) DiscoverSmem {
@@ -823,13 +814,11 @@ ta_status ta_launch_discover(ta_window *h) {
     a.tt = h->d_triples; a.cm = h->d_comms; a.sum = h->d_load_sum; a.misc = h->d_misc;
     a.status = h->d_status; a.prekey = h->d_keys; a.hist = h->d_hist;
     a.slot_cnt = h->cnt_windows ? h->d_slot_cnt : nullptr;
-    a.sbits = sbits; a.ibits = 0;
+    a.sbits = sbits;
     TA_CHECK_CUDA(h, cudaFuncSetAttribute(k_discover_staged, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                           (int)sizeof(DiscoverSmem)));
     const int64_t tiles = (h->n + DS_TILE - 1) / DS_TILE;
-#ifndef DS_CTAS_PER_SM
 #define DS_CTAS_PER_SM 4
-#endif
     const int grid = (int)(tiles < 148 * DS_CTAS_PER_SM ? tiles : 148 * DS_CTAS_PER_SM);
     ta_launch(k_discover_staged, grid, DS_THREADS, sizeof(DiscoverSmem), h->stream, a);
     h->tkeep = -1;  // read back with the other results of the pass

@@ -146,17 +146,6 @@ __device__ __forceinline__ void load8_i64(const int64_t *col, int64_t p0, int64_
     for (int j = 0; j < 8; j++) v[j] = p0 + j < n ? col[p0 + j] : 0;
   }
 }
-__device__ __forceinline__ void store8_i64(int64_t *col, int64_t p0, int64_t n, const i64 *v) {
-  if (p0 + 8 <= n) {
-    longlong2 *ps = reinterpret_cast<longlong2 *>(col + p0);
-#pragma unroll
-    for (int j = 0; j < 4; j++) ps[j] = make_longlong2(v[2 * j], v[2 * j + 1]);
-  } else {
-#pragma unroll
-    for (int j = 0; j < 8; j++)
-      if (p0 + j < n) col[p0 + j] = v[j];
-  }
-}
 __device__ __forceinline__ void store8_i32(int32_t *col, int64_t p0, int64_t n, const int32_t *v) {
   if (p0 + 8 <= n) {
     int4 *ps = reinterpret_cast<int4 *>(col + p0);
@@ -187,50 +176,6 @@ __device__ __forceinline__ void loadn_i16(const int16_t *col, int64_t p0, int64_
     for (int j = 0; j < IT; j++) v[j] = p0 + j < n ? col[p0 + j] : fill;
   }
 }
-template <int IT>
-__device__ __forceinline__ void loadn_i64(const int64_t *col, int64_t p0, int64_t n, i64 *v) {
-  if (IT <= 2) {
-    for (int j = 0; j < IT; j++) v[j] = p0 + j < n ? col[p0 + j] : 0;
-    return;
-  }
-  if (p0 + IT <= n) {
-    const longlong2 *ps = reinterpret_cast<const longlong2 *>(col + p0);
-#pragma unroll
-    for (int j = 0; j < IT / 2; j++) {
-      const longlong2 x = ps[j];
-      v[2 * j] = x.x;
-      v[2 * j + 1] = x.y;
-    }
-  } else {
-#pragma unroll
-    for (int j = 0; j < IT; j++) v[j] = p0 + j < n ? col[p0 + j] : 0;
-  }
-}
-template <int IT>
-__device__ __forceinline__ void storen_i64(int64_t *col, int64_t p0, int64_t n, const i64 *v) {
-  if (p0 + IT <= n) {
-    longlong2 *ps = reinterpret_cast<longlong2 *>(col + p0);
-#pragma unroll
-    for (int j = 0; j < IT / 2; j++) ps[j] = make_longlong2(v[2 * j], v[2 * j + 1]);
-  } else {
-#pragma unroll
-    for (int j = 0; j < IT; j++)
-      if (p0 + j < n) col[p0 + j] = v[j];
-  }
-}
-template <int IT>
-__device__ __forceinline__ void storen_i32(int32_t *col, int64_t p0, int64_t n, const int32_t *v) {
-  if (p0 + IT <= n) {
-    int4 *ps = reinterpret_cast<int4 *>(col + p0);
-#pragma unroll
-    for (int j = 0; j < IT / 4; j++) ps[j] = make_int4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
-  } else {
-#pragma unroll
-    for (int j = 0; j < IT; j++)
-      if (p0 + j < n) col[p0 + j] = v[j];
-  }
-}
-
 // Ordered compaction of the sorted positions whose kind is in `kind_mask`: 256 threads x 32
 // positions per tile, vector loads of the kind column, one tile scan.
 #define CK_THREADS 256

@@ -17,17 +17,11 @@
 
 #define RS_BINS 256
 // descriptors of earlier tiles fetched together in the look back (1 = one at a time)
-#ifndef RS_LOOKBACK_BATCH
 #define RS_LOOKBACK_BATCH 4
-#endif
 
 // resident CTAs per SM the register allocation is sized for (pairs, keys only)
-#ifndef RSP_MINB
 #define RSP_MINB 2
-#endif
-#ifndef RSK_MINB
 #define RSK_MINB 4
-#endif
 
 struct RadixArgs {
   const u64 *keys_in;
@@ -177,7 +171,6 @@ __device__ __forceinline__ void radix_tile(const RadixArgs &a, RadixSmem<THREADS
           : "r"(dv), "r"(1u << b));
     }
     if (!FULL && !valid) m = 0;
-#ifndef RS_RANK_READBACK
     // The lowest peer adds the group size to the warp's digit counter and hands the counter's
     // old value to its peers by a shuffle; a peer's rank is that value plus the number of peers
     // below it.  No read-back of the counter and no warp barrier: the rows of a thread are
@@ -189,18 +182,6 @@ __device__ __forceinline__ void radix_tile(const RadixArgs &a, RadixSmem<THREADS
     old = __shfl_sync(0xffffffffu, old, leader < 0 ? lane : leader);
     rd[j] = (int)(((old + (u32)__popc(m & lt)) << 8) | d);
   }
-#else
-    // one population count per key: the number of peers at or above the lane.  The lowest
-    // peer adds the group size to the warp's digit counter; every peer then reads the counter
-    // back and steps down from its new value.
-    const u32 above1 = (u32)__popc(m >> lane);
-    if (valid && (m & lt) == 0) atomicAdd(&wh[d], above1);
-    __syncwarp();
-    const u32 after = valid ? wh[d] : 0u;
-    rd[j] = (int)(((after - above1) << 8) | d);
-    __syncwarp();
-  }
-#endif
   __syncthreads();
   // per digit: the CTA's count, exclusive starts of the digits, and per warp the tile-local
   // start of its run (so the scatter needs one shared load per key)
@@ -366,20 +347,14 @@ __global__ void __launch_bounds__(THREADS, VALS ? RSP_MINB : RSK_MINB) k_radix_p
 // tile shapes
 #define RSP_THREADS 384  // pairs
 #define RSP_ITEMS 12
-#ifndef RSK_THREADS
 #define RSK_THREADS 256  // keys only
-#endif
-#ifndef RSK_ITEMS
 #define RSK_ITEMS 16
-#endif
 // Up to RS_SMALL keys a pass waits for its one round of CTAs, not for the chip: half the keys per thread
 // (60 k records 384 -> 377 us for the whole analysis, 500 k 587 -> 575, 1.2 M 818 -> 810; a quarter
 // of them makes the look back longer than it saves).
 #define RSK_ITEMS_SMALL 8
 #define RSP_ITEMS_SMALL 6  // pairs (100 k expert records, 8 k collectives: 628 -> 596 us)
-#ifndef RS_SMALL
 #define RS_SMALL (2ll << 20)
-#endif
 
 // digit histograms of every pass (used when the caller has none)
 __global__ void __launch_bounds__(256) k_radix_hist(const u64 *keys, int64_t n, SortPlan plan,

@@ -158,7 +158,6 @@ struct ta_window {
 
   // sort products
   ta_sort_result sorted;
-  int32_t *d_lane_code;      // per lane: window << tbits | triple rank
   int32_t *d_lane_slot;      // per lane: window * n_pids + pid rank
   int32_t *d_lane_dom_end;   // per lane: first position behind the run of lanes of the same domain
   int32_t *d_lane_dev_base;  // per device lane: number of device records in earlier lanes

@@ -176,9 +176,7 @@ __device__ __forceinline__ u32 gather_index(u64 k, const GatherArgs &a) {
 // equal coarse keys are counted by bit operations on one vote (loops over neighbouring keys, with a
 // fifth of the records in runs, made every warp diverge: 410 instructions per warp), and no warp
 // waits for the others at the end.
-#ifndef GT_MINB
 #define GT_MINB 8
-#endif
 template <bool PACKED, bool ONE>
 __global__ void __launch_bounds__(256, GT_MINB) k_gather(GatherArgs a) {
   TA_PDL();
@@ -358,7 +356,7 @@ __device__ __forceinline__ void lane_table(const int32_t *lane_start, int64_t n_
                                                      int64_t n_valid, int32_t *lane_window,
                                                      int32_t *lane_pid, int16_t *lane_stream,
                                                      int16_t *lane_domain, int32_t *lane_off,
-                                                     int32_t *lane_code, int32_t *lane_slot,
+                                                     int32_t *lane_slot,
                                                      int32_t *lane_dom_end, int32_t *lane_dom_next,
                                                      int32_t *lane_dev_base, int32_t *n_lanes_out,
                                                      int64_t cap, const int32_t *status, u64 *tmp) {
@@ -384,7 +382,6 @@ __device__ __forceinline__ void lane_table(const int32_t *lane_start, int64_t n_
         lane_stream[l] = code_stream(code);
         lane_domain[l] = code_domain(code);
         lane_off[l] = st;
-        lane_code[l] = (int32_t)c;
         lane_slot[l] = w * n_pids + tt->pid_rank[t];
       }
     }
@@ -447,14 +444,14 @@ __global__ void __launch_bounds__(1024) k_lane_table(const int32_t *lane_start, 
                                                      int64_t n_valid, int32_t *lane_window,
                                                      int32_t *lane_pid, int16_t *lane_stream,
                                                      int16_t *lane_domain, int32_t *lane_off,
-                                                     int32_t *lane_code, int32_t *lane_slot,
+                                                     int32_t *lane_slot,
                                                      int32_t *lane_dom_end, int32_t *lane_dom_next,
                                                      int32_t *lane_dev_base, int32_t *n_lanes_out,
                                                      int64_t cap, const int32_t *status,
                                                      SlotRanges ranges, Tail tail) {
   TA_PDL();
   __shared__ u64 tmp[33];
-  lane_table(lane_start, n_codes, tbits, n_pids, tt, n_valid, lane_window, lane_pid, lane_stream, lane_domain, lane_off, lane_code, lane_slot, lane_dom_end, lane_dom_next, lane_dev_base, n_lanes_out, cap, status, tmp);
+  lane_table(lane_start, n_codes, tbits, n_pids, tt, n_valid, lane_window, lane_pid, lane_stream, lane_domain, lane_off, lane_slot, lane_dom_end, lane_dom_next, lane_dev_base, n_lanes_out, cap, status, tmp);
   if (!ta_failed(status)) slot_ranges(ranges, tmp);
   run_tail(tail);
 }
@@ -468,7 +465,7 @@ struct LaneRows {
   int64_t n_valid;
   int32_t *lane_window, *lane_pid;
   int16_t *lane_stream, *lane_domain;
-  int32_t *lane_off, *lane_code, *lane_slot, *lane_dom_end, *lane_dom_next, *lane_dev_base, *n_lanes_out;
+  int32_t *lane_off, *lane_slot, *lane_dom_end, *lane_dom_next, *lane_dev_base, *n_lanes_out;
   const u64 *n_lanes;  // total of the first scan
   int64_t bound;       // lanes <= bound
 };
@@ -487,7 +484,6 @@ struct LaneCodeOut {
     t.lane_stream[l] = code_stream(code);
     t.lane_domain[l] = code_domain(code);
     t.lane_off[l] = t.lane_start[c] - 1;
-    t.lane_code[l] = (int32_t)c;
     t.lane_slot[l] = w * t.n_pids + t.tt->pid_rank[r];
   }
 };
@@ -559,7 +555,7 @@ ta_status ta_run_sort_timeline(ta_window *h) {
 
   // result buffers (kept until ta_free)
   size_t keep = Carver::pad(n * 4) + 3 * Carver::pad(n * 8) + 3 * Carver::pad(n * 4) +
-                2 * Carver::pad(n * 2) + 7 * Carver::pad(lane_cap * 4) + 2 * Carver::pad(lane_cap * 2) +
+                2 * Carver::pad(n * 2) + 6 * Carver::pad(lane_cap * 4) + 2 * Carver::pad(lane_cap * 2) +
                 Carver::pad((lane_cap + 1) * 4) + Carver::pad((size_t)n_slots * 24) + 512;
   void *kb = ta_dalloc(h, keep);
   if (!kb) return TA_ERR_OOM;
@@ -569,7 +565,7 @@ ta_status ta_run_sort_timeline(ta_window *h) {
   int32_t *c_pid = ck.take<int32_t>(n), *c_name = ck.take<int32_t>(n), *c_seq = ck.take<int32_t>(n);
   int16_t *c_stream = ck.take<int16_t>(n), *c_kind = ck.take<int16_t>(n);
   int32_t *lane_window = ck.take<int32_t>(lane_cap), *lane_pid = ck.take<int32_t>(lane_cap);
-  int32_t *lane_code = ck.take<int32_t>(lane_cap), *lane_slot = ck.take<int32_t>(lane_cap);
+  int32_t *lane_slot = ck.take<int32_t>(lane_cap);
   int16_t *lane_stream = ck.take<int16_t>(lane_cap), *lane_domain = ck.take<int16_t>(lane_cap);
   int32_t *lane_off = ck.take<int32_t>(lane_cap + 1);
   int32_t *lane_dom_end = ck.take<int32_t>(lane_cap);
@@ -708,11 +704,11 @@ ta_status ta_run_sort_timeline(ta_window *h) {
     if (n_codes <= LT_ONE_CTA || n == 0) {
       // (few codes: fewer warps to wait for at each of its barriers)
       ta_launch(k_lane_table, 1, n_codes <= 256 && n_slots <= 256 ? 256 : 1024, 0, st, lane_start, n_codes, h->tbits, h->n_pids > 0 ? h->n_pids : 1, h->d_triples,
-                h->n_valid, lane_window, lane_pid, lane_stream, lane_domain, lane_off, lane_code, lane_slot,
+                h->n_valid, lane_window, lane_pid, lane_stream, lane_domain, lane_off, lane_slot,
                 lane_dom_end, lane_dom_next, lane_dev_base, n_lanes_dev, lane_cap, h->d_status, ranges, ta_tail(h, 1));
     } else {
       LaneRows t{lane_start, h->tbits, h->n_pids > 0 ? h->n_pids : 1, h->d_triples, h->n_valid,
-                 lane_window, lane_pid, lane_stream, lane_domain, lane_off, lane_code, lane_slot,
+                 lane_window, lane_pid, lane_stream, lane_domain, lane_off, lane_slot,
                  lane_dom_end, lane_dom_next, lane_dev_base, n_lanes_dev, nullptr, lane_cap - 1};
       Carver cs(sort_tmp);  // the sort is done with its temporaries by the time the scans run
       ScanTemp s1, s2, s3;
@@ -750,7 +746,6 @@ ta_status ta_run_sort_timeline(ta_window *h) {
   r.pid = c_pid; r.name_id = c_name; r.seq = c_seq; r.stream = c_stream; r.kind = c_kind;
   r.lane_window = lane_window; r.lane_pid = lane_pid; r.lane_stream = lane_stream;
   r.lane_domain = lane_domain; r.lane_off = lane_off;
-  h->d_lane_code = lane_code;
   h->d_lane_slot = lane_slot;
   h->d_lane_dom_end = lane_dom_end;
   h->d_lane_dev_base = lane_dev_base;
