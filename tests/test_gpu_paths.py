@@ -300,3 +300,39 @@ def test_operators_at_the_first_instant_there_is(n):
         assert np.array_equal(s.numpy("perm"), o.get("perm"))
         for k in ("parent", "depth"):
             assert np.array_equal(a.numpy(k), o.get(k)), k
+
+
+@pytest.mark.parametrize("hashed", [False, True])
+def test_join_of_more_records_than_launches_are_counted_on_the_way(hashed):
+    """From 24 M records on, launches with a kernel are counted by a pass of their own, which also
+    tells whether some have several (graph replays): both ways to address the table."""
+    import torch
+    from oracle.ta_oracle import Oracle
+    from paper_2609_40247_b200 import ta
+    from runners import ATTR_KEYS, JOIN_KEYS, ROLLUP_KEYS, assert_same
+    wl = synth.make_workload("c3", 0.39, truth=False)
+    ev = wl.events
+    assert len(ev) > 24 << 20
+    kernels = np.nonzero(ev["kind"] == 3)[0]
+    again = kernels[5::97]  # the kernel of the record two kernels before in the list gets a second one
+    same = ev["pid"][again] == ev["pid"][kernels[3::97][:len(again)]]
+    ev["corr_id"][again[same]] = ev["corr_id"][kernels[3::97][:len(again)][same]]
+    if hashed:
+        joins = ev["kind"] != 5
+        with np.errstate(over="ignore"):
+            ev["corr_id"][joins] *= np.int64(-7046029254386353131)
+    o = Oracle(ev, wl.win_off, wl.win_t0, wl.win_t1)
+    o.load()
+    o.sort()
+    o.correlate()
+    assert o.attribute() == 0
+    o.rollup()
+    want = {k: o.get(k) for k in JOIN_KEYS + ATTR_KEYS + ROLLUP_KEYS}
+    assert int(want["kernels_of_launch"].max()) > 1 and int(want["join_sum"]["n_orphan_launch"].sum()) > 0
+    buf = torch.from_numpy(np.ascontiguousarray(ev).view(np.uint8).reshape(-1)).cuda()
+    with ta.Window(buf, wl.win_off, wl.win_t0, wl.win_t1) as w:
+        w.sort_timeline()
+        j, a = w.correlate_launches(), w.attribute_operators()
+        r = w.rollup_operators()
+        got = {k: res.numpy(k) for res, names in ((j, JOIN_KEYS), (a, ATTR_KEYS), (r, ROLLUP_KEYS)) for k in names}
+    assert_same(want, got)
