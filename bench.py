@@ -208,11 +208,12 @@ def lsd_model_bytes_per_event(wl):
 
 
 def built_path_bytes_per_event(wl, radix_bytes_per_event):
-    """Algorithmic bytes per record of the path AS BUILT, kernel by kernel (reads + writes of
-    every column or table a kernel touches, fills and read-modify-write atomics included;
-    lookups that stay in cache across a tile are counted once per record).  The radix passes
-    enter with the bytes the library reports for them (16 B per record and pass for packed
-    keys).  f_x = share of the records of kind x."""
+    """Algorithmic bytes per record of the path as it was before kernels were added up from the
+    launch side, kernel by kernel (fills of the operators' columns, three atomics per kernel, a
+    pass of its own for the launch statistics): what earlier lines of this benchmark divided by,
+    reported beside touched_bytes_per_event so that they can be compared.  The radix passes enter
+    with the bytes the library reports for them (16 B per record and pass for packed keys).
+    f_x = share of the records of kind x."""
     ev = wl.events
     n = max(len(ev), 1)
     kinds = np.bincount(np.clip(ev["kind"].astype(np.int64), 0, 6), minlength=7)[:6] / n
@@ -232,6 +233,36 @@ def built_path_bytes_per_event(wl, radix_bytes_per_event):
         "gaps": 2.0 + f_d * 16.0 + 8.0,
         "aggregate": (2.0 + f_d * 20.0) + (2.0 + f_o * 24.0),
         "collectives": 8.0 + 2.0 + f_c * 100.0,       # wait fill, kind, compaction + pair sort + groups
+    }
+    return sum(parts.values()), parts
+
+
+def touched_bytes_per_event(wl, radix_bytes_per_event):
+    """Algorithmic bytes per record of the path AS BUILT, kernel by kernel: reads and writes of
+    every column or table a kernel touches, clearings and read-modify-write atomics included.
+    Lookups that stay in cache across a tile count once per record, rows that are written again
+    while they are in cache once.  The radix passes enter with the bytes the library reports for
+    them (16 B per record and pass for packed keys).  f_x = share of the records of kind x."""
+    ev = wl.events
+    n = max(len(ev), 1)
+    kinds = np.bincount(np.clip(ev["kind"].astype(np.int64), 0, 6), minlength=7)[:6] / n
+    f_o, f_api, f_l, f_k, f_m, f_c = (float(x) for x in kinds)
+    f_K, f_h, f_d = f_k + f_m, f_o + f_api + f_l, f_k + f_m + f_c
+    counted_apart = 4.0 if n >= 24 << 20 else 0.0     # launches with kernels, by a pass of their own
+    parts = {
+        "discover": 40.0 + 8.0,                       # records in, one word per record out
+        "radix passes": radix_bytes_per_event,        # keys in, keys out, per pass
+        "gather": 8.0 + 40.0 + 44.0,                  # key, record (random), 8 columns + perm
+        "join": 4.0 + f_l * 4.0                       # kernel counts and table cleared
+                + f_h * 10.0 + f_l * 4.0              # build: kind, corr of host records; table entry
+                + f_d * 18.0 + f_K * 20.0 + 20.0      # probe: kind, corr, ts; entry, launch ts/te; 3 outputs
+                + f_K * 8.0 + f_h * counted_apart,    # count and kernel at the launch
+        "attribute": f_h * 2.0 + f_o * 8.0            # tile stacks: kinds, ends of operators
+                     + f_h * 26.0 + f_K * 16.0 + 33.0  # resolve: kind, ts pair, count, kernel; its ts pair; 6 outputs
+                     + f_d * 6.0 + f_K * 4.0 + 4.0,   # inherit: kind, launch_of; parent; op_of
+        "gaps": f_d * 16.0 + 8.0,
+        "aggregate": f_d * 22.0 + f_h * 6.0 + f_o * 20.0,
+        "collectives": 8.0 + 2.0 + f_c * 100.0,       # waits cleared, kind, compaction + pair sort + groups
     }
     return sum(parts.values()), parts
 
@@ -495,15 +526,18 @@ def main():
         lsd_bytes, key_bits, passes, parts = lsd_model_bytes_per_event(wl)
         per_gpu = value / world
         radix_per_event = (radix_bytes / radix_steps / n) if (n_pass > 0 and n > 0) else 0.0
-        built_bytes, built_parts = built_path_bytes_per_event(wl, radix_per_event)
+        built_bytes, built_parts = touched_bytes_per_event(wl, radix_per_event)
+        before_bytes, _ = built_path_bytes_per_event(wl, radix_per_event)
         line["hbm_model"] = {
-            # headline: the bytes the path as built touches (kernel by kernel, built_path_bytes_per_event)
+            # headline: the bytes the path as built touches (kernel by kernel, touched_bytes_per_event)
             "built_bytes_per_event": round(built_bytes, 2),
             "built_parts": {k: round(v, 2) for k, v in built_parts.items()},
             "radix_passes_per_step": (n_pass / radix_steps) if n_pass else 0,
             "frac_of_measured_peak": per_gpu * built_bytes / (peak * 1e9),
             "frac_of_nominal_8TBs": per_gpu * built_bytes / 8.0e12,
             "target_ms_for_half_of_measured_peak": 2e3 * n * built_bytes / (peak * 1e9),
+            # what lines of builds whose attribution went by the device side were divided by
+            "frac_of_measured_peak_device_side_attribution_model": per_gpu * before_bytes / (peak * 1e9),
             # secondary: the byte model of an LSD sort of (key, index) pairs, one pass per key
             # byte - a different algorithm's bytes - and the compulsory bytes alone
             "lsd_bytes_per_event": round(lsd_bytes, 2), "lsd_key_bits": key_bits, "lsd_passes": passes,

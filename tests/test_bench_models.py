@@ -40,3 +40,23 @@ def test_built_path_model_adds_its_parts_and_takes_the_radix_bytes_as_given():
     # every other part depends on the kind mix only
     assert all(parts[k] == parts2[k] for k in parts if k != "radix passes")
     assert 380.0 < total < 410.0
+
+
+def test_touched_bytes_model_on_the_c3_mix():
+    """The path as built, by hand: 36 + 28 bytes per host and device record where columns are read,
+    69 of outputs and counters, per launch, kernel and operator what its table entry costs."""
+    wl = synth.make_workload("c3", 0.01, truth=False)
+    total, parts = bench.touched_bytes_per_event(wl, 64.0)
+    assert abs(total - sum(parts.values())) < 1e-9
+    assert parts["radix passes"] == 64.0 and parts["discover"] == 48.0 and parts["gather"] == 92.0
+    m = _mix(wl.events)
+    f_h = m["op"] + m["api"] + m["launch"]
+    f_K = m["kernel"] + m["memcpy"]
+    f_d = f_K + m["coll"]
+    assert abs(f_h + f_d - 1.0) < 1e-9
+    want = (48 + 64 + 92 + (4 + 20 + 10 * f_h + 18 * f_d + 8 * m["launch"] + 28 * f_K)
+            + (37 + 28 * f_h + 8 * m["op"] + 6 * f_d + 20 * f_K) + (8 + 16 * f_d)
+            + (22 * f_d + 6 * f_h + 20 * m["op"]) + (10 + 100 * m["coll"]))
+    assert abs(total - want) < 1e-9
+    before, _ = bench.built_path_bytes_per_event(wl, 64.0)
+    assert 350.0 < total < before
