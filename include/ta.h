@@ -19,7 +19,10 @@
  *     ordinary host memory.  Result structs are filled with device pointers
  *     OWNED BY THE HANDLE (valid until ta_free) and host scalars.  Host-side
  *     per-window summary arrays are CALLER-OWNED, W entries, and are filled
- *     after one stream synchronisation at the end of the call.
+ *     when the call returns: it waits for its work on the stream, by polling a
+ *     word in page-locked memory that its last kernel writes, or by a stream
+ *     synchronisation (large results, and where the device's schedule flags ask
+ *     for blocking or yielding waits).
  *   - Every kernel is enqueued on env.cuda_stream.  Every call that takes a
  *     handle (and ta_load_window) makes env.device the current device of the
  *     calling thread and leaves it current when it returns.
@@ -383,7 +386,7 @@ ta_status ta_match_collectives(ta_window *h, const ta_comm_size *sizes,
  * All arrays are device memory owned by the handle, n_rows entries each.
  * Limits: as ta_load_window, and windows x pids < 2^22 (TA_ERR_TOO_LARGE).
  * Errors: TA_ERR_ORDER before ta_sort_timeline; TA_ERR_OOM; TA_ERR_CUDA;
- * TA_ERR_TIMEOUT.  One stream synchronisation at the end. */
+ * TA_ERR_TIMEOUT.  One wait, at the end. */
 typedef struct ta_overlap_result {
   int64_t n_rows;
   const int32_t *d_window, *d_pid;
@@ -415,7 +418,7 @@ ta_status ta_device_overlap(ta_window *h, ta_overlap_result *out);
  * and device peaks that a 40-byte record does not carry: see ta_operator_sol.
  * All arrays are device memory owned by the handle, n entries each.
  * Errors: TA_ERR_ORDER unless ta_attribute_operators returned TA_OK;
- * TA_ERR_OOM; TA_ERR_CUDA.  One stream synchronisation at the end. */
+ * TA_ERR_OOM; TA_ERR_CUDA.  One wait, at the end. */
 typedef struct ta_rollup_summary {
   int64_t n_graph_launches, n_graph_kernels, max_kernels_per_launch;
 } ta_rollup_summary;
@@ -460,7 +463,7 @@ ta_status ta_rollup_operators(ta_window *h, ta_rollup_result *out,
  * worst case of adding 10^7 positive doubles in another order).
  * All arrays are device memory owned by the handle, n entries each.
  * Errors: TA_ERR_ORDER unless ta_attribute_operators returned TA_OK;
- * TA_ERR_INVALID_ARG; TA_ERR_OOM; TA_ERR_CUDA.  One stream synchronisation. */
+ * TA_ERR_INVALID_ARG; TA_ERR_OOM; TA_ERR_CUDA.  One wait. */
 typedef struct ta_sol_summary {
   int64_t n_resolved, n_no_kernels, n_no_counts, sum_top_ns;
   double sum_flops, sum_bytes, max_sol;
@@ -504,7 +507,7 @@ ta_status ta_operator_sol(ta_window *h, const double *flops, const double *bytes
  * ta_aggregate_ops(h, 1 << TA_KIND_OP, 2, ...): operators with op_gap_ns > 0.
  * All arrays are device memory owned by the handle.
  * Errors: TA_ERR_ORDER before ta_correlate_launches; TA_ERR_INVALID_ARG;
- * TA_ERR_OOM; TA_ERR_CUDA; TA_ERR_TIMEOUT.  One stream synchronisation. */
+ * TA_ERR_OOM; TA_ERR_CUDA; TA_ERR_TIMEOUT.  One wait. */
 enum { TA_BLAME_NO_LAUNCH = 0, TA_BLAME_SUBMISSION = 1, TA_BLAME_QUEUED = 2, TA_BLAME_TAIL = 3 };
 
 typedef struct ta_blame_summary {
@@ -572,9 +575,9 @@ void ta_free(ta_window *h);
  * Limits: window span and the longest record < 2^40 ns each, windows x pids <
  * 2^22 (TA_ERR_TOO_LARGE).
  * Errors: TA_ERR_ORDER before ta_correlate_launches; TA_ERR_OOM; TA_ERR_CUDA;
- * TA_ERR_TIMEOUT.  Two stream synchronisations (three when some stream lane
- * does not end its records in ascending order and the device records have to
- * be sorted by end time). */
+ * TA_ERR_TIMEOUT.  One wait while windows x pids <= 1024, every stream lane ends
+ * its records in ascending order and at most 8192 waits of the host are on the
+ * paths' way; else two, or three (the device records are sorted by end time then). */
 enum {
   TA_CP_KERNEL = 0, TA_CP_MEMCPY = 1, TA_CP_COLL = 2, TA_CP_LAUNCH_LATENCY = 3,
   TA_CP_STREAM_DELAY = 4, TA_CP_IN_CALL = 5, TA_CP_BETWEEN_CALLS = 6, TA_CP_WAIT_TAIL = 7
@@ -647,12 +650,12 @@ ta_status ta_lane_gaps_noalloc_host(const int64_t *ts_start, const int64_t *ts_e
  * Helpers around the results and their memory.
  *
  * ta_fetch: copies `count` device regions of the handle's results to host memory
- * (dst[i] <- src[i], bytes[i]) with one synchronisation of env.cuda_stream.
- * Regions of up to 128 KB are gathered by one kernel.
+ * (dst[i] <- src[i], bytes[i]) with one wait for env.cuda_stream.  Regions of up to
+ * 128 KB are gathered by one kernel.
  * ta_block_of: the allocation a result pointer of this handle lies in.
  * ta_chunk_*: an allocator for ta_env that hands out pieces of one block of device
  * memory the caller has obtained, for callers whose own allocator is expensive
- * to call (an analysis makes some thirty requests); a request that does not
+ * to call (an analysis makes some twenty requests); a request that does not
  * fit goes to the caller's alloc / release.  Use it as
  *   env.alloc = ta_chunk_alloc; env.release = ta_chunk_release; env.ctx = ta_chunk_open(...);
  * one chunk per handle, closed after ta_free; the block itself stays the caller's.

@@ -839,7 +839,9 @@ ta_status ta_run_attribute(ta_window *h, ta_attr_summary *out_summary) {
   // stacks in front of its tiles itself (60 k records 400 us with 256, 387 with 128), 256 up to some
   // three million (1.2 M: 833 with 512, 822), 1024 from ten rounds of the 148 * 32 warps
   // k_attr_resolve keeps on the chip (66.8 M: 782 us of the kernel with 512, 750, and half the stacks); 512
-  // between, where the last round's slowest warps show (16.8 M: 342 us of the kernel with 1024, 263).
+  // between, where the last round's slowest warps show (16.8 M: 342 us of the kernel with 1024, 263; from
+  // some 24 M on the call is 2 % faster with 1024: 28 M experts 579 and 571 us, prefill 698 and 669, 60 M
+  // 1108 and 1074).
   const int per_tile = n <= 128ll * AT_FAN * AT_FAN ? 128 : n <= (3 << 20) ? 256 : n <= 10ll * 148 * 32 * 1024 ? 512 : 1024;
   const int64_t tiles = (n + per_tile - 1) / per_tile;
   size_t keep = 3 * Carver::pad(nn * 4) + Carver::pad(nn) + 3 * Carver::pad(nn * 8) + 256;

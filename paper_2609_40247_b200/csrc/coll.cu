@@ -310,7 +310,7 @@ ta_status ta_run_collectives(ta_window *h, const ta_comm_size *sizes, int32_t n_
   TA_TRY((launch_scan<OpAdd, CollHeadIn, CollHeadOut>(h, m, hin, hout, OpAdd(), s2)));
   // The group tables are sized by the number of groups when that is worth a round trip; while
   // the bound "one group per COLL record" keeps them under 1 GiB they are sized by the bound
-  // and the count comes back with the call's one synchronisation.
+  // and the count comes back with the call's one wait.
   u64 ng64 = 0;
   const bool bounded = (u64)m * 60 <= (1ull << 30);
   if (!bounded) {

@@ -579,7 +579,7 @@ ta_status ta_run_gaps(ta_window *h, int64_t min_gap, ta_gap_result *out) {
     ta_launch(k_gap_list_order, (unsigned)((m + 255) / 256), 256, 0, st, ulist, ukeys, bits, rank, m, list, h->d_status);
     TA_CHECK_CUDA(h, cudaGetLastError());
     // both kernels are still queued: their temporaries go back after the handle's next
-    // synchronisation (the list itself is used in stream order like every other result)
+    // wait (the list itself is used in stream order like every other result)
     ta_dfree_later(h, tb);
     ta_dfree_later(h, lt);
     tb = lt = nullptr;

@@ -496,8 +496,10 @@ ta_status ta_run_correlate(ta_window *h, ta_join_summary *out_summary) {
   a.launch_of = launch_of; a.kol = kol; a.kernel_of = h->d_kernel_of; a.multi = (u32 *)&h->d_status[ST_MULTI]; a.latency = latency; a.qdelay = qdelay; a.sum = d_sum;
   a.status = h->d_status;
   // Rows per warp: 12, fewer where that would be less than a round of the 148 * 24 warps on the chip
-  // (1.2 M records: 101 us with 12, 90 with 8), 24 where it leaves twenty rounds and more (66.8 M: 730 us
-  // with 12, 690 with 24; 16.8 M: 182 with 12, 233 with 32, whose last warps run long).
+  // (1.2 M records: 101 us with 12, 90 with 8), 24 where it leaves twenty rounds and more.  The call with 12
+  // and with 24 rows: experts, 20 M records 315 and 345 us, 36 M 512 and 545, 52 M 761 and 811, 60 M 922 and
+  // 914, 66.8 M 40 less; prefill 20 M 366 and 330, 52 M 1163 and 984, 60 M 1359 and 1197.  The line lies where
+  // neither loses.
   int64_t rows = n / 32 / (148 * 32);
   rows = rows < JP_ROWS ? JP_ROWS : rows > 12 ? 12 : rows / JP_ROWS * JP_ROWS;
   if (n > (int64_t)20 * 148 * 24 * 24 * 32) rows = 24;

@@ -5,7 +5,7 @@
 // array instead of memory obtained from an allocator.  A call is one clearing of 128
 // bytes, one kernel, and a host that watches the page-locked row the kernel's last
 // tile writes (a second kernel where a lane's records do not end in ascending order).
-// Bound by latency: 64 k records take 28 us through the Python binding, of which
+// Bound by latency: 64 k records take 30 us through the Python binding, of which
 // the kernel is 5 (two clearings, a scan, two copies back and a synchronisation: 62).
 #include "ta_internal.cuh"
 

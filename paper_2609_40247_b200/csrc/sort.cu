@@ -55,7 +55,7 @@ __device__ __forceinline__ u64 prekey_to_key(const PrekeyInfo &k, u64 w64, int w
   return (hi << k.ibits) | (u64)(i - k.off[w]);
 }
 
-// Tile descriptors of the pair passes (the small sorts: long-gap list, collective keys) carry the
+// Tile descriptors of the pair passes (the small sorts: collective keys, the dropped tail, symbols) carry the
 // pass they belong to, so that one clearing of the descriptor array serves every pass of a sort:
 // [status, 2 bits][pass tag, 6 bits][count, 56 bits]; a descriptor whose tag is not the running
 // pass's is as good as empty.  The keys-only passes (the timeline sort: 16 k tiles) keep plain
@@ -411,7 +411,9 @@ static size_t min_tile(int64_t n) {
 }
 
 // Descriptors of all passes are cleared at once while that is little memory (keys-only passes: 1 KB
-// per tile and pass); for more records each keys-only pass has the one array cleared in front of it.
+// per tile and pass); for more records each keys-only pass has the one array cleared in front of it (the
+// launches it saves are worth some 10 us at any size - 20 M records 874 us with a clearing per pass, 863
+// without, 60 M 2531 and 2520 - and the memory grows: 29 MB at the line, 117 at 66.8 M).
 #define RS_AT_ONCE (1ll << 24)
 static size_t state_bytes(int64_t n) {
   const int64_t tile = (int64_t)min_tile(n);

@@ -127,7 +127,7 @@ struct ta_window {
   std::vector<size_t> alloc_bytes;  // their sizes, same order
   char *zero_pool;   // cleared when the window was loaded, handed out by ta_zalloc
   size_t zero_bytes, zero_used;
-  std::vector<void *> deferred;  // temporaries to release after the next synchronisation
+  std::vector<void *> deferred;  // temporaries to release after the next wait
 
   ResultStage out;  // results of the call in progress on their way to the host
 
@@ -287,7 +287,7 @@ ta_status ta_run_critpath(ta_window *h, ta_critpath_result *out, ta_critpath_sum
 // ta_read_status / ta_sync_fetch, and holds what *dev_src holds once all kernels launched before
 // that have run, whatever was launched before or after this.
 ta_status ta_queue_d2h(ta_window *h, void *dst, const void *dev_src, size_t bytes);
-// One stream synchronisation: delivers the queued copies and releases deferred temporaries.
+// One wait for all that is queued: delivers the noted copies and releases deferred temporaries.
 ta_status ta_sync_fetch(ta_window *h);
 // The same, with the device status words.
 ta_status ta_read_status(ta_window *h, int32_t *host_words /*ST_WORDS*/);
@@ -306,7 +306,7 @@ struct Tail {
   volatile u32 *seq_word;
 };
 Tail ta_tail(ta_window *h, int64_t grid);
-// Releases a temporary that queued work may still use: after the next synchronisation.
+// Releases a temporary that queued work may still use: after the next wait.
 void ta_dfree_later(ta_window *h, void *p);
 
 

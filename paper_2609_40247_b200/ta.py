@@ -302,9 +302,11 @@ def _place(device, stream_ptr):
     return at
 
 
-# An analysis makes some thirty requests for memory, each a call from C into Python.  Windows of up
+# An analysis makes some twenty requests for memory, each a call from C into Python.  Windows of up
 # to CHUNK_RECORDS records take one block up front, sized for the results and temporaries of the
 # seven calls, and the library hands out pieces of it; what does not fit is requested as before.
+# Above that the block saves 0.5 % (28 M records 2607 and 2585 us) and is more than 3 GB, of which
+# a caller who only sorts uses half.
 CHUNK_RECORDS = 1 << 24
 CHUNK_BYTES_PER_RECORD = 176
 CHUNK_BYTES_FIXED = 4 << 20
@@ -422,7 +424,10 @@ class _Result:
 
     def tensor(self, name):
         """Zero-copy torch view (uint8 for struct arrays) of a device result; valid while
-        the window is open."""
+        the window is open.  In a window of up to CHUNK_RECORDS records on torch's memory it is a
+        part of one block taken for all results (176 bytes per record and 4 MB), which goes
+        back to torch once the window is closed and none of its tensors is referenced any
+        more: copy what is to be kept for long."""
         field, _, size, count = self._table[name]
         nbytes = count(self) * size
         ptr = getattr(self._raw, field)
