@@ -415,7 +415,7 @@ class _Result:
         self._blocks = window._blocks
         self._raw = raw
         self._host = {}      # tables fetched with another one and not asked for yet
-        self._shown = set()  # fields the caller has a tensor of and may write to: read when asked for
+        self._shown = {}     # fields the caller has a tensor of and may write to: read when asked for
         self.__dict__.update(extra or {})
 
     def _spec(self, name):
@@ -433,8 +433,7 @@ class _Result:
         ptr = getattr(self._raw, field)
         if nbytes == 0 or not ptr:
             return self._blocks.empty()
-        self._shown.add(field)
-        self._host.pop(field, None)
+        self._shown[field] = True
         t = _part(self._blocks.last, ptr, nbytes) if _part else None
         return self._blocks.part(ptr, nbytes) if t is None else t
 
@@ -466,10 +465,7 @@ class _Result:
         st = self._handle.lib.ta_fetch(self._handle.ptr, m, dst, src, num)
         if st != 0:
             raise TaError(st, "ta_fetch")
-        for field, array in arrays[1:]:
-            self._host[field] = array
-            if field in self._shown:  # a tensor was handed out meanwhile, by another thread
-                self._host.pop(field, None)
+        self._host.update(arrays[1:])
         return arrays[0][1]
 
     def numpy(self, name):
@@ -480,7 +476,8 @@ class _Result:
         if count(self) == 0 or not getattr(self._raw, field):
             out = np.empty(0, dtype=dt)
         else:
-            out = self._host.pop(field, None) if self._handle.ptr else None  # (none of a closed window)
+            # (none of a closed window)
+            out = self._host.pop(field, None) if self._handle.ptr and field not in self._shown else None
             if out is None:
                 out = self._fetch(name)
         if field.endswith("_hist"):
@@ -714,8 +711,12 @@ class Window:
         size = CHUNK_BYTES_FIXED + self.n * CHUNK_BYTES_PER_RECORD
         try:
             # (without a stream of the caller's choice the window is on the device's current one)
-            with _plain(), contextlib.nullcontext() if stream is None else torch.cuda.stream(stream):
-                t = torch.empty(size, dtype=torch.uint8, device=torch.device("cuda", h.device))
+            device = torch.device("cuda", h.device)
+            if stream is None and not torch.is_inference_mode_enabled():
+                t = torch.empty(size, dtype=torch.uint8, device=device)
+            else:
+                with _plain(), contextlib.nullcontext() if stream is None else torch.cuda.stream(stream):
+                    t = torch.empty(size, dtype=torch.uint8, device=device)
         except RuntimeError:  # out of memory, or whatever else the allocator in use has to say
             return  # piece by piece, as far as it goes
         base = t.data_ptr()
