@@ -188,7 +188,9 @@ __device__ __forceinline__ void agg_flush(const AggArgs &a, AggSmem &s) {
     }
   }
   __syncthreads();
-  // histogram bins: one thread per (slot, bin)
+  // histogram bins: one thread per (slot, bin).  Not unrolled: fetching the longer code costs a window of
+  // 60 k records 1.5 us a call (24.5 and 23.7 us against 26.1 and 25.7), and saves 16.8 M two of 135
+#pragma unroll 1
   for (int i = threadIdx.x; i < AG_SLOTS * TA_NBINS; i += AG_THREADS) {
     const int sl = i / TA_NBINS, b = i - sl * TA_NBINS;
     const u32 c = s.hist[sl][b];
