@@ -655,7 +655,7 @@ ta_status ta_lane_gaps_noalloc_host(const int64_t *ts_start, const int64_t *ts_e
  * ta_block_of: the allocation a result pointer of this handle lies in.
  * ta_chunk_*: an allocator for ta_env that hands out pieces of one block of device
  * memory the caller has obtained, for callers whose own allocator is expensive
- * to call (an analysis makes some twenty requests); a request that does not
+ * to call (the seven calls make 13 to 19 requests); a request that does not
  * fit goes to the caller's alloc / release.  Use it as
  *   env.alloc = ta_chunk_alloc; env.release = ta_chunk_release; env.ctx = ta_chunk_open(...);
  * one chunk per handle, closed after ta_free; the block itself stays the caller's.

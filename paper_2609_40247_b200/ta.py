@@ -302,7 +302,7 @@ def _place(device, stream_ptr):
     return at
 
 
-# An analysis makes some twenty requests for memory, each a call from C into Python.  Windows of up
+# The seven calls make 13 to 19 requests for memory, each a call from C into Python.  Windows of up
 # to CHUNK_RECORDS records take one block up front, sized for the results and temporaries of the
 # seven calls, and the library hands out pieces of it; what does not fit is requested as before.
 # Above that the block saves 0.5 % (28 M records 2607 and 2585 us) and is more than 3 GB, of which
