@@ -439,18 +439,23 @@ __device__ __forceinline__ void run_tail(const Tail &t, Before before) {
   __shared__ int s_last;
   if (t.m == 0) return;
   __syncthreads();
-  if (threadIdx.x == 0) {
+  if (gridDim.x > 1) {  // (the block barrier does for a CTA alone)
+    if (threadIdx.x == 0) {
+      __threadfence();
+      s_last = atomicInc(t.ticket, gridDim.x - 1) == gridDim.x - 1;  // (wraps back to 0)
+    }
+    __syncthreads();
+    if (!s_last) return;
     __threadfence();
-    s_last = gridDim.x == 1 || atomicInc(t.ticket, gridDim.x - 1) == gridDim.x - 1;  // (wraps back to 0)
   }
-  __syncthreads();
-  if (!s_last) return;
-  __threadfence();
   before();
-  for (int e = 0; e < t.m; e++) {
-    const u32 *s = (const u32 *)t.src[e];
-    u32 *d = (u32 *)(t.pin_dev + t.off[e]);
-    for (unsigned i = threadIdx.x; i < t.bytes[e] / 4; i += blockDim.x) d[i] = __ldcg(s + i);
+  // the words of all regions side by side: one after the other each is a round trip to L2 more
+  for (unsigned i = threadIdx.x;; i += blockDim.x) {
+    unsigned k = i;
+    int e = 0;
+    while (e < t.m && k >= t.bytes[e] / 4) k -= t.bytes[e++] / 4;
+    if (e == t.m) break;
+    ((u32 *)(t.pin_dev + t.off[e]))[k] = __ldcg((const u32 *)t.src[e] + k);
   }
   __syncthreads();
   if (threadIdx.x == 0) {
