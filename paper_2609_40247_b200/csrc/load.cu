@@ -55,11 +55,24 @@ struct PlanWindows {
   int64_t v[3 * TA_PLAN_WINDOWS + 1];  // off, t0, t1 as they lie in memory
   int n;                               // 0: the bounds were copied
 };
+// What the handle has to find cleared is cleared by the other CTAs meanwhile (a fill in front of the
+// plan was one operation more in a row, and the plan waited for it to end).
+struct PlanClear {
+  uint4 *p;
+  int64_t n;  // of 16 bytes each
+};
 __global__ void __launch_bounds__(PL_THREADS) k_plan(const ta_event *ev, int64_t n, int64_t *off,
                                                      const int64_t *t0, const int64_t *t1, int W,
                                                      int sbits, int64_t max_span, int64_t max_win,
-                                                     int64_t *misc, PlanWindows pw) {
+                                                     int64_t *misc, PlanWindows pw, PlanClear clear) {
   TA_PDL();
+  if (blockIdx.x > 0) {
+    const int64_t step = (int64_t)(gridDim.x - 1) * PL_THREADS;
+#pragma unroll 4
+    for (int64_t i = (int64_t)(blockIdx.x - 1) * PL_THREADS + threadIdx.x; i < clear.n; i += step)
+      clear.p[i] = make_uint4(0, 0, 0, 0);
+    return;
+  }
   if (threadIdx.x < pw.n) off[threadIdx.x] = pw.v[threadIdx.x];
   if (threadIdx.x < 16) {  // [0] / [1] smallest / largest name, [3] / [4] sequence number, the rest 0
     const int k = threadIdx.x;
@@ -787,7 +800,7 @@ static int grid_for(int64_t n, int threads, int per_sm) {
   return (int)(g < 1 ? 1 : (g > cap ? cap : g));
 }
 
-ta_status ta_launch_discover(ta_window *h) {
+ta_status ta_launch_discover(ta_window *h, void *zero, size_t zero_bytes, int32_t spin) {
   h->tkeep = 0;
   h->fast_keys = 0;
   int64_t max_span = 1, max_win = 1;
@@ -804,8 +817,13 @@ ta_status ta_launch_discover(ta_window *h) {
     memcpy(pw.v + h->W + 1, h->h_t0.data(), (size_t)h->W * 8);
     memcpy(pw.v + 2 * h->W + 1, h->h_t1.data(), (size_t)h->W * 8);
   }
-  ta_launch(k_plan, 1, PL_THREADS, 0, h->stream, h->events, h->n, h->d_off, h->d_t0, h->d_t1, h->W, sbits, max_span,
-            max_win, h->d_misc, pw);
+  // (64 KB a CTA and more: 128 MB in a round of two CTAs per SM)
+  const PlanClear clear{(uint4 *)zero, (int64_t)(zero_bytes / 16)};
+  const int64_t parts = ((int64_t)zero_bytes + (64 << 10) - 1) / (64 << 10);
+  ta_launch(k_plan, 1 + (unsigned)(parts < 296 ? parts : 296), PL_THREADS, 0, h->stream, h->events, h->n, h->d_off,
+            h->d_t0, h->d_t1, h->W, sbits, max_span, max_win, h->d_misc, pw, clear);
+  if (spin > 0)
+    TA_CHECK_CUDA(h, cudaMemcpyAsync(h->d_status + ST_SPIN, &spin, sizeof(spin), cudaMemcpyHostToDevice, h->stream));
   if (h->n > 0) {
     // plan the time resolution (above), then the pass over the records, which also takes the histograms of
     // the time passes and counts the records per triple

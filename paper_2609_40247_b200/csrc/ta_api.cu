@@ -507,7 +507,7 @@ static ta_status load_impl(ta_window *h, const ta_event *events, int32_t on_devi
   const int W = h->W;
   cudaStream_t st = h->stream;
   // one device block: [off | t0 | t1 | misc], filled by the planning kernel (by a copy when there
-  // are many windows), and everything that starts at zero, cleared by one fill: [status | load
+  // are many windows), and everything that starts at zero, cleared by that kernel too: [status | load
   // summaries | digit histograms | triple table | communicator table | pool for the later calls]
   const size_t up_words = (size_t)(W + 1) + 2 * (size_t)W + 16;
   // the pool: kernel counts (4 bytes per record), the join's table (some 2), the sort's descriptors (1.3),
@@ -540,6 +540,7 @@ static ta_status load_impl(ta_window *h, const ta_event *events, int32_t on_devi
   h->d_comms = c.take<CommTable>(1);
   char *zero_end = (char *)h->d_comms + sizeof(h->d_comms->slots);
   static_assert(offsetof(CommTable, slots) == 0, "slots come first");
+  static_assert(offsetof(TripleTable, slots) % 16 == 0 && sizeof(h->d_comms->slots) % 16 == 0, "cleared in 16-byte words");
   h->d_keys = (u64 *)ta_dalloc(h, (size_t)(n > 0 ? n : 1) * 8);
   if (!h->d_keys) return TA_ERR_OOM;
 
@@ -559,10 +560,6 @@ static ta_status load_impl(ta_window *h, const ta_event *events, int32_t on_devi
     // a pageable source is staged by the runtime before the call returns
     TA_CHECK_CUDA(h, cudaMemcpyAsync(up, host.data(), host.size() * 8, cudaMemcpyHostToDevice, st));
   }
-  TA_CHECK_CUDA(h, cudaMemsetAsync(zero_begin, 0, zero_end - zero_begin, st));
-  const int32_t spin = g_ta_spin_limit.load();
-  if (spin > 0)
-    TA_CHECK_CUDA(h, cudaMemcpyAsync(h->d_status + ST_SPIN, &spin, sizeof(spin), cudaMemcpyHostToDevice, st));
 
   int32_t words[ST_WORDS];
   int64_t misc[16];
@@ -572,7 +569,7 @@ static ta_status load_impl(ta_window *h, const ta_event *events, int32_t on_devi
   TA_TRY(ta_queue_d2h(h, h->h_comm_sorted.data(), h->d_comms->sorted_id, TA_COMMS_AT_ONCE * sizeof(u64)));
   TA_TRY(ta_queue_d2h(h, words, h->d_status, sizeof(words)));
   TA_TRY(ta_queue_d2h(h, sums.data(), h->d_load_sum, W * sizeof(ta_load_summary)));
-  TA_TRY(ta_launch_discover(h));
+  TA_TRY(ta_launch_discover(h, zero_begin, (size_t)(zero_end - zero_begin), g_ta_spin_limit.load()));
   TA_TRY(ta_sync_fetch(h));
   if (words[ST_ERR]) return (ta_status)words[ST_ERR];
   h->n_triples = words[ST_N_TRIPLES];

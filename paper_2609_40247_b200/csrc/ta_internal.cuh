@@ -252,7 +252,8 @@ SortPlan ta_make_plan(int lo_bit, int hi_bit);
 ta_status ta_upload(ta_window *h, void *dst, const void *host_src, size_t bytes);  // host -> device on the handle's stream
 void ta_upload_age();  // a handle has gone away
 // load.cu
-ta_status ta_launch_discover(ta_window *h);
+// Clears `zero` (whole 16-byte words) on the way; spin: poll limit of the handle's waits, 0 = the default.
+ta_status ta_launch_discover(ta_window *h, void *zero, size_t zero_bytes, int32_t spin);
 ta_status ta_launch_rank_triples(ta_window *h);
 ta_status ta_launch_load(ta_window *h, bool allow_packed);
 // timeline.cu
