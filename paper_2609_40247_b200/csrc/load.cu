@@ -13,7 +13,7 @@
 //                   itself and no separate key pass is needed;
 //   k_top_hist_*    digit histograms of the passes over the (window, lane) bits of several windows,
 //                   from the records counted per window and triple, or from the words when there
-//                   are too many windows for that (of one window: see k_radix_scan_hist);
+//                   are too many windows for that (of one window: k_rank);
 //   k_rank_*        one CTA each: sort and rank the few triples / communicator ids;
 //   k_load_pre      turns those words into keys in place - [dropped][window][triple
 //                   rank][(ts_start - t0) >> dshift]{[index in window]} - and takes the
@@ -473,7 +473,7 @@ __global__ void __launch_bounds__(DS_THREADS, 4) k_discover_staged(DiscoverArgs 
 }
 
 // ---- histograms of the passes over the (dropped, window, triple rank) bits ------------------
-// (of a single window they follow from the records counted per triple: k_radix_scan_hist)
+// (of a single window they follow from the records counted per triple, in k_rank)
 struct TopHistArgs {
   SortPlan plan;        // the whole plan; passes [n_time, n_pass) are the top passes
   int n_time;
@@ -586,7 +586,7 @@ __device__ __forceinline__ void block_sort(u64 *buf, int n) {
 // of triples: the occupied slots are packed to the front in any order, as code << 13 | slot, so
 // that the sorted entry names its slot; the table is read once and only its occupied slots are
 // written (two passes over all slots in block-scan rounds and a serial pid walk took 20 us).
-__device__ __forceinline__ void rank_triples(TripleTable *tt, const u32 *slot_cnt, int32_t *status,
+__device__ __forceinline__ int rank_triples(TripleTable *tt, const u32 *slot_cnt, int32_t *status,
                                              u64 *buf /* TA_TRIPLE_SLOTS */) {
   __shared__ u64 tmp[33];
   __shared__ int n_tr;
@@ -625,6 +625,7 @@ __device__ __forceinline__ void rank_triples(TripleTable *tt, const u32 *slot_cn
     status[ST_N_TRIPLES] = n;
     status[ST_N_PIDS] = pids;
   }
+  return n;
 }
 
 // One CTA: sorts and ranks the communicator ids.
@@ -661,14 +662,78 @@ __device__ __forceinline__ void rank_comms(CommTable *cm, int32_t *status, u64 *
   }
 }
 
-// Both rankings in one launch: CTA 0 the triples, CTA 1 the communicator ids (they are
-// independent, and two single-CTA kernels one after the other cost a launch latency more).
+// Of one window: where the digits of every radix pass begin in its output, the exclusive scan of
+// the digit histograms, a warp per pass (a launch of its own in front of the first pass otherwise).  The passes over the
+// time bits are counted; those over the (dropped, triple rank) bits follow from the records per triple, and
+// dropped records have time digits 0.
+struct RankBins {
+  const u32 *hist;
+  const int64_t *misc;
+  const ta_load_summary *sum;  // null: several windows
+  u32 *bin_offset;
+};
+__device__ __forceinline__ void scan_bins(u32 (&v)[8], u32 *out) {
+  const int lane = threadIdx.x & 31;
+  u32 mine = 0;
+#pragma unroll
+  for (int k = 0; k < 8; k++) mine += v[k];
+  u32 ex = (u32)warp_scan_inclusive((u64)mine, OpAdd()) - mine;
+#pragma unroll
+  for (int k = 0; k < 8; k++) {
+    out[lane * 8 + k] = ex;
+    ex += v[k];
+  }
+}
+__device__ __forceinline__ void rank_time_bins(const RankBins &b) {
+  const int lane = threadIdx.x & 31, p = threadIdx.x >> 5;
+  const SortPlan tp = ta_plan_bits(0, (int)b.misc[6]);
+  if (p >= tp.n_pass || tp.n_pass > 5) return;  // (more: the passes are counted anew)
+  const u32 dropped = (u32)(b.sum->n_bad_kind + b.sum->n_bad_interval + b.sum->n_out_of_window);
+  u32 v[8];
+#pragma unroll
+  for (int k = 0; k < 8; k++) v[k] = b.hist[p * 256 + lane * 8 + k] + (lane + k == 0 ? dropped : 0u);
+  scan_bins(v, b.bin_offset + p * 256);
+}
+// n triples are ranked, their counts written
+__device__ __forceinline__ void rank_top_bins(const RankBins &b, const TripleTable *tt, int n, u32 *sh /* 512 */) {
+  const int lane = threadIdx.x & 31, p = threadIdx.x >> 5;
+  const int n_time = ta_plan_bits(0, (int)b.misc[6]).n_pass;
+  const u32 dropped = (u32)(b.sum->n_bad_kind + b.sum->n_bad_interval + b.sum->n_out_of_window);
+  int tbits = 0;
+  while (n > 1 && (n - 1) >> tbits) tbits++;
+  const int L = tbits + (dropped ? 1 : 0);
+  if (L == 0 || n_time > 5) return;
+  const SortPlan lp = ta_plan_bits(0, L);  // two passes at most
+  for (int i = threadIdx.x; i < 512; i += blockDim.x) sh[i] = 0;
+  __syncthreads();
+  for (int r = threadIdx.x; r <= n; r += blockDim.x) {
+    const u32 code = r < n ? (u32)r : 1u << tbits, c = r < n ? tt->rank_cnt[r] : dropped;
+    if (c)
+      for (int q = 0; q < lp.n_pass; q++) atomicAdd(&sh[q * 256 + ((code >> lp.shift[q]) & ((1u << lp.bits[q]) - 1u))], c);
+  }
+  __syncthreads();
+  if (p >= lp.n_pass) return;
+  u32 v[8];
+#pragma unroll
+  for (int k = 0; k < 8; k++) v[k] = sh[p * 256 + lane * 8 + k];
+  scan_bins(v, b.bin_offset + (n_time + p) * 256);
+}
+
+// Both rankings in one launch: CTA 0 the triples, CTA 1 the communicator ids, CTA 2 the time bins (they are
+// independent, and single-CTA kernels one after the other cost a launch latency more each).
 __global__ void __launch_bounds__(1024) k_rank(TripleTable *tt, CommTable *cm, const u32 *slot_cnt,
-                                               int32_t *status, Tail tail) {
+                                               int32_t *status, RankBins bins, Tail tail) {
   TA_PDL();
   extern __shared__ u64 rank_buf[];  // TA_TRIPLE_SLOTS
-  if (blockIdx.x == 0) rank_triples(tt, slot_cnt, status, rank_buf);
-  else rank_comms(cm, status, rank_buf);
+  if (blockIdx.x == 0) {
+    const int n = rank_triples(tt, slot_cnt, status, rank_buf);
+    __syncthreads();
+    if (bins.sum) rank_top_bins(bins, tt, n, reinterpret_cast<u32 *>(rank_buf));
+  } else if (blockIdx.x == 1) {
+    rank_comms(cm, status, rank_buf);
+  } else {
+    rank_time_bins(bins);
+  }
   run_tail(tail);
 }
 
@@ -844,8 +909,10 @@ ta_status ta_launch_discover(ta_window *h, void *zero, size_t zero_bytes, int32_
   }
   TA_CHECK_CUDA(h, cudaFuncSetAttribute(k_rank, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         TA_TRIPLE_SLOTS * (int)sizeof(u64)));
-  ta_launch(k_rank, 2, 1024, TA_TRIPLE_SLOTS * sizeof(u64), h->stream, h->d_triples, h->d_comms, h->d_slot_cnt,
-            h->d_status, ta_tail(h, 2));
+  const bool one = h->W == 1;
+  const RankBins bins{h->d_hist, h->d_misc, one ? h->d_load_sum : nullptr, h->d_bin_offset};
+  ta_launch(k_rank, one ? 3 : 2, 1024, TA_TRIPLE_SLOTS * sizeof(u64), h->stream, h->d_triples, h->d_comms, h->d_slot_cnt,
+            h->d_status, bins, ta_tail(h, one ? 3 : 2));
   TA_CHECK_CUDA(h, cudaGetLastError());
   return TA_OK;
 }
@@ -872,7 +939,6 @@ ta_status ta_launch_load(ta_window *h, bool allow_packed) {
   h->ibits = ta_bit_len((uint64_t)(max_win - 1));
   if (h->ibits < 1) h->ibits = 1;
   h->fast_keys = 0;
-  h->top.rank_cnt = nullptr;
   if (allow_packed && h->prekeys && h->tkeep > 0 && h->tkeep <= h->sbits) {
     // The staged discovery pass took the histograms of the passes over the time bits kept, and
     // the lane sizes give those of the passes above them: the first radix pass can build the
@@ -893,12 +959,7 @@ ta_status ta_launch_load(ta_window *h, bool allow_packed) {
       h->plan.n_pass = tp.n_pass + n_top;
       h->fast_keys = 1;
       if (h->n == 0) return TA_OK;
-      if (h->W == 1) {  // k_radix_scan_hist completes the histograms
-        TopHist &t = h->top;
-        t.plan = h->plan; t.n_time = tp.n_pass; t.top_lo = h->ibits + T; t.tbits = h->tbits; t.wbits = h->wbits;
-        t.n_triples = h->n_triples; t.n_dropped = (u32)(h->n - h->n_valid); t.rank_cnt = h->d_triples->rank_cnt;
-        return TA_OK;
-      }
+      if (h->W == 1) return TA_OK;  // k_rank has scanned the histograms
       TopHistArgs a;
       memset(&a, 0, sizeof(a));
       a.plan = h->plan; a.n_time = tp.n_pass; a.top_lo = h->ibits + T;

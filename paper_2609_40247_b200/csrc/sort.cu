@@ -376,30 +376,12 @@ __global__ void __launch_bounds__(256) k_radix_hist(const u64 *keys, int64_t n, 
 }
 
 // exclusive scan of each pass's histogram: one CTA of 256 threads per pass
-__global__ void __launch_bounds__(256) k_radix_scan_hist(const u32 *hist, u32 *bin_offset, TopHist top) {
+__global__ void __launch_bounds__(256) k_radix_scan_hist(const u32 *hist, u32 *bin_offset) {
   TA_PDL();
   __shared__ u64 tmp[33];
-  __shared__ u32 sh[RS_BINS];
   const int p = blockIdx.x, tid = threadIdx.x;
   u64 total;
-  u32 v;
-  if (top.rank_cnt && p >= top.n_time) {  // from the records counted per lane
-    sh[tid] = 0;
-    __syncthreads();
-    const int shift = top.plan.shift[p] - top.top_lo;
-    const u32 mask = (1u << top.plan.bits[p]) - 1u;
-    for (int r = tid; r < top.n_triples; r += 256) {
-      const u32 c = top.rank_cnt[r];
-      if (c) atomicAdd(&sh[(u32)((u64)r >> shift) & mask], c);
-    }
-    if (tid == 0 && top.n_dropped) atomicAdd(&sh[(u32)((1ull << (top.wbits + top.tbits)) >> shift) & mask], top.n_dropped);
-    __syncthreads();
-    v = sh[tid];
-  } else {
-    v = hist[p * RS_BINS + tid];
-    if (top.rank_cnt && tid == 0) v += top.n_dropped;  // their time digits are 0
-  }
-  u64 ex = block_scan_exclusive<OpAdd>((u64)v, OpAdd(), tmp, &total);
+  const u64 ex = block_scan_exclusive<OpAdd>((u64)hist[p * RS_BINS + tid], OpAdd(), tmp, &total);
   bin_offset[p * RS_BINS + tid] = (u32)ex;
 }
 
@@ -448,12 +430,12 @@ static cudaError_t launch_pass(const RadixArgs &a, int bits, unsigned tiles, cud
 // alternate between the scratch and the final buffers such that the last pass
 // writes the final ones; keys_in / vals_in are only read (pairs with vals_in null:
 // the value of element i is i).  keys_in must not alias scratch or final.
-// `hist` = precomputed [pass][256] digit histograms, or null.
+// `hist` = precomputed [pass][256] digit histograms, or null; `bins` = their scan (hist is not used then), or null.
 template <bool VALS, int ITEMS>
 static ta_status radix_sort(ta_window *h, const u64 *keys_in, const u32 *vals_in, u64 *keys_scratch,
                             u32 *vals_scratch, u64 *keys_final, u32 *vals_final, int64_t n,
                             const SortPlan &plan, const u32 *hist, void *temp,
-                            bool first_pass_unstable, const PrekeyInfo *prekey, const TopHist *top) {
+                            bool first_pass_unstable, const PrekeyInfo *prekey, const u32 *bins) {
   if (n <= 0) return TA_OK;
   constexpr int THREADS = VALS ? RSP_THREADS : RSK_THREADS;
   constexpr int TILE = THREADS * ITEMS;
@@ -473,17 +455,17 @@ static ta_status radix_sort(ta_window *h, const u64 *keys_in, const u32 *vals_in
   u64 *state = cz.take<u64>(per_pass * arrays);
   u32 *counter = cz.take<u32>(16);
   if (!zeroed) TA_CHECK_CUDA(h, cudaMemsetAsync(state, 0, zero, st));
-  if (!hist) {
+  if (!hist && !bins) {
     u32 *own_hist = cz.take<u32>(10 * RS_BINS);
     int64_t want = (n + 255) / 256;
     int grid = (int)(want < 148 * 8 ? want : 148 * 8);
     ta_launch(k_radix_hist, grid, 256, 0, st, keys_in, n, plan, own_hist);
     hist = own_hist;
   }
-  TopHist th;
-  if (top) th = *top;
-  else memset(&th, 0, sizeof(th));
-  ta_launch(k_radix_scan_hist, plan.n_pass, 256, 0, st, hist, bin_offset, th);
+  if (!bins) {
+    ta_launch(k_radix_scan_hist, plan.n_pass, 256, 0, st, hist, bin_offset);
+    bins = bin_offset;
+  }
   const u64 *kin = keys_in;
   const u32 *vin = vals_in;
   for (int p = 0; p < plan.n_pass; p++) {
@@ -492,7 +474,7 @@ static ta_status radix_sort(ta_window *h, const u64 *keys_in, const u32 *vals_in
     a.keys_in = kin; a.keys_out = to_final ? keys_final : keys_scratch;
     a.vals_in = vin; a.vals_out = to_final ? vals_final : vals_scratch;
     a.n = n; a.shift = plan.shift[p];
-    a.bin_offset = bin_offset + p * RS_BINS;
+    a.bin_offset = bins + p * RS_BINS;
     if (!VALS && p > 0 && !at_once)  // untagged descriptors: cleared in front of every pass
       TA_CHECK_CUDA(h, cudaMemsetAsync(state, 0, per_pass * sizeof(u64), st));
     a.tile_state = state + (at_once && !VALS ? (size_t)p * per_pass : 0); a.tile_counter = counter + p; a.status = h->d_status;
@@ -532,8 +514,8 @@ ta_status ta_radix_sort_pairs(ta_window *h, const u64 *keys_in, const u32 *vals_
 
 ta_status ta_radix_sort_keys(ta_window *h, const u64 *keys_in, u64 *keys_scratch, u64 *keys_final,
                              int64_t n, const SortPlan &plan, const u32 *hist, void *temp,
-                             bool first_pass_unstable, const PrekeyInfo *prekey, const TopHist *top) {
+                             bool first_pass_unstable, const PrekeyInfo *prekey, const u32 *bin_offset) {
   auto sort = n <= RS_SMALL ? radix_sort<false, RSK_ITEMS_SMALL> : radix_sort<false, RSK_ITEMS>;
   return sort(h, keys_in, nullptr, keys_scratch, nullptr, keys_final, nullptr, n, plan, hist, temp,
-              first_pass_unstable, prekey, top);
+              first_pass_unstable, prekey, bin_offset);
 }

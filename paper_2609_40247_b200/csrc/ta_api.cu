@@ -519,7 +519,7 @@ static ta_status load_impl(ta_window *h, const ta_event *events, int32_t on_devi
   h->zero_bytes = n <= TA_ZERO_POOL_RECORDS ? Carver::pad((size_t)n * 16 + (3u << 20)) : 0;
   size_t bytes = Carver::pad(up_words * 8) + Carver::pad(ST_WORDS * 4) +
                  Carver::pad(sizeof(TripleTable)) + Carver::pad(sizeof(CommTable)) +
-                 Carver::pad(W * sizeof(ta_load_summary)) + Carver::pad(10 * 256 * 4) +
+                 Carver::pad(W * sizeof(ta_load_summary)) + 2 * Carver::pad(10 * 256 * 4) +
                  Carver::pad(cnt_bytes) + h->zero_bytes + 256;
   void *b = ta_dalloc(h, bytes);
   if (!b) return TA_ERR_OOM;
@@ -529,6 +529,7 @@ static ta_status load_impl(ta_window *h, const ta_event *events, int32_t on_devi
   h->d_t0 = up + (W + 1);
   h->d_t1 = h->d_t0 + W;
   h->d_misc = h->d_t1 + W;
+  h->d_bin_offset = c.take<u32>(10 * 256);
   h->d_triples = c.take<TripleTable>(1);  // (only its first part, the slots, has to be cleared)
   char *zero_begin = (char *)h->d_triples->slots;
   static_assert(offsetof(TripleTable, slots) + sizeof(h->d_triples->slots) == sizeof(TripleTable), "slots come last");

@@ -79,15 +79,6 @@ static inline SortPlan ta_plan_bits(int lo_bit, int hi_bit) {
   return p;
 }
 
-// What the scan of the digit histograms still has to add to them: the (window, lane) digits of a
-// single window from the records counted per triple, and the dropped records of every pass.
-struct TopHist {
-  SortPlan plan;        // passes [n_time, n_pass) are over the bits above top_lo
-  int n_time, top_lo, tbits, wbits, n_triples;
-  u32 n_dropped;
-  const u32 *rank_cnt;  // records per triple rank; null: the histograms are complete
-};
-
 // Device -> host results on their way.  They go through a page-locked block and are handed to their
 // destinations after one wait (a copy into pageable memory would block until it is done).
 struct ResultStage {
@@ -154,7 +145,7 @@ struct ta_window {
   int cnt_windows;             // W, or 0 when there are too many windows to count by window and slot
   int64_t min_name, max_name, max_dur;
   SortPlan plan;
-  TopHist top;
+  u32 *d_bin_offset;           // [pass][256]: of one window, the digits' first places, made by the ranking of the triples
 
   // sort products
   ta_sort_result sorted;
@@ -246,7 +237,7 @@ struct PrekeyInfo {
 ta_status ta_radix_sort_keys(ta_window *h, const u64 *keys_in, u64 *keys_scratch, u64 *keys_final,
                              int64_t n, const SortPlan &plan, const u32 *hist /*nullable*/,
                              void *temp, bool first_pass_unstable, const PrekeyInfo *prekey = nullptr,
-                             const TopHist *top = nullptr);
+                             const u32 *bin_offset = nullptr);
 SortPlan ta_make_plan(int lo_bit, int hi_bit);
 // upload.cu
 ta_status ta_upload(ta_window *h, void *dst, const void *host_src, size_t bytes);  // host -> device on the handle's stream

@@ -610,7 +610,7 @@ ta_status ta_run_sort_timeline(ta_window *h) {
         PrekeyInfo pre{h->d_off, h->W, h->d_triples->rank_of_slot, h->tbits, h->wbits,
                        h->sbits - h->dshift, h->dshift, h->ibits};
         TA_TRY(ta_radix_sort_keys(h, h->d_keys, kscr, skeys, n, h->plan, h->d_hist, sort_tmp, true,
-                                  h->fast_keys ? &pre : nullptr, &h->top));
+                                  h->fast_keys ? &pre : nullptr, h->fast_keys && h->W == 1 ? h->d_bin_offset : nullptr));
         if (n > h->n_valid)
           ta_launch(k_unpack_tail, nblk(n - h->n_valid, 256), 256, 0, st, skeys, h->n_valid, n, pi, perm, h->d_status);
       }
