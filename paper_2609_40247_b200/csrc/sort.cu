@@ -413,10 +413,12 @@ static cudaError_t launch_pass(const RadixArgs &a, int bits, unsigned tiles, cud
 #define RS_CASE(B)                                                                                  \
   case B: {                                                                                         \
     auto kern = k_radix_pass<THREADS, ITEMS, VALS, B, STABLE, PREKEY>;                                     \
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,         \
-                                         (int)sizeof(Smem));                                        \
-    if (e != cudaSuccess) return e;                                                                 \
-    ta_launch(kern, tiles, THREADS, sizeof(Smem), st, a);                                             \
+    if (sizeof(Smem) > (48u << 10)) { /* (what a kernel may have without being asked) */             \
+      cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,       \
+                                           (int)sizeof(Smem));                                      \
+      if (e != cudaSuccess) return e;                                                               \
+    }                                                                                               \
+    ta_launch(kern, tiles + (PREKEY ? a.pk.aside.parts : 0u), THREADS, sizeof(Smem), st, a);          \
     return cudaGetLastError();                                                                      \
   }
   switch (bits) {
