@@ -13,6 +13,7 @@
 // shared-memory atomic and as many warp votes as the digit has bits.
 #include <cstring>
 
+#include "lanes.cuh"
 #include "ta_internal.cuh"
 
 #define RS_BINS 256
@@ -318,6 +319,10 @@ __global__ void __launch_bounds__(THREADS, VALS ? RSP_MINB : RSK_MINB) k_radix_p
   extern __shared__ __align__(16) unsigned char smem_raw[];
   RadixSmem<THREADS, ITEMS> &s = *reinterpret_cast<RadixSmem<THREADS, ITEMS> *>(smem_raw);
   const int tid = threadIdx.x;
+  if (PREKEY && blockIdx.x < a.pk.aside.parts) {
+    timeline_aside(a.pk.aside, blockIdx.x, a.status, s.scan_tmp);
+    return;
+  }
   if (tid == 0) {
     s.tile = (int)atomicAdd(a.tile_counter, 1u);
     s.fail = ta_failed(a.status) ? 1 : 0;

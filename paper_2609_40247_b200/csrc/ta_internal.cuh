@@ -154,6 +154,7 @@ struct ta_window {
   int32_t *d_lane_dev_base;  // per device lane: number of device records in earlier lanes
   int32_t *d_lane_dom_next;  // per lane: index of the first later lane of the other domain
   int64_t n_device;          // kept device records
+  int max_dev_lanes;         // device lanes of a process, at most (neighbouring processes without host lanes count together)
   i64 *d_slot_min, *d_slot_max;               // per slot: corr_id range of its LAUNCH records
   i64 *d_slot_base;                           // per slot: offset of its range when all ranges are laid end to end, -1 = empty
   std::vector<int64_t> h_slot_min, h_slot_max;  // host copies (INT64_MAX / INT64_MIN when none)
@@ -227,12 +228,32 @@ ta_status ta_radix_sort_pairs(ta_window *h, const u64 *keys_in, const u32 *vals_
                               u64 *keys_scratch, u32 *vals_scratch, u64 *keys_final,
                               u32 *vals_final, int64_t n, const SortPlan &plan,
                               const u32 *hist /*nullable*/, void *temp);
+// The lane table of a window or a batch.
+struct LaneTable {
+  const int32_t *lane_start;  // per lane code: first position + 1, 0 = no record
+  int64_t n_codes;
+  int tbits, n_pids;
+  const TripleTable *tt;
+  int64_t n_valid, cap;
+  int32_t *lane_window, *lane_pid;
+  int16_t *lane_stream, *lane_domain;
+  int32_t *lane_off, *lane_slot, *lane_dom_end, *lane_dom_next, *lane_dev_base, *n_lanes_out;
+};
+// What further CTAs of the first pass make, of one window whose records are counted per triple: the lane
+// table, and (rounds > 0) the order of the gather's tiles.  parts = 0: nothing.
+struct TimelineAside {
+  LaneTable lanes;
+  int n_triples;
+  u32 parts, n_tiles, rounds;
+  u32 *order;
+};
 // How the first pass of the timeline sort turns a discovery word into a key on the fly.
 struct PrekeyInfo {
   const int64_t *off;          // window offsets (device), W + 1
   int W;
   const int32_t *rank_of_slot; // triple slot -> rank
   int tbits, wbits, tsb, dshift, ibits;  // tsb = time bits kept
+  TimelineAside aside;
 };
 ta_status ta_radix_sort_keys(ta_window *h, const u64 *keys_in, u64 *keys_scratch, u64 *keys_final,
                              int64_t n, const SortPlan &plan, const u32 *hist /*nullable*/,

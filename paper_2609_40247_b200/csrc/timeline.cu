@@ -13,6 +13,7 @@
 // Dropped records (the tail) are ordered by the full tuple with a chain of stable sorts.
 #include <climits>
 
+#include "lanes.cuh"
 #include "records.cuh"
 #include "scan.cuh"
 #include "ta_internal.cuh"
@@ -144,7 +145,15 @@ __global__ void __launch_bounds__(256) k_tail_place(const u32 *idx, const u32 *r
 }
 
 // ---- step 4: gather records into sorted columns + lane heads ---------------
+// Tiles of a round of the gather's order (a wave of CTAs; 148 to 4736 are within 1 %), and records per
+// process from which the order is made: below some 100 MB the records of a process stay in L2 from its
+// first lane to its last, and in lane order the writes lie closer together (prefill, 4 processes, the kernel
+// without and with the order: 8 M records 174 and 174 us, 16.8 M 425 and 398; experts, 16 processes, 8 M 154
+// and 158, 66.8 M 1388 and 1258).
+#define GO_ROUND 1184
+#define GO_MIN 2500000
 struct GatherArgs {
+  const u32 *order;   // tiles in the order they are taken, null: as they lie
   const ta_event *ev;
   u32 *perm;          // pairs: input; packed keys: written here for the kept records
   const u64 *keys;
@@ -178,8 +187,7 @@ __device__ __forceinline__ u32 gather_index(u64 k, const GatherArgs &a) {
 // waits for the others at the end.
 #define GT_MINB 8
 template <bool PACKED, bool ONE>
-__global__ void __launch_bounds__(256, GT_MINB) k_gather(GatherArgs a) {
-  TA_PDL();
+__device__ __forceinline__ void gather_tile(const GatherArgs &a) {
   __shared__ int s_slot[8];
   __shared__ u64 s_mx[8], s_mn[8];
   __shared__ u32 s_done;
@@ -189,13 +197,14 @@ __global__ void __launch_bounds__(256, GT_MINB) k_gather(GatherArgs a) {
   if (failed) return;
   // positions fit 32 bits (n < 2^31): 32-bit indices keep the address arithmetic of the nine
   // column stores and of the neighbour reads short
-  const u32 p = blockIdx.x * blockDim.x + threadIdx.x;
+  const u32 p = (a.order ? a.order[blockIdx.x] : blockIdx.x) * 256u + threadIdx.x;
   const u32 n = (u32)a.n, nv = (u32)a.n_valid;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const u64 k = p < nv ? a.keys[p] : 0;
   u64 kprev = __shfl_up_sync(0xffffffffu, k, 1);
   if (lane == 0 && p > 0 && p < nv) kprev = a.keys[p - 1];
   const u64 knext = PACKED && lane == 31 && p + 1 < nv ? a.keys[p + 1] : 0;
+  const bool head = !ONE && p < nv && (p == 0 || (kprev >> a.sbits) != (k >> a.sbits));  // of its lane
   u32 idx = 0;
   if (p < n) idx = PACKED && p < nv ? gather_index<ONE>(k, a) : a.perm[p];
   Rec r;
@@ -266,7 +275,7 @@ __global__ void __launch_bounds__(256, GT_MINB) k_gather(GatherArgs a) {
     a.kind[dst] = r.kind;
     if (p < nv) {
       const u64 code = k >> a.sbits;
-      if (p == 0 || (kprev >> a.sbits) != code) a.lane_start[code] = (int32_t)p + 1;
+      if (head) a.lane_start[code] = (int32_t)p + 1;
       if (r.kind == TA_KIND_LAUNCH) {
         slot = (int)(code >> a.tbits) * a.n_pids + a.tt->pid_rank[code & ((1ull << a.tbits) - 1)];
         mx = (u64)r.corr ^ (1ull << 63);
@@ -330,7 +339,7 @@ __device__ __forceinline__ void slot_ranges(const SlotRanges &a, u64 *tmp) {
     const int64_t s = s0 + threadIdx.x;
     u64 size = 0;
     if (s < a.n_slots) {
-      const u64 mx = a.code[s], mn_inv = a.code[a.n_slots + s];
+        const u64 mx = __ldcg(&a.code[s]), mn_inv = __ldcg(&a.code[a.n_slots + s]);
       const bool any = mx != 0 || mn_inv != 0;
       a.slot_max[s] = any ? (i64)(mx ^ (1ull << 63)) : INT64_MIN;
       a.slot_min[s] = any ? (i64)((~mn_inv) ^ (1ull << 63)) : INT64_MAX;
@@ -342,6 +351,17 @@ __device__ __forceinline__ void slot_ranges(const SlotRanges &a, u64 *tmp) {
     base += total;
   }
 }
+// Of one window whose lane table is there already the ranges are all that is left behind the gather: up to
+// the grids that carry a tail its last CTA makes them.
+template <bool PACKED, bool ONE, bool TAIL>
+__global__ void __launch_bounds__(256, GT_MINB) k_gather(GatherArgs a, SlotRanges ranges, Tail tail) {
+  TA_PDL();
+  gather_tile<PACKED, ONE>(a);
+  __shared__ u64 tmp[TAIL ? 33 : 1];
+  if (TAIL) run_tail(tail, [&] {
+    if (!ta_failed(a.status)) slot_ranges(ranges, tmp);
+  });
+}
 __global__ void __launch_bounds__(1024) k_slot_ranges(SlotRanges a, const int32_t *status, Tail tail) {
   TA_PDL();
   __shared__ u64 tmp[33];
@@ -349,123 +369,17 @@ __global__ void __launch_bounds__(1024) k_slot_ranges(SlotRanges a, const int32_
   run_tail(tail);
 }
 
-// One CTA: compacts the non-empty lane codes into the lane table (code order is
-// canonical order).  For few codes; k_scan with the functors below does the same for many.
-__device__ __forceinline__ void lane_table(const int32_t *lane_start, int64_t n_codes,
-                                                     int tbits, int n_pids, const TripleTable *tt,
-                                                     int64_t n_valid, int32_t *lane_window,
-                                                     int32_t *lane_pid, int16_t *lane_stream,
-                                                     int16_t *lane_domain, int32_t *lane_off,
-                                                     int32_t *lane_slot,
-                                                     int32_t *lane_dom_end, int32_t *lane_dom_next,
-                                                     int32_t *lane_dev_base, int32_t *n_lanes_out,
-                                                     int64_t cap, const int32_t *status, u64 *tmp) {
-  __shared__ u64 base;
-  if (ta_failed(status)) {  // no lanes: every later call then finds nothing to index
-    if (threadIdx.x == 0) { n_lanes_out[0] = 0; n_lanes_out[1] = 0; }
-    return;
-  }
-  if (threadIdx.x == 0) base = 0;
-  __syncthreads();
-  for (int64_t c0 = 0; c0 < n_codes; c0 += blockDim.x) {
-    int64_t c = c0 + threadIdx.x;
-    int32_t st = c < n_codes ? lane_start[c] - 1 : -1;
-    u64 total;
-    u64 ex = block_scan_exclusive<OpAdd>(st >= 0 ? 1ull : 0ull, OpAdd(), tmp, &total);
-    if (st >= 0) {
-      int64_t l = (int64_t)(base + ex);
-      if (l < cap) {
-        int w = (int)(c >> tbits), t = (int)(c & ((1ll << tbits) - 1));
-        u64 code = tt->sorted_code[t];
-        lane_window[l] = w;
-        lane_pid[l] = code_pid(code);
-        lane_stream[l] = code_stream(code);
-        lane_domain[l] = code_domain(code);
-        lane_off[l] = st;
-        lane_slot[l] = w * n_pids + tt->pid_rank[t];
-      }
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) base += total;
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
-    int64_t L = (int64_t)base;
-    if (L < cap + 1) lane_off[L] = (int32_t)n_valid;
-    *n_lanes_out = (int32_t)L;
-  }
-  __syncthreads();
-  // per lane: the first later lane of the other domain, and the position where it begins (host
-  // and device lanes alternate per (window, pid), so the runs are a few lanes long - but a batch
-  // of device-only windows is one long run, hence a scan and no walk).  Going backwards over
-  // the lanes, the nearest boundary at or behind lane l is a running maximum of
-  // L - (index of the lane behind a boundary); chunks of blockDim.x lanes, carried in `base`.
-  const int64_t L = (int64_t)base < cap ? (int64_t)base : cap;
-  __syncthreads();  // every thread has read the lane count before `base` is reused
-  if (threadIdx.x == 0) base = 0;
-  __syncthreads();
-  for (int64_t r0 = 0; r0 < L; r0 += blockDim.x) {
-    const int64_t r = r0 + threadIdx.x;  // reversed lane index
-    const int64_t l = L - 1 - r;
-    u64 v = 0;
-    if (r < L && l + 1 < L && lane_domain[l + 1] != lane_domain[l]) v = (u64)(L - (l + 1));
-    u64 total;
-    const u64 ex = block_scan_exclusive<OpMax>(v, OpMax(), tmp, &total);
-    if (r < L) {
-      u64 best = ex > v ? ex : v;
-      best = best > base ? best : base;
-      const int64_t m = best ? L - (int64_t)best : L;
-      lane_dom_end[l] = m < L ? lane_off[m] : (int32_t)n_valid;
-      lane_dom_next[l] = (int32_t)m;  // index of the first later lane of the other domain (L if none)
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) base = base > total ? base : total;
-    __syncthreads();
-  }
-  // per device lane: how many device records sit in earlier lanes (their index once the device
-  // records are taken out in order); n_lanes_out[1] = the number of device records
-  if (threadIdx.x == 0) base = 0;
-  __syncthreads();
-  for (int64_t l0 = 0; l0 < L; l0 += blockDim.x) {
-    const int64_t l = l0 + threadIdx.x;
-    u64 sz = 0;
-    if (l < L && lane_domain[l] == 1) sz = (u64)((l + 1 < L ? lane_off[l + 1] : (int32_t)n_valid) - lane_off[l]);
-    u64 total;
-    const u64 ex = block_scan_exclusive<OpAdd>(sz, OpAdd(), tmp, &total);
-    if (l < L) lane_dev_base[l] = (int32_t)(base + ex);
-    __syncthreads();
-    if (threadIdx.x == 0) base += total;
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) n_lanes_out[1] = (int32_t)base;
-}
-__global__ void __launch_bounds__(1024) k_lane_table(const int32_t *lane_start, int64_t n_codes,
-                                                     int tbits, int n_pids, const TripleTable *tt,
-                                                     int64_t n_valid, int32_t *lane_window,
-                                                     int32_t *lane_pid, int16_t *lane_stream,
-                                                     int16_t *lane_domain, int32_t *lane_off,
-                                                     int32_t *lane_slot,
-                                                     int32_t *lane_dom_end, int32_t *lane_dom_next,
-                                                     int32_t *lane_dev_base, int32_t *n_lanes_out,
-                                                     int64_t cap, const int32_t *status,
-                                                     SlotRanges ranges, Tail tail) {
+__global__ void __launch_bounds__(1024) k_lane_table(LaneTable t, const int32_t *status, SlotRanges ranges, Tail tail) {
   TA_PDL();
   __shared__ u64 tmp[33];
-  lane_table(lane_start, n_codes, tbits, n_pids, tt, n_valid, lane_window, lane_pid, lane_stream, lane_domain, lane_off, lane_slot, lane_dom_end, lane_dom_next, lane_dev_base, n_lanes_out, cap, status, tmp);
+  lane_table<false>(t, status, tmp);
   if (!ta_failed(status)) slot_ranges(ranges, tmp);
   run_tail(tail);
 }
 
 // The same for many codes (a batch of 512 windows has 65 k of them, and one CTA was bound by the
 // scattered writes it has to make alone: 165 us): three scans over as many CTAs as it takes.
-struct LaneRows {
-  const int32_t *lane_start;
-  int tbits, n_pids;
-  const TripleTable *tt;
-  int64_t n_valid;
-  int32_t *lane_window, *lane_pid;
-  int16_t *lane_stream, *lane_domain;
-  int32_t *lane_off, *lane_slot, *lane_dom_end, *lane_dom_next, *lane_dev_base, *n_lanes_out;
+struct LaneRows : LaneTable {
   const u64 *n_lanes;  // total of the first scan
   int64_t bound;       // lanes <= bound
 };
@@ -507,6 +421,7 @@ struct LaneDomOut {
     const int64_t m = best ? L - (int64_t)best : L;
     t.lane_dom_end[l] = m < L ? t.lane_off[m] : (int32_t)t.n_valid;
     t.lane_dom_next[l] = (int32_t)m;
+    if (t.lane_domain[l] == 1 && (l == 0 || t.lane_domain[l - 1] != 1)) atomicMax(&t.n_lanes_out[2], (int32_t)(m - l));
   }
 };
 struct LaneDevIn {
@@ -571,19 +486,22 @@ ta_status ta_run_sort_timeline(ta_window *h) {
   int32_t *lane_dom_end = ck.take<int32_t>(lane_cap);
   int32_t *lane_dev_base = ck.take<int32_t>(lane_cap);
   int32_t *lane_dom_next = ck.take<int32_t>(lane_cap);
-  int32_t *n_lanes_dev = ck.take<int32_t>(2);  // [0] lanes, [1] device records
+  int32_t *n_lanes_dev = ck.take<int32_t>(3);  // [0] lanes, [1] device records, [2] device lanes of a process at most
   h->d_slot_min = ck.take<i64>(3 * n_slots);
   h->d_slot_max = h->d_slot_min + n_slots;
   h->d_slot_base = h->d_slot_max + n_slots;
 
   // temporaries (released at the end of the call)
-  size_t tmp_bytes = 2 * Carver::pad(n * 8) + Carver::pad(n * 4) + ta_sort_temp_bytes(n) +
+  const u32 tiles = (u32)((n + 255) / 256);
+  const bool by_round = h->packed && h->fast_keys && h->W == 1 && n / (h->n_pids > 0 ? h->n_pids : 1) >= GO_MIN;
+  size_t tmp_bytes = 2 * Carver::pad(n * 8) + Carver::pad(n * 4) + Carver::pad(by_round ? (size_t)tiles * 4 : 0) + ta_sort_temp_bytes(n) +
                      2 * scan_temp_bytes(lane_cap) + scan_temp_bytes(n_codes) + 512;
   void *tb = ta_dalloc(h, tmp_bytes);
   if (!tb) return TA_ERR_OOM;
   Carver ct(tb);
   u64 *kscr = ct.take<u64>(n), *skeys = ct.take<u64>(n);
   u32 *vscr = ct.take<u32>(n);
+  u32 *order = ct.take<u32>(by_round ? tiles : 0);
   ta_status zs;
   // cleared: first positions per lane code, correlation-id ranges per slot
   const size_t zero_bytes = Carver::pad((size_t)n_codes * 4) + Carver::pad((size_t)n_slots * 16);
@@ -594,7 +512,14 @@ ta_status ta_run_sort_timeline(ta_window *h) {
   u64 *slot_code = cz.take<u64>(2 * n_slots);
   void *sort_tmp = ct.base + ct.off;
 
-  int32_t n_lanes_host[2] = {0, 0};
+  // of one window the lanes follow from the counts of the load, beside the first pass
+  const bool lanes_early = h->W == 1 && h->packed && h->fast_keys && n > 0;
+  const LaneTable lanes{lane_start, n_codes, h->tbits, h->n_pids > 0 ? h->n_pids : 1, h->d_triples, h->n_valid, lane_cap,
+                        lane_window, lane_pid, lane_stream, lane_domain, lane_off, lane_slot,
+                        lane_dom_end, lane_dom_next, lane_dev_base, n_lanes_dev};
+  const SlotRanges ranges{slot_code, n_slots, h->d_slot_min, h->d_slot_max, h->d_slot_base};
+  bool tailed = false;  // the gather did the ranges and brings the results
+  int32_t n_lanes_host[3] = {0, 0, 0};
   // Packed keys settle the order down to a coarse time; the gather ranks the members of a run
   // of equal coarse keys itself.  A run too long for that is reported at the end, and the
   // second attempt sorts (key, index) pairs at full time resolution.
@@ -602,13 +527,28 @@ ta_status ta_run_sort_timeline(ta_window *h) {
     int32_t words[ST_WORDS];
     h->h_slot_min.resize((size_t)n_slots);
     h->h_slot_max.resize((size_t)n_slots);
+    auto fetch = [&]() -> ta_status {
+      TA_TRY(ta_queue_d2h(h, n_lanes_host, n_lanes_dev, 3 * sizeof(int32_t)));
+      TA_TRY(ta_queue_d2h(h, words, h->d_status, sizeof(words)));
+      TA_TRY(ta_queue_d2h(h, h->h_slot_min.data(), h->d_slot_min, n_slots * 8));
+      return ta_queue_d2h(h, h->h_slot_max.data(), h->d_slot_max, n_slots * 8);
+    };
     if (attempt) TA_CHECK_CUDA(h, cudaMemsetAsync(zb, 0, zero_bytes, st));
     if (n > 0) {
       if (h->packed) {
         // keys carry the index: 8-byte elements, fewer bytes per pass
         PackInfo pi{h->ibits, h->ibits + h->tbits + (h->sbits - h->dshift), h->wbits, h->d_off};
         PrekeyInfo pre{h->d_off, h->W, h->d_triples->rank_of_slot, h->tbits, h->wbits,
-                       h->sbits - h->dshift, h->dshift, h->ibits};
+                       h->sbits - h->dshift, h->dshift, h->ibits, TimelineAside()};
+        if (lanes_early) {
+          TimelineAside &x = pre.aside;
+          x.lanes = lanes;
+          x.lanes.n_codes = x.n_triples = h->n_triples;
+          x.n_tiles = tiles;
+          x.rounds = by_round ? (tiles + GO_ROUND - 1) / GO_ROUND : 0;
+          x.order = order;
+          x.parts = 1 + x.rounds;
+        }
         TA_TRY(ta_radix_sort_keys(h, h->d_keys, kscr, skeys, n, h->plan, h->d_hist, sort_tmp, true,
                                   h->fast_keys ? &pre : nullptr, h->fast_keys && h->W == 1 ? h->d_bin_offset : nullptr));
         if (n > h->n_valid)
@@ -685,6 +625,7 @@ ta_status ta_run_sort_timeline(ta_window *h) {
       }
       // step 4
       GatherArgs g;
+      g.order = h->packed && by_round ? order : nullptr;
       g.ev = h->events; g.perm = perm; g.keys = skeys; g.n = n; g.n_valid = h->n_valid;
       g.packed = h->packed; g.ibits = h->ibits; g.wbits = h->wbits; g.off = h->d_off;
       g.wshift = h->ibits + h->tbits + (h->sbits - h->dshift);
@@ -693,23 +634,26 @@ ta_status ta_run_sort_timeline(ta_window *h) {
       g.stream = c_stream; g.kind = c_kind; g.lane_start = lane_start;
       g.tt = h->d_triples; g.tbits = h->tbits; g.n_pids = h->n_pids > 0 ? h->n_pids : 1;
       g.slot_code = slot_code; g.n_slots = n_slots; g.status = h->d_status;
-      auto gather = h->packed ? (h->W == 1 ? k_gather<true, true> : k_gather<true, false>) : k_gather<false, false>;
-      ta_launch(gather, nblk(n, 256), 256, 0, st, g);
-    }
-    TA_TRY(ta_queue_d2h(h, n_lanes_host, n_lanes_dev, 2 * sizeof(int32_t)));
-    TA_TRY(ta_queue_d2h(h, words, h->d_status, sizeof(words)));
-    for (int q = 0; q < 2; q++)
-      TA_TRY(ta_queue_d2h(h, q ? h->h_slot_max.data() : h->h_slot_min.data(), q ? h->d_slot_max : h->d_slot_min, n_slots * 8));
-    const SlotRanges ranges{slot_code, n_slots, h->d_slot_min, h->d_slot_max, h->d_slot_base};
-    if (n_codes <= LT_ONE_CTA || n == 0) {
-      // (few codes: fewer warps to wait for at each of its barriers)
-      ta_launch(k_lane_table, 1, n_codes <= 256 && n_slots <= 256 ? 256 : 1024, 0, st, lane_start, n_codes, h->tbits, h->n_pids > 0 ? h->n_pids : 1, h->d_triples,
-                h->n_valid, lane_window, lane_pid, lane_stream, lane_domain, lane_off, lane_slot,
-                lane_dom_end, lane_dom_next, lane_dev_base, n_lanes_dev, lane_cap, h->d_status, ranges, ta_tail(h, 1));
+      TA_TRY(fetch());
+      const unsigned grid = (unsigned)nblk(n, 256);
+      Tail tail;
+      if (lanes_early && h->packed && grid <= 1024) tail = ta_tail(h, grid);
+      tailed = tail.m > 0;
+      auto gather = !h->packed ? k_gather<false, false, false>
+                    : !lanes_early ? k_gather<true, false, false>
+                    : tailed ? k_gather<true, true, true> : k_gather<true, true, false>;
+      ta_launch(gather, grid, 256, 0, st, g, ranges, tail);
     } else {
-      LaneRows t{lane_start, h->tbits, h->n_pids > 0 ? h->n_pids : 1, h->d_triples, h->n_valid,
-                 lane_window, lane_pid, lane_stream, lane_domain, lane_off, lane_slot,
-                 lane_dom_end, lane_dom_next, lane_dev_base, n_lanes_dev, nullptr, lane_cap - 1};
+      TA_TRY(fetch());
+    }
+    if (tailed) {
+    } else if (lanes_early) {
+      ta_launch(k_slot_ranges, 1, n_slots <= 256 ? 256 : 1024, 0, st, ranges, h->d_status, ta_tail(h, 1));
+    } else if (n_codes <= LT_ONE_CTA || n == 0) {
+      // (few codes: fewer warps to wait for at each of its barriers)
+      ta_launch(k_lane_table, 1, n_codes <= 256 && n_slots <= 256 ? 256 : 1024, 0, st, lanes, h->d_status, ranges, ta_tail(h, 1));
+    } else {
+      LaneRows t{lanes, nullptr, lane_cap - 1};
       Carver cs(sort_tmp);  // the sort is done with its temporaries by the time the scans run
       ScanTemp s1, s2, s3;
       cs.off += scan_temp_carve(cs.base + cs.off, n_codes, &s1);
@@ -717,7 +661,7 @@ ta_status ta_run_sort_timeline(ta_window *h) {
       cs.off += scan_temp_carve(cs.base + cs.off, t.bound, &s3);
       TA_CHECK_CUDA(h, cudaMemsetAsync(sort_tmp, 0, cs.off, st));
       t.n_lanes = s1.total;
-      TA_CHECK_CUDA(h, cudaMemsetAsync(n_lanes_dev, 0, 8, st));
+      TA_CHECK_CUDA(h, cudaMemsetAsync(n_lanes_dev, 0, 12, st));
       TA_TRY((launch_scan<OpAdd, LaneCodeIn, LaneCodeOut>(h, n_codes, LaneCodeIn{t}, LaneCodeOut{t}, OpAdd(), s1)));
       TA_TRY((launch_scan<OpMax, LaneDomIn, LaneDomOut>(h, t.bound, LaneDomIn{t}, LaneDomOut{t}, OpMax(), s2)));
       TA_TRY((launch_scan<OpAdd, LaneDevIn, LaneDevOut>(h, t.bound, LaneDevIn{t}, LaneDevOut{t}, OpAdd(), s3)));
@@ -738,6 +682,7 @@ ta_status ta_run_sort_timeline(ta_window *h) {
 
   const int32_t n_lanes = n_lanes_host[0];
   h->n_device = n_lanes_host[1];
+  h->max_dev_lanes = n_lanes_host[2];
   ta_sort_result &r = h->sorted;
   r.n = n; r.n_valid = h->n_valid; r.n_lanes = n_lanes; r.n_windows = h->W;
   r.perm = (const int32_t *)perm;

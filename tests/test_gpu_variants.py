@@ -1,0 +1,55 @@
+"""The two sides of each rule that chooses a way by sizes, value ranges or lanes, at the sizes where
+they can go wrong, bit for bit against the oracle."""
+import numpy as np
+import pytest
+
+from paper_2609_40247_b200.synth import EVENT_DTYPE
+from test_gpu_parity import both
+
+pytestmark = pytest.mark.gpu
+
+T0 = 1_700_000_000_000_000_000
+
+
+def _device(n, starts, durations, pid=0, stream=0, kind=3, name=0):
+    ev = np.zeros(n, dtype=EVENT_DTYPE)
+    ev["ts_start"], ev["ts_end"] = starts, starts + durations
+    ev["pid"], ev["stream"], ev["kind"], ev["name_id"] = pid, stream, kind, name
+    ev["corr_id"] = -1 - np.arange(n)
+    return ev
+
+
+@pytest.mark.parametrize("lanes,per", [(1, 3), (2, 255), (257, 9), (1030, 3), (40, 700)])
+def test_lane_table_from_the_counts_of_the_load(lanes, per):
+    """Lanes of one window from the records counted per triple: one to several rounds of the CTA that
+    makes the table, host and device lanes in any order, some records dropped."""
+    rng = np.random.default_rng(lanes)
+    n = lanes * per
+    ev = np.zeros(n, dtype=EVENT_DTYPE)
+    lane = rng.permutation(np.arange(n) % lanes)
+    ev["pid"] = lane // 5 - lanes // 10
+    ev["stream"] = lane % 5
+    ev["kind"] = np.where(lane % 5 < 2, 1, 3)
+    ev["ts_start"] = T0 + rng.integers(0, 10**9, n)
+    ev["ts_end"] = ev["ts_start"] + rng.integers(1, 10**5, n)
+    ev["corr_id"] = np.arange(n)
+    both(ev, [0, n], [T0], [T0 + 10**9])
+    ev["kind"][::11] = 7
+    both(ev, [0, n], [T0], [T0 + 10**9])
+
+
+def test_gather_takes_the_lanes_of_large_processes_together():
+    """One process with more records than the gather's order of tiles begins at: two lanes of very
+    different lengths and a dropped tail that begins inside a tile."""
+    n = 2_700_001
+    rng = np.random.default_rng(3)
+    ev = np.zeros(n, dtype=EVENT_DTYPE)
+    device = np.arange(n) % 7 > 2
+    ev["kind"] = np.where(device, 3, 2)
+    ev["stream"] = np.where(device, np.where(np.arange(n) % 5000 == 4, 9, 1), 0)
+    ev["ts_start"] = T0 + np.arange(n) * 5000 + rng.integers(0, 5000, n)
+    ev["ts_end"] = ev["ts_start"] + 2000
+    ev["corr_id"] = np.arange(n) // 2
+    ev = ev[np.argsort(np.arange(n) // 4096 * 2 + device, kind="stable")]
+    ev["kind"][5::4001] = 7
+    both(ev, [0, n], [T0], [T0 + n * 5000], min_gap=50_000_000)
