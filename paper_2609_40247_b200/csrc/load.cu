@@ -939,18 +939,28 @@ ta_status ta_launch_load(ta_window *h, bool allow_packed) {
   h->ibits = ta_bit_len((uint64_t)(max_win - 1));
   if (h->ibits < 1) h->ibits = 1;
   h->fast_keys = 0;
+  h->xbits = 0;
   if (allow_packed && h->prekeys && h->tkeep > 0 && h->tkeep <= h->sbits) {
     // The staged discovery pass took the histograms of the passes over the time bits kept, and
     // the lane sizes give those of the passes above them: the first radix pass can build the
     // keys from the discovery words, no key pass is needed.  Passes over time bits and passes
     // over (dropped, window, triple rank) bits never share a digit.
     const int T = h->tkeep, L = hd + h->wbits + h->tbits;
-    const SortPlan tp = ta_plan_bits(h->ibits, h->ibits + T);
-    const SortPlan lp = ta_plan_bits(h->ibits + T, h->ibits + T + L);
+    // What is left of the 64 bits goes to further time bits below those that are sorted: the gather
+    // ranks the records of a cell by them, without a look at the records.  Bursts are what gains by it: the
+    // gather of 16.8 M prefill records, 82 % of them in cells with others and seven to a cell, takes 393 us
+    // and 422 without; of 66.8 M expert records, 22 % and two, 1262 and 1255, and 512 windows of 65 k records
+    // lost 490 to 468: windows of a batch go without.
+    const int spare = h->W == 1 ? 64 - (T + L + h->ibits) : 0;
+    const int X = spare < 0 ? 0 : spare < h->sbits - T ? spare : h->sbits - T;
+    const int lo = h->ibits + X;
+    const SortPlan tp = ta_plan_bits(lo, lo + T);
+    const SortPlan lp = ta_plan_bits(lo + T, lo + T + L);
     const int n_top = L > 0 ? lp.n_pass : 0;
     if (T + L + h->ibits <= 64 && tp.n_pass <= 5 && tp.n_pass + n_top <= 10) {
       h->packed = 1;
-      h->dshift = h->sbits - T;
+      h->xbits = X;
+      h->dshift = h->sbits - T - X;
       h->plan = tp;
       for (int q = 0; q < n_top; q++) {
         h->plan.shift[tp.n_pass + q] = lp.shift[q];
@@ -962,7 +972,7 @@ ta_status ta_launch_load(ta_window *h, bool allow_packed) {
       if (h->W == 1) return TA_OK;  // k_rank has scanned the histograms
       TopHistArgs a;
       memset(&a, 0, sizeof(a));
-      a.plan = h->plan; a.n_time = tp.n_pass; a.top_lo = h->ibits + T;
+      a.plan = h->plan; a.n_time = tp.n_pass; a.top_lo = lo + T;
       a.tbits = h->tbits; a.wbits = h->wbits; a.tt = h->d_triples; a.hist = h->d_hist;
       a.prekey = h->d_keys; a.n = h->n; a.off = h->d_off; a.W = h->W;
       // (512 windows of 65 k records: 211 us from the words)

@@ -139,6 +139,7 @@ struct ta_window {
   int n_triples, n_pids;
   int sbits, tbits, wbits, has_dropped;
   int packed, dshift, ibits;   // packed keys: low ibits = index inside the window, dshift low time bits dropped
+  int xbits;                   // packed keys: low time bits of the key that the passes leave unsorted
   int tkeep;                   // time bits the planning kernel decided to keep (0 = it did not run)
   int fast_keys;               // the first radix pass builds the keys from the discovery words itself
   u32 *d_slot_cnt;             // kept records per (window, triple slot) of the first cnt_windows windows

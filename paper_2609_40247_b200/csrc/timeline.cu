@@ -160,6 +160,8 @@ struct GatherArgs {
   int64_t n, n_valid;
   int sbits;          // key bits below the lane code (time bits kept [+ index bits])
   int packed, ibits, wshift, wbits;
+  int cshift;         // packed keys: bits below the cell, which the passes did not sort
+  u32 xmask;          // those of them above the index
   const int64_t *off;
   // corr_id range of the LAUNCH records per (window, pid) slot, for the join
   const TripleTable *tt;
@@ -209,49 +211,70 @@ __device__ __forceinline__ void gather_tile(const GatherArgs &a) {
   if (p < n) idx = PACKED && p < nv ? gather_index<ONE>(k, a) : a.perm[p];
   Rec r;
   if (p < n) r = load_rec(a.ev, idx);
-  u32 dst = p;  // where the record goes: p, or its place inside a run of equal coarse keys
+  u32 dst = p;  // where the record goes: p, or its place inside a run of equal cells
   if (PACKED) {
     // packed keys order the records down to a coarse time only: members of a run of equal
     // (lane, coarse time) sit in no particular order (the first radix pass is not stable) and
-    // are ranked here by (ts_start, -ts_end, input index)
-    const u64 hk = k >> a.ibits;
-    const u32 eq = __ballot_sync(0xffffffffu, p < nv && p > 0 && (kprev >> a.ibits) == hk);
-    const bool next = __any_sync(0xffffffffu, lane == 31 && p + 1 < nv && (knext >> a.ibits) == hk);
+    // are ranked here by (ts_start, -ts_end, input index): of one window by the time bits the passes left
+    // alone, and by the records where those are the same
+    constexpr bool FINE = ONE;
+    const u64 hk = k >> a.cshift;
+    const u32 eq = __ballot_sync(0xffffffffu, p < nv && p > 0 && (kprev >> a.cshift) == hk);
+    const bool next = __any_sync(0xffffffffu, lane == 31 && p + 1 < nv && (knext >> a.cshift) == hk);
     if (eq || next) {
-      // equal keys in front of the record and behind it, as far as the warp reaches
+      const u32 fine = FINE ? (u32)(k >> a.ibits) & a.xmask : 0u;
+      // equal cells in front of the record and behind it, as far as the warp reaches
       int before = __clz((int)~(eq << (31 - lane)));
       int after = lane < 31 ? __ffs((int)~(eq >> (lane + 1))) - 1 : 0;
       // a run that meets the warp's edge goes on in memory
       const bool open = p < nv && (before == lane + 1 || (lane + after == 31 && next));
       int rank = 0;
-      // the others: every member is compared with the one d places in front of it, and what it
+      const int rounds = __reduce_max_sync(0xffffffffu, open ? 0 : before);
+      // every member is compared with the one d places in front of it, and what it
       // learns holds the other way round for that one
-      for (int d = 1;; d++) {
+      for (int d = 1; d <= rounds; d++) {
         const bool me = !open && before >= d;
         const u32 m = __ballot_sync(0xffffffffu, me);
-        if (m == 0) break;
-        const i64 os = __shfl_up_sync(0xffffffffu, r.ts_start, d);
-        bool first = os < r.ts_start;
-        if (__any_sync(0xffffffffu, me && os == r.ts_start)) {
-          const i64 oe = __shfl_up_sync(0xffffffffu, r.ts_end, d);
-          const u32 oi = __shfl_up_sync(0xffffffffu, idx, d);
-          first = first || (os == r.ts_start && (oe > r.ts_end || (oe == r.ts_end && oi < idx)));
+        bool first;
+        if (FINE) {
+          const u32 of = __shfl_up_sync(0xffffffffu, fine, d);
+          first = of < fine;
+          if (__any_sync(0xffffffffu, me && of == fine)) {
+            const i64 os = __shfl_up_sync(0xffffffffu, r.ts_start, d);
+            const i64 oe = __shfl_up_sync(0xffffffffu, r.ts_end, d);
+            const u32 oi = __shfl_up_sync(0xffffffffu, idx, d);
+            first = first || (of == fine && (os < r.ts_start || (os == r.ts_start && (oe > r.ts_end || (oe == r.ts_end && oi < idx)))));
+          }
+        } else {
+          const i64 os = __shfl_up_sync(0xffffffffu, r.ts_start, d);
+          first = os < r.ts_start;
+          if (__any_sync(0xffffffffu, me && os == r.ts_start)) {
+            const i64 oe = __shfl_up_sync(0xffffffffu, r.ts_end, d);
+            const u32 oi = __shfl_up_sync(0xffffffffu, idx, d);
+            first = first || (os == r.ts_start && (oe > r.ts_end || (oe == r.ts_end && oi < idx)));
+          }
         }
         const u32 b = __ballot_sync(0xffffffffu, me && first);
         rank += (me && first ? 1 : 0) + (int)(((m & ~b) >> d) >> lane & 1u);
       }
       if (open) {
         if (before == lane + 1)
-          while (before <= TA_TIE_RUN_MAX && p > (u32)before && (a.keys[p - before - 1] >> a.ibits) == hk) before++;
+          while (before <= TA_TIE_RUN_MAX && p > (u32)before && (a.keys[p - before - 1] >> a.cshift) == hk) before++;
         if (lane + after == 31)
-          while (after <= TA_TIE_RUN_MAX && p + after + 1 < nv && (a.keys[p + after + 1] >> a.ibits) == hk) after++;
+          while (after <= TA_TIE_RUN_MAX && p + after + 1 < nv && (a.keys[p + after + 1] >> a.cshift) == hk) after++;
         if (before + after + 1 > TA_TIE_RUN_MAX) {
           a.status[ST_LONG_RUN] = 1;  // the caller starts over with full-resolution keys
           before = after = 0;
         }
         for (int q = -before; q <= after; q++) {
           if (q == 0) continue;
-          const u32 oi = gather_index<ONE>(a.keys[p + q], a);
+          const u64 ok = a.keys[p + q];
+          const u32 of = FINE ? (u32)(ok >> a.ibits) & a.xmask : 0u;
+          if (of != fine) {
+            rank += of < fine ? 1 : 0;
+            continue;
+          }
+          const u32 oi = gather_index<ONE>(ok, a);
           const i64 *o = reinterpret_cast<const i64 *>(a.ev) + (u64)oi * 5;
           const i64 os = o[0], oe = o[1];
           const bool first = os < r.ts_start || (os == r.ts_start && (oe > r.ts_end || (oe == r.ts_end && oi < idx)));
@@ -628,6 +651,7 @@ ta_status ta_run_sort_timeline(ta_window *h) {
       g.order = h->packed && by_round ? order : nullptr;
       g.ev = h->events; g.perm = perm; g.keys = skeys; g.n = n; g.n_valid = h->n_valid;
       g.packed = h->packed; g.ibits = h->ibits; g.wbits = h->wbits; g.off = h->d_off;
+      g.cshift = h->ibits + h->xbits; g.xmask = (u32)((1ull << h->xbits) - 1);
       g.wshift = h->ibits + h->tbits + (h->sbits - h->dshift);
       g.sbits = h->packed ? h->ibits + (h->sbits - h->dshift) : h->sbits;
       g.ts_start = c_ts; g.ts_end = c_te; g.corr = c_corr; g.pid = c_pid; g.name = c_name; g.seq = c_seq;

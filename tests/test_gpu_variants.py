@@ -19,6 +19,22 @@ def _device(n, starts, durations, pid=0, stream=0, kind=3, name=0):
     return ev
 
 
+@pytest.mark.parametrize("run", [1, 2, 31, 33, 47, 48, 49, 64, 65])
+@pytest.mark.parametrize("step", [0, 1, 3])
+def test_runs_of_records_in_one_cell_of_the_sort_key(run, step):
+    """Bursts whose records share the sorted bits of the key, before and beyond the length that is
+    ranked in place, told apart by the bits below (step 3), by the records (0: equal starts) or by
+    both, in a window long enough for coarse cells; bursts cross tiles of 256 at every offset."""
+    bursts = 700 // run + 40
+    at = T0 + np.repeat(np.sort(np.random.default_rng(run).choice(10**6, bursts, replace=False)) * 30_000, run)
+    starts = at + np.tile(np.arange(run) * step, bursts)
+    ev = _device(len(starts), starts, 5 + np.tile(np.arange(run) % 3, bursts), stream=np.arange(len(starts)) % 2)
+    ev = ev[np.random.default_rng(7).permutation(len(ev))]
+    for windows in (1, 2):
+        off = [0, len(ev)] if windows == 1 else [0, len(ev) // 3, len(ev)]
+        both(ev, off, [T0] * windows, [T0 + 31 * 10**9] * windows)
+
+
 @pytest.mark.parametrize("lanes,per", [(1, 3), (2, 255), (257, 9), (1030, 3), (40, 700)])
 def test_lane_table_from_the_counts_of_the_load(lanes, per):
     """Lanes of one window from the records counted per triple: one to several rounds of the CTA that
