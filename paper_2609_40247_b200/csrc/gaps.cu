@@ -470,6 +470,39 @@ __global__ void __launch_bounds__(256) k_gap_list_order(const ta_long_gap *src, 
   dst[rank[k >> 6] + __popcll(bits[k >> 6] & ((1ull << (k & 63u)) - 1ull))] = src[i];
 }
 
+// Both steps in one CTA for a short bitmap and list: what a launch costs more than the work.
+#define GL_THREADS 1024
+#define GL_WORDS 8192    // words of the bitmap (262 k records)
+#define GL_ENTRIES 8192
+__global__ void __launch_bounds__(GL_THREADS) k_gap_list_one(const ta_long_gap *src, const u32 *key, const u64 *bits,
+                                                             int n_bits, int m, ta_long_gap *dst, const int32_t *status) {
+  TA_PDL();
+  __shared__ u64 tmp[33];
+  __shared__ u32 rank[GL_WORDS];
+  if (ta_failed(status)) return;
+  constexpr int PER = GL_WORDS / GL_THREADS;
+  const int w0 = threadIdx.x * PER;
+  u32 c[PER], mine = 0;
+#pragma unroll
+  for (int k = 0; k < PER; k++) {
+    c[k] = w0 + k < n_bits ? (u32)__popcll(bits[w0 + k]) : 0u;
+    mine += c[k];
+  }
+  u64 total;
+  u32 r = (u32)block_scan_exclusive<OpAdd>((u64)mine, OpAdd(), tmp, &total);
+#pragma unroll
+  for (int k = 0; k < PER; k++) {
+    rank[w0 + k] = r;
+    r += c[k];
+  }
+  __syncthreads();
+#pragma unroll 2
+  for (int i = threadIdx.x; i < m; i += GL_THREADS) {
+    const u32 k = key[i];
+    dst[rank[k >> 6] + __popcll(bits[k >> 6] & ((1ull << (k & 63u)) - 1ull))] = src[i];
+  }
+}
+
 ta_status ta_run_gaps(ta_window *h, int64_t min_gap, ta_gap_result *out) {
   const int64_t n = h->n;
   const int L = h->sorted.n_lanes;
@@ -573,10 +606,14 @@ ta_status ta_run_gaps(ta_window *h, int64_t min_gap, ta_gap_result *out) {
   if (m > 0) {
     list = (ta_long_gap *)ta_dalloc(h, (size_t)m * sizeof(ta_long_gap));
     if (!list) return TA_ERR_OOM;
-    GapBitsIn bi{bits};
-    GapBitsOut bo{rank};
-    TA_TRY((launch_scan<OpAdd, GapBitsIn, GapBitsOut>(h, n_bits, bi, bo, OpAdd(), scan)));
-    ta_launch(k_gap_list_order, (unsigned)((m + 255) / 256), 256, 0, st, ulist, ukeys, bits, rank, m, list, h->d_status);
+    if (n_bits <= GL_WORDS && m <= GL_ENTRIES) {
+      ta_launch(k_gap_list_one, 1, GL_THREADS, 0, st, ulist, ukeys, bits, (int)n_bits, (int)m, list, h->d_status);
+    } else {
+      GapBitsIn bi{bits};
+      GapBitsOut bo{rank};
+      TA_TRY((launch_scan<OpAdd, GapBitsIn, GapBitsOut>(h, n_bits, bi, bo, OpAdd(), scan)));
+      ta_launch(k_gap_list_order, (unsigned)((m + 255) / 256), 256, 0, st, ulist, ukeys, bits, rank, m, list, h->d_status);
+    }
     TA_CHECK_CUDA(h, cudaGetLastError());
     // both kernels are still queued: their temporaries go back after the handle's next
     // wait (the list itself is used in stream order like every other result)

@@ -69,3 +69,14 @@ def test_gather_takes_the_lanes_of_large_processes_together():
     ev = ev[np.argsort(np.arange(n) // 4096 * 2 + device, kind="stable")]
     ev["kind"][5::4001] = 7
     both(ev, [0, n], [T0], [T0 + n * 5000], min_gap=50_000_000)
+
+
+@pytest.mark.parametrize("n", [8192, 262_143, 262_145, 300_000])
+def test_long_gaps_ordered_by_one_cta_and_by_many(n):
+    """Lists and bitmaps around the size one CTA puts in order: every record behind a long gap, and one
+    in ninety."""
+    for every in (1, 90):
+        wait = np.where(np.arange(n) % every == 0, 700, 0)
+        starts = T0 + np.cumsum(wait + 10)
+        ev = _device(n, starts, 10, stream=np.arange(n) % 3)
+        both(ev, [0, n], [T0], [T0 + (1 << 35)], min_gap=500 if every > 1 else 1)
