@@ -304,8 +304,16 @@ __global__ void __launch_bounds__(GP_THREADS, GP_MINB) k_gaps(GapArgs a, Tail ta
 // with eight consecutive records, each with its own lane walk, took 270 warp instructions per 32
 // records and bound the kernel: 480 us for 66.8 M records).  Statistics of the CTA's first GR_LANES
 // lanes are folded on chip.
+// Long gaps are collected on chip and take their places in the list with one add per CTA: in a window of
+// stalls every row has some (a fifth of the records of a prefill window), and an add per row on the one
+// cursor, at about a nanosecond each, was all the kernel did (16.8 M prefill records 165 us, 85 now).
 #define GR_LANES 4
+#define GR_LIST 512
 __device__ __forceinline__ void gaps_rows(const GapArgs &a, int rows) {
+  __shared__ ta_long_gap s_list[GR_LIST];
+  __shared__ u32 s_key[GR_LIST];
+  __shared__ u32 s_n;
+  __shared__ u64 s_base;
   __shared__ u64 s_sum[GR_LANES][3];  // busy, idle, gaps
   __shared__ i64 s_max[GR_LANES];
   __shared__ u32 s_hist[GR_LANES][TA_NBINS];
@@ -315,6 +323,7 @@ __device__ __forceinline__ void gaps_rows(const GapArgs &a, int rows) {
   for (int i = tid; i < GR_LANES * TA_NBINS; i += GP_THREADS) (&s_hist[0][0])[i] = 0;
   if (tid < GR_LANES * 3) (&s_sum[0][0])[tid] = 0;
   if (tid < GR_LANES) s_max[tid] = 0;
+  if (tid == 0) s_n = 0;
   const int64_t span = (int64_t)rows * 32;
   const int64_t begin = ((int64_t)blockIdx.x * (GP_THREADS / 32) + warp) * span;
   const int64_t end = min(begin + span, a.n), vend = min(end, a.n_valid);
@@ -388,17 +397,27 @@ __device__ __forceinline__ void gaps_rows(const GapArgs &a, int rows) {
           a.lane_gaps[l].n_events = lane_end - off;
         }
       }
-      // long-gap list: the warp reserves its entries with one add on the cursor (they are put in
-      // order afterwards)
+      // long-gap list (put in order afterwards): what finds no room on chip takes its place in memory
+      // with an add per row
       const bool lg = g > 0 && g >= a.min_gap;
       if (__any_sync(0xffffffffu, lg || lt)) {
         const u32 m_g = __ballot_sync(0xffffffffu, lg), m_t = __ballot_sync(0xffffffffu, lt);
-        const u32 below = (1u << lane) - 1u;
+        const u32 below = (1u << lane) - 1u, n_g = (u32)__popc(m_g), cnt = n_g + (u32)__popc(m_t);
+        u32 at = 0;
+        if (lane == 0) at = atomicAdd(&s_n, cnt);
+        at = __shfl_sync(0xffffffffu, at, 0);
+        const u32 room = at < GR_LIST ? min(cnt, GR_LIST - at) : 0u;
         u64 base = 0;
-        if (lane == 0) base = atomicAdd(a.n_long, (u64)(__popc(m_g) + __popc(m_t)));
-        base = __shfl_sync(0xffffffffu, base, 0);
-        if (lg) gap_append(a, (i64)base + __popc(m_g & below), ta_long_gap{l, (int32_t)p, P, g}, (u32)p << 1);
-        if (lt) gap_append(a, (i64)base + __popc(m_g) + __popc(m_t & below), ta_long_gap{l, -1, w1 - tl, tl}, (u32)p << 1 | 1u);
+        if (room < cnt) {
+          if (lane == 0) base = atomicAdd(a.n_long, (u64)(cnt - room));
+          base = __shfl_sync(0xffffffffu, base, 0);
+        }
+        auto put = [&](u32 k, const ta_long_gap &x, u32 key) {
+          if (k < room) { s_list[at + k] = x; s_key[at + k] = key; }
+          else gap_append(a, (i64)(base + (k - room)), x, key);
+        };
+        if (lg) put((u32)__popc(m_g & below), ta_long_gap{l, (int32_t)p, P, g}, (u32)p << 1);
+        if (lt) put(n_g + (u32)__popc(m_t & below), ta_long_gap{l, -1, w1 - tl, tl}, (u32)p << 1 | 1u);
       }
     }
     pos = seg_end;
@@ -425,6 +444,12 @@ __device__ __forceinline__ void gaps_rows(const GapArgs &a, int rows) {
   }
   for (int64_t p = max(begin, vend) + lane; p < end; p += 32) a.gap_before[p] = 0;  // dropped records
   __syncthreads();
+  const u32 listed = min(s_n, (u32)GR_LIST);
+  if (listed) {  // the same in every thread
+    if (tid == 0) s_base = atomicAdd(a.n_long, (u64)listed);
+    __syncthreads();
+    for (u32 i = tid; i < listed; i += GP_THREADS) gap_append(a, (i64)(s_base + i), s_list[i], s_key[i]);
+  }
   for (int i = tid; i < GR_LANES * (TA_NBINS + 4); i += GP_THREADS) {
     const int li = i / (TA_NBINS + 4), k = i - li * (TA_NBINS + 4), ll = l0 + li;
     if (ll >= a.n_lanes) continue;
