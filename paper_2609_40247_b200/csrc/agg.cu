@@ -463,19 +463,24 @@ __device__ __forceinline__ void agg_rows_here(int G, const AggRowOut &o, u64 *to
   __shared__ u64 tmp[33];
   __shared__ u32 s_cell[AG_ROWS_HERE];
   const int g = threadIdx.x;
-  const u64 c = g < G ? __ldcg(&o.cnt[g]) : 0;
+  // everything a row takes is asked for together (one field after the other, each is a round trip to L2)
+  const bool in = g < G;
+  const u64 c = in ? __ldcg(&o.cnt[g]) : 0, sum = in ? __ldcg(&o.sum[g]) : 0, minc = in ? __ldcg(&o.minc[g]) : 0,
+            maxb = in ? __ldcg(&o.maxb[g]) : 0;
+  const int slot = in ? g / (int)o.R : 0, r = in ? g - slot * (int)o.R : 0;
+  const int32_t pid = in ? o.tt->pid_value[slot % o.n_pids] : 0;
+  const int32_t name = in && o.name_of ? o.name_of[r] : (int32_t)(o.min_name + r);
   u64 rows;
   const u64 row = block_scan_exclusive<OpAdd>(c ? 1ull : 0ull, OpAdd(), tmp, &rows);
   if (c) {
     s_cell[row] = (u32)g;
-    const int slot = g / (int)o.R, r = g - slot * (int)o.R;
     o.g_window[row] = slot / o.n_pids;
-    o.g_pid[row] = o.tt->pid_value[slot % o.n_pids];
-    o.g_name[row] = o.name_of ? o.name_of[r] : (int32_t)(o.min_name + r);
+    o.g_pid[row] = pid;
+    o.g_name[row] = name;
     o.g_count[row] = (int64_t)c;
-    o.g_sum[row] = (int64_t)__ldcg(&o.sum[g]);
-    o.g_min[row] = (int64_t)((~__ldcg(&o.minc[g])) ^ (1ull << 63));
-    o.g_max[row] = (int64_t)(__ldcg(&o.maxb[g]) ^ (1ull << 63));
+    o.g_sum[row] = (int64_t)sum;
+    o.g_min[row] = (int64_t)((~minc) ^ (1ull << 63));
+    o.g_max[row] = (int64_t)(maxb ^ (1ull << 63));
   }
   if (g == 0) {
     *total = rows;
@@ -484,9 +489,18 @@ __device__ __forceinline__ void agg_rows_here(int G, const AggRowOut &o, u64 *to
   __syncthreads();
   const uint4 *src = reinterpret_cast<const uint4 *>(o.hist);
   uint4 *dst = reinterpret_cast<uint4 *>(o.g_hist);
-  for (int i = g; i < (int)rows * (TA_NBINS / 4); i += AG_THREADS) {
-    const int r = i / (TA_NBINS / 4);
-    dst[i] = __ldcg(src + s_cell[r] * (TA_NBINS / 4) + (i - r * (TA_NBINS / 4)));
+  const int words = (int)rows * (TA_NBINS / 4);
+  constexpr int BATCH = 5;
+  for (int i0 = g; i0 < words; i0 += AG_THREADS * BATCH) {
+    uint4 v[BATCH];
+#pragma unroll
+    for (int k = 0; k < BATCH; k++) {
+      const int i = i0 + k * AG_THREADS, q = i / (TA_NBINS / 4);
+      if (i < words) v[k] = __ldcg(src + s_cell[q] * (TA_NBINS / 4) + (i - q * (TA_NBINS / 4)));
+    }
+#pragma unroll
+    for (int k = 0; k < BATCH; k++)
+      if (i0 + k * AG_THREADS < words) dst[i0 + k * AG_THREADS] = v[k];
   }
 }
 
