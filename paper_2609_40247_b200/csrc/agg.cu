@@ -31,7 +31,14 @@
 #define AG_THREADS 256
 #define AG_ITEMS 4
 #define AG_STEP (AG_THREADS * AG_ITEMS)
-#define AG_SLOTS 256
+// Slots of a CTA's table: 512 (a CTA of 8192 records of a window with 4096 symbols meets some 700, and what
+// finds no slot goes to memory by itself), 256 where a window has no more cells than that.
+#define AG_SLOTS_LOG2 9
+#define AG_SLOTS_FEW_LOG2 8
+#define AG_PROBES 8
+// bins a CTA counts on chip, 64 ns to 67 ms; others are rare and go to the row in memory
+#define AG_BIN0 6
+#define AG_BINS 20
 #define AG_ITEM (8 * AG_STEP)    // positions per CTA at most
 static_assert(AG_ITEM < (1 << 15), "a CTA's bins are 16 bits wide, the limbs of its sums 17 bits in a word");
 
@@ -142,14 +149,17 @@ __device__ __forceinline__ int64_t row_of(const AggArgs &a, int64_t g) {
   return (int64_t)a.rank[g >> 5] + __popc(a.bits[g >> 5] & ((1u << (g & 31)) - 1u));
 }
 
+// Values below 2^32 ns (four seconds; larger ones go to the row in memory), so that everything is native
+// 32-bit shared-memory atomics: 64-bit extremes are compare-and-swap loops, and with their 16 bytes and all
+// 40 bins a slot was twice as large.
+template <int LOG2>
 struct AggSmem {
-  int32_t key[AG_SLOTS];
-  // the sum in limbs of 17 bits (the third takes the rest, modulo 2^32): native 32-bit shared-memory
-  // atomics only, and one of them for a value below 131 us; the count is the sum of the bins
-  u32 sum[3][AG_SLOTS];
-  u64 minc[AG_SLOTS];
-  u64 maxb[AG_SLOTS];
-  uint16_t hist[AG_SLOTS][TA_NBINS];
+  static constexpr int SLOTS = 1 << LOG2;
+  int32_t key[SLOTS];
+  u32 sum[2][SLOTS];  // limbs of 17 and 15 bits: one atomic for a value below 131 us; the count is the sum of the bins
+  u32 minc[SLOTS];    // complement of the smallest
+  u32 max[SLOTS];
+  uint16_t hist[SLOTS][AG_BINS];
 };
 
 __device__ __forceinline__ void agg_global_add(const AggArgs &a, int64_t g, u64 cnt, u64 sum, u64 minc,
@@ -161,18 +171,22 @@ __device__ __forceinline__ void agg_global_add(const AggArgs &a, int64_t g, u64 
   atomicMax(&a.d_maxb[g], maxb);
 }
 
-__device__ __forceinline__ void agg_clear(AggSmem &s) {
+template <int LOG2>
+__device__ __forceinline__ void agg_clear(AggSmem<LOG2> &s) {
+  constexpr int AG_SLOTS = 1 << LOG2;
   for (int i = threadIdx.x; i < AG_SLOTS; i += AG_THREADS) {
     s.key[i] = -1;
-    s.sum[0][i] = s.sum[1][i] = s.sum[2][i] = 0;
+    s.sum[0][i] = s.sum[1][i] = 0;
     s.minc[i] = 0;
-    s.maxb[i] = 0;
+    s.max[i] = 0;
   }
   u32 *hw = reinterpret_cast<u32 *>(&s.hist[0][0]);
-  for (int i = threadIdx.x; i < AG_SLOTS * TA_NBINS / 2; i += AG_THREADS) hw[i] = 0;
+  for (int i = threadIdx.x; i < AG_SLOTS * AG_BINS / 2; i += AG_THREADS) hw[i] = 0;
 }
 
-__device__ __forceinline__ void agg_flush(const AggArgs &a, AggSmem &s) {
+template <int LOG2>
+__device__ __forceinline__ void agg_flush(const AggArgs &a, AggSmem<LOG2> &s) {
+  constexpr int AG_SLOTS = 1 << LOG2;
   __syncthreads();
   for (int i = threadIdx.x; i < AG_SLOTS; i += AG_THREADS) {
     int32_t k = s.key[i];
@@ -182,19 +196,19 @@ __device__ __forceinline__ void agg_flush(const AggArgs &a, AggSmem &s) {
       const u32 *hw = reinterpret_cast<const u32 *>(&s.hist[i][0]);
       u32 cnt = 0;
 #pragma unroll
-      for (int b = 0; b < TA_NBINS / 2; b++) cnt += (hw[b] & 0xFFFFu) + (hw[b] >> 16);
-      agg_global_add(a, k, cnt, (u64)s.sum[0][i] + ((u64)s.sum[1][i] << 17) + ((u64)s.sum[2][i] << 34),
-                     s.minc[i], s.maxb[i]);
+      for (int b = 0; b < AG_BINS / 2; b++) cnt += (hw[b] & 0xFFFFu) + (hw[b] >> 16);
+      agg_global_add(a, k, cnt, (u64)s.sum[0][i] + ((u64)s.sum[1][i] << 17), ~((u64)(u32)~s.minc[i] ^ (1ull << 63)),
+                     (u64)s.max[i] ^ (1ull << 63));
     }
   }
   __syncthreads();
   // histogram bins: one thread per (slot, bin).  Not unrolled: fetching the longer code costs a window of
   // 60 k records 1.5 us a call (24.5 and 23.7 us against 26.1 and 25.7), and saves 16.8 M two of 135
 #pragma unroll 1
-  for (int i = threadIdx.x; i < AG_SLOTS * TA_NBINS; i += AG_THREADS) {
-    const int sl = i / TA_NBINS, b = i - sl * TA_NBINS;
+  for (int i = threadIdx.x; i < AG_SLOTS * AG_BINS; i += AG_THREADS) {
+    const int sl = i / AG_BINS, b = i - sl * AG_BINS;
     const u32 c = s.hist[sl][b];
-    if (c) atomicAdd(&a.d_hist[(size_t)s.key[sl] * TA_NBINS + b], c);
+    if (c) atomicAdd(&a.d_hist[(size_t)s.key[sl] * TA_NBINS + AG_BIN0 + b], c);
   }
 }
 
@@ -302,9 +316,9 @@ __global__ void __launch_bounds__(AG_THREADS) k_agg_mark(AggArgs a) {
   }
 }
 
-template <bool TABLE>
+template <bool TABLE, int LOG2>
 __device__ __forceinline__ void agg_chunk(const AggArgs &a) {
-  __shared__ AggSmem s;
+  __shared__ AggSmem<LOG2> s;
   if (ta_failed(a.status)) return;
   LaneWalker lw(a.lane_off, a.n_lanes, a.n_valid, a.n_valid);
   {
@@ -339,31 +353,36 @@ __device__ __forceinline__ void agg_chunk(const AggArgs &a) {
         const int64_t g = (int64_t)a.lane_slot[lane] * a.R + name_rank_of<TABLE>(a, nm[j]);
         const u64 vb = (u64)v[j] ^ (1ull << 63);
         const int bin = log2_bin(v[j]);
-        u32 hsh = (u32)g * 2654435761u;
-        int slot = (int)(hsh >> 24) & (AG_SLOTS - 1);
+        const u32 hsh = (u32)g * 2654435761u;
+        int slot = (int)(hsh >> (32 - LOG2));
         bool placed = false;
-        for (int probe = 0; probe < 8; probe++) {
-          int32_t cur = s.key[slot];
-          if (cur == (int32_t)g) { placed = true; break; }
-          if (cur == -1) {
-            int32_t old = atomicCAS(&s.key[slot], -1, (int32_t)g);
-            if (old == -1 || old == (int32_t)g) { placed = true; break; }
+        if ((u64)v[j] < 1ull << 32)
+          for (int probe = 0; probe < AG_PROBES; probe++) {
+            const int32_t cur = s.key[slot];
+            if (cur == (int32_t)g) { placed = true; break; }
+            if (cur == -1) {
+              const int32_t old = atomicCAS(&s.key[slot], -1, (int32_t)g);
+              if (old == -1 || old == (int32_t)g) { placed = true; break; }
+            }
+            slot = (slot + 1) & ((1 << LOG2) - 1);
           }
-          slot = (slot + 1) & (AG_SLOTS - 1);
-        }
         if (placed) {
           // values are durations (>= 0), fewer than 2^15 adds per CTA: 2^15 x 2^17 fits a word
-          const u64 uv = (u64)v[j];
-          atomicAdd(&s.sum[0][slot], (u32)(uv & 0x1FFFF));
-          if (uv >> 17) atomicAdd(&s.sum[1][slot], (u32)((uv >> 17) & 0x1FFFF));
-          if (uv >> 34) atomicAdd(&s.sum[2][slot], (u32)(uv >> 34));
-          // 64-bit min/max in shared memory are compare-and-swap loops: skip them unless the
-          // value would actually move the extreme (rare once a slot has seen a few records)
-          if (~vb > s.minc[slot]) atomicMax(&s.minc[slot], ~vb);
-          if (vb > s.maxb[slot]) atomicMax(&s.maxb[slot], vb);
-          // 16-bit bins packed two per word
-          u32 *hw = reinterpret_cast<u32 *>(&s.hist[slot][0]) + (bin >> 1);
-          atomicAdd(hw, (bin & 1) ? 0x10000u : 1u);
+          const u32 uv = (u32)v[j];
+          atomicAdd(&s.sum[0][slot], uv & 0x1FFFFu);
+          if (uv >> 17) atomicAdd(&s.sum[1][slot], uv >> 17);
+          // an atomic only where the value would move the extreme (rare once a slot has seen a few records)
+          if (~uv > s.minc[slot]) atomicMax(&s.minc[slot], ~uv);
+          if (uv > s.max[slot]) atomicMax(&s.max[slot], uv);
+          const u32 b = (u32)(bin - AG_BIN0);
+          if (b < AG_BINS) {  // 16-bit bins packed two per word
+            u32 *hw = reinterpret_cast<u32 *>(&s.hist[slot][0]) + (b >> 1);
+            atomicAdd(hw, (b & 1) ? 0x10000u : 1u);
+          } else {
+            const int64_t row = row_of(a, g);
+            atomicAdd(&a.d_cnt[row], 1ull);
+            atomicAdd(&a.d_hist[(size_t)row * TA_NBINS + bin], 1u);
+          }
         } else {
           const int64_t row = row_of(a, g);
           agg_global_add(a, row, 1, (u64)v[j], ~vb, vb);
@@ -459,6 +478,7 @@ __global__ void __launch_bounds__(AC_THREADS) k_agg_rows(int64_t G, AggRowOut o,
 
 // The same for a few cells, by the last CTA of k_agg.
 #define AG_ROWS_HERE AG_THREADS
+static_assert(AG_ROWS_HERE <= 1 << AG_SLOTS_FEW_LOG2, "a slot for every cell");
 __device__ __forceinline__ void agg_rows_here(int G, const AggRowOut &o, u64 *total) {
   __shared__ u64 tmp[33];
   __shared__ u32 s_cell[AG_ROWS_HERE];
@@ -508,7 +528,7 @@ __device__ __forceinline__ void agg_rows_here(int G, const AggRowOut &o, u64 *to
 template <bool TABLE, bool TAIL>
 __global__ void __launch_bounds__(AG_THREADS, 6) k_agg(AggArgs a, int rows_here, AggRowOut o, u64 *total, Tail tail) {
   TA_PDL();
-  agg_chunk<TABLE>(a);
+  agg_chunk<TABLE, TAIL ? AG_SLOTS_FEW_LOG2 : AG_SLOTS_LOG2>(a);
   if (TAIL) run_tail(tail, [&] {
     if (rows_here && !ta_failed(a.status)) agg_rows_here(rows_here, o, total);
   });

@@ -71,6 +71,18 @@ def test_gather_takes_the_lanes_of_large_processes_together():
     both(ev, [0, n], [T0], [T0 + n * 5000], min_gap=50_000_000)
 
 
+@pytest.mark.parametrize("value", [0, 63, 64, 65, 131_071, 131_072, (1 << 26) - 1, 1 << 26, (1 << 32) - 1, 1 << 32, 1 << 36])
+@pytest.mark.parametrize("names", [1, 513, 3000])
+def test_aggregates_of_values_on_and_off_chip(value, names):
+    """Durations around the bins and the word a CTA keeps on chip, mixed with ordinary ones, for as many
+    symbols as it has rows and more."""
+    rng = np.random.default_rng(value % 1000 + names)
+    n = 9000
+    dur = np.where(rng.random(n) < 0.3, value, rng.integers(500, 10**6, n))
+    ev = _device(n, T0 + np.arange(n) * 1000, dur, name=rng.integers(0, names, n))
+    both(ev, [0, n], [T0], [T0 + 10**9])
+
+
 @pytest.mark.parametrize("n", [8192, 262_143, 262_145, 300_000])
 def test_long_gaps_ordered_by_one_cta_and_by_many(n):
     """Lists and bitmaps around the size one CTA puts in order: every record behind a long gap, and one
