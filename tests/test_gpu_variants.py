@@ -3,6 +3,7 @@ they can go wrong, bit for bit against the oracle."""
 import numpy as np
 import pytest
 
+from helpers import make_events
 from paper_2609_40247_b200.synth import EVENT_DTYPE
 from test_gpu_parity import both
 
@@ -81,6 +82,32 @@ def test_aggregates_of_values_on_and_off_chip(value, names):
     dur = np.where(rng.random(n) < 0.3, value, rng.integers(500, 10**6, n))
     ev = _device(n, T0 + np.arange(n) * 1000, dur, name=rng.integers(0, names, n))
     both(ev, [0, n], [T0], [T0 + 10**9])
+
+
+@pytest.mark.parametrize("pids,seqs,gap", [(2, 40, 1), (2, 20_000, 1), (64, 30, 1), (65, 30, 1), (8, 900, 1), (8, 50, 1000), (3, 1, 1)])
+@pytest.mark.parametrize("windows", [1, 3])
+def test_collectives_addressed_and_sorted(pids, seqs, gap, windows):
+    """Groups in a table of cells (dense numbers, up to 64 processes) and by sorting (sparse numbers, more
+    processes), with processes that take part twice or not at all, ties of the last arrival, a communicator
+    of unknown size."""
+    rng = np.random.default_rng(pids * 1000 + seqs + windows)
+    parts, off = [], [0]
+    for w in range(windows):
+        rows = []
+        for c in range(3):
+            for q in range(seqs):
+                t = T0 + w * 10**10 + (q * 3 + c) * 10**5
+                end = t + 90_000 + int(rng.integers(0, 100))
+                for p in range(pids):
+                    if rng.random() < 0.02:
+                        continue
+                    for _ in range(1 + (rng.random() < 0.02)):
+                        rows.append(("COLL", p - 1, 7, t + int(rng.integers(0, 4)) * 1000, end, 1000 + c, 5, q * gap - 3))
+        ev = make_events(rows)
+        parts.append(ev[rng.permutation(len(ev))])
+        off.append(off[-1] + len(ev))
+    both(np.concatenate(parts), off, [T0 + w * 10**10 for w in range(windows)],
+         [T0 + w * 10**10 + 5 * 10**9 for w in range(windows)], comm_sizes=[(1000, pids), (1001, pids + 1)])
 
 
 @pytest.mark.parametrize("n", [8192, 262_143, 262_145, 300_000])
