@@ -6,15 +6,17 @@
 //
 // The measure of a union of intervals taken in start order is
 //   sum_i max(0, e_i - max(s_i, P_i)),   P_i = max of the ends seen before i,
-// the same recurrence as the per-stream gap scan, so the step is: take the device
-// records of every process out of their stream lanes, sort them by (window, process,
-// ts_start) - keys that carry the record's index in their low bits when (process slot, time,
-// index) fit 64 bits, (key, index) pairs otherwise - and run ONE chained max-scan with three channels
-// (all records, computation, communication).  The measure of the intersection follows
+// the same recurrence as the per-stream gap scan, so the step is: bring the device
+// records of every process out of their stream lanes into one order by ts_start and run ONE
+// chained max-scan with three channels (all records, computation, communication).  The lanes of a process
+// are in that order already, so the records of a few lanes are merged (k_ov_merge); those of
+// many are sorted by (window, process, ts_start) - keys that carry the record's index in their low
+// bits when (process slot, time, index) fit 64 bits, (key, index) pairs otherwise.  The measure of the intersection follows
 // from the three unions: |A n B| = |A| + |B| - |A u B|.  Scanned values are tagged with
 // the (window, process) slot in their upper bits, as in the gap scan, so a prefix that
 // belongs to an earlier process is recognised and ignored.
-// HBM-bound on the sort: 8 B + 8 B (keys) or 12 B + 12 B (pairs) per device record and pass.
+// Merging reads 18 B and writes 16 B per device record; the sort moves 8 B + 8 B (keys) or 12 B + 12 B
+// (pairs) per device record and pass, and the scan then gathers.
 #include <climits>
 #include <cstring>
 
@@ -86,8 +88,136 @@ __global__ void __launch_bounds__(OV_THREADS) k_ov_keys(OvKeyArgs a) {
   }
 }
 
+// ---- merging the lanes of a process -------------------------------------------------------
+// A record's place among its process's is its place in its lane plus, for every other lane, the number
+// of records that begin before it.  A warp takes rows of 32 records of one lane; where it is in the other
+// lanes it keeps in cursors (thread j: lane j), a row looks at the next 32 starts behind each, and every
+// thread finds its place among those by five shuffles.
+#define OM_LANES 16   // device lanes of a process at most: a row costs some fifty instructions per lane
+#define OM_WARPS 8
+#define OM_FAR 0xFFFFFFF0ull
+struct OvMergeArgs {
+  int64_t n_valid, m;
+  int n_lanes;
+  const int64_t *ts, *te;
+  const int16_t *kind;
+  const int32_t *lane_off, *lane_slot, *lane_window, *lane_dom_end, *lane_dom_next, *lane_dev_base;
+  const int16_t *lane_domain;
+  const int64_t *t0, *t1;
+  ulonglong2 *out;  // per device record in order: (ts_start - t0) << 1 | not a kernel; slot << 40 | clipped end - t0
+  const int32_t *status;
+};
+__global__ void __launch_bounds__(OM_WARPS * 32) k_ov_merge(OvMergeArgs a, int rows) {
+  TA_PDL();
+  if (ta_failed(a.status)) return;
+  const int lane = threadIdx.x & 31;
+  const int64_t span = (int64_t)rows * 32;
+  const int64_t begin = ((int64_t)blockIdx.x * OM_WARPS + (threadIdx.x >> 5)) * span, end = min(begin + span, a.n_valid);
+  if (begin >= end) return;
+  int l = tile_lane_search(a.lane_off, a.n_lanes, begin);
+  for (int64_t pos = begin; pos < end;) {
+    if (a.lane_domain[l] != 1) {
+      pos = a.lane_dom_end[l];
+      l = a.lane_dom_next[l];
+      continue;
+    }
+    const int64_t off = a.lane_off[l], lane_end = a.lane_off[l + 1], seg_end = min(lane_end, end);
+    const int slot = a.lane_slot[l], w = a.lane_window[l];
+    const i64 w0 = a.t0[w], w1 = a.t1[w];
+    // the process's device lanes [f, f + k): neighbours of l
+    const int around = l - (OM_LANES - 1) + lane;  // threads 0 .. 2 * OM_LANES - 2
+    const bool same = lane < 2 * OM_LANES - 1 && around >= 0 && around < a.n_lanes && a.lane_slot[around] == slot &&
+                      a.lane_domain[around] == 1;
+    const u32 m = __ballot_sync(0xffffffffu, same);
+    const int f = l - (OM_LANES - 1) + (__ffs((int)m) - 1), k = __popc(m);
+    // records of lane f + lane that come in front of the segment's first
+    int64_t cur = 0, cur_end = 0;
+    int32_t cur_off = 0;
+    i64 s = 0, e = 0;
+    int kd = 0;
+    if (pos + lane < seg_end) { s = a.ts[pos + lane]; e = a.te[pos + lane]; kd = a.kind[pos + lane]; }
+    if (lane < k && f + lane != l) {
+      cur = cur_off = a.lane_off[f + lane];
+      cur_end = a.lane_off[f + lane + 1];
+      const i64 s0 = a.ts[pos];
+      int64_t hi = cur_end;
+      while (cur < hi) {
+        const int64_t mid = (cur + hi) >> 1;
+        const i64 v = a.ts[mid];
+        if (v < s0 || (v == s0 && f + lane < l)) cur = mid + 1;
+        else hi = mid;
+      }
+    }
+    const int64_t base = a.lane_dev_base[f];
+    for (; pos < seg_end; pos += 32) {
+      const int64_t p = pos + lane;
+      const bool in = p < seg_end;
+      const i64 cs = s, ce = min(e, w1);
+      const int ck = kd;
+      if (p + 32 < seg_end) { s = a.ts[p + 32]; e = a.te[p + 32]; kd = a.kind[p + 32]; }
+      int64_t rank = p - off;
+      const i64 s0 = __shfl_sync(0xffffffffu, cs, 0);
+      const int last = (int)min((int64_t)31, seg_end - pos - 1);
+      // starts relative to the row's first; rows that span four seconds and more are searched in memory
+      const u64 rel64 = in ? (u64)(cs - s0) : 0;
+      if (__all_sync(0xffffffffu, rel64 < OM_FAR)) {
+        for (int j = 0; j < k; j++) {
+          if (f + j == l) continue;
+          int64_t c = __shfl_sync(0xffffffffu, cur, j);
+          const int64_t c_end = __shfl_sync(0xffffffffu, cur_end, j);
+          // starts are coded from 1 on, 0: before the row's first.  Of records that begin together those
+          // of the lanes in front come first.
+          const u32 key = (u32)rel64 + (f + j < l ? 2u : 1u);
+          u32 found = 0;
+          for (;;) {
+            u32 v = 0xFFFFFFFFu;
+            if (c + lane < c_end) {
+              const i64 x = a.ts[c + lane] - s0;
+              v = x >= (i64)OM_FAR ? 0xFFFFFFFFu : x < 0 ? 0u : (u32)x + 1;
+            }
+            // how many of the 32 are below the key
+            u32 lo = 0;
+#pragma unroll
+            for (int step = 16; step > 0; step >>= 1) {
+              const u32 x = __shfl_sync(0xffffffffu, v, (int)(lo + step - 1));
+              if (x < key) lo += step;
+            }
+            const u32 top = __shfl_sync(0xffffffffu, v, 31);
+            if (lo == 31 && top < key) lo = 32;
+            found += lo;
+            const u32 gone = __shfl_sync(0xffffffffu, lo, last);
+            c += gone;
+            if (gone < 32) break;
+          }
+          rank += __shfl_sync(0xffffffffu, cur, j) - __shfl_sync(0xffffffffu, cur_off, j) + (int64_t)found;
+          if (lane == j) cur = c;
+        }
+      } else {
+        for (int j = 0; j < k; j++) {
+          if (f + j == l) continue;
+          int64_t lo = __shfl_sync(0xffffffffu, cur, j), hi = __shfl_sync(0xffffffffu, cur_end, j);
+          while (in && lo < hi) {
+            const int64_t mid = (lo + hi) >> 1;
+            const i64 v = a.ts[mid];
+            if (v < cs || (v == cs && f + j < l)) lo = mid + 1;
+            else hi = mid;
+          }
+          rank += lo - __shfl_sync(0xffffffffu, cur_off, j);
+          const int64_t c = __shfl_sync(0xffffffffu, lo, last);
+          if (lane == j) cur = c;
+        }
+      }
+      if (in && (u64)(base + rank) < (u64)a.m)
+        a.out[base + rank] = make_ulonglong2((u64)(cs - w0) << 1 | (ck != TA_KIND_KERNEL), (u64)slot << 40 | (u64)(ce - w0));
+    }
+    pos = seg_end;
+    if (lane_end <= end) l++;
+  }
+}
+
 struct OvScanArgs {
   int64_t m;          // device records
+  const ulonglong2 *merged;
   const u64 *keys;    // sorted
   const u32 *pos;     // sorted position: of element i (pairs), or of device record index c (packed keys)
   int idxbits;        // packed keys: low bits hold the device record index; 0 = pairs
@@ -101,6 +231,7 @@ struct OvScanArgs {
   int32_t *status;
 };
 
+template <bool MERGED>
 __global__ void __launch_bounds__(OV_THREADS, 3) k_ov_scan(OvScanArgs a) {
   TA_PDL();
   __shared__ u64 tmp[3][33];
@@ -115,34 +246,47 @@ __global__ void __launch_bounds__(OV_THREADS, 3) k_ov_scan(OvScanArgs a) {
   if (s_fail) return;  // the sort gave up: the keys name no records
   const int tile = s_tile;
   const int64_t i0 = (int64_t)tile * OV_TILE + (int64_t)tid * OV_ITEMS;
-  // keys and positions of the thread's eight records, then the gathers, all issued together
-  u64 key[OV_ITEMS];
-  u32 pp[OV_ITEMS];
-  i64 en[OV_ITEMS];
-  int16_t kd[OV_ITEMS];
-#pragma unroll
-  for (int j = 0; j < OV_ITEMS; j++) {
-    const bool in = i0 + j < a.m;
-    key[j] = in ? a.keys[i0 + j] : ~0ull;
-    if (a.idxbits) {
-      pp[j] = in ? a.pos[key[j] & ((1ull << a.idxbits) - 1)] : 0u;
-      key[j] >>= a.idxbits;
-    } else {
-      pp[j] = in ? a.pos[i0 + j] : 0u;
-    }
-  }
-#pragma unroll
-  for (int j = 0; j < OV_ITEMS; j++) {
-    const bool in = i0 + j < a.m;
-    en[j] = in ? a.te[pp[j]] : 0;
-    kd[j] = in ? a.kind[pp[j]] : (int16_t)-1;
-  }
-  const u64 tsmask = (1ull << a.tsbits) - 1;
   u64 val[OV_ITEMS];   // (slot + 1) << 40 | clipped end - window start
   i64 srel[OV_ITEMS];  // ts_start - window start
   int slot_of[OV_ITEMS];
+  int ch_of[OV_ITEMS]; // 1 computation, 2 communication
   u64 run[3] = {0, 0, 0};
-  {
+  if constexpr (MERGED) {
+    ulonglong2 x[OV_ITEMS];
+#pragma unroll
+    for (int j = 0; j < OV_ITEMS; j++) x[j] = i0 + j < a.m ? a.merged[i0 + j] : make_ulonglong2(0, ~0ull);
+#pragma unroll
+    for (int j = 0; j < OV_ITEMS; j++) {
+      const bool in = i0 + j < a.m;
+      slot_of[j] = in ? (int)(x[j].y >> 40) : -1;
+      srel[j] = (i64)(x[j].x >> 1);
+      ch_of[j] = 1 + (int)(x[j].x & 1u);
+      val[j] = in ? x[j].y + (1ull << 40) : 0;
+    }
+  } else {
+    // keys and positions of the thread's eight records, then the gathers, all issued together
+    u64 key[OV_ITEMS];
+    u32 pp[OV_ITEMS];
+    i64 en[OV_ITEMS];
+    int16_t kd[OV_ITEMS];
+#pragma unroll
+    for (int j = 0; j < OV_ITEMS; j++) {
+      const bool in = i0 + j < a.m;
+      key[j] = in ? a.keys[i0 + j] : ~0ull;
+      if (a.idxbits) {
+        pp[j] = in ? a.pos[key[j] & ((1ull << a.idxbits) - 1)] : 0u;
+        key[j] >>= a.idxbits;
+      } else {
+        pp[j] = in ? a.pos[i0 + j] : 0u;
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < OV_ITEMS; j++) {
+      const bool in = i0 + j < a.m;
+      en[j] = in ? a.te[pp[j]] : 0;
+      kd[j] = in ? a.kind[pp[j]] : (int16_t)-1;
+    }
+    const u64 tsmask = (1ull << a.tsbits) - 1;
     int wl = -1;
     i64 w0 = 0, w1 = 0;
 #pragma unroll
@@ -150,6 +294,7 @@ __global__ void __launch_bounds__(OV_THREADS, 3) k_ov_scan(OvScanArgs a) {
       val[j] = 0;
       srel[j] = 0;
       slot_of[j] = -1;
+      ch_of[j] = kd[j] == TA_KIND_KERNEL ? 1 : 2;
       if (kd[j] < 0) continue;
       const int slot = (int)(key[j] >> a.tsbits);
       const int w = slot / a.n_pids;
@@ -158,10 +303,13 @@ __global__ void __launch_bounds__(OV_THREADS, 3) k_ov_scan(OvScanArgs a) {
       slot_of[j] = slot;
       srel[j] = (i64)(key[j] & tsmask);
       val[j] = ((u64)(slot + 1) << 40) | (u64)ce;
-      run[0] = max(run[0], val[j]);
-      const int ch = kd[j] == TA_KIND_KERNEL ? 1 : 2;
-      run[ch] = max(run[ch], val[j]);
     }
+  }
+#pragma unroll
+  for (int j = 0; j < OV_ITEMS; j++) {
+    run[0] = max(run[0], val[j]);
+    if (ch_of[j] == 1) run[1] = max(run[1], val[j]);
+    else run[2] = max(run[2], val[j]);
   }
   u64 pre[3];
 #pragma unroll
@@ -188,7 +336,7 @@ __global__ void __launch_bounds__(OV_THREADS, 3) k_ov_scan(OvScanArgs a) {
     const int slot = slot_of[j];
     if (slot < 0) continue;
     const i64 ce = (i64)(val[j] & OV_LOW);
-    const int ch = kd[j] == TA_KIND_KERNEL ? 1 : 2;
+    const int ch = ch_of[j];
     u64 add[4] = {1, 0, 0, 0};
 #pragma unroll
     for (int c = 0; c < 3; c++) {
@@ -285,47 +433,65 @@ ta_status ta_run_overlap(ta_window *h, ta_overlap_result *out) {
   ro.d_exposed = ck.take<int64_t>(n_slots);
 
   const int64_t tiles = (m + OV_TILE - 1) / OV_TILE;
-  size_t tb = 3 * Carver::pad((size_t)m * 8) + 3 * Carver::pad((size_t)m * 4) + ta_sort_temp_bytes(m) +
-              3 * Carver::pad((size_t)tiles * 8) + Carver::pad(64) + Carver::pad((size_t)n_slots * 32) +
-              scan_temp_bytes(n_slots) + 512;
+  const bool merge = h->max_dev_lanes <= OM_LANES;
+  size_t tb = merge ? Carver::pad((size_t)m * 16) : 3 * Carver::pad((size_t)m * 8) + 3 * Carver::pad((size_t)m * 4) + ta_sort_temp_bytes(m);
+  tb += scan_temp_bytes(n_slots) + 512;
   void *tmpb = ta_dalloc(h, tb);
   if (!tmpb) return TA_ERR_OOM;
   Carver ct(tmpb);
-  u64 *k_in = ct.take<u64>(m), *k_scr = ct.take<u64>(m), *k_fin = ct.take<u64>(m);
-  u32 *v_in = ct.take<u32>(m), *v_scr = ct.take<u32>(m), *v_fin = ct.take<u32>(m);
-  char *zb = ct.base + ct.off;
+  ta_status zs;
+  void *zb = ta_zalloc(h, 3 * Carver::pad((size_t)tiles * 8) + Carver::pad(64) + Carver::pad((size_t)n_slots * 32), &zs);
+  if (!zb) return zs;
+  Carver cz(zb);
   OvScanArgs sa;
-  for (int c = 0; c < 3; c++) sa.st[c] = ct.take<u64>(tiles);
-  sa.counter = (u32 *)ct.take<u64>(8);
-  sa.acc = ct.take<u64>(n_slots * 4);
-  TA_CHECK_CUDA(h, cudaMemsetAsync(zb, 0, (ct.base + ct.off) - zb, st));
-  void *sort_tmp = ct.base + ct.off; ct.off += ta_sort_temp_bytes(m);
-  void *scan_mem = ct.base + ct.off;
-
-  OvKeyArgs ka;
-  ka.n = h->n; ka.n_valid = h->n_valid; ka.n_lanes = h->sorted.n_lanes;
-  ka.ts = h->sorted.ts_start;
-  ka.lane_off = h->sorted.lane_off; ka.lane_slot = h->d_lane_slot; ka.lane_window = h->sorted.lane_window;
-  ka.lane_dom_end = h->d_lane_dom_end; ka.lane_dev_base = h->d_lane_dev_base;
-  ka.lane_domain = h->sorted.lane_domain; ka.t0 = h->d_t0; ka.tsbits = tsbits; ka.idxbits = idxbits;
-  ka.keys = k_in; ka.pos = v_in; ka.status = h->d_status;
-  const int64_t key_tiles = (h->n_valid + OV_TILE - 1) / OV_TILE;
-  ta_launch(k_ov_keys, (unsigned)key_tiles, OV_THREADS, 0, st, ka);
-  TA_CHECK_CUDA(h, cudaGetLastError());
-  if (idxbits) {
-    TA_TRY(ta_radix_sort_keys(h, k_in, k_scr, k_fin, m,
-                              ta_make_plan(idxbits, idxbits + tsbits + slot_bits), nullptr, sort_tmp,
-                              true));  // coverage sums do not depend on the order of equal starts
-    sa.pos = v_in;
+  memset(&sa, 0, sizeof(sa));
+  for (int c = 0; c < 3; c++) sa.st[c] = cz.take<u64>(tiles);
+  sa.counter = (u32 *)cz.take<u64>(8);
+  sa.acc = cz.take<u64>(n_slots * 4);
+  if (merge) {
+    OvMergeArgs ma;
+    ma.n_valid = h->n_valid; ma.m = m; ma.n_lanes = h->sorted.n_lanes;
+    ma.ts = h->sorted.ts_start; ma.te = h->sorted.ts_end; ma.kind = h->sorted.kind;
+    ma.lane_off = h->sorted.lane_off; ma.lane_slot = h->d_lane_slot; ma.lane_window = h->sorted.lane_window;
+    ma.lane_dom_end = h->d_lane_dom_end; ma.lane_dom_next = h->d_lane_dom_next; ma.lane_dev_base = h->d_lane_dev_base;
+    ma.lane_domain = h->sorted.lane_domain; ma.t0 = h->d_t0; ma.t1 = h->d_t1;
+    ma.out = ct.take<ulonglong2>(m); ma.status = h->d_status;
+    sa.merged = ma.out;
+    // rows per warp: as many as leave the chip two rounds of warps; the search of the cursors is paid once per warp
+    int64_t rows = h->n_valid / 32 / (148 * 64);
+    rows = rows < 4 ? 4 : rows > 32 ? 32 : rows;
+    ta_launch(k_ov_merge, (unsigned)((h->n_valid + rows * OM_WARPS * 32 - 1) / (rows * OM_WARPS * 32)), OM_WARPS * 32, 0, st, ma, (int)rows);
   } else {
-    TA_TRY(ta_radix_sort_pairs(h, k_in, v_in, k_scr, v_scr, k_fin, v_fin, m,
-                               ta_make_plan(0, tsbits + slot_bits), nullptr, sort_tmp));
-    sa.pos = v_fin;
+    u64 *k_in = ct.take<u64>(m), *k_scr = ct.take<u64>(m), *k_fin = ct.take<u64>(m);
+    u32 *v_in = ct.take<u32>(m), *v_scr = ct.take<u32>(m), *v_fin = ct.take<u32>(m);
+    void *sort_tmp = ct.base + ct.off; ct.off += ta_sort_temp_bytes(m);
+    OvKeyArgs ka;
+    ka.n = h->n; ka.n_valid = h->n_valid; ka.n_lanes = h->sorted.n_lanes;
+    ka.ts = h->sorted.ts_start;
+    ka.lane_off = h->sorted.lane_off; ka.lane_slot = h->d_lane_slot; ka.lane_window = h->sorted.lane_window;
+    ka.lane_dom_end = h->d_lane_dom_end; ka.lane_dev_base = h->d_lane_dev_base;
+    ka.lane_domain = h->sorted.lane_domain; ka.t0 = h->d_t0; ka.tsbits = tsbits; ka.idxbits = idxbits;
+    ka.keys = k_in; ka.pos = v_in; ka.status = h->d_status;
+    const int64_t key_tiles = (h->n_valid + OV_TILE - 1) / OV_TILE;
+    ta_launch(k_ov_keys, (unsigned)key_tiles, OV_THREADS, 0, st, ka);
+    TA_CHECK_CUDA(h, cudaGetLastError());
+    if (idxbits) {
+      TA_TRY(ta_radix_sort_keys(h, k_in, k_scr, k_fin, m,
+                                ta_make_plan(idxbits, idxbits + tsbits + slot_bits), nullptr, sort_tmp,
+                                true));  // coverage sums do not depend on the order of equal starts
+      sa.pos = v_in;
+    } else {
+      TA_TRY(ta_radix_sort_pairs(h, k_in, v_in, k_scr, v_scr, k_fin, v_fin, m,
+                                 ta_make_plan(0, tsbits + slot_bits), nullptr, sort_tmp));
+      sa.pos = v_fin;
+    }
+    sa.keys = k_fin;
   }
-  sa.m = m; sa.keys = k_fin; sa.idxbits = idxbits;
+  void *scan_mem = ct.base + ct.off;
+  sa.m = m; sa.idxbits = idxbits;
   sa.te = h->sorted.ts_end; sa.kind = h->sorted.kind; sa.t0 = h->d_t0; sa.t1 = h->d_t1;
   sa.tsbits = tsbits; sa.n_pids = n_pids; sa.status = h->d_status;
-  ta_launch(k_ov_scan, (unsigned)tiles, OV_THREADS, 0, st, sa);
+  ta_launch(merge ? k_ov_scan<true> : k_ov_scan<false>, (unsigned)tiles, OV_THREADS, 0, st, sa);
   TA_CHECK_CUDA(h, cudaGetLastError());
 
   ro.acc = sa.acc; ro.tt = h->d_triples; ro.t0 = h->d_t0; ro.t1 = h->d_t1; ro.n_pids = n_pids;
@@ -339,6 +505,7 @@ ta_status ta_run_overlap(ta_window *h, ta_overlap_result *out) {
   TA_TRY((launch_scan<OpAdd, OvRowIn, OvRowOut>(h, n_slots, ri, ro, OpAdd(), s3, true)));
   TA_TRY(ta_sync_fetch(h));
   ta_dfree(h, tmpb);
+  ta_dfree(h, zb);
   if (words[ST_ERR]) return (ta_status)words[ST_ERR];
   out->n_rows = (int64_t)rows;
   out->d_window = ro.d_window; out->d_pid = ro.d_pid; out->d_n_events = ro.d_n_events;

@@ -110,6 +110,26 @@ def test_collectives_addressed_and_sorted(pids, seqs, gap, windows):
          [T0 + w * 10**10 + 5 * 10**9 for w in range(windows)], comm_sizes=[(1000, pids), (1001, pids + 1)])
 
 
+@pytest.mark.parametrize("lanes", [1, 2, 15, 16, 17, 33])
+@pytest.mark.parametrize("spread", [20, 10**6, 1 << 31])
+def test_overlap_of_merged_and_of_sorted_lanes(lanes, spread):
+    """Streams of a process merged (up to sixteen) and sorted: many equal starts, rows of 32 records that
+    span more than 2^32 ns, lanes of one record beside long ones, two processes and two windows."""
+    rng = np.random.default_rng(lanes * 7 + spread % 97)
+    parts, off = [], [0]
+    for w in range(2):
+        ev = []
+        for pid in (1, 2):
+            for s in range(lanes):
+                n = int(rng.integers(1, 4)) if s % 3 == 1 else int(rng.integers(100, 400))
+                starts = T0 + np.minimum(np.sort(rng.integers(0, max(1, spread * 100), n)), (1 << 38) - 1)
+                ev.append(_device(n, starts, rng.integers(0, spread * 3, n), pid=pid, stream=s, kind=rng.integers(3, 6, n)))
+        ev = np.concatenate(ev)
+        parts.append(ev[rng.permutation(len(ev))])
+        off.append(off[-1] + len(ev))
+    both(np.concatenate(parts), off, [T0] * 2, [T0 + (1 << 38)] * 2)
+
+
 @pytest.mark.parametrize("n", [8192, 262_143, 262_145, 300_000])
 def test_long_gaps_ordered_by_one_cta_and_by_many(n):
     """Lists and bitmaps around the size one CTA puts in order: every record behind a long gap, and one
