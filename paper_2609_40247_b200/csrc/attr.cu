@@ -34,9 +34,7 @@
 #define AT_THREADS 256
 #define AT_CAP 16
 #define AS_MINB 4
-// k_attr_ops: four records per thread keep it at 64 registers, four CTAs per SM (eight records and
-// three CTAs measured 0.12 ms slower on the 66.8 M record window: the kernel waits on gathers)
-#define AT_OPS_MINB 4
+#define AT_OPS_MINB 6
 
 struct AttrArgs {
   int64_t n, n_valid;
@@ -674,8 +672,6 @@ __global__ void __launch_bounds__(AS_WARPS * 32, AS_MINB) k_attr_resolve(AttrArg
 }
 
 // ---- device records inherit the operator of their launch ------------------------
-#define AT_OPS_ITEMS 4
-#define AT_OPS_TILE (AT_THREADS * AT_OPS_ITEMS)
 // adds kernels to an operator's row in memory (whose first / last are identities while it has none)
 __device__ __forceinline__ void attr_row_add(const AttrArgs &a, int32_t r, int cnt, i64 first, i64 last, i64 ns) {
   atomicAdd(&a.op_n[r], cnt);
@@ -697,113 +693,112 @@ __device__ __forceinline__ void attr_emit(ta_attr_summary *sm, const u64 *t) {
   if (t[1]) atomicAdd((u64 *)&sm->n_no_launch, t[1]);
   if (t[2]) atomicAdd((u64 *)&sm->n_no_op, t[2]);
 }
+// A warp takes `rows` x 32 positions, 32 records of ONE lane per row, AO_ROWS rows at a time with the launches
+// of the next ones on their way; no warp waits for another before the end.  (Four records per thread
+// of a CTA's tile, the lanes walked by every thread behind two block barriers: 243 us of 66.8 M records and 67 of 16.8 M, where this
+// takes 117 and 37; four CTAs per SM 124 and 37, eight 128 and 43; 8 rows 159 and 44, 32 rows 113 and 75.)
 // MULTI: some launch has more than one kernel; those kernels are added to their operator here.
+#define AO_ROWS 4
+#define AO_MAX 16
 template <bool MULTI>
-__device__ __forceinline__ void attr_ops(const AttrArgs &a) {
-  constexpr int IT = AT_OPS_ITEMS;
-  __shared__ u64 red[3][AT_THREADS / 32];
-  __shared__ int s_lane0, s_lane1;
+__device__ __forceinline__ void attr_ops(const AttrArgs &a, int rows) {
+  __shared__ u32 red[3][AT_THREADS / 32];
+  __shared__ int red_w[AT_THREADS / 32];
   if (ta_failed(a.status)) return;
   if (blockIdx.x < a.spill_blocks) {
     attr_spill(a);
     return;
   }
-  const int tid = threadIdx.x, lane = tid & 31;
-  const int64_t tile_start = (int64_t)(blockIdx.x - a.spill_blocks) * AT_OPS_TILE;
-  const int64_t p0 = tile_start + (int64_t)tid * IT;
-  if (tid == 0) { s_lane0 = -1; s_lane1 = -1; }
-  __syncthreads();
-  if (tid < 32 && tile_start < a.n_valid && a.n_lanes > 0) {
-    int l = tile_lane_search(a.lane_off, a.n_lanes, tile_start);
-    if (lane == 0) s_lane0 = l;
-  }
-  __syncthreads();
-  const int l0 = s_lane0;
-  // A tile of host lanes holds no device record: nothing to read, op_of = -1 throughout.
-  if (l0 >= 0 && span_outside_domain(a.lane_domain, a.lane_dom_end, l0,
-                                     min(tile_start + AT_OPS_TILE, a.n_valid), 1)) {
-    if (p0 + IT <= a.n) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t span = (int64_t)rows * 32;
+  const int64_t begin = min(((int64_t)(blockIdx.x - a.spill_blocks) * (AT_THREADS / 32) + warp) * span, a.n);
+  const int64_t end = min(begin + span, a.n), vend = min(end, a.n_valid);
+  u32 cnt[3] = {0, 0, 0};  // attributed, no launch, no operator
+  int cur = -1;            // window they are of
+  auto flush = [&]() {
+    u64 t[3];
 #pragma unroll
-      for (int q = 0; q < IT / 4; q++) *reinterpret_cast<int4 *>(a.op_of + p0 + 4 * q) = make_int4(-1, -1, -1, -1);
-    } else {
-      for (int j = 0; j < IT; j++)
-        if (p0 + j < a.n) a.op_of[p0 + j] = -1;
+    for (int k = 0; k < 3; k++) {
+      t[k] = __reduce_add_sync(0xffffffffu, cnt[k]);
+      cnt[k] = 0;
     }
-    return;
-  }
-  // kinds and launches of the thread's records are requested together (launch_of is -1 wherever
-  // the record is no matched kernel or copy, so the gather below needs no kind), then the parents
-  // of the launches: two rounds of memory latency instead of three
-  int16_t kd[IT];
-  loadn_i16<IT>(a.kind, p0, a.n, 0, kd);
-  int32_t lo[IT], op[IT];
-#pragma unroll
-  for (int j = 0; j < IT; j++) { lo[j] = -1; op[j] = -1; }
-  if (p0 + IT <= a.n) {
-#pragma unroll
-    for (int q = 0; q < IT / 4; q++) {
-      const int4 x = *reinterpret_cast<const int4 *>(a.launch_of + p0 + 4 * q);
-      lo[4 * q] = x.x; lo[4 * q + 1] = x.y; lo[4 * q + 2] = x.z; lo[4 * q + 3] = x.w;
+    if (lane == 0) attr_emit(&a.sum[cur], t);
+  };
+  int l = begin < vend ? tile_lane_search(a.lane_off, a.n_lanes, begin) : 0;
+  for (int64_t pos = begin; pos < vend;) {
+    if (a.lane_domain[l] != 1) {  // host lanes hold no device record
+      const int64_t stop = min((int64_t)a.lane_dom_end[l], vend);
+      for (int64_t p = pos + lane; p < stop; p += 32) a.op_of[p] = -1;
+      pos = stop;
+      l = a.lane_dom_next[l];
+      continue;
     }
-  } else {
+    const int64_t lane_end = a.lane_off[l + 1], e = min(lane_end, vend);
+    const int win = a.lane_window[l];
+    if (win != cur) {
+      if (cur >= 0) flush();
+      cur = win;
+    }
+    // (launch_of is -1 wherever the record is no matched kernel or copy: the gather needs no kind)
+    int lo[AO_ROWS], kd[AO_ROWS];
+    auto ask = [&](int64_t p) {
 #pragma unroll
-    for (int j = 0; j < IT; j++)
-      if (p0 + j < a.n) lo[j] = a.launch_of[p0 + j];
-  }
-#pragma unroll
-  for (int j = 0; j < IT; j++)
-    if (lo[j] >= 0) op[j] = a.parent[lo[j]];
-  unsigned pm = 0;
-#pragma unroll
-  for (int j = 0; j < IT; j++)
-    if (p0 + j < a.n_valid && (kd[j] == TA_KIND_KERNEL || kd[j] == TA_KIND_MEMCPY)) pm |= 1u << j;
-  u64 acc[3] = {0, 0, 0};  // attributed, no launch, no operator, for the thread's first window
-  int wm = -1;
-  {
-    int l = l0;
-    int64_t next_off = l >= 0 ? (int64_t)a.lane_off[l + 1] : LLONG_MAX;
-    int win = l >= 0 ? a.lane_window[l] : 0;
-#pragma unroll
-    for (int j = 0; j < IT; j++) {
-      if (!(pm & (1u << j))) { op[j] = -1; continue; }
-      const int64_t p = p0 + j;
-      if (p >= next_off) {
-        do { l++; next_off = a.lane_off[l + 1]; } while (p >= next_off);
-        win = a.lane_window[l];
+      for (int r = 0; r < AO_ROWS; r++) {
+        const int64_t q = p + 32 * r + lane;
+        lo[r] = -1;
+        kd[r] = 0;
+        if (q < e) { lo[r] = a.launch_of[q]; kd[r] = a.kind[q]; }
       }
-      if (MULTI && lo[j] >= 0 && op[j] >= 0 && a.kol[lo[j]] > 1) {
-        const i64 s = a.ts[p], e = a.te[p];
-        attr_row_add(a, op[j], 1, s, e, e - s);
+    };
+    ask(pos);
+    for (; pos < e; pos += 32 * AO_ROWS) {
+      int op[AO_ROWS], from[AO_ROWS];
+#pragma unroll
+      for (int r = 0; r < AO_ROWS; r++) {
+        from[r] = lo[r];
+        op[r] = lo[r] >= 0 ? a.parent[lo[r]] : -1;
+        cnt[1] += lo[r] < 0 && (kd[r] == TA_KIND_KERNEL || kd[r] == TA_KIND_MEMCPY);
       }
-      if (wm < 0) wm = win;
-      if (win == wm) {
-        acc[0] += lo[j] >= 0 && op[j] >= 0;
-        acc[1] += lo[j] < 0;
-        acc[2] += lo[j] >= 0 && op[j] < 0;
-      } else {
-        const u64 one[3] = {lo[j] >= 0 && op[j] >= 0, lo[j] < 0, lo[j] >= 0 && op[j] < 0};
-        attr_emit(&a.sum[win], one);
+      ask(pos + 32 * AO_ROWS);
+#pragma unroll
+      for (int r = 0; r < AO_ROWS; r++) {
+        const int64_t q = pos + 32 * r + lane;
+        if (q >= e) continue;
+        a.op_of[q] = op[r];
+        cnt[0] += op[r] >= 0;
+        cnt[2] += from[r] >= 0 && op[r] < 0;
+        if (MULTI && op[r] >= 0 && a.kol[from[r]] > 1) {
+          const i64 s = a.ts[q], t = a.te[q];
+          attr_row_add(a, op[r], 1, s, t, t - s);
+        }
       }
     }
-    const int64_t plast = min(tile_start + AT_OPS_TILE, a.n_valid) - 1;
-    if (plast >= p0 && plast < p0 + IT) {
-      while (plast >= next_off) { l++; next_off = a.lane_off[l + 1]; }
-      s_lane1 = l;
-    }
+    pos = e;
+    if (lane_end == e) l++;
   }
-  if (p0 + IT <= a.n) {
+  for (int64_t p = max(begin, vend) + lane; p < end; p += 32) a.op_of[p] = -1;  // dropped records
+  // the CTA's figures: one addition where its warps are in one window
 #pragma unroll
-    for (int q = 0; q < IT / 4; q++)
-      *reinterpret_cast<int4 *>(a.op_of + p0 + 4 * q) = make_int4(op[4 * q], op[4 * q + 1], op[4 * q + 2], op[4 * q + 3]);
-  } else {
-#pragma unroll
-    for (int j = 0; j < IT; j++)
-      if (p0 + j < a.n) a.op_of[p0 + j] = op[j];
+  for (int k = 0; k < 3; k++) {
+    const u32 t = __reduce_add_sync(0xffffffffu, cnt[k]);
+    if (lane == 0) red[k][warp] = t;
   }
+  if (lane == 0) red_w[warp] = cur;
   __syncthreads();
-  if (l0 < 0) return;
-  fold_by_window<3, 0, AT_THREADS / 32>(acc, wm, a.lane_window[l0], a.lane_window[s_lane1], red,
-                                        [&](int w, const u64 *t) { attr_emit(&a.sum[w], t); });
+  if (threadIdx.x != 0) return;
+  u64 t[3] = {0, 0, 0};
+  int w = -1;
+  for (int x = 0; x < AT_THREADS / 32; x++) {
+    if (red_w[x] < 0) continue;
+    if (red_w[x] != w) {
+      if (w >= 0) attr_emit(&a.sum[w], t);
+      w = red_w[x];
+      t[0] = t[1] = t[2] = 0;
+    }
+#pragma unroll
+    for (int k = 0; k < 3; k++) t[k] += red[k][x];
+  }
+  if (w >= 0) attr_emit(&a.sum[w], t);
 }
 
 // operators that were open at the end of their tile and got no kernels from anywhere: no identities
@@ -822,9 +817,9 @@ __global__ void __launch_bounds__(256) k_attr_finalize(AttrArgs a, Tail tail) {
 }
 // With a tail the last CTA does the work of k_attr_finalize (of a few tiles).
 template <bool MULTI, bool TAIL>
-__global__ void __launch_bounds__(AT_THREADS, AT_OPS_MINB) k_attr_ops(AttrArgs a, Tail tail) {
+__global__ void __launch_bounds__(AT_THREADS, AT_OPS_MINB) k_attr_ops(AttrArgs a, int rows, Tail tail) {
   TA_PDL();
-  attr_ops<MULTI>(a);
+  attr_ops<MULTI>(a, rows);
   if (TAIL) run_tail(tail, [&] {
     if (ta_failed(a.status)) return;
     for (int64_t i = threadIdx.x; i < a.n_tiles * AT_CAP; i += AT_THREADS) attr_finalize(a, i);
@@ -919,14 +914,17 @@ ta_status ta_run_attribute(ta_window *h, ta_attr_summary *out_summary) {
     // (a tile owes something to few operators of earlier ones, as a rule)
     const int64_t sb = (tiles * 2 + AT_THREADS - 1) / AT_THREADS;
     a.spill_blocks = (unsigned)(sb < 148 * 2 ? sb : 148 * 2);
-    const unsigned ob = a.spill_blocks + (unsigned)((n + AT_OPS_TILE - 1) / AT_OPS_TILE);
+    // rows per warp: 16, fewer while that would be less than two rounds of the 148 * 48 warps on the chip
+    int64_t rows = n / 32 / (148 * 96) / AO_ROWS * AO_ROWS;
+    rows = rows < AO_ROWS ? AO_ROWS : rows > AO_MAX ? AO_MAX : rows;
+    const unsigned ob = a.spill_blocks + (unsigned)((n + rows * AT_THREADS - 1) / (rows * AT_THREADS));
     // the last step in the last CTA of this one, for a few tiles (16 entries each)
     const int64_t entries = tiles * AT_CAP;
     Tail tail;
     if (entries <= 4 * AT_THREADS) tail = ta_tail(h, ob);
     auto ops = h->multi_launch ? (tail.m ? k_attr_ops<true, true> : k_attr_ops<true, false>)
                                : (tail.m ? k_attr_ops<false, true> : k_attr_ops<false, false>);
-    ta_launch(ops, ob, AT_THREADS, 0, st, a, tail);
+    ta_launch(ops, ob, AT_THREADS, 0, st, a, (int)rows, tail);
     if (tail.m == 0) {
       const int64_t fb = (entries + 255) / 256;
       ta_launch(k_attr_finalize, (unsigned)fb, 256, 0, st, a, ta_tail(h, fb));

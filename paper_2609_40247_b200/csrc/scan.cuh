@@ -247,45 +247,6 @@ static inline ta_status launch_compact_kind(ta_window *h, const int16_t *kind, i
   return TA_OK;
 }
 
-// Folds per-thread figures of a tile into per-window rows: v[0 .. NS) are sums, v[NS .. NS + NM)
-// maxima, w the window they belong to (-1: the thread has none), w_first / w_last the windows of
-// the tile's first and last record.  Lanes are short in a batch of many windows (a tile meets a
-// dozen of them), windows are not: a tile inside one window takes one block reduction and one
-// emit, a tile that meets several takes one emit per warp that lies inside one of them.
-// red: (NS + NM) x WARPS words of shared memory.  Called by all threads of the CTA.
-template <int NS, int NM, int WARPS, class Emit>
-__device__ __forceinline__ void fold_by_window(u64 (&v)[NS + NM], int w, int w_first, int w_last,
-                                               u64 (*red)[WARPS], Emit emit) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const u32 has = __ballot_sync(0xffffffffu, w >= 0);
-  const int w0 = has ? __shfl_sync(0xffffffffu, w, __ffs(has) - 1) : -1;
-  const bool one = w_first == w_last;
-  if (one || __all_sync(0xffffffffu, w < 0 || w == w0)) {
-    if (has || one) {
-#pragma unroll
-      for (int k = 0; k < NS; k++) v[k] = warp_reduce(w >= 0 ? v[k] : 0ull, OpAdd());
-#pragma unroll
-      for (int k = NS; k < NS + NM; k++) v[k] = warp_reduce(w >= 0 ? v[k] : 0ull, OpMax());
-    }
-    if (!one && has && lane == 0) emit(w0, v);
-  } else if (w >= 0) {
-    emit(w, v);
-  }
-  if (!one) return;  // the same in every thread of the CTA
-  if (lane == 0)
-#pragma unroll
-    for (int k = 0; k < NS + NM; k++) red[k][warp] = v[k];
-  __syncthreads();
-  if (warp == 0) {
-#pragma unroll
-    for (int k = 0; k < NS + NM; k++) {
-      const u64 x = lane < WARPS ? red[k][lane] : 0ull;
-      v[k] = k < NS ? warp_reduce(x, OpAdd()) : warp_reduce(x, OpMax());
-    }
-    if (lane == 0) emit(w_first, v);
-  }
-}
-
 // Walks the lane table along ascending sorted positions.
 struct LaneWalker {
   const int32_t *lane_off;
