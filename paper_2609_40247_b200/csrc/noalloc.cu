@@ -2,9 +2,11 @@
 // must not allocate device memory (see include/ta.h).  Same arithmetic as the
 // per-lane part of ta_stream_gaps; the sums, the tile descriptors of the chained
 // max-scan, the tile counter and the status word live in a fixed file-scope device
-// array instead of memory obtained from an allocator.  A call is one clearing of 128
-// bytes, one kernel, and a host that watches the page-locked row the kernel's last
-// tile writes (a second kernel where a lane's records do not end in ascending order).
+// array instead of memory obtained from an allocator.  A call is one kernel and a host
+// that watches the page-locked row the kernel's last tile writes (a second kernel where a
+// lane's records do not end in ascending order).  There are two sets of sums: the last tile
+// clears the set of the next call, which clears both itself when it does not follow a call that
+// was alone on the device and succeeded.
 // Bound by latency: 64 k records take 30 us through the Python binding, of which
 // the kernel is 5 (two clearings, a scan, two copies back and a synchronisation: 62).
 #include "ta_internal.cuh"
@@ -21,7 +23,7 @@
 #define NF_ITEMS 4
 #define NF_TILE (NA_THREADS * NF_ITEMS)
 
-// what the kernels of a call add up; cleared in front of each of them
+// what the kernels of a call add up
 struct NaSums {
   u64 busy, idle, n_gaps, max_gap;
   i64 first_start, last_end;
@@ -29,8 +31,9 @@ struct NaSums {
   u32 not_ascending;   // scan-free run: a record ends before the one in front of it
   int32_t status[ST_WORDS];
   u32 counter;         // tile tickets of the scan
-  u32 pad[3];
+  u32 pad[5];
 };
+static_assert(sizeof(NaSums) % 16 == 0, "cleared in words of 16 bytes");
 // the result in page-locked host memory, next to the device row the caller asked for
 struct NaHost {
   ta_lane_gaps row;
@@ -39,10 +42,12 @@ struct NaHost {
   volatile u32 seq;  // the call's number, written last
 };
 struct NaScratch {
-  NaSums sum;
+  NaSums sum[2];                // calls take them in turn
   u64 state[NA_MAX_TILES + 1];  // tile descriptors of the max-scan
   NaHost host;                  // stands in where no memory could be page-locked, and is copied
 };
+
+__device__ __forceinline__ NaSums *na_sums(NaScratch *sc, u32 seq) { return &sc->sum[seq & 1u]; }
 
 // Every device that loads the library holds this array until the process exits.
 // In host code `g_na_scratch` is only a stand-in for the symbol, not a device
@@ -62,7 +67,7 @@ __device__ __forceinline__ void na_finish(u64 sb, u64 si, u64 ng, u64 mg, int64_
   if (tid != 0) return;
   u64 a = 0, b = 0, c = 0, d = 0;
   for (int w = 0; w < NA_THREADS / 32; w++) { a += red[0][w]; b += red[1][w]; c += red[2][w]; d = d > red[3][w] ? d : red[3][w]; }
-  NaSums *s = &sc->sum;
+  NaSums *s = na_sums(sc, seq);
   if (a) atomicAdd(&s->busy, a);
   if (b) atomicAdd(&s->idle, b);
   if (c) atomicAdd(&s->n_gaps, c);
@@ -75,6 +80,9 @@ __device__ __forceinline__ void na_finish(u64 sb, u64 si, u64 ng, u64 mg, int64_
   r.n_gaps = (i64)__ldcg(&s->n_gaps); r.max_gap = (i64)__ldcg(&s->max_gap);
   r.first_start = __ldcg(&s->first_start); r.last_end = __ldcg(&s->last_end);
   *out = r;
+  uint4 *next = reinterpret_cast<uint4 *>(na_sums(sc, seq + 1));
+#pragma unroll
+  for (int k = 0; k < (int)(sizeof(NaSums) / 16); k++) next[k] = make_uint4(0, 0, 0, 0);
   host->row = r;
   host->err = __ldcg(&s->status[ST_ERR]);
   host->not_ascending = __ldcg(&s->not_ascending);
@@ -155,8 +163,9 @@ __global__ void __launch_bounds__(NA_THREADS) k_lane_gaps_ascending(const int64_
   }
   u64 sb = 0, si = 0, ng = 0, mg = 0;
   bool descends = false;
-  t.walk(pre, p0, n, W0, W1, gap_before, &sc->sum, &sb, &si, &ng, &mg, &descends);
-  if (descends) sc->sum.not_ascending = 1u;
+  NaSums *sum = na_sums(sc, seq);
+  t.walk(pre, p0, n, W0, W1, gap_before, sum, &sb, &si, &ng, &mg, &descends);
+  if (descends) sum->not_ascending = 1u;
   na_finish(sb, si, ng, mg, n, red, sc, out, host, seq);
 }
 
@@ -171,7 +180,8 @@ __global__ void __launch_bounds__(NA_THREADS) k_lane_gaps_noalloc(const int64_t 
   __shared__ u64 s_excl;
   __shared__ int s_tile, s_fail;
   const int tid = threadIdx.x;
-  if (tid == 0) s_tile = (int)atomicAdd(&sc->sum.counter, 1u);
+  NaSums *sum = na_sums(sc, seq);
+  if (tid == 0) s_tile = (int)atomicAdd(&sum->counter, 1u);
   __syncthreads();
   const int tile = s_tile;
   const int64_t p0 = (int64_t)tile * NA_TILE + (int64_t)tid * NA_ITEMS;
@@ -181,14 +191,14 @@ __global__ void __launch_bounds__(NA_THREADS) k_lane_gaps_noalloc(const int64_t 
   u64 thread_excl = block_scan_exclusive<OpMax>(t.run, OpMax(), tmp, &tile_max);
   if (tid < 32) {
     bool failed;
-    u64 e = tile_lookback<OpMax>(sc->state, tile, tile_max, OpMax(), sc->sum.status, &failed);
+    u64 e = tile_lookback<OpMax>(sc->state, tile, tile_max, OpMax(), sum->status, &failed);
     if (tid == 0) { s_excl = e; s_fail = failed ? 1 : 0; }
   }
   __syncthreads();
   u64 sb = 0, si = 0, ng = 0, mg = 0;
   if (!s_fail) {  // a bounded wait that gave up: the status word says so, the tile writes nothing
     bool descends = false;
-    t.walk(s_excl > thread_excl ? s_excl : thread_excl, p0, n, W0, W1, gap_before, &sc->sum, &sb, &si, &ng, &mg,
+    t.walk(s_excl > thread_excl ? s_excl : thread_excl, p0, n, W0, W1, gap_before, sum, &sb, &si, &ng, &mg,
            &descends);
   }
   na_finish(sb, si, ng, mg, n, red, sc, out, host, seq);
@@ -199,11 +209,15 @@ struct NaDevice {
   NaScratch *scratch;
   NaHost *host, *host_dev;
   u32 seq;
+  u32 cleared_for;  // number of the call whose set of sums is clear, 0 = none is known to be
+  int inside;       // calls in progress
+  bool met;         // ... and two of them have been at the same time since there was none
 };
 static std::mutex g_na_guard;
 static NaDevice g_na_device[64];
 
-static NaDevice *na_device(u32 *seq) {
+// clear: the call has to clear the sums itself.  na_leave ends what this begins.
+static NaDevice *na_enter(u32 *seq, bool *clear) {
   int dev = -1;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
   std::lock_guard<std::mutex> lock(g_na_guard);
@@ -226,9 +240,27 @@ static NaDevice *na_device(u32 *seq) {
     }
     d.scratch = (NaScratch *)p;
   }
-  *seq = ++d.seq;
+  if (++d.seq == 0) ++d.seq;
+  *seq = d.seq;
+  *clear = d.inside > 0 || d.cleared_for != d.seq;
+  d.cleared_for = 0;
+  if (d.inside++ > 0) d.met = true;
   return &d;
 }
+// Calls that met on the device race for its sums (the caller's mistake): none of them leaves a set to
+// the next.
+static void na_leave(NaDevice *d, u32 seq, bool ok) {
+  std::lock_guard<std::mutex> lock(g_na_guard);
+  if (ok && !d->met && d->seq == seq) d->cleared_for = seq + 1 ? seq + 1 : 0;
+  if (--d->inside == 0) d->met = false;
+}
+struct NaCall {
+  NaDevice *d;
+  u32 seq;
+  bool clear, ok;
+  NaCall() : d(nullptr), seq(0), clear(true), ok(false) { d = na_enter(&seq, &clear); }
+  ~NaCall() { if (d) na_leave(d, seq, ok); }
+};
 
 extern "C" ta_status ta_lane_gaps_noalloc_host(const int64_t *ts_start, const int64_t *ts_end, int64_t n,
                                                int64_t win_t0, int64_t win_t1, int64_t *gap_before,
@@ -240,9 +272,6 @@ extern "C" ta_status ta_lane_gaps_noalloc_host(const int64_t *ts_start, const in
   if (n > NA_MAX_RECORDS) return TA_ERR_TOO_LARGE;  // the fixed scratch array covers no more
   if ((uint64_t)win_t1 - (uint64_t)win_t0 >= (1ull << 40)) return TA_ERR_TOO_LARGE;
   cudaStream_t st = (cudaStream_t)cuda_stream;
-  u32 seq = 0;
-  NaDevice *d = na_device(&seq);
-  if (!d) return TA_ERR_CUDA;
   if (n == 0) {
     ta_lane_gaps empty = {0, win_t1 - win_t0, 0, 1, win_t1 - win_t0, 0, win_t0};
     if (cudaMemcpyAsync(lane_out, &empty, sizeof(empty), cudaMemcpyHostToDevice, st) != cudaSuccess)
@@ -250,10 +279,16 @@ extern "C" ta_status ta_lane_gaps_noalloc_host(const int64_t *ts_start, const in
     if (host_row) *host_row = empty;
     return cudaStreamSynchronize(st) == cudaSuccess ? TA_OK : TA_ERR_CUDA;
   }
+  NaCall call;
+  NaDevice *d = call.d;
+  if (!d) return TA_ERR_CUDA;
+  const u32 seq = call.seq;
   NaScratch *sc = d->scratch;
   for (int scan = 0; scan < 2; scan++) {
-    // the array keeps the previous call's contents: clear what must start at zero
-    if (cudaMemsetAsync(sc, 0, scan ? sizeof(NaScratch) : sizeof(NaSums), st) != cudaSuccess) return TA_ERR_CUDA;
+    // the array keeps the previous call's contents: clear what must start at zero (a fill and the wait for
+    // it in front of the kernel cost 1.4 us of 30)
+    if ((scan || call.clear) && cudaMemsetAsync(sc, 0, scan ? sizeof(NaScratch) : sizeof(sc->sum), st) != cudaSuccess)
+      return TA_ERR_CUDA;
     const int64_t tile = scan ? NA_TILE : NF_TILE;
     const unsigned tiles = (unsigned)((n + tile - 1) / tile);
     if (scan)
@@ -274,8 +309,10 @@ extern "C" ta_status ta_lane_gaps_noalloc_host(const int64_t *ts_start, const in
     std::atomic_thread_fence(std::memory_order_acquire);
     if (h->err) return (ta_status)h->err;
     if (host_row) *host_row = h->row;
-    if (!h->not_ascending) break;
-    if (scan) break;
+    if (scan || !h->not_ascending) {
+      call.ok = true;
+      break;
+    }
     if (d->host) d->host->seq = seq - 1;  // the scan announces itself again
   }
   return TA_OK;

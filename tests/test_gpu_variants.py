@@ -139,3 +139,36 @@ def test_long_gaps_ordered_by_one_cta_and_by_many(n):
         starts = T0 + np.cumsum(wait + 10)
         ev = _device(n, starts, 10, stream=np.arange(n) % 3)
         both(ev, [0, n], [T0], [T0 + (1 << 35)], min_gap=500 if every > 1 else 1)
+
+
+@pytest.mark.parametrize("order", ["aaaa", "adad", "ddaa", "aeda"])
+def test_noalloc_calls_that_follow_one_another(order):
+    """The sums of a call are cleared by the one in front of it: lanes that end their records in
+    ascending order (a) and that do not (d: the scan runs too), refused calls between them (e), of
+    different sizes."""
+    import torch
+    from paper_2609_40247_b200 import ta
+    rng = np.random.default_rng(11)
+    for i, kind in enumerate(order * 2):
+        n = (1, 1023, 1025, 70_001)[(i + len(order)) % 4]
+        start = T0 + np.cumsum(rng.integers(1, 1000, n))
+        end = start + (rng.integers(0, 300, n) if kind == "a" else 0)
+        if kind == "a":
+            end = np.maximum.accumulate(end)
+        elif n > 1:
+            end[n // 2] += 10**6
+        if kind == "e":
+            with pytest.raises(ta.TaError):
+                ta.lane_gaps_noalloc(torch.zeros(3, dtype=torch.int64, device="cuda"),
+                                     torch.zeros(3, dtype=torch.int64, device="cuda"), 5, 5)
+            continue
+        t1 = int(end.max()) + 12345
+        gap, row = ta.lane_gaps_noalloc(torch.from_numpy(start).cuda(), torch.from_numpy(end).cuda(), T0, t1)
+        before = np.concatenate([[T0], np.maximum.accumulate(end)[:-1]])
+        want = np.maximum(start - before, 0)
+        tail = t1 - int(end.max())
+        assert np.array_equal(gap.cpu().numpy(), want)
+        assert int(row["idle"]) == int(want.sum()) + tail and int(row["n_events"]) == n
+        assert int(row["busy"]) == int(np.maximum(end - np.maximum(start, before), 0).sum())
+        assert int(row["n_gaps"]) == int((want > 0).sum()) + 1 and int(row["last_end"]) == int(end.max())
+        assert int(row["max_gap"]) == max(int(want.max()), tail) and int(row["first_start"]) == int(start[0])
