@@ -78,9 +78,9 @@ struct CpArgs {
   int32_t *prev_node;   // host nodes: the node before it in its lane, or -1
   int32_t *head;        // nodes: head of the run (host: -1 = the run reaches the lane start)
   int32_t *entry;       // [position of a run head] where the walk entered that run, or -1
-  int32_t *entry_lane;  // [lane] the same for host runs that reach the lane start
+  int32_t *entry_lane;  // [lane] the same for host runs that reach the lane start: position + 1, 0 = none
   u64 *slot_host_te;    // per slot: latest end among host nodes (order-preserving code, 0 = none)
-  int32_t *slot_host_pos;  // per slot: highest position among the host nodes that end then
+  int32_t *slot_host_pos;  // per slot: highest position among the host nodes that end then (0 = none yet)
   u64 *st_a, *st_b;     // tile descriptors of the two scans
   u32 *counter;
   u32 *n_eff;           // length of the list below
@@ -233,6 +233,11 @@ __global__ void __launch_bounds__(CP_THREADS, 3) k_cp_classify(CpArgs a) {
   const int64_t tile_end = min(tile_start + CP_TILE, a.n_valid);
   const int64_t p0 = tile_start + (int64_t)threadIdx.x * CP_ITEMS;
   if (p0 >= tile_end) return;
+  {  // nothing entered, nothing listed (fills of their own cost two launches)
+    const int32_t none[CP_ITEMS] = {-1, -1, -1, -1, -1, -1, -1, -1};
+    store8_i32(a.entry, p0, a.n, none);
+    store8_i32(a.id_of, p0, a.n, none);
+  }
   int16_t kd[CP_ITEMS];
   i64 s[CP_ITEMS], e[CP_ITEMS];
   load8_i16(a.kind, p0, a.n, -1, kd);
@@ -489,7 +494,7 @@ __device__ __forceinline__ int32_t cp_follow(const CpArgs &a, int32_t d, bool re
   const int32_t l = a.launch_of[h];
   const int32_t e = a.head[l];
   if (e < 0) {
-    if (record) a.entry_lane[lane_of_pos(a.lane_off, a.n_lanes, l)] = l;
+    if (record) a.entry_lane[lane_of_pos(a.lane_off, a.n_lanes, l)] = l + 1;
     return -1;
   }
   if (record) a.entry[e] = l;
@@ -549,7 +554,7 @@ __device__ __forceinline__ int32_t cp_start_slot(const CpArgs &a, int64_t slot) 
     } else {       // the sink ran: the walk enters its host run at its START
       atomicAdd(&acc[6], (u64)(a.te[sink] - a.ts[sink]));
       const int32_t e = a.head[sink];
-      if (e < 0) a.entry_lane[lane_of_pos(a.lane_off, a.n_lanes, sink)] = sink;
+      if (e < 0) a.entry_lane[lane_of_pos(a.lane_off, a.n_lanes, sink)] = sink + 1;
       else {
         a.entry[e] = sink;
         first = a.id_of[e];
@@ -665,7 +670,7 @@ __global__ void __launch_bounds__(CP_THREADS) k_cp_mark(CpArgs a) {
       ln.to(p);
       bool on;
       if (cp_device(kd[j])) on = hd[j] >= 0 && a.entry[hd[j]] >= p;
-      else on = (hd[j] >= 0 ? a.entry[hd[j]] : a.entry_lane[ln.l]) >= p;
+      else on = (hd[j] >= 0 ? a.entry[hd[j]] : a.entry_lane[ln.l] - 1) >= p;
       const bool as_head = !cp_device(kd[j]) && a.entry[p] >= 0;  // a wait the walk left through its END
       if (!on && !as_head) continue;
       flags |= 1ull << (8 * j);
@@ -795,7 +800,8 @@ ta_status ta_run_critpath(ta_window *h, ta_critpath_result *out, ta_critpath_sum
   ro.p_reason = ck.take<int32_t>(n_slots);
   ro.p_begin = ck.take<int64_t>(n_slots); ro.p_end = ck.take<int64_t>(n_slots);
   ro.p_ns = ck.take<int64_t>(n_slots * 8);
-  TA_CHECK_CUDA(h, cudaMemsetAsync(on_path, 0, (size_t)nn, st));
+  // (k_cp_mark writes the column for all kept records)
+  if (nn > h->n_valid) TA_CHECK_CUDA(h, cudaMemsetAsync(on_path + h->n_valid, 0, (size_t)(nn - h->n_valid), st));
   out->on_path = on_path;
   if (h->n_valid <= 0) {
     h->d_on_path = on_path;
@@ -804,10 +810,7 @@ ta_status ta_run_critpath(ta_window *h, ta_critpath_result *out, ta_critpath_sum
 
   const int64_t tiles = (h->n_valid + CP_TILE - 1) / CP_TILE;
   const int64_t mm = m > 0 ? m : 1;
-  size_t tb = Carver::pad((size_t)nn) + 6 * Carver::pad((size_t)nn * 4) + Carver::pad((size_t)(n_lanes + 1) * 4) +
-              2 * Carver::pad((size_t)tiles * 8) + Carver::pad(64) + Carver::pad((size_t)n_slots * 8) +
-              Carver::pad((size_t)n_slots * 4) + Carver::pad((size_t)n_slots * CP_ACC * 8) +
-              scan_temp_bytes(n_slots) + CP_CHAIN_MAX * 5 + 1024;
+  size_t tb = Carver::pad((size_t)nn) + 6 * Carver::pad((size_t)nn * 4) + scan_temp_bytes(n_slots) + CP_CHAIN_MAX * 5 + 1024;
   void *tmpb = ta_dalloc(h, tb);
   if (!tmpb) return TA_ERR_OOM;
   Carver ct(tmpb);
@@ -820,22 +823,24 @@ ta_status ta_run_critpath(ta_window *h, ta_critpath_result *out, ta_critpath_sum
   a.eff_pos = ct.take<u32>(nn);
   int32_t *list_jump = ct.take<int32_t>(CP_CHAIN_MAX);
   uint8_t *list_mark = ct.take<uint8_t>(CP_CHAIN_MAX);
-  // zeroed block
-  char *zb = ct.base + ct.off;
-  a.st_a = ct.take<u64>(tiles); a.st_b = ct.take<u64>(tiles);
-  a.counter = (u32 *)ct.take<u64>(8);
-  a.n_eff = a.counter + 2;
-  a.not_ascending = a.counter + 3;
-  a.slot_host_te = ct.take<u64>(n_slots);
-  a.acc = ct.take<u64>(n_slots * CP_ACC);
-  const size_t zbytes = (ct.base + ct.off) - zb;
-  // block filled with -1
-  char *fb = ct.base + ct.off;
   a.entry = ct.take<int32_t>(nn);
   a.id_of = ct.take<int32_t>(nn);
-  a.entry_lane = ct.take<int32_t>(n_lanes + 1);
-  a.slot_host_pos = ct.take<int32_t>(n_slots);
-  const size_t fbytes = (ct.base + ct.off) - fb;
+  // zeroed block
+  const size_t zbytes = 2 * Carver::pad((size_t)tiles * 8) + Carver::pad(64) + Carver::pad((size_t)n_slots * 8) +
+                        Carver::pad((size_t)n_slots * CP_ACC * 8) + Carver::pad((size_t)(n_lanes + 1) * 4) +
+                        Carver::pad((size_t)n_slots * 4);
+  ta_status zs;
+  void *zb = ta_zalloc(h, zbytes, &zs);
+  if (!zb) return zs;
+  Carver cz(zb);
+  a.st_a = cz.take<u64>(tiles); a.st_b = cz.take<u64>(tiles);
+  a.counter = (u32 *)cz.take<u64>(8);
+  a.n_eff = a.counter + 2;
+  a.not_ascending = a.counter + 3;
+  a.slot_host_te = cz.take<u64>(n_slots);
+  a.acc = cz.take<u64>(n_slots * CP_ACC);
+  a.entry_lane = cz.take<int32_t>(n_lanes + 1);
+  a.slot_host_pos = cz.take<int32_t>(n_slots);
   void *scan_mem = ct.base + ct.off;
 
   a.n = n; a.n_valid = h->n_valid; a.m = m; a.n_lanes = n_lanes; a.n_pids = n_pids; a.n_slots = n_slots;
@@ -878,8 +883,7 @@ ta_status ta_run_critpath(ta_window *h, ta_critpath_result *out, ta_critpath_sum
   };
   for (int attempt = 0; attempt < 2; attempt++) {
     a.use_sort = attempt;
-    TA_CHECK_CUDA(h, cudaMemsetAsync(zb, 0, zbytes, st));
-    TA_CHECK_CUDA(h, cudaMemsetAsync(fb, 0xff, fbytes, st));
+    if (attempt) TA_CHECK_CUDA(h, cudaMemsetAsync(zb, 0, zbytes, st));
     if (a.use_sort && m > 0) {
       sortb = ta_dalloc(h, 3 * Carver::pad((size_t)mm * 8) + 3 * Carver::pad((size_t)mm * 4) + ta_sort_temp_bytes(mm) + 256);
       if (!sortb) return TA_ERR_OOM;
@@ -957,6 +961,7 @@ ta_status ta_run_critpath(ta_window *h, ta_critpath_result *out, ta_critpath_sum
   if (lb) ta_dfree(h, lb);
   if (sortb) ta_dfree(h, sortb);
   ta_dfree(h, tmpb);
+  ta_dfree(h, zb);
   if (words[ST_ERR]) return (ta_status)words[ST_ERR];
   for (int64_t s = 0; s < n_slots; s++) {
     const u64 *r = &hacc[(size_t)s * CP_ACC];
