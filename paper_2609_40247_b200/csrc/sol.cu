@@ -163,8 +163,11 @@ __device__ __forceinline__ void operator_sol(const SolArgs &a, int64_t n_tiles, 
       src[j] = -1;
       if (!(ops & (1u << j))) continue;
       const int64_t p = p0 + j;
-      if (a.op_n[p] > 0) top[j] = a.op_last[p] - a.op_first[p];
-      if (top[j] > 0) src[j] = a.perm[p];
+      // (requested together, whatever the count turns out to be: two rounds of latency less)
+      const int32_t cnt = a.op_n[p], at = a.perm[p];
+      const i64 first = a.op_first[p], last = a.op_last[p];
+      if (cnt > 0) top[j] = last - first;
+      if (top[j] > 0) src[j] = at;
     }
     double f[SO_ITEMS], b[SO_ITEMS];
 #pragma unroll
