@@ -671,7 +671,7 @@ class Window:
             else:
                 env.alloc, env.release, env.ctx = _torch_alloc, _torch_release, _place(dev, sptr)
                 if self.n <= CHUNK_RECORDS:
-                    self._take_chunk(env, stream)
+                    self._take_chunk(env, stream, 0 if on_device else nbytes)
         env.cuda_stream = sptr
         env.device = dev
         self.load_summary, summary_at = _rows(self.W, LOAD_SUM)
@@ -702,13 +702,14 @@ class Window:
 
         self._handle.callbacks = env.alloc, env.release = _ALLOC_T(_alloc), _RELEASE_T(_release)
 
-    def _take_chunk(self, env, stream):
+    def _take_chunk(self, env, stream, copy_bytes):
         import torch
         _views()
         h = self._handle
         if torch.are_deterministic_algorithms_enabled() and torch.utils.deterministic.fill_uninitialized_memory:
             return  # (torch would write all of it first; the allocator the pieces come from does not)
-        size = CHUNK_BYTES_FIXED + self.n * CHUNK_BYTES_PER_RECORD
+        # (records from the host have their copy in it as well: without it the later calls went back to torch)
+        size = CHUNK_BYTES_FIXED + self.n * CHUNK_BYTES_PER_RECORD + copy_bytes
         try:
             # (without a stream of the caller's choice the window is on the device's current one)
             device = torch.device("cuda", h.device)
