@@ -24,6 +24,8 @@
 
 #define BL_THREADS 256
 #define BL_TILE (BL_THREADS * 4)
+#define BL_TILE_FEW BL_THREADS  // tiles of windows that have up to BL_FEW of them
+#define BL_FEW 1024
 #define BL_LANES 64
 #define BL_GAPS 768    // gaps staged on chip: 18 KB, five CTAs per SM
 
@@ -167,18 +169,23 @@ __device__ __forceinline__ i64 gap_time_within(const Gaps &g, int64_t first, int
   return gap_time_before(g, first, ie, e) - gap_time_before(g, first, is, s);
 }
 
-// One tile of 1024 positions per CTA.  An operator's charge is two binary searches in each of its
+// One tile of 1024 (256) positions per CTA.  An operator's charge is two binary searches in each of its
 // process's streams, a chain of some thirty dependent reads per stream; the operators of the tile are
 // listed first and the (operator, stream) pairs are dealt out over the threads, so that no lane idles
 // beside a launch record and no thread walks eight streams one after the other (one thread per eight
 // records: 120 us for a prefill window of 250 k records, 195 us for 8 M decode records).  The gaps
 // that can matter to the tile are few, as a rule, and are searched on chip.
+// A window of few tiles leaves SMs idle and waits for a tile's rounds of pairs, ten of them in a prefill
+// window of 250 k records: a quarter of the tile takes 51 us to 25 there (half: 33).  Where there are tiles
+// enough the searches that a tile makes once count instead (8 M records 72 us, 88 by halves, 143 by
+// quarters); the line is where a call's last CTA still brings its results back.
+template <int TILE>
 __device__ __forceinline__ void blame_ops(const BlameArgs &a) {
   __shared__ int s_lane0, s_n, s_most;
-  __shared__ u64 s_sum[BL_TILE];
-  __shared__ uint16_t s_op[BL_TILE];
-  __shared__ int32_t s_dlo[BL_TILE];
-  __shared__ uint16_t s_dn[BL_TILE];
+  __shared__ u64 s_sum[TILE];
+  __shared__ uint16_t s_op[TILE];
+  __shared__ int32_t s_dlo[TILE];
+  __shared__ uint16_t s_dn[TILE];
   __shared__ int s_d0;                       // first device lane of the tile's operators, -1: there are several processes
   __shared__ i64 s_from, s_to;               // earliest start, latest end among them
   __shared__ int32_t s_lo[BL_LANES], s_hi[BL_LANES];  // per stream: the gaps that can matter to them
@@ -187,7 +194,7 @@ __device__ __forceinline__ void blame_ops(const BlameArgs &a) {
   __shared__ u64 s_pre[BL_GAPS];
   if (ta_failed(a.status)) return;
   const int tid = threadIdx.x;
-  const int64_t tile_start = (int64_t)blockIdx.x * BL_TILE;
+  const int64_t tile_start = (int64_t)blockIdx.x * TILE;
   if (tile_start >= a.n_valid) return;
   if (tid < 32) {
     const int l = tile_lane_search(a.lane_off, a.n_lanes, tile_start);
@@ -195,12 +202,12 @@ __device__ __forceinline__ void blame_ops(const BlameArgs &a) {
   }
   __syncthreads();
   const int l0 = s_lane0;
-  const int64_t tile_end = min(tile_start + BL_TILE, a.n_valid);
+  const int64_t tile_end = min(tile_start + TILE, a.n_valid);
   if (span_outside_domain(a.lane_domain, a.lane_dom_end, l0, tile_end, 0)) return;
   int l = l0, cur = -1, dlo = 0, dn = 0;
   i64 from = INT64_MAX, to = INT64_MIN;
   int64_t next_off = a.lane_off[l + 1];
-  constexpr int PER = BL_TILE / BL_THREADS;
+  constexpr int PER = TILE / BL_THREADS;
   bool op[PER];
 #pragma unroll
   for (int k = 0; k < PER; k++) {
@@ -225,7 +232,12 @@ __device__ __forceinline__ void blame_ops(const BlameArgs &a) {
         dlo = a.lane_dom_next[l];
         int dhi = dlo;
         const int slot = a.lane_slot[l];
-        while (dhi < a.n_lanes && a.lane_domain[dhi] == 1 && a.lane_slot[dhi] == slot) dhi++;
+        // slots do not descend: the run of device lanes is this process's if its last lane is (one
+        // lane after the other: 8 M records 82 us)
+        const int run_end = dlo < a.n_lanes ? a.lane_dom_next[dlo] : dlo;
+        if (run_end > dlo && a.lane_slot[run_end - 1] == slot) dhi = run_end;
+        else
+          while (dhi < run_end && a.lane_slot[dhi] == slot) dhi++;
         dn = dhi - dlo;
       }
     }
@@ -307,10 +319,10 @@ __device__ __forceinline__ void blame_ops(const BlameArgs &a) {
   for (int i = tid; i < ops; i += BL_THREADS)
     if (s_sum[i]) a.op_gap_ns[tile_start + s_op[i]] = (i64)s_sum[i];
 }
-template <bool TAIL>
+template <int TILE, bool TAIL>
 __global__ void __launch_bounds__(BL_THREADS) k_blame_ops(BlameArgs a, Tail tail) {
   TA_PDL();
-  blame_ops(a);
+  blame_ops<TILE>(a);
   if (TAIL) run_tail(tail);
 }
 
@@ -363,14 +375,18 @@ ta_status ta_run_blame(ta_window *h, const ta_gap_result *gaps, ta_blame_result 
   GapLenOut go{a.pre};
   TA_TRY((launch_scan<OpAdd, GapLenIn, GapLenOut>(h, m, gi, go, OpAdd(), s1)));
   ta_launch(k_blame_lanes, (unsigned)((L + 1 + 255) / 256), 256, 0, st, a);
-  const int64_t tiles = (h->n_valid + BL_TILE - 1) / BL_TILE;
+  const bool few = h->n_valid <= (int64_t)BL_TILE_FEW * BL_FEW;
+  const int tile = few ? BL_TILE_FEW : BL_TILE;
+  const int64_t tiles = (h->n_valid + tile - 1) / tile;
   std::vector<u64> hc((size_t)W * 4), hn((size_t)W * 4);
   int32_t words[ST_WORDS];
   TA_TRY(ta_queue_d2h(h, hc.data(), a.win_count, (size_t)W * 32));
   TA_TRY(ta_queue_d2h(h, hn.data(), a.win_ns, (size_t)W * 32));
   TA_TRY(ta_queue_d2h(h, words, h->d_status, sizeof(words)));
   const Tail tail = ta_tail(h, tiles);
-  ta_launch(tail.m ? k_blame_ops<true> : k_blame_ops<false>, (unsigned)tiles, BL_THREADS, 0, st, a, tail);
+  ta_launch(few ? (tail.m ? k_blame_ops<BL_TILE_FEW, true> : k_blame_ops<BL_TILE_FEW, false>)
+                : (tail.m ? k_blame_ops<BL_TILE, true> : k_blame_ops<BL_TILE, false>),
+            (unsigned)tiles, BL_THREADS, 0, st, a, tail);
   TA_CHECK_CUDA(h, cudaGetLastError());
   TA_TRY(ta_sync_fetch(h));
   ta_dfree(h, tmpb);

@@ -172,3 +172,32 @@ def test_noalloc_calls_that_follow_one_another(order):
         assert int(row["busy"]) == int(np.maximum(end - np.maximum(start, before), 0).sum())
         assert int(row["n_gaps"]) == int((want > 0).sum()) + 1 and int(row["last_end"]) == int(end.max())
         assert int(row["max_gap"]) == max(int(want.max()), tail) and int(row["first_start"]) == int(start[0])
+
+
+@pytest.mark.parametrize("n", [255, 257, 1023, 1025, 262_144, 262_145])
+def test_gaps_charged_to_operators_by_tiles_of_either_size(n):
+    """Operators four deep on two threads of one process, beside a process without streams and one with
+    nothing but streams: around the smaller tile, the larger one and the line between them."""
+    rng = np.random.default_rng(n)
+    k = np.arange(n)
+    ev = np.zeros(n, dtype=EVENT_DTYPE)
+    device = k % 5 > 2
+    ev["pid"] = np.where(k % 97 == 3, 2, np.where(k % 97 == 1, 1, 0))
+    device = np.where(ev["pid"] == 1, False, np.where(ev["pid"] == 2, True, device))
+    ev["stream"] = np.where(device, k // 5 % 7, k // 3 % 2)
+    ev["kind"] = np.where(device, 3, 2)
+    ev["ts_start"] = T0 + 100 + k * 20
+    ev["ts_end"] = ev["ts_start"] + np.where(device, rng.integers(1, 60, n), 10)
+    ev["corr_id"] = k
+    for pid in (0, 1):
+        for thread in (0, 1):
+            at = k[~device & (ev["pid"] == pid) & (ev["stream"] == thread)]
+            for level, every in enumerate((7200, 720, 36, 9)):
+                if len(at) < 2:
+                    continue
+                first = np.arange(0, len(at), every)  # of every block, one record later per level
+                last = np.minimum(first + every, len(at)) - 1
+                head = np.minimum(first + level, last)
+                ev["kind"][at[head]] = 0
+                ev["ts_end"][at[head]] = T0 + 100 + at[last] * 20 + 18 - 2 * level
+    both(ev[rng.permutation(n)], [0, n], [T0], [T0 + 10**9], min_gap=30)
