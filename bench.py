@@ -262,7 +262,7 @@ def touched_bytes_per_event(wl, radix_bytes_per_event):
                      + f_d * 6.0 + f_K * 4.0 + 4.0,   # inherit: kind, launch_of; parent; op_of
         "gaps": f_d * 16.0 + 8.0,
         "aggregate": f_d * 22.0 + f_h * 6.0 + f_o * 20.0,
-        "collectives": 8.0 + 2.0 + f_c * 84.0,        # waits cleared, kind; member, list entry twice, cell, wait
+        "collectives": 8.0 + 2.0 + f_c * 100.0,       # waits cleared, kind, compaction + pair sort + groups
     }
     return sum(parts.values()), parts
 
