@@ -89,129 +89,160 @@ __global__ void __launch_bounds__(OV_THREADS) k_ov_keys(OvKeyArgs a) {
 }
 
 // ---- merging the lanes of a process -------------------------------------------------------
-// A record's place among its process's is its place in its lane plus, for every other lane, the number
-// of records that begin before it.  A warp takes rows of 32 records of one lane; where it is in the other
-// lanes it keeps in cursors (thread j: lane j), a row looks at the next 32 starts behind each, and every
-// thread finds its place among those by five shuffles.
-#define OM_LANES 16   // device lanes of a process at most: a row costs some fifty instructions per lane
-#define OM_WARPS 8
-#define OM_FAR 0xFFFFFFF0ull
+// Every lane is cut at its first record and behind every OM_STEP records (lanes of a process at different
+// ones of them, so that lanes in step are cut at different times).  Where a cut falls in the other lanes is
+// searched, and the number of cuts in front of it is its place among the cuts of the process: between
+// neighbouring cuts there is at most OM_STEP records of each lane, whatever the lanes look like - a stream of
+// 300 copies beside one of 2 M kernels, streams that work in turns, lanes of one record.  A CTA merges the
+// records between two cuts on chip.
+// (Warps that took rows of 32 records of one lane, with cursors they moved through the others: 300 records
+// beside 2 M took 11.6 ms, because one warp went through all of them; 100 us so, and 226 by sorting.)
+// A record is searched in every other lane, so many lanes are sorted.  A call on even lanes of 4 M records
+// together, merged and sorted: 2 lanes 177 and 336 us, 8 264 and 340, 12 328 and 334, 14 368 and 335; of
+// 250 k: 2 lanes 55 and 97, 12 88 and 95, 16 98 and 96.
+#define OM_LANES 12    // device lanes of a process at most
+#define OM_STEP 256
+#define OM_THREADS 256
 struct OvMergeArgs {
-  int64_t n_valid, m;
-  int n_lanes;
+  int64_t m;
+  int n_lanes, n_cuts;  // places for cuts; not all are taken
+  int width;            // of a row of `cut`: device lanes of a process at most, and one
   const int64_t *ts, *te;
   const int16_t *kind;
-  const int32_t *lane_off, *lane_slot, *lane_window, *lane_dom_end, *lane_dom_next, *lane_dev_base;
+  const int32_t *lane_off, *lane_slot, *lane_window, *lane_dev_base;
   const int16_t *lane_domain;
   const int64_t *t0, *t1;
+  u32 *lanes;    // per place: (first lane of the process + 1) << 5 | its lanes, 0 = no cut
+  int32_t *cut;  // per place: device records in front of the cut, then where the lanes of the process go on
   ulonglong2 *out;  // per device record in order: (ts_start - t0) << 1 | not a kernel; slot << 40 | clipped end - t0
   const int32_t *status;
 };
-__global__ void __launch_bounds__(OM_WARPS * 32) k_ov_merge(OvMergeArgs a, int rows) {
+// First place of the cuts of lane l: a lane of c records has at most c / OM_STEP + 2.
+__device__ __forceinline__ int ov_cut_base(const OvMergeArgs &a, int l) { return a.lane_dev_base[l] / OM_STEP + 2 * l; }
+// Cuts in front of record c of a lane whose cuts are `phase` records early.
+__device__ __forceinline__ int ov_cuts_before(int c, int phase) { return c ? (c + phase + OM_STEP - 1) / OM_STEP : 0; }
+
+// A warp per cut.  It searches all lanes at the same time: of k lanes, 32 / k threads each, so many probes a round.
+__global__ void __launch_bounds__(OM_THREADS) k_ov_cuts(OvMergeArgs a) {
   TA_PDL();
   if (ta_failed(a.status)) return;
-  const int lane = threadIdx.x & 31;
-  const int64_t span = (int64_t)rows * 32;
-  const int64_t begin = ((int64_t)blockIdx.x * OM_WARPS + (threadIdx.x >> 5)) * span, end = min(begin + span, a.n_valid);
-  if (begin >= end) return;
-  int l = tile_lane_search(a.lane_off, a.n_lanes, begin);
-  for (int64_t pos = begin; pos < end;) {
-    if (a.lane_domain[l] != 1) {
-      pos = a.lane_dom_end[l];
-      l = a.lane_dom_next[l];
-      continue;
+  const int lane = threadIdx.x & 31, q = (int)(blockIdx.x * (OM_THREADS / 32) + (threadIdx.x >> 5));
+  if (q >= a.n_cuts) return;
+  int l = 0;
+  for (int hi = a.n_lanes; hi - l > 1;) {
+    const int step = (hi - l + 31) >> 5, at = l + lane * step;
+    const u32 b = __ballot_sync(0xffffffffu, at < hi && ov_cut_base(a, at) <= q);
+    l += (31 - __clz((int)b)) * step;  // (the first lane begins at 0: thread 0 always qualifies)
+    hi = min(hi, l + step);
+  }
+  if (a.lane_domain[l] != 1) return;
+  // the process's device lanes [f, f + k): neighbours of l
+  const int around = l - (OM_LANES - 1) + lane;  // threads 0 .. 2 * OM_LANES - 2
+  const bool same = lane < 2 * OM_LANES - 1 && around >= 0 && around < a.n_lanes && a.lane_slot[around] == a.lane_slot[l] &&
+                    a.lane_domain[around] == 1;
+  const u32 mask = __ballot_sync(0xffffffffu, same);
+  const int f = l - (OM_LANES - 1) + (__ffs((int)mask) - 1), k = __popc(mask);
+  if (k > a.width - 1) return;
+  const int s = q - ov_cut_base(a, l), own = l - f;
+  const int p = s ? s * OM_STEP - own * OM_STEP / k : 0;
+  const int off = a.lane_off[l];
+  if (p >= a.lane_off[l + 1] - off) return;
+  const i64 x = a.ts[off + p];
+  int probes = 32;
+  while (probes * k > 32) probes >>= 1;
+  const int j = lane / probes, t = lane & (probes - 1);
+  const bool in = j < k && t == 0;
+  int lo = 0, hi = 0, joff = 0;
+  if (j < k) {
+    joff = a.lane_off[f + j];
+    if (j == own) lo = hi = p;
+    else hi = a.lane_off[f + j + 1] - joff;
+  }
+  // records of lane f + j in front of the cut; of records that begin together those of the lanes in front come first
+  while (__any_sync(0xffffffffu, lo < hi)) {
+    const int w = (hi - lo + probes) / (probes + 1), at = lo + (t + 1) * w - 1;
+    bool front = false;
+    if (lo < hi && at < hi) {
+      const i64 v = a.ts[joff + at];
+      front = v < x || (v == x && j < own);
     }
-    const int64_t off = a.lane_off[l], lane_end = a.lane_off[l + 1], seg_end = min(lane_end, end);
-    const int slot = a.lane_slot[l], w = a.lane_window[l];
-    const i64 w0 = a.t0[w], w1 = a.t1[w];
-    // the process's device lanes [f, f + k): neighbours of l
-    const int around = l - (OM_LANES - 1) + lane;  // threads 0 .. 2 * OM_LANES - 2
-    const bool same = lane < 2 * OM_LANES - 1 && around >= 0 && around < a.n_lanes && a.lane_slot[around] == slot &&
-                      a.lane_domain[around] == 1;
-    const u32 m = __ballot_sync(0xffffffffu, same);
-    const int f = l - (OM_LANES - 1) + (__ffs((int)m) - 1), k = __popc(m);
-    // records of lane f + lane that come in front of the segment's first
-    int64_t cur = 0, cur_end = 0;
-    int32_t cur_off = 0;
-    i64 s = 0, e = 0;
-    int kd = 0;
-    if (pos + lane < seg_end) { s = a.ts[pos + lane]; e = a.te[pos + lane]; kd = a.kind[pos + lane]; }
-    if (lane < k && f + lane != l) {
-      cur = cur_off = a.lane_off[f + lane];
-      cur_end = a.lane_off[f + lane + 1];
-      const i64 s0 = a.ts[pos];
-      int64_t hi = cur_end;
-      while (cur < hi) {
-        const int64_t mid = (cur + hi) >> 1;
-        const i64 v = a.ts[mid];
-        if (v < s0 || (v == s0 && f + lane < l)) cur = mid + 1;
+    const u32 all = __ballot_sync(0xffffffffu, front);
+    const int n = __popc((all >> (j * probes)) & (0xffffffffu >> (32 - probes)));
+    if (lo < hi) {
+      lo += n * w;
+      if (n < probes) hi = min(hi, lo + w - 1);
+    }
+  }
+  const u32 place = __reduce_add_sync(0xffffffffu, in ? (u32)ov_cuts_before(lo, j * OM_STEP / k) : 0u) + (u32)ov_cut_base(a, f);
+  const u32 front = __reduce_add_sync(0xffffffffu, in ? (u32)lo : 0u);
+  if (place >= (u32)a.n_cuts) return;
+  int32_t *row = a.cut + (int64_t)place * a.width;
+  if (lane == 0) {
+    a.lanes[place] = (u32)(f + 1) << 5 | (u32)k;
+    row[0] = a.lane_dev_base[f] + (int32_t)front;
+  }
+  if (in) row[1 + j] = joff + lo;
+}
+
+__global__ void __launch_bounds__(OM_THREADS) k_ov_merge(OvMergeArgs a) {
+  TA_PDL();
+  extern __shared__ u64 ov_key[];  // ts_start - t0 of the records between the cuts, lane by lane
+  __shared__ int s_from[OM_LANES], s_pre[OM_LANES + 1];
+  if (ta_failed(a.status)) return;
+  const int i = (int)blockIdx.x, tid = (int)threadIdx.x;
+  const u32 lanes = a.lanes[i], next = i + 1 < a.n_cuts ? a.lanes[i + 1] : 0u;
+  if (!lanes) return;
+  const int f = (int)(lanes >> 5) - 1, k = (int)(lanes & 31u);
+  const int32_t *row = a.cut + (int64_t)i * a.width;
+  if (tid < 32) {
+    int from = 0, n = 0;
+    if (tid < k) {
+      from = row[1 + tid];
+      n = (next == lanes ? row[a.width + 1 + tid] : a.lane_off[f + tid + 1]) - from;
+      n = min(max(n, 0), OM_STEP);
+    }
+    const int upto = (int)warp_scan_inclusive((u64)n, OpAdd());
+    if (tid < k) {
+      s_from[tid] = from;
+      s_pre[tid + 1] = upto;
+    }
+    if (tid == 0) s_pre[0] = 0;
+  }
+  const int slot = a.lane_slot[f], w = a.lane_window[f];
+  const i64 w0 = a.t0[w], w1 = a.t1[w];
+  const int first = row[0];
+  __syncthreads();
+  const int total = s_pre[k];
+  auto lane_of = [&](int e) {
+    int j = 0;
+    while (e >= s_pre[j + 1]) j++;
+    return j;
+  };
+  for (int e = tid; e < total; e += OM_THREADS) {
+    const int j = lane_of(e);
+    ov_key[e] = (u64)(a.ts[s_from[j] + e - s_pre[j]] - w0);
+  }
+  __syncthreads();
+  for (int e = tid; e < total; e += OM_THREADS) {
+    const int own = lane_of(e), p = s_from[own] + e - s_pre[own];
+    const i64 te = a.te[p], end = te < w1 ? te : w1;
+    const int kd = a.kind[p];
+    const u64 x = ov_key[e];
+    int rank = e - s_pre[own];
+    for (int j = 0; j < k; j++) {
+      if (j == own) continue;
+      int lo = s_pre[j], hi = s_pre[j + 1];
+      const int at = lo;
+      const u64 y = x + (j < own ? 1 : 0);
+      while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if (ov_key[mid] < y) lo = mid + 1;
         else hi = mid;
       }
+      rank += lo - at;
     }
-    const int64_t base = a.lane_dev_base[f];
-    for (; pos < seg_end; pos += 32) {
-      const int64_t p = pos + lane;
-      const bool in = p < seg_end;
-      const i64 cs = s, ce = min(e, w1);
-      const int ck = kd;
-      if (p + 32 < seg_end) { s = a.ts[p + 32]; e = a.te[p + 32]; kd = a.kind[p + 32]; }
-      int64_t rank = p - off;
-      const i64 s0 = __shfl_sync(0xffffffffu, cs, 0);
-      const int last = (int)min((int64_t)31, seg_end - pos - 1);
-      // starts relative to the row's first; rows that span four seconds and more are searched in memory
-      const u64 rel64 = in ? (u64)(cs - s0) : 0;
-      if (__all_sync(0xffffffffu, rel64 < OM_FAR)) {
-        for (int j = 0; j < k; j++) {
-          if (f + j == l) continue;
-          int64_t c = __shfl_sync(0xffffffffu, cur, j);
-          const int64_t c_end = __shfl_sync(0xffffffffu, cur_end, j);
-          // starts are coded from 1 on, 0: before the row's first.  Of records that begin together those
-          // of the lanes in front come first.
-          const u32 key = (u32)rel64 + (f + j < l ? 2u : 1u);
-          u32 found = 0;
-          for (;;) {
-            u32 v = 0xFFFFFFFFu;
-            if (c + lane < c_end) {
-              const i64 x = a.ts[c + lane] - s0;
-              v = x >= (i64)OM_FAR ? 0xFFFFFFFFu : x < 0 ? 0u : (u32)x + 1;
-            }
-            // how many of the 32 are below the key
-            u32 lo = 0;
-#pragma unroll
-            for (int step = 16; step > 0; step >>= 1) {
-              const u32 x = __shfl_sync(0xffffffffu, v, (int)(lo + step - 1));
-              if (x < key) lo += step;
-            }
-            const u32 top = __shfl_sync(0xffffffffu, v, 31);
-            if (lo == 31 && top < key) lo = 32;
-            found += lo;
-            const u32 gone = __shfl_sync(0xffffffffu, lo, last);
-            c += gone;
-            if (gone < 32) break;
-          }
-          rank += __shfl_sync(0xffffffffu, cur, j) - __shfl_sync(0xffffffffu, cur_off, j) + (int64_t)found;
-          if (lane == j) cur = c;
-        }
-      } else {
-        for (int j = 0; j < k; j++) {
-          if (f + j == l) continue;
-          int64_t lo = __shfl_sync(0xffffffffu, cur, j), hi = __shfl_sync(0xffffffffu, cur_end, j);
-          while (in && lo < hi) {
-            const int64_t mid = (lo + hi) >> 1;
-            const i64 v = a.ts[mid];
-            if (v < cs || (v == cs && f + j < l)) lo = mid + 1;
-            else hi = mid;
-          }
-          rank += lo - __shfl_sync(0xffffffffu, cur_off, j);
-          const int64_t c = __shfl_sync(0xffffffffu, lo, last);
-          if (lane == j) cur = c;
-        }
-      }
-      if (in && (u64)(base + rank) < (u64)a.m)
-        a.out[base + rank] = make_ulonglong2((u64)(cs - w0) << 1 | (ck != TA_KIND_KERNEL), (u64)slot << 40 | (u64)(ce - w0));
-    }
-    pos = seg_end;
-    if (lane_end <= end) l++;
+    if ((u64)(first + rank) < (u64)a.m)
+      a.out[first + rank] = make_ulonglong2(x << 1 | (kd != TA_KIND_KERNEL), (u64)slot << 40 | (u64)(end - w0));
   }
 }
 
@@ -433,14 +464,19 @@ ta_status ta_run_overlap(ta_window *h, ta_overlap_result *out) {
   ro.d_exposed = ck.take<int64_t>(n_slots);
 
   const int64_t tiles = (m + OV_TILE - 1) / OV_TILE;
-  const bool merge = h->max_dev_lanes <= OM_LANES;
-  size_t tb = merge ? Carver::pad((size_t)m * 16) : 3 * Carver::pad((size_t)m * 8) + 3 * Carver::pad((size_t)m * 4) + ta_sort_temp_bytes(m);
+  // Merging takes no more memory than sorting: short lanes have cuts that are as large as their records.
+  const int width = h->max_dev_lanes + 1;
+  const int64_t n_cuts = m / OM_STEP + 2 * (int64_t)h->sorted.n_lanes + 1;
+  const bool merge = h->max_dev_lanes <= OM_LANES && n_cuts * (width + 1) * 4 <= 16 * m + (64 << 10);
+  size_t tb = merge ? Carver::pad((size_t)m * 16) + Carver::pad((size_t)n_cuts * width * 4)
+                    : 3 * Carver::pad((size_t)m * 8) + 3 * Carver::pad((size_t)m * 4) + ta_sort_temp_bytes(m);
   tb += scan_temp_bytes(n_slots) + 512;
   void *tmpb = ta_dalloc(h, tb);
   if (!tmpb) return TA_ERR_OOM;
   Carver ct(tmpb);
   ta_status zs;
-  void *zb = ta_zalloc(h, 3 * Carver::pad((size_t)tiles * 8) + Carver::pad(64) + Carver::pad((size_t)n_slots * 32), &zs);
+  void *zb = ta_zalloc(h, 3 * Carver::pad((size_t)tiles * 8) + Carver::pad(64) + Carver::pad((size_t)n_slots * 32) +
+                              (merge ? Carver::pad((size_t)n_cuts * 4) : 0), &zs);
   if (!zb) return zs;
   Carver cz(zb);
   OvScanArgs sa;
@@ -450,19 +486,17 @@ ta_status ta_run_overlap(ta_window *h, ta_overlap_result *out) {
   sa.acc = cz.take<u64>(n_slots * 4);
   if (merge) {
     OvMergeArgs ma;
-    ma.n_valid = h->n_valid; ma.m = m; ma.n_lanes = h->sorted.n_lanes;
+    ma.m = m; ma.n_lanes = h->sorted.n_lanes; ma.n_cuts = (int)n_cuts; ma.width = width;
     ma.ts = h->sorted.ts_start; ma.te = h->sorted.ts_end; ma.kind = h->sorted.kind;
     ma.lane_off = h->sorted.lane_off; ma.lane_slot = h->d_lane_slot; ma.lane_window = h->sorted.lane_window;
-    ma.lane_dom_end = h->d_lane_dom_end; ma.lane_dom_next = h->d_lane_dom_next; ma.lane_dev_base = h->d_lane_dev_base;
-    ma.lane_domain = h->sorted.lane_domain; ma.t0 = h->d_t0; ma.t1 = h->d_t1;
-    ma.out = ct.take<ulonglong2>(m); ma.status = h->d_status;
+    ma.lane_dev_base = h->d_lane_dev_base; ma.lane_domain = h->sorted.lane_domain; ma.t0 = h->d_t0; ma.t1 = h->d_t1;
+    ma.out = ct.take<ulonglong2>(m); ma.cut = ct.take<int32_t>(n_cuts * width); ma.lanes = cz.take<u32>(n_cuts);
+    ma.status = h->d_status;
     sa.merged = ma.out;
-    // rows per warp: as many as leave the chip two rounds of warps; the search of the cursors is paid once per warp
-    int64_t rows = h->n_valid / 32 / (148 * 64);
-    // (a row is a chain of a step per lane, so small windows take one per warp: 250 k records 34 us with four,
-    // 25 with two, 20 with one)
-    rows = rows < 1 ? 1 : rows > 32 ? 32 : rows;
-    ta_launch(k_ov_merge, (unsigned)((h->n_valid + rows * OM_WARPS * 32 - 1) / (rows * OM_WARPS * 32)), OM_WARPS * 32, 0, st, ma, (int)rows);
+    const size_t smem = (size_t)h->max_dev_lanes * OM_STEP * sizeof(u64);
+    static_assert(OM_LANES * OM_STEP * sizeof(u64) <= 40u << 10 && 2 * OM_LANES - 1 <= 32, "within what a kernel has without being asked");
+    ta_launch(k_ov_cuts, (unsigned)((n_cuts + OM_THREADS / 32 - 1) / (OM_THREADS / 32)), OM_THREADS, 0, st, ma);
+    ta_launch(k_ov_merge, (unsigned)n_cuts, OM_THREADS, smem, st, ma);
   } else {
     u64 *k_in = ct.take<u64>(m), *k_scr = ct.take<u64>(m), *k_fin = ct.take<u64>(m);
     u32 *v_in = ct.take<u32>(m), *v_scr = ct.take<u32>(m), *v_fin = ct.take<u32>(m);

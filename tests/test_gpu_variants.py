@@ -130,6 +130,64 @@ def test_overlap_of_merged_and_of_sorted_lanes(lanes, spread):
     both(np.concatenate(parts), off, [T0] * 2, [T0 + (1 << 38)] * 2)
 
 
+@pytest.mark.parametrize("lanes", [2, 3, 11, 12, 13])
+@pytest.mark.parametrize("filling", ["around a cut", "in step", "in turns", "one sparse", "one early"])
+def test_overlap_of_lanes_of_any_filling(lanes, filling):
+    """Lanes of a process as long as the parts they are merged in (one record less, one more), all at the same
+    times, one after the other, and a few records spread over or in front of full lanes; two processes."""
+    rng = np.random.default_rng(lanes)
+    parts = []
+    for pid in (1, 2):
+        for s in range(lanes):
+            n = {"around a cut": (255, 256, 257, 511, 513, 1, 0)[(s + pid) % 7], "in step": 1000, "in turns": 4 * 300,
+                 "one sparse": 40 if s == 1 else 9000, "one early": 300 if s == 1 else 5000}[filling]
+            k = np.arange(n)
+            starts = {"around a cut": np.sort(rng.integers(0, 300, n)), "in step": k * 100,
+                      "in turns": (k // 300 * lanes + s) * 300 + k % 300, "one sparse": np.sort(rng.integers(0, 10**6, n)),
+                      "one early": k // 3 if s == 1 else np.sort(rng.integers(80, 10**6, n))}[filling]
+            parts.append(_device(n, T0 + starts, rng.integers(0, 250, n), pid=pid, stream=s, kind=rng.integers(3, 6, n)))
+    ev = np.concatenate(parts)
+    ev["corr_id"][ev["kind"] == 5] = 7  # one communicator
+    both(ev[rng.permutation(len(ev))], [0, len(ev)], [T0], [T0 + 10**9])
+
+
+@pytest.mark.parametrize("pids,windows", [(90, 1), (1300, 4)])
+def test_overlap_of_many_lanes_of_one_record(pids, windows):
+    """Processes of a host lane and two streams of one or two records: merged where their cuts are few, sorted
+    where the table of cuts would be larger than what sorting takes."""
+    pid, window = np.tile(np.arange(pids), windows), np.repeat(np.arange(windows), pids)
+    t = T0 + window * 10**6
+    ev = np.concatenate([_device(len(t), t + 5 + s * 3 + pid % 7, 4 + pid % 5, pid=pid, stream=s, kind=kind)
+                         for s, kind in ((0, 1), (0, 3), (1, 4), (1, 3))])
+    ev = ev[np.argsort(np.tile(window, 4), kind="stable")]
+    both(ev, np.arange(windows + 1) * pids * 4, T0 + np.arange(windows) * 10**6, T0 + np.arange(1, windows + 1) * 10**6)
+
+
+def test_overlap_of_a_sparse_lane_beside_a_full_one_takes_no_longer():
+    """300 records spread over 2 M others: with the sparse lane walked record by record through the full one
+    the call took 60 times what it takes of two even lanes; both take about the same."""
+    import torch
+    from paper_2609_40247_b200 import ta
+    rng = np.random.default_rng(5)
+    times = []
+    for sizes in ((2_000_000, 300), (1_000_150, 1_000_150)):
+        ev = np.concatenate([_device(n, T0 + np.sort(rng.integers(0, 30 * 10**9, n)), 1000, stream=s)
+                             for s, n in enumerate(sizes)])
+        buf = torch.from_numpy(ev.view(np.uint8).reshape(-1)).cuda()
+        with ta.Window(buf, [0, len(ev)], [T0], [T0 + 30 * 10**9]) as w:
+            w.sort_timeline()
+            best = float("inf")
+            for _ in range(8):
+                a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+                a.record()
+                w.device_overlap()
+                b.record()
+                b.synchronize()
+                best = min(best, a.elapsed_time(b))
+        times.append(best)
+    assert times[0] < 5 * times[1], times
+
+
 @pytest.mark.parametrize("n", [8192, 262_143, 262_145, 300_000])
 def test_long_gaps_ordered_by_one_cta_and_by_many(n):
     """Lists and bitmaps around the size one CTA puts in order: every record behind a long gap, and one
