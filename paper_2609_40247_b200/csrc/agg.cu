@@ -36,9 +36,12 @@
 #define AG_SLOTS_LOG2 9
 #define AG_SLOTS_FEW_LOG2 8
 #define AG_PROBES 8
-// bins a CTA counts on chip, 64 ns to 67 ms; others are rare and go to the row in memory
+// bins a slot holds, 64 ns to 17 ms; the counts of others share a table
 #define AG_BIN0 6
-#define AG_BINS 20
+#define AG_BINS 18
+#define AG_ODD_LOG2 9
+// slots of values from 2^32 ns on (four seconds): there are few of them, but of few symbols
+#define AG_WIDE_LOG2 5
 #define AG_ITEM (8 * AG_STEP)    // positions per CTA at most
 static_assert(AG_ITEM < (1 << 15), "a CTA's bins are 16 bits wide, the limbs of its sums 17 bits in a word");
 
@@ -149,18 +152,26 @@ __device__ __forceinline__ int64_t row_of(const AggArgs &a, int64_t g) {
   return (int64_t)a.rank[g >> 5] + __popc(a.bits[g >> 5] & ((1u << (g & 31)) - 1u));
 }
 
-// Values below 2^32 ns (four seconds; larger ones go to the row in memory), so that everything is native
-// 32-bit shared-memory atomics: 64-bit extremes are compare-and-swap loops, and with their 16 bytes and all
-// 40 bins a slot was twice as large.
+// Values below 2^32 ns, so that everything is native 32-bit shared-memory atomics: 64-bit extremes are
+// compare-and-swap loops, and with their 16 bytes and all 40 bins a slot was twice as large.  What a CTA holds
+// is paid for by the cache: the two tables of 66.8 M records take 576 us, with bins from 1 ns on (38 KB a CTA) 646.
+// Bins and values that a slot has no room for are added up on chip all the same, in tables of their own: in
+// memory the records of no length or of a second meet at the rows of their symbols (a call on 8 M of 4 / 200
+// symbols, all of no length: 2570 / 1480 us, 93 / 189 so; one in twenty of 100 ms: 217 / 187 and 99 / 172).
 template <int LOG2>
 struct AggSmem {
-  static constexpr int SLOTS = 1 << LOG2;
+  static constexpr int SLOTS = 1 << LOG2, ODD = 1 << AG_ODD_LOG2, WIDE = 1 << AG_WIDE_LOG2;
   int32_t key[SLOTS];
   u32 sum[2][SLOTS];  // limbs of 17 and 15 bits: one atomic for a value below 131 us; the count is the sum of the bins
   u32 minc[SLOTS];    // complement of the smallest
   u32 max[SLOTS];
   uint16_t hist[SLOTS][AG_BINS];
+  u32 odd[ODD];       // (slot << 6 | bin) + 1 << 16 | count; slots from SLOTS on are wide ones
+  int32_t wide_key[WIDE];
+  u32 wide_sum[3][WIDE];  // limbs of 17 and 17 bits and the rest, modulo 2^32
+  u64 wide_minc[WIDE], wide_maxb[WIDE];
 };
+static_assert(((1 << AG_SLOTS_LOG2) + (1 << AG_WIDE_LOG2)) << 6 < 1 << 16 && AG_ITEM < 1 << 16, "a slot and a bin in 16 bits, a count in 16");
 
 __device__ __forceinline__ void agg_global_add(const AggArgs &a, int64_t g, u64 cnt, u64 sum, u64 minc,
                                                u64 maxb) {
@@ -173,26 +184,86 @@ __device__ __forceinline__ void agg_global_add(const AggArgs &a, int64_t g, u64 
 
 template <int LOG2>
 __device__ __forceinline__ void agg_clear(AggSmem<LOG2> &s) {
-  constexpr int AG_SLOTS = 1 << LOG2;
-  for (int i = threadIdx.x; i < AG_SLOTS; i += AG_THREADS) {
+  for (int i = threadIdx.x; i < s.SLOTS; i += AG_THREADS) {
     s.key[i] = -1;
     s.sum[0][i] = s.sum[1][i] = 0;
     s.minc[i] = 0;
     s.max[i] = 0;
   }
   u32 *hw = reinterpret_cast<u32 *>(&s.hist[0][0]);
-  for (int i = threadIdx.x; i < AG_SLOTS * AG_BINS / 2; i += AG_THREADS) hw[i] = 0;
+  for (int i = threadIdx.x; i < s.SLOTS * AG_BINS / 2; i += AG_THREADS) hw[i] = 0;
+  for (int i = threadIdx.x; i < s.ODD; i += AG_THREADS) s.odd[i] = 0;
+  for (int i = threadIdx.x; i < s.WIDE; i += AG_THREADS) {
+    s.wide_key[i] = -1;
+    s.wide_sum[0][i] = s.wide_sum[1][i] = s.wide_sum[2][i] = 0;
+    s.wide_minc[i] = s.wide_maxb[i] = 0;
+  }
+}
+
+// the slot of cell g, claimed if it has none; -1: no room near
+template <int LOG2>
+__device__ __forceinline__ int agg_slot(int32_t *key, int32_t g) {
+  int slot = (int)((u32)g * 2654435761u >> (32 - LOG2));
+  for (int probe = 0; probe < AG_PROBES; probe++) {
+    const int32_t cur = key[slot];
+    if (cur == g) return slot;
+    if (cur == -1) {
+      const int32_t old = atomicCAS(&key[slot], -1, g);
+      if (old == -1 || old == g) return slot;
+    }
+    slot = (slot + 1) & ((1 << LOG2) - 1);
+  }
+  return -1;
+}
+
+// What agg_chunk leaves: the bin of a value whose slot (at) does not hold it, and wide values (of cell at).
+template <int LOG2>
+__device__ __forceinline__ void agg_rest(const AggArgs &a, AggSmem<LOG2> &s, int32_t at, i64 v) {
+  const int bin = log2_bin(v);
+  int slot = at;
+  if (v >> 32) {
+    const u64 vb = (u64)v ^ (1ull << 63);
+    slot = v > 0 ? agg_slot<AG_WIDE_LOG2>(s.wide_key, at) : -1;
+    if (slot < 0) {
+      const int64_t row = row_of(a, at);
+      atomicAdd(&a.d_cnt[row], 1ull);
+      atomicAdd(&a.d_sum[row], (u64)v);
+      if (~vb > __ldcg(&a.d_minc[row])) atomicMax(&a.d_minc[row], ~vb);
+      if (vb > __ldcg(&a.d_maxb[row])) atomicMax(&a.d_maxb[row], vb);
+      atomicAdd(&a.d_hist[(size_t)row * TA_NBINS + bin], 1u);
+      return;
+    }
+    atomicAdd(&s.wide_sum[0][slot], (u32)v & 0x1FFFFu);
+    atomicAdd(&s.wide_sum[1][slot], (u32)(v >> 17) & 0x1FFFFu);
+    atomicAdd(&s.wide_sum[2][slot], (u32)(v >> 34));
+    if (~vb > s.wide_minc[slot]) atomicMax(&s.wide_minc[slot], ~vb);
+    if (vb > s.wide_maxb[slot]) atomicMax(&s.wide_maxb[slot], vb);
+    slot += s.SLOTS;
+  }
+  const u32 key = (u32)(slot << 6 | bin) + 1;
+  int o = (int)(key * 2654435761u >> (32 - AG_ODD_LOG2));
+  for (int probe = 0; probe < AG_PROBES; probe++) {
+    u32 cur = s.odd[o];
+    if (cur == 0) cur = atomicCAS(&s.odd[o], 0u, key << 16);
+    if (cur == 0 || cur >> 16 == key) {
+      atomicAdd(&s.odd[o], 1u);
+      return;
+    }
+    o = (o + 1) & (s.ODD - 1);
+  }
+  const int64_t row = row_of(a, slot < s.SLOTS ? s.key[slot] : s.wide_key[slot - s.SLOTS]);
+  atomicAdd(&a.d_cnt[row], 1ull);
+  atomicAdd(&a.d_hist[(size_t)row * TA_NBINS + bin], 1u);
 }
 
 template <int LOG2>
 __device__ __forceinline__ void agg_flush(const AggArgs &a, AggSmem<LOG2> &s) {
-  constexpr int AG_SLOTS = 1 << LOG2;
   __syncthreads();
-  for (int i = threadIdx.x; i < AG_SLOTS; i += AG_THREADS) {
+  for (int i = threadIdx.x; i < s.SLOTS; i += AG_THREADS) {
     int32_t k = s.key[i];
     if (k >= 0) {
       k = (int32_t)row_of(a, k);
-      s.key[i] = k;  // the row, for the bins below
+      s.key[i] = k;
       const u32 *hw = reinterpret_cast<const u32 *>(&s.hist[i][0]);
       u32 cnt = 0;
 #pragma unroll
@@ -201,11 +272,25 @@ __device__ __forceinline__ void agg_flush(const AggArgs &a, AggSmem<LOG2> &s) {
                      (u64)s.max[i] ^ (1ull << 63));
     }
   }
+  for (int i = threadIdx.x; i < s.WIDE; i += AG_THREADS)
+    if (s.wide_key[i] >= 0) {
+      const int32_t k = (int32_t)row_of(a, s.wide_key[i]);
+      s.wide_key[i] = k;
+      agg_global_add(a, k, 0, (u64)s.wide_sum[0][i] + ((u64)s.wide_sum[1][i] << 17) + ((u64)s.wide_sum[2][i] << 34),
+                     s.wide_minc[i], s.wide_maxb[i]);
+    }
   __syncthreads();
+  for (int i = threadIdx.x; i < s.ODD; i += AG_THREADS)
+    if (s.odd[i]) {
+      const u32 sb = (s.odd[i] >> 16) - 1, sl = sb >> 6, c = s.odd[i] & 0xFFFFu;
+      const int32_t row = sl < s.SLOTS ? s.key[sl] : s.wide_key[sl - s.SLOTS];
+      atomicAdd(&a.d_cnt[row], (u64)c);
+      atomicAdd(&a.d_hist[(size_t)row * TA_NBINS + (sb & 63u)], c);
+    }
   // histogram bins: one thread per (slot, bin).  Not unrolled: fetching the longer code costs a window of
   // 60 k records 1.5 us a call (24.5 and 23.7 us against 26.1 and 25.7), and saves 16.8 M two of 135
 #pragma unroll 1
-  for (int i = threadIdx.x; i < AG_SLOTS * AG_BINS; i += AG_THREADS) {
+  for (int i = threadIdx.x; i < s.SLOTS * AG_BINS; i += AG_THREADS) {
     const int sl = i / AG_BINS, b = i - sl * AG_BINS;
     const u32 c = s.hist[sl][b];
     if (c) atomicAdd(&a.d_hist[(size_t)s.key[sl] * TA_NBINS + AG_BIN0 + b], c);
@@ -346,48 +431,49 @@ __device__ __forceinline__ void agg_chunk(const AggArgs &a) {
       i64 v[AG_ITEMS];
       int32_t nm[AG_ITEMS];
       agg_select(a, p0, end, sel, v, nm);
+      u32 rest = 0;
 #pragma unroll
       for (int j = 0; j < AG_ITEMS; j++) {
         if (!sel[j]) continue;
         const int lane = lw.at(p0 + j);
-        const int64_t g = (int64_t)a.lane_slot[lane] * a.R + name_rank_of<TABLE>(a, nm[j]);
-        const u64 vb = (u64)v[j] ^ (1ull << 63);
-        const int bin = log2_bin(v[j]);
-        const u32 hsh = (u32)g * 2654435761u;
-        int slot = (int)(hsh >> (32 - LOG2));
-        bool placed = false;
-        if ((u64)v[j] < 1ull << 32)
-          for (int probe = 0; probe < AG_PROBES; probe++) {
-            const int32_t cur = s.key[slot];
-            if (cur == (int32_t)g) { placed = true; break; }
-            if (cur == -1) {
-              const int32_t old = atomicCAS(&s.key[slot], -1, (int32_t)g);
-              if (old == -1 || old == (int32_t)g) { placed = true; break; }
-            }
-            slot = (slot + 1) & ((1 << LOG2) - 1);
-          }
-        if (placed) {
-          // values are durations (>= 0), fewer than 2^15 adds per CTA: 2^15 x 2^17 fits a word
-          const u32 uv = (u32)v[j];
-          atomicAdd(&s.sum[0][slot], uv & 0x1FFFFu);
-          if (uv >> 17) atomicAdd(&s.sum[1][slot], uv >> 17);
-          // an atomic only where the value would move the extreme (rare once a slot has seen a few records)
-          if (~uv > s.minc[slot]) atomicMax(&s.minc[slot], ~uv);
-          if (uv > s.max[slot]) atomicMax(&s.max[slot], uv);
-          const u32 b = (u32)(bin - AG_BIN0);
-          if (b < AG_BINS) {  // 16-bit bins packed two per word
-            u32 *hw = reinterpret_cast<u32 *>(&s.hist[slot][0]) + (b >> 1);
-            atomicAdd(hw, (b & 1) ? 0x10000u : 1u);
-          } else {
-            const int64_t row = row_of(a, g);
-            atomicAdd(&a.d_cnt[row], 1ull);
-            atomicAdd(&a.d_hist[(size_t)row * TA_NBINS + bin], 1u);
-          }
-        } else {
+        const int32_t g = nm[j] = (int32_t)((int64_t)a.lane_slot[lane] * a.R + name_rank_of<TABLE>(a, nm[j]));
+        if ((u64)v[j] >> 32) {
+          rest |= 1u << j;
+          continue;
+        }
+        const int slot = agg_slot<LOG2>(s.key, g), bin = log2_bin(v[j]);
+        if (slot < 0) {
           const int64_t row = row_of(a, g);
+          const u64 vb = (u64)v[j] ^ (1ull << 63);
           agg_global_add(a, row, 1, (u64)v[j], ~vb, vb);
           atomicAdd(&a.d_hist[(size_t)row * TA_NBINS + bin], 1u);
+          continue;
         }
+        // values are durations (>= 0), fewer than 2^15 adds per CTA: 2^15 x 2^17 fits a word
+        const u32 uv = (u32)v[j];
+        atomicAdd(&s.sum[0][slot], uv & 0x1FFFFu);
+        if (uv >> 17) atomicAdd(&s.sum[1][slot], uv >> 17);
+        // an atomic only where the value would move the extreme (rare once a slot has seen a few records)
+        if (~uv > s.minc[slot]) atomicMax(&s.minc[slot], ~uv);
+        if (uv > s.max[slot]) atomicMax(&s.max[slot], uv);
+        const u32 b = (u32)(bin - AG_BIN0);
+        if (b < AG_BINS) {  // 16-bit bins packed two per word
+          u32 *hw = reinterpret_cast<u32 *>(&s.hist[slot][0]) + (b >> 1);
+          atomicAdd(hw, (b & 1) ? 0x10000u : 1u);
+        } else {
+          rest |= 1u << j;
+          nm[j] = slot;
+        }
+      }
+#pragma unroll 1
+      for (; rest; rest &= rest - 1) {
+        const int j = __ffs((int)rest) - 1;
+        i64 vj = v[0];
+        int32_t at = nm[0];
+#pragma unroll
+        for (int k = 1; k < AG_ITEMS; k++)
+          if (j == k) { vj = v[k]; at = nm[k]; }
+        agg_rest(a, s, at, vj);
       }
     }
   }

@@ -84,6 +84,42 @@ def test_aggregates_of_values_on_and_off_chip(value, names):
     both(ev, [0, n], [T0], [T0 + 10**9])
 
 
+@pytest.mark.parametrize("names", [1, 5, 31, 33, 300])
+def test_aggregates_of_values_of_every_size(names):
+    """Durations from nothing to minutes, so that most bins are in none of the slots a CTA keeps and more symbols
+    than it has room for have values beyond its words."""
+    rng = np.random.default_rng(names)
+    n = 30_000
+    dur = (2.0 ** rng.uniform(0, 37, n)).astype(np.int64) - 1
+    ev = _device(n, T0 + np.arange(n) * 1000, dur, name=rng.integers(0, names, n))
+    both(ev, [0, n], [T0], [T0 + 10**9], agg_masks=(56, 8))
+
+
+def test_aggregate_of_records_of_no_length_takes_no_longer():
+    """Values outside the bins of a slot were added up in memory, at the rows of a few symbols: 30 times as long."""
+    import torch
+    from paper_2609_40247_b200 import ta
+    n = 4_000_000
+    rng = np.random.default_rng(2)
+    times = {}
+    for label, dur in (("ordinary", rng.integers(1000, 10**6, n)), ("none", 0), ("one in twenty long", np.where(rng.random(n) < 0.05, 10**8, 9000))):
+        ev = _device(n, T0 + np.arange(n) * 5000, dur, name=np.arange(n) % 4)
+        ev["corr_id"] = -1
+        buf = torch.from_numpy(ev.view(np.uint8).reshape(-1)).cuda()
+        with ta.Window(buf, [0, n], [T0], [T0 + 30 * 10**9]) as w:
+            w.sort_timeline()
+            best = float("inf")
+            for _ in range(8):
+                a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+                a.record()
+                w.aggregate_ops(ta.DEVICE_KINDS, 0)
+                b.record()
+                b.synchronize()
+                best = min(best, a.elapsed_time(b))
+        times[label] = best
+    assert times["none"] < 4 * times["ordinary"] and times["one in twenty long"] < 4 * times["ordinary"], times
+
+
 @pytest.mark.parametrize("pids,seqs,gap", [(2, 40, 1), (2, 20_000, 1), (64, 30, 1), (65, 30, 1), (8, 900, 1), (8, 50, 1000), (3, 1, 1)])
 @pytest.mark.parametrize("windows", [1, 3])
 def test_collectives_addressed_and_sorted(pids, seqs, gap, windows):
