@@ -54,13 +54,12 @@ __device__ __forceinline__ u64 coll_rank(const CollCtx &c, i64 id, int32_t *stat
 __global__ void __launch_bounds__(256) k_coll_keys(CollCtx c, u64 *keys, int32_t *slot_of, int32_t *status) {
   TA_PDL();
   __shared__ int s_lane0;
-  if (ta_failed(status)) return;
   int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   // the compacted positions ascend: the lane of the CTA's first record is searched once, the
-  // others walk on from it
-  if (threadIdx.x == 0) s_lane0 = lane_of_pos(c.lane_off, c.n_lanes, c.posc[min(j, c.m - 1)]);
+  // others walk on from it.  One thread asks for the error word: another CTA may set it meanwhile (coll_rank).
+  if (threadIdx.x == 0) s_lane0 = ta_failed(status) ? -1 : lane_of_pos(c.lane_off, c.n_lanes, c.posc[min(j, c.m - 1)]);
   __syncthreads();
-  if (j >= c.m) return;
+  if (s_lane0 < 0 || j >= c.m) return;
   const u32 p = c.posc[j];
   const int lane = coll_lane(c, s_lane0, p);
   const u64 rank = coll_rank(c, c.corr[p], status), w = (u64)c.lane_window[lane];
@@ -209,10 +208,12 @@ __global__ void __launch_bounds__(CT_THREADS) k_coll_cells(CollCtx c, CollCells 
   TA_PDL();
   __shared__ u64 tmp[33];
   __shared__ uint16_t s_pos[CT_TILE];
-  __shared__ int s_lane0;
+  __shared__ int s_lane0, s_fail;
   __shared__ u32 s_base;
-  if (ta_failed(status)) return;
   const int tid = threadIdx.x;
+  // (one thread asks: another CTA may set the word meanwhile, and warps that leave would leave the others
+  // without their part of the list)
+  if (tid == 0) s_fail = ta_failed(status) ? 1 : 0;
   const int64_t start = (int64_t)blockIdx.x * CT_TILE, p0 = start + (int64_t)tid * CT_ITEMS;
   int16_t kd[CT_ITEMS];
 #pragma unroll
@@ -229,7 +230,7 @@ __global__ void __launch_bounds__(CT_THREADS) k_coll_cells(CollCtx c, CollCells 
   u64 total;
   u32 at = (u32)block_scan_exclusive<OpAdd>((u64)__popc(sel), OpAdd(), tmp, &total);
   const u32 count = (u32)total;
-  if (count == 0) return;
+  if (count == 0 || s_fail) return;  // (the scan has met a block barrier)
   for (; sel; sel &= sel - 1) s_pos[at++] = (uint16_t)(tid * CT_ITEMS + __ffs((int)sel) - 1);
   if (tid < 32) {
     const int l = tile_lane_search(c.lane_off, c.n_lanes, start);

@@ -268,3 +268,27 @@ def test_a_failed_handle_fails_the_aggregate_of_symbols_spread_wide():
             w.inject_device_error(TA_ERR_TIMEOUT)
             for mask in (ta.DEVICE_KINDS, 1, 63):
                 assert _status(lambda: w.aggregate_ops(mask, 0)) == TA_ERR_TIMEOUT
+
+
+@pytest.mark.parametrize("gap", [1, 1000])
+def test_communicators_the_load_has_not_seen(gap):
+    """Ids written over the sorted column after the sort are in no table: every CTA that meets one says so while
+    others begin, in the way by cells (gap 1) and by sorting (1000); the call fails and frees, and the
+    next analysis is unaffected."""
+    import torch
+    TA_ERR_OVERFLOW = 6
+    n = 1 << 18
+    k = np.arange(n)
+    ev = np.zeros(n, dtype=ta.EVENT_DTYPE)
+    ev["ts_start"], ev["pid"], ev["kind"] = 1000 + k, k % 4, np.where(k % 3 == 0, 5, 3)
+    ev["ts_end"] = ev["ts_start"] + 50
+    ev["corr_id"], ev["seq"] = np.where(k % 3 == 0, 77, -1), k // 12 * gap
+    buf = torch.from_numpy(ev.view(np.uint8).reshape(-1)).cuda()
+    with ta.Window(buf, [0, n], [0], [n + 2000]) as w:
+        s = w.sort_timeline()
+        s.tensor("corr_id").view(torch.int64)[::2] = 1234567
+        torch.cuda.synchronize()
+        assert _status(lambda: w.match_collectives([(77, 4)])) == TA_ERR_OVERFLOW
+        assert _status(w.correlate_launches) == TA_ERR_OVERFLOW
+    a = (ev, [0, n], [0], [n + 2000])
+    assert_same(run_oracle(*a, comm_sizes=[(77, 4)]), run_gpu(*a, comm_sizes=[(77, 4)]))
