@@ -183,7 +183,7 @@ struct CollCells {
   u64 *end;     // latest end
   u64 *who;     // processes seen
   u32 *more;    // members beyond the first of a process
-  u64 *done;    // latest start << 1 | the group counts
+  u64 *done;    // latest start << 1 | the group counts: written over `early`
   int64_t n;    // cells
   int64_t range, per_window;  // sequence numbers; cells of a window
   const int64_t *t0;
@@ -538,11 +538,26 @@ ta_status ta_run_collectives(ta_window *h, const ta_comm_size *sizes, int32_t n_
   u64 *r_maxw = cz.take<u64>(n_slots), *r_nstrag = cz.take<u64>(n_slots);
 
   // Cells of the direct table.  Up to two per member (and a few thousand): clearing and scanning them
-  // costs less than sorting the members.
+  // costs less than sorting the members.  They are taken from the handle's cleared pool; where it has no room
+  // (long windows) the way by cells must not ask for more memory than sorting does, 112 bytes per member and more.
   const unsigned __int128 all_cells = (unsigned __int128)h->W * (unsigned)h->n_comms * (uint64_t)(h->max_seq - h->min_seq + 1);
-  const bool cells = n_pids <= CC_MAX_PIDS && all_cells <= (unsigned __int128)(2 * m + 4096);
+  bool cells = n_pids <= CC_MAX_PIDS && all_cells <= (unsigned __int128)(2 * m + 4096);
   const int64_t nc = cells ? (int64_t)all_cells : 0;
+  const size_t cells_zeroed = 4 * Carver::pad((size_t)nc * 8) + Carver::pad((size_t)nc * 4) + Carver::pad(4) + scan_temp_bytes(nc);
+  const size_t cells_temp = Carver::pad((size_t)m * 8) + 3 * Carver::pad((size_t)m * 4) + Carver::pad((size_t)h->n_comms * 4) +
+                            scan_temp_bytes(n_slots) + 256;
+  const size_t sort_list = Carver::pad((size_t)m * 4) + scan_temp_bytes(n) + 256;
+  const size_t sort_temp = 3 * Carver::pad((size_t)m * 8) + 4 * Carver::pad((size_t)m * 4) + Carver::pad((size_t)(m + 1) * 4) +
+                           Carver::pad((size_t)h->n_comms * 4) + ta_sort_temp_bytes(m) + scan_temp_bytes(m) +
+                           scan_temp_bytes(n_slots) + 512;
+  auto rows_bytes = [](int64_t ng) { return 5 * Carver::pad((size_t)ng * 4) + 5 * Carver::pad((size_t)ng * 8) + 256; };
+  // Sorting: the group tables are sized by the number of groups when that is worth a round trip; while
+  // the bound "one group per COLL record" keeps them under 1 GiB they are sized by the bound
+  // and the count comes back with the call's one wait.
+  const bool bounded = (u64)m * 60 <= (1ull << 30);
   void *t1 = nullptr, *t2, *zc = nullptr;
+  if (cells && !(zc = ta_zpool(h, cells_zeroed)))
+    cells = cells_zeroed + cells_temp + rows_bytes(nc < m ? nc : m) <= sort_list + sort_temp + (bounded ? rows_bytes(m) : 0);
   u64 ng64 = 0;
   const u64 *ng_dev = nullptr;
   CollMemberArgs ma;
@@ -551,7 +566,7 @@ ta_status ta_run_collectives(ta_window *h, const ta_comm_size *sizes, int32_t n_
   memset(&ga, 0, sizeof(ga));
   void *scan3;
   auto rows_of = [&](int64_t ng) -> bool {
-    void *outb = ta_dalloc(h, 5 * Carver::pad((size_t)ng * 4) + 5 * Carver::pad((size_t)ng * 8) + 256);
+    void *outb = ta_dalloc(h, rows_bytes(ng));
     if (!outb) return false;
     Carver co(outb);
     ga.g_window = co.take<int32_t>(ng); ga.g_seq = co.take<int32_t>(ng); ga.g_n = co.take<int32_t>(ng);
@@ -563,22 +578,20 @@ ta_status ta_run_collectives(ta_window *h, const ta_comm_size *sizes, int32_t n_
   if (cells) {
     // 1. to 3. members to their cells; 4. the cells that are groups
     if (!rows_of(nc < m ? nc : m)) return TA_ERR_OOM;
-    t2 = ta_dalloc(h, Carver::pad((size_t)nc * 8) + Carver::pad((size_t)m * 8) + 3 * Carver::pad((size_t)m * 4) +
-                          Carver::pad((size_t)h->n_comms * 4) + scan_temp_bytes(n_slots) + 256);
+    t2 = ta_dalloc(h, cells_temp);
     if (!t2) return TA_ERR_OOM;
     Carver c2(t2);
     CollCells x;
-    x.done = c2.take<u64>(nc);
     CollList list;
     list.rel = c2.take<u64>(m);
     list.pos = c2.take<u32>(m); list.cell = c2.take<u32>(m);
     list.slot = c2.take<int32_t>(m);
     int32_t *d_expected = c2.take<int32_t>(h->n_comms);
     scan3 = c2.base + c2.off;
-    zc = ta_zalloc(h, 4 * Carver::pad((size_t)nc * 8) + Carver::pad((size_t)nc * 4) + Carver::pad(4) + scan_temp_bytes(nc), &zs);
-    if (!zc) return zs;
+    if (!zc && !(zc = ta_zalloc(h, cells_zeroed, &zs))) return zs;
     Carver cc(zc);
     x.late = cc.take<u64>(nc); x.early = cc.take<u64>(nc); x.end = cc.take<u64>(nc); x.who = cc.take<u64>(nc);
+    x.done = x.early;
     x.more = cc.take<u32>(nc);
     list.n = cc.take<u32>(1);
     ScanTemp s2;
@@ -601,8 +614,7 @@ ta_status ta_run_collectives(ta_window *h, const ta_comm_size *sizes, int32_t n_
     cx.posc = list.pos;
   } else {
     // 1. compaction
-    size_t t1b = Carver::pad((size_t)m * 4) + scan_temp_bytes(n) + 256;
-    t1 = ta_dalloc(h, t1b);
+    t1 = ta_dalloc(h, sort_list);
     if (!t1) return TA_ERR_OOM;
     Carver c1(t1);
     u32 *pos_all = c1.take<u32>(m);
@@ -612,10 +624,7 @@ ta_status ta_run_collectives(ta_window *h, const ta_comm_size *sizes, int32_t n_
     TA_TRY(launch_compact_kind(h, h->sorted.kind, h->n_valid, 1u << TA_KIND_COLL, pos_all, s1, reinterpret_cast<i64 *>(wait_ns), nn));
     cx.posc = pos_all;
     // 2. keys + sort; 3. heads
-    size_t t2b = 3 * Carver::pad((size_t)m * 8) + 4 * Carver::pad((size_t)m * 4) + Carver::pad((size_t)(m + 1) * 4) +
-                 Carver::pad((size_t)h->n_comms * 4) +
-                 ta_sort_temp_bytes(m) + scan_temp_bytes(m) + scan_temp_bytes(n_slots) + 512;
-    t2 = ta_dalloc(h, t2b);
+    t2 = ta_dalloc(h, sort_temp);
     if (!t2) return TA_ERR_OOM;
     Carver c2(t2);
     u64 *k_in = c2.take<u64>(m), *k_s = c2.take<u64>(m), *ks = c2.take<u64>(m);
@@ -636,10 +645,6 @@ ta_status ta_run_collectives(ta_window *h, const ta_comm_size *sizes, int32_t n_
     CollHeadIn hin{ks};
     CollHeadOut hout{cs, gid_of_c, gstart};
     TA_TRY((launch_scan<OpAdd, CollHeadIn, CollHeadOut>(h, m, hin, hout, OpAdd(), s2)));
-    // The group tables are sized by the number of groups when that is worth a round trip; while
-    // the bound "one group per COLL record" keeps them under 1 GiB they are sized by the bound
-    // and the count comes back with the call's one wait.
-    const bool bounded = (u64)m * 60 <= (1ull << 30);
     if (!bounded) {
       TA_TRY(ta_queue_d2h(h, &ng64, s2.total, 8));
       TA_TRY(ta_sync_fetch(h));

@@ -146,6 +146,33 @@ def test_collectives_addressed_and_sorted(pids, seqs, gap, windows):
          [T0 + w * 10**10 + 5 * 10**9 for w in range(windows)], comm_sizes=[(1000, pids), (1001, pids + 1)])
 
 
+@pytest.mark.parametrize("pids,gap", [(1, 1), (1, 2), (2, 3), (8, 1), (8, 9), (4, 100)])
+def test_collectives_take_no_more_memory_by_cells_than_by_sorting(pids, gap):
+    """Nothing but collectives, so that the handle's pool has no room for the cells: from one cell per group and
+    eight members to two cells per member, and to numbers too sparse for cells."""
+    import torch
+    from paper_2609_40247_b200 import ta
+    n = 160_000
+    k = np.arange(n)
+    ev = _device(n, T0 + k // pids * 500 + k % 7, 100, pid=k % pids, kind=5)
+    ev["corr_id"], ev["seq"] = 3, k // pids * gap
+    both(ev, [0, n], [T0], [T0 + 10**9], comm_sizes=[(3, pids)])
+    buf = torch.from_numpy(ev.view(np.uint8).reshape(-1)).cuda()
+    dev, stream = buf.device.index, torch.cuda.current_stream().cuda_stream
+    asked = []
+
+    def alloc(nbytes):
+        asked.append(nbytes)
+        return torch.cuda.caching_allocator_alloc(nbytes, dev, stream)
+
+    with ta.Window(buf, [0, n], [T0], [T0 + 10**9], alloc_fn=alloc, release_fn=torch.cuda.caching_allocator_delete) as w:
+        w.sort_timeline()
+        del asked[:]
+        w.match_collectives([(3, pids)])
+    # sorting: waits 8, list 4, keys 24, indices and groups 20, rows 60; and descriptors
+    assert sum(asked) <= 120 * n + (1 << 20), asked
+
+
 @pytest.mark.parametrize("lanes", [1, 2, 15, 16, 17, 33])
 @pytest.mark.parametrize("spread", [20, 10**6, 1 << 31])
 def test_overlap_of_merged_and_of_sorted_lanes(lanes, spread):
