@@ -938,6 +938,8 @@ ta_status ta_launch_load(ta_window *h, bool allow_packed) {
   if (((int64_t)h->W << h->tbits) > (1ll << 24)) return TA_ERR_TOO_LARGE;
   h->ibits = ta_bit_len((uint64_t)(max_win - 1));
   if (h->ibits < 1) h->ibits = 1;
+  // A single lane has no bits of its own; what names it is shifted all the same, by 63 at most.
+  const int lane_bits = hd + h->wbits + h->tbits, room = 64 - (lane_bits > 0 ? lane_bits : 1) - h->ibits;
   h->fast_keys = 0;
   h->xbits = 0;
   if (allow_packed && h->prekeys && h->tkeep > 0 && h->tkeep <= h->sbits) {
@@ -945,19 +947,19 @@ ta_status ta_launch_load(ta_window *h, bool allow_packed) {
     // the lane sizes give those of the passes above them: the first radix pass can build the
     // keys from the discovery words, no key pass is needed.  Passes over time bits and passes
     // over (dropped, window, triple rank) bits never share a digit.
-    const int T = h->tkeep, L = hd + h->wbits + h->tbits;
+    const int T = h->tkeep, L = lane_bits;
     // What is left of the 64 bits goes to further time bits below those that are sorted: the gather
     // ranks the records of a cell by them, without a look at the records.  Bursts are what gains by it: the
     // gather of 16.8 M prefill records, 82 % of them in cells with others and seven to a cell, takes 393 us
     // and 422 without; of 66.8 M expert records, 22 % and two, 1262 and 1255, and 512 windows of 65 k records
     // lost 490 to 468: windows of a batch go without.
-    const int spare = h->W == 1 ? 64 - (T + L + h->ibits) : 0;
+    const int spare = h->W == 1 ? room - T : 0;
     const int X = spare < 0 ? 0 : spare < h->sbits - T ? spare : h->sbits - T;
     const int lo = h->ibits + X;
     const SortPlan tp = ta_plan_bits(lo, lo + T);
     const SortPlan lp = ta_plan_bits(lo + T, lo + T + L);
     const int n_top = L > 0 ? lp.n_pass : 0;
-    if (T + L + h->ibits <= 64 && tp.n_pass <= 5 && tp.n_pass + n_top <= 10) {
+    if (T <= room && tp.n_pass <= 5 && tp.n_pass + n_top <= 10) {
       h->packed = 1;
       h->xbits = X;
       h->dshift = h->sbits - T - X;
@@ -984,7 +986,7 @@ ta_status ta_launch_load(ta_window *h, bool allow_packed) {
       return TA_OK;  // the words stay in d_keys (h->prekeys stays set): a retry can still use them
     }
   }
-  int drop = total + h->ibits - 64;
+  int drop = h->sbits - room;
   if (drop < 0) drop = 0;
   h->packed = allow_packed && drop <= TA_PACK_MAX_DROP && drop < h->sbits;
   if (h->packed) {

@@ -36,6 +36,38 @@ def test_runs_of_records_in_one_cell_of_the_sort_key(run, step):
         both(ev, off, [T0] * windows, [T0 + 31 * 10**9] * windows)
 
 
+@pytest.mark.parametrize("lanes", [1, 900])
+def test_keys_that_fill_their_word(lanes):
+    """A window as long as one may be, with enough lanes and records that the key has no room for all time bits
+    below the sorted ones: bursts told apart by those it has, by those it has not, and by the records."""
+    rng = np.random.default_rng(lanes)
+    n = 40_000
+    at = rng.integers(0, 1 << 20, n // 8) << 19
+    start = T0 + (at[:, None] + rng.integers(0, 4, (n // 8, 8)) * rng.choice([0, 1, 3, 64, 4000], (n // 8, 1))).reshape(-1)
+    ev = _device(n, start, rng.integers(0, 3, n), pid=np.repeat(rng.integers(0, lanes, n // 8), 8), kind=2)
+    both(ev[rng.permutation(n)], [0, n], [T0], [T0 + (1 << 40) - 1])
+
+
+def test_one_lane_whose_key_is_all_time_and_index():
+    """2^23 records and more of one thread in the longest window: 40 bits of time and 24 of the index."""
+    import torch
+    from paper_2609_40247_b200 import ta
+    n = (1 << 23) + 77
+    rng = np.random.default_rng(0)
+    ev = np.zeros(n, dtype=EVENT_DTYPE)
+    ev["ts_start"] = T0 + np.sort(rng.integers(0, 1 << 39, n)) + (1 << 38)
+    ev["ts_end"] = ev["ts_start"] + 1 + np.arange(n) % 3
+    ev["corr_id"], ev["kind"] = 1000 - np.arange(n), 2
+    ev = ev[np.concatenate([np.arange(i, n, 64) for i in range(64)])]
+    buf = torch.from_numpy(ev.view(np.uint8).reshape(-1)).cuda()
+    with ta.Window(buf, [0, n], [T0], [T0 + (1 << 40) - 1]) as w:
+        s = w.sort_timeline()
+        want = np.lexsort((np.arange(n), -ev["ts_end"], ev["ts_start"]))
+        assert np.array_equal(s.numpy("perm"), want) and s.n_lanes == 1
+        j = w.correlate_launches()
+        assert int(j.join_sum["n_launch"][0]) == int(j.join_sum["n_orphan_launch"][0]) == n
+
+
 @pytest.mark.parametrize("lanes,per", [(1, 3), (2, 255), (257, 9), (1030, 3), (40, 700)])
 def test_lane_table_from_the_counts_of_the_load(lanes, per):
     """Lanes of one window from the records counted per triple: one to several rounds of the CTA that
