@@ -89,8 +89,8 @@ __global__ void __launch_bounds__(OV_THREADS) k_ov_keys(OvKeyArgs a) {
 }
 
 // ---- merging the lanes of a process -------------------------------------------------------
-// Every lane is cut at its first record and behind every OM_STEP records (lanes of a process at different
-// ones of them, so that lanes in step are cut at different times).  Where a cut falls in the other lanes is
+// A process is cut in front of its first record, and every lane of it behind every OM_STEP records (lanes at
+// different ones of them, so that lanes in step are cut at different times).  Where a cut falls in the other lanes is
 // searched, and the number of cuts in front of it is its place among the cuts of the process: between
 // neighbouring cuts there is at most OM_STEP records of each lane, whatever the lanes look like - a stream of
 // 300 copies beside one of 2 M kernels, streams that work in turns, lanes of one record.  A CTA merges the
@@ -102,7 +102,9 @@ __global__ void __launch_bounds__(OV_THREADS) k_ov_keys(OvKeyArgs a) {
 // 250 k: 2 lanes 55 and 97, 12 88 and 95, 16 98 and 96.
 #define OM_LANES 12    // device lanes of a process at most
 #define OM_STEP 256
+#define OM_CUTS_FEW 8192  // places for cuts that cost a small window no more than its launches
 #define OM_THREADS 256
+#define OM_GRID (148 * 32)  // CTAs that merge where most places are empty (short lanes)
 struct OvMergeArgs {
   int64_t m;
   int n_lanes, n_cuts;  // places for cuts; not all are taken
@@ -117,10 +119,11 @@ struct OvMergeArgs {
   ulonglong2 *out;  // per device record in order: (ts_start - t0) << 1 | not a kernel; slot << 40 | clipped end - t0
   const int32_t *status;
 };
-// First place of the cuts of lane l: a lane of c records has at most c / OM_STEP + 2.
-__device__ __forceinline__ int ov_cut_base(const OvMergeArgs &a, int l) { return a.lane_dev_base[l] / OM_STEP + 2 * l; }
+// First place of the cuts of lane l: a lane of c records has at most c / OM_STEP + 1, the process's own among
+// those of its first lane.
+__device__ __forceinline__ int ov_cut_base(const OvMergeArgs &a, int l) { return a.lane_dev_base[l] / OM_STEP + l; }
 // Cuts in front of record c of a lane whose cuts are `phase` records early.
-__device__ __forceinline__ int ov_cuts_before(int c, int phase) { return c ? (c + phase + OM_STEP - 1) / OM_STEP : 0; }
+__device__ __forceinline__ int ov_cuts_before(int c, int phase) { return c + phase > 0 ? (c + phase - 1) / OM_STEP : 0; }
 
 // A warp per cut.  It searches all lanes at the same time: of k lanes, 32 / k threads each, so many probes a round.
 __global__ void __launch_bounds__(OM_THREADS) k_ov_cuts(OvMergeArgs a) {
@@ -143,7 +146,7 @@ __global__ void __launch_bounds__(OM_THREADS) k_ov_cuts(OvMergeArgs a) {
   const u32 mask = __ballot_sync(0xffffffffu, same);
   const int f = l - (OM_LANES - 1) + (__ffs((int)mask) - 1), k = __popc(mask);
   if (k > a.width - 1) return;
-  const int s = q - ov_cut_base(a, l), own = l - f;
+  const int own = l - f, s = q - ov_cut_base(a, l) + (own > 0);  // cut s of its lane; s = 0: of the process
   const int p = s ? s * OM_STEP - own * OM_STEP / k : 0;
   const int off = a.lane_off[l];
   if (p >= a.lane_off[l + 1] - off) return;
@@ -156,7 +159,7 @@ __global__ void __launch_bounds__(OM_THREADS) k_ov_cuts(OvMergeArgs a) {
   if (j < k) {
     joff = a.lane_off[f + j];
     if (j == own) lo = hi = p;
-    else hi = a.lane_off[f + j + 1] - joff;
+    else if (s) hi = a.lane_off[f + j + 1] - joff;
   }
   // records of lane f + j in front of the cut; of records that begin together those of the lanes in front come first
   while (__any_sync(0xffffffffu, lo < hi)) {
@@ -173,7 +176,7 @@ __global__ void __launch_bounds__(OM_THREADS) k_ov_cuts(OvMergeArgs a) {
       if (n < probes) hi = min(hi, lo + w - 1);
     }
   }
-  const u32 place = __reduce_add_sync(0xffffffffu, in ? (u32)ov_cuts_before(lo, j * OM_STEP / k) : 0u) + (u32)ov_cut_base(a, f);
+  const u32 place = __reduce_add_sync(0xffffffffu, in && s ? (u32)ov_cuts_before(lo, j * OM_STEP / k) : 0u) + (s > 0) + (u32)ov_cut_base(a, f);
   const u32 front = __reduce_add_sync(0xffffffffu, in ? (u32)lo : 0u);
   if (place >= (u32)a.n_cuts) return;
   int32_t *row = a.cut + (int64_t)place * a.width;
@@ -189,60 +192,63 @@ __global__ void __launch_bounds__(OM_THREADS) k_ov_merge(OvMergeArgs a) {
   extern __shared__ u64 ov_key[];  // ts_start - t0 of the records between the cuts, lane by lane
   __shared__ int s_from[OM_LANES], s_pre[OM_LANES + 1];
   if (ta_failed(a.status)) return;
-  const int i = (int)blockIdx.x, tid = (int)threadIdx.x;
-  const u32 lanes = a.lanes[i], next = i + 1 < a.n_cuts ? a.lanes[i + 1] : 0u;
-  if (!lanes) return;
-  const int f = (int)(lanes >> 5) - 1, k = (int)(lanes & 31u);
-  const int32_t *row = a.cut + (int64_t)i * a.width;
-  if (tid < 32) {
-    int from = 0, n = 0;
-    if (tid < k) {
-      from = row[1 + tid];
-      n = (next == lanes ? row[a.width + 1 + tid] : a.lane_off[f + tid + 1]) - from;
-      n = min(max(n, 0), OM_STEP);
-    }
-    const int upto = (int)warp_scan_inclusive((u64)n, OpAdd());
-    if (tid < k) {
-      s_from[tid] = from;
-      s_pre[tid + 1] = upto;
-    }
-    if (tid == 0) s_pre[0] = 0;
-  }
-  const int slot = a.lane_slot[f], w = a.lane_window[f];
-  const i64 w0 = a.t0[w], w1 = a.t1[w];
-  const int first = row[0];
-  __syncthreads();
-  const int total = s_pre[k];
-  auto lane_of = [&](int e) {
-    int j = 0;
-    while (e >= s_pre[j + 1]) j++;
-    return j;
-  };
-  for (int e = tid; e < total; e += OM_THREADS) {
-    const int j = lane_of(e);
-    ov_key[e] = (u64)(a.ts[s_from[j] + e - s_pre[j]] - w0);
-  }
-  __syncthreads();
-  for (int e = tid; e < total; e += OM_THREADS) {
-    const int own = lane_of(e), p = s_from[own] + e - s_pre[own];
-    const i64 te = a.te[p], end = te < w1 ? te : w1;
-    const int kd = a.kind[p];
-    const u64 x = ov_key[e];
-    int rank = e - s_pre[own];
-    for (int j = 0; j < k; j++) {
-      if (j == own) continue;
-      int lo = s_pre[j], hi = s_pre[j + 1];
-      const int at = lo;
-      const u64 y = x + (j < own ? 1 : 0);
-      while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if (ov_key[mid] < y) lo = mid + 1;
-        else hi = mid;
+  const int tid = (int)threadIdx.x;
+  for (int i = (int)blockIdx.x; i < a.n_cuts; i += (int)gridDim.x) {
+    const u32 lanes = a.lanes[i], next = i + 1 < a.n_cuts ? a.lanes[i + 1] : 0u;
+    if (!lanes) continue;
+    const int f = (int)(lanes >> 5) - 1, k = (int)(lanes & 31u);
+    const int32_t *row = a.cut + (int64_t)i * a.width;
+    __syncthreads();  // the round before is done with the shared arrays
+    if (tid < 32) {
+      int from = 0, n = 0;
+      if (tid < k) {
+        from = row[1 + tid];
+        n = (next == lanes ? row[a.width + 1 + tid] : a.lane_off[f + tid + 1]) - from;
+        n = min(max(n, 0), OM_STEP);
       }
-      rank += lo - at;
+      const int upto = (int)warp_scan_inclusive((u64)n, OpAdd());
+      if (tid < k) {
+        s_from[tid] = from;
+        s_pre[tid + 1] = upto;
+      }
+      if (tid == 0) s_pre[0] = 0;
     }
-    if ((u64)(first + rank) < (u64)a.m)
-      a.out[first + rank] = make_ulonglong2(x << 1 | (kd != TA_KIND_KERNEL), (u64)slot << 40 | (u64)(end - w0));
+    const int slot = a.lane_slot[f], w = a.lane_window[f];
+    const i64 w0 = a.t0[w], w1 = a.t1[w];
+    const int first = row[0];
+    __syncthreads();
+    const int total = s_pre[k];
+    auto lane_of = [&](int e) {
+      int j = 0;
+      while (e >= s_pre[j + 1]) j++;
+      return j;
+    };
+    for (int e = tid; e < total; e += OM_THREADS) {
+      const int j = lane_of(e);
+      ov_key[e] = (u64)(a.ts[s_from[j] + e - s_pre[j]] - w0);
+    }
+    __syncthreads();
+    for (int e = tid; e < total; e += OM_THREADS) {
+      const int own = lane_of(e), p = s_from[own] + e - s_pre[own];
+      const i64 te = a.te[p], end = te < w1 ? te : w1;
+      const int kd = a.kind[p];
+      const u64 x = ov_key[e];
+      int rank = e - s_pre[own];
+      for (int j = 0; j < k; j++) {
+        if (j == own) continue;
+        int lo = s_pre[j], hi = s_pre[j + 1];
+        const int at = lo;
+        const u64 y = x + (j < own ? 1 : 0);
+        while (lo < hi) {
+          const int mid = (lo + hi) >> 1;
+          if (ov_key[mid] < y) lo = mid + 1;
+          else hi = mid;
+        }
+        rank += lo - at;
+      }
+      if ((u64)(first + rank) < (u64)a.m)
+        a.out[first + rank] = make_ulonglong2(x << 1 | (kd != TA_KIND_KERNEL), (u64)slot << 40 | (u64)(end - w0));
+    }
   }
 }
 
@@ -464,10 +470,12 @@ ta_status ta_run_overlap(ta_window *h, ta_overlap_result *out) {
   ro.d_exposed = ck.take<int64_t>(n_slots);
 
   const int64_t tiles = (m + OV_TILE - 1) / OV_TILE;
-  // Merging takes no more memory than sorting: short lanes have cuts that are as large as their records.
+  // Short lanes have places for cuts that nothing is between, and a table of them that is larger than what
+  // sorting takes: 2.9 M records in lanes of 120 196 us merged and 312 sorted, 1 M in lanes of eight 325 and 186.
   const int width = h->max_dev_lanes + 1;
-  const int64_t n_cuts = m / OM_STEP + 2 * (int64_t)h->sorted.n_lanes + 1;
-  const bool merge = h->max_dev_lanes <= OM_LANES && n_cuts * (width + 1) * 4 <= 16 * m + (64 << 10);
+  const int64_t n_cuts = m / OM_STEP + (int64_t)h->sorted.n_lanes + 1;
+  const bool merge = h->max_dev_lanes <= OM_LANES && n_cuts <= (m / 32 > OM_CUTS_FEW ? m / 32 : OM_CUTS_FEW) &&
+                     n_cuts * (width + 1) * 4 <= 16 * m + (64 << 10);
   size_t tb = merge ? Carver::pad((size_t)m * 16) + Carver::pad((size_t)n_cuts * width * 4)
                     : 3 * Carver::pad((size_t)m * 8) + 3 * Carver::pad((size_t)m * 4) + ta_sort_temp_bytes(m);
   tb += scan_temp_bytes(n_slots) + 512;
@@ -496,7 +504,9 @@ ta_status ta_run_overlap(ta_window *h, ta_overlap_result *out) {
     const size_t smem = (size_t)h->max_dev_lanes * OM_STEP * sizeof(u64);
     static_assert(OM_LANES * OM_STEP * sizeof(u64) <= 40u << 10 && 2 * OM_LANES - 1 <= 32, "within what a kernel has without being asked");
     ta_launch(k_ov_cuts, (unsigned)((n_cuts + OM_THREADS / 32 - 1) / (OM_THREADS / 32)), OM_THREADS, 0, st, ma);
-    ta_launch(k_ov_merge, (unsigned)n_cuts, OM_THREADS, smem, st, ma);
+    // (a CTA per place else: 12 even lanes of 4 M records 328 us, by that grid 350)
+    const bool empty = h->sorted.n_lanes > m / OM_STEP && n_cuts > OM_GRID;
+    ta_launch(k_ov_merge, (unsigned)(empty ? OM_GRID : n_cuts), OM_THREADS, smem, st, ma);
   } else {
     u64 *k_in = ct.take<u64>(m), *k_scr = ct.take<u64>(m), *k_fin = ct.take<u64>(m);
     u32 *v_in = ct.take<u32>(m), *v_scr = ct.take<u32>(m), *v_fin = ct.take<u32>(m);

@@ -258,18 +258,34 @@ def test_overlap_of_many_lanes_of_one_record(pids, windows):
     both(ev, np.arange(windows + 1) * pids * 4, T0 + np.arange(windows) * 10**6, T0 + np.arange(1, windows + 1) * 10**6)
 
 
-def test_overlap_of_a_sparse_lane_beside_a_full_one_takes_no_longer():
-    """300 records spread over 2 M others: with the sparse lane walked record by record through the full one
-    the call took 60 times what it takes of two even lanes; both take about the same."""
+@pytest.mark.parametrize("shape", ["sparse beside full", "short lanes"])
+def test_overlap_takes_no_longer_on_lanes_of_another_filling(shape):
+    """300 records spread over 2 M others (with the sparse lane walked record by record through the full one the
+    call took 60 times what it takes of two even lanes) and 2000 windows of 64 lanes of eight records (ten
+    times, merged): both take about what two even lanes of as many records take."""
     import torch
     from paper_2609_40247_b200 import ta
     rng = np.random.default_rng(5)
+
+    def even(n):
+        return [(np.concatenate([_device(n // 2, T0 + np.sort(rng.integers(0, 30 * 10**9, n // 2)), 1000, stream=s)
+                                 for s in (0, 1)]), 1)]
+    if shape == "short lanes":
+        k = np.arange(1 << 20)
+        odd = [(_device(len(k), T0 + k // 512 * 10**6 + k % 512 * 1000, 700, pid=k // 64 % 8 * 3, stream=k % 8), 2048)]
+        host = _device(2048 * 8, T0 + np.arange(2048 * 8) // 8 * 10**6, 10, pid=np.arange(2048 * 8) % 8 * 3, kind=1)
+        odd = [(np.concatenate([odd[0][0], host]), 2048)]
+    else:
+        odd = [(np.concatenate([_device(n, T0 + np.sort(rng.integers(0, 30 * 10**9, n)), 1000, stream=s)
+                                for s, n in enumerate((2_000_000, 300))]), 1)]
     times = []
-    for sizes in ((2_000_000, 300), (1_000_150, 1_000_150)):
-        ev = np.concatenate([_device(n, T0 + np.sort(rng.integers(0, 30 * 10**9, n)), 1000, stream=s)
-                             for s, n in enumerate(sizes)])
+    for ev, windows in odd + even(len(odd[0][0])):
+        window = (ev["ts_start"] - T0) // 10**6 if windows > 1 else np.zeros(len(ev), dtype=np.int64)
+        ev = ev[np.argsort(window, kind="stable")]
+        off = np.concatenate([[0], np.cumsum(np.bincount(window, minlength=windows))])
+        span = 10**6 if windows > 1 else 30 * 10**9
         buf = torch.from_numpy(ev.view(np.uint8).reshape(-1)).cuda()
-        with ta.Window(buf, [0, len(ev)], [T0], [T0 + 30 * 10**9]) as w:
+        with ta.Window(buf, off, T0 + np.arange(windows) * span, T0 + np.arange(1, windows + 1) * span) as w:
             w.sort_timeline()
             best = float("inf")
             for _ in range(8):
