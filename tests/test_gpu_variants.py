@@ -310,6 +310,98 @@ def test_long_gaps_ordered_by_one_cta_and_by_many(n):
         both(ev, [0, n], [T0], [T0 + (1 << 35)], min_gap=500 if every > 1 else 1)
 
 
+@pytest.mark.parametrize("n,every", [(8191, 1), (8192, 1), (262_144, 400), (262_145, 400)])
+def test_long_gaps_at_the_limits_of_one_cta(n, every):
+    """A list of 8192 entries and one more (a gap in front of every record and one behind the last), and a
+    bitmap of 8192 words and one more with a list far below."""
+    wait = np.where(np.arange(n) % every == 0, 700, 0)
+    _, g = both(_device(n, T0 + np.cumsum(wait + 10), 10), [0, n], [T0], [T0 + (1 << 35)], min_gap=500)
+    assert len(g["long_gaps"]) == (n + every - 1) // every + 1
+
+
+@pytest.mark.parametrize("comms", [31, 32, 33, 64])
+def test_collectives_of_communicators_few_and_many(comms):
+    """Communicator sizes that travel with the launch, and those that are copied: right, too small, not given."""
+    rng = np.random.default_rng(comms)
+    seqs, pids = 20, 3
+    k = np.arange(comms * seqs * pids)
+    ev = _device(len(k), T0 + k * 50 + rng.integers(0, 500, len(k)), 40, pid=k % pids, kind=5)
+    ev["corr_id"], ev["seq"] = 10**12 - k // pids % comms * 7, k // (pids * comms)
+    ev = ev[rng.permutation(len(ev))[:-5]]
+    sizes = [(10**12 - c * 7, pids + (c % 5 == 2)) for c in range(comms) if c % 4 != 3]
+    both(ev, [0, len(ev)], [T0], [T0 + 10**9], comm_sizes=sizes)
+
+
+@pytest.mark.parametrize("windows", [1, 2])
+@pytest.mark.parametrize("beyond", [0, 1])
+def test_collectives_at_the_limit_of_the_cells(beyond, windows):
+    """As many cells as two per member and 4096, and one per window more."""
+    m = 600 * windows
+    last = (2 * m + 4096) // windows - 1 + beyond  # largest sequence number: last + 1 cells a window
+    k = np.arange(600)
+    one = _device(600, k // 2 * 300, 100, pid=k % 2, kind=5)
+    one["corr_id"], one["seq"] = 9, np.where(k // 2 == 299, last, k // 2 * 3)
+    parts = []
+    for w in range(windows):
+        parts.append(one.copy())
+        parts[-1]["ts_start"] += T0 + w * 10**6
+        parts[-1]["ts_end"] += T0 + w * 10**6
+    both(np.concatenate(parts), np.arange(windows + 1) * 600, T0 + np.arange(windows) * 10**6,
+         T0 + np.arange(1, windows + 1) * 10**6, comm_sizes=[(9, 2)])
+
+
+@pytest.mark.parametrize("run", [1, 200])
+def test_gather_order_of_processes_of_uneven_size(run):
+    """Two processes of 4.9 M and 0.2 M records, whose lanes are taken by turns, one of them without records in the
+    first half; with a run of equal times too long to be ranked in place (200) the order is not used."""
+    n = 5_100_001
+    rng = np.random.default_rng(run)
+    k = np.arange(n)
+    ev = np.zeros(n, dtype=EVENT_DTYPE)
+    ev["pid"] = np.where(k % 25 == 3, 4, 2)
+    device = k % 7 > 2
+    ev["kind"] = np.where(device, 3, 2)
+    ev["stream"] = np.where(device, np.where((k % 5 == 4) & (k > n // 2), 9, 1), 0)
+    ev["ts_start"] = T0 + k * 5000 + rng.integers(0, 5000, n)
+    ev["ts_start"][1000:1000 + run] = T0 + 7
+    ev["ts_end"] = ev["ts_start"] + 2000
+    ev["corr_id"] = k // 2
+    ev = ev[np.argsort(k // 4096 * 2 + device, kind="stable")]
+    both(ev, [0, n], [T0], [T0 + n * 5000], min_gap=50_000_000)
+
+
+def test_noalloc_call_that_fails_leaves_nothing_to_the_next():
+    """A call under stream capture is refused when it comes to wait, after it has taken its place among the
+    calls; what follows clears the sums itself."""
+    import torch
+    from paper_2609_40247_b200 import ta
+    start = torch.arange(5000, dtype=torch.int64, device="cuda") * 100 + T0
+    end = start + 60
+    gap, lane = torch.empty_like(start), torch.zeros(ta.LANE_GAPS.itemsize, dtype=torch.uint8, device="cuda")
+
+    def check():
+        _, row = ta.lane_gaps_noalloc(start, end, T0, T0 + 10**6, gap, lane)
+        assert int(row["busy"]) == 300_000 and int(row["n_gaps"]) == 5000 and int(row["n_events"]) == 5000
+        assert int(gap.sum()) == 4999 * 40
+
+    check()
+    check()
+    for _ in range(3):
+        graph, refused = torch.cuda.CUDAGraph(), False
+        try:
+            with torch.cuda.graph(graph):
+                try:
+                    ta.lane_gaps_noalloc(start, end, T0, T0 + 10**6, gap, lane)
+                except ta.TaError:
+                    refused = True
+        except RuntimeError:
+            pass  # the capture ends with the error
+        assert refused
+        torch.cuda.synchronize()
+        check()
+    check()
+
+
 @pytest.mark.parametrize("order", ["aaaa", "adad", "ddaa", "aeda"])
 def test_noalloc_calls_that_follow_one_another(order):
     """The sums of a call are cleared by the one in front of it: lanes that end their records in
