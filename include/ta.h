@@ -610,8 +610,8 @@ ta_status ta_critical_path(ta_window *h, ta_critpath_result *out,
  * allocates on the device.  (Its first call on a device asks for a hundred bytes of
  * page-locked host memory, which may synchronise the device, and does without if there
  * are none.)
- * Its scratch (tile descriptors of the scan, a counter, a status word: about
- * 16 KB) is a fixed array inside the library image, which every GPU that loads
+ * Its scratch (tile descriptors of the scan, two sets of sums, counters and status
+ * words: about 16 KB) is a fixed array inside the library image, which every GPU that loads
  * the library holds until the process exits.
  *
  * Input: the records of one device lane of one window [win_t0, win_t1), already
@@ -629,9 +629,10 @@ ta_status ta_critical_path(ta_window *h, ta_critpath_result *out,
  * which the CUDA runtime may load the library's code and the scratch array onto
  * the device (lazy module loading), which does take device memory: make it once
  * at start-up, before the heap is reserved, not at the first moment of need.  All calls on a device share the
- * one scratch array, which keeps the previous call's contents; each call clears
- * it first, so two calls that overlap on the GPU (different streams or threads)
- * race and must be serialised by the caller.  The call enqueues its work on
+ * one scratch array.  They take its two sets of sums in turn: a call's last block clears
+ * the set of the next call, and a call that does not follow one that was alone on
+ * the device and succeeded clears both first.  Two calls that overlap on the GPU
+ * (different streams or threads) race and must be serialised by the caller.  The call enqueues its work on
  * cuda_stream, waits for it and returns TA_OK, TA_ERR_INVALID_ARG,
  * TA_ERR_TOO_LARGE, TA_ERR_CUDA or TA_ERR_TIMEOUT.
  */

@@ -2,14 +2,18 @@
 // are linked, and every rank's wait for the last arrival is measured (cross-process
 // links: Sec. 6.1 "Execution progress and state"; ranks held up by a late one: Sec. 9.2).  Group key (window, comm_id, seq).
 //
-//   1. compact the COLL records (a few percent of the window), in sorted-
-//      position order, which is pid-major;
-//   2. stable pair sort by (window | communicator rank | seq - min seq): the
-//      members of a group become adjacent and stay ordered by pid;
-//   3. group heads by comparing neighbours, group ids by a scan;
-//   4. one thread per group: arrival range, skew, straggler, flags;
-//   5. one thread per member in pid-major order: wait, and per-(window, pid)
-//      totals folded per CTA before they touch global memory.
+// Sequence numbers count up per communicator, so the keys of a window's groups fill a table well, and a
+// collective's members meet in one of its cells:
+//
+//   1. every COLL record adds itself to its cell (k_coll_cells), which lists it for 3 on the way;
+//   2. the cells that hold a group, in order, become rows: arrival range, skew, straggler, flags (k_coll_rows);
+//   3. one thread per member: wait, and per-(window, pid) totals folded per CTA before they touch
+//      global memory (k_coll_members).
+//
+// With more than 64 processes, numbers too sparse, or no memory for as many cells, the members are sorted instead:
+// compaction in sorted-position order, which is pid-major; stable pair sort by (window | communicator rank |
+// seq - min seq), so that the members of a group become adjacent and stay ordered by pid; group heads by
+// comparing neighbours, group ids by a scan; one thread per group; then 3.
 #include <algorithm>
 #include <climits>
 #include <vector>

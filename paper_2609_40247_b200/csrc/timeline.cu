@@ -362,7 +362,7 @@ __device__ __forceinline__ void slot_ranges(const SlotRanges &a, u64 *tmp) {
     const int64_t s = s0 + threadIdx.x;
     u64 size = 0;
     if (s < a.n_slots) {
-        const u64 mx = __ldcg(&a.code[s]), mn_inv = __ldcg(&a.code[a.n_slots + s]);
+      const u64 mx = __ldcg(&a.code[s]), mn_inv = __ldcg(&a.code[a.n_slots + s]);
       const bool any = mx != 0 || mn_inv != 0;
       a.slot_max[s] = any ? (i64)(mx ^ (1ull << 63)) : INT64_MIN;
       a.slot_min[s] = any ? (i64)((~mn_inv) ^ (1ull << 63)) : INT64_MAX;
