@@ -238,8 +238,9 @@ def built_path_bytes_per_event(wl, radix_bytes_per_event):
 
 
 def touched_bytes_per_event(wl, radix_bytes_per_event):
-    """Algorithmic bytes per record of the path AS BUILT (but for the collectives, see there), kernel by kernel: reads and writes of
-    every column or table a kernel touches, clearings and read-modify-write atomics included.
+    """Algorithmic bytes per record of the path AS BUILT (but for the collectives, see there), kernel
+    by kernel: reads and writes of every column or table a kernel touches, clearings and
+    read-modify-write atomics included.
     Lookups that stay in cache across a tile count once per record, rows that are written again
     while they are in cache once.  The radix passes enter with the bytes the library reports for
     them (16 B per record and pass for packed keys).  f_x = share of the records of kind x."""
@@ -263,7 +264,7 @@ def touched_bytes_per_event(wl, radix_bytes_per_event):
         "gaps": f_d * 16.0 + 8.0,
         "aggregate": f_d * 22.0 + f_h * 6.0 + f_o * 20.0,
         # waits cleared, kind; members as by compaction, pair sort and groups, so that figures of
-        # different builds compare (by cells they touch 84 bytes: 1.3 less per record of 372 on c3)
+        # different builds compare (by cells they touch 76 bytes: 1.9 less per record of 372 on c3)
         "collectives": 8.0 + 2.0 + f_c * 100.0,
     }
     return sum(parts.values()), parts

@@ -159,9 +159,8 @@ __global__ void __launch_bounds__(256) k_coll_groups(CollGroupArgs a) {
 
 struct CollMemberArgs {
   CollCtx c;
-  const int32_t *slot_of;
   // sorted groups
-  const int32_t *gid_of_c;
+  const int32_t *slot_of, *gid_of_c;
   const int64_t *g_max;
   const int32_t *g_flags;
   // cells
@@ -195,6 +194,7 @@ struct CollCells {
   int32_t few[CC_FEW];        // (a copy costs more than the kernel)
 };
 
+static_assert(24 + CC_REL_BITS <= 64, "fewer than 2^24 slots");
 // A CTA takes 8192 sorted positions: it picks out the COLL records, clears the wait column, and has its threads
 // add the records to their cells, one each.  The list it leaves for k_coll_members is in order inside a
 // tile; tiles take their places as they come.
@@ -203,8 +203,7 @@ struct CollCells {
 #define CT_TILE (CT_THREADS * CT_ITEMS)
 struct CollList {
   u32 *pos, *cell;
-  u64 *rel;       // start relative to the window
-  int32_t *slot;
+  u64 *rel;       // slot << CC_REL_BITS | start relative to the window
   u32 *n;
 };
 __global__ void __launch_bounds__(CT_THREADS) k_coll_cells(CollCtx c, CollCells x, const int16_t *kind, int64_t n_valid,
@@ -267,8 +266,7 @@ __global__ void __launch_bounds__(CT_THREADS) k_coll_cells(CollCtx c, CollCells 
     if (seen & bit) atomicAdd(&x.more[cell], 1u);
     o.pos[base + j] = p;
     o.cell[base + j] = (u32)cell;
-    o.rel[base + j] = rel;
-    o.slot[base + j] = slot;
+    o.rel[base + j] = (u64)slot << CC_REL_BITS | rel;
   }
 }
 
@@ -388,6 +386,7 @@ __device__ __forceinline__ void coll_members(const CollMemberArgs &a) {
   __shared__ int s_same;
   __shared__ u64 red[4][8];
   if (ta_failed(a.status)) return;
+  auto slot_at = [&](int64_t i) { return CELLS ? (int)(a.rel_of[i] >> CC_REL_BITS) : a.slot_of[i]; };
   int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const bool in = j < a.c.m;
   int slot = -1;
@@ -398,7 +397,7 @@ __device__ __forceinline__ void coll_members(const CollMemberArgs &a) {
     bool counts;
     if (CELLS) {
       const u64 d = a.done[a.cell_of[j]];
-      w = (i64)(d >> 1) - (i64)a.rel_of[j];
+      w = (i64)(d >> 1) - (i64)(a.rel_of[j] & ((1ull << CC_REL_BITS) - 1));
       counts = d & 1u;
     } else {
       int g = a.gid_of_c[j];
@@ -406,12 +405,12 @@ __device__ __forceinline__ void coll_members(const CollMemberArgs &a) {
       counts = a.g_flags[g] == 0;
     }
     a.wait_ns[p] = w;
-    slot = a.slot_of[j];
+    slot = slot_at(j);
     if (counts) { ok = 1; wait = (u64)w; }
   }
   if (threadIdx.x == 0) s_same = 1;
   __syncthreads();
-  const int block_first = a.slot_of[min((int64_t)blockIdx.x * blockDim.x, a.c.m - 1)];
+  const int block_first = slot_at(min((int64_t)blockIdx.x * blockDim.x, a.c.m - 1));
   if (in && slot != block_first) s_same = 0;
   __syncthreads();
   if (s_same) {
@@ -543,12 +542,12 @@ ta_status ta_run_collectives(ta_window *h, const ta_comm_size *sizes, int32_t n_
 
   // Cells of the direct table.  Up to two per member (and a few thousand): clearing and scanning them
   // costs less than sorting the members.  They are taken from the handle's cleared pool; where it has no room
-  // (long windows) the way by cells must not ask for more memory than sorting does, 112 bytes per member and more.
+  // (long windows) the way by cells must not ask for more memory than sorting does, some 108 bytes per member.
   const unsigned __int128 all_cells = (unsigned __int128)h->W * (unsigned)h->n_comms * (uint64_t)(h->max_seq - h->min_seq + 1);
   bool cells = n_pids <= CC_MAX_PIDS && all_cells <= (unsigned __int128)(2 * m + 4096);
   const int64_t nc = cells ? (int64_t)all_cells : 0;
   const size_t cells_zeroed = 4 * Carver::pad((size_t)nc * 8) + Carver::pad((size_t)nc * 4) + Carver::pad(4) + scan_temp_bytes(nc);
-  const size_t cells_temp = Carver::pad((size_t)m * 8) + 3 * Carver::pad((size_t)m * 4) + Carver::pad((size_t)h->n_comms * 4) +
+  const size_t cells_temp = Carver::pad((size_t)m * 8) + 2 * Carver::pad((size_t)m * 4) + Carver::pad((size_t)h->n_comms * 4) +
                             scan_temp_bytes(n_slots) + 256;
   const size_t sort_list = Carver::pad((size_t)m * 4) + scan_temp_bytes(n) + 256;
   const size_t sort_temp = 3 * Carver::pad((size_t)m * 8) + 4 * Carver::pad((size_t)m * 4) + Carver::pad((size_t)(m + 1) * 4) +
@@ -589,7 +588,6 @@ ta_status ta_run_collectives(ta_window *h, const ta_comm_size *sizes, int32_t n_
     CollList list;
     list.rel = c2.take<u64>(m);
     list.pos = c2.take<u32>(m); list.cell = c2.take<u32>(m);
-    list.slot = c2.take<int32_t>(m);
     int32_t *d_expected = c2.take<int32_t>(h->n_comms);
     scan3 = c2.base + c2.off;
     if (!zc && !(zc = ta_zalloc(h, cells_zeroed, &zs))) return zs;
@@ -614,7 +612,7 @@ ta_status ta_run_collectives(ta_window *h, const ta_comm_size *sizes, int32_t n_
                      ga.g_end, r_nstrag, h->d_triples};
     ta_launch(k_coll_rows, (unsigned)((nc + CW_TILE - 1) / CW_TILE), CW_THREADS, 0, st, cx, x, o, s2, h->d_status);
     ng_dev = s2.total;
-    ma.cell_of = list.cell; ma.rel_of = list.rel; ma.done = x.done; ma.slot_of = list.slot;
+    ma.cell_of = list.cell; ma.rel_of = list.rel; ma.done = x.done;
     cx.posc = list.pos;
   } else {
     // 1. compaction
